@@ -265,6 +265,7 @@ int faar_create(faar_ctx** out, int device, void* stream) {
   c->tune_wide = -1;
   c->last_gemm_split = 0;
   for (int i = 0; i < FAAR_GEMM_VARIANTS; ++i) c->gemm_max_pairs[i] = 0;
+  c->fp4_max_pairs[0] = c->fp4_max_pairs[1] = 0;
   c->wsoft_ws = nullptr;
   c->wsoft_beta = 0.f;
   c->copy_stream = nullptr;

@@ -131,6 +131,13 @@ def test_own_nvfp4_gemm_at_the_down_proj_size(ctx):
     _check_nvfp4_gemm(ctx, 2048, 8192, 4096, seed=1, sample=64)
 
 
+@pytest.mark.parametrize("O,K,T", [(2300, 288, 2100), (4100, 1312, 3000), (2304, 32, 2304)])
+def test_own_nvfp4_gemm_with_wide_tiles(ctx, O, K, T):
+    """Enough output for 256 x 256 tiles on every CTA pair, with two or three tiles on some (both accumulators, which
+    share columns): ragged edges in all three sizes, one and several stages per tile."""
+    _check_nvfp4_gemm(ctx, O, K, T, seed=O + K, sample=128)
+
+
 def test_own_nvfp4_gemm_agrees_with_the_layer_path(ctx):
     """X_q W_final^T computed two ways by this library: the FP4 GEMM on the packed operands, and the BF16
     tensor-core GEMM (frozen-target call) on the same values written out in BF16 (activations: units times
