@@ -680,8 +680,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer (leader CTA only) ----------------
-    if (lane == 0 && rank == 0) {
+    // ---------------- MMA issuer (leader CTA only; the whole warp, converged: see faar_elect_one) ----------------
+    if (rank == 0) {
       int stage = 0; uint32_t phase = 0;
       int it = 0;
       bool ok = true;
@@ -691,34 +691,39 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const uint32_t acc_phase = WIDE ? it & 1 : (it >> 1) & 1;
         ok = mbar_wait(tempty_bar(acc), acc_phase ^ 1u, ac, 0x200u | acc);
         if (ok && WIDE) ok = mbar_wait(tempty_bar(1), acc_phase ^ 1u, ac, 0x201u);
+        ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + acc * BN_MAX;
         const uint32_t idesc = make_idesc(WIDE ? BN_MAX : tile_coord(p, tile, m_tiles).w, A_MN ? 1 : 0, B_MN ? 1 : 0);
         for (int kb = 0; kb < k_blocks; ++kb) {
-          ok = mbar_wait(full_bar(stage), phase, ac, 0x300u | stage);
+          ok = __all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, ac, 0x300u | stage));
           if (!ok) break;
           tc_fence_after();
           const uint32_t sa = base + stage * C::STAGE_BYTES, sb = sa + C::A_BYTES;
           const uint64_t da = A_MN ? make_smem_desc_mn(sa) : make_smem_desc(sa);
           const uint64_t db = B_MN ? make_smem_desc_mn(sb) : make_smem_desc(sb);
           constexpr uint32_t ka = A_MN ? MN_KSTEP : 2u, kbs = B_MN ? MN_KSTEP : 2u;
+          if (faar_elect_one()) {
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
-            // advancing 16 bf16 = 32 bytes inside the swizzled row: +2 in the 16-byte address field
-            // (MN-major: 16 rows of 128 bytes further on)
-            tc_mma_bf16(tmem_d, da + ka * k, db + kbs * k, idesc, (kb | k) != 0 ? 1u : 0u);
-            if (WIDE)
-              tc_mma_bf16(tmem_d + BN_MAX, da + 2u * k, make_smem_desc(sb + C::BH_BYTES) + 2u * k, idesc,
-                          (kb | k) != 0 ? 1u : 0u);
+            for (int k = 0; k < BK / UMMA_K; ++k) {
+              // advancing 16 bf16 = 32 bytes inside the swizzled row: +2 in the 16-byte address field
+              // (MN-major: 16 rows of 128 bytes further on)
+              tc_mma_bf16(tmem_d, da + ka * k, db + kbs * k, idesc, (kb | k) != 0 ? 1u : 0u);
+              if (WIDE)
+                tc_mma_bf16(tmem_d + BN_MAX, da + 2u * k, make_smem_desc(sb + C::BH_BYTES) + 2u * k, idesc,
+                            (kb | k) != 0 ? 1u : 0u);
+            }
+            tc_commit_pair(empty_bar(stage));          // frees this stage in both CTAs
           }
-          tc_commit_pair(empty_bar(stage));            // frees this stage in both CTAs
+          __syncwarp();
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok) {
+        if (ok && faar_elect_one()) {
           tc_commit_pair(tfull_bar(acc));              // accumulator ready in both CTAs
           if (WIDE) tc_commit_pair(tfull_bar(1));
         }
+        __syncwarp();
       }
     }
   } else {
