@@ -11,7 +11,8 @@
 //   m is the row's reference, not its running maximum: it moves to a tile's maximum only when that exceeds it by
 //   more than 2^8 (probabilities stay below 2^8, the final division by their sum and lse = m + log2(sum) are
 //   exact either way); only then is O rescaled, in tensor memory, between two P V products.
-// Q, K_j, V_j arrive by TMA (two stages for K and V).  A fifth warp's lane 0 issues every copy and every MMA; the
+// Q, K_j, V_j arrive by TMA (two stages for K and V).  A fifth warp issues every copy and every MMA (by one lane of a
+// converged warp: fwd 145.5 -> 140.6 us, bwd 385 -> 354 us at 4 x 2048 tokens, 32 heads, against a lane-0 branch); the
 // scores have two buffers in tensor memory, so S of tile j + 1 is formed while the warps work on tile j, and two
 // CTAs per SM overlap what remains serial (softmax -> P V).
 // Rows of a query tile beyond the sequence end compute on whatever rows follow in memory (or zeros past the
@@ -224,57 +225,71 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   auto sV = [&](int s) { return base + OFF_V + (uint32_t)s * KV_BYTES; };
 
   if (warp == 4) {
-    // ---------------- copies and MMAs: one thread ----------------
-    if (lane == 0) {
-      auto load_k = [&](int j) { bar_expect(kfull(j & 1), KV_BYTES); tma_2d(sK(j & 1), &tmK, g * HD, (int)(seq0 + (long long)j * KT), kfull(j & 1)); };
-      auto load_v = [&](int j) { bar_expect(vfull(j & 1), KV_BYTES); tma_2d(sV(j & 1), &tmV, g * HD, (int)(seq0 + (long long)j * KT), vfull(j & 1)); };
+    // ---------------- copies and MMAs: one lane of this warp, which stays converged (see faar_elect_one) ----------
+    const bool lead = lane == 0;
+    auto wait = [&](uint32_t bar, uint32_t parity, uint32_t code) {
+      return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
+    };
+    auto load_k = [&](int j) {
+      if (lead) { bar_expect(kfull(j & 1), KV_BYTES); tma_2d(sK(j & 1), &tmK, g * HD, (int)(seq0 + (long long)j * KT), kfull(j & 1)); }
+      __syncwarp();
+    };
+    auto load_v = [&](int j) {
+      if (lead) { bar_expect(vfull(j & 1), KV_BYTES); tma_2d(sV(j & 1), &tmV, g * HD, (int)(seq0 + (long long)j * KT), vfull(j & 1)); }
+      __syncwarp();
+    };
+    if (lead) {
       bar_expect(bar_q, Q_BYTES);
       tma_2d(sQ, &tmQ, h * HD, (int)(seq0 + q0), bar_q);
-      load_k(0); load_v(0);
-      if (n_kt > 1) { load_k(1); load_v(1); }
-      bool ok = bar_wait(bar_q, 0u, abort_flag, 0xA01u);
-      const uint32_t id_s = idesc(0), id_pv = idesc(1);
-      // S of tile j into score buffer j & 1.  The scores of tile j + 1 are issued before this thread waits for the
-      // probabilities of tile j, so the tensor cores form them while the four warps work on tile j.
-      auto issue_s = [&](int j) {
-        const uint64_t da = desc_k_major(sQ), db = desc_k_major(sK(j & 1));
+    }
+    load_k(0); load_v(0);
+    if (n_kt > 1) { load_k(1); load_v(1); }
+    bool ok = wait(bar_q, 0u, 0xA01u);
+    const uint32_t id_s = idesc(0), id_pv = idesc(1);
+    // S of tile j into score buffer j & 1.  The scores of tile j + 1 are issued before this warp waits for the
+    // probabilities of tile j, so the tensor cores form them while the four warps work on tile j.
+    auto issue_s = [&](int j) {
+      const uint64_t da = desc_k_major(sQ), db = desc_k_major(sK(j & 1));
+      if (faar_elect_one()) {
 #pragma unroll
         for (int k = 0; k < HD / 16; ++k) mma(tmem + 64u * (uint32_t)(j & 1), da + 2u * k, db + 2u * k, id_s, k != 0 ? 1u : 0u);
         commit(bar_s(j & 1));
-      };
-      if (ok) ok = bar_wait(kfull(0), 0u, abort_flag, 0xA10u);
-      if (ok) { fence_after(); issue_s(0); }
-      for (int j = 0; j < n_kt && ok; ++j) {
-        const int st = j & 1;
-        const uint32_t ph = (uint32_t)((j >> 1) & 1);
-        if (j + 1 < n_kt) {
-          ok = bar_wait(kfull((j + 1) & 1), (uint32_t)(((j + 1) >> 1) & 1), abort_flag, 0xA10u | ((j + 1) & 1));
-          // its score buffer last held tile j - 1
-          if (ok && j >= 1) ok = bar_wait(bar_sfree((j + 1) & 1), (uint32_t)(((j - 1) >> 1) & 1), abort_flag, 0xA20u);
-          if (!ok) break;
-          fence_after();
-          issue_s(j + 1);
-        }
-        // P_j written (into P buffer j & 1): S_j has been read, so its K stage is free
-        ok = bar_wait(bar_p, (uint32_t)(j & 1), abort_flag, 0xA30u);
+      }
+      __syncwarp();
+    };
+    if (ok) ok = wait(kfull(0), 0u, 0xA10u);
+    if (ok) { fence_after(); issue_s(0); }
+    for (int j = 0; j < n_kt && ok; ++j) {
+      const int st = j & 1;
+      const uint32_t ph = (uint32_t)((j >> 1) & 1);
+      if (j + 1 < n_kt) {
+        ok = wait(kfull((j + 1) & 1), (uint32_t)(((j + 1) >> 1) & 1), 0xA10u | ((j + 1) & 1));
+        // its score buffer last held tile j - 1
+        if (ok && j >= 1) ok = wait(bar_sfree((j + 1) & 1), (uint32_t)(((j - 1) >> 1) & 1), 0xA20u);
         if (!ok) break;
-        if (j + 2 < n_kt) load_k(j + 2);
-        ok = bar_wait(vfull(st), ph, abort_flag, 0xA40u | st);
-        // P V_{j-1} complete: its V stage is free
-        if (ok && j > 0) ok = bar_wait(bar_o, (uint32_t)((j - 1) & 1), abort_flag, 0xA50u);
-        if (!ok) break;
-        if (j >= 1 && j + 1 < n_kt) load_v(j + 1);
         fence_after();
-        {
-          const uint64_t db = desc_n_major(sV(st));
-          const uint32_t ta = tmem + 192u + 32u * (uint32_t)st;      // P_j: 16 contraction steps = 8 columns
+        issue_s(j + 1);
+      }
+      // P_j written (into P buffer j & 1): S_j has been read, so its K stage is free
+      ok = wait(bar_p, (uint32_t)(j & 1), 0xA30u);
+      if (!ok) break;
+      if (j + 2 < n_kt) load_k(j + 2);
+      ok = wait(vfull(st), ph, 0xA40u | st);
+      // P V_{j-1} complete: its V stage is free
+      if (ok && j > 0) ok = wait(bar_o, (uint32_t)((j - 1) & 1), 0xA50u);
+      if (!ok) break;
+      if (j >= 1 && j + 1 < n_kt) load_v(j + 1);
+      fence_after();
+      const uint64_t db = desc_n_major(sV(st));
+      const uint32_t ta = tmem + 192u + 32u * (uint32_t)st;          // P_j: 16 contraction steps = 8 columns
+      if (faar_elect_one()) {
 #pragma unroll
-          for (int k = 0; k < KT / 16; ++k) mma_ts(tmem + 128u, ta + 8u * k, db + 128u * k, id_pv, (j | k) != 0 ? 1u : 0u);
-        }
+        for (int k = 0; k < KT / 16; ++k) mma_ts(tmem + 128u, ta + 8u * k, db + 128u * k, id_pv, (j | k) != 0 ? 1u : 0u);
         commit(bar_o);
       }
-      if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }   // copies in flight
+      __syncwarp();
     }
+    if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }   // copies in flight
   } else {
     // ---------------- softmax: thread = query row = tensor-memory lane ----------------
     const int row = 32 * warp + lane;
@@ -459,56 +474,67 @@ attn_dq64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   auto sV = [&](int s) { return sK(s) + KV_BYTES; };
 
   if (warp == 8) {
-    if (lane == 0) {
-      auto load_kv = [&](int j) {
-        const int st = j % DQ_STAGES;
+    const bool lead = lane == 0;
+    auto wait = [&](uint32_t bar, uint32_t parity, uint32_t code) {
+      return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
+    };
+    auto load_kv = [&](int j) {
+      const int st = j % DQ_STAGES;
+      if (lead) {
         bar_expect(kvfull(st), 2 * KV_BYTES);
         tma_2d(sK(st), &tmK, g * HD, (int)(seq0 + (long long)j * KT), kvfull(st));
         tma_2d(sV(st), &tmV, g * HD, (int)(seq0 + (long long)j * KT), kvfull(st));
-      };
+      }
+      __syncwarp();
+    };
+    if (lead) {
       bar_expect(bar_qd, 2 * Q_BYTES);
       tma_2d(sQ, &tmQ, h * HD, (int)(seq0 + q0), bar_qd);
       tma_2d(sDO, &tmDO, h * HD, (int)(seq0 + q0), bar_qd);
-      load_kv(0);
-      if (n_kt > 1) load_kv(1);
-      bool ok = bar_wait(bar_qd, 0u, abort_flag, 0xC01u);
-      const uint32_t id_k = idesc(0), id_n = idesc(1);
-      auto issue_dq = [&](int j) {                            // dQ += dS_j K_j
-        const uint64_t db = desc_n_major(sK(j % DQ_STAGES));
+    }
+    load_kv(0);
+    if (n_kt > 1) load_kv(1);
+    bool ok = wait(bar_qd, 0u, 0xC01u);
+    const uint32_t id_k = idesc(0), id_n = idesc(1);
+    auto issue_dq = [&](int j) {                              // dQ += dS_j K_j
+      const uint64_t db = desc_n_major(sK(j % DQ_STAGES));
+      if (faar_elect_one()) {
 #pragma unroll
         for (int k = 0; k < KT / 16; ++k) mma_ts(tmem + 128u, tmem + 192u + 8u * k, db + 128u * k, id_n, (j | k) != 0 ? 1u : 0u);
         commit(bar_done);
-      };
-      for (int j = 0; j < n_kt && ok; ++j) {
-        const int st = j % DQ_STAGES;
-        if (j >= 1 && j + 1 < n_kt) {                         // stage of tile j + 1 last held tile j - 2
-          if (j >= 2) ok = bar_wait(bar_done, (uint32_t)((j - 2) & 1), abort_flag, 0xC10u);
-          if (!ok) break;
-          load_kv(j + 1);
-        }
-        ok = bar_wait(kvfull(st), (uint32_t)((j / DQ_STAGES) & 1), abort_flag, 0xC20u | st);
-        if (ok && j > 0) ok = bar_wait(bar_sfree, (uint32_t)((j - 1) & 1), abort_flag, 0xC30u);
+      }
+      __syncwarp();
+    };
+    for (int j = 0; j < n_kt && ok; ++j) {
+      const int st = j % DQ_STAGES;
+      if (j >= 1 && j + 1 < n_kt) {                           // stage of tile j + 1 last held tile j - 2
+        if (j >= 2) ok = wait(bar_done, (uint32_t)((j - 2) & 1), 0xC10u);
+        if (!ok) break;
+        load_kv(j + 1);
+      }
+      ok = wait(kvfull(st), (uint32_t)((j / DQ_STAGES) & 1), 0xC20u | st);
+      if (ok && j > 0) ok = wait(bar_sfree, (uint32_t)((j - 1) & 1), 0xC30u);
+      if (!ok) break;
+      fence_after();
+      const uint64_t dq_ = desc_k_major(sQ), dk_ = desc_k_major(sK(st)), dd = desc_k_major(sDO), dv_ = desc_k_major(sV(st));
+      if (faar_elect_one()) {
+#pragma unroll
+        for (int k = 0; k < HD / 16; ++k) mma(tmem, dq_ + 2u * k, dk_ + 2u * k, id_k, k != 0 ? 1u : 0u);
+#pragma unroll
+        for (int k = 0; k < HD / 16; ++k) mma(tmem + 64u, dd + 2u * k, dv_ + 2u * k, id_k, k != 0 ? 1u : 0u);
+        commit(bar_s);
+      }
+      __syncwarp();
+      if (j > 0) {
+        ok = wait(bar_ds, (uint32_t)((j - 1) & 1), 0xC40u);
         if (!ok) break;
         fence_after();
-        {
-          const uint64_t dq_ = desc_k_major(sQ), dk_ = desc_k_major(sK(st)), dd = desc_k_major(sDO), dv_ = desc_k_major(sV(st));
-#pragma unroll
-          for (int k = 0; k < HD / 16; ++k) mma(tmem, dq_ + 2u * k, dk_ + 2u * k, id_k, k != 0 ? 1u : 0u);
-#pragma unroll
-          for (int k = 0; k < HD / 16; ++k) mma(tmem + 64u, dd + 2u * k, dv_ + 2u * k, id_k, k != 0 ? 1u : 0u);
-        }
-        commit(bar_s);
-        if (j > 0) {
-          ok = bar_wait(bar_ds, (uint32_t)((j - 1) & 1), abort_flag, 0xC40u);
-          if (!ok) break;
-          fence_after();
-          issue_dq(j - 1);
-        }
+        issue_dq(j - 1);
       }
-      if (ok) ok = bar_wait(bar_ds, (uint32_t)((n_kt - 1) & 1), abort_flag, 0xC50u);
-      if (ok) { fence_after(); issue_dq(n_kt - 1); }
-      if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
     }
+    if (ok) ok = wait(bar_ds, (uint32_t)((n_kt - 1) & 1), 0xC50u);
+    if (ok) { fence_after(); issue_dq(n_kt - 1); }
+    if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
   } else {
     const int row = 32 * (warp & 3) + lane, half = warp >> 2;    // this thread: columns 32 half .. 32 half + 31 of its row
     const int qi = q0 + row;
@@ -660,65 +686,76 @@ attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   auto q0_of = [&](int i) { return (qt0 + i % per_head) * KT; };
 
   if (warp == 8) {
-    if (lane == 0) {
-      auto load_item = [&](int i) {
-        const int st = i % KV_STAGES;
+    const bool lead = lane == 0;
+    auto wait = [&](uint32_t bar, uint32_t parity, uint32_t code) {
+      return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
+    };
+    auto load_item = [&](int i) {
+      const int st = i % KV_STAGES;
+      if (lead) {
         bar_expect(qfull(st), 2 * KV_BYTES);
         tma_2d(sQ(st), &tmQ, head_of(i) * HD, (int)(seq0 + q0_of(i)), qfull(st));
         tma_2d(sDO(st), &tmDO, head_of(i) * HD, (int)(seq0 + q0_of(i)), qfull(st));
-      };
+      }
+      __syncwarp();
+    };
+    if (lead) {
       bar_expect(bar_kv, 2 * Q_BYTES);
       tma_2d(sKt, &tmK, g * HD, (int)(seq0 + k0), bar_kv);
       tma_2d(sVt, &tmV, g * HD, (int)(seq0 + k0), bar_kv);
-      load_item(0);
-      if (n_it > 1) load_item(1);
-      if (n_it > 2) load_item(2);
-      bool ok = bar_wait(bar_kv, 0u, abort_flag, 0xE01u);
-      const uint32_t id_k = idesc(0), id_n = idesc(1);
-      auto issue_s = [&](int i) {                              // S^T and dP^T of item i
-        const int st = i % KV_STAGES;
-        const uint64_t dk_ = desc_k_major(sKt), dq_ = desc_k_major(sQ(st)), dv_ = desc_k_major(sVt), dd = desc_k_major(sDO(st));
+    }
+    load_item(0);
+    if (n_it > 1) load_item(1);
+    if (n_it > 2) load_item(2);
+    bool ok = wait(bar_kv, 0u, 0xE01u);
+    const uint32_t id_k = idesc(0), id_n = idesc(1);
+    auto issue_s = [&](int i) {                                // S^T and dP^T of item i
+      const int st = i % KV_STAGES;
+      const uint64_t dk_ = desc_k_major(sKt), dq_ = desc_k_major(sQ(st)), dv_ = desc_k_major(sVt), dd = desc_k_major(sDO(st));
+      if (faar_elect_one()) {
 #pragma unroll
         for (int k = 0; k < HD / 16; ++k) mma(tmem, dk_ + 2u * k, dq_ + 2u * k, id_k, k != 0 ? 1u : 0u);
 #pragma unroll
         for (int k = 0; k < HD / 16; ++k) mma(tmem + 64u, dv_ + 2u * k, dd + 2u * k, id_k, k != 0 ? 1u : 0u);
         commit(bar_s(i & 1));
-      };
-      if (ok) ok = bar_wait(qfull(0), 0u, abort_flag, 0xE10u);
-      if (ok) { fence_after(); issue_s(0); }
-      for (int i = 0; i < n_it && ok; ++i) {
-        if (i + 3 < n_it) {                                    // its stage last held item i - 1: wait for that item's
-          if (i >= 1) ok = bar_wait(bar_done((i - 1) & 1), (uint32_t)(((i - 1) >> 1) & 1), abort_flag, 0xE40u);   // MMAs
-          if (!ok) break;
-          load_item(i + 3);
-        }
-        ok = bar_wait(bar_pds(i & 1), (uint32_t)((i >> 1) & 1), abort_flag, 0xE30u);
+      }
+      __syncwarp();
+    };
+    if (ok) ok = wait(qfull(0), 0u, 0xE10u);
+    if (ok) { fence_after(); issue_s(0); }
+    for (int i = 0; i < n_it && ok; ++i) {
+      if (i + 3 < n_it) {                                      // its stage last held item i - 1: wait for that item's
+        if (i >= 1) ok = wait(bar_done((i - 1) & 1), (uint32_t)(((i - 1) >> 1) & 1), 0xE40u);   // MMAs
+        if (!ok) break;
+        load_item(i + 3);
+      }
+      ok = wait(bar_pds(i & 1), (uint32_t)((i >> 1) & 1), 0xE30u);
+      if (!ok) break;
+      fence_after();
+      // A operands from tensor memory: contraction steps 0, 1 (queries 0..31) in columns 0..15 of the buffer,
+      // steps 2, 3 (queries 32..63) in columns 32..47
+      const int st = i % KV_STAGES;
+      const uint64_t dd = desc_n_major(sDO(st)), dq_ = desc_n_major(sQ(st));
+      if (faar_elect_one()) {
+#pragma unroll
+        for (int k = 0; k < KT / 16; ++k)
+          mma_ts(tmem + 128u, tmem + (uint32_t)(32 * (k >> 1) + 8 * (k & 1)), dd + 128u * k, id_n, (i | k) != 0 ? 1u : 0u);
+#pragma unroll
+        for (int k = 0; k < KT / 16; ++k)
+          mma_ts(tmem + 192u, tmem + 64u + (uint32_t)(32 * (k >> 1) + 8 * (k & 1)), dq_ + 128u * k, id_n, (i | k) != 0 ? 1u : 0u);
+        commit(bar_done(i & 1));
+      }
+      __syncwarp();
+      if (i + 1 < n_it) {
+        // the next item's score products overwrite P^T / dS^T: after the accumulating products have read them
+        ok = wait(qfull((i + 1) % KV_STAGES), (uint32_t)(((i + 1) / KV_STAGES) & 1), 0xE10u);
+        if (ok) ok = wait(bar_done(i & 1), (uint32_t)((i >> 1) & 1), 0xE20u);
         if (!ok) break;
         fence_after();
-        {
-          // A operands from tensor memory: contraction steps 0, 1 (queries 0..31) in columns 0..15 of the buffer,
-          // steps 2, 3 (queries 32..63) in columns 32..47
-          const int st = i % KV_STAGES;
-          const uint64_t dd = desc_n_major(sDO(st)), dq_ = desc_n_major(sQ(st));
-#pragma unroll
-          for (int k = 0; k < KT / 16; ++k)
-            mma_ts(tmem + 128u, tmem + (uint32_t)(32 * (k >> 1) + 8 * (k & 1)), dd + 128u * k, id_n, (i | k) != 0 ? 1u : 0u);
-#pragma unroll
-          for (int k = 0; k < KT / 16; ++k)
-            mma_ts(tmem + 192u, tmem + 64u + (uint32_t)(32 * (k >> 1) + 8 * (k & 1)), dq_ + 128u * k, id_n, (i | k) != 0 ? 1u : 0u);
-        }
-        commit(bar_done(i & 1));
-        if (i + 1 < n_it) {
-          // the next item's score products overwrite P^T / dS^T: after the accumulating products have read them
-          ok = bar_wait(qfull((i + 1) % KV_STAGES), (uint32_t)(((i + 1) / KV_STAGES) & 1), abort_flag, 0xE10u);
-          if (ok) ok = bar_wait(bar_done(i & 1), (uint32_t)((i >> 1) & 1), abort_flag, 0xE20u);
-          if (!ok) break;
-          fence_after();
-          issue_s(i + 1);
-        }
+        issue_s(i + 1);
       }
-      if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
     }
+    if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
   } else {
     const int row = 32 * (warp & 3) + lane, half = warp >> 2;    // this thread: queries 32 half .. 32 half + 31 of an item
     const int kj = k0 + row;
