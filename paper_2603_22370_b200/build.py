@@ -5,12 +5,14 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfaar.so")
 LIB_DEBUG = os.path.join(HERE, "libfaar_debug.so")     # -DFAAR_DEBUG: epilogue stores checked against tensor extents
+BINDING = os.path.join(HERE, "_faarbind.so")           # native argument marshalling, for this interpreter
 SOURCES = ["faar_api.cu", "faar_elementwise.cu", "faar_gemm.cu", "faar_static_scratch.cu", "faar_align.cu", "faar_glue.cu", "faar_fp4_gemm.cu", "faar_attention.cu", "faar_attention_tc.cu"]
 
 
@@ -25,8 +27,19 @@ def needs_build(lib: str = LIB) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "faar.h")]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != "faar_binding.cpp"] + [os.path.join(ROOT, "include", "faar.h")]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _build_binding(force: bool = False):
+    src, header = os.path.join(CSRC, "faar_binding.cpp"), os.path.join(ROOT, "include", "faar.h")
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= max(os.path.getmtime(src), os.path.getmtime(header)):
+        return
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I",
+           sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"), src, "-o", BINDING, "-ldl"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
 
 
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
@@ -35,6 +48,7 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     writes (a store that would leave it is skipped and reported through the workspace status word).  The
     binding loads it when FAAR_LIB names it."""
     lib = LIB_DEBUG if debug else LIB
+    _build_binding(force)
     if not force and not needs_build(lib):
         return lib
     cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -1,6 +1,7 @@
 // extern "C" entry points of libfaar.so: argument validation, workspace carving,
 // kernel sequencing.  No device memory is allocated here.
 #include <math.h>
+#include <atomic>
 #include <initializer_list>
 #include <new>
 
@@ -202,6 +203,28 @@ faar_prof_scope::faar_prof_scope(faar_ctx* ctx, int kernel_id) : c(ctx), pair(-1
   pair = i;
 }
 
+int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes) {
+  for (const void* k : c->smem_set)
+    if (k == kernel) return 0;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) c->smem_set.push_back(kernel);
+  return (int)e;
+}
+
+int faar_max_pairs(faar_ctx* c, int slot, const void* kernel, cudaLaunchConfig_t* cfg) {
+  constexpr int DEVICES = 64;
+  static std::atomic<int> known[DEVICES][FAAR_PAIR_KERNELS];       // 0 = not asked yet
+  const bool keep = c->device < DEVICES;
+  int n = keep ? known[c->device][slot].load(std::memory_order_relaxed) : 0;
+  if (n) return n;
+  cfg->gridDim = dim3(2 * (c->num_sms / 2), 1, 1);
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kernel, cfg);
+  if (e != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = c->num_sms / 2; }
+  if (n > c->num_sms / 2) n = c->num_sms / 2;
+  if (keep) known[c->device][slot].store(n, std::memory_order_relaxed);
+  return n;
+}
+
 faar_prof_scope::~faar_prof_scope() {
   if (pair >= 0) cudaEventRecord(c->prof_events[2 * pair + 1], c->stream);
 }
@@ -264,8 +287,6 @@ int faar_create(faar_ctx** out, int device, void* stream) {
   c->tune_attention_fragments = 0;
   c->tune_wide = -1;
   c->last_gemm_split = 0;
-  for (int i = 0; i < FAAR_GEMM_VARIANTS; ++i) c->gemm_max_pairs[i] = 0;
-  c->fp4_max_pairs[0] = c->fp4_max_pairs[1] = 0;
   c->wsoft_ws = nullptr;
   c->wsoft_beta = 0.f;
   c->copy_stream = nullptr;

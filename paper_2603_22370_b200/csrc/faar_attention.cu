@@ -838,12 +838,12 @@ template <int D> constexpr int dq_smem() { return 4 * AT * (D + 8) * 2 + 2 * 4 *
 
 template <int D>
 int launch_fwd(faar_ctx* ctx, const AttnParams& p) {
-  cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd_smem<D>());
-  if (e != cudaSuccess) return (int)e;
+  int e = faar_allow_smem(ctx, (const void*)attn_fwd_kernel<D>, fwd_smem<D>());
+  if (e) return e;
   dim3 grid((p.S + AT - 1) / AT, p.H, p.B);
   if (D == HD && ctx->tune_attention_fragments != 1) {
-    e = cudaFuncSetAttribute(attn_fwd64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FWD64_SMEM);
-    if (e != cudaSuccess) return (int)e;
+    e = faar_allow_smem(ctx, (const void*)attn_fwd64_kernel, FWD64_SMEM);
+    if (e) return e;
   }
   faar_prof_scope ps(ctx, FAAR_K_ATTENTION);
   if (D == HD && ctx->tune_attention_fragments == 0)
@@ -858,11 +858,11 @@ int launch_fwd(faar_ctx* ctx, const AttnParams& p) {
 
 template <int D>
 int launch_bwd(faar_ctx* ctx, const AttnParams& p, float* dsum) {
-  cudaError_t e = cudaFuncSetAttribute(attn_dkv_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, dkv_smem<D>());
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_dq_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, dq_smem<D>());
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_dkv64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD64_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(attn_dq64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD64_SMEM);
-  if (e != cudaSuccess) return (int)e;
+  int e = faar_allow_smem(ctx, (const void*)attn_dkv_kernel<D>, dkv_smem<D>());
+  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_kernel<D>, dq_smem<D>());
+  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dkv64_kernel, BWD64_SMEM);
+  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq64_kernel, BWD64_SMEM);
+  if (e) return e;
   faar_prof_scope ps(ctx, FAAR_K_ATTENTION);
   long long rows = (long long)p.B * p.H * ((p.S + 256 / D - 1) / (256 / D));      // warp passes of the row-sum kernel
   long long blocks = (rows + 3) / 4;

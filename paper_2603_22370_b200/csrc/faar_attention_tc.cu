@@ -885,8 +885,7 @@ int faar_launch_attention_fwd64_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, 
   if (!e) e = head_map(ctx, &tmK, k, T, Hkv * HD, ldk, KT);
   if (!e) e = head_map(ctx, &tmV, v, T, Hkv * HD, ldk, KT);
   if (e) return e;
-  cudaError_t ce = cudaFuncSetAttribute(attn_fwd64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-  if (ce != cudaSuccess) return (int)ce;
+  if ((e = faar_allow_smem(ctx, (const void*)attn_fwd64_tc_kernel, SMEM))) return e;
   TcParams p;
   p.out = reinterpret_cast<__nv_bfloat16*>(out); p.lse = lse; p.ldo = ldo; p.B = B; p.S = S; p.H = H; p.Hkv = Hkv;
   p.scale_log2 = scale_log2;
@@ -906,8 +905,7 @@ int faar_launch_attention_dq64_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, c
   if (!e) e = head_map(ctx, &tmK, k, T, Hkv * HD, ldk, KT);
   if (!e) e = head_map(ctx, &tmV, v, T, Hkv * HD, ldk, KT);
   if (e) return e;
-  cudaError_t ce = cudaFuncSetAttribute(attn_dq64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DQ_SMEM);
-  if (ce != cudaSuccess) return (int)ce;
+  if ((e = faar_allow_smem(ctx, (const void*)attn_dq64_tc_kernel, DQ_SMEM))) return e;
   TcBwdParams p = {};
   p.lse = lse; p.dsum = dsum; p.dq = reinterpret_cast<__nv_bfloat16*>(dq); p.ldq = ldq; p.ldk = ldk;
   p.B = B; p.S = S; p.H = H; p.Hkv = Hkv; p.scale_log2 = scale_log2; p.inv_sqrt_d = scale_log2 / 1.4426950408889634f;
@@ -927,8 +925,7 @@ int faar_launch_attention_dkv64_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, 
   if (!e) e = head_map(ctx, &tmK, k, T, Hkv * HD, ldk, QT);
   if (!e) e = head_map(ctx, &tmV, v, T, Hkv * HD, ldk, QT);
   if (e) return e;
-  cudaError_t ce = cudaFuncSetAttribute(attn_dkv64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, KV_SMEM);
-  if (ce != cudaSuccess) return (int)ce;
+  if ((e = faar_allow_smem(ctx, (const void*)attn_dkv64_tc_kernel, KV_SMEM))) return e;
   TcBwdParams p = {};
   p.lse = lse; p.dsum = dsum; p.dk = reinterpret_cast<__nv_bfloat16*>(dk); p.dv = reinterpret_cast<__nv_bfloat16*>(dv);
   p.ldq = ldq; p.ldk = ldk; p.B = B; p.S = S; p.H = H; p.Hkv = Hkv; p.scale_log2 = scale_log2;

@@ -389,18 +389,11 @@ int launch4(faar_ctx* ctx, const uint8_t* A, const uint8_t* sfa, const uint8_t* 
   cfg.stream = ctx->stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  int& max_pairs = ctx->fp4_max_pairs[BN == 256];
-  if (max_pairs == 0) {            // how many CTA pairs the device can hold at once, asked once per context
-    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C4::SMEM);
-    if (ce != cudaSuccess) return (int)ce;
-    cfg.gridDim = dim3(2 * (ctx->num_sms / 2), 1, 1);
-    int n = 0;
-    ce = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-    if (ce != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = ctx->num_sms / 2; }
-    max_pairs = n < ctx->num_sms / 2 ? n : ctx->num_sms / 2;
-  }
+  int e = faar_allow_smem(ctx, (const void*)kern, C4::SMEM);
+  if (e) return e;
+  const int max_pairs = faar_max_pairs(ctx, FAAR_GEMM_VARIANTS + (BN == 256), (const void*)kern, &cfg);
   CUtensorMap tmA, tmB, tmSA, tmSB;
-  int e = byte_map(ctx, &tmA, A, p.M, p.K, TM);
+  e = byte_map(ctx, &tmA, A, p.M, p.K, TM);
   if (!e) e = byte_map(ctx, &tmB, B, p.N, p.K, BN / 2);
   if (!e) e = scale_map(ctx, &tmSA, sfa, (p.M + 127) / 128, p.k_tiles, 1);
   if (!e) e = scale_map(ctx, &tmSB, sfb, (p.N + 127) / 128, p.k_tiles, C4::N_SFB);

@@ -1007,11 +1007,13 @@ int pick_full_cols(const faar_ctx* ctx, int M, int N, int bn, int pairs) {
     const int rest = N - full_cols * bn;
     const long long half_tiles = rest > 0 ? (long long)m_tiles * ((rest + bn / 2 - 1) / (bn / 2)) : 0;
     const long long total = full_tiles + half_tiles;
+    // a pair's load depends on how many full and how many half tiles it gets, which change only at two pair numbers
     double worst = 0.0;
-    for (int p = 0; p < pairs && p < total; ++p) {
-      double load = 0.0, last = 0.0;
-      for (long long t = p; t < total; t += pairs) { last = t < full_tiles ? 1.0 : 0.75; load += last; }
-      load += 0.4 * last;
+    const long long cand[3] = {0, full_tiles % pairs, total % pairs};
+    for (long long p : cand) {
+      if (p >= total) continue;
+      const long long nt = (total - p + pairs - 1) / pairs, nf = full_tiles > p ? (full_tiles - p + pairs - 1) / pairs : 0;
+      const double last = nt > nf ? 0.75 : 1.0, load = nf + 0.75 * (nt - nf) + 0.4 * last;
       if (load > worst) worst = load;
     }
     if (best < 0.0 || worst < best - 1e-9) { best = worst; best_full = full_cols; }
@@ -1037,8 +1039,8 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   static_assert(C::SMEM_BYTES <= SMEM_LIMIT, "shared memory budget");
   static_assert(C::EPI_WARPS <= MAX_EPI_WARPS, "partials budget");
   auto kern = faar_gemm_kernel<MODE, OPT, WIDE, MN>;
-  cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
-  if (ce != cudaSuccess) return (int)ce;
+  int e = faar_allow_smem(ctx, (const void*)kern, C::SMEM_BYTES);
+  if (e) return e;
   cudaLaunchConfig_t cfg = base_cfg;
   cfg.dynamicSmemBytes = C::SMEM_BYTES;
   kp.bn = bn;
@@ -1046,7 +1048,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   if (a->b_mn && bn != BN_MAX) kp.n_full_cols = (a->N + bn - 1) / bn;      // half tiles of a 128-wide tile would be 32 columns per CTA
   CUtensorMap tmA, tmB, tmBh;
   kp.a_mn = a->a_mn; kp.b_mn = a->b_mn;
-  int e = a->a_mn ? make_map_mn(ctx, &tmA, a->A, a->Kc, a->M, a->lda) : make_map(ctx, &tmA, a->A, a->M, a->Kc, a->lda, BM);
+  e = a->a_mn ? make_map_mn(ctx, &tmA, a->A, a->Kc, a->M, a->lda) : make_map(ctx, &tmA, a->A, a->M, a->Kc, a->lda, BM);
   if (e) return e;
   if (a->b_mn) {
     e = make_map_mn(ctx, &tmB, a->B, a->Kc, a->N, a->ldb);    // one map serves full and half-width tiles
@@ -1054,7 +1056,8 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   } else {
     e = make_map(ctx, &tmB, a->B, a->N, a->Kc, a->ldb, bn / 2);
     if (e) return e;
-    e = make_map(ctx, &tmBh, a->B, a->N, a->Kc, a->ldb, bn % 32 == 0 ? bn / 4 : bn / 2);   // half-width tiles
+    if (kp.n_full_cols * bn < a->N) e = make_map(ctx, &tmBh, a->B, a->N, a->Kc, a->ldb, bn % 32 == 0 ? bn / 4 : bn / 2);   // half-width tiles
+    else tmBh = tmB;
   }
   if (e) return e;
   const long long m_tiles = (a->M + 2 * BM - 1) / (2 * BM);
@@ -1068,7 +1071,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   ctx->last_gemm_pairs = pairs;
   ctx->last_gemm_split = WIDE ? 0 : (a->N + bn - 1) / bn - kp.n_full_cols;
   faar_prof_scope ps(ctx, MODE == FAAR_GEMM_REF ? FAAR_K_GEMM_REF : (MODE == FAAR_GEMM_FWD ? FAAR_K_GEMM_FWD : FAAR_K_GEMM_BWD));
-  ce = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmBh, kp);
+  cudaError_t ce = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmBh, kp);
   if (ce != cudaSuccess) return (int)ce;
   return (int)cudaGetLastError();
 }
@@ -1089,20 +1092,10 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
   cfg.stream = ctx->stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  // how many CTA pairs the device can hold at once (a GPC with an odd SM count strands one SM); asked once
-  // per context and kernel mode, with the context's device current (every variant takes one CTA per SM)
-  int& max_pairs = ctx->gemm_max_pairs[MODE == FAAR_GEMM_BWD ? 2 + OPT : MODE];
-  if (max_pairs == 0) {
-    auto kern = faar_gemm_kernel<MODE, OPT, false, 0>;
-    cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
-    if (ce != cudaSuccess) return (int)ce;
-    cfg.gridDim = dim3(2 * (ctx->num_sms / 2), 1, 1);
-    int n = 0;
-    ce = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-    if (ce != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = ctx->num_sms / 2; }
-    if (n > ctx->num_sms / 2) n = ctx->num_sms / 2;
-    max_pairs = n;
-  }
+  auto kern = faar_gemm_kernel<MODE, OPT, false, 0>;               // every variant takes one CTA per SM
+  const int e = faar_allow_smem(ctx, (const void*)kern, C::SMEM_BYTES);
+  if (e) return e;
+  const int max_pairs = faar_max_pairs(ctx, MODE == FAAR_GEMM_BWD ? 2 + OPT : MODE, (const void*)kern, &cfg);
   const int bn = pick_bn(ctx, MODE, a->M, a->N, max_pairs, a->b_mn != 0);
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
   // which operand layouts a mode is ever launched with: the plain product with A untransposed (input gradient),

@@ -10,6 +10,7 @@
 #include <vector>
 
 constexpr int FAAR_GEMM_VARIANTS = 8;     // REF, FWD, BWD x 4 optimiser / chaining variants
+constexpr int FAAR_PAIR_KERNELS = FAAR_GEMM_VARIANTS + 2;   // and the NVFP4 GEMM's 128- and 256-wide tiles
 
 struct faar_ctx {
   int device;
@@ -22,9 +23,7 @@ struct faar_ctx {
   int tune_wide;                          // 1 = 256 x 512 GEMM tiles wherever the shape allows; -1 (default), 0 = never
   int tune_attention_fragments;           // head_dim 64 attention: 0 = tcgen05 kernels, 2 = mma.sync kernels, 1 = the shared-memory fragment kernels
   int last_gemm_bn, last_gemm_pairs, last_gemm_split;   // what the last GEMM launch used
-  // CTA pairs this context's device can hold at once, per GEMM kernel instantiation (0 = not asked yet)
-  int gemm_max_pairs[FAAR_GEMM_VARIANTS];
-  int fp4_max_pairs[2];                   // the same for the NVFP4 GEMM's 128- and 256-wide tiles
+  std::vector<const void*> smem_set;      // kernels whose dynamic shared-memory limit has been raised on this device
   // chained steps: the workspace and the beta of the forward operand that the last backward call wrote
   const void* wsoft_ws;
   float wsoft_beta;
@@ -47,6 +46,13 @@ struct faar_prof_scope {
   faar_prof_scope(faar_ctx* ctx, int kernel_id);
   ~faar_prof_scope();
 };
+
+// Raises a kernel's dynamic shared-memory limit, once per context (the call costs about as much host time as a launch's
+// argument checks and every launch of a small layer would pay it).  The context's device is current.
+int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes);
+// How many CTA pairs of `kernel` (launched as *cfg, a cluster of two, its grid ignored) the context's device holds at once:
+// a fact of device and kernel (a GPC with an odd SM count strands one SM), asked once per device and process.
+int faar_max_pairs(faar_ctx* c, int slot, const void* kernel, cudaLaunchConfig_t* cfg);
 
 // ---- workspace layout -------------------------------------------------------
 // [0, 256)            header: word 0 = status (0 = ok), word 2 = count of dW-GEMM

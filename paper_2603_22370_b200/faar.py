@@ -1,4 +1,5 @@
-"""ctypes binding of libfaar.so.  Argument marshalling only: every function
+"""Binding of libfaar.so (ctypes; the calls that enqueue work go through the native marshalling module
+_faarbind, which is several microseconds a call faster).  Argument marshalling only: every function
 below has the name and the arguments of the C entry point it calls; tensors
 are torch CUDA tensors whose `data_ptr()` is handed through.  There is no
 fallback: if the library is missing or a call fails, an exception is raised.
@@ -113,6 +114,23 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_native = None
+
+
+def _fast():
+    """The native marshalling module, bound to the same library as lib()."""
+    global _native
+    if _native is None:
+        lib()
+        try:
+            from . import _faarbind
+        except ImportError as e:
+            raise ImportError(f"{e}; run `python -m paper_2603_22370_b200.build`") from e
+        _faarbind.load(LIB_PATH)
+        _native = _faarbind
+    return _native
+
+
 def status_string(status: int) -> str:
     return lib().faar_status_string(int(status)).decode()
 
@@ -124,10 +142,6 @@ def _p(t):
         return C.c_void_p(t)
     assert t.is_cuda, "device tensors only"
     return C.c_void_p(t.data_ptr())
-
-
-def C_size(t) -> C.c_size_t:
-    return C.c_size_t(t.numel())
 
 
 def _check(status: int, where: str):
@@ -157,12 +171,14 @@ class Context:
         self.device = device
         s = stream.cuda_stream if stream is not None else torch.cuda.current_stream(device).cuda_stream
         _check(lib().faar_create(C.byref(self._h), device, C.c_void_p(s)), "faar_create")
+        self._n = self._h.value                     # the handle as the native marshalling takes it
         self.ws = None
 
     def close(self):
         if self._h:
             lib().faar_destroy(self._h)
             self._h = C.c_void_p(0)
+            self._n = None
 
     def __del__(self):
         try:
@@ -215,7 +231,7 @@ def workspace_size(shape: Shape) -> int:
 
 
 def workspace_init(ctx: Context, ws: torch.Tensor):
-    _check(lib().faar_workspace_init(ctx._h, _p(ws), C.c_size_t(ws.numel())), "faar_workspace_init")
+    _check(_fast().faar_workspace_init(ctx._n, ws, ws.numel()), "faar_workspace_init")
 
 
 def selftest_wait_timeout(ctx: Context, ws: torch.Tensor, limit_us: int = 1000):
@@ -232,25 +248,23 @@ def check_status(ctx: Context, ws: torch.Tensor) -> int:
 
 
 def softquant_init(ctx, shape, W, s_global_in, scales, s_global_out, code, V_init, ws):
-    _check(lib().faar_softquant_init(ctx._h, C.byref(shape), _p(W), C.c_float(s_global_in), _p(scales),
-                                     _p(s_global_out), _p(code), _p(V_init), _p(ws), C.c_size_t(ws.numel())),
-           "faar_softquant_init")
+    _check(_fast().faar_softquant_init(ctx._n, shape, W, s_global_in, scales, s_global_out, code, V_init, ws,
+           ws.numel()), "faar_softquant_init")
 
 
 def softquant_eval(ctx, shape, V, code, scales, s_global, beta, W_soft, h, W_soft_bf16=None):
-    _check(lib().faar_softquant_eval(ctx._h, C.byref(shape), _p(V), _p(code), _p(scales), _p(s_global),
-                                     C.c_float(beta), _p(W_soft), _p(h), _p(W_soft_bf16)), "faar_softquant_eval")
+    _check(_fast().faar_softquant_eval(ctx._n, shape, V, code, scales, s_global, beta, W_soft, h, W_soft_bf16),
+           "faar_softquant_eval")
 
 
 def softquant_operand_f32(ctx, shape, V, code, scales, s_global, beta, W_operand):
-    _check(lib().faar_softquant_operand_f32(ctx._h, C.byref(shape), _p(V), _p(code), _p(scales), _p(s_global),
-                                            C.c_float(beta), _p(W_operand)), "faar_softquant_operand_f32")
+    _check(_fast().faar_softquant_operand_f32(ctx._n, shape, V, code, scales, s_global, beta, W_operand),
+           "faar_softquant_operand_f32")
 
 
 def act_fakequant(ctx, T, K, X, ldx, s_global_in, Xq_units, ldq, s_global_out, packed, scales, ws):
-    _check(lib().faar_act_fakequant(ctx._h, T, K, _p(X), C.c_int64(ldx), C.c_float(s_global_in), _p(Xq_units),
-                                    C.c_int64(ldq), _p(s_global_out), _p(packed), _p(scales), _p(ws),
-                                    C.c_size_t(ws.numel())), "faar_act_fakequant")
+    _check(_fast().faar_act_fakequant(ctx._n, T, K, X, ldx, s_global_in, Xq_units, ldq, s_global_out, packed, scales,
+           ws, ws.numel()), "faar_act_fakequant")
 
 
 def align_loss_workspace_size(T, vocab) -> int:
@@ -260,56 +274,52 @@ def align_loss_workspace_size(T, vocab) -> int:
 
 
 def align_loss(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, dZ_q, dH_q, loss_out2, ws):
-    _check(lib().faar_align_loss(ctx._h, T, vocab, hidden, _p(Z_fp), _p(Z_q), C.c_int64(ldz), _p(H_fp), _p(H_q),
-                                 C.c_int64(ldh), C.c_float(tau), C.c_float(lambda_kl), _p(dZ_q), _p(dH_q), _p(loss_out2),
-                                 _p(ws), C.c_size_t(ws.numel())), "faar_align_loss")
+    _check(_fast().faar_align_loss(ctx._n, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, dZ_q,
+           dH_q, loss_out2, ws, ws.numel()), "faar_align_loss")
 
 
 def swizzle_scales(ctx, rows, cols, scales, scales_tiled):
-    _check(lib().faar_swizzle_scales(ctx._h, rows, cols, _p(scales), _p(scales_tiled), C.c_size_t(scales_tiled.numel())),
+    _check(_fast().faar_swizzle_scales(ctx._n, rows, cols, scales, scales_tiled, scales_tiled.numel()),
            "faar_swizzle_scales")
 
 
 def silu_mul(ctx, rows, cols, gate, ldg, up, ldu, out, ldo):
-    _check(lib().faar_silu_mul(ctx._h, rows, cols, _p(gate), ldg, _p(up), ldu, _p(out), ldo), "faar_silu_mul")
+    _check(_fast().faar_silu_mul(ctx._n, rows, cols, gate, ldg, up, ldu, out, ldo), "faar_silu_mul")
 
 
 def rmsnorm(ctx, rows, cols, x, ldx, g, eps, y, ldy, rstd=None):
-    _check(lib().faar_rmsnorm(ctx._h, rows, cols, _p(x), ldx, _p(g), eps, _p(y), ldy, _p(rstd)), "faar_rmsnorm")
+    _check(_fast().faar_rmsnorm(ctx._n, rows, cols, x, ldx, g, eps, y, ldy, rstd), "faar_rmsnorm")
 
 
 def rmsnorm_bwd(ctx, rows, cols, dy, lddy, x, ldx, g, rstd, add, ldadd, dx, lddx):
-    _check(lib().faar_rmsnorm_bwd(ctx._h, rows, cols, _p(dy), lddy, _p(x), ldx, _p(g), _p(rstd), _p(add), ldadd, _p(dx), lddx),
-           "faar_rmsnorm_bwd")
+    _check(_fast().faar_rmsnorm_bwd(ctx._n, rows, cols, dy, lddy, x, ldx, g, rstd, add, ldadd, dx, lddx), "faar_rmsnorm_bwd")
 
 
 def add_rmsnorm(ctx, rows, cols, a, lda, b, ldb, total, lds, g, eps, y, ldy, rstd=None):
-    _check(lib().faar_add_rmsnorm(ctx._h, rows, cols, _p(a), C.c_int64(lda), _p(b), C.c_int64(ldb), _p(total), C.c_int64(lds),
-                                  _p(g), C.c_float(eps), _p(y), C.c_int64(ldy), _p(rstd)), "faar_add_rmsnorm")
+    _check(_fast().faar_add_rmsnorm(ctx._n, rows, cols, a, lda, b, ldb, total, lds, g, eps, y, ldy, rstd),
+           "faar_add_rmsnorm")
 
 
 def rmsnorm_bwd_sum(ctx, rows, cols, dy, dy2, dy3, lddy, x, ldx, g, rstd, add, ldadd, dx, lddx):
-    _check(lib().faar_rmsnorm_bwd_sum(ctx._h, rows, cols, _p(dy), _p(dy2), _p(dy3), C.c_int64(lddy), _p(x), C.c_int64(ldx),
-                                      _p(g), _p(rstd), _p(add), C.c_int64(ldadd), _p(dx), C.c_int64(lddx)),
-           "faar_rmsnorm_bwd_sum")
+    _check(_fast().faar_rmsnorm_bwd_sum(ctx._n, rows, cols, dy, dy2, dy3, lddy, x, ldx, g, rstd, add, ldadd, dx,
+           lddx), "faar_rmsnorm_bwd_sum")
 
 
 def rope(ctx, rows, n_heads, head_dim, x, ldx, positions, theta, inverse, y, ldy):
-    _check(lib().faar_rope(ctx._h, rows, n_heads, head_dim, _p(x), ldx, _p(positions), theta, int(inverse), _p(y), ldy),
-           "faar_rope")
+    _check(_fast().faar_rope(ctx._n, rows, n_heads, head_dim, x, ldx, positions, theta, int(inverse), y, ldy), "faar_rope")
 
 
 def silu_mul_bwd(ctx, rows, cols, dout, ldd, gate, ldg, up, ldu, dgate, lddg, dup, lddu):
-    _check(lib().faar_silu_mul_bwd(ctx._h, rows, cols, _p(dout), ldd, _p(gate), ldg, _p(up), ldu, _p(dgate), lddg, _p(dup),
-                                   lddu), "faar_silu_mul_bwd")
+    _check(_fast().faar_silu_mul_bwd(ctx._n, rows, cols, dout, ldd, gate, ldg, up, ldu, dgate, lddg, dup, lddu),
+           "faar_silu_mul_bwd")
 
 
 def embedding(ctx, rows, cols, vocab, table, ldt, tokens, out, ldo):
-    _check(lib().faar_embedding(ctx._h, rows, cols, vocab, _p(table), ldt, _p(tokens), _p(out), ldo), "faar_embedding")
+    _check(_fast().faar_embedding(ctx._n, rows, cols, vocab, table, ldt, tokens, out, ldo), "faar_embedding")
 
 
 def add(ctx, rows, cols, a, lda, b, ldb, out, ldo):
-    _check(lib().faar_add(ctx._h, rows, cols, _p(a), lda, _p(b), ldb, _p(out), ldo), "faar_add")
+    _check(_fast().faar_add(ctx._n, rows, cols, a, lda, b, ldb, out, ldo), "faar_add")
 
 
 def tune_wide_tiles(ctx, mode: int):
@@ -330,55 +340,50 @@ def tune_attention(ctx, mode: int):
 
 
 def attention_fwd(ctx, batch, seq, n_heads, n_kv_heads, head_dim, q, ldq, k, v, ldkv, out, ldo, lse):
-    _check(lib().faar_attention_fwd(ctx._h, batch, seq, n_heads, n_kv_heads, head_dim, _p(q), ldq, _p(k), _p(v), ldkv,
-                                    _p(out), ldo, _p(lse)), "faar_attention_fwd")
+    _check(_fast().faar_attention_fwd(ctx._n, batch, seq, n_heads, n_kv_heads, head_dim, q, ldq, k, v, ldkv, out, ldo,
+           lse), "faar_attention_fwd")
 
 
 def attention_bwd(ctx, batch, seq, n_heads, n_kv_heads, head_dim, q, ldq, k, v, ldkv, out, dout, ldo, lse, dsum, dq, dk, dv):
-    _check(lib().faar_attention_bwd(ctx._h, batch, seq, n_heads, n_kv_heads, head_dim, _p(q), ldq, _p(k), _p(v), ldkv,
-                                    _p(out), _p(dout), ldo, _p(lse), _p(dsum), _p(dq), _p(dk), _p(dv)), "faar_attention_bwd")
+    _check(_fast().faar_attention_bwd(ctx._n, batch, seq, n_heads, n_kv_heads, head_dim, q, ldq, k, v, ldkv, out,
+           dout, ldo, lse, dsum, dq, dk, dv), "faar_attention_bwd")
 
 
 def nvfp4_gemm(ctx, M, N, K, A_packed, A_scales_tiled, A_s_global, B_packed, B_scales_tiled, B_s_global, C, ldc, ws):
-    _check(lib().faar_nvfp4_gemm(ctx._h, M, N, K, _p(A_packed), _p(A_scales_tiled), _p(A_s_global), _p(B_packed),
-                                 _p(B_scales_tiled), _p(B_s_global), _p(C), ldc, _p(ws), C_size(ws)), "faar_nvfp4_gemm")
+    _check(_fast().faar_nvfp4_gemm(ctx._n, M, N, K, A_packed, A_scales_tiled, A_s_global, B_packed, B_scales_tiled,
+           B_s_global, C, ldc, ws, ws.numel()), "faar_nvfp4_gemm")
 
 
 def transpose_bf16(ctx, rows, cols, inp, ld_in, out, ld_out):
-    _check(lib().faar_transpose_bf16(ctx._h, rows, cols, _p(inp), C.c_int64(ld_in), _p(out), C.c_int64(ld_out)),
-           "faar_transpose_bf16")
+    _check(_fast().faar_transpose_bf16(ctx._n, rows, cols, inp, ld_in, out, ld_out), "faar_transpose_bf16")
 
 
 def layer_ref(ctx, shape, X, W, Y_ref, ws):
-    _check(lib().faar_layer_ref(ctx._h, C.byref(shape), _p(X), _p(W), _p(Y_ref), _p(ws), C.c_size_t(ws.numel())),
-           "faar_layer_ref")
+    _check(_fast().faar_layer_ref(ctx._n, shape, X, W, Y_ref, ws, ws.numel()), "faar_layer_ref")
 
 
 def layer_fwd(ctx, shape, hp, X, Y_ref, V, code, scales, s_global, dYt, loss_mse, Y_q, ws):
-    _check(lib().faar_layer_fwd(ctx._h, C.byref(shape), C.byref(hp), _p(X), _p(Y_ref), _p(V), _p(code), _p(scales),
-                                _p(s_global), _p(dYt), _p(loss_mse), _p(Y_q), _p(ws), C.c_size_t(ws.numel())),
-           "faar_layer_fwd")
+    _check(_fast().faar_layer_fwd(ctx._n, shape, hp, X, Y_ref, V, code, scales, s_global, dYt, loss_mse, Y_q, ws,
+           ws.numel()), "faar_layer_fwd")
 
 
 def layer_dx(ctx, shape, beta, dY, V, code, scales, s_global, WsoftT, dX, ws):
-    _check(lib().faar_layer_dx(ctx._h, C.byref(shape), C.c_float(beta), _p(dY), _p(V), _p(code), _p(scales),
-                               _p(s_global), _p(WsoftT), _p(dX), _p(ws), C.c_size_t(ws.numel())), "faar_layer_dx")
+    _check(_fast().faar_layer_dx(ctx._n, shape, beta, dY, V, code, scales, s_global, WsoftT, dX, ws, ws.numel()),
+           "faar_layer_dx")
 
 
 def layer_dx_operand(ctx, shape, dY, Wsoft, dX, ws):
-    _check(lib().faar_layer_dx_operand(ctx._h, C.byref(shape), _p(dY), _p(Wsoft), _p(dX), _p(ws), C.c_size_t(ws.numel())),
-           "faar_layer_dx_operand")
+    _check(_fast().faar_layer_dx_operand(ctx._n, shape, dY, Wsoft, dX, ws, ws.numel()), "faar_layer_dx_operand")
 
 
 def round_loss(ctx, V, N, loss_round, ws):
-    _check(lib().faar_round_loss(ctx._h, _p(V), C.c_int64(N), _p(loss_round), _p(ws), C.c_size_t(ws.numel())),
-           "faar_round_loss")
+    _check(_fast().faar_round_loss(ctx._n, V, N, loss_round, ws, ws.numel()), "faar_round_loss")
 
 
 def round_loss_static(ctx, V, N, loss_round):
     """Round Loss without a workspace: for callers that may not allocate device memory.  The scratch
     is a fixed array inside libfaar.so; N is limited to round_loss_static_max_n()."""
-    _check(lib().faar_round_loss_static(ctx._h, _p(V), C.c_int64(N), _p(loss_round)), "faar_round_loss_static")
+    _check(_fast().faar_round_loss_static(ctx._n, V, N, loss_round), "faar_round_loss_static")
 
 
 def round_loss_static_max_n() -> int:
@@ -386,53 +391,44 @@ def round_loss_static_max_n() -> int:
 
 
 def layer_bwd(ctx, shape, hp, dYt, Xt, V, code, scales, s_global, adam_m, adam_u, dV, ws):
-    _check(lib().faar_layer_bwd(ctx._h, C.byref(shape), C.byref(hp), _p(dYt), _p(Xt), _p(V), _p(code), _p(scales),
-                                _p(s_global), _p(adam_m), _p(adam_u), _p(dV), _p(ws), C.c_size_t(ws.numel())),
-           "faar_layer_bwd")
+    _check(_fast().faar_layer_bwd(ctx._n, shape, hp, dYt, Xt, V, code, scales, s_global, adam_m, adam_u, dV, ws,
+           ws.numel()), "faar_layer_bwd")
 
 
 def layer_bwd_rowmajor(ctx, shape, hp, dY, X, V, code, scales, s_global, adam_m, adam_u, dV, ws):
-    _check(lib().faar_layer_bwd_rowmajor(ctx._h, C.byref(shape), C.byref(hp), _p(dY), _p(X), _p(V), _p(code), _p(scales),
-                                _p(s_global), _p(adam_m), _p(adam_u), _p(dV), _p(ws), C.c_size_t(ws.numel())),
-           "faar_layer_bwd_rowmajor")
+    _check(_fast().faar_layer_bwd_rowmajor(ctx._n, shape, hp, dY, X, V, code, scales, s_global, adam_m, adam_u, dV,
+           ws, ws.numel()), "faar_layer_bwd_rowmajor")
 
 
 def layer_step(ctx, shape, hp, X, Xt, Y_ref, V, code, scales, s_global, adam_m, adam_u, loss_out2, ws):
-    _check(lib().faar_layer_step(ctx._h, C.byref(shape), C.byref(hp), _p(X), _p(Xt), _p(Y_ref), _p(V), _p(code),
-                                 _p(scales), _p(s_global), _p(adam_m), _p(adam_u), _p(loss_out2), _p(ws),
-                                 C.c_size_t(ws.numel())), "faar_layer_step")
+    _check(_fast().faar_layer_step(ctx._n, shape, hp, X, Xt, Y_ref, V, code, scales, s_global, adam_m, adam_u,
+           loss_out2, ws, ws.numel()), "faar_layer_step")
 
 
 def harden_pack(ctx, shape, V, code, scales, s_global, packed, scales_out, decisions, W_final, wfinal_dtype=F32):
-    _check(lib().faar_harden_pack(ctx._h, C.byref(shape), _p(V), _p(code), _p(scales), _p(s_global), _p(packed),
-                                  _p(scales_out), _p(decisions), _p(W_final), C.c_int(wfinal_dtype)),
-           "faar_harden_pack")
+    _check(_fast().faar_harden_pack(ctx._n, shape, V, code, scales, s_global, packed, scales_out, decisions, W_final,
+           wfinal_dtype), "faar_harden_pack")
 
 
 def layer_step_host(ctx, shape, hp, X_host, Y_ref_host, W, X_dev, Xt_dev, Yref_dev, V, code, scales, s_global, adam_m,
                     adam_u, loss_dev2, loss_host2, ws):
     """X_host, Y_ref_host, loss_host2 are (pinned) CPU tensors; the rest are device tensors.  Y_ref_host None:
     the target is computed on the device from the copied X and W."""
-    _check(lib().faar_layer_step_host(ctx._h, C.byref(shape), C.byref(hp), C.c_void_p(X_host.data_ptr()),
-                                      C.c_void_p(Y_ref_host.data_ptr() if Y_ref_host is not None else 0), _p(W),
-                                      _p(X_dev), _p(Xt_dev), _p(Yref_dev), _p(V),
-                                      _p(code), _p(scales), _p(s_global), _p(adam_m), _p(adam_u), _p(loss_dev2),
-                                      C.c_void_p(loss_host2.data_ptr()), _p(ws), C.c_size_t(ws.numel())),
-           "faar_layer_step_host")
+    _check(_fast().faar_layer_step_host(ctx._n, shape, hp, X_host.data_ptr(),
+           None if Y_ref_host is None else Y_ref_host.data_ptr(), W, X_dev, Xt_dev, Yref_dev, V, code, scales, s_global, adam_m, adam_u, loss_dev2,
+           loss_host2.data_ptr(), ws, ws.numel()), "faar_layer_step_host")
 
 
 def nvfp4_expand(ctx, rows, K, packed, scales, out, ld):
-    _check(lib().faar_nvfp4_expand(ctx._h, rows, K, _p(packed), _p(scales), _p(out), C.c_int64(ld)), "faar_nvfp4_expand")
+    _check(_fast().faar_nvfp4_expand(ctx._n, rows, K, packed, scales, out, ld), "faar_nvfp4_expand")
 
 
 def layer_step_host_nvfp4(ctx, shape, hp, Xpacked_host, Xscales_host, Y_ref_host, Xpacked_dev, Xscales_dev, Xq_dev, Yref_dev,
                           V, code, scales, s_global, adam_m, adam_u, loss_dev2, loss_host2, ws):
     """Host tensors (pinned): packed codes, block scales, frozen target, the two-float loss."""
-    _check(lib().faar_layer_step_host_nvfp4(
-        ctx._h, C.byref(shape), C.byref(hp), C.c_void_p(Xpacked_host.data_ptr()), C.c_void_p(Xscales_host.data_ptr()),
-        C.c_void_p(Y_ref_host.data_ptr()), _p(Xpacked_dev), _p(Xscales_dev), _p(Xq_dev), _p(Yref_dev), _p(V), _p(code),
-        _p(scales), _p(s_global), _p(adam_m), _p(adam_u), _p(loss_dev2), C.c_void_p(loss_host2.data_ptr()), _p(ws),
-        C.c_size_t(ws.numel())), "faar_layer_step_host_nvfp4")
+    _check(_fast().faar_layer_step_host_nvfp4(ctx._n, shape, hp, Xpacked_host.data_ptr(), Xscales_host.data_ptr(),
+           Y_ref_host.data_ptr(), Xpacked_dev, Xscales_dev, Xq_dev, Yref_dev, V, code, scales, s_global, adam_m,
+           adam_u, loss_dev2, loss_host2.data_ptr(), ws, ws.numel()), "faar_layer_step_host_nvfp4")
 
 
 class KernelTime(C.Structure):
