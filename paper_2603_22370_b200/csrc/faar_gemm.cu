@@ -270,28 +270,39 @@ struct KParams {
 
 // Tile t of the launch: the first n_full_cols tile columns are bn wide, the remaining columns bn/2
 // (half-width tiles fill the last, partly empty wave of the CTA pairs and halve the epilogue that
-// nothing overlaps).  Tiles are numbered row block fastest, all full-width tiles first.
+// nothing overlaps).  All full-width tiles come first.  Tiles are numbered in bands of RASTER_ROWS row blocks, inside
+// a band row block fastest: the tiles that run at one time (74) then form a nearly square patch of the output, which
+// needs the fewest distinct operand rows.  With row blocks fastest over the whole height the LM head's product
+// (128 256 x 8192 outputs, 501 row blocks) read its 525 MB of weights from DRAM once per token tile.
+constexpr int RASTER_ROWS = 8;
 struct TileCoord { int m0, n0, w; };
+__device__ __forceinline__ void raster(int t, int m_tiles, int n_cols, int& m, int& n) {
+  const int band = t / (RASTER_ROWS * n_cols), first = band * RASTER_ROWS;
+  const int rows = min(RASTER_ROWS, m_tiles - first), r = t - first * n_cols;
+  n = r / rows;
+  m = first + r - n * rows;
+}
+__device__ __forceinline__ int half_columns(const KParams& p) {
+  const int rest = p.N - p.n_full_cols * p.bn;                    // columns covered by half-width tiles
+  return rest > 0 ? (rest + p.bn / 2 - 1) / (p.bn / 2) : 0;
+}
 __device__ __forceinline__ TileCoord tile_coord(const KParams& p, int t, int m_tiles) {
   const int full_tiles = m_tiles * p.n_full_cols;
   TileCoord c;
+  int m, n;
   if (t < full_tiles) {
-    c.m0 = (t % m_tiles) * (2 * BM);
-    c.n0 = (t / m_tiles) * p.bn;
+    raster(t, m_tiles, p.n_full_cols, m, n);
+    c.n0 = n * p.bn;
     c.w = p.bn;
   } else {
-    const int u = t - full_tiles;
-    c.m0 = (u % m_tiles) * (2 * BM);
-    c.n0 = p.n_full_cols * p.bn + (u / m_tiles) * (p.bn / 2);
+    raster(t - full_tiles, m_tiles, half_columns(p), m, n);
+    c.n0 = p.n_full_cols * p.bn + n * (p.bn / 2);
     c.w = p.bn / 2;
   }
+  c.m0 = m * (2 * BM);
   return c;
 }
-__device__ __forceinline__ int tile_count(const KParams& p, int m_tiles) {
-  const int rest = p.N - p.n_full_cols * p.bn;                    // columns covered by half-width tiles
-  const int half_cols = rest > 0 ? (rest + p.bn / 2 - 1) / (p.bn / 2) : 0;
-  return m_tiles * (p.n_full_cols + half_cols);
-}
+__device__ __forceinline__ int tile_count(const KParams& p, int m_tiles) { return m_tiles * (p.n_full_cols + half_columns(p)); }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
@@ -419,6 +430,28 @@ __device__ __forceinline__ float epi_fwd(const KParams& p, int o, int t0, const 
         if (FAAR_DBG_OK(p, q, 2, p.Yout, p.ext_yout, 1u)) *q = __float2bfloat16_rn(__uint_as_float(acc[j]) * p.act_scale);
       }
   }
+  return ss;
+}
+
+// The same for a chunk inside the matrix, 16 target values held as BF16 pairs (transposed target), no Y_q wanted: two
+// values at a time, which keeps the whole epilogue in registers.
+__device__ __forceinline__ float epi_fwd_vec(const KParams& p, int o, int t0, const uint32_t (&acc)[16], const uint4& ya, const uint4& yb) {
+  if (o >= p.M) return 0.f;
+  const uint32_t w[8] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
+  float ss = 0.f;
+  uint32_t d[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float r0 = __uint_as_float(acc[2 * i]) * p.act_scale - __uint_as_float(w[i] << 16);
+    const float r1 = __uint_as_float(acc[2 * i + 1]) * p.act_scale - __uint_as_float(w[i] & 0xFFFF0000u);
+    ss = fmaf(r0, r0, ss);
+    ss = fmaf(r1, r1, ss);
+    d[i] = pack_bf16x2(p.mse2c * r0, p.mse2c * r1);
+  }
+  uint4* d4 = reinterpret_cast<uint4*>(p.dYt + (long long)o * p.ld_dyt + t0);
+  if (!FAAR_DBG_OK(p, d4, 32, p.dYt, p.ext_dyt, 2u)) return ss;
+  d4[0] = make_uint4(d[0], d[1], d[2], d[3]);
+  d4[1] = make_uint4(d[4], d[5], d[6], d[7]);
   return ss;
 }
 
@@ -611,6 +644,10 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int total_tiles = WIDE ? m_tiles * ((p.N + WIDE_BN - 1) / WIDE_BN) : tile_count(p, m_tiles);
   const int k_blocks = (p.Kc + BK - 1) / BK;
 
+  if (threadIdx.x == 64) {                             // the copies' descriptors, fetched during the set-up
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     // accumulator-empty barriers are used in the leader only: every epilogue warp of both CTAs arrives there
@@ -736,6 +773,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     float s_global = 0.f;
     if (MODE == FAAR_GEMM_BWD) s_global = *p.s_global;
     uint32_t pn = 0;                                   // panels this quarter has staged so far
+    const bool yvec_ok = MODE == FAAR_GEMM_FWD && p.yref_t && p.yref_dtype == FAAR_BF16 && p.Yout == nullptr;
     bool dead = false;
     // One pass per accumulator buffer that fills: a tile, or (WIDE) a 256-column half of a tile.
     for (int vt = 0;; ++vt) {
@@ -744,10 +782,6 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       if (tile >= total_tiles) break;
       const int acc = WIDE ? vt & 1 : it & 1;
       const uint32_t acc_phase = WIDE ? it & 1 : (it >> 1) & 1;
-      bool ok = mbar_wait(tfull_bar(acc), acc_phase, ac, 0x400u | acc);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      tc_fence_after();
       TileCoord tc;
       if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * WIDE_BN + acc * BN_MAX; tc.w = BN_MAX; }
       else tc = tile_coord(p, tile, m_tiles);
@@ -756,6 +790,24 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int col_begin = cg * cols_per_warp;
       const int col_end = min(col_begin + cols_per_warp, TW);
       const int o = m0 + quarter * 32 + lane;
+      // FWD with a transposed BF16 target, columns inside the matrix: this lane's target values (128 at most, sixteen
+      // 16-byte loads) are requested before the wait for the accumulator, so their latency lies under the main loop
+      const bool yvec = yvec_ok && n0 + col_end <= p.N;
+      uint4 yraw[MODE == FAAR_GEMM_FWD ? 16 : 1];
+      if constexpr (MODE == FAAR_GEMM_FWD) {
+        static_assert(BN_MAX / C::COL_GROUPS == 128, "a warp's columns of the widest tile");
+        if (yvec && o < p.M) {
+          const uint4* y4 = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.Yref) +
+                                                           (long long)o * p.ldy + n0 + col_begin);
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (col_begin + 16 * q < col_end) { yraw[2 * q] = y4[2 * q]; yraw[2 * q + 1] = y4[2 * q + 1]; }
+        }
+      }
+      bool ok = mbar_wait(tfull_bar(acc), acc_phase, ac, 0x400u | acc);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
       const uint32_t trow = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN_MAX);
       if constexpr (MODE == FAAR_GEMM_BWD) {
         // PW-column panels, staged by the four warps of this lane quarter together (see epi_bwd_rows)
@@ -808,37 +860,15 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
         continue;
       } else {
-        if (MODE == FAAR_GEMM_FWD && p.yref_t && p.yref_dtype == FAAR_BF16) {
-          // transposed BF16 target: this lane's 64 values of four chunks are requested together
-          // (eight 16-byte loads in flight), so a tile costs two load latencies instead of one per chunk
-#pragma unroll 1
-          for (int cb = col_begin; cb < col_end; cb += 64) {
-            if (n0 + cb >= p.N) break;                   // warp-uniform
-            uint4 yraw[8];
-            if (o < p.M) {
-              const uint4* y4 = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.Yref) +
-                                                               (long long)o * p.ldy + n0 + cb);
+        if (MODE == FAAR_GEMM_FWD && yvec) {
 #pragma unroll
-              for (int q = 0; q < 4; ++q)
-                if (cb + 16 * q < col_end && n0 + cb + 16 * q < p.N) { yraw[2 * q] = y4[2 * q]; yraw[2 * q + 1] = y4[2 * q + 1]; }
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int c = cb + 16 * q;
-              if (c < col_end && n0 + c < p.N) {         // warp-uniform
-                uint32_t r[16];
-                tmem_ld16(trow + (uint32_t)c, r);
-                tmem_ld_wait();
-                const uint32_t w[8] = {yraw[2 * q].x, yraw[2 * q].y, yraw[2 * q].z, yraw[2 * q].w,
-                                       yraw[2 * q + 1].x, yraw[2 * q + 1].y, yraw[2 * q + 1].z, yraw[2 * q + 1].w};
-                float yr[16];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                  yr[2 * i] = __uint_as_float(w[i] << 16);
-                  yr[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-                }
-                warp_acc += epi_fwd(p, o, n0 + c, r, yr);
-              }
+          for (int q = 0; q < 8; ++q) {
+            const int c = col_begin + 16 * q;
+            if (c < col_end) {                           // warp-uniform
+              uint32_t r[16];
+              tmem_ld16(trow + (uint32_t)c, r);
+              tmem_ld_wait();
+              warp_acc += epi_fwd_vec(p, o, n0 + c, r, yraw[2 * q], yraw[2 * q + 1]);
             }
           }
         } else {
@@ -879,11 +909,12 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   }
 
   if constexpr (MODE == FAAR_GEMM_BWD) {
-    // Final loss sums by whichever CTA finishes last: always the same partials in the same order
-    // (strided double accumulation, then a tree), so the result does not depend on which CTA it is.
+    // Final loss sums by whichever CTA finishes last: always the same partials in the same order (strided double
+    // accumulation, then a tree over lanes and one over warps), so the result does not depend on which CTA it is.
     if (p.fin_out2 != nullptr) {
-      double* sh = reinterpret_cast<double*>(smem);          // the operand ring is idle by now
-      volatile int* last_flag = reinterpret_cast<volatile int*>(smem + 256 * sizeof(double));
+      constexpr int WARPS = C::THREADS / 32;
+      double* sh = reinterpret_cast<double*>(smem);          // [2][WARPS]; the operand ring is idle by now
+      volatile int* last_flag = reinterpret_cast<volatile int*>(smem + 2 * WARPS * sizeof(double));
       if (threadIdx.x == 0) {
         __threadfence();                                     // this CTA's partials, ordered by the barrier above
         int last = 0;
@@ -900,20 +931,20 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       __syncthreads();
       if (*last_flag) {
         const int n_round = (int)gridDim.x * C::EPI_WARPS;
-        for (int which = 0; which < 2; ++which) {
-          const float* src = which ? p.partials : p.fin_mse_partials;
-          const int n = which ? n_round : p.fin_n_mse;
-          double acc = 0.0;
-          if (threadIdx.x < 256)
-            for (int i = threadIdx.x; i < n; i += 256) acc += (double)__ldcg(src + i);
-          __syncthreads();
-          if (threadIdx.x < 256) sh[threadIdx.x] = acc;
-          __syncthreads();
-          for (int st = 128; st > 0; st >>= 1) {
-            if (threadIdx.x < st) sh[threadIdx.x] += sh[threadIdx.x + st];
-            __syncthreads();
-          }
-          if (threadIdx.x == 0) p.fin_out2[which] = (float)(sh[0] * (double)(which ? p.fin_scale_round : p.fin_scale_mse));
+        double mse = 0.0, rnd = 0.0;
+        for (int i = threadIdx.x; i < p.fin_n_mse; i += C::THREADS) mse += (double)__ldcg(p.fin_mse_partials + i);
+        for (int i = threadIdx.x; i < n_round; i += C::THREADS) rnd += (double)__ldcg(p.partials + i);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          mse += __shfl_xor_sync(0xffffffffu, mse, o);
+          rnd += __shfl_xor_sync(0xffffffffu, rnd, o);
+        }
+        if (lane == 0) { sh[warp] = mse; sh[WARPS + warp] = rnd; }
+        __syncthreads();
+        if (threadIdx.x < 2) {
+          double t = 0.0;
+          for (int w = 0; w < WARPS; ++w) t += sh[threadIdx.x * WARPS + w];
+          p.fin_out2[threadIdx.x] = (float)(t * (double)(threadIdx.x ? p.fin_scale_round : p.fin_scale_mse));
         }
       }
     }
