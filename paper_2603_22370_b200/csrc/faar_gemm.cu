@@ -37,6 +37,7 @@ constexpr int PANEL_BYTES = 32 * PW * 4;       // one 32-row x PW-column FP32 pa
 constexpr int SMEM_LIMIT = 227 * 1024;
 constexpr int CTL_BYTES = 512;
 constexpr int MAX_EPI_WARPS = 16;
+constexpr int MAX_STAGES = 10;
 
 // The tile width bn (accumulator columns, a multiple of 16 up to 256) is a launch parameter chosen by
 // the host (pick_bn).  Shared memory and tensor memory are laid out for the widest tile.
@@ -52,14 +53,17 @@ template <int MODE, bool WIDE = false> struct Cfg {
   static constexpr int THREADS = 32 * (2 + EPI_WARPS);
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int BH_BYTES = (BN_MAX / 2) * BK * 2;       // this CTA's 128 rows of one 256-column B tile
-  static constexpr int B_BYTES = WIDE ? 2 * BH_BYTES : BH_BYTES;   // slot size
+  static constexpr int B_BYTES = WIDE ? 2 * BH_BYTES : BH_BYTES;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int EPI_BYTES = MODE == FAAR_GEMM_BWD ? 4 * PANEL_BYTES : 0;
-  static constexpr int FIT = (SMEM_LIMIT - 1024 - CTL_BYTES - EPI_BYTES) / STAGE_BYTES;
-  static constexpr int STAGES = FIT > 8 ? 8 : FIT;
+  // The ring: as many stages of the launch's tile width as fit (a stage is the A rows plus bn / 2 rows of B: 32 KB for
+  // 256 columns, 18 KB for 32), at most MAX_STAGES.  A small launch's main loop runs at stages / latency, so narrow
+  // tiles get the deeper ring.
+  static constexpr int RING_BYTES = (SMEM_LIMIT - 1024 - CTL_BYTES - EPI_BYTES) / 1024 * 1024;
+  static constexpr int MIN_STAGES = RING_BYTES / STAGE_BYTES;
   static constexpr int TMEM_COLS = 2 * BN_MAX;                 // two accumulator buffers
   static constexpr int COL_GROUPS = EPI_WARPS / 4;             // warps sharing one TMEM lane quarter
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024 /*alignment slack*/ + CTL_BYTES;
+  static constexpr int SMEM_BYTES = RING_BYTES + EPI_BYTES + 1024 /*alignment slack*/ + CTL_BYTES;
 };
 
 // ---- PTX wrappers ------------------------------------------------------------------------
@@ -244,6 +248,7 @@ __device__ __forceinline__ uint32_t make_idesc(int bn, int a_mn = 0, int b_mn = 
 struct KParams {
   int M, N, Kc;
   int bn;                 // tile width
+  int stages, stage_bytes;   // ring depth, bytes of a stage (both CTAs alike)
   int n_full_cols;        // tile columns of full width; the columns after them are bn/2 wide (tail split)
   int a_mn, b_mn;         // operand stored with M (N) contiguous, [Kc, M] / [Kc, N], instead of [M, Kc] / [N, Kc]
   uint32_t* status;
@@ -259,9 +264,17 @@ struct KParams {
   // BWD: M = O, N = K
   float* V; const uint8_t* code; const uint8_t* scales; const float* s_global;
   float* adam_m; float* adam_u; float* dV;
-  float beta, lam_over_n, lr, b1, b2, eps, inv_bc1, inv_bc2; int opt;
+  // constants of the update, derived once on the host: as kernel parameters they are operands of the instructions that
+  // use them and take no registers
+  float bl, hbl;                    // beta log2(e) (e^x as 2^(x log2 e)), -bl / 2
+  float sbeta;                      // beta act_scale / 2 (the narrowest interval is 0.5 wide)
+  float lam4;                       // -4 lambda / N: (lambda / N) (4 - 8 v) = lam4 (2 v - 1)
+  float b1, b2, c1, c2, eps;        // c = 1 - b
+  float nstep;                      // -lr / bias correction 1 (Adam), -lr (gradient descent)
+  float rbc2;                       // sqrt(u / bc2) = sqrt(u) rbc2
+  float nbl_next, hbl_next;         // the next step's Eq. 3 (faar_operand_consts)
   // BWD, optional: the next step's BF16 forward operand, from the updated v (null = not wanted)
-  __nv_bfloat16* wsoft_next; float beta_next;
+  __nv_bfloat16* wsoft_next;
   // BWD, optional: the CTA that finishes last also forms the step's two loss values
   uint32_t* fin_counter;            // workspace word, zero between launches
   const float* fin_mse_partials; int fin_n_mse; float fin_scale_mse;
@@ -478,74 +491,63 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // 4 (l % LPR)..+3, so that one warp instruction moves 512 bytes of V / m / u as 32 / LPR row pieces of
 // 4 PW contiguous bytes each: whole lines as 16-byte vectors.  (A panel of 128 columns gives one 512-byte
 // piece per instruction but leaves room for five TMA stages only; the sixth stage is worth more.)
-// The per-weight state of RPG such instructions is requested together before any of it is computed
-// (one measured fastest: the sixteen warps of a CTA already keep 24 KB of state loads in flight).
-// FULL: the panel lies wholly inside the matrix (no bounds tests).
+// The per-weight state of the next instruction is requested before the current one's is computed, and a panel's first
+// before the panel is staged (a tile's first before its accumulator is ready): a request takes 600-800 clocks, the
+// arithmetic of one instruction's weights about 400, and a small launch has nothing else to hide the former.
 // o_first: output feature of panel row 0; k_first: input feature of panel column 0; k_end: first
 // input feature beyond the tile (or the matrix).
 // Returns the Round Loss contribution of the pre-update v's.
-constexpr int RPG = 1;
 constexpr int LPR = PW / 4;                     // lanes per panel row
 constexpr int RPI = 32 / LPR;                   // rows per warp instruction
 constexpr int ITS = 8 / RPI;                    // instructions per warp and panel
-template <int OPT, bool FULL>
+struct RowState { float4 v, m, u; uint32_t cw, sb; };
+// State of this lane's four weights of instruction `it` of the panel whose row 0 / column 0 is (o_first, k_first), or
+// nothing if they lie outside the matrix or at or beyond column k_end.
+template <int OPT>
+__device__ __forceinline__ bool load_row_state(const KParams& p, int lane, int sub, int o_first, int k_first, int k_end, int it,
+                                               uint64_t stream, RowState& st) {
+  const int row = o_first + 8 * sub + lane / LPR + RPI * it, col = k_first + 4 * (lane % LPR);
+  const bool ok = row < p.M && col < k_end;
+  if (ok) {
+    const long long e = (long long)row * p.N + col;
+    st.v = ldg128_stream(p.V + e, stream);
+    st.cw = *reinterpret_cast<const uint16_t*>(p.code + (e >> 1));
+    st.sb = p.scales[e >> 4];
+    if (OPT & 1) {
+      st.m = ldg128_stream(p.adam_m + e, stream);
+      st.u = ldg128_stream(p.adam_u + e, stream);
+    }
+  }
+  return ok;
+}
+// `st` / `st_ok` hold the state of instruction 0 on entry; on return those of instruction 0 of the panel at column
+// k_next (unless k_next >= k_end).
+template <int OPT>
 __device__ __forceinline__ float epi_bwd_rows(const KParams& p, uint32_t panel, int lane, int sub, int o_first,
-                                              int k_first, int k_end, float s_global) {
+                                              int k_first, int k_next, int k_end, float s_global, RowState& st, bool& st_ok) {
   const int cu = lane % LPR;                                       // 16-byte unit of the row
-  const int kcol = k_first + 4 * cu;
-  const bool col_ok = FULL || kcol < k_end;
   const int r0 = 8 * sub + lane / LPR;                             // this lane's row in the first instruction
-  const long long e0 = (long long)(o_first + r0) * p.N + kcol;     // row r0 element of this lane
-  float* const Vp = p.V + e0;
-  float* const Mp = p.adam_m + e0;
-  float* const Up = p.adam_u + e0;
-  const uint8_t* const Cp = p.code + (e0 >> 1);
-  const uint8_t* const Sp = p.scales + (e0 >> 4);
-  const float bl = p.beta * 1.44269504088896341f;                 // beta log2(e): e^x as 2^(x log2 e)
-  const float hbl = -0.5f * bl;
-  const float c1 = 1.f - p.b1, c2 = 1.f - p.b2;
-  const float step_size = p.lr * p.inv_bc1;
-  const float rbc2 = sqrtf(p.inv_bc2);                            // sqrt(u / bc2) = sqrt(u) sqrt(1 / bc2)
-  const float lam4 = -4.f * p.lam_over_n;                         // (lambda / N) (4 - 8 v) = lam4 (2 v - 1)
-  float nbl_next, hbl_next;                                       // OPT & 2: constants of the next step's Eq. 3
-  faar_operand_consts(p.beta_next, &nbl_next, &hbl_next);
+  const long long e0 = (long long)(o_first + r0) * p.N + k_first + 4 * cu;         // row r0 element of this lane
   const uint64_t stream = l2_policy_stream();
   const uint64_t vkeep = l2_policy_keep();       // the updated V is the next kernel's input (soft weights)
   float tt = 0.f, n_el = 0.f;                                     // sum of (2 v - 1)^2, elements seen
 #pragma unroll
-  for (int grp = 0; grp < ITS / RPG; ++grp) {
-    float4 v[RPG], m[RPG], u[RPG];
-    uint32_t cw[RPG], sb[RPG];
-    bool ok[RPG];
-#pragma unroll
-    for (int q = 0; q < RPG; ++q) {
-      const int i = RPI * (RPG * grp + q);                              // row r0 + i
-      ok[q] = FULL || (col_ok && o_first + r0 + i < p.M);
-      if (ok[q]) {
-        const int off = i * p.N;
-        v[q] = ldg128_stream(Vp + off, stream);
-        cw[q] = *reinterpret_cast<const uint16_t*>(Cp + (off >> 1));
-        sb[q] = Sp[off >> 4];
-        if (OPT & 1) {
-          m[q] = ldg128_stream(Mp + off, stream);
-          u[q] = ldg128_stream(Up + off, stream);
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < RPG; ++q) {
-      if (ok[q]) {
-        const int i = RPI * (RPG * grp + q);
-        const int row = r0 + i;
-        const int off = i * p.N;
+  for (int it = 0; it < ITS; ++it) {
+    const RowState cur = st;
+    const bool ok = st_ok;
+    st_ok = it + 1 < ITS ? load_row_state<OPT>(p, lane, sub, o_first, k_first, k_end, it + 1, stream, st)
+                         : load_row_state<OPT>(p, lane, sub, o_first, k_next, k_end, 0, stream, st);
+    {
+      if (ok) {
+        const int row = r0 + RPI * it;
+        const long long e = e0 + (long long)(RPI * it) * p.N;
         const float4 g4 = lds128(panel + (uint32_t)row * (4u * PW) + (uint32_t)((cu ^ (row & 7)) << 4));
         const float G[4] = {g4.x, g4.y, g4.z, g4.w};
-        const float vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-        // s beta / 2 (the narrowest interval is 0.5 wide); act_scale: G = act_scale * acc
-        const float sc = __fmul_rn(faar_e4m3_to_float(sb[q]), s_global);
-        const float sbh = sc * (0.5f * p.beta * p.act_scale);
+        const float vv[4] = {cur.v.x, cur.v.y, cur.v.z, cur.v.w};
+        const float sc = __fmul_rn(faar_e4m3_to_float(cur.sb), s_global);
+        const float sbh = sc * p.sbeta;
         // byte j: log2 of (interval width / 0.5) of element j, looked up by its interval index k (0 0 0 0 1 1 2)
-        const uint32_t ksel = cw[q] & 0x7777u;
+        const uint32_t ksel = cur.cw & 0x7777u;
         const uint32_t wlog = __byte_perm(0u, 0x00020101u, ksel);
         // OPT & 2: bytes 3 and 2 of the lower node's float (0 .5 1 1.5 2 3 4) by the same look-up
         uint32_t lo_hi = 0u, lo_lo = 0u;
@@ -557,51 +559,51 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, uint32_t panel, 
         float g[4], vn[4], mn[4], un[4];
         float mm[4], uu[4];
         if (OPT & 1) {
-          mm[0] = m[q].x; mm[1] = m[q].y; mm[2] = m[q].z; mm[3] = m[q].w;
-          uu[0] = u[q].x; uu[1] = u[q].y; uu[2] = u[q].z; uu[3] = u[q].w;
+          mm[0] = cur.m.x; mm[1] = cur.m.y; mm[2] = cur.m.z; mm[3] = cur.m.w;
+          uu[0] = cur.u.x; uu[1] = cur.u.y; uu[2] = cur.u.z; uu[3] = cur.u.w;
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const float ex = ex2_approx(-fabsf(fmaf(bl, vv[j], hbl)));         // e^-|beta (v - 0.5)|
+          const float ex = ex2_approx(-fabsf(fmaf(p.bl, vv[j], p.hbl)));         // e^-|beta (v - 0.5)|
           const float hs = rcp_approx(1.0f + ex);
           const float dh = ex * hs * hs;                                     // h (1 - h)
           // dh times the width factor by an add to its exponent field (a dh flushed to 0 becomes ~1e-38), then
           // the sign of w from bit 3 of the nibble
           const uint32_t wexp = (j < 3 ? wlog << (23 - 8 * j) : wlog >> 1) & 0x01800000u;
-          const uint32_t sgn = (cw[q] << (28 - 4 * j)) & 0x80000000u;
+          const uint32_t sgn = (cur.cw << (28 - 4 * j)) & 0x80000000u;
           float chain = sbh * __uint_as_float(__float_as_uint(dh) + wexp);
           chain = __uint_as_float(__float_as_uint(chain) ^ sgn);
           const float t = fmaf(2.f, vv[j], -1.f);
-          g[j] = fmaf(G[j], chain, lam4 * t);
+          g[j] = fmaf(G[j], chain, p.lam4 * t);
           tt = fmaf(t, t, tt);
           if (OPT & 1) {
-            mn[j] = fmaf(p.b1, mm[j], c1 * g[j]);
-            un[j] = fmaf(p.b2, uu[j], c2 * g[j] * g[j]);
-            const float den = fmaf(sqrt_approx(un[j]), rbc2, p.eps);
-            vn[j] = __saturatef(fmaf(-step_size, mn[j] * rcp_approx(den), vv[j]));   // clip to [0, 1]
+            mn[j] = fmaf(p.b1, mm[j], p.c1 * g[j]);
+            un[j] = fmaf(p.b2, uu[j], p.c2 * g[j] * g[j]);
+            const float den = fmaf(sqrt_approx(un[j]), p.rbc2, p.eps);
+            vn[j] = __saturatef(fmaf(p.nstep, mn[j] * rcp_approx(den), vv[j]));   // clip to [0, 1]
           } else {
-            vn[j] = __saturatef(fmaf(-p.lr, g[j], vv[j]));
+            vn[j] = __saturatef(fmaf(p.nstep, g[j], vv[j]));
           }
           if (OPT & 2) {
             // Eq. 2 / Eq. 3 at the updated v with the next step's beta: (lo + h width) s with the sign of w, in
             // the soft-weights kernel's operations, so that the BF16 operand is the same bit for bit
             const float lo = __uint_as_float(__byte_perm(lo_hi, lo_lo, (uint32_t)((j << 12) | ((4 + j) << 8))) & 0xFFFF0000u);
             const float wd = __uint_as_float(0x3F000000u + wexp);
-            const float mag = faar_operand_weight(faar_sigmoid_operand(nbl_next, hbl_next, vn[j]), lo, wd, sc);
+            const float mag = faar_operand_weight(faar_sigmoid_operand(p.nbl_next, p.hbl_next, vn[j]), lo, wd, sc);
             wn[j] = __uint_as_float(__float_as_uint(mag) ^ sgn);
           }
         }
-        // one check covers the five stores below: they share the element offset e0 + off
-        if (!FAAR_DBG_OK(p, Vp + off, 16, p.V, p.ext_state, 3u)) continue;
-        if ((OPT & 2) && !FAAR_DBG_OK(p, p.wsoft_next + e0 + off, 8, p.wsoft_next, p.ext_wsoft, 4u)) continue;
+        // one check covers the five stores below: they share the element offset e
+        if (!FAAR_DBG_OK(p, p.V + e, 16, p.V, p.ext_state, 3u)) continue;
+        if ((OPT & 2) && !FAAR_DBG_OK(p, p.wsoft_next + e, 8, p.wsoft_next, p.ext_wsoft, 4u)) continue;
         if (OPT & 2)
-          *reinterpret_cast<uint2*>(p.wsoft_next + e0 + off) = make_uint2(pack_bf16x2(wn[0], wn[1]), pack_bf16x2(wn[2], wn[3]));
-        if (p.dV) stg128_stream(p.dV + e0 + off, g[0], g[1], g[2], g[3], stream);
+          *reinterpret_cast<uint2*>(p.wsoft_next + e) = make_uint2(pack_bf16x2(wn[0], wn[1]), pack_bf16x2(wn[2], wn[3]));
+        if (p.dV) stg128_stream(p.dV + e, g[0], g[1], g[2], g[3], stream);
         if (OPT & 1) {
-          stg128_stream(Mp + off, mn[0], mn[1], mn[2], mn[3], stream);
-          stg128_stream(Up + off, un[0], un[1], un[2], un[3], stream);
+          stg128_stream(p.adam_m + e, mn[0], mn[1], mn[2], mn[3], stream);
+          stg128_stream(p.adam_u + e, un[0], un[1], un[2], un[3], stream);
         }
-        stg128_stream(Vp + off, vn[0], vn[1], vn[2], vn[3], vkeep);
+        stg128_stream(p.V + e, vn[0], vn[1], vn[2], vn[3], vkeep);
         n_el += 4.f;
       }
     }
@@ -624,16 +626,18 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;       // the same offset in both CTAs of the pair
   uint8_t* smem = smem_raw + (base - raw);
-  const uint32_t epi_u32 = base + C::STAGES * C::STAGE_BYTES;
-  uint8_t* ctl = smem + C::STAGES * C::STAGE_BYTES + C::EPI_BYTES;
+  const int STAGES = p.stages;
+  const uint32_t STAGE_BYTES = (uint32_t)p.stage_bytes;
+  const uint32_t epi_u32 = base + C::RING_BYTES;
+  uint8_t* ctl = smem + C::RING_BYTES + C::EPI_BYTES;
   const uint32_t ctl_u32 = epi_u32 + C::EPI_BYTES;
   // control block: full[S], empty[S], tmem_full[2], tmem_empty[2], tmem base, abort flag
   auto full_bar = [&](int s) { return ctl_u32 + 8u * s; };
-  auto empty_bar = [&](int s) { return ctl_u32 + 8u * (C::STAGES + s); };
-  auto tfull_bar = [&](int a) { return ctl_u32 + 8u * (2 * C::STAGES + a); };
-  auto tempty_bar = [&](int a) { return ctl_u32 + 8u * (2 * C::STAGES + 2 + a); };
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(ctl + 8 * (2 * C::STAGES + 4));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(ctl + 8 * (2 * C::STAGES + 4) + 4);
+  auto empty_bar = [&](int s) { return ctl_u32 + 8u * (MAX_STAGES + s); };
+  auto tfull_bar = [&](int a) { return ctl_u32 + 8u * (2 * MAX_STAGES + a); };
+  auto tempty_bar = [&](int a) { return ctl_u32 + 8u * (2 * MAX_STAGES + 2 + a); };
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(ctl + 8 * (2 * MAX_STAGES + 4));
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(ctl + 8 * (2 * MAX_STAGES + 4) + 4);
   const AbortCtl ac{abort_flag, p.status};
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -649,7 +653,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
   }
   if (threadIdx.x == 0) {
-    for (int s = 0; s < C::STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
+    for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     // accumulator-empty barriers are used in the leader only: every epilogue warp of both CTAs arrives there
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 2 * C::EPI_WARPS); }
     for (int q = 0; q < 8; ++q) mbar_init(ctl_u32 + 256u + 8u * q, 4);   // panel staged / panel consumed, per lane quarter
@@ -687,7 +691,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int kb = 0; kb < k_blocks; ++kb) {
           ok = mbar_wait(empty_bar(stage), phase ^ 1u, ac, 0x100u | stage);
           if (!ok) break;
-          const uint32_t sa = base + stage * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+          const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + C::A_BYTES;
           // the leader's barrier collects the bytes of both CTAs' copies
           if (rank == 0)
             mbar_expect_tx(full_bar(stage), WIDE ? 2u * (uint32_t)(C::A_BYTES + C::B_BYTES)
@@ -707,7 +711,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
           // second column half (rows beyond the matrix arrive as zeros)
           if (WIDE) tma_load_2d(sb + C::BH_BYTES, &tmB, kb * BK, n0 + BN_MAX, leader_full, keep);
-          if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
       if (!ok) {
@@ -737,7 +741,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           ok = __all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, ac, 0x300u | stage));
           if (!ok) break;
           tc_fence_after();
-          const uint32_t sa = base + stage * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+          const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + C::A_BYTES;
           const uint64_t da = A_MN ? make_smem_desc_mn(sa) : make_smem_desc(sa);
           const uint64_t db = B_MN ? make_smem_desc_mn(sb) : make_smem_desc(sb);
           constexpr uint32_t ka = A_MN ? MN_KSTEP : 2u, kbs = B_MN ? MN_KSTEP : 2u;
@@ -754,7 +758,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             tc_commit_pair(empty_bar(stage));          // frees this stage in both CTAs
           }
           __syncwarp();
-          if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (ok && faar_elect_one()) {
           tc_commit_pair(tfull_bar(acc));              // accumulator ready in both CTAs
@@ -773,6 +777,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     float s_global = 0.f;
     if (MODE == FAAR_GEMM_BWD) s_global = *p.s_global;
     uint32_t pn = 0;                                   // panels this quarter has staged so far
+    RowState row_state;                                // BWD: state requested ahead
+    bool row_ok = false;
     const bool yvec_ok = MODE == FAAR_GEMM_FWD && p.yref_t && p.yref_dtype == FAAR_BF16 && p.Yout == nullptr;
     bool dead = false;
     // One pass per accumulator buffer that fills: a tile, or (WIDE) a 256-column half of a tile.
@@ -804,6 +810,9 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (col_begin + 16 * q < col_end) { yraw[2 * q] = y4[2 * q]; yraw[2 * q + 1] = y4[2 * q + 1]; }
         }
       }
+      const int k_end = min(p.N, n0 + TW);               // BWD: columns of this tile that exist
+      if constexpr (MODE == FAAR_GEMM_BWD)
+        row_ok = load_row_state<OPT>(p, lane, ew >> 2, m0 + quarter * 32, n0, k_end, 0, l2_policy_stream(), row_state);
       bool ok = mbar_wait(tfull_bar(acc), acc_phase, ac, 0x400u | acc);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -833,21 +842,17 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               sts128(panel + (uint32_t)lane * (4u * PW) + (uint32_t)(((4 * sub + u) ^ (lane & 7)) << 4), r[4 * u],
                      r[4 * u + 1], r[4 * u + 2], r[4 * u + 3]);
           }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(pfull);
           if (pc + PW >= TW || n0 + pc + PW >= p.N) {    // this warp's last read of the accumulator
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), 0));
             released = true;
           }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(pfull);
           okp = mbar_wait(pfull, pn & 1u, ac, 0x600u | quarter);
           if (!__all_sync(0xffffffffu, okp)) { dead = true; break; }
-          const int k_end = min(p.N, n0 + TW);           // columns of this tile that exist
-          if (o_first + 32 <= p.M && n0 + pc + PW <= k_end)
-            warp_acc += epi_bwd_rows<OPT, true>(p, panel, lane, sub, o_first, n0 + pc, k_end, s_global);
-          else
-            warp_acc += epi_bwd_rows<OPT, false>(p, panel, lane, sub, o_first, n0 + pc, k_end, s_global);
+          warp_acc += epi_bwd_rows<OPT>(p, panel, lane, sub, o_first, n0 + pc, n0 + pc + PW, k_end, s_global, row_state, row_ok);
           __syncwarp();
           if (lane == 0) mbar_arrive(pdone);
           ++pn;
@@ -1000,25 +1005,41 @@ int make_map_mn(faar_ctx* ctx, CUtensorMap* map, const void* ptr, int kc_rows, i
   return r == CUDA_SUCCESS ? 0 : (int)cudaErrorInvalidValue;
 }
 
-// Tile width for an M x N output.  A tile's time is set by the operand bytes it pulls through the SM (A rows
-// are not shared between tiles), not by its columns, so 256-wide tiles win wherever they were measured
-// against narrower ones that fill more CTA pairs (down_proj-, gate-, q- and k_proj-shaped layers), with one
-// exception: the dW GEMM of a small layer, whose per-weight epilogue is heavy, gains from spreading 128-wide
-// tiles over twice as many pairs while fewer than half of the pairs would have a 256-wide tile.  A tile is
-// never wider than the output rounded up to 32 columns.
-int pick_bn_k_major(const faar_ctx* ctx, int mode, int M, int N, int pairs);
-int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int pairs, bool b_mn) {
-  const int bn = pick_bn_k_major(ctx, mode, M, N, pairs);
-  // an N-contiguous B comes in boxes of 64 columns per CTA: widths 128 and 256 only
-  return b_mn && bn % 128 != 0 ? (N <= 128 ? 128 : BN_MAX) : bn;
-}
-int pick_bn_k_major(const faar_ctx* ctx, int mode, int M, int N, int pairs) {
-  if (ctx->tune_bn >= 128 && ctx->tune_bn <= BN_MAX && ctx->tune_bn % 16 == 0) return ctx->tune_bn;
+// Tile width for an M x N output over k_blocks blocks of the contraction.  While 256-wide tiles give every CTA pair one,
+// they win: a tile's time is set by the operand bytes it pulls through the SM, and the A rows are the same for any
+// width.  A smaller problem is a matter of latency: its tiles run at once, each brings its share of the epilogue, and
+// narrower tiles spread that over more SMs.
+// REF, FWD: the width with the smallest estimated time of the busiest pair (microseconds).  A k block costs the ring's
+// latency, or what the L2 needs for all pairs' operands (about 10 TB/s); the epilogue 0.8 / 0.6 per 64 columns.
+// Measured (width before -> after): product [260, 1024] over 512 8.8 -> 6.2 us (128 -> 32), forward kernel of a
+// 128 x 256 layer at 1024 tokens 12.8 -> 10.7 us, input gradient [192, 128] over 384 11.1 -> 8.9 us.
+// BWD: its per-weight epilogue is bound by instruction issue and a tile of it has a fixed cost of several microseconds,
+// so only 128-wide tiles (cut into halves of 64 by pick_full_cols while pairs are idle) while fewer than half of the
+// pairs would have a 256-wide one; 32-wide tiles: dW kernel of a 128 x 256 layer 19.2 -> 18.8 us, of a 1024 x 3600 layer
+// 33.6 -> 51 us.
+int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs, bool b_mn) {
+  if (ctx->tune_bn >= 128 && ctx->tune_bn <= BN_MAX && ctx->tune_bn % 16 == 0)
+    return b_mn && ctx->tune_bn % 128 != 0 ? (N <= 128 ? 128 : BN_MAX) : ctx->tune_bn;   // boxes of 64 columns per CTA
   const long long m_tiles = (M + 2 * BM - 1) / (2 * BM);
-  int bn = BN_MAX;
-  if (N < BN_MAX) bn = N <= 128 ? 128 : (N + 31) / 32 * 32;
-  if (mode == FAAR_GEMM_BWD && 2 * m_tiles * ((N + BN_MAX - 1) / BN_MAX) < pairs) bn = 128;
-  return bn;
+  if (mode == FAAR_GEMM_BWD) {
+    if (N <= 128 || 2 * m_tiles * ((N + BN_MAX - 1) / BN_MAX) < pairs) return 128;
+    return N < BN_MAX && !b_mn ? (N + 31) / 32 * 32 : BN_MAX;
+  }
+  const int widest = N > 128 ? (N < BN_MAX ? (N + 31) / 32 * 32 : BN_MAX) : (N > 64 ? 128 : (N > 32 ? 64 : 32));
+  if (m_tiles * ((N + widest - 1) / widest) >= pairs) return widest;
+  const double epi64 = mode == FAAR_GEMM_FWD ? 0.6 : 0.8;
+  int best = widest;
+  double best_cost = 1e30;
+  for (int bn = widest; bn >= 32; bn = bn > 128 ? 128 : bn / 2) {
+    const long long tiles = m_tiles * ((N + bn - 1) / bn);
+    const long long waves = (tiles + pairs - 1) / pairs, active = tiles < pairs ? tiles : pairs;
+    const double l2 = 2.0 * active * (BM + bn / 2) * BK * 2 / 1e7;
+    const double latency = bn > 128 ? 0.22 : (bn > 64 ? 0.19 : 0.16);
+    const double loop = k_blocks * (l2 > latency ? l2 : latency), epi = epi64 * bn / 64.0;
+    const double cost = waves * loop + epi + (waves - 1) * (epi > loop ? epi - loop : 0.0);
+    if (cost < best_cost - 1e-9) { best_cost = cost; best = bn; }
+  }
+  return best;
 }
 
 // How many trailing tile columns to cut into half-width tiles.  Tiles go to CTA pairs round-robin, all
@@ -1028,7 +1049,7 @@ int pick_bn_k_major(const faar_ctx* ctx, int mode, int M, int N, int pairs) {
 int pick_full_cols(const faar_ctx* ctx, int M, int N, int bn, int pairs) {
   const int m_tiles = (M + 2 * BM - 1) / (2 * BM);
   const int n_cols = (N + bn - 1) / bn;
-  if (bn % 32 != 0) return n_cols;
+  if (bn % 32 != 0 || bn <= 64) return n_cols;
   if (ctx->tune_tail >= 0) return ctx->tune_tail < n_cols ? n_cols - ctx->tune_tail : 0;
   double best = -1.0;
   int best_full = n_cols;
@@ -1066,7 +1087,7 @@ template <int MODE, int OPT, bool WIDE, int MN>
 int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_out, int bn, int max_pairs,
                    const cudaLaunchConfig_t& base_cfg) {
   using C = Cfg<MODE, WIDE>;
-  static_assert(C::STAGES >= 3, "ring too short");
+  static_assert(C::MIN_STAGES >= 3, "ring too short");
   static_assert(C::SMEM_BYTES <= SMEM_LIMIT, "shared memory budget");
   static_assert(C::EPI_WARPS <= MAX_EPI_WARPS, "partials budget");
   auto kern = faar_gemm_kernel<MODE, OPT, WIDE, MN>;
@@ -1075,6 +1096,8 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   cudaLaunchConfig_t cfg = base_cfg;
   cfg.dynamicSmemBytes = C::SMEM_BYTES;
   kp.bn = bn;
+  kp.stage_bytes = WIDE ? C::STAGE_BYTES : C::A_BYTES + (int)faar_align_up((size_t)(bn / 2) * BK * 2, 1024);   // whole 8-row swizzle atoms
+  kp.stages = C::RING_BYTES / kp.stage_bytes < MAX_STAGES ? C::RING_BYTES / kp.stage_bytes : MAX_STAGES;
   kp.n_full_cols = WIDE ? 0 : pick_full_cols(ctx, a->M, a->N, bn, max_pairs);
   if (a->b_mn && bn != BN_MAX) kp.n_full_cols = (a->N + bn - 1) / bn;      // half tiles of a 128-wide tile would be 32 columns per CTA
   CUtensorMap tmA, tmB, tmBh;
@@ -1127,7 +1150,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
   const int e = faar_allow_smem(ctx, (const void*)kern, C::SMEM_BYTES);
   if (e) return e;
   const int max_pairs = faar_max_pairs(ctx, MODE == FAAR_GEMM_BWD ? 2 + OPT : MODE, (const void*)kern, &cfg);
-  const int bn = pick_bn(ctx, MODE, a->M, a->N, max_pairs, a->b_mn != 0);
+  const int bn = pick_bn(ctx, MODE, a->M, a->N, (a->Kc + BK - 1) / BK, max_pairs, a->b_mn != 0);
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
   // which operand layouts a mode is ever launched with: the plain product with A untransposed (input gradient),
   // the dW product with B or with both untransposed
@@ -1169,9 +1192,14 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* a, int* n_partials_out
   kp.dYt = a->dYt; kp.ld_dyt = a->ld_dyt; kp.mse2c = a->mse2c; kp.act_scale = a->act_scale; kp.partials = a->partials;
   kp.V = a->V; kp.code = a->code; kp.scales = a->scales; kp.s_global = a->s_global;
   kp.adam_m = a->adam_m; kp.adam_u = a->adam_u; kp.dV = a->dV;
-  kp.beta = a->beta; kp.lam_over_n = a->lam_over_n; kp.lr = a->lr; kp.b1 = a->b1; kp.b2 = a->b2; kp.eps = a->eps;
-  kp.inv_bc1 = a->inv_bc1; kp.inv_bc2 = a->inv_bc2; kp.opt = a->opt;
-  kp.wsoft_next = a->wsoft_next; kp.beta_next = a->beta_next;
+  kp.bl = a->beta * 1.44269504088896341f; kp.hbl = -0.5f * kp.bl;
+  kp.sbeta = 0.5f * a->beta * a->act_scale;
+  kp.lam4 = -4.f * a->lam_over_n;
+  kp.b1 = a->b1; kp.b2 = a->b2; kp.c1 = 1.f - a->b1; kp.c2 = 1.f - a->b2; kp.eps = a->eps;
+  kp.nstep = a->opt == 1 ? -(a->lr * a->inv_bc1) : -a->lr;
+  kp.rbc2 = sqrtf(a->inv_bc2);
+  kp.nbl_next = -(a->beta_next * 1.4426950408889634f); kp.hbl_next = -0.5f * kp.nbl_next;
+  kp.wsoft_next = a->wsoft_next;
   kp.fin_counter = a->fin_counter; kp.fin_mse_partials = a->fin_mse_partials; kp.fin_n_mse = a->fin_n_mse;
   kp.fin_scale_mse = a->fin_scale_mse; kp.fin_scale_round = a->fin_scale_round; kp.fin_out2 = a->fin_out2;
   // the BWD epilogue forms row offsets of up to 7 rows in 32-bit element counts (the entry points refuse
