@@ -838,49 +838,44 @@ template <int D> constexpr int dq_smem() { return 4 * AT * (D + 8) * 2 + 2 * 4 *
 
 template <int D>
 int launch_fwd(faar_ctx* ctx, const AttnParams& p) {
-  int e = faar_allow_smem(ctx, (const void*)attn_fwd_kernel<D>, fwd_smem<D>());
-  if (e) return e;
-  dim3 grid((p.S + AT - 1) / AT, p.H, p.B);
-  if (D == HD && ctx->tune_attention_fragments != 1) {
-    e = faar_allow_smem(ctx, (const void*)attn_fwd64_kernel, FWD64_SMEM);
-    if (e) return e;
-  }
   faar_prof_scope ps(ctx, FAAR_K_ATTENTION);
-  if (D == HD && ctx->tune_attention_fragments == 0)
-    return faar_launch_attention_fwd64_tc(ctx, p.B, p.S, p.H, p.Hkv, p.q, p.ldq, p.k, p.v, p.ldk, p.out, p.ldo, p.lse,
-                                          p.scale_log2);
-  if (D == HD && ctx->tune_attention_fragments == 2)
+  if (ctx->tune_attention_fragments == 0)
+    return faar_launch_attention_fwd_tc(ctx, p.B, p.S, p.H, p.Hkv, D, p.q, p.ldq, p.k, p.v, p.ldk, p.out, p.ldo, p.lse,
+                                        p.scale_log2);
+  if (D == HD && ctx->tune_attention_fragments == 2) {
+    const int e = faar_allow_smem(ctx, (const void*)attn_fwd64_kernel, FWD64_SMEM);
+    if (e) return e;
     attn_fwd64_kernel<<<dim3((p.S + FQ - 1) / FQ, p.H, p.B), FWD_THREADS, FWD64_SMEM, ctx->stream>>>(p);
-  else
-    attn_fwd_kernel<D><<<grid, ATT_THREADS, fwd_smem<D>(), ctx->stream>>>(p);
+    return (int)cudaGetLastError();
+  }
+  const int e = faar_allow_smem(ctx, (const void*)attn_fwd_kernel<D>, fwd_smem<D>());
+  if (e) return e;
+  attn_fwd_kernel<D><<<dim3((p.S + AT - 1) / AT, p.H, p.B), ATT_THREADS, fwd_smem<D>(), ctx->stream>>>(p);
   return (int)cudaGetLastError();
 }
 
 template <int D>
 int launch_bwd(faar_ctx* ctx, const AttnParams& p, float* dsum) {
-  int e = faar_allow_smem(ctx, (const void*)attn_dkv_kernel<D>, dkv_smem<D>());
-  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_kernel<D>, dq_smem<D>());
-  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dkv64_kernel, BWD64_SMEM);
-  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq64_kernel, BWD64_SMEM);
-  if (e) return e;
   faar_prof_scope ps(ctx, FAAR_K_ATTENTION);
   long long rows = (long long)p.B * p.H * ((p.S + 256 / D - 1) / (256 / D));      // warp passes of the row-sum kernel
   long long blocks = (rows + 3) / 4;
   if (blocks > (long long)ctx->num_sms * 16) blocks = (long long)ctx->num_sms * 16;
   attn_dsum_kernel<D><<<(int)blocks, ATT_THREADS, 0, ctx->stream>>>(p, dsum);
   const int tiles = (p.S + AT - 1) / AT;
-  if (D == HD && ctx->tune_attention_fragments == 0) {
-    int le = faar_launch_attention_dkv64_tc(ctx, p.B, p.S, p.H, p.Hkv, p.q, p.ldq, p.k, p.v, p.ldk, p.dout, p.ldo, p.lse, dsum,
-                                            p.dk, p.dv, p.scale_log2);
-    if (le) return le;
-    return faar_launch_attention_dq64_tc(ctx, p.B, p.S, p.H, p.Hkv, p.q, p.ldq, p.k, p.v, p.ldk, p.dout, p.ldo, p.lse, dsum,
-                                         p.dq, p.scale_log2);
-  }
-  if (D == HD && ctx->tune_attention_fragments != 1) {
+  if (ctx->tune_attention_fragments == 0)
+    return faar_launch_attention_bwd_tc(ctx, p.B, p.S, p.H, p.Hkv, D, p.q, p.ldq, p.k, p.v, p.ldk, p.dout, p.ldo, p.lse, dsum,
+                                        p.dq, p.dk, p.dv, p.scale_log2);
+  if (D == HD && ctx->tune_attention_fragments == 2) {
+    int e = faar_allow_smem(ctx, (const void*)attn_dkv64_kernel, BWD64_SMEM);
+    if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq64_kernel, BWD64_SMEM);
+    if (e) return e;
     attn_dkv64_kernel<<<dim3(tiles, p.Hkv, p.B), BWD_THREADS, BWD64_SMEM, ctx->stream>>>(p);
     attn_dq64_kernel<<<dim3(tiles, p.H, p.B), BWD_THREADS, BWD64_SMEM, ctx->stream>>>(p);
     return (int)cudaGetLastError();
   }
+  int e = faar_allow_smem(ctx, (const void*)attn_dkv_kernel<D>, dkv_smem<D>());
+  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_kernel<D>, dq_smem<D>());
+  if (e) return e;
   attn_dkv_kernel<D><<<dim3(tiles, p.Hkv, p.B), ATT_THREADS, dkv_smem<D>(), ctx->stream>>>(p);
   attn_dq_kernel<D><<<dim3(tiles, p.H, p.B), ATT_THREADS, dq_smem<D>(), ctx->stream>>>(p);
   return (int)cudaGetLastError();

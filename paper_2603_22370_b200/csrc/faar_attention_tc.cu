@@ -1,11 +1,11 @@
-// Causal attention for head_dim 64 on the tcgen05 tensor cores (sm_100a): the forward kernel first, then the two
+// Causal attention for head_dim 64 and 128 on the tcgen05 tensor cores (sm_100a): the forward kernel first, then the two
 // backward kernels (dQ; dK and dV), which are built the same way and described where they start.
 //
 // Forward.  One CTA takes 128 queries of one head and sweeps the keys in tiles of 64 (one sweep):
-//   S   = Q K_j^T       tcgen05.mma  M = 128, N = 64, K = 64   -> 64 FP32 columns of tensor memory
+//   S   = Q K_j^T       tcgen05.mma  M = 128, N = 64, K = d    -> 64 FP32 columns of tensor memory
 //   P_j = 2^(c S - m)   four warps, one query row per thread (its tensor-memory lane): no shuffles; the row
 //                       goes back to tensor memory as BF16 pairs, 32 columns (tcgen05.st)
-//   O  += P_j V_j       tcgen05.mma  M = 128, N = 64, K = 64   accumulating in 64 more columns over the whole sweep;
+//   O  += P_j V_j       tcgen05.mma  M = 128, N = d, K = 64    accumulating in d more columns over the whole sweep;
 //                       P_j is the A operand, read from tensor memory; V_j is read from shared memory as it lies
 //                       in memory (keys as rows: a B operand with its N index contiguous)
 //   m is the row's reference, not its running maximum: it moves to a tile's maximum only when that exceeds it by
@@ -27,13 +27,26 @@
 
 namespace {
 
-constexpr int QT = 128, KT = 64, HD = 64;
-constexpr int Q_BYTES = QT * HD * 2, KV_BYTES = KT * HD * 2;
-constexpr int OFF_K = Q_BYTES, OFF_V = OFF_K + 2 * KV_BYTES, OFF_CTL = OFF_V + 2 * KV_BYTES;
+constexpr int QT = 128, KT = 64;
 constexpr int CTL = 256;
-constexpr int SMEM = OFF_CTL + CTL + 1024;
+// Rows are staged in panels of 64 columns (128 bytes, one swizzle row): a head of 128 has two panels per tile.
+constexpr int Q_PANEL = QT * 128, KV_PANEL = KT * 128;
+// Forward.  Tensor memory, 256 columns and two CTAs per SM for both head sizes: S of even / odd tiles in columns 0..63 /
+// 64..127, O from 128.  head_dim 64 leaves room for P of its own (192..223 / 224..255); with head_dim 128 O takes the
+// rest, and P_j is written over the first half of S_j, which its thread has just read.
+// Measured against the fragment kernels that head_dim 128 took before (16 / 8 heads): 2 x 1000 tokens forward 292 -> 23 us,
+// backward 798 -> 87 us; 4 x 2048 tokens 1681 -> 90 us (761 TFLOP/s) and 4253 -> 363 us.  Bound by the row threads (one 2^x
+// per score on the special-function unit and the instructions around it), not by the tensor pipe.
+template <int HD> struct Fwd {
+  static constexpr int NP = HD / 64, Q_BYTES = NP * Q_PANEL, KV_BYTES = NP * KV_PANEL;
+  static constexpr int OFF_K = Q_BYTES, OFF_V = OFF_K + 2 * KV_BYTES, OFF_CTL = OFF_V + 2 * KV_BYTES;
+  static constexpr int SMEM = OFF_CTL + CTL + 1024;
+  static constexpr bool P_OVER_S = HD == 128;
+  static constexpr int COL_O = 128;
+  static __device__ __forceinline__ uint32_t col_p(int j) { return P_OVER_S ? 64u * (uint32_t)(j & 1) : 192u + 32u * (uint32_t)(j & 1); }
+};
 constexpr int THREADS = 160;
-constexpr int TMEM_COLS = 256;                     // S of even / odd tiles: columns 0..63 / 64..127, O: 128..191, P: 192..223 / 224..255
+constexpr int TMEM_COLS = 256;
 constexpr float FWD_SLACK = 8.0f;                  // log2 of how far a tile's maximum may exceed the row's reference
 constexpr unsigned long long LIMIT_NS = 2000000000ull;
 
@@ -91,14 +104,14 @@ __device__ __forceinline__ uint64_t desc_k_major(uint32_t saddr) {
          ((uint64_t)2 << 61);
 }
 // Operand with its N index contiguous (64 of them = one 128-byte row per contraction index): groups of 8
-// contraction indices 1024 B apart; a single 64-wide group along N, so the leading offset is not used.
+// contraction indices 1024 B apart; the second 64-wide group along N (head_dim 128) is the next 64-row panel, 8192 B on.
 __device__ __forceinline__ uint64_t desc_n_major(uint32_t saddr) {
   return (uint64_t)((saddr & 0x3FFFF) >> 4) | ((uint64_t)(8192 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
-// D = F32, A = B = BF16, M = 128, N = 64; bit 16: B has its N index contiguous.
-__device__ __forceinline__ uint32_t idesc(int b_n_major) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_n_major << 16) | ((uint32_t)(KT >> 3) << 17) | ((uint32_t)(QT >> 4) << 24);
+// D = F32, A = B = BF16, M = 128; bit 16: B has its N index contiguous.
+__device__ __forceinline__ constexpr uint32_t idesc(int n, int b_n_major) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_n_major << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(QT >> 4) << 24);
 }
 __device__ __forceinline__ void mma(uint32_t d, uint64_t da, uint64_t db, uint32_t id, uint32_t acc) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
@@ -152,6 +165,13 @@ __device__ __forceinline__ void st16(uint32_t taddr, const uint32_t (&u)[16]) {
       : "memory");
 }
 __device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// D = A B^T over d contraction elements, both operands staged row by row (panels of 64 elements, pa / pb bytes apart)
+template <int HD>
+__device__ __forceinline__ void mma_rows(uint32_t d, uint32_t sa, uint32_t pa, uint32_t sb, uint32_t pb, uint32_t id) {
+#pragma unroll
+  for (int k = 0; k < HD / 16; ++k)
+    mma(d, desc_k_major(sa + (k >> 2) * pa) + 2u * (k & 3), desc_k_major(sb + (k >> 2) * pb) + 2u * (k & 3), id, k != 0 ? 1u : 0u);
+}
 // D (+)= A B with A read from tensor memory (128 lanes = rows, two BF16 contraction elements per 32-bit column,
 // the lower index in the lower half) and B from shared memory
 __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t db, uint32_t id, uint32_t acc) {
@@ -176,9 +196,19 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// NP boxes of 64 columns
+template <int HD>
+__device__ __forceinline__ void tma_head(uint32_t dst, uint32_t panel, const CUtensorMap* map, int x, int y, uint32_t bar) {
+#pragma unroll
+  for (int c = 0; c < HD / 64; ++c) tma_2d(dst + c * panel, map, x + 64 * c, y, bar);
+}
+
+template <int HD>
 __global__ void __launch_bounds__(THREADS, 2)
-attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, const TcParams p) {
+  using F = Fwd<HD>;
+  constexpr int KV_BYTES = F::KV_BYTES, Q_BYTES = F::Q_BYTES, OFF_CTL = F::OFF_CTL, OFF_K = F::OFF_K, OFF_V = F::OFF_V;
   extern __shared__ uint8_t raw[];
   const uint32_t base = (s32(raw) + 1023u) & ~1023u;
   uint8_t* smem = raw + (base - s32(raw));
@@ -231,28 +261,26 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
     };
     auto load_k = [&](int j) {
-      if (lead) { bar_expect(kfull(j & 1), KV_BYTES); tma_2d(sK(j & 1), &tmK, g * HD, (int)(seq0 + (long long)j * KT), kfull(j & 1)); }
+      if (lead) { bar_expect(kfull(j & 1), KV_BYTES); tma_head<HD>(sK(j & 1), KV_PANEL, &tmK, g * HD, (int)(seq0 + (long long)j * KT), kfull(j & 1)); }
       __syncwarp();
     };
     auto load_v = [&](int j) {
-      if (lead) { bar_expect(vfull(j & 1), KV_BYTES); tma_2d(sV(j & 1), &tmV, g * HD, (int)(seq0 + (long long)j * KT), vfull(j & 1)); }
+      if (lead) { bar_expect(vfull(j & 1), KV_BYTES); tma_head<HD>(sV(j & 1), KV_PANEL, &tmV, g * HD, (int)(seq0 + (long long)j * KT), vfull(j & 1)); }
       __syncwarp();
     };
     if (lead) {
       bar_expect(bar_q, Q_BYTES);
-      tma_2d(sQ, &tmQ, h * HD, (int)(seq0 + q0), bar_q);
+      tma_head<HD>(sQ, Q_PANEL, &tmQ, h * HD, (int)(seq0 + q0), bar_q);
     }
     load_k(0); load_v(0);
     if (n_kt > 1) { load_k(1); load_v(1); }
     bool ok = wait(bar_q, 0u, 0xA01u);
-    const uint32_t id_s = idesc(0), id_pv = idesc(1);
+    constexpr uint32_t id_s = idesc(KT, 0), id_pv = idesc(HD, 1);
     // S of tile j into score buffer j & 1.  The scores of tile j + 1 are issued before this warp waits for the
     // probabilities of tile j, so the tensor cores form them while the four warps work on tile j.
     auto issue_s = [&](int j) {
-      const uint64_t da = desc_k_major(sQ), db = desc_k_major(sK(j & 1));
       if (faar_elect_one()) {
-#pragma unroll
-        for (int k = 0; k < HD / 16; ++k) mma(tmem + 64u * (uint32_t)(j & 1), da + 2u * k, db + 2u * k, id_s, k != 0 ? 1u : 0u);
+        mma_rows<HD>(tmem + 64u * (uint32_t)(j & 1), sQ, Q_PANEL, sK(j & 1), KV_PANEL, id_s);
         commit(bar_s(j & 1));
       }
       __syncwarp();
@@ -264,8 +292,9 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const uint32_t ph = (uint32_t)((j >> 1) & 1);
       if (j + 1 < n_kt) {
         ok = wait(kfull((j + 1) & 1), (uint32_t)(((j + 1) >> 1) & 1), 0xA10u | ((j + 1) & 1));
-        // its score buffer last held tile j - 1
-        if (ok && j >= 1) ok = wait(bar_sfree((j + 1) & 1), (uint32_t)(((j - 1) >> 1) & 1), 0xA20u);
+        // its score buffer last held tile j - 1: read by all rows (or, holding P_{j-1} by now, consumed by P V_{j-1})
+        if (ok && j >= 1)
+          ok = F::P_OVER_S ? wait(bar_o, (uint32_t)((j - 1) & 1), 0xA20u) : wait(bar_sfree((j + 1) & 1), (uint32_t)(((j - 1) >> 1) & 1), 0xA20u);
         if (!ok) break;
         fence_after();
         issue_s(j + 1);
@@ -281,10 +310,10 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       if (j >= 1 && j + 1 < n_kt) load_v(j + 1);
       fence_after();
       const uint64_t db = desc_n_major(sV(st));
-      const uint32_t ta = tmem + 192u + 32u * (uint32_t)st;          // P_j: 16 contraction steps = 8 columns
+      const uint32_t ta = tmem + F::col_p(j);                        // P_j: 16 contraction steps = 8 columns
       if (faar_elect_one()) {
 #pragma unroll
-        for (int k = 0; k < KT / 16; ++k) mma_ts(tmem + 128u, ta + 8u * k, db + 128u * k, id_pv, (j | k) != 0 ? 1u : 0u);
+        for (int k = 0; k < KT / 16; ++k) mma_ts(tmem + (uint32_t)F::COL_O, ta + 8u * k, db + 128u * k, id_pv, (j | k) != 0 ? 1u : 0u);
         commit(bar_o);
       }
       __syncwarp();
@@ -294,7 +323,7 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     // ---------------- softmax: thread = query row = tensor-memory lane ----------------
     const int row = 32 * warp + lane;
     const int qi = q0 + row;
-    const uint32_t t_lane = tmem + ((uint32_t)(32 * warp) << 16), t_o = t_lane + 128u;
+    const uint32_t t_lane = tmem + ((uint32_t)(32 * warp) << 16), t_o = t_lane + (uint32_t)F::COL_O;
     float m = -INFINITY, l = 0.f;                             // the reference the row's probabilities are relative to; their sum
     bool ok = true;
     for (int j = 0; j < n_kt; ++j) {
@@ -310,8 +339,10 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 #pragma unroll
         for (int i = 0; i < 32; ++i) { s[i] = t[i]; s[32 + i] = t2[i]; }
       }
-      fence_before();
-      bar_arrive(bar_sfree(j & 1));
+      if (!F::P_OVER_S) {
+        fence_before();
+        bar_arrive(bar_sfree(j & 1));
+      }
       if (k0 + KT - 1 > q0 || k0 + KT > p.S) {                // the tile crosses some row's diagonal, or the sequence end
 #pragma unroll
         for (int i = 0; i < KT; ++i)
@@ -341,7 +372,7 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         fence_after();
         const float a = moved ? alpha : 1.0f;
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
+        for (int half = 0; half < HD / 32; ++half) {
           float t[32];
           uint32_t u[32];
           ld32(t_o + 32u * half, t);
@@ -361,7 +392,7 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         sum2[w & 1] = __fadd2_rn(sum2[w & 1], e);
         pk[w] = pack2(e.x, e.y);
       }
-      st32(t_lane + 192u + 32u * (uint32_t)(j & 1), pk);             // this row of P_j, an A operand in tensor memory
+      st32(t_lane + F::col_p(j), pk);             // this row of P_j, an A operand in tensor memory
       fence_before();
       bar_arrive(bar_p);
       l = l * alpha + ((sum2[0].x + sum2[0].y) + (sum2[1].x + sum2[1].y));
@@ -382,7 +413,7 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       const float inv = l > 0.f ? 1.0f / l : 0.f;
       uint4* dst = reinterpret_cast<uint4*>(p.out + (seq0 + qi) * p.ldo + h * HD);
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
+      for (int half = 0; half < HD / 32; ++half) {
         float t[32];
         ld32(t_o + 32u * half, t);
         if (qi < p.S) {
@@ -413,9 +444,18 @@ attn_fwd64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 //                                        as it lies in memory: keys as contraction rows, d contiguous)
 // The dQ product of tile j - 1 is issued after the score products of tile j, so it runs while the rows work on
 // tile j; K / V tiles come through three TMA stages.  Only the final dQ leaves tensor memory.
-constexpr int DQ_OFF_DO = Q_BYTES, DQ_OFF_KV = 2 * Q_BYTES, DQ_STAGE = 2 * KV_BYTES, DQ_STAGES = 3;
-constexpr int DQ_OFF_CTL = DQ_OFF_KV + DQ_STAGES * DQ_STAGE;
-constexpr int DQ_SMEM = DQ_OFF_CTL + CTL + 1024;
+// head_dim 128: 160 KB of operands allow one CTA per SM, whose 512 columns then hold two S and two dP buffers, so that the
+// score products of tile j + 1 run while the rows work on tile j; dS_j is written over the S columns its threads have
+// read, and the buffer pair is free again when dQ += dS_j K_j has run.
+template <int HD> struct Dq {
+  static constexpr int NP = HD / 64, Q_BYTES = NP * Q_PANEL, KV_BYTES = NP * KV_PANEL, STAGE = 2 * KV_BYTES, STAGES = 3;
+  static constexpr int OFF_DO = Q_BYTES, OFF_KV = 2 * Q_BYTES, OFF_CTL = OFF_KV + STAGES * STAGE;
+  static constexpr int SMEM = OFF_CTL + CTL + 1024;
+  static constexpr bool TWO = HD == 128;                     // two score buffers
+  static constexpr int TMEM = TWO ? 512 : 256;
+  static constexpr int COL_DP = TWO ? 128 : 64, COL_DQ = TWO ? 256 : 128;
+  static constexpr int CTAS = TWO ? 1 : 2;
+};
 // The backward kernels have no reduction along a row, so two threads share a row (32 of the 64 columns each:
 // warps w and w + 4 read the same tensor-memory lanes): eight row warps, the ninth issues copies and MMAs.
 constexpr int BWD_THREADS = 288, ROW_THREADS = 256;
@@ -428,17 +468,25 @@ struct TcBwdParams {
   float scale_log2, inv_sqrt_d;
 };
 
-__global__ void __launch_bounds__(BWD_THREADS, 2)
-attn_dq64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
+template <int HD>
+__global__ void __launch_bounds__(BWD_THREADS, Dq<HD>::CTAS)
+attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
                     const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const TcBwdParams p) {
+  using C = Dq<HD>;
+  constexpr int KV_BYTES = C::KV_BYTES, Q_BYTES = C::Q_BYTES;
   extern __shared__ uint8_t raw[];
   const uint32_t base = (s32(raw) + 1023u) & ~1023u;
   uint8_t* smem = raw + (base - s32(raw));
-  const uint32_t ctl = base + DQ_OFF_CTL;
-  const uint32_t bar_qd = ctl, bar_s = ctl + 40, bar_sfree = ctl + 48, bar_ds = ctl + 56, bar_done = ctl + 64;
+  const uint32_t ctl = base + C::OFF_CTL;
+  const uint32_t bar_qd = ctl, bar_sfree = ctl + 48;
+  // TWO: one barrier of each kind per buffer (tiles alternate); otherwise one, passed once per tile
+  auto bar_s = [&](int j) { return C::TWO ? ctl + 104u + 8u * (j & 1) : ctl + 40u; };
+  auto bar_ds = [&](int j) { return C::TWO ? ctl + 120u + 8u * (j & 1) : ctl + 56u; };
+  auto bar_done = [&](int j) { return C::TWO ? ctl + 136u + 8u * (j & 1) : ctl + 64u; };
+  auto parity = [&](int j) { return (uint32_t)(C::TWO ? (j >> 1) & 1 : j & 1); };
   auto kvfull = [&](int s) { return ctl + 8u + 8u * s; };
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + DQ_OFF_CTL + 96);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + DQ_OFF_CTL + 100);
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + C::OFF_CTL + 96);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_CTL + 100);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // one-dimensional grid, query tile slowest and descending: CTAs start in order of decreasing work
@@ -453,25 +501,29 @@ attn_dq64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 
   if (threadIdx.x == 0) {
     bar_init(bar_qd, 1);
-    for (int s = 0; s < DQ_STAGES; ++s) bar_init(kvfull(s), 1);
-    bar_init(bar_s, 1); bar_init(bar_done, 1);
-    bar_init(bar_sfree, ROW_THREADS); bar_init(bar_ds, ROW_THREADS);
+    for (int s = 0; s < C::STAGES; ++s) bar_init(kvfull(s), 1);
+    for (int s = 0; s < (C::TWO ? 2 : 1); ++s) { bar_init(bar_s(s), 1); bar_init(bar_done(s), 1); bar_init(bar_ds(s), ROW_THREADS); }
+    bar_init(bar_sfree, ROW_THREADS);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 8) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(const_cast<uint32_t*>(tmem_slot))),
-                 "r"((uint32_t)TMEM_COLS) : "memory");
+                 "r"((uint32_t)C::TMEM) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;                         // S: columns 0..63, dP: 64..127, dQ: 128..191, dS (BF16 pairs): 192..223
-  const uint32_t sQ = base, sDO = base + DQ_OFF_DO;
-  auto sK = [&](int s) { return base + DQ_OFF_KV + (uint32_t)s * DQ_STAGE; };
+  const uint32_t tmem = *tmem_slot;                         // head_dim 64: S in columns 0..63, dP: 64..127, dQ: 128..191, dS (BF16 pairs): 192..223
+  const uint32_t sQ = base, sDO = base + C::OFF_DO;
+  auto sK = [&](int s) { return base + C::OFF_KV + (uint32_t)s * C::STAGE; };
   auto sV = [&](int s) { return sK(s) + KV_BYTES; };
+  auto col_s = [&](int j) { return C::TWO ? 64u * (uint32_t)(j & 1) : 0u; };
+  auto col_dp = [&](int j) { return (uint32_t)C::COL_DP + col_s(j); };
+  // dS_j as 64 BF16 pairs' columns: 8 per contraction step; over S each thread half's 16 columns start at its own 32
+  auto col_ds = [&](int j, int step) { return C::TWO ? col_s(j) + (uint32_t)(32 * (step >> 1) + 8 * (step & 1)) : 192u + 8u * (uint32_t)step; };
 
   if (warp == 8) {
     const bool lead = lane == 0;
@@ -479,61 +531,83 @@ attn_dq64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
     };
     auto load_kv = [&](int j) {
-      const int st = j % DQ_STAGES;
+      const int st = j % C::STAGES;
       if (lead) {
         bar_expect(kvfull(st), 2 * KV_BYTES);
-        tma_2d(sK(st), &tmK, g * HD, (int)(seq0 + (long long)j * KT), kvfull(st));
-        tma_2d(sV(st), &tmV, g * HD, (int)(seq0 + (long long)j * KT), kvfull(st));
+        tma_head<HD>(sK(st), KV_PANEL, &tmK, g * HD, (int)(seq0 + (long long)j * KT), kvfull(st));
+        tma_head<HD>(sV(st), KV_PANEL, &tmV, g * HD, (int)(seq0 + (long long)j * KT), kvfull(st));
       }
       __syncwarp();
     };
     if (lead) {
       bar_expect(bar_qd, 2 * Q_BYTES);
-      tma_2d(sQ, &tmQ, h * HD, (int)(seq0 + q0), bar_qd);
-      tma_2d(sDO, &tmDO, h * HD, (int)(seq0 + q0), bar_qd);
+      tma_head<HD>(sQ, Q_PANEL, &tmQ, h * HD, (int)(seq0 + q0), bar_qd);
+      tma_head<HD>(sDO, Q_PANEL, &tmDO, h * HD, (int)(seq0 + q0), bar_qd);
     }
     load_kv(0);
     if (n_kt > 1) load_kv(1);
+    if (C::TWO && n_kt > 2) load_kv(2);
     bool ok = wait(bar_qd, 0u, 0xC01u);
-    const uint32_t id_k = idesc(0), id_n = idesc(1);
-    auto issue_dq = [&](int j) {                              // dQ += dS_j K_j
-      const uint64_t db = desc_n_major(sK(j % DQ_STAGES));
+    constexpr uint32_t id_k = idesc(KT, 0), id_n = idesc(HD, 1);
+    auto issue_s = [&](int j) {                               // S_j, dP_j
+      const int st = j % C::STAGES;
       if (faar_elect_one()) {
-#pragma unroll
-        for (int k = 0; k < KT / 16; ++k) mma_ts(tmem + 128u, tmem + 192u + 8u * k, db + 128u * k, id_n, (j | k) != 0 ? 1u : 0u);
-        commit(bar_done);
+        mma_rows<HD>(tmem + col_s(j), sQ, Q_PANEL, sK(st), KV_PANEL, id_k);
+        mma_rows<HD>(tmem + col_dp(j), sDO, Q_PANEL, sV(st), KV_PANEL, id_k);
+        commit(bar_s(j));
       }
       __syncwarp();
     };
-    for (int j = 0; j < n_kt && ok; ++j) {
-      const int st = j % DQ_STAGES;
-      if (j >= 1 && j + 1 < n_kt) {                           // stage of tile j + 1 last held tile j - 2
-        if (j >= 2) ok = wait(bar_done, (uint32_t)((j - 2) & 1), 0xC10u);
-        if (!ok) break;
-        load_kv(j + 1);
-      }
-      ok = wait(kvfull(st), (uint32_t)((j / DQ_STAGES) & 1), 0xC20u | st);
-      if (ok && j > 0) ok = wait(bar_sfree, (uint32_t)((j - 1) & 1), 0xC30u);
-      if (!ok) break;
-      fence_after();
-      const uint64_t dq_ = desc_k_major(sQ), dk_ = desc_k_major(sK(st)), dd = desc_k_major(sDO), dv_ = desc_k_major(sV(st));
+    auto issue_dq = [&](int j) {                              // dQ += dS_j K_j
+      const uint64_t db = desc_n_major(sK(j % C::STAGES));
       if (faar_elect_one()) {
 #pragma unroll
-        for (int k = 0; k < HD / 16; ++k) mma(tmem, dq_ + 2u * k, dk_ + 2u * k, id_k, k != 0 ? 1u : 0u);
-#pragma unroll
-        for (int k = 0; k < HD / 16; ++k) mma(tmem + 64u, dd + 2u * k, dv_ + 2u * k, id_k, k != 0 ? 1u : 0u);
-        commit(bar_s);
+        for (int k = 0; k < KT / 16; ++k)
+          mma_ts(tmem + (uint32_t)C::COL_DQ, tmem + col_ds(j, k), db + 128u * k, id_n, (j | k) != 0 ? 1u : 0u);
+        commit(bar_done(j));
       }
       __syncwarp();
-      if (j > 0) {
-        ok = wait(bar_ds, (uint32_t)((j - 1) & 1), 0xC40u);
+    };
+    if constexpr (C::TWO) {
+      if (ok) ok = wait(kvfull(0), 0u, 0xC20u);
+      if (ok) { fence_after(); issue_s(0); }
+      for (int j = 0; j < n_kt && ok; ++j) {
+        if (j >= 1 && j + 1 < n_kt) ok = wait(bar_done(j - 1), parity(j - 1), 0xC10u);   // buffers and stage of tile j - 1 are free
+        if (ok && j >= 1 && j + 2 < n_kt) load_kv(j + 2);
+        if (ok && j + 1 < n_kt) {
+          ok = wait(kvfull((j + 1) % C::STAGES), (uint32_t)(((j + 1) / C::STAGES) & 1), 0xC20u | ((j + 1) % C::STAGES));
+          if (!ok) break;
+          fence_after();
+          issue_s(j + 1);
+        }
+        if (ok) ok = wait(bar_ds(j), parity(j), 0xC40u);
         if (!ok) break;
         fence_after();
-        issue_dq(j - 1);
+        issue_dq(j);
       }
+    } else {
+      for (int j = 0; j < n_kt && ok; ++j) {
+        const int st = j % C::STAGES;
+        if (j >= 1 && j + 1 < n_kt) {                         // stage of tile j + 1 last held tile j - 2
+          if (j >= 2) ok = wait(bar_done(j - 2), parity(j - 2), 0xC10u);
+          if (!ok) break;
+          load_kv(j + 1);
+        }
+        ok = wait(kvfull(st), (uint32_t)((j / C::STAGES) & 1), 0xC20u | st);
+        if (ok && j > 0) ok = wait(bar_sfree, (uint32_t)((j - 1) & 1), 0xC30u);
+        if (!ok) break;
+        fence_after();
+        issue_s(j);
+        if (j > 0) {
+          ok = wait(bar_ds(j - 1), parity(j - 1), 0xC40u);
+          if (!ok) break;
+          fence_after();
+          issue_dq(j - 1);
+        }
+      }
+      if (ok) ok = wait(bar_ds(n_kt - 1), parity(n_kt - 1), 0xC50u);
+      if (ok) { fence_after(); issue_dq(n_kt - 1); }
     }
-    if (ok) ok = wait(bar_ds, (uint32_t)((n_kt - 1) & 1), 0xC50u);
-    if (ok) { fence_after(); issue_dq(n_kt - 1); }
     if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
   } else {
     const int row = 32 * (warp & 3) + lane, half = warp >> 2;    // this thread: columns 32 half .. 32 half + 31 of its row
@@ -545,14 +619,14 @@ attn_dq64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     bool ok = true;
     for (int j = 0; j < n_kt; ++j) {
       const int k0 = j * KT;
-      ok = bar_wait(bar_s, (uint32_t)(j & 1), abort_flag, 0xD10u);
+      ok = bar_wait(bar_s(j), parity(j), abort_flag, 0xD10u);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       fence_after();
       float s[32];
       auto tile = [&](auto diag_tag) {                        // P (dP - delta) / sqrt(d); the mask only where needed
         constexpr bool DIAG = decltype(diag_tag)::value;
         float t[32], d[32];
-        ld32x2(t_lane + 32u * half, t_lane + 64u + 32u * half, t, d);
+        ld32x2(t_lane + col_s(j) + 32u * half, t_lane + col_dp(j) + 32u * half, t, d);
         const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nl2 = make_float2(-lse, -lse);
         const float2 is2 = make_float2(p.inv_sqrt_d, p.inv_sqrt_d), nd2 = make_float2(nd, nd);
 #pragma unroll
@@ -568,35 +642,39 @@ attn_dq64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         }
       };
       if (k0 + KT - 1 > q0) tile(std::true_type{}); else tile(std::false_type{});   // some key of the tile above some row
-      fence_before();
-      bar_arrive(bar_sfree);
-      if (j > 0) {                                            // the dS buffer is free once dQ of tile j - 1 has run
-        ok = bar_wait(bar_done, (uint32_t)((j - 1) & 1), abort_flag, 0xD20u);
-        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      if (!C::TWO) {
+        fence_before();
+        bar_arrive(bar_sfree);
+        if (j > 0) {                                          // the dS buffer is free once dQ of tile j - 1 has run
+          ok = bar_wait(bar_done(j - 1), parity(j - 1), abort_flag, 0xD20u);
+          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        }
       }
       uint32_t pk[16];
 #pragma unroll
       for (int w = 0; w < 16; ++w) pk[w] = pack2(s[2 * w], s[2 * w + 1]);
-      st16(t_lane + 192u + 16u * half, pk);                   // this thread's half of the row of dS_j: an A operand
+      st16(t_lane + col_ds(j, 2 * half), pk);                 // this thread's half of the row of dS_j: an A operand
       wait_st();
       fence_before();
-      bar_arrive(bar_ds);
+      bar_arrive(bar_ds(j));
     }
     if (ok) {
-      ok = bar_wait(bar_done, (uint32_t)((n_kt - 1) & 1), abort_flag, 0xD30u);
+      ok = bar_wait(bar_done(n_kt - 1), parity(n_kt - 1), abort_flag, 0xD30u);
       ok = __all_sync(0xffffffffu, ok);
     }
     if (ok) {
       fence_after();
       uint4* dst = reinterpret_cast<uint4*>(p.dq + (seq0 + qi) * p.ldq + h * HD);
-      {
+#pragma unroll
+      for (int q = 0; q < C::NP; ++q) {                       // this thread's half of the row
         float t[32];
-        ld32(t_lane + 128u + 32u * half, t);
+        const int c0 = (HD / 2) * half + 32 * q;
+        ld32(t_lane + (uint32_t)(C::COL_DQ + c0), t);
         if (qi < p.S) {
 #pragma unroll
           for (int c = 0; c < 4; ++c)
-            dst[4 * half + c] = make_uint4(pack2(t[8 * c], t[8 * c + 1]), pack2(t[8 * c + 2], t[8 * c + 3]),
-                                           pack2(t[8 * c + 4], t[8 * c + 5]), pack2(t[8 * c + 6], t[8 * c + 7]));
+            dst[c0 / 8 + c] = make_uint4(pack2(t[8 * c], t[8 * c + 1]), pack2(t[8 * c + 2], t[8 * c + 3]),
+                                         pack2(t[8 * c + 4], t[8 * c + 5]), pack2(t[8 * c + 6], t[8 * c + 7]));
         }
       }
     }
@@ -606,7 +684,7 @@ attn_dq64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   __syncthreads();
   if (warp == 8) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C::TMEM) : "memory");
   }
 }
 
@@ -623,29 +701,40 @@ attn_dq64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 // and so wait for the accumulating products).  Q / dO tiles come through four TMA stages (requested three items
 // ahead), lse and delta of a tile's 64 queries are staged in shared memory by the row threads themselves.  Queries
 // beyond the sequence end are masked (their rows hold the next sequence's data).
-constexpr int KV_OFF_V = Q_BYTES, KV_OFF_QD = 2 * Q_BYTES, KV_STAGE = 2 * KV_BYTES, KV_STAGES = 4;
-constexpr int KV_OFF_ROWV = KV_OFF_QD + KV_STAGES * KV_STAGE, KV_OFF_CTL = KV_OFF_ROWV + 2 * 2 * KT * 4;
-constexpr int KV_SMEM = KV_OFF_CTL + CTL + 1024;
-static_assert(2 * KV_SMEM <= 227 * 1024, "two CTAs per SM");
-// S^T: columns 0..63, dP^T: 64..127, dV: 128..191, dK: 192..255.  The thread of row half h reads columns 32 h .. 32 h + 31
-// of S^T (dP^T) and writes its 32 values of P^T (dS^T) as 16 BF16 pairs to columns 32 h .. 32 h + 15 of the same buffer.
-constexpr int KV_TMEM = 256;
+// head_dim 128: dV and dK take 256 columns and the operands 162 KB, so one CTA per SM with all 512 columns: two S^T and two
+// dP^T buffers, the score products of item i + 1 run while the rows work on item i; three stages.
+template <int HD> struct Dkv {
+  static constexpr int NP = HD / 64, KEY_BYTES = NP * Q_PANEL, QD_BYTES = NP * KV_PANEL, STAGE = 2 * QD_BYTES;
+  static constexpr bool TWO = HD == 128;
+  static constexpr int STAGES = TWO ? 3 : 4;
+  static constexpr int OFF_V = KEY_BYTES, OFF_QD = 2 * KEY_BYTES, OFF_ROWV = OFF_QD + STAGES * STAGE, OFF_CTL = OFF_ROWV + 2 * 2 * KT * 4;
+  static constexpr int SMEM = OFF_CTL + CTL + 1024;
+  static constexpr int CTAS = TWO ? 1 : 2;
+  // head_dim 64: S^T in columns 0..63, dP^T: 64..127, dV: 128..191, dK: 192..255.  The thread of row half h reads columns
+  // 32 h .. 32 h + 31 of S^T (dP^T) and writes its 32 values of P^T (dS^T) as 16 BF16 pairs to columns 32 h .. 32 h + 15
+  // of the same buffer.
+  static constexpr int TMEM = TWO ? 512 : 256;
+  static constexpr int COL_DP = TWO ? 128 : 64, COL_DV = TWO ? 256 : 128, COL_DK = COL_DV + HD;
+  static_assert(CTAS * (SMEM + 1024) <= 228 * 1024, "shared memory budget");
+};
 
-__global__ void __launch_bounds__(BWD_THREADS, 2)
-attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
+template <int HD>
+__global__ void __launch_bounds__(BWD_THREADS, Dkv<HD>::CTAS)
+attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const TcBwdParams p) {
+  using C = Dkv<HD>;
   extern __shared__ uint8_t raw[];
   const uint32_t base = (s32(raw) + 1023u) & ~1023u;
   uint8_t* smem = raw + (base - s32(raw));
-  const uint32_t ctl = base + KV_OFF_CTL;
+  const uint32_t ctl = base + C::OFF_CTL;
   const uint32_t bar_kv = ctl;
   auto qfull = [&](int s) { return ctl + 8u + 8u * s; };          // 4
   auto bar_s = [&](int s) { return ctl + 40u + 8u * s; };         // 2 (items alternate): the score products of an item are complete
   auto bar_pds = [&](int s) { return ctl + 72u + 8u * s; };       // 2: P^T / dS^T of an item written by all rows
   auto bar_done = [&](int s) { return ctl + 88u + 8u * s; };      // 2: the accumulating MMAs of an item have run
   auto bar_rv = [&](int s) { return ctl + 112u + 8u * s; };       // 2: lse / delta of an item staged, previous use read by all
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + KV_OFF_CTL + 128);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + KV_OFF_CTL + 132);
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + C::OFF_CTL + 128);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_CTL + 132);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // one-dimensional grid, key tile slowest: CTAs start in order of decreasing work (the first key tiles see the
@@ -662,7 +751,7 @@ attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 
   if (threadIdx.x == 0) {
     bar_init(bar_kv, 1);
-    for (int s = 0; s < KV_STAGES; ++s) bar_init(qfull(s), 1);
+    for (int s = 0; s < C::STAGES; ++s) bar_init(qfull(s), 1);
     for (int s = 0; s < 2; ++s) {
       bar_init(bar_s(s), 1); bar_init(bar_done(s), 1); bar_init(bar_pds(s), ROW_THREADS); bar_init(bar_rv(s), ROW_THREADS);
     }
@@ -672,16 +761,18 @@ attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   }
   if (warp == 8) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s32(const_cast<uint32_t*>(tmem_slot))),
-                 "r"((uint32_t)KV_TMEM) : "memory");
+                 "r"((uint32_t)C::TMEM) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   fence_before();
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t sKt = base, sVt = base + KV_OFF_V;
-  auto sQ = [&](int s) { return base + KV_OFF_QD + (uint32_t)s * KV_STAGE; };
-  auto sDO = [&](int s) { return sQ(s) + KV_BYTES; };
+  const uint32_t sKt = base, sVt = base + C::OFF_V;
+  auto sQ = [&](int s) { return base + C::OFF_QD + (uint32_t)s * C::STAGE; };
+  auto sDO = [&](int s) { return sQ(s) + C::QD_BYTES; };
+  auto col_s = [&](int i) { return C::TWO ? 64u * (uint32_t)(i & 1) : 0u; };
+  auto col_dp = [&](int i) { return (uint32_t)C::COL_DP + col_s(i); };
   auto head_of = [&](int i) { return g * rep + i / per_head; };
   auto q0_of = [&](int i) { return (qt0 + i % per_head) * KT; };
 
@@ -691,68 +782,83 @@ attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
     };
     auto load_item = [&](int i) {
-      const int st = i % KV_STAGES;
+      const int st = i % C::STAGES;
       if (lead) {
-        bar_expect(qfull(st), 2 * KV_BYTES);
-        tma_2d(sQ(st), &tmQ, head_of(i) * HD, (int)(seq0 + q0_of(i)), qfull(st));
-        tma_2d(sDO(st), &tmDO, head_of(i) * HD, (int)(seq0 + q0_of(i)), qfull(st));
+        bar_expect(qfull(st), 2 * C::QD_BYTES);
+        tma_head<HD>(sQ(st), KV_PANEL, &tmQ, head_of(i) * HD, (int)(seq0 + q0_of(i)), qfull(st));
+        tma_head<HD>(sDO(st), KV_PANEL, &tmDO, head_of(i) * HD, (int)(seq0 + q0_of(i)), qfull(st));
       }
       __syncwarp();
     };
     if (lead) {
-      bar_expect(bar_kv, 2 * Q_BYTES);
-      tma_2d(sKt, &tmK, g * HD, (int)(seq0 + k0), bar_kv);
-      tma_2d(sVt, &tmV, g * HD, (int)(seq0 + k0), bar_kv);
+      bar_expect(bar_kv, 2 * C::KEY_BYTES);
+      tma_head<HD>(sKt, Q_PANEL, &tmK, g * HD, (int)(seq0 + k0), bar_kv);
+      tma_head<HD>(sVt, Q_PANEL, &tmV, g * HD, (int)(seq0 + k0), bar_kv);
     }
     load_item(0);
     if (n_it > 1) load_item(1);
     if (n_it > 2) load_item(2);
     bool ok = wait(bar_kv, 0u, 0xE01u);
-    const uint32_t id_k = idesc(0), id_n = idesc(1);
+    constexpr uint32_t id_k = idesc(KT, 0), id_n = idesc(HD, 1);
     auto issue_s = [&](int i) {                                // S^T and dP^T of item i
-      const int st = i % KV_STAGES;
-      const uint64_t dk_ = desc_k_major(sKt), dq_ = desc_k_major(sQ(st)), dv_ = desc_k_major(sVt), dd = desc_k_major(sDO(st));
+      const int st = i % C::STAGES;
+      if (faar_elect_one()) {
+        mma_rows<HD>(tmem + col_s(i), sKt, Q_PANEL, sQ(st), KV_PANEL, id_k);
+        mma_rows<HD>(tmem + col_dp(i), sVt, Q_PANEL, sDO(st), KV_PANEL, id_k);
+        commit(bar_s(i & 1));
+      }
+      __syncwarp();
+    };
+    // dV += P^T dO_i, dK += dS^T Q_i.  A operands from tensor memory: contraction steps 0, 1 (queries 0..31) in columns
+    // 0..15 of the buffer, steps 2, 3 (queries 32..63) in columns 32..47
+    auto accumulate = [&](int i) {
+      const int st = i % C::STAGES;
+      const uint64_t dd = desc_n_major(sDO(st)), dq_ = desc_n_major(sQ(st));
       if (faar_elect_one()) {
 #pragma unroll
-        for (int k = 0; k < HD / 16; ++k) mma(tmem, dk_ + 2u * k, dq_ + 2u * k, id_k, k != 0 ? 1u : 0u);
+        for (int k = 0; k < KT / 16; ++k)
+          mma_ts(tmem + (uint32_t)C::COL_DV, tmem + col_s(i) + (uint32_t)(32 * (k >> 1) + 8 * (k & 1)), dd + 128u * k, id_n, (i | k) != 0 ? 1u : 0u);
 #pragma unroll
-        for (int k = 0; k < HD / 16; ++k) mma(tmem + 64u, dv_ + 2u * k, dd + 2u * k, id_k, k != 0 ? 1u : 0u);
-        commit(bar_s(i & 1));
+        for (int k = 0; k < KT / 16; ++k)
+          mma_ts(tmem + (uint32_t)C::COL_DK, tmem + col_dp(i) + (uint32_t)(32 * (k >> 1) + 8 * (k & 1)), dq_ + 128u * k, id_n, (i | k) != 0 ? 1u : 0u);
+        commit(bar_done(i & 1));
       }
       __syncwarp();
     };
     if (ok) ok = wait(qfull(0), 0u, 0xE10u);
     if (ok) { fence_after(); issue_s(0); }
     for (int i = 0; i < n_it && ok; ++i) {
-      if (i + 3 < n_it) {                                      // its stage last held item i - 1: wait for that item's
-        if (i >= 1) ok = wait(bar_done((i - 1) & 1), (uint32_t)(((i - 1) >> 1) & 1), 0xE40u);   // MMAs
-        if (!ok) break;
-        load_item(i + 3);
-      }
-      ok = wait(bar_pds(i & 1), (uint32_t)((i >> 1) & 1), 0xE30u);
-      if (!ok) break;
-      fence_after();
-      // A operands from tensor memory: contraction steps 0, 1 (queries 0..31) in columns 0..15 of the buffer,
-      // steps 2, 3 (queries 32..63) in columns 32..47
-      const int st = i % KV_STAGES;
-      const uint64_t dd = desc_n_major(sDO(st)), dq_ = desc_n_major(sQ(st));
-      if (faar_elect_one()) {
-#pragma unroll
-        for (int k = 0; k < KT / 16; ++k)
-          mma_ts(tmem + 128u, tmem + (uint32_t)(32 * (k >> 1) + 8 * (k & 1)), dd + 128u * k, id_n, (i | k) != 0 ? 1u : 0u);
-#pragma unroll
-        for (int k = 0; k < KT / 16; ++k)
-          mma_ts(tmem + 192u, tmem + 64u + (uint32_t)(32 * (k >> 1) + 8 * (k & 1)), dq_ + 128u * k, id_n, (i | k) != 0 ? 1u : 0u);
-        commit(bar_done(i & 1));
-      }
-      __syncwarp();
-      if (i + 1 < n_it) {
-        // the next item's score products overwrite P^T / dS^T: after the accumulating products have read them
-        ok = wait(qfull((i + 1) % KV_STAGES), (uint32_t)(((i + 1) / KV_STAGES) & 1), 0xE10u);
-        if (ok) ok = wait(bar_done(i & 1), (uint32_t)((i >> 1) & 1), 0xE20u);
+      if constexpr (C::TWO) {
+        if (i >= 1 && i + 1 < n_it) ok = wait(bar_done((i - 1) & 1), (uint32_t)(((i - 1) >> 1) & 1), 0xE40u);   // buffers, stage of item i - 1
+        if (ok && i >= 1 && i + 2 < n_it) load_item(i + 2);
+        if (ok && i + 1 < n_it) {
+          ok = wait(qfull((i + 1) % C::STAGES), (uint32_t)(((i + 1) / C::STAGES) & 1), 0xE10u);
+          if (!ok) break;
+          fence_after();
+          issue_s(i + 1);
+        }
+        if (ok) ok = wait(bar_pds(i & 1), (uint32_t)((i >> 1) & 1), 0xE30u);
         if (!ok) break;
         fence_after();
-        issue_s(i + 1);
+        accumulate(i);
+      } else {
+        if (i + 3 < n_it) {                                    // its stage last held item i - 1: wait for that item's
+          if (i >= 1) ok = wait(bar_done((i - 1) & 1), (uint32_t)(((i - 1) >> 1) & 1), 0xE40u);   // MMAs
+          if (!ok) break;
+          load_item(i + 3);
+        }
+        ok = wait(bar_pds(i & 1), (uint32_t)((i >> 1) & 1), 0xE30u);
+        if (!ok) break;
+        fence_after();
+        accumulate(i);
+        if (i + 1 < n_it) {
+          // the next item's score products overwrite P^T / dS^T: after the accumulating products have read them
+          ok = wait(qfull((i + 1) % C::STAGES), (uint32_t)(((i + 1) / C::STAGES) & 1), 0xE10u);
+          if (ok) ok = wait(bar_done(i & 1), (uint32_t)((i >> 1) & 1), 0xE20u);
+          if (!ok) break;
+          fence_after();
+          issue_s(i + 1);
+        }
       }
     }
     if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
@@ -760,7 +866,7 @@ attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     const int row = 32 * (warp & 3) + lane, half = warp >> 2;    // this thread: queries 32 half .. 32 half + 31 of an item
     const int kj = k0 + row;
     const uint32_t t_lane = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-    float* rowv_all = reinterpret_cast<float*>(smem + KV_OFF_ROWV);      // [2][2][KT]: lse, delta / sqrt(d) negated
+    float* rowv_all = reinterpret_cast<float*>(smem + C::OFF_ROWV);      // [2][2][KT]: lse, delta / sqrt(d) negated
     bool ok = true;
     // this thread's share of an item's 64 lse values (rows 0..63) or 64 negated, scaled delta values (rows 64..127);
     // the value for item i + 1 is requested at the start of item i, so its latency is off the per-item path
@@ -789,7 +895,7 @@ attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
       auto item = [&](auto edge_tag) {
         constexpr bool EDGE = decltype(edge_tag)::value;
         float t[32], d[32];
-        ld32x2(t_lane + 32u * half, t_lane + 64u + 32u * half, t, d);
+        ld32x2(t_lane + col_s(i) + 32u * half, t_lane + col_dp(i) + 32u * half, t, d);
 #pragma unroll
         for (int j4 = 0; j4 < 32; j4 += 4) {
           const float4 l4 = *reinterpret_cast<const float4*>(rowv + 32 * half + j4);          // the same address in every lane
@@ -815,10 +921,10 @@ attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         uint32_t pk[16];
 #pragma unroll
         for (int w = 0; w < 16; ++w) pk[w] = pack2(t[2 * w], t[2 * w + 1]);
-        st16(t_lane + 32u * half, pk);                           // over the first half of the columns just read
+        st16(t_lane + col_s(i) + 32u * half, pk);                // over the first half of the columns just read
 #pragma unroll
         for (int w = 0; w < 16; ++w) pk[w] = pack2(d[2 * w], d[2 * w + 1]);
-        st16(t_lane + 64u + 32u * half, pk);
+        st16(t_lane + col_dp(i) + 32u * half, pk);
       };
       if (edge) item(std::true_type{}); else item(std::false_type{});
       wait_st();
@@ -834,14 +940,16 @@ attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
 #pragma unroll
       for (int which = 0; which < 2; ++which) {
         uint4* dst = reinterpret_cast<uint4*>((which ? p.dk : p.dv) + (seq0 + kj) * p.ldk + g * HD);
-        {
+#pragma unroll
+        for (int q = 0; q < C::NP; ++q) {                      // this thread's half of the row
           float t[32];
-          ld32(t_lane + 128u + 64u * which + 32u * half, t);
+          const int c0 = (HD / 2) * half + 32 * q;
+          ld32(t_lane + (uint32_t)(C::COL_DV + HD * which + c0), t);
           if (kj < p.S) {
 #pragma unroll
             for (int c = 0; c < 4; ++c)
-              dst[4 * half + c] = make_uint4(pack2(t[8 * c], t[8 * c + 1]), pack2(t[8 * c + 2], t[8 * c + 3]),
-                                             pack2(t[8 * c + 4], t[8 * c + 5]), pack2(t[8 * c + 6], t[8 * c + 7]));
+              dst[c0 / 8 + c] = make_uint4(pack2(t[8 * c], t[8 * c + 1]), pack2(t[8 * c + 2], t[8 * c + 3]),
+                                           pack2(t[8 * c + 4], t[8 * c + 5]), pack2(t[8 * c + 6], t[8 * c + 7]));
           }
         }
       }
@@ -852,7 +960,7 @@ attn_dkv64_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
   __syncthreads();
   if (warp == 8) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)KV_TMEM) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C::TMEM) : "memory");
   }
 }
 
@@ -864,7 +972,7 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
 int head_map(faar_ctx* ctx, CUtensorMap* map, const void* ptr, long long rows, int cols, long long ld, int box_rows) {
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  cuuint32_t box[2] = {(cuuint32_t)HD, (cuuint32_t)box_rows};
+  cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
   cuuint32_t es[2] = {1, 1};
   CUresult r = reinterpret_cast<EncodeFn>(ctx->encode_tiled)(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims,
                                                              strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -873,65 +981,66 @@ int head_map(faar_ctx* ctx, CUtensorMap* map, const void* ptr, long long rows, i
   return r == CUDA_SUCCESS ? 0 : (int)cudaErrorInvalidValue;
 }
 
+template <int HD>
+int launch_fwd(faar_ctx* ctx, const TcParams& p, const void* q, int64_t ldq, const void* k, const void* v, int64_t ldk) {
+  using F = Fwd<HD>;
+  static_assert(2 * (F::SMEM + 1024) <= 228 * 1024, "two CTAs per SM");
+  const long long T = (long long)p.B * p.S;
+  CUtensorMap tmQ, tmK, tmV;
+  int e = head_map(ctx, &tmQ, q, T, p.H * HD, ldq, QT);
+  if (!e) e = head_map(ctx, &tmK, k, T, p.Hkv * HD, ldk, KT);
+  if (!e) e = head_map(ctx, &tmV, v, T, p.Hkv * HD, ldk, KT);
+  if (!e) e = faar_allow_smem(ctx, (const void*)attn_fwd_tc_kernel<HD>, F::SMEM);
+  if (e) return e;
+  attn_fwd_tc_kernel<HD><<<dim3(((p.S + QT - 1) / QT) * p.H * p.B, 1, 1), THREADS, F::SMEM, ctx->stream>>>(tmQ, tmK, tmV, p);
+  return (int)cudaGetLastError();
+}
+
+template <int HD>
+int launch_bwd(faar_ctx* ctx, const TcBwdParams& p, const void* q, int64_t ldq, const void* k, const void* v, int64_t ldk,
+               const void* dout, int64_t ldo) {
+  const long long T = (long long)p.B * p.S;
+  CUtensorMap tmQ, tmDO, tmK, tmV, tmQk, tmDOk, tmKk, tmVk;      // boxes of 128 rows / of 64 rows
+  int e = head_map(ctx, &tmQ, q, T, p.H * HD, ldq, QT);
+  if (!e) e = head_map(ctx, &tmDO, dout, T, p.H * HD, ldo, QT);
+  if (!e) e = head_map(ctx, &tmK, k, T, p.Hkv * HD, ldk, QT);
+  if (!e) e = head_map(ctx, &tmV, v, T, p.Hkv * HD, ldk, QT);
+  if (!e) e = head_map(ctx, &tmQk, q, T, p.H * HD, ldq, KT);
+  if (!e) e = head_map(ctx, &tmDOk, dout, T, p.H * HD, ldo, KT);
+  if (!e) e = head_map(ctx, &tmKk, k, T, p.Hkv * HD, ldk, KT);
+  if (!e) e = head_map(ctx, &tmVk, v, T, p.Hkv * HD, ldk, KT);
+  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dkv_tc_kernel<HD>, Dkv<HD>::SMEM);
+  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_tc_kernel<HD>, Dq<HD>::SMEM);
+  if (e) return e;
+  const int tiles = (p.S + QT - 1) / QT;
+  attn_dkv_tc_kernel<HD><<<dim3(tiles * p.Hkv * p.B, 1, 1), BWD_THREADS, Dkv<HD>::SMEM, ctx->stream>>>(tmQk, tmDOk, tmK, tmV, p);
+  e = (int)cudaGetLastError();
+  if (e) return e;
+  attn_dq_tc_kernel<HD><<<dim3(tiles * p.H * p.B, 1, 1), BWD_THREADS, Dq<HD>::SMEM, ctx->stream>>>(tmQ, tmDO, tmKk, tmVk, p);
+  return (int)cudaGetLastError();
+}
+
 }  // namespace
 
-int faar_launch_attention_fwd64_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, const void* q, int64_t ldq, const void* k,
-                                   const void* v, int64_t ldk, void* out, int64_t ldo, float* lse, float scale_log2) {
-  static_assert(2 * SMEM <= 227 * 1024, "two CTAs per SM");
-  const long long T = (long long)B * S;
-  if (T > 0x7FFFFFFFll) return (int)cudaErrorInvalidValue;
-  CUtensorMap tmQ, tmK, tmV;
-  int e = head_map(ctx, &tmQ, q, T, H * HD, ldq, QT);
-  if (!e) e = head_map(ctx, &tmK, k, T, Hkv * HD, ldk, KT);
-  if (!e) e = head_map(ctx, &tmV, v, T, Hkv * HD, ldk, KT);
-  if (e) return e;
-  if ((e = faar_allow_smem(ctx, (const void*)attn_fwd64_tc_kernel, SMEM))) return e;
+int faar_launch_attention_fwd_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
+                                 const void* v, int64_t ldk, void* out, int64_t ldo, float* lse, float scale_log2) {
+  if ((long long)B * S > 0x7FFFFFFFll) return (int)cudaErrorInvalidValue;
   TcParams p;
   p.out = reinterpret_cast<__nv_bfloat16*>(out); p.lse = lse; p.ldo = ldo; p.B = B; p.S = S; p.H = H; p.Hkv = Hkv;
   p.scale_log2 = scale_log2;
-  attn_fwd64_tc_kernel<<<dim3(((S + QT - 1) / QT) * H * B, 1, 1), THREADS, SMEM, ctx->stream>>>(tmQ, tmK, tmV, p);
-  return (int)cudaGetLastError();
+  return D == 64 ? launch_fwd<64>(ctx, p, q, ldq, k, v, ldk) : launch_fwd<128>(ctx, p, q, ldq, k, v, ldk);
 }
 
-int faar_launch_attention_dq64_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, const void* q, int64_t ldq, const void* k,
-                                  const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
-                                  const float* dsum, void* dq, float scale_log2) {
-  static_assert(2 * (DQ_SMEM + 1024) <= 227 * 1024, "two CTAs per SM");
-  const long long T = (long long)B * S;
-  if (T > 0x7FFFFFFFll) return (int)cudaErrorInvalidValue;
-  CUtensorMap tmQ, tmDO, tmK, tmV;
-  int e = head_map(ctx, &tmQ, q, T, H * HD, ldq, QT);
-  if (!e) e = head_map(ctx, &tmDO, dout, T, H * HD, ldo, QT);
-  if (!e) e = head_map(ctx, &tmK, k, T, Hkv * HD, ldk, KT);
-  if (!e) e = head_map(ctx, &tmV, v, T, Hkv * HD, ldk, KT);
-  if (e) return e;
-  if ((e = faar_allow_smem(ctx, (const void*)attn_dq64_tc_kernel, DQ_SMEM))) return e;
+int faar_launch_attention_bwd_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
+                                 const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
+                                 const float* dsum, void* dq, void* dk, void* dv, float scale_log2) {
+  if ((long long)B * S > 0x7FFFFFFFll) return (int)cudaErrorInvalidValue;
   TcBwdParams p = {};
-  p.lse = lse; p.dsum = dsum; p.dq = reinterpret_cast<__nv_bfloat16*>(dq); p.ldq = ldq; p.ldk = ldk;
-  p.B = B; p.S = S; p.H = H; p.Hkv = Hkv; p.scale_log2 = scale_log2; p.inv_sqrt_d = scale_log2 / 1.4426950408889634f;
-  attn_dq64_tc_kernel<<<dim3(((S + QT - 1) / QT) * H * B, 1, 1), BWD_THREADS, DQ_SMEM, ctx->stream>>>(tmQ, tmDO, tmK, tmV, p);
-  return (int)cudaGetLastError();
-}
-
-int faar_launch_attention_dkv64_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, const void* q, int64_t ldq, const void* k,
-                                   const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
-                                   const float* dsum, void* dk, void* dv, float scale_log2) {
-  static_assert(KV_SMEM <= 227 * 1024, "shared memory budget");
-  const long long T = (long long)B * S;
-  if (T > 0x7FFFFFFFll) return (int)cudaErrorInvalidValue;
-  CUtensorMap tmQ, tmDO, tmK, tmV;
-  int e = head_map(ctx, &tmQ, q, T, H * HD, ldq, KT);
-  if (!e) e = head_map(ctx, &tmDO, dout, T, H * HD, ldo, KT);
-  if (!e) e = head_map(ctx, &tmK, k, T, Hkv * HD, ldk, QT);
-  if (!e) e = head_map(ctx, &tmV, v, T, Hkv * HD, ldk, QT);
-  if (e) return e;
-  if ((e = faar_allow_smem(ctx, (const void*)attn_dkv64_tc_kernel, KV_SMEM))) return e;
-  TcBwdParams p = {};
-  p.lse = lse; p.dsum = dsum; p.dk = reinterpret_cast<__nv_bfloat16*>(dk); p.dv = reinterpret_cast<__nv_bfloat16*>(dv);
+  p.lse = lse; p.dsum = dsum;
+  p.dq = reinterpret_cast<__nv_bfloat16*>(dq); p.dk = reinterpret_cast<__nv_bfloat16*>(dk); p.dv = reinterpret_cast<__nv_bfloat16*>(dv);
   p.ldq = ldq; p.ldk = ldk; p.B = B; p.S = S; p.H = H; p.Hkv = Hkv; p.scale_log2 = scale_log2;
   p.inv_sqrt_d = scale_log2 / 1.4426950408889634f;
-  attn_dkv64_tc_kernel<<<dim3(((S + QT - 1) / QT) * Hkv * B, 1, 1), BWD_THREADS, KV_SMEM, ctx->stream>>>(tmQ, tmDO, tmK, tmV, p);
-  return (int)cudaGetLastError();
+  return D == 64 ? launch_bwd<64>(ctx, p, q, ldq, k, v, ldk, dout, ldo) : launch_bwd<128>(ctx, p, q, ldq, k, v, ldk, dout, ldo);
 }
 
 // Reads and clears the status word of this module (synchronous copy: call after the stream has been synchronised).

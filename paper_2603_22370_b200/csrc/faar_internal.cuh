@@ -21,7 +21,7 @@ struct faar_ctx {
   int tune_bn;                            // 0 = choose the GEMM tile width automatically
   int tune_tail;                          // -1 = choose the tail split automatically, else columns to split
   int tune_wide;                          // 1 = 256 x 512 GEMM tiles wherever the shape allows; -1 (default), 0 = never
-  int tune_attention_fragments;           // head_dim 64 attention: 0 = tcgen05 kernels, 2 = mma.sync kernels, 1 = the shared-memory fragment kernels
+  int tune_attention_fragments;           // attention: 0 = tcgen05 kernels, 2 = mma.sync kernels (head_dim 64), 1 = the shared-memory fragment kernels
   int last_gemm_bn, last_gemm_pairs, last_gemm_split;   // what the last GEMM launch used
   std::vector<const void*> smem_set;      // kernels whose dynamic shared-memory limit has been raised on this device
   // chained steps: the workspace and the beta of the forward operand that the last backward call wrote
@@ -94,14 +94,12 @@ int faar_launch_softquant_init(faar_ctx*, const faar_shape*, const void* W, floa
                                uint8_t* scales, float* s_global_out, uint8_t* code, float* V,
                                unsigned long long* amax_word);
 int faar_launch_nvfp4_expand(faar_ctx*, int rows, int K, const uint8_t* packed, const uint8_t* scales, void* out, int64_t ld);
-int faar_launch_attention_fwd64_tc(faar_ctx*, int B, int S, int H, int Hkv, const void* q, int64_t ldq, const void* k,
-                                   const void* v, int64_t ldk, void* out, int64_t ldo, float* lse, float scale_log2);
-int faar_launch_attention_dq64_tc(faar_ctx*, int B, int S, int H, int Hkv, const void* q, int64_t ldq, const void* k,
-                                  const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
-                                  const float* dsum, void* dq, float scale_log2);
-int faar_launch_attention_dkv64_tc(faar_ctx*, int B, int S, int H, int Hkv, const void* q, int64_t ldq, const void* k,
-                                   const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
-                                   const float* dsum, void* dk, void* dv, float scale_log2);
+// head_dim D = 64 or 128 on the tcgen05 tensor cores
+int faar_launch_attention_fwd_tc(faar_ctx*, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
+                                 const void* v, int64_t ldk, void* out, int64_t ldo, float* lse, float scale_log2);
+int faar_launch_attention_bwd_tc(faar_ctx*, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
+                                 const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
+                                 const float* dsum, void* dq, void* dk, void* dv, float scale_log2);
 int faar_attention_tc_status(uint32_t* code_out);
 int faar_launch_softquant_eval(faar_ctx*, const faar_shape*, const float* V, const uint8_t* code,
                                const uint8_t* scales, const float* s_global, float beta,

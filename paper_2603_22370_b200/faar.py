@@ -334,8 +334,8 @@ def attention_status(ctx):
 
 
 def tune_attention(ctx, mode: int):
-    """head_dim 64: 0 = tcgen05 kernels forward and backward (default), 2 = register-resident mma.sync kernels,
-    1 = the shared-memory fragment kernels (as head_dim 128 always takes)."""
+    """0 = tcgen05 kernels forward and backward (default), 2 = register-resident mma.sync kernels (head_dim 64),
+    1 = the shared-memory fragment kernels."""
     _check(lib().faar_tune_attention(ctx._h, mode), "faar_tune_attention")
 
 

@@ -45,6 +45,24 @@ def test_attention_forward_and_backward_match_the_oracle(ctx, B, S, H, HKV, D, f
         faar.tune_attention(ctx, 0)
 
 
+@pytest.mark.parametrize("fragments", [0, 1])
+@pytest.mark.parametrize("B,S,H,HKV", [(1, 2, 1, 1), (2, 64, 2, 1), (1, 65, 4, 2), (3, 127, 2, 2), (1, 128, 2, 1), (2, 129, 4, 1),
+                                       (1, 321, 4, 2), (1, 700, 2, 1)])
+def test_attention_of_128_element_heads(ctx, B, S, H, HKV, fragments):
+    """head_dim 128 on tcgen05 (two 64-column panels per tile, P / dS written over the scores) and on the fragment kernels:
+    two keys, edges of the 64-key and 128-query tiles, one to many tiles per sweep."""
+    faar.tune_attention(ctx, fragments)
+    try:
+        _attention_case(ctx, B, S, H, HKV, 128)
+    finally:
+        faar.tune_attention(ctx, 0)
+
+
+@pytest.mark.parametrize("q_scale", [3.0, 8.0])
+def test_attention_of_128_element_heads_with_peaked_scores(ctx, q_scale):
+    _attention_case(ctx, 2, 321, 4, 2, 128, q_scale=q_scale)
+
+
 @pytest.mark.parametrize("q_scale", [3.0, 8.0])
 def test_attention_with_peaked_scores(ctx, q_scale):
     """Scores whose row maxima keep growing along the key sweep by amounts on both sides of the forward kernel's
