@@ -100,6 +100,7 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
 
 __global__ void __launch_bounds__(AL_THREADS, 1)
 align_loss_kernel(const AlignParams p) {
+  faar_pdl_sync();
   __shared__ float wred[4][AL_WARPS];
   __shared__ float row[2];                                         // log2-sum-exp of the token's row: fp, q
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -249,6 +250,6 @@ int faar_launch_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const vo
   const int grid = T < ctx->num_sms ? T : ctx->num_sms;
   *n_partials = grid;
   faar_prof_scope ps(ctx, FAAR_K_ALIGN_LOSS);
-  align_loss_kernel<<<grid, AL_THREADS, 0, ctx->stream>>>(p);
+  faar_launch_pdl(ctx, align_loss_kernel, dim3(grid), dim3(AL_THREADS), 0, p);
   return (int)cudaGetLastError();
 }

@@ -54,6 +54,7 @@ __device__ __forceinline__ void load_tile(__nv_bfloat16 (*tile)[D + 8], const __
 template <int D>
 __global__ void __launch_bounds__(ATT_THREADS)
 attn_fwd_kernel(const AttnParams p) {
+  faar_pdl_sync();
   extern __shared__ __align__(128) uint8_t att_smem[];
   auto Qs = reinterpret_cast<__nv_bfloat16(*)[D + 8]>(att_smem);
   auto Ks = reinterpret_cast<__nv_bfloat16(*)[D + 8]>(att_smem + AT * (D + 8) * 2);
@@ -177,6 +178,7 @@ attn_fwd_kernel(const AttnParams p) {
 template <int D>
 __global__ void __launch_bounds__(ATT_THREADS)
 attn_dsum_kernel(const AttnParams p, float* dsum) {
+  faar_pdl_sync();
   constexpr int LPR = D / 8, RPW = 32 / LPR;                 // lanes per row, rows per warp
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sub = lane / LPR, c = (lane % LPR) * 8;
@@ -214,6 +216,7 @@ attn_dsum_kernel(const AttnParams p, float* dsum) {
 template <int D>
 __global__ void __launch_bounds__(ATT_THREADS)
 attn_dkv_kernel(const AttnParams p) {
+  faar_pdl_sync();
   extern __shared__ __align__(128) uint8_t att_smem[];
   constexpr int TILE = AT * (D + 8) * 2;
   auto Ks = reinterpret_cast<__nv_bfloat16(*)[D + 8]>(att_smem);
@@ -349,6 +352,7 @@ attn_dkv_kernel(const AttnParams p) {
 template <int D>
 __global__ void __launch_bounds__(ATT_THREADS)
 attn_dq_kernel(const AttnParams p) {
+  faar_pdl_sync();
   extern __shared__ __align__(128) uint8_t att_smem[];
   constexpr int TILE = AT * (D + 8) * 2;
   auto Qs = reinterpret_cast<__nv_bfloat16(*)[D + 8]>(att_smem);
@@ -569,6 +573,7 @@ constexpr int STAGE_ELEMS = 2 * AT * LDS;            // a K tile and a V tile; e
 constexpr int FWD64_SMEM = 3 * STAGE_ELEMS * 2;
 __global__ void __launch_bounds__(FWD_THREADS, 2)
 attn_fwd64_kernel(const AttnParams p) {
+  faar_pdl_sync();
   extern __shared__ __align__(128) uint8_t att_smem[];
   auto stage_k = [&](int s) { return reinterpret_cast<__nv_bfloat16(*)[LDS]>(att_smem) + (size_t)s * 2 * AT; };
   auto stage_v = [&](int s) { return stage_k(s) + AT; };
@@ -673,6 +678,7 @@ constexpr int BWD_THREADS = 128;
 constexpr int BWD64_SMEM = 3 * STAGE_ELEMS * 2 + 3 * 2 * AT * 4;      // three stages + their lse / dsum rows (dK, dV kernel)
 __global__ void __launch_bounds__(BWD_THREADS, 3)
 attn_dq64_kernel(const AttnParams p) {
+  faar_pdl_sync();
   extern __shared__ __align__(128) uint8_t att_smem[];
   auto stage_k = [&](int s) { return reinterpret_cast<__nv_bfloat16(*)[LDS]>(att_smem) + (size_t)s * 2 * AT; };
   auto stage_v = [&](int s) { return stage_k(s) + AT; };
@@ -749,6 +755,7 @@ attn_dq64_kernel(const AttnParams p) {
 // mask: their Q and dO rows are zero, so whatever P and dS they get adds nothing to dV or dK.
 __global__ void __launch_bounds__(BWD_THREADS, 2)
 attn_dkv64_kernel(const AttnParams p) {
+  faar_pdl_sync();
   extern __shared__ __align__(128) uint8_t att_smem[];
   auto stage_q = [&](int s) { return reinterpret_cast<__nv_bfloat16(*)[LDS]>(att_smem) + (size_t)s * 2 * AT; };
   auto stage_d = [&](int s) { return stage_q(s) + AT; };
@@ -845,12 +852,12 @@ int launch_fwd(faar_ctx* ctx, const AttnParams& p) {
   if (D == HD && ctx->tune_attention_fragments == 2) {
     const int e = faar_allow_smem(ctx, (const void*)attn_fwd64_kernel, FWD64_SMEM);
     if (e) return e;
-    attn_fwd64_kernel<<<dim3((p.S + FQ - 1) / FQ, p.H, p.B), FWD_THREADS, FWD64_SMEM, ctx->stream>>>(p);
+    faar_launch_pdl(ctx, attn_fwd64_kernel, dim3((p.S + FQ - 1) / FQ, p.H, p.B), dim3(FWD_THREADS), FWD64_SMEM, p);
     return (int)cudaGetLastError();
   }
   const int e = faar_allow_smem(ctx, (const void*)attn_fwd_kernel<D>, fwd_smem<D>());
   if (e) return e;
-  attn_fwd_kernel<D><<<dim3((p.S + AT - 1) / AT, p.H, p.B), ATT_THREADS, fwd_smem<D>(), ctx->stream>>>(p);
+  faar_launch_pdl(ctx, attn_fwd_kernel<D>, dim3((p.S + AT - 1) / AT, p.H, p.B), dim3(ATT_THREADS), fwd_smem<D>(), p);
   return (int)cudaGetLastError();
 }
 
@@ -860,7 +867,7 @@ int launch_bwd(faar_ctx* ctx, const AttnParams& p, float* dsum) {
   long long rows = (long long)p.B * p.H * ((p.S + 256 / D - 1) / (256 / D));      // warp passes of the row-sum kernel
   long long blocks = (rows + 3) / 4;
   if (blocks > (long long)ctx->num_sms * 16) blocks = (long long)ctx->num_sms * 16;
-  attn_dsum_kernel<D><<<(int)blocks, ATT_THREADS, 0, ctx->stream>>>(p, dsum);
+  faar_launch_pdl(ctx, attn_dsum_kernel<D>, dim3((int)blocks), dim3(ATT_THREADS), 0, p, dsum);
   const int tiles = (p.S + AT - 1) / AT;
   if (ctx->tune_attention_fragments == 0)
     return faar_launch_attention_bwd_tc(ctx, p.B, p.S, p.H, p.Hkv, D, p.q, p.ldq, p.k, p.v, p.ldk, p.dout, p.ldo, p.lse, dsum,
@@ -869,15 +876,15 @@ int launch_bwd(faar_ctx* ctx, const AttnParams& p, float* dsum) {
     int e = faar_allow_smem(ctx, (const void*)attn_dkv64_kernel, BWD64_SMEM);
     if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq64_kernel, BWD64_SMEM);
     if (e) return e;
-    attn_dkv64_kernel<<<dim3(tiles, p.Hkv, p.B), BWD_THREADS, BWD64_SMEM, ctx->stream>>>(p);
-    attn_dq64_kernel<<<dim3(tiles, p.H, p.B), BWD_THREADS, BWD64_SMEM, ctx->stream>>>(p);
+    faar_launch_pdl(ctx, attn_dkv64_kernel, dim3(tiles, p.Hkv, p.B), dim3(BWD_THREADS), BWD64_SMEM, p);
+    faar_launch_pdl(ctx, attn_dq64_kernel, dim3(tiles, p.H, p.B), dim3(BWD_THREADS), BWD64_SMEM, p);
     return (int)cudaGetLastError();
   }
   int e = faar_allow_smem(ctx, (const void*)attn_dkv_kernel<D>, dkv_smem<D>());
   if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_kernel<D>, dq_smem<D>());
   if (e) return e;
-  attn_dkv_kernel<D><<<dim3(tiles, p.Hkv, p.B), ATT_THREADS, dkv_smem<D>(), ctx->stream>>>(p);
-  attn_dq_kernel<D><<<dim3(tiles, p.H, p.B), ATT_THREADS, dq_smem<D>(), ctx->stream>>>(p);
+  faar_launch_pdl(ctx, attn_dkv_kernel<D>, dim3(tiles, p.Hkv, p.B), dim3(ATT_THREADS), dkv_smem<D>(), p);
+  faar_launch_pdl(ctx, attn_dq_kernel<D>, dim3(tiles, p.H, p.B), dim3(ATT_THREADS), dq_smem<D>(), p);
   return (int)cudaGetLastError();
 }
 

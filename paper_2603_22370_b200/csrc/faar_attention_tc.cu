@@ -250,6 +250,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  faar_pdl_sync();                                          // set-up done; now wait for the previous kernel's data
   const uint32_t sQ = base;
   auto sK = [&](int s) { return base + OFF_K + (uint32_t)s * KV_BYTES; };
   auto sV = [&](int s) { return base + OFF_V + (uint32_t)s * KV_BYTES; };
@@ -517,6 +518,7 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;                         // head_dim 64: S in columns 0..63, dP: 64..127, dQ: 128..191, dS (BF16 pairs): 192..223
+  faar_pdl_sync();                                          // set-up done; now wait for the previous kernel's data
   const uint32_t sQ = base, sDO = base + C::OFF_DO;
   auto sK = [&](int s) { return base + C::OFF_KV + (uint32_t)s * C::STAGE; };
   auto sV = [&](int s) { return sK(s) + KV_BYTES; };
@@ -768,6 +770,7 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  faar_pdl_sync();                                          // set-up done; now wait for the previous kernel's data
   const uint32_t sKt = base, sVt = base + C::OFF_V;
   auto sQ = [&](int s) { return base + C::OFF_QD + (uint32_t)s * C::STAGE; };
   auto sDO = [&](int s) { return sQ(s) + C::QD_BYTES; };
@@ -992,7 +995,7 @@ int launch_fwd(faar_ctx* ctx, const TcParams& p, const void* q, int64_t ldq, con
   if (!e) e = head_map(ctx, &tmV, v, T, p.Hkv * HD, ldk, KT);
   if (!e) e = faar_allow_smem(ctx, (const void*)attn_fwd_tc_kernel<HD>, F::SMEM);
   if (e) return e;
-  attn_fwd_tc_kernel<HD><<<dim3(((p.S + QT - 1) / QT) * p.H * p.B, 1, 1), THREADS, F::SMEM, ctx->stream>>>(tmQ, tmK, tmV, p);
+  faar_launch_pdl(ctx, attn_fwd_tc_kernel<HD>, dim3(((p.S + QT - 1) / QT) * p.H * p.B, 1, 1), dim3(THREADS), F::SMEM, tmQ, tmK, tmV, p);
   return (int)cudaGetLastError();
 }
 
@@ -1013,10 +1016,10 @@ int launch_bwd(faar_ctx* ctx, const TcBwdParams& p, const void* q, int64_t ldq, 
   if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_tc_kernel<HD>, Dq<HD>::SMEM);
   if (e) return e;
   const int tiles = (p.S + QT - 1) / QT;
-  attn_dkv_tc_kernel<HD><<<dim3(tiles * p.Hkv * p.B, 1, 1), BWD_THREADS, Dkv<HD>::SMEM, ctx->stream>>>(tmQk, tmDOk, tmK, tmV, p);
+  faar_launch_pdl(ctx, attn_dkv_tc_kernel<HD>, dim3(tiles * p.Hkv * p.B, 1, 1), dim3(BWD_THREADS), Dkv<HD>::SMEM, tmQk, tmDOk, tmK, tmV, p);
   e = (int)cudaGetLastError();
   if (e) return e;
-  attn_dq_tc_kernel<HD><<<dim3(tiles * p.H * p.B, 1, 1), BWD_THREADS, Dq<HD>::SMEM, ctx->stream>>>(tmQ, tmDO, tmKk, tmVk, p);
+  faar_launch_pdl(ctx, attn_dq_tc_kernel<HD>, dim3(tiles * p.H * p.B, 1, 1), dim3(BWD_THREADS), Dq<HD>::SMEM, tmQ, tmDO, tmKk, tmVk, p);
   return (int)cudaGetLastError();
 }
 

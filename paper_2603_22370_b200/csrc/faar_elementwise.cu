@@ -29,7 +29,7 @@ __device__ __forceinline__ int64_t w_offset(int64_t g, uint32_t groups_per_row, 
 template <bool BF16IN>
 __global__ void __launch_bounds__(EW_THREADS)
 amax_kernel(const void* __restrict__ W, int O, int K, int64_t ldw, unsigned long long* amax_word, uint32_t epoch) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel waits for this one's end itself
+  faar_pdl_sync();
   const uint32_t groups_per_row = K / 8;
   const int64_t total = (int64_t)O * groups_per_row;
   const bool dense = ldw == K;
@@ -293,7 +293,7 @@ softquant_init_kernel(const void* __restrict__ W, int O, int K, int64_t ldw,
                       uint8_t* __restrict__ scales, float* __restrict__ s_global_out,
                       uint8_t* __restrict__ code, float* __restrict__ V) {
   __shared__ uint4 stage[EW_THREADS * 4];
-  asm volatile("griddepcontrol.wait;" ::: "memory");      // the maximum (and W itself) may come from the kernel before
+  faar_pdl_sync();                                        // the maximum (and W itself) may come from the kernel before
   const float s_global = tensor_scale(s_global_in, amax_word);
   if (blockIdx.x == 0 && threadIdx.x == 0) *s_global_out = s_global;
   const float d = __fmul_rn(s_global, 6.0f);
@@ -340,34 +340,37 @@ softquant_init_kernel(const void* __restrict__ W, int O, int K, int64_t ldw,
 // magnitude (Eq. 7 applied to the initial position).  The output holds sign * node * block scale, which
 // needs at most 7 significant bits and is therefore exact in BF16; the FP32 tensor scale stays outside
 // (X_q = Xq_units * s_global) and is applied by the GEMM epilogues.
-// From the bracket: t = [v >= 0.5] (v - 0.5 is a multiple of 2^-25, so a saturating FMA by 2^25 gives 0 or 1),
-// node = (j + t) * spacing, magnitude code = k + t.
-template <bool FAST>
-__device__ __forceinline__ void nearest_block(const float (&w)[16], float s, float sg, uint32_t (&o)[8], uint32_t (&cw)[2]) {
-  float q[16];
-  block_quotients<FAST>(w, s, q);
+// The nearest node comes from the hardware conversion to E2M1, which rounds ties to the even code; setting the lowest
+// mantissa bit of the quotient first turns that into ties to the larger magnitude: every midpoint of the grid has that
+// bit clear, so a quotient on a midpoint moves above it, and one below a midpoint stays below.  The codes convert back
+// to F16 pairs (nodes exactly); shifting the magnitude bits right by three makes them BF16 values scaled by 2^-112 (the
+// difference of the exponent biases), which the block scale times 2^112 undoes in one exact packed product.
+// 42 -> 14 thread instructions per value: [4096, 8192] 54 -> 29 us (153 MB; the maximum pass excluded), now bound by HBM.
+__device__ __forceinline__ uint32_t to_e2m1x2(float lo, float hi) {             // one byte: lo in bits 3:0
+  uint32_t r;
+  asm("{\n\t.reg .b8 b;\n\tcvt.rn.satfinite.e2m1x2.f32 b, %1, %2;\n\tcvt.u32.u8 %0, b;\n\t}" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+__device__ __forceinline__ uint32_t e2m1x2_to_f16x2(uint32_t byte) {
+  uint32_t r;
+  asm("{\n\t.reg .b8 b;\n\tcvt.u8.u32 b, %1;\n\tcvt.rn.f16x2.e2m1x2 %0, b;\n\t}" : "=r"(r) : "r"(byte));
+  return r;
+}
+__device__ __forceinline__ void nearest_block(const float (&q)[16], float sg, uint32_t (&o)[8], uint32_t (&cw)[2]) {
+  const uint32_t sgb = __float_as_uint(sg * 0x1p112f);                          // at most 4 significant bits: the high half
+  const uint32_t sg2w = __byte_perm(sgb, sgb, 0x3232);
+  const __nv_bfloat162 sg2 = *reinterpret_cast<const __nv_bfloat162*>(&sg2w);
+  uint32_t by[8];
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    float n[8];
-#pragma unroll
-    for (int i = 0; i < 8; i += 2) {
-      float out[2];
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int x = 8 * h + i + e;
-        const grid_pos g = locate(q[x]);
-        const float t = __saturatef(__fmaf_rn(g.v, 0x1p25f, 1.0f - 0x1p24f));
-        const float neg = negative_flag<FAST>(w[x], q[x]);
-        n[i + e] = __fmaf_rn(8.0f, neg, __fadd_rn(g.k, t));
-        const float spacing_sg = __fmul_rn(__fmaf_rn(0.5f, g.t1, __fadd_rn(0.5f, g.t2)), sg);   // {.5, 1, 2} * sg
-        const float mag = __fmul_rn(__fadd_rn(g.j, t), spacing_sg);                          // exact: 3 x 4 bits at most
-        out[e] = __fmul_rn(mag, __fmaf_rn(-2.0f, neg, 1.0f));
-      }
-      // both values have zero low halves: the BF16 pair is the two high halves
-      o[(8 * h + i) >> 1] = __byte_perm(__float_as_uint(out[0]), __float_as_uint(out[1]), 0x7632);
-    }
-    cw[h] = pack_nibbles(n);
+  for (int i = 0; i < 8; ++i) {
+    by[i] = to_e2m1x2(__uint_as_float(__float_as_uint(q[2 * i]) | 1u), __uint_as_float(__float_as_uint(q[2 * i + 1]) | 1u));
+    const uint32_t h = e2m1x2_to_f16x2(by[i]);
+    const uint32_t b = ((h >> 3) & 0x0FFF0FFFu) | (h & 0x80008000u);
+    const __nv_bfloat162 x = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&b), sg2);
+    o[i] = *reinterpret_cast<const uint32_t*>(&x);
   }
+  cw[0] = __byte_perm(__byte_perm(by[0], by[1], 0x0040), __byte_perm(by[2], by[3], 0x0040), 0x5410);
+  cw[1] = __byte_perm(__byte_perm(by[4], by[5], 0x0040), __byte_perm(by[6], by[7], 0x0040), 0x5410);
 }
 
 __global__ void __launch_bounds__(EW_THREADS, 3)
@@ -375,7 +378,7 @@ act_fakequant_kernel(const __nv_bfloat16* __restrict__ X, int T, int K, int64_t 
                      const unsigned long long* __restrict__ amax_word, __nv_bfloat16* __restrict__ Xq, int64_t ldq,
                      float* __restrict__ s_global_out, uint8_t* __restrict__ packed, uint8_t* __restrict__ scales) {
   __shared__ uint4 stage[EW_THREADS * 2];
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  faar_pdl_sync();
   const float s_global = tensor_scale(s_global_in, amax_word);
   if (blockIdx.x == 0 && threadIdx.x == 0) *s_global_out = s_global;
   const float d = __fmul_rn(s_global, 6.0f);
@@ -402,8 +405,17 @@ act_fakequant_kernel(const __nv_bfloat16* __restrict__ X, int T, int K, int64_t 
     uint32_t cw[2];
     uint4 oq[2];
     uint32_t(&o)[8] = *reinterpret_cast<uint32_t(*)[8]>(oq);
-    if (fast_division_ok(s, amax, has_minute)) nearest_block<true>(w, s, sg, o, cw);
-    else nearest_block<false>(w, s, sg, o, cw);
+    float q[16];
+    // a quotient far below the smallest midpoint need not be exact, so minute values take the fast path here (and -0.0
+    // becomes +0.0 in its residual corrections)
+    if (fast_division_ok(s, amax, false)) {
+      block_quotients<true>(w, s, q);
+    } else {
+      block_quotients<false>(w, s, q);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) q[i] = copysignf(q[i], w[i] < 0.f ? -1.0f : 1.0f);
+    }
+    nearest_block(q, sg, o, cw);
     if (dense_out) {
       const int64_t warp_first = b0 + (threadIdx.x & ~31);
       if (warp_first < total) {
@@ -428,6 +440,7 @@ act_fakequant_kernel(const __nv_bfloat16* __restrict__ X, int T, int K, int64_t 
 __global__ void __launch_bounds__(EW_THREADS)
 nvfp4_expand_kernel(const uint8_t* __restrict__ packed, const uint8_t* __restrict__ scales, int rows, int K,
                     __nv_bfloat16* __restrict__ out, int64_t ld) {
+  faar_pdl_sync();
   const uint32_t blocks_per_row = K / 16;
   const int64_t total = (int64_t)rows * blocks_per_row;
   for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < total; b += (int64_t)gridDim.x * blockDim.x) {
@@ -530,6 +543,7 @@ softquant_eval_kernel(const float* __restrict__ V, const uint8_t* __restrict__ c
 // ---- Round Loss partial sums ------------------------------------------------------------
 __global__ void __launch_bounds__(EW_THREADS)
 round_partials_kernel(const float* __restrict__ V, int64_t N, float* __restrict__ partials) {
+  faar_pdl_sync();
   float acc = 0.f;
   const int64_t n4 = N / 4;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
@@ -557,6 +571,7 @@ round_partials_kernel(const float* __restrict__ V, int64_t N, float* __restrict_
 __global__ void __launch_bounds__(256)
 finalize_kernel(const float* __restrict__ p0, int n0, float scale0, float* out0,
                 const float* __restrict__ p1, int n1, float scale1, float* out1) {
+  faar_pdl_sync();
   __shared__ double sh[256];
   for (int which = 0; which < 2; ++which) {
     const float* p = which ? p1 : p0;
@@ -582,6 +597,7 @@ harden_pack_kernel(const float* __restrict__ V, const uint8_t* __restrict__ code
                    const uint8_t* __restrict__ scales, const float* __restrict__ s_global_p,
                    int64_t n_groups, uint8_t* __restrict__ packed, uint8_t* __restrict__ scales_out,
                    uint8_t* __restrict__ decisions, void* __restrict__ W_final, int wfinal_dtype) {
+  faar_pdl_sync();
   const float s_global = W_final ? *s_global_p : 0.f;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n_groups;
        g += (int64_t)gridDim.x * blockDim.x) {
@@ -629,23 +645,52 @@ harden_pack_kernel(const float* __restrict__ V, const uint8_t* __restrict__ code
 
 // ---- block scales into the tiled order of block-scaled tensor-core GEMMs ----------------------------
 // Output: 128 x 4 tiles of 512 bytes, tiles of a row band first; byte (r, c) of a tile at
-// (r % 32) * 16 + (r / 32) * 4 + c; rows and columns beyond the matrix are zero.  One thread per output
-// 4-byte word (the four columns of one row of one tile).
+// (r % 32) * 16 + (r / 32) * 4 + c; rows and columns beyond the matrix are zero.  One CTA per 128 rows x 64 columns: rows
+// come in as 16-byte vectors where the row pitch allows, pass through shared memory (pitch 17 words: the reads of a
+// warp, one column of 32 rows, fall on 32 banks) and leave as the 8 KB of 16 consecutive tiles, 16 bytes per thread
+// (rows r, r + 32, r + 64, r + 96).  One thread per 4-byte word, reading 4 bytes of a row each, took 10.4 us for
+// [4096, 512] (2 MB), this 3.9 us.
+constexpr int SZ_COLS = 64, SZ_PITCH = SZ_COLS / 4 + 1;
 __global__ void __launch_bounds__(EW_THREADS)
-swizzle_scales_kernel(const uint8_t* __restrict__ in, int rows, int cols, uint32_t* __restrict__ out, int64_t n_words) {
-  const int col_tiles = (cols + 3) / 4;
-  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n_words; w += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t tile = w >> 7;
-    const int in_tile = (int)(w & 127);                 // (r % 32) * 4 + r / 32
-    const int r = (int)(tile / col_tiles) * 128 + (in_tile & 3) * 32 + (in_tile >> 2);
-    const int c0 = (int)(tile % col_tiles) * 4;
-    uint32_t v = 0;
-    if (r < rows) {
+swizzle_scales_kernel(const uint8_t* __restrict__ in, int rows, int cols, uint32_t* __restrict__ out, int col_tiles) {
+  __shared__ uint32_t tile[128 * SZ_PITCH];
+  const int r0 = blockIdx.y * 128, c0 = blockIdx.x * SZ_COLS;
+  const bool vec = cols % 16 == 0 && (reinterpret_cast<uintptr_t>(in) & 15) == 0;
+  const bool out_vec = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+  faar_pdl_sync();
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (c0 + j < cols) v |= (uint32_t)in[(int64_t)r * cols + c0 + j] << (8 * j);
+  for (int i = 0; i < 2; ++i) {
+    const int idx = threadIdx.x + EW_THREADS * i, r = idx >> 2, c = c0 + 16 * (idx & 3);
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (r0 + r < rows && c < cols) {
+      const uint8_t* src = in + (int64_t)(r0 + r) * cols + c;
+      if (vec) {
+        v = *reinterpret_cast<const uint4*>(src);
+      } else {
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (c + j < cols) w[j >> 2] |= (uint32_t)src[j] << (8 * (j & 3));
+        v = make_uint4(w[0], w[1], w[2], w[3]);
+      }
     }
-    out[w] = v;
+    uint32_t* t = tile + r * SZ_PITCH + 4 * (idx & 3);
+    t[0] = v.x; t[1] = v.y; t[2] = v.z; t[3] = v.w;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int idx = threadIdx.x + EW_THREADS * i, ct = idx >> 5, r = idx & 31;       // column tile of the chunk, row of the quarter
+    if (c0 / 4 + ct < col_tiles) {
+      const uint32_t* t = tile + r * SZ_PITCH + ct;
+      uint32_t* dst = out + (((int64_t)blockIdx.y * col_tiles + c0 / 4 + ct) * 32 + r) * 4;
+      if (out_vec) {
+        *reinterpret_cast<uint4*>(dst) = make_uint4(t[0], t[32 * SZ_PITCH], t[64 * SZ_PITCH], t[96 * SZ_PITCH]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dst[j] = t[32 * j * SZ_PITCH];
+      }
+    }
   }
 }
 
@@ -653,6 +698,7 @@ swizzle_scales_kernel(const uint8_t* __restrict__ in, int rows, int cols, uint32
 __global__ void __launch_bounds__(256)
 transpose_bf16_kernel(const uint16_t* __restrict__ in, int rows, int cols, int64_t ld_in,
                       uint16_t* __restrict__ out, int64_t ld_out) {
+  faar_pdl_sync();
   __shared__ uint16_t tile[64][66];
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;   // 64 x 4
@@ -676,6 +722,7 @@ transpose_bf16_kernel(const uint16_t* __restrict__ in, int rows, int cols, int64
 __global__ void __launch_bounds__(256)
 transpose_bf16_vec_kernel(const uint16_t* __restrict__ in, int rows, int cols, int64_t ld_in,
                           uint16_t* __restrict__ out, int64_t ld_out) {
+  faar_pdl_sync();
   __shared__ __align__(16) uint32_t tile[64][36];
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   {
@@ -714,22 +761,6 @@ int grid_for(const faar_ctx* ctx, int64_t work_items, int per_sm) {
 
 }  // namespace
 
-// Launch with stream serialisation relaxed: the kernel's CTAs may be scheduled while the kernel before
-// it drains; the kernel itself waits (griddepcontrol.wait) before it touches global memory.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_relaxed(faar_ctx* ctx, void (*kernel)(KArgs...), int grid, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3(EW_THREADS, 1, 1);
-  cfg.stream = ctx->stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
 // Serial number of a tensor-maximum pass, shared by all contexts of the process (a workspace may pass from one
 // context to another).  0 is what a freshly initialised workspace header holds and is skipped.
 static std::atomic<uint32_t> g_amax_epoch{0};
@@ -745,9 +776,9 @@ static int launch_amax(faar_ctx* ctx, bool bf16, const void* W, int rows, int K,
   const int64_t groups = (int64_t)rows * (K / 8);
   faar_prof_scope ps(ctx, FAAR_K_AMAX);
   const int grid = grid_for(ctx, (groups + 7) / 8, 8);
-  if (bf16) amax_kernel<true><<<grid, EW_THREADS, 0, ctx->stream>>>(W, rows, K, ld, amax_word, epoch);
-  else amax_kernel<false><<<grid, EW_THREADS, 0, ctx->stream>>>(W, rows, K, ld, amax_word, epoch);
-  return (int)cudaGetLastError();
+  const cudaError_t e = faar_launch_pdl(ctx, bf16 ? amax_kernel<true> : amax_kernel<false>, dim3(grid), dim3(EW_THREADS), 0, W, rows,
+                                        K, ld, amax_word, epoch);
+  return e != cudaSuccess ? (int)e : (int)cudaGetLastError();
 }
 
 int faar_launch_softquant_init(faar_ctx* ctx, const faar_shape* s, const void* W, float s_global_in,
@@ -759,8 +790,8 @@ int faar_launch_softquant_init(faar_ctx* ctx, const faar_shape* s, const void* W
     if (e) return e;
   }
   faar_prof_scope ps(ctx, FAAR_K_SOFTQUANT_INIT);
-  cudaError_t e = launch_relaxed(ctx, s->w_dtype == FAAR_BF16 ? softquant_init_kernel<true> : softquant_init_kernel<false>,
-                                 grid_for(ctx, blocks, 3), W, s->O, s->K, s->ldw, s_global_in,
+  cudaError_t e = faar_launch_pdl(ctx, s->w_dtype == FAAR_BF16 ? softquant_init_kernel<true> : softquant_init_kernel<false>,
+                                 dim3(grid_for(ctx, blocks, 3)), dim3(EW_THREADS), 0, W, s->O, s->K, s->ldw, s_global_in,
                                  (const unsigned long long*)amax_word, scales, s_global_out, code, V);
   if (e != cudaSuccess) return (int)e;
   return (int)cudaGetLastError();
@@ -775,7 +806,7 @@ int faar_launch_act_fakequant(faar_ctx* ctx, int T, int K, const void* X, int64_
     if (e) return e;
   }
   faar_prof_scope ps(ctx, FAAR_K_ACT_FAKEQUANT);
-  cudaError_t e = launch_relaxed(ctx, act_fakequant_kernel, grid_for(ctx, blocks, 3),
+  cudaError_t e = faar_launch_pdl(ctx, act_fakequant_kernel, dim3(grid_for(ctx, blocks, 3)), dim3(EW_THREADS), 0,
                                  reinterpret_cast<const __nv_bfloat16*>(X), T, K, ldx, s_global_in,
                                  (const unsigned long long*)amax_word, reinterpret_cast<__nv_bfloat16*>(Xq), ldq,
                                  s_global_out, packed, scales);
@@ -787,7 +818,7 @@ int faar_launch_nvfp4_expand(faar_ctx* ctx, int rows, int K, const uint8_t* pack
                              int64_t ld) {
   const int64_t blocks = (int64_t)rows * (K / 16);
   faar_prof_scope ps(ctx, FAAR_K_ACT_FAKEQUANT);
-  nvfp4_expand_kernel<<<grid_for(ctx, blocks, 8), EW_THREADS, 0, ctx->stream>>>(packed, scales, rows, K,
+  faar_launch_pdl(ctx, nvfp4_expand_kernel, dim3(grid_for(ctx, blocks, 8)), dim3(EW_THREADS), 0, packed, scales, rows, K,
                                                                                reinterpret_cast<__nv_bfloat16*>(out), ld);
   return (int)cudaGetLastError();
 }
@@ -797,17 +828,8 @@ int faar_launch_softquant_eval(faar_ctx* ctx, const faar_shape* s, const float* 
                                float* h, __nv_bfloat16* W_bf16, float* W_operand_f32) {
   const int64_t groups = (int64_t)s->O * (s->K / 8);
   faar_prof_scope ps(ctx, FAAR_K_SOFT_WEIGHTS);
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3(grid_for(ctx, groups, 8), 1, 1);
-  cfg.blockDim = dim3(EW_THREADS, 1, 1);
-  cfg.stream = ctx->stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, softquant_eval_kernel, V, code, scales, s_global, beta, (int64_t)groups, W_soft,
-                                     h, W_bf16, W_operand_f32);
+  cudaError_t e = faar_launch_pdl(ctx, softquant_eval_kernel, dim3(grid_for(ctx, groups, 8)), dim3(EW_THREADS), 0, V, code, scales,
+                                  s_global, beta, (int64_t)groups, W_soft, h, W_bf16, W_operand_f32);
   if (e != cudaSuccess) return (int)e;
   return (int)cudaGetLastError();
 }
@@ -819,20 +841,26 @@ int faar_launch_transpose_bf16(faar_ctx* ctx, int rows, int cols, const void* in
   const bool vec = cols % 8 == 0 && ld_in % 8 == 0 && ld_out % 8 == 0 && ld_out >= (int64_t)(rows + 7) / 8 * 8 &&
                    ((uintptr_t)in & 15) == 0 && ((uintptr_t)out & 15) == 0;
   if (vec) {
-    transpose_bf16_vec_kernel<<<grid, 256, 0, ctx->stream>>>(reinterpret_cast<const uint16_t*>(in), rows, cols, ld_in,
+    faar_launch_pdl(ctx, transpose_bf16_vec_kernel, dim3(grid), dim3(256), 0, reinterpret_cast<const uint16_t*>(in), rows, cols, ld_in,
                                                              reinterpret_cast<uint16_t*>(out), ld_out);
     return (int)cudaGetLastError();
   }
-  transpose_bf16_kernel<<<grid, 256, 0, ctx->stream>>>(reinterpret_cast<const uint16_t*>(in), rows, cols, ld_in,
+  faar_launch_pdl(ctx, transpose_bf16_kernel, dim3(grid), dim3(256), 0, reinterpret_cast<const uint16_t*>(in), rows, cols, ld_in,
                                                        reinterpret_cast<uint16_t*>(out), ld_out);
   return (int)cudaGetLastError();
 }
 
 int faar_launch_swizzle_scales(faar_ctx* ctx, int rows, int cols, const uint8_t* in, uint8_t* out) {
-  const int64_t n_words = (int64_t)((rows + 127) / 128) * ((cols + 3) / 4) * 128;
+  const int col_tiles = (cols + 3) / 4, bands = (rows + 127) / 128;
   faar_prof_scope ps(ctx, FAAR_K_HARDEN_PACK);
-  swizzle_scales_kernel<<<grid_for(ctx, n_words, 8), EW_THREADS, 0, ctx->stream>>>(in, rows, cols,
-                                                                                  reinterpret_cast<uint32_t*>(out), n_words);
+  // a grid's y extent is limited to 65535: more bands than that (8.4 M rows) go in several launches
+  for (int b0 = 0; b0 < bands; b0 += 65535) {
+    const int nb = bands - b0 < 65535 ? bands - b0 : 65535;
+    cudaError_t e = faar_launch_pdl(ctx, swizzle_scales_kernel, dim3((cols + SZ_COLS - 1) / SZ_COLS, nb), dim3(EW_THREADS), 0,
+                                    in + (int64_t)b0 * 128 * cols, rows - 128 * b0, cols,
+                                    reinterpret_cast<uint32_t*>(out + (int64_t)b0 * col_tiles * 512), col_tiles);
+    if (e != cudaSuccess) return (int)e;
+  }
   return (int)cudaGetLastError();
 }
 
@@ -840,7 +868,7 @@ int faar_launch_round_partials(faar_ctx* ctx, const float* V, int64_t N, float* 
   int grid = grid_for(ctx, (N + 3) / 4, 4);
   if (grid > FAAR_MAX_PARTIALS) grid = FAAR_MAX_PARTIALS;
   faar_prof_scope ps(ctx, FAAR_K_ROUND_LOSS);
-  round_partials_kernel<<<grid, EW_THREADS, 0, ctx->stream>>>(V, N, partials);
+  faar_launch_pdl(ctx, round_partials_kernel, dim3(grid), dim3(EW_THREADS), 0, V, N, partials);
   *n_partials = grid;
   return (int)cudaGetLastError();
 }
@@ -848,7 +876,7 @@ int faar_launch_round_partials(faar_ctx* ctx, const float* V, int64_t N, float* 
 int faar_launch_finalize(faar_ctx* ctx, const float* p0, int n0, float scale0, float* out0, const float* p1,
                          int n1, float scale1, float* out1) {
   faar_prof_scope ps(ctx, FAAR_K_FINALIZE);
-  finalize_kernel<<<1, 256, 0, ctx->stream>>>(p0, n0, scale0, out0, p1, n1, scale1, out1);
+  faar_launch_pdl(ctx, finalize_kernel, dim3(1), dim3(256), 0, p0, n0, scale0, out0, p1, n1, scale1, out1);
   return (int)cudaGetLastError();
 }
 
@@ -857,7 +885,7 @@ int faar_launch_harden_pack(faar_ctx* ctx, const faar_shape* s, const float* V, 
                             uint8_t* scales_out, uint8_t* decisions, void* W_final, int wfinal_dtype) {
   const int64_t groups = (int64_t)s->O * (s->K / 8);
   faar_prof_scope ps(ctx, FAAR_K_HARDEN_PACK);
-  harden_pack_kernel<<<grid_for(ctx, groups, 8), EW_THREADS, 0, ctx->stream>>>(
+  faar_launch_pdl(ctx, harden_pack_kernel, dim3(grid_for(ctx, groups, 8)), dim3(EW_THREADS), 0, 
       V, code, scales, s_global, groups, packed, scales_out, decisions, W_final, wfinal_dtype);
   return (int)cudaGetLastError();
 }

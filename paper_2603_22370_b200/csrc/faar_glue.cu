@@ -47,6 +47,7 @@ __device__ __forceinline__ int split_row_step() { return gridDim.y * blockDim.y;
 __global__ void __launch_bounds__(GL_THREADS)
 silu_mul_kernel(const __nv_bfloat16* gate, int64_t ldg, const __nv_bfloat16* up, int64_t ldu, __nv_bfloat16* out, int64_t ldo,
                 int rows, int groups) {
+  faar_pdl_sync();
   const int cg = split_group();
   if (cg >= groups) return;
   const int col = 8 * cg, step = split_row_step();
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(GL_THREADS)
 rmsnorm_kernel(const __nv_bfloat16* x, int64_t ldx, const __nv_bfloat16* b, int64_t ldb, __nv_bfloat16* sum_out, int64_t lds,
                const float* __restrict__ g, float eps, __nv_bfloat16* y, int64_t ldy, float* __restrict__ rstd_out, int rows,
                int cols) {
+  faar_pdl_sync();
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int n_groups = cols / 8;
@@ -183,6 +185,7 @@ __global__ void __launch_bounds__(GL_THREADS)
 rmsnorm_bwd_kernel(const __nv_bfloat16* dy, const __nv_bfloat16* dy2, const __nv_bfloat16* dy3, int64_t lddy,
                    const __nv_bfloat16* x, int64_t ldx, const float* __restrict__ g, const float* __restrict__ rstd_in,
                    const __nv_bfloat16* add, int64_t ldadd, __nv_bfloat16* dx, int64_t lddx, int rows, int cols) {
+  faar_pdl_sync();
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int n_groups = cols / 8;
@@ -245,6 +248,7 @@ template <int HPT>
 __global__ void __launch_bounds__(GL_THREADS)
 rope_kernel(const __nv_bfloat16* x, int64_t ldx, const int* __restrict__ pos, __nv_bfloat16* y, int64_t ldy, int rows,
             int groups, int head_dim, float log2_theta, int inverse) {
+  faar_pdl_sync();
   const int cg = split_group();
   if (cg >= groups) return;
   const int half = head_dim / 2, gph = half / 8;                    // 8-element groups per half head
@@ -289,6 +293,7 @@ rope_kernel(const __nv_bfloat16* x, int64_t ldx, const int* __restrict__ pos, __
 __global__ void __launch_bounds__(GL_THREADS)
 silu_mul_bwd_kernel(const __nv_bfloat16* dout, int64_t ldd, const __nv_bfloat16* gate, int64_t ldg, const __nv_bfloat16* up,
                     int64_t ldu, __nv_bfloat16* dgate, int64_t lddg, __nv_bfloat16* dup, int64_t lddu, int rows, int groups) {
+  faar_pdl_sync();
   const int cg = split_group();
   if (cg >= groups) return;
   const int col = 8 * cg;
@@ -312,6 +317,7 @@ silu_mul_bwd_kernel(const __nv_bfloat16* dout, int64_t ldd, const __nv_bfloat16*
 __global__ void __launch_bounds__(GL_THREADS)
 embedding_kernel(const __nv_bfloat16* __restrict__ table, int64_t ldt, const int* __restrict__ tokens, int vocab,
                  __nv_bfloat16* __restrict__ out, int64_t ldo, int rows, int groups) {
+  faar_pdl_sync();
   const int cg = split_group();
   if (cg >= groups) return;
   const int col = 8 * cg;
@@ -327,6 +333,7 @@ embedding_kernel(const __nv_bfloat16* __restrict__ table, int64_t ldt, const int
 __global__ void __launch_bounds__(GL_THREADS)
 add_kernel(const __nv_bfloat16* a, int64_t lda, const __nv_bfloat16* b, int64_t ldb, __nv_bfloat16* out, int64_t ldo, int rows,
            int groups) {
+  faar_pdl_sync();
   const int cg = split_group();
   if (cg >= groups) return;
   const int col = 8 * cg;
@@ -371,7 +378,7 @@ int faar_launch_silu_mul(faar_ctx* ctx, int rows, int cols, const void* gate, in
                          void* out, int64_t ldo) {
   faar_prof_scope ps(ctx, FAAR_K_GLUE);
   const Split sp = glue_split(ctx, (rows + 1) / 2, cols / 8);
-  silu_mul_kernel<<<sp.grid, sp.block, 0, ctx->stream>>>(
+  faar_launch_pdl(ctx, silu_mul_kernel, sp.grid, sp.block, 0, 
       reinterpret_cast<const __nv_bfloat16*>(gate), ldg, reinterpret_cast<const __nv_bfloat16*>(up), ldu,
       reinterpret_cast<__nv_bfloat16*>(out), ldo, rows, cols / 8);
   return (int)cudaGetLastError();
@@ -387,9 +394,9 @@ int faar_launch_rmsnorm(faar_ctx* ctx, int rows, int cols, const void* x, int64_
   auto* sp = reinterpret_cast<__nv_bfloat16*>(sum_out);
   auto* yp = reinterpret_cast<__nv_bfloat16*>(y);
   if (cols <= 8 * 32 * 8)
-    rmsnorm_kernel<8><<<grid, GL_THREADS, 0, ctx->stream>>>(xp, ldx, bp, ldb, sp, lds, g, eps, yp, ldy, rstd, rows, cols);
+    faar_launch_pdl(ctx, rmsnorm_kernel<8>, dim3(grid), dim3(GL_THREADS), 0, xp, ldx, bp, ldb, sp, lds, g, eps, yp, ldy, rstd, rows, cols);
   else
-    rmsnorm_kernel<0><<<grid, GL_THREADS, 0, ctx->stream>>>(xp, ldx, bp, ldb, sp, lds, g, eps, yp, ldy, rstd, rows, cols);
+    faar_launch_pdl(ctx, rmsnorm_kernel<0>, dim3(grid), dim3(GL_THREADS), 0, xp, ldx, bp, ldb, sp, lds, g, eps, yp, ldy, rstd, rows, cols);
   return (int)cudaGetLastError();
 }
 
@@ -405,7 +412,7 @@ int faar_launch_rmsnorm_bwd(faar_ctx* ctx, int rows, int cols, const void* dy, c
   auto* xp = reinterpret_cast<const __nv_bfloat16*>(x);
   auto* ap = reinterpret_cast<const __nv_bfloat16*>(add);
   auto* op = reinterpret_cast<__nv_bfloat16*>(dx);
-  rmsnorm_bwd_kernel<<<grid, GL_THREADS, 0, ctx->stream>>>(d1, d2, d3, lddy, xp, ldx, g, rstd, ap, ldadd, op, lddx, rows, cols);
+  faar_launch_pdl(ctx, rmsnorm_bwd_kernel, dim3(grid), dim3(GL_THREADS), 0, d1, d2, d3, lddy, xp, ldx, g, rstd, ap, ldadd, op, lddx, rows, cols);
   return (int)cudaGetLastError();
 }
 
@@ -418,9 +425,9 @@ int faar_launch_rope(faar_ctx* ctx, int rows, int n_heads, int head_dim, const v
   auto* xp = reinterpret_cast<const __nv_bfloat16*>(x);
   auto* yp = reinterpret_cast<__nv_bfloat16*>(y);
   if (four)
-    rope_kernel<4><<<sp.grid, sp.block, 0, ctx->stream>>>(xp, ldx, pos, yp, ldy, rows, groups, head_dim, log2f(theta), inverse);
+    faar_launch_pdl(ctx, rope_kernel<4>, sp.grid, sp.block, 0, xp, ldx, pos, yp, ldy, rows, groups, head_dim, log2f(theta), inverse);
   else
-    rope_kernel<1><<<sp.grid, sp.block, 0, ctx->stream>>>(xp, ldx, pos, yp, ldy, rows, groups, head_dim, log2f(theta), inverse);
+    faar_launch_pdl(ctx, rope_kernel<1>, sp.grid, sp.block, 0, xp, ldx, pos, yp, ldy, rows, groups, head_dim, log2f(theta), inverse);
   return (int)cudaGetLastError();
 }
 
@@ -428,7 +435,7 @@ int faar_launch_silu_mul_bwd(faar_ctx* ctx, int rows, int cols, const void* dout
                              const void* up, int64_t ldu, void* dgate, int64_t lddg, void* dup, int64_t lddu) {
   faar_prof_scope ps(ctx, FAAR_K_GLUE);
   const Split sp = glue_split(ctx, rows, cols / 8);
-  silu_mul_bwd_kernel<<<sp.grid, sp.block, 0, ctx->stream>>>(
+  faar_launch_pdl(ctx, silu_mul_bwd_kernel, sp.grid, sp.block, 0, 
       reinterpret_cast<const __nv_bfloat16*>(dout), ldd, reinterpret_cast<const __nv_bfloat16*>(gate), ldg,
       reinterpret_cast<const __nv_bfloat16*>(up), ldu, reinterpret_cast<__nv_bfloat16*>(dgate), lddg,
       reinterpret_cast<__nv_bfloat16*>(dup), lddu, rows, cols / 8);
@@ -439,7 +446,7 @@ int faar_launch_embedding(faar_ctx* ctx, int rows, int cols, int vocab, const vo
                           void* out, int64_t ldo) {
   faar_prof_scope ps(ctx, FAAR_K_GLUE);
   const Split sp = glue_split(ctx, rows, cols / 8);
-  embedding_kernel<<<sp.grid, sp.block, 0, ctx->stream>>>(
+  faar_launch_pdl(ctx, embedding_kernel, sp.grid, sp.block, 0, 
       reinterpret_cast<const __nv_bfloat16*>(table), ldt, tokens, vocab, reinterpret_cast<__nv_bfloat16*>(out), ldo, rows,
       cols / 8);
   return (int)cudaGetLastError();
@@ -449,7 +456,7 @@ int faar_launch_add(faar_ctx* ctx, int rows, int cols, const void* a, int64_t ld
                     int64_t ldo) {
   faar_prof_scope ps(ctx, FAAR_K_GLUE);
   const Split sp = glue_split(ctx, rows, cols / 8);
-  add_kernel<<<sp.grid, sp.block, 0, ctx->stream>>>(
+  faar_launch_pdl(ctx, add_kernel, sp.grid, sp.block, 0, 
       reinterpret_cast<const __nv_bfloat16*>(a), lda, reinterpret_cast<const __nv_bfloat16*>(b), ldb,
       reinterpret_cast<__nv_bfloat16*>(out), ldo, rows, cols / 8);
   return (int)cudaGetLastError();

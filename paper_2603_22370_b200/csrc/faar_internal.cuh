@@ -54,6 +54,23 @@ int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes);
 // a fact of device and kernel (a GPC with an odd SM count strands one SM), asked once per device and process.
 int faar_max_pairs(faar_ctx* c, int slot, const void* kernel, cudaLaunchConfig_t* cfg);
 
+// Launch with stream serialisation relaxed (programmatic dependent launch): the kernel's CTAs may be scheduled while the
+// kernel before it drains; the kernel itself waits (faar_pdl_sync) before it touches global memory.
+template <typename... KArgs, typename... Args>
+static inline cudaError_t faar_launch_pdl(faar_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // ---- workspace layout -------------------------------------------------------
 // [0, 256)            header: word 0 = status (0 = ok), word 2 = count of dW-GEMM
 //                     CTAs that have finished (zero between launches), bytes 16..23 = tensor maximum of

@@ -63,6 +63,23 @@ def test_act_fakequant_bit_exact(ctx, T, K, ldx, sg_in):
     assert torch.equal(Xq, Xq2)
 
 
+@pytest.mark.parametrize("sg_in", [0.0, 2.0 ** -7, 0.013])
+@pytest.mark.parametrize("spread", [4, 24, 120])
+def test_act_fakequant_over_the_bf16_range(ctx, sg_in, spread):
+    """Random BF16 bit patterns over `spread` binades (blocks that mix ordinary, minute and zero values of either sign, and
+    quotients on and next to every midpoint): codes, scales and values bit for bit."""
+    rng = np.random.default_rng(spread)
+    T, K = 256, 512
+    bits = (rng.integers(0, 2, (T, K)) << 15) | (rng.integers(129 - spread, 130, (T, K)) << 7) | rng.integers(0, 128, (T, K))
+    bits[rng.random((T, K)) < 0.02] &= 0x8000                          # +0.0 and -0.0
+    X = (bits.astype(np.uint32) << 16).view(np.float32)
+    Xq, sx, packed, scales = _quantise(ctx, X, sg_in)
+    units, sg, packed_o, scales_o = fo.act_fake_quant(X, sg_in)
+    assert host(sx)[0] == sg
+    assert np.array_equal(host(scales), scales_o) and np.array_equal(host(packed), packed_o)
+    assert np.array_equal(host(Xq).astype(np.float64), units)
+
+
 @pytest.mark.parametrize("O,K,T", [(300, 1040, 600), (128, 256, 1024)])
 def test_layer_step_on_quantised_activations(ctx, O, K, T):
     W, X = inputs.config2(9, O, K, T)

@@ -174,3 +174,21 @@ def test_nvfp4_gemm_argument_checks(ctx):
     assert call(A=px.view(-1)[1:]) == faar.ERR_ALIGN
     assert call(ws_bytes=16) == faar.ERR_WORKSPACE
     lay.check()
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 1), (127, 3), (128, 64), (129, 65), (300, 16), (257, 80), (64, 515)])
+@pytest.mark.parametrize("offset", [0, 4])
+def test_tiled_scales_at_the_edges_of_a_block(ctx, rows, cols, offset):
+    """One CTA takes 128 rows x 64 columns: partial bands and chunks, row pitches with and without 16-byte vectors, an
+    output that is only word-aligned; every byte against the definition of the layout, padding zero."""
+    g = torch.Generator(device=DEV).manual_seed(rows + cols)
+    s = torch.randint(0, 256, (rows, cols), dtype=torch.uint8, device=DEV, generator=g)
+    n = (rows + 127) // 128 * ((cols + 3) // 4) * 512
+    buf = torch.full((n + 16,), 7, dtype=torch.uint8, device=DEV)
+    faar.swizzle_scales(ctx, rows, cols, s, buf[offset:offset + n])
+    torch.cuda.synchronize()
+    pad = np.zeros(((rows + 127) // 128 * 128, (cols + 3) // 4 * 4), dtype=np.uint8)
+    pad[:rows, :cols] = host(s)
+    want = pad.reshape(-1, 4, 32, (cols + 3) // 4, 4).transpose(0, 3, 2, 1, 4).reshape(-1)
+    got = host(buf)
+    assert np.array_equal(got[offset:offset + n], want) and np.all(got[:offset] == 7) and np.all(got[offset + n:] == 7)
