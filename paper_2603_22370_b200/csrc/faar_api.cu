@@ -556,9 +556,16 @@ int faar_layer_ref(faar_ctx* ctx, const faar_shape* s, const void* X, const void
   FAAR_DEVICE_GUARD(ctx);
   faar_gemm_args a = {};
   a.mode = FAAR_GEMM_REF;
-  a.M = s->O; a.N = s->T; a.Kc = s->K;
-  a.A = W; a.lda = s->ldw;
-  a.B = X; a.ldb = s->ldx;
+  a.Kc = s->K;
+  if (s->yref_transposed) {                // Y^T[O, T]: one row per output feature
+    a.M = s->O; a.N = s->T;
+    a.A = W; a.lda = s->ldw;
+    a.B = X; a.ldb = s->ldx;
+  } else {
+    a.M = s->T; a.N = s->O;
+    a.A = X; a.lda = s->ldx;
+    a.B = W; a.ldb = s->ldw;
+  }
   a.status = reinterpret_cast<uint32_t*>(workspace);
   a.Yout = Y_ref; a.yout_dtype = s->yref_dtype; a.ldy = s->ldy; a.yref_t = s->yref_transposed;
   return cuda_fail(ctx, faar_launch_gemm(ctx, &a, nullptr));
@@ -583,13 +590,13 @@ int faar_layer_dx(faar_ctx* ctx, const faar_shape* s, float beta, const void* dY
   if (ctx->wsoft_ws == workspace) ctx->wsoft_ws = nullptr;     // the operand slot is overwritten below
   int e = faar_launch_softquant_eval(ctx, s, V, code, scales, s_global, beta, nullptr, nullptr, wsoft);
   if (e) return cuda_fail(ctx, e);
-  // dX^T[K,T] = W_soft^T[K,O] * dY[T,O]^T, written transposed as dX[T,K].  W_soft [O,K] is that A operand with
-  // its M index (k) contiguous and the contraction index (o) as the row: read as it is.
+  // dX[T,K] = dY[T,O] W_soft[O,K]: W_soft is the B operand with its N index (k) contiguous and the contraction index (o)
+  // as the row: read as it is.
   faar_gemm_args a = {};
   a.mode = FAAR_GEMM_REF;
-  a.M = s->K; a.N = s->T; a.Kc = s->O;
-  a.A = wsoft; a.lda = s->K; a.a_mn = 1;
-  a.B = dY; a.ldb = s->ldy;
+  a.M = s->T; a.N = s->K; a.Kc = s->O;
+  a.A = dY; a.lda = s->ldy;
+  a.B = wsoft; a.ldb = s->K; a.b_mn = 1;
   a.status = reinterpret_cast<uint32_t*>(ws);
   a.Yout = dX; a.yout_dtype = FAAR_BF16; a.ldy = s->ldx;
   return cuda_fail(ctx, faar_launch_gemm(ctx, &a, nullptr));
@@ -604,12 +611,12 @@ int faar_layer_dx_operand(faar_ctx* ctx, const faar_shape* s, const void* dY, co
   if (s->ldy % 8 || s->ldx % 8 || s->ldw % 8 || !aligned16(dY) || !aligned16(Wsoft) || !aligned16(dX)) return FAAR_ERR_ALIGN;
   if ((st = check_ws(s, workspace, workspace_bytes))) return st;
   FAAR_DEVICE_GUARD(ctx);
-  // dX^T[K,T] = W_soft^T[K,O] * dY[T,O]^T written transposed as dX[T,K], as in faar_layer_dx
+  // dX[T,K] = dY[T,O] W_soft[O,K], as in faar_layer_dx
   faar_gemm_args a = {};
   a.mode = FAAR_GEMM_REF;
-  a.M = s->K; a.N = s->T; a.Kc = s->O;
-  a.A = Wsoft; a.lda = s->ldw; a.a_mn = 1;
-  a.B = dY; a.ldb = s->ldy;
+  a.M = s->T; a.N = s->K; a.Kc = s->O;
+  a.A = dY; a.lda = s->ldy;
+  a.B = Wsoft; a.ldb = s->ldw; a.b_mn = 1;
   a.status = reinterpret_cast<uint32_t*>(workspace);
   a.Yout = dX; a.yout_dtype = FAAR_BF16; a.ldy = s->ldx;
   return cuda_fail(ctx, faar_launch_gemm(ctx, &a, nullptr));

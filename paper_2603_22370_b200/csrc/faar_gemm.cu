@@ -17,7 +17,8 @@
 //   REF : Y_fp = X W^T                                   (Procedure step 8)
 //   FWD : r = Y_q - Y_ref, sum r^2, dY = 2c r -> dY^T     (steps 9-10, Eq. 5 first term)
 //   BWD : G = dY^T X -> dV -> optimiser update + clip     (step 13, Eq. 5, with Eq. 2/3 chain rule)
-// In all of them the accumulator row (TMEM lane) is the output feature o.
+// In FWD and BWD the accumulator row (TMEM lane) is the output feature o.  In REF it is a row of the result as it lies in
+// memory (a token, or an output feature if the target is wanted transposed), so that a lane's 16 columns are contiguous.
 //
 // Every wait on an mbarrier is bounded: after about two seconds the waiting thread records a code in
 // the status word, raises a CTA-wide abort flag and every role leaves its loop; both CTAs then meet at
@@ -237,6 +238,7 @@ __device__ __forceinline__ uint64_t make_smem_desc_mn(uint32_t saddr) {
 }
 constexpr int MN_BOX = 64;                         // M / N elements per MN-major TMA box
 constexpr int MN_BOX_BYTES = MN_BOX * BK * 2;      // 8192
+__host__ __device__ constexpr int mn_boxes(int columns) { return (columns + MN_BOX - 1) / MN_BOX; }
 constexpr uint32_t MN_KSTEP = (UMMA_K * 128) >> 4; // 16 contraction indices on: 2048 B in the address field
 // Instruction descriptor: D = F32, A = B = BF16, M = 256 (the CTA pair), N = bn; bits 15 / 16 say that A / B is
 // MN-major instead of K-major.
@@ -250,13 +252,14 @@ struct KParams {
   int bn;                 // tile width
   int stages, stage_bytes;   // ring depth, bytes of a stage (both CTAs alike)
   int n_full_cols;        // tile columns of full width; the columns after them are bn/2 wide (tail split)
-  int a_mn, b_mn;         // operand stored with M (N) contiguous, [Kc, M] / [Kc, N], instead of [M, Kc] / [N, Kc]
   uint32_t* status;
   long long ext_yout, ext_dyt, ext_state, ext_wsoft;   // bytes of Yout, dYt, each of V / m / u / dV, wsoft_next (debug checks)
   // REF / FWD
   void* Yout; int yout_dtype; long long ldy;
   const void* Yref; int yref_dtype;
-  int yref_t;             // Y_ref / Y_out stored transposed: [O, ldy] with ldy >= T rounded up to 16
+  int yref_t;             // FWD: Y_ref / Y_q stored transposed, [O, ldy] with ldy >= T rounded up to 16
+  int y_store;            // REF: rows of Yout take 16 columns as 3: one 32-byte store, padded (columns beyond N are written as 0),
+                          // 2: one 32-byte store, 1: 16-byte stores, 0: single values
   __nv_bfloat16* dYt; long long ld_dyt;
   float mse2c;
   float act_scale;        // FWD: Y_q = act_scale * acc; BWD: G = act_scale * acc
@@ -339,44 +342,61 @@ __device__ __forceinline__ bool dbg_in_range(const KParams& p, const void* ptr, 
 #endif
 
 // ---- epilogues: one call handles 16 accumulator columns of one row ---------------------------
-// REF: write acc to Y[t, o].
-__device__ __forceinline__ void epi_ref(const KParams& p, int o, int t0, const uint32_t (&acc)[16]) {
-  if (o >= p.M) return;
-  if (p.yref_t) {                                    // row o of the transposed target: 16 contiguous values
-    // (the row is padded to a multiple of 16, so a full vector store stays inside it)
+__device__ __forceinline__ void stg256(void* ptr, const uint32_t (&w)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(ptr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]),
+               "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+}
+// REF: write acc to row `row`, columns c0..c0+15 of Y.  A whole 32-byte sector per lane and instruction: with the output
+// feature in the lane and the token in the column (2-byte stores, 64 bytes per warp instruction) the epilogue of a
+// 256-wide tile took 7.4-9 us, most of it after the last product of a launch.
+__device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const uint32_t (&acc)[16]) {
+  if (row >= p.M) return;
+  const long long off = (long long)row * p.ldy + c0;
+  if (p.y_store >= 2 && (p.y_store == 3 || c0 + 16 <= p.N)) {
+    const bool whole = c0 + 16 <= p.N;
     if (p.yout_dtype == FAAR_BF16) {
-      uint4* d4 = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.Yout) + (long long)o * p.ldy + t0);
-      float a[16];
+      __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + off;
+      uint32_t w[8];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) a[j] = (t0 + j < p.N) ? __uint_as_float(acc[j]) : 0.f;
-      if (!FAAR_DBG_OK(p, d4, 32, p.Yout, p.ext_yout, 1u)) return;
-      d4[0] = make_uint4(pack_bf16x2(a[0], a[1]), pack_bf16x2(a[2], a[3]), pack_bf16x2(a[4], a[5]), pack_bf16x2(a[6], a[7]));
-      d4[1] = make_uint4(pack_bf16x2(a[8], a[9]), pack_bf16x2(a[10], a[11]), pack_bf16x2(a[12], a[13]), pack_bf16x2(a[14], a[15]));
+      for (int j = 0; j < 8; ++j)
+        w[j] = pack_bf16x2(whole || c0 + 2 * j < p.N ? __uint_as_float(acc[2 * j]) : 0.f,
+                           whole || c0 + 2 * j + 1 < p.N ? __uint_as_float(acc[2 * j + 1]) : 0.f);
+      if (FAAR_DBG_OK(p, y, 32, p.Yout, p.ext_yout, 1u)) stg256(y, w);
     } else {
-      float4* d4 = reinterpret_cast<float4*>(reinterpret_cast<float*>(p.Yout) + (long long)o * p.ldy + t0);
-      if (!FAAR_DBG_OK(p, d4, 64, p.Yout, p.ext_yout, 1u)) return;
+      float* y = reinterpret_cast<float*>(p.Yout) + off;
+      if (!FAAR_DBG_OK(p, y, 64, p.Yout, p.ext_yout, 1u)) return;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        d4[q] = make_float4((t0 + 4 * q < p.N) ? __uint_as_float(acc[4 * q]) : 0.f,
-                            (t0 + 4 * q + 1 < p.N) ? __uint_as_float(acc[4 * q + 1]) : 0.f,
-                            (t0 + 4 * q + 2 < p.N) ? __uint_as_float(acc[4 * q + 2]) : 0.f,
-                            (t0 + 4 * q + 3 < p.N) ? __uint_as_float(acc[4 * q + 3]) : 0.f);
+      for (int h = 0; h < 2; ++h) {
+        uint32_t w[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[j] = whole || c0 + 8 * h + j < p.N ? acc[8 * h + j] : 0u;
+        stg256(y + 8 * h, w);
+      }
     }
     return;
   }
+  const int n = min(16, p.N - c0);
+  if (p.yout_dtype == FAAR_BF16) {
+    __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + off;
+    if (p.y_store && n == 16) {
+      if (!FAAR_DBG_OK(p, y, 32, p.Yout, p.ext_yout, 1u)) return;
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    int t = t0 + j;
-    if (t < p.N) {
-      float a = __uint_as_float(acc[j]);
-      if (p.yout_dtype == FAAR_BF16) {
-        __nv_bfloat16* q = reinterpret_cast<__nv_bfloat16*>(p.Yout) + (long long)t * p.ldy + o;
-        if (FAAR_DBG_OK(p, q, 2, p.Yout, p.ext_yout, 1u)) *q = __float2bfloat16_rn(a);
-      } else {
-        float* q = reinterpret_cast<float*>(p.Yout) + (long long)t * p.ldy + o;
-        if (FAAR_DBG_OK(p, q, 4, p.Yout, p.ext_yout, 1u)) *q = a;
+      for (int h = 0; h < 2; ++h) {
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = pack_bf16x2(__uint_as_float(acc[8 * h + 2 * j]), __uint_as_float(acc[8 * h + 2 * j + 1]));
+        reinterpret_cast<uint4*>(y)[h] = make_uint4(w[0], w[1], w[2], w[3]);
       }
+      return;
     }
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (j < n && FAAR_DBG_OK(p, y + j, 2, p.Yout, p.ext_yout, 1u)) y[j] = __float2bfloat16_rn(__uint_as_float(acc[j]));
+  } else {
+    float* y = reinterpret_cast<float*>(p.Yout) + off;
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (j < n && FAAR_DBG_OK(p, y + j, 4, p.Yout, p.ext_yout, 1u)) y[j] = __uint_as_float(acc[j]);
   }
 }
 
@@ -695,7 +715,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           // the leader's barrier collects the bytes of both CTAs' copies
           if (rank == 0)
             mbar_expect_tx(full_bar(stage), WIDE ? 2u * (uint32_t)(C::A_BYTES + C::B_BYTES)
-                                                 : 2u * (uint32_t)(C::A_BYTES + (tc.w / 2) * BK * 2));
+                                                 : 2u * (uint32_t)(C::A_BYTES + (B_MN ? mn_boxes(tc.w / 2) * MN_BOX : tc.w / 2) * BK * 2));
           const uint32_t leader_full = map_to_cta(full_bar(stage), 0);
           if (A_MN) {                                          // two boxes of 64 rows of A, each [64 k][64 m]
             tma_load_2d(sa, &tmA, m0, kb * BK, leader_full, keep);
@@ -703,7 +723,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           } else {
             tma_load_2d(sa, &tmA, kb * BK, m0, leader_full, keep);
           }
-          if (B_MN) {                                          // w/2 = 128 or 64 rows of B: two boxes or one
+          if (B_MN) {                                          // this CTA's w / 2 columns of B, in boxes of 64
             tma_load_2d(sb, &tmB, n0, kb * BK, leader_full, keep);
             if (tc.w / 2 > MN_BOX) tma_load_2d(sb + MN_BOX_BYTES, &tmB, n0 + MN_BOX, kb * BK, leader_full, keep);
           } else {
@@ -877,15 +897,22 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
           }
         } else {
+          // REF: two chunks' accumulators in flight (a warp's column count is a multiple of 16: the second may be absent)
+          constexpr int STEP = MODE == FAAR_GEMM_REF ? 32 : 16;
 #pragma unroll 1
-          for (int c = col_begin; c < col_end; c += 16) {
+          for (int c = col_begin; c < col_end; c += STEP) {
             if (n0 + c >= p.N) break;                    // warp-uniform
             uint32_t r[16];
             tmem_ld16(trow + (uint32_t)c, r);
-            tmem_ld_wait();
             if (MODE == FAAR_GEMM_REF) {
+              const bool second = c + 16 < col_end && n0 + c + 16 < p.N;
+              uint32_t r2[16];
+              if (second) tmem_ld16(trow + (uint32_t)(c + 16), r2);
+              tmem_ld_wait();
               epi_ref(p, o, n0 + c, r);
+              if (second) epi_ref(p, o, n0 + c + 16, r2);
             } else {
+              tmem_ld_wait();
               float yr[16];
               load_yref(p, o, n0 + c, yr);
               warp_acc += epi_fwd(p, o, n0 + c, r, yr);
@@ -1010,7 +1037,7 @@ int make_map_mn(faar_ctx* ctx, CUtensorMap* map, const void* ptr, int kc_rows, i
 // width.  A smaller problem is a matter of latency: its tiles run at once, each brings its share of the epilogue, and
 // narrower tiles spread that over more SMs.
 // REF, FWD: the width with the smallest estimated time of the busiest pair (microseconds).  A k block costs the ring's
-// latency, or what the L2 needs for all pairs' operands (about 10 TB/s); the epilogue 0.8 / 0.6 per 64 columns.
+// latency, or what the L2 needs for all pairs' operands (about 10 TB/s); the epilogue 0.4 / 0.6 per 64 columns.
 // Measured (width before -> after): product [260, 1024] over 512 8.8 -> 6.2 us (128 -> 32), forward kernel of a
 // 128 x 256 layer at 1024 tokens 12.8 -> 10.7 us, input gradient [192, 128] over 384 11.1 -> 8.9 us.
 // BWD: its per-weight epilogue is bound by instruction issue and a tile of it has a fixed cost of several microseconds,
@@ -1019,15 +1046,15 @@ int make_map_mn(faar_ctx* ctx, CUtensorMap* map, const void* ptr, int kc_rows, i
 // 33.6 -> 51 us.
 int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs, bool b_mn) {
   if (ctx->tune_bn >= 128 && ctx->tune_bn <= BN_MAX && ctx->tune_bn % 16 == 0)
-    return b_mn && ctx->tune_bn % 128 != 0 ? (N <= 128 ? 128 : BN_MAX) : ctx->tune_bn;   // boxes of 64 columns per CTA
+    return b_mn ? (ctx->tune_bn + 31) / 32 * 32 : ctx->tune_bn;      // a CTA's first column of an N-contiguous B: 32-byte aligned
   const long long m_tiles = (M + 2 * BM - 1) / (2 * BM);
   if (mode == FAAR_GEMM_BWD) {
     if (N <= 128 || 2 * m_tiles * ((N + BN_MAX - 1) / BN_MAX) < pairs) return 128;
-    return N < BN_MAX && !b_mn ? (N + 31) / 32 * 32 : BN_MAX;
+    return N < BN_MAX ? (N + 31) / 32 * 32 : BN_MAX;
   }
   const int widest = N > 128 ? (N < BN_MAX ? (N + 31) / 32 * 32 : BN_MAX) : (N > 64 ? 128 : (N > 32 ? 64 : 32));
   if (m_tiles * ((N + widest - 1) / widest) >= pairs) return widest;
-  const double epi64 = mode == FAAR_GEMM_FWD ? 0.6 : 0.8;
+  const double epi64 = mode == FAAR_GEMM_FWD ? 0.6 : 0.4;
   int best = widest;
   double best_cost = 1e30;
   for (int bn = widest; bn >= 32; bn = bn > 128 ? 128 : bn / 2) {
@@ -1079,8 +1106,9 @@ int pick_full_cols(const faar_ctx* ctx, int M, int N, int bn, int pairs) {
 // power-capped jobs of whole decoder blocks the same launch and the q / o projections lose 6-10 %; the dW GEMM
 // loses 29 % (its long epilogue is no longer hidden) and the plain product loses whenever it needs more than
 // one wave.  No rule was found that wins consistently, so the default never takes them.
-bool pick_wide(const faar_ctx* ctx, int N, int bn) {
-  return ctx->tune_wide == 1 && bn == BN_MAX && N > BN_MAX;
+bool pick_wide(const faar_ctx* ctx, int mode, int M, int N, int bn) {
+  const int tokens = mode == FAAR_GEMM_REF && M > N ? M : N;           // REF may have the tokens as its rows
+  return ctx->tune_wide == 1 && bn == BN_MAX && tokens > BN_MAX;
 }
 
 template <int MODE, int OPT, bool WIDE, int MN>
@@ -1096,12 +1124,10 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   cudaLaunchConfig_t cfg = base_cfg;
   cfg.dynamicSmemBytes = C::SMEM_BYTES;
   kp.bn = bn;
-  kp.stage_bytes = WIDE ? C::STAGE_BYTES : C::A_BYTES + (int)faar_align_up((size_t)(bn / 2) * BK * 2, 1024);   // whole 8-row swizzle atoms
+  kp.stage_bytes = WIDE ? C::STAGE_BYTES : C::A_BYTES + (a->b_mn ? mn_boxes(bn / 2) * MN_BOX_BYTES : (int)faar_align_up((size_t)(bn / 2) * BK * 2, 1024));   // whole swizzle atoms
   kp.stages = C::RING_BYTES / kp.stage_bytes < MAX_STAGES ? C::RING_BYTES / kp.stage_bytes : MAX_STAGES;
   kp.n_full_cols = WIDE ? 0 : pick_full_cols(ctx, a->M, a->N, bn, max_pairs);
-  if (a->b_mn && bn != BN_MAX) kp.n_full_cols = (a->N + bn - 1) / bn;      // half tiles of a 128-wide tile would be 32 columns per CTA
   CUtensorMap tmA, tmB, tmBh;
-  kp.a_mn = a->a_mn; kp.b_mn = a->b_mn;
   e = a->a_mn ? make_map_mn(ctx, &tmA, a->A, a->Kc, a->M, a->lda) : make_map(ctx, &tmA, a->A, a->M, a->Kc, a->lda, BM);
   if (e) return e;
   if (a->b_mn) {
@@ -1152,17 +1178,17 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
   const int max_pairs = faar_max_pairs(ctx, MODE == FAAR_GEMM_BWD ? 2 + OPT : MODE, (const void*)kern, &cfg);
   const int bn = pick_bn(ctx, MODE, a->M, a->N, (a->Kc + BK - 1) / BK, max_pairs, a->b_mn != 0);
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
-  // which operand layouts a mode is ever launched with: the plain product with A untransposed (input gradient),
-  // the dW product with B or with both untransposed
+  // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient), the dW
+  // product with B or with both untransposed
   if constexpr (MODE == FAAR_GEMM_REF) {
-    if (mn == 1) return launch_variant<MODE, OPT, false, 1>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+    if (mn == 2) return launch_variant<MODE, OPT, false, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   }
   if constexpr (MODE == FAAR_GEMM_BWD) {
     if (mn == 2) return launch_variant<MODE, OPT, false, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
     if (mn == 3) return launch_variant<MODE, OPT, false, 3>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   }
   if (mn != 0) return (int)cudaErrorInvalidValue;
-  if (pick_wide(ctx, a->N, bn)) return launch_variant<MODE, OPT, true, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+  if (pick_wide(ctx, MODE, a->M, a->N, bn)) return launch_variant<MODE, OPT, true, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   return launch_variant<MODE, OPT, false, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
 }
 
@@ -1180,9 +1206,13 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* a, int* n_partials_out
   kp.M = a->M; kp.N = a->N; kp.Kc = a->Kc; kp.bn = BN_MAX; kp.n_full_cols = 0; kp.status = a->status;
   {
     const long long ysz = a->yout_dtype == FAAR_BF16 ? 2 : 4;
-    // Y is [N(T), ldy] or, transposed, [M(O), ldy]; the last row ends after its last valid (or padded) column
-    kp.ext_yout = a->Yout ? (a->yref_t ? ((long long)(a->M - 1) * a->ldy + (a->N + 15) / 16 * 16)
-                                       : ((long long)(a->N - 1) * a->ldy + a->M)) * ysz : 0;
+    // the last row ends after its last valid (or padded) column; REF and the transposed FWD layout: [M, ldy], else [N(T), ldy]
+    const bool rows_m = a->mode == FAAR_GEMM_REF || a->yref_t;
+    kp.ext_yout = a->Yout ? (rows_m ? ((long long)(a->M - 1) * a->ldy + (a->yref_t ? (a->N + 15) / 16 * 16 : a->N))
+                                    : ((long long)(a->N - 1) * a->ldy + a->M)) * ysz : 0;
+    const bool al32 = a->ldy * ysz % 32 == 0 && (reinterpret_cast<uintptr_t>(a->Yout) & 31) == 0;
+    const bool al16 = a->ldy * ysz % 16 == 0 && (reinterpret_cast<uintptr_t>(a->Yout) & 15) == 0;
+    kp.y_store = al32 ? (a->yref_t ? 3 : 2) : (al16 ? 1 : 0);
     kp.ext_dyt = a->dYt ? ((long long)(a->M - 1) * a->ld_dyt + a->N) * 2 : 0;
     kp.ext_state = (long long)a->M * a->N * 4;
     kp.ext_wsoft = (long long)a->M * a->N * 2;

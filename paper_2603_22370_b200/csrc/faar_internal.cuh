@@ -172,9 +172,9 @@ struct faar_gemm_args {
   int a_mn, b_mn;         // 1: the operand is stored with M (N) contiguous instead: A[Kc, M] (lda), B[Kc, N] (ldb)
   uint32_t* status;       // workspace status word
   // REF / FWD
-  void* Yout; int yout_dtype; int64_t ldy;     // [N(T), M(O)] written transposed; nullable in FWD
+  void* Yout; int yout_dtype; int64_t ldy;     // REF: [M, ldy]; FWD: [N(T), M(O)] written transposed, nullable
   const void* Yref; int yref_dtype;            // FWD
-  int yref_t;                                  // REF, FWD: Y stored transposed [O, ldy]
+  int yref_t;                                  // FWD: Y stored transposed [O, ldy]; REF: rows of Yout padded to 16 columns
   __nv_bfloat16* dYt; int64_t ld_dyt;          // FWD: [M(O), ld_dyt]
   float mse2c;                                 // FWD: 2 * mse_scale
   float act_scale;                             // FWD, BWD: tensor scale of quantised activations (1 = none)
