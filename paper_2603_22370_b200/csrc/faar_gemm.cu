@@ -251,7 +251,9 @@ struct KParams {
   int M, N, Kc;
   int bn;                 // tile width
   int stages, stage_bytes;   // ring depth, bytes of a stage (both CTAs alike)
-  int n_full_cols;        // tile columns of full width; the columns after them are bn/2 wide (tail split)
+  int n_main;             // tile columns of bn; a last column with at most bn/2 columns of the matrix (narrow) is extra
+  int narrow;             // 1: there is such a column; its tiles are bn/2 wide
+  int n_full;             // the first n_full tiles of the main columns are bn wide, the others come as two halves (tail split)
   uint32_t* status;
   long long ext_yout, ext_dyt, ext_state, ext_wsoft;   // bytes of Yout, dYt, each of V / m / u / dV, wsoft_next (debug checks)
   // REF / FWD
@@ -284,8 +286,8 @@ struct KParams {
   float fin_scale_round; float* fin_out2;   // {L_MSE, L_round}; null = no final sums here
 };
 
-// Tile t of the launch: the first n_full_cols tile columns are bn wide, the remaining columns bn/2
-// (half-width tiles fill the last, partly empty wave of the CTA pairs and halve the epilogue that
+// Tile t of the launch: the first n_full tiles of the raster are bn wide, each of the others is taken as two tiles of
+// bn/2 (half-width tiles even out the last, partly empty wave of the CTA pairs and halve the epilogue that
 // nothing overlaps).  All full-width tiles come first.  Tiles are numbered in bands of RASTER_ROWS row blocks, inside
 // a band row block fastest: the tiles that run at one time (74) then form a nearly square patch of the output, which
 // needs the fewest distinct operand rows.  With row blocks fastest over the whole height the LM head's product
@@ -298,27 +300,26 @@ __device__ __forceinline__ void raster(int t, int m_tiles, int n_cols, int& m, i
   n = r / rows;
   m = first + r - n * rows;
 }
-__device__ __forceinline__ int half_columns(const KParams& p) {
-  const int rest = p.N - p.n_full_cols * p.bn;                    // columns covered by half-width tiles
-  return rest > 0 ? (rest + p.bn / 2 - 1) / (p.bn / 2) : 0;
-}
 __device__ __forceinline__ TileCoord tile_coord(const KParams& p, int t, int m_tiles) {
-  const int full_tiles = m_tiles * p.n_full_cols;
+  const int halves = 2 * (m_tiles * p.n_main - p.n_full);
+  const int u = t - p.n_full;
   TileCoord c;
   int m, n;
-  if (t < full_tiles) {
-    raster(t, m_tiles, p.n_full_cols, m, n);
-    c.n0 = n * p.bn;
-    c.w = p.bn;
+  if (u < halves) {
+    raster(u < 0 ? t : p.n_full + (u >> 1), m_tiles, p.n_main, m, n);
+    c.n0 = n * p.bn + (u > 0 ? (u & 1) * (p.bn / 2) : 0);
+    c.w = u < 0 ? p.bn : p.bn / 2;
   } else {
-    raster(t - full_tiles, m_tiles, half_columns(p), m, n);
-    c.n0 = p.n_full_cols * p.bn + n * (p.bn / 2);
+    m = u - halves;
+    c.n0 = p.n_main * p.bn;
     c.w = p.bn / 2;
   }
   c.m0 = m * (2 * BM);
   return c;
 }
-__device__ __forceinline__ int tile_count(const KParams& p, int m_tiles) { return m_tiles * (p.n_full_cols + half_columns(p)); }
+__device__ __forceinline__ int tile_count(const KParams& p, int m_tiles) {
+  return 2 * m_tiles * p.n_main - p.n_full + (p.narrow ? m_tiles : 0);
+}
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
@@ -1041,7 +1042,7 @@ int make_map_mn(faar_ctx* ctx, CUtensorMap* map, const void* ptr, int kc_rows, i
 // Measured (width before -> after): product [260, 1024] over 512 8.8 -> 6.2 us (128 -> 32), forward kernel of a
 // 128 x 256 layer at 1024 tokens 12.8 -> 10.7 us, input gradient [192, 128] over 384 11.1 -> 8.9 us.
 // BWD: its per-weight epilogue is bound by instruction issue and a tile of it has a fixed cost of several microseconds,
-// so only 128-wide tiles (cut into halves of 64 by pick_full_cols while pairs are idle) while fewer than half of the
+// so only 128-wide tiles (cut into halves of 64 by pick_full while pairs are idle) while fewer than half of the
 // pairs would have a 256-wide one; 32-wide tiles: dW kernel of a 128 x 256 layer 19.2 -> 18.8 us, of a 1024 x 3600 layer
 // 33.6 -> 51 us.
 int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs, bool b_mn) {
@@ -1069,34 +1070,39 @@ int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs
   return best;
 }
 
-// How many trailing tile columns to cut into half-width tiles.  Tiles go to CTA pairs round-robin, all
-// full-width tiles first.  A half tile costs 0.75 of a full one (its A rows are loaded all the same), and
-// the epilogue of a pair's last tile is not overlapped by anything (0.4 of that tile's cost).  Returns the
-// number of full-width columns that minimises the busiest pair's time (ties: fewer half tiles).
-int pick_full_cols(const faar_ctx* ctx, int M, int N, int bn, int pairs) {
-  const int m_tiles = (M + 2 * BM - 1) / (2 * BM);
-  const int n_cols = (N + bn - 1) / bn;
-  if (bn % 32 != 0 || bn <= 64) return n_cols;
-  if (ctx->tune_tail >= 0) return ctx->tune_tail < n_cols ? n_cols - ctx->tune_tail : 0;
+// How many tiles of the raster stay whole.  Tiles go to CTA pairs round-robin, all whole tiles first.  A half tile costs
+// 0.75 of a whole one (its A rows are loaded all the same), and the epilogue of a pair's last tile is not overlapped by
+// anything (0.4 of that tile's cost).  Returns the number that minimises the busiest pair's time (ties: fewer halves).
+// A pair's load depends on how many whole and how many half tiles it gets, which change only at two pair numbers.
+// Cutting single tiles instead of whole tile columns matters for tall grids, whose columns hold many tiles: [8192, 2048]
+// over 8192 is 256 tiles of 256 on 74 pairs, 3.46 waves: 212 us with no column worth cutting, 191 us with 34 tiles cut.
+int pick_full(faar_ctx* ctx, int mode, int m_tiles, int n_main, int narrow, int bn, int pairs) {
+  const int main = m_tiles * n_main, tail = narrow ? m_tiles : 0;
+  if (bn % 32 != 0 || bn <= 32) return main;
+  if (ctx->tune_tail >= 0) {
+    const long long cut = (long long)(ctx->tune_tail > narrow ? ctx->tune_tail - narrow : 0) * m_tiles;
+    return cut < main ? main - (int)cut : 0;
+  }
+  if (mode != FAAR_GEMM_BWD && main + tail <= pairs) return main;        // the width was chosen for this case (pick_bn)
+  for (const auto& k : ctx->split_plans)
+    if (k.mode == mode && k.m_tiles == m_tiles && k.n_main == n_main && k.narrow == narrow && k.bn == bn) return k.full;
   double best = -1.0;
-  int best_full = n_cols;
-  for (int split = 0; split <= n_cols && split <= 16; ++split) {
-    const int full_cols = n_cols - split;
-    const long long full_tiles = (long long)m_tiles * full_cols;
-    const int rest = N - full_cols * bn;
-    const long long half_tiles = rest > 0 ? (long long)m_tiles * ((rest + bn / 2 - 1) / (bn / 2)) : 0;
-    const long long total = full_tiles + half_tiles;
-    // a pair's load depends on how many full and how many half tiles it gets, which change only at two pair numbers
+  int best_full = main;
+  const int least = main > 2 * pairs ? main - 2 * pairs : 0;
+  for (int full = main; full >= least; --full) {
+    const int total = 2 * main - full + tail;
     double worst = 0.0;
-    const long long cand[3] = {0, full_tiles % pairs, total % pairs};
-    for (long long p : cand) {
+    const int cand[3] = {0, full % pairs, total % pairs};
+    for (int p : cand) {
       if (p >= total) continue;
-      const long long nt = (total - p + pairs - 1) / pairs, nf = full_tiles > p ? (full_tiles - p + pairs - 1) / pairs : 0;
+      const int nt = (total - p + pairs - 1) / pairs, nf = full > p ? (full - p + pairs - 1) / pairs : 0;
       const double last = nt > nf ? 0.75 : 1.0, load = nf + 0.75 * (nt - nf) + 0.4 * last;
       if (load > worst) worst = load;
     }
-    if (best < 0.0 || worst < best - 1e-9) { best = worst; best_full = full_cols; }
+    if (best < 0.0 || worst < best - 1e-9) { best = worst; best_full = full; }
   }
+  auto& slot = ctx->split_plans[ctx->next_plan++ % FAAR_SPLIT_PLANS];
+  slot = {mode, m_tiles, n_main, narrow, bn, best_full};
   return best_full;
 }
 
@@ -1126,7 +1132,10 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   kp.bn = bn;
   kp.stage_bytes = WIDE ? C::STAGE_BYTES : C::A_BYTES + (a->b_mn ? mn_boxes(bn / 2) * MN_BOX_BYTES : (int)faar_align_up((size_t)(bn / 2) * BK * 2, 1024));   // whole swizzle atoms
   kp.stages = C::RING_BYTES / kp.stage_bytes < MAX_STAGES ? C::RING_BYTES / kp.stage_bytes : MAX_STAGES;
-  kp.n_full_cols = WIDE ? 0 : pick_full_cols(ctx, a->M, a->N, bn, max_pairs);
+  const int m_tiles = (a->M + 2 * BM - 1) / (2 * BM), n_cols = (a->N + bn - 1) / bn;
+  kp.narrow = !WIDE && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
+  kp.n_main = n_cols - kp.narrow;
+  kp.n_full = WIDE ? 0 : pick_full(ctx, MODE, m_tiles, kp.n_main, kp.narrow, bn, max_pairs);
   CUtensorMap tmA, tmB, tmBh;
   e = a->a_mn ? make_map_mn(ctx, &tmA, a->A, a->Kc, a->M, a->lda) : make_map(ctx, &tmA, a->A, a->M, a->Kc, a->lda, BM);
   if (e) return e;
@@ -1136,20 +1145,19 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   } else {
     e = make_map(ctx, &tmB, a->B, a->N, a->Kc, a->ldb, bn / 2);
     if (e) return e;
-    if (kp.n_full_cols * bn < a->N) e = make_map(ctx, &tmBh, a->B, a->N, a->Kc, a->ldb, bn % 32 == 0 ? bn / 4 : bn / 2);   // half-width tiles
+    if (kp.narrow || kp.n_full < m_tiles * kp.n_main) e = make_map(ctx, &tmBh, a->B, a->N, a->Kc, a->ldb, bn % 32 == 0 ? bn / 4 : bn / 2);   // half-width tiles
     else tmBh = tmB;
   }
   if (e) return e;
-  const long long m_tiles = (a->M + 2 * BM - 1) / (2 * BM);
-  const int rest_cols = a->N - kp.n_full_cols * bn;
-  const long long tiles = WIDE ? m_tiles * ((a->N + WIDE_BN - 1) / WIDE_BN)
-                               : m_tiles * (kp.n_full_cols + (rest_cols > 0 ? (rest_cols + bn / 2 - 1) / (bn / 2) : 0));
+  const long long tiles = WIDE ? (long long)m_tiles * ((a->N + WIDE_BN - 1) / WIDE_BN)
+                               : 2ll * m_tiles * kp.n_main - kp.n_full + (kp.narrow ? m_tiles : 0);
   const int pairs = (int)(tiles < max_pairs ? tiles : max_pairs);
   cfg.gridDim = dim3(2 * pairs, 1, 1);
   if (n_partials_out) *n_partials_out = 2 * pairs * C::EPI_WARPS;
   ctx->last_gemm_bn = WIDE ? WIDE_BN : bn;
   ctx->last_gemm_pairs = pairs;
-  ctx->last_gemm_split = WIDE ? 0 : (a->N + bn - 1) / bn - kp.n_full_cols;
+  // in columns' worth of tiles
+  ctx->last_gemm_split = WIDE ? 0 : kp.narrow + (m_tiles * kp.n_main - kp.n_full + m_tiles - 1) / m_tiles;
   faar_prof_scope ps(ctx, MODE == FAAR_GEMM_REF ? FAAR_K_GEMM_REF : (MODE == FAAR_GEMM_FWD ? FAAR_K_GEMM_FWD : FAAR_K_GEMM_BWD));
   cudaError_t ce = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmBh, kp);
   if (ce != cudaSuccess) return (int)ce;
@@ -1203,7 +1211,7 @@ int faar_gemm_max_partials(const faar_ctx* ctx, int, int) { return ctx->num_sms 
 
 int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* a, int* n_partials_out) {
   KParams kp;
-  kp.M = a->M; kp.N = a->N; kp.Kc = a->Kc; kp.bn = BN_MAX; kp.n_full_cols = 0; kp.status = a->status;
+  kp.M = a->M; kp.N = a->N; kp.Kc = a->Kc; kp.bn = BN_MAX; kp.n_main = kp.narrow = kp.n_full = 0; kp.status = a->status;
   {
     const long long ysz = a->yout_dtype == FAAR_BF16 ? 2 : 4;
     // the last row ends after its last valid (or padded) column; REF and the transposed FWD layout: [M, ldy], else [N(T), ldy]

@@ -12,6 +12,9 @@
 constexpr int FAAR_GEMM_VARIANTS = 8;     // REF, FWD, BWD x 4 optimiser / chaining variants
 constexpr int FAAR_PAIR_KERNELS = FAAR_GEMM_VARIANTS + 2;   // and the NVFP4 GEMM's 128- and 256-wide tiles
 
+constexpr int FAAR_SPLIT_PLANS = 16;
+struct faar_split_plan { int mode, m_tiles, n_main, narrow, bn, full; };   // GEMM tail split of a tile grid, as chosen
+
 struct faar_ctx {
   int device;
   int num_sms;
@@ -24,6 +27,8 @@ struct faar_ctx {
   int tune_attention_fragments;           // attention: 0 = tcgen05 kernels, 2 = mma.sync kernels (head_dim 64), 1 = the shared-memory fragment kernels
   int last_gemm_bn, last_gemm_pairs, last_gemm_split;   // what the last GEMM launch used
   std::vector<const void*> smem_set;      // kernels whose dynamic shared-memory limit has been raised on this device
+  faar_split_plan split_plans[FAAR_SPLIT_PLANS];          // the last ones used
+  unsigned next_plan;
   // chained steps: the workspace and the beta of the forward operand that the last backward call wrote
   const void* wsoft_ws;
   float wsoft_beta;
