@@ -545,6 +545,59 @@ FAAR_API int faar_attention_bwd(faar_ctx* ctx, int batch, int seq, int n_heads, 
                                 int64_t ldq, const void* k, const void* v, int64_t ldkv, const void* out, const void* dout,
                                 int64_t ldo, const float* lse, float* dsum, void* dq, void* dk, void* dv);
 
+/* ---- passes of a whole decoder model ------------------------------------------------
+ * Procedure steps 16-17 (both forward passes) and 21-23 (backward with the update of every V), each enqueued by one
+ * call: the launches of the entry points above, block by block, without a host round trip per launch.  Linears that
+ * read the same input are one group: their rows are stacked in W and Wsoft, their rounding state stays per linear.
+ * The soft weights a quantised forward pass formed are what the backward pass of the same step reads. */
+typedef struct {
+  int rows;                     /* output features                               */
+  float* V;                     /* [rows, K]; code, scales as elsewhere          */
+  const uint8_t* code;
+  const uint8_t* scales;
+  const float* s_global;
+  float* adam_m;                /* null for gradient descent                     */
+  float* adam_u;
+  float* dV;                    /* [rows, K] out, nullable (backward)            */
+} faar_linear;
+typedef struct {
+  int n;                        /* linears in the group, at most 3               */
+  const void* W;                /* frozen weights, stacked [sum rows, K] bf16    */
+  void* Wsoft;                  /* soft weights, stacked [sum rows, K] bf16      */
+  faar_linear lin[3];
+} faar_linear_group;
+typedef struct {
+  faar_linear_group qkv, o, gate_up, down;
+  const float* attn_norm;       /* [hidden]                                      */
+  const float* mlp_norm;
+} faar_block;
+/* Sizes as in the model's configuration; head_dim 64 or 128; vocab, hidden and ffn multiples of 16.
+ * embed, lm_head: [vocab, hidden] bf16; lm_head_t: [hidden, ld_lm_head_t] bf16, its transpose (backward only);
+ * final_norm: [hidden] float; blocks: host array of n_layers. */
+typedef struct {
+  int vocab, hidden, n_layers, n_heads, n_kv_heads, head_dim, ffn;
+  float eps, theta;
+  const void* embed;
+  const void* lm_head;
+  const void* lm_head_t;
+  int64_t ld_lm_head_t;
+  const float* final_norm;
+  const faar_block* blocks;
+} faar_model;
+/* Bytes of the activation arena of a forward pass (keep != 0: of one whose activations the backward pass will read)
+ * and of the backward pass's scratch memory (host out-pointers; both are caller-owned, 256-byte aligned). */
+FAAR_API int faar_model_sizes(const faar_model* model, int batch, int seq, int keep, size_t* arena_bytes, size_t* scratch_bytes);
+/* tokens, positions: [batch*seq] ints on the device.  quantised = 0: frozen weights; 1: soft weights at temperature beta,
+ * left in every group's Wsoft.  Z out: [batch*seq, vocab] bf16; H out: [batch*seq, hidden] bf16 (after the final norm). */
+FAAR_API int faar_model_forward(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* tokens, const int* positions,
+                                int quantised, float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H,
+                                void* workspace, size_t workspace_bytes);
+/* From the loss gradients at the logits (dZ, row stride ldz) and at the last hidden state (dH) back to every V, which is
+ * updated in place.  arena: of the quantised forward pass with keep != 0 of the same step. */
+FAAR_API int faar_model_backward(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* positions,
+                                 const faar_hparams* hp, void* arena, size_t arena_bytes, const void* dZ, int64_t ldz, const void* dH,
+                                 void* scratch, size_t scratch_bytes, void* workspace, size_t workspace_bytes);
+
 /* ---- GEMM on the deployable operands -----------------------------------------
  * "Hardening and Inference": the hardened weights are NVFP4 tensors that the hardware multiplies as they
  * are.  This call does that on the block-scaled FP4 tensor-core path: C = (sA sB) A B^T, every element of A

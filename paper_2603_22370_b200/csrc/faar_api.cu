@@ -110,6 +110,16 @@ int fwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const v
   return faar_launch_gemm(ctx, &a, n_partials);
 }
 
+// Temperature, optimiser and bias corrections of a dW launch.
+void set_update(faar_gemm_args* a, const faar_hparams* hp) {
+  a->beta = hp->beta;
+  a->lr = hp->lr; a->b1 = hp->beta1; a->b2 = hp->beta2; a->eps = hp->eps; a->opt = hp->opt;
+  if (hp->opt == 1) {
+    a->inv_bc1 = (float)(1.0 / (1.0 - pow((double)hp->beta1, (double)hp->step)));
+    a->inv_bc2 = (float)(1.0 / (1.0 - pow((double)hp->beta2, (double)hp->step)));
+  }
+}
+
 int bwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const void* dYt, const void* Xt,
              float* V, const uint8_t* code, const uint8_t* scales, const float* s_global, float* adam_m,
              float* adam_u, float* dV, uint8_t* ws, const faar_ws_layout& l, int* n_partials,
@@ -138,9 +148,8 @@ int bwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const v
   }
   a.status = reinterpret_cast<uint32_t*>(ws);
   a.partials = reinterpret_cast<float*>(ws + l.off_round_partials);
-  a.V = V; a.code = code; a.scales = scales; a.s_global = s_global;
-  a.adam_m = adam_m; a.adam_u = adam_u; a.dV = dV;
-  a.beta = hp->beta;
+  a.n_seg = 1;
+  a.seg[0] = {V, code, scales, s_global, adam_m, adam_u, dV, (float)((double)hp->lambda_round / ((double)s->O * (double)s->K)), s->O};
   if (hp->beta_next > 0.f) {
     a.wsoft_next = reinterpret_cast<__nv_bfloat16*>(ws + l.off_wsoft);
     a.beta_next = hp->beta_next;
@@ -150,12 +159,7 @@ int bwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const v
     ctx->wsoft_ws = nullptr;               // V moves on without a matching operand
   }
   a.act_scale = hp->act_scale > 0.f ? hp->act_scale : 1.0f;
-  a.lam_over_n = (float)((double)hp->lambda_round / ((double)s->O * (double)s->K));
-  a.lr = hp->lr; a.b1 = hp->beta1; a.b2 = hp->beta2; a.eps = hp->eps; a.opt = hp->opt;
-  if (hp->opt == 1) {
-    a.inv_bc1 = (float)(1.0 / (1.0 - pow((double)hp->beta1, (double)hp->step)));
-    a.inv_bc2 = (float)(1.0 / (1.0 - pow((double)hp->beta2, (double)hp->step)));
-  }
+  set_update(&a, hp);
   return faar_launch_gemm(ctx, &a, n_partials);
 }
 
@@ -201,6 +205,28 @@ faar_prof_scope::faar_prof_scope(faar_ctx* ctx, int kernel_id) : c(ctx), pair(-1
   c->prof_kernel.push_back(kernel_id);
   c->prof_used = i + 1;
   pair = i;
+}
+
+int faar_check_hparams(const faar_hparams* hp, bool need_opt) { return check_hp(hp, need_opt); }
+
+int faar_bwd_group(faar_ctx* ctx, int n_seg, faar_bwd_state* seg, int T, int K, const faar_hparams* hp, const void* dY, int64_t ldy,
+                   const void* X, int64_t ldx, void* workspace) {
+  uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
+  faar_gemm_args a = {};
+  a.mode = FAAR_GEMM_BWD;
+  for (int i = 0; i < n_seg; ++i) {
+    seg[i].lam_over_n = (float)((double)hp->lambda_round / ((double)seg[i].rows * (double)K));
+    a.seg[i] = seg[i];
+    a.M += seg[i].rows;
+  }
+  a.n_seg = n_seg; a.N = K; a.Kc = T;
+  a.A = dY; a.lda = ldy; a.a_mn = 1;
+  a.B = X; a.ldb = ldx; a.b_mn = 1;
+  a.status = reinterpret_cast<uint32_t*>(ws);
+  a.partials = reinterpret_cast<float*>(ws + FAAR_WS_HEADER) + FAAR_MAX_PARTIALS;
+  a.act_scale = hp->act_scale > 0.f ? hp->act_scale : 1.0f;
+  set_update(&a, hp);
+  return faar_launch_gemm(ctx, &a, nullptr);
 }
 
 int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes) {

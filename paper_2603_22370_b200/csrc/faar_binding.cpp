@@ -5,7 +5,8 @@
 // a vectorcall function whose argument conversion is generated from the entry point's own C declaration:
 //   pointer            None, an int (address), or a CUDA tensor (its data_ptr(); a host tensor is refused)
 //   faar_shape /
-//   faar_hparams       the binding's ctypes structure, by its buffer
+//   faar_hparams /
+//   faar_model         the binding's ctypes structure, by its buffer
 //   int, size_t, float Python numbers
 // A function returns the call's status; raising is the Python side's business.  The GIL is released for the call.
 // The module holds no device code and does not link libfaar.so: load(path) opens the library the process binds (the
@@ -63,7 +64,7 @@ template <> struct Arg<float> {
 };
 template <class T> struct Arg<T, std::enable_if_t<std::is_pointer_v<T>>> {
   using E = std::remove_cv_t<std::remove_pointer_t<T>>;
-  static constexpr bool STRUCT = std::is_same_v<E, faar_shape> || std::is_same_v<E, faar_hparams>;
+  static constexpr bool STRUCT = std::is_same_v<E, faar_shape> || std::is_same_v<E, faar_hparams> || std::is_same_v<E, faar_model>;
   T v;
   bool set(PyObject* o) {
     if constexpr (STRUCT) {                        // copied, so nothing is held while the GIL is released
@@ -92,7 +93,7 @@ template <class T> struct Arg<T, std::enable_if_t<std::is_pointer_v<T>>> {
   X(faar_layer_bwd_rowmajor) X(faar_layer_step) X(faar_layer_step_host) X(faar_nvfp4_expand)                              \
   X(faar_layer_step_host_nvfp4) X(faar_harden_pack) X(faar_align_loss) X(faar_swizzle_scales) X(faar_rmsnorm)             \
   X(faar_rmsnorm_bwd) X(faar_add_rmsnorm) X(faar_rmsnorm_bwd_sum) X(faar_rope) X(faar_silu_mul_bwd) X(faar_embedding)     \
-  X(faar_add) X(faar_attention_fwd) X(faar_attention_bwd) X(faar_nvfp4_gemm)
+  X(faar_add) X(faar_attention_fwd) X(faar_attention_bwd) X(faar_nvfp4_gemm) X(faar_model_forward) X(faar_model_backward)
 
 enum {
 #define SLOT(name) SLOT_##name,

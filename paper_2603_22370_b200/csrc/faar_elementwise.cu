@@ -540,6 +540,49 @@ softquant_eval_kernel(const float* __restrict__ V, const uint8_t* __restrict__ c
   }
 }
 
+// The BF16 operand alone, for up to three linears whose output rows are stacked in `out`: one launch for the linears of a
+// decoder block that share an input.  Each segment's bases are moved back by its first group, so that groups of the
+// launch index them; a segment starts at a multiple of eight rows.
+struct SoftSegment { const float* V; const uint8_t* code; const uint8_t* scales; const float* s_global; };
+struct SoftGroup { SoftSegment seg[FAAR_MAX_SEGMENTS]; int64_t end[FAAR_MAX_SEGMENTS - 1]; };
+__global__ void __launch_bounds__(EW_THREADS)
+soft_weights_group_kernel(const __grid_constant__ SoftGroup sg, float beta, int64_t n_groups, __nv_bfloat16* __restrict__ out) {
+  __shared__ float2 lut[16];
+  if (threadIdx.x < 16) {
+    const int k = threadIdx.x & 7;
+    const float sgn = (threadIdx.x & 8) ? -1.f : 1.f;
+    lut[threadIdx.x] = make_float2(sgn * faar_node(k), sgn * faar_width(k));
+  }
+  __syncthreads();
+  faar_pdl_sync();
+  float nbl, hbl;
+  faar_operand_consts(beta, &nbl, &hbl);
+  const float sg0 = *sg.seg[0].s_global, sg1 = *sg.seg[1].s_global, sg2 = *sg.seg[2].s_global;
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n_groups; g += (int64_t)gridDim.x * blockDim.x) {
+    const int i = (g >= sg.end[0]) + (g >= sg.end[1]);
+    const SoftSegment& s = sg.seg[i];
+    const int64_t e = g * 8;
+    const float4* vp = reinterpret_cast<const float4*>(s.V + e);
+    const float4 a = vp[0], b = vp[1];
+    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    const uint32_t cw = *reinterpret_cast<const uint32_t*>(s.code + e / 2);
+    const float sc = __fmul_rn(faar_e4m3_to_float(s.scales[e / 16]), i == 0 ? sg0 : (i == 1 ? sg1 : sg2));
+    uint32_t o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float w[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float2 nw = lut[(cw >> (8 * j + 4 * h)) & 0xF];
+        w[h] = faar_operand_weight(faar_sigmoid_operand(nbl, hbl, v[2 * j + h]), nw.x, nw.y, sc);
+      }
+      const __nv_bfloat162 p2 = __floats2bfloat162_rn(w[0], w[1]);
+      o[j] = *reinterpret_cast<const uint32_t*>(&p2);
+    }
+    *reinterpret_cast<uint4*>(out + e) = make_uint4(o[0], o[1], o[2], o[3]);
+  }
+}
+
 // ---- Round Loss partial sums ------------------------------------------------------------
 __global__ void __launch_bounds__(EW_THREADS)
 round_partials_kernel(const float* __restrict__ V, int64_t N, float* __restrict__ partials) {
@@ -832,6 +875,23 @@ int faar_launch_softquant_eval(faar_ctx* ctx, const faar_shape* s, const float* 
                                   s_global, beta, (int64_t)groups, W_soft, h, W_bf16, W_operand_f32);
   if (e != cudaSuccess) return (int)e;
   return (int)cudaGetLastError();
+}
+
+int faar_launch_soft_weights_group(faar_ctx* ctx, int n_seg, const faar_bwd_state* seg, int K, float beta, __nv_bfloat16* out) {
+  SoftGroup g = {};
+  int64_t row0 = 0;
+  for (int i = 0; i < FAAR_MAX_SEGMENTS; ++i) {
+    if (i) g.end[i - 1] = i < n_seg ? row0 * (K / 8) : INT64_MAX;
+    const faar_bwd_state& b = seg[i < n_seg ? i : 0];
+    const int64_t e0 = i < n_seg ? row0 * K : 0;
+    g.seg[i] = {b.V - e0, b.code - e0 / 2, b.scales - e0 / 16, b.s_global};
+    if (i < n_seg) row0 += b.rows;
+  }
+  const int64_t groups = row0 * (K / 8);
+  faar_prof_scope ps(ctx, FAAR_K_SOFT_WEIGHTS);
+  const cudaError_t e = faar_launch_pdl(ctx, soft_weights_group_kernel, dim3(grid_for(ctx, groups, 8)), dim3(EW_THREADS), 0, g, beta,
+                                        groups, out);
+  return e != cudaSuccess ? (int)e : (int)cudaGetLastError();
 }
 
 int faar_launch_transpose_bf16(faar_ctx* ctx, int rows, int cols, const void* in, int64_t ld_in, void* out,

@@ -247,6 +247,14 @@ __device__ __forceinline__ uint32_t make_idesc(int bn, int a_mn = 0, int b_mn = 
          ((uint32_t)(bn >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
 }
 
+// One linear's per-weight state (faar_bwd_state); the bases are moved back by its first row, so that rows of the launch
+// index them.
+struct Segment {
+  float* V; const uint8_t* code; const uint8_t* scales; const float* s_global;
+  float* adam_m; float* adam_u; float* dV;
+  float lam4;                       // -4 lambda / N: (lambda / N) (4 - 8 v) = lam4 (2 v - 1)
+};
+
 struct KParams {
   int M, N, Kc;
   int bn;                 // tile width
@@ -267,13 +275,12 @@ struct KParams {
   float act_scale;        // FWD: Y_q = act_scale * acc; BWD: G = act_scale * acc
   float* partials;
   // BWD: M = O, N = K
-  float* V; const uint8_t* code; const uint8_t* scales; const float* s_global;
-  float* adam_m; float* adam_u; float* dV;
+  Segment seg[FAAR_MAX_SEGMENTS];
+  int seg_end[FAAR_MAX_SEGMENTS - 1];   // first rows of segments 1 and 2
   // constants of the update, derived once on the host: as kernel parameters they are operands of the instructions that
   // use them and take no registers
   float bl, hbl;                    // beta log2(e) (e^x as 2^(x log2 e)), -bl / 2
   float sbeta;                      // beta act_scale / 2 (the narrowest interval is 0.5 wide)
-  float lam4;                       // -4 lambda / N: (lambda / N) (4 - 8 v) = lam4 (2 v - 1)
   float b1, b2, c1, c2, eps;        // c = 1 - b
   float nstep;                      // -lr / bias correction 1 (Adam), -lr (gradient descent)
   float rbc2;                       // sqrt(u / bc2) = sqrt(u) rbc2
@@ -525,18 +532,18 @@ struct RowState { float4 v, m, u; uint32_t cw, sb; };
 // State of this lane's four weights of instruction `it` of the panel whose row 0 / column 0 is (o_first, k_first), or
 // nothing if they lie outside the matrix or at or beyond column k_end.
 template <int OPT>
-__device__ __forceinline__ bool load_row_state(const KParams& p, int lane, int sub, int o_first, int k_first, int k_end, int it,
+__device__ __forceinline__ bool load_row_state(const KParams& p, const Segment& g, int lane, int sub, int o_first, int k_first, int k_end, int it,
                                                uint64_t stream, RowState& st) {
   const int row = o_first + 8 * sub + lane / LPR + RPI * it, col = k_first + 4 * (lane % LPR);
   const bool ok = row < p.M && col < k_end;
   if (ok) {
     const long long e = (long long)row * p.N + col;
-    st.v = ldg128_stream(p.V + e, stream);
-    st.cw = *reinterpret_cast<const uint16_t*>(p.code + (e >> 1));
-    st.sb = p.scales[e >> 4];
+    st.v = ldg128_stream(g.V + e, stream);
+    st.cw = *reinterpret_cast<const uint16_t*>(g.code + (e >> 1));
+    st.sb = g.scales[e >> 4];
     if (OPT & 1) {
-      st.m = ldg128_stream(p.adam_m + e, stream);
-      st.u = ldg128_stream(p.adam_u + e, stream);
+      st.m = ldg128_stream(g.adam_m + e, stream);
+      st.u = ldg128_stream(g.adam_u + e, stream);
     }
   }
   return ok;
@@ -544,7 +551,7 @@ __device__ __forceinline__ bool load_row_state(const KParams& p, int lane, int s
 // `st` / `st_ok` hold the state of instruction 0 on entry; on return those of instruction 0 of the panel at column
 // k_next (unless k_next >= k_end).
 template <int OPT>
-__device__ __forceinline__ float epi_bwd_rows(const KParams& p, uint32_t panel, int lane, int sub, int o_first,
+__device__ __forceinline__ float epi_bwd_rows(const KParams& p, const Segment& sg, uint32_t panel, int lane, int sub, int o_first,
                                               int k_first, int k_next, int k_end, float s_global, RowState& st, bool& st_ok) {
   const int cu = lane % LPR;                                       // 16-byte unit of the row
   const int r0 = 8 * sub + lane / LPR;                             // this lane's row in the first instruction
@@ -556,8 +563,8 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, uint32_t panel, 
   for (int it = 0; it < ITS; ++it) {
     const RowState cur = st;
     const bool ok = st_ok;
-    st_ok = it + 1 < ITS ? load_row_state<OPT>(p, lane, sub, o_first, k_first, k_end, it + 1, stream, st)
-                         : load_row_state<OPT>(p, lane, sub, o_first, k_next, k_end, 0, stream, st);
+    st_ok = it + 1 < ITS ? load_row_state<OPT>(p, sg, lane, sub, o_first, k_first, k_end, it + 1, stream, st)
+                         : load_row_state<OPT>(p, sg, lane, sub, o_first, k_next, k_end, 0, stream, st);
     {
       if (ok) {
         const int row = r0 + RPI * it;
@@ -595,7 +602,7 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, uint32_t panel, 
           float chain = sbh * __uint_as_float(__float_as_uint(dh) + wexp);
           chain = __uint_as_float(__float_as_uint(chain) ^ sgn);
           const float t = fmaf(2.f, vv[j], -1.f);
-          g[j] = fmaf(G[j], chain, p.lam4 * t);
+          g[j] = fmaf(G[j], chain, sg.lam4 * t);
           tt = fmaf(t, t, tt);
           if (OPT & 1) {
             mn[j] = fmaf(p.b1, mm[j], p.c1 * g[j]);
@@ -615,16 +622,16 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, uint32_t panel, 
           }
         }
         // one check covers the five stores below: they share the element offset e
-        if (!FAAR_DBG_OK(p, p.V + e, 16, p.V, p.ext_state, 3u)) continue;
+        if (!FAAR_DBG_OK(p, sg.V + e, 16, sg.V, p.ext_state, 3u)) continue;
         if ((OPT & 2) && !FAAR_DBG_OK(p, p.wsoft_next + e, 8, p.wsoft_next, p.ext_wsoft, 4u)) continue;
         if (OPT & 2)
           *reinterpret_cast<uint2*>(p.wsoft_next + e) = make_uint2(pack_bf16x2(wn[0], wn[1]), pack_bf16x2(wn[2], wn[3]));
-        if (p.dV) stg128_stream(p.dV + e, g[0], g[1], g[2], g[3], stream);
+        if (sg.dV) stg128_stream(sg.dV + e, g[0], g[1], g[2], g[3], stream);
         if (OPT & 1) {
-          stg128_stream(p.adam_m + e, mn[0], mn[1], mn[2], mn[3], stream);
-          stg128_stream(p.adam_u + e, un[0], un[1], un[2], un[3], stream);
+          stg128_stream(sg.adam_m + e, mn[0], mn[1], mn[2], mn[3], stream);
+          stg128_stream(sg.adam_u + e, un[0], un[1], un[2], un[3], stream);
         }
-        stg128_stream(p.V + e, vn[0], vn[1], vn[2], vn[3], vkeep);
+        stg128_stream(sg.V + e, vn[0], vn[1], vn[2], vn[3], vkeep);
         n_el += 4.f;
       }
     }
@@ -639,7 +646,7 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, uint32_t panel, 
 template <int MODE, int OPT, bool WIDE, int MN>
 __global__ void __launch_bounds__(Cfg<MODE, WIDE>::THREADS, 1)
 faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                 const __grid_constant__ CUtensorMap tmBh, const KParams p) {
+                 const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ KParams p) {
   using C = Cfg<MODE, WIDE>;
   constexpr bool A_MN = (MN & 1) != 0, B_MN = (MN & 2) != 0;
   const int BN = p.bn;
@@ -796,7 +803,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int cg = ew >> 2;                            // which of the warps sharing this lane quarter
     float warp_acc = 0.f;
     float s_global = 0.f;
-    if (MODE == FAAR_GEMM_BWD) s_global = *p.s_global;
+    if (MODE == FAAR_GEMM_BWD) s_global = *p.seg[0].s_global;
     uint32_t pn = 0;                                   // panels this quarter has staged so far
     RowState row_state;                                // BWD: state requested ahead
     bool row_ok = false;
@@ -832,8 +839,13 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
       }
       const int k_end = min(p.N, n0 + TW);               // BWD: columns of this tile that exist
-      if constexpr (MODE == FAAR_GEMM_BWD)
-        row_ok = load_row_state<OPT>(p, lane, ew >> 2, m0 + quarter * 32, n0, k_end, 0, l2_policy_stream(), row_state);
+      // the linear this warp's 8 rows belong to (several only with both operands row-major)
+      const int o_warp = m0 + quarter * 32 + 8 * (ew >> 2);
+      const Segment& seg = p.seg[MODE == FAAR_GEMM_BWD && MN == 3 ? (o_warp >= p.seg_end[0]) + (o_warp >= p.seg_end[1]) : 0];
+      if constexpr (MODE == FAAR_GEMM_BWD) {
+        if (MN == 3) s_global = *seg.s_global;
+        row_ok = load_row_state<OPT>(p, seg, lane, ew >> 2, m0 + quarter * 32, n0, k_end, 0, l2_policy_stream(), row_state);
+      }
       bool ok = mbar_wait(tfull_bar(acc), acc_phase, ac, 0x400u | acc);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -873,7 +885,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
           okp = mbar_wait(pfull, pn & 1u, ac, 0x600u | quarter);
           if (!__all_sync(0xffffffffu, okp)) { dead = true; break; }
-          warp_acc += epi_bwd_rows<OPT>(p, panel, lane, sub, o_first, n0 + pc, n0 + pc + PW, k_end, s_global, row_state, row_ok);
+          warp_acc += epi_bwd_rows<OPT>(p, seg, panel, lane, sub, o_first, n0 + pc, n0 + pc + PW, k_end, s_global, row_state, row_ok);
           __syncwarp();
           if (lane == 0) mbar_arrive(pdone);
           ++pn;
@@ -1228,11 +1240,26 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* a, int* n_partials_out
   kp.Yout = a->Yout; kp.yout_dtype = a->yout_dtype; kp.ldy = a->ldy;
   kp.Yref = a->Yref; kp.yref_dtype = a->yref_dtype; kp.yref_t = a->yref_t;
   kp.dYt = a->dYt; kp.ld_dyt = a->ld_dyt; kp.mse2c = a->mse2c; kp.act_scale = a->act_scale; kp.partials = a->partials;
-  kp.V = a->V; kp.code = a->code; kp.scales = a->scales; kp.s_global = a->s_global;
-  kp.adam_m = a->adam_m; kp.adam_u = a->adam_u; kp.dV = a->dV;
+  if (a->mode == FAAR_GEMM_BWD) {
+    long long row0 = 0;
+    for (int i = 0; i < FAAR_MAX_SEGMENTS; ++i) {
+      Segment& k = kp.seg[i];
+      if (i >= a->n_seg) {
+        k = Segment();
+        if (i) kp.seg_end[i - 1] = 0x7FFFFFFF;
+        continue;
+      }
+      const faar_bwd_state& g = a->seg[i];
+      const long long e0 = row0 * a->N;
+      if (i) kp.seg_end[i - 1] = (int)row0;
+      k.V = g.V - e0; k.code = g.code - e0 / 2; k.scales = g.scales - e0 / 16; k.s_global = g.s_global;
+      k.adam_m = g.adam_m ? g.adam_m - e0 : nullptr; k.adam_u = g.adam_u ? g.adam_u - e0 : nullptr; k.dV = g.dV ? g.dV - e0 : nullptr;
+      k.lam4 = -4.f * g.lam_over_n;
+      row0 += g.rows;
+    }
+  }
   kp.bl = a->beta * 1.44269504088896341f; kp.hbl = -0.5f * kp.bl;
   kp.sbeta = 0.5f * a->beta * a->act_scale;
-  kp.lam4 = -4.f * a->lam_over_n;
   kp.b1 = a->b1; kp.b2 = a->b2; kp.c1 = 1.f - a->b1; kp.c2 = 1.f - a->b2; kp.eps = a->eps;
   kp.nstep = a->opt == 1 ? -(a->lr * a->inv_bc1) : -a->lr;
   kp.rbc2 = sqrtf(a->inv_bc2);

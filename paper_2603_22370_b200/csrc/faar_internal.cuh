@@ -111,6 +111,16 @@ static inline faar_ws_layout faar_ws_plan(const faar_shape* s) {
   return l;
 }
 
+// The per-weight state a dW product updates: one linear, or (row-major operands) up to three whose output rows are
+// stacked, each with its own tensors and Round Loss weight.
+constexpr int FAAR_MAX_SEGMENTS = 3;
+struct faar_bwd_state {
+  float* V; const uint8_t* code; const uint8_t* scales; const float* s_global;
+  float* adam_m; float* adam_u; float* dV;
+  float lam_over_n;
+  int rows;               // output rows of this linear (a multiple of 8 where several are stacked)
+};
+
 // ---- launchers (each returns a cudaError_t as int) ---------------------------
 int faar_launch_softquant_init(faar_ctx*, const faar_shape*, const void* W, float s_global_in,
                                uint8_t* scales, float* s_global_out, uint8_t* code, float* V,
@@ -127,6 +137,8 @@ int faar_launch_softquant_eval(faar_ctx*, const faar_shape*, const float* V, con
                                const uint8_t* scales, const float* s_global, float beta,
                                float* W_soft, float* h, __nv_bfloat16* W_soft_bf16,
                                float* W_operand_f32 = nullptr);
+// BF16 soft weights of up to three linears stacked by output rows (seg: V, code, scales, s_global, rows)
+int faar_launch_soft_weights_group(faar_ctx*, int n_seg, const faar_bwd_state* seg, int K, float beta, __nv_bfloat16* out);
 int faar_launch_act_fakequant(faar_ctx*, int T, int K, const void* X, int64_t ldx, float s_global_in, void* Xq,
                               int64_t ldq, float* s_global_out, uint8_t* packed, uint8_t* scales,
                               unsigned long long* amax_word);
@@ -167,6 +179,12 @@ int faar_launch_harden_pack(faar_ctx*, const faar_shape*, const float* V, const 
                             const uint8_t* scales, const float* s_global, uint8_t* packed,
                             uint8_t* scales_out, uint8_t* decisions, void* W_final, int wfinal_dtype);
 
+// dW products with chain rule and update on row-major operands dY [T, ldy], X [T, ldx]; the segments' rows stacked in dY's
+// columns.  hp has been checked.
+int faar_bwd_group(faar_ctx*, int n_seg, faar_bwd_state* seg, int T, int K, const faar_hparams* hp, const void* dY, int64_t ldy,
+                   const void* X, int64_t ldx, void* workspace);
+int faar_check_hparams(const faar_hparams* hp, bool need_opt);
+
 enum { FAAR_GEMM_REF = 0, FAAR_GEMM_FWD = 1, FAAR_GEMM_BWD = 2 };
 
 struct faar_gemm_args {
@@ -185,9 +203,8 @@ struct faar_gemm_args {
   float act_scale;                             // FWD, BWD: tensor scale of quantised activations (1 = none)
   float* partials;                             // FWD: sum r^2 partials; BWD: Round Loss partials
   // BWD: M = O, N = K
-  float* V; const uint8_t* code; const uint8_t* scales; const float* s_global;
-  float* adam_m; float* adam_u; float* dV;
-  float beta, lam_over_n, lr, b1, b2, eps, inv_bc1, inv_bc2; int opt;
+  int n_seg; faar_bwd_state seg[FAAR_MAX_SEGMENTS];
+  float beta, lr, b1, b2, eps, inv_bc1, inv_bc2; int opt;
   // BWD, optional: also write the next step's BF16 operand W_soft(V', beta_next) (null = not wanted)
   __nv_bfloat16* wsoft_next; float beta_next;
   // BWD, optional: final loss sums by the last CTA (fin_out2 null = not wanted)

@@ -1,0 +1,305 @@
+// Forward and backward passes of a whole decoder model (full-model alignment, Procedure steps 16-17 and 21-23): the
+// sequence of kernel launches for every block, enqueued by one call.  No arithmetic here and no kernels of its own.
+//
+// Why native: a pass is a chain of 25 launches per block, many of a few microseconds each.  Issued one by one from Python
+// they cost 7.5 us of host time each, more than the kernels of a small model take: an alignment step of two 128-wide blocks
+// on 192 tokens took 770 us for 500 us of device time.  Activations live in one caller-owned arena per pass at
+// offsets that depend on the sizes alone.
+#include "faar_internal.cuh"
+
+namespace {
+
+size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+
+struct Sizes {
+  size_t T;
+  int d, qd, kvd, qkv, f, H;
+  size_t seq_rows;                            // floats of one lse array
+};
+Sizes sizes(const faar_model* m, int batch, int seq) {
+  Sizes s;
+  s.T = (size_t)batch * seq;
+  s.d = m->hidden; s.qd = m->n_heads * m->head_dim; s.kvd = m->n_kv_heads * m->head_dim; s.qkv = s.qd + 2 * s.kvd; s.f = m->ffn;
+  s.H = m->n_heads;
+  s.seq_rows = s.T * m->n_heads;
+  return s;
+}
+
+// Byte offsets of a block's saved activations inside its part of the arena.
+struct BlockLayout {
+  size_t x_in, hn, rstd1, qkv, a, lse, x_mid, rstd2, mn, gu, act, bytes;
+  explicit BlockLayout(const Sizes& s) {
+    size_t o = 0;
+    auto take = [&](size_t n) { const size_t at = o; o += align256(n); return at; };
+    x_in = take(s.T * s.d * 2); hn = take(s.T * s.d * 2); rstd1 = take(s.T * 4);
+    qkv = take(s.T * s.qkv * 2); a = take(s.T * s.qd * 2); lse = take(s.seq_rows * 4);
+    x_mid = take(s.T * s.d * 2); rstd2 = take(s.T * 4); mn = take(s.T * s.d * 2);
+    gu = take(s.T * 2 * s.f * 2); act = take(s.T * s.f * 2);
+    bytes = o;
+  }
+};
+// keep: one part per block, then the final norm's input and rstd, then the temporary; otherwise two parts used in turn.
+struct Arena {
+  BlockLayout b;
+  size_t parts, x_last, rstd_f, tmp, total;
+  Arena(const Sizes& s, int n_layers, bool keep) : b(s) {
+    parts = keep ? n_layers : (n_layers < 2 ? n_layers : 2);
+    x_last = parts * b.bytes;
+    rstd_f = x_last + align256(s.T * s.d * 2);
+    tmp = rstd_f + align256(s.T * 4);
+    total = tmp + align256(s.T * s.d * 2);
+  }
+};
+struct Scratch {
+  size_t dhz, dx, dact, dgu, dn, da, dqkv, dsum, total;
+  explicit Scratch(const Sizes& s) {
+    size_t o = 0;
+    auto take = [&](size_t n) { const size_t at = o; o += align256(n); return at; };
+    dhz = take(s.T * s.d * 2); dx = take(s.T * s.d * 2); dact = take(s.T * s.f * 2); dgu = take(s.T * 2 * s.f * 2);
+    dn = take(s.T * s.d * 2); da = take(s.T * s.qd * 2); dqkv = take(s.T * s.qkv * 2); dsum = take(s.seq_rows * 4);
+    total = o;
+  }
+};
+
+// Y[T, O] = X[T, K] W[O, K]^T, or with w_rows_contract: Y[T, O] = X[T, K] W[K, O]
+int product(faar_ctx* ctx, size_t T, int O, int K, const void* X, int64_t ldx, const void* W, int64_t ldw, bool w_rows_contract,
+            void* Y, int64_t ldy, void* ws) {
+  faar_gemm_args a = {};
+  a.mode = FAAR_GEMM_REF;
+  a.M = (int)T; a.N = O; a.Kc = K;
+  a.A = X; a.lda = ldx;
+  a.B = W; a.ldb = ldw; a.b_mn = w_rows_contract;
+  a.status = reinterpret_cast<uint32_t*>(ws);
+  a.Yout = Y; a.yout_dtype = FAAR_BF16; a.ldy = ldy;
+  return faar_launch_gemm(ctx, &a, nullptr);
+}
+
+int group_rows(const faar_linear_group& g) {
+  int r = 0;
+  for (int i = 0; i < g.n; ++i) r += g.lin[i].rows;
+  return r;
+}
+int segments(const faar_linear_group& g, faar_bwd_state (&seg)[FAAR_MAX_SEGMENTS]) {
+  for (int i = 0; i < g.n; ++i) {
+    const faar_linear& l = g.lin[i];
+    seg[i] = {l.V, l.code, l.scales, l.s_global, l.adam_m, l.adam_u, l.dV, 0.f, l.rows};
+  }
+  return g.n;
+}
+// A group's forward product: frozen weights, or soft weights formed first.
+int group_forward(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* X, bool quantised, float beta, void* Y, void* ws) {
+  const int rows = group_rows(g);
+  if (quantised) {
+    faar_bwd_state seg[FAAR_MAX_SEGMENTS];
+    const int n = segments(g, seg);
+    const int e = faar_launch_soft_weights_group(ctx, n, seg, K, beta, reinterpret_cast<__nv_bfloat16*>(g.Wsoft));
+    if (e) return e;
+  }
+  return product(ctx, T, rows, K, X, K, quantised ? g.Wsoft : g.W, K, false, Y, rows, ws);
+}
+// A group's backward: the gradient towards the common input, then the update of every V (at the pre-update soft weights).
+int group_backward(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp,
+                   void* dX, void* ws) {
+  const int rows = group_rows(g);
+  int e = product(ctx, T, K, rows, dY, rows, g.Wsoft, K, true, dX, K, ws);
+  if (e) return e;
+  faar_bwd_state seg[FAAR_MAX_SEGMENTS];
+  const int n = segments(g, seg);
+  return faar_bwd_group(ctx, n, seg, (int)T, K, hp, dY, rows, X, K, ws);
+}
+
+bool aligned(const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+int check_group(const faar_linear_group& g, int n, const int* rows, bool quantised, const faar_hparams* hp) {
+  if (g.n != n) return FAAR_ERR_INVALID_ARG;
+  if (quantised ? !aligned(g.Wsoft) : !aligned(g.W)) return g.W || g.Wsoft ? FAAR_ERR_ALIGN : FAAR_ERR_INVALID_ARG;
+  for (int i = 0; i < n; ++i) {
+    const faar_linear& l = g.lin[i];
+    if (l.rows != rows[i]) return FAAR_ERR_SHAPE;
+    if (!quantised) continue;
+    if (!l.V || !l.code || !l.scales || !l.s_global) return FAAR_ERR_INVALID_ARG;
+    if (hp && hp->opt == 1 && (!l.adam_m || !l.adam_u)) return FAAR_ERR_INVALID_ARG;
+    if (!aligned(l.V) || !aligned(l.code) || (l.adam_m && !aligned(l.adam_m)) || (l.adam_u && !aligned(l.adam_u)) ||
+        (l.dV && !aligned(l.dV)))
+      return FAAR_ERR_ALIGN;
+  }
+  return FAAR_OK;
+}
+int check_model(const faar_ctx* ctx, const faar_model* m, int batch, int seq, bool quantised, const faar_hparams* hp, const void* ws,
+                size_t ws_bytes) {
+  if (!ctx || !m || !m->blocks || !m->embed || !m->lm_head || !m->final_norm) return FAAR_ERR_INVALID_ARG;
+  if (batch <= 0 || seq <= 0 || (long long)batch * seq > 0x7FFFFFFFll || m->n_layers <= 0 || m->n_heads <= 0 || m->n_kv_heads <= 0 ||
+      m->n_heads % m->n_kv_heads || (m->head_dim != 64 && m->head_dim != 128))
+    return FAAR_ERR_SHAPE;
+  if (m->vocab <= 0 || m->vocab % 16 || m->hidden <= 0 || m->hidden % 16 || m->ffn <= 0 || m->ffn % 16) return FAAR_ERR_SHAPE;
+  if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < FAAR_WS_HEADER + 2 * sizeof(float) * FAAR_MAX_PARTIALS)
+    return FAAR_ERR_WORKSPACE;
+  const int qd = m->n_heads * m->head_dim, kvd = m->n_kv_heads * m->head_dim;
+  const int qkv[3] = {qd, kvd, kvd}, one[1] = {m->hidden}, gu[2] = {m->ffn, m->ffn};
+  for (int l = 0; l < m->n_layers; ++l) {
+    const faar_block& b = m->blocks[l];
+    if (!b.attn_norm || !b.mlp_norm) return FAAR_ERR_INVALID_ARG;
+    int st = check_group(b.qkv, 3, qkv, quantised, hp);
+    if (!st) st = check_group(b.o, 1, one, quantised, hp);
+    if (!st) st = check_group(b.gate_up, 2, gu, quantised, hp);
+    if (!st) st = check_group(b.down, 1, one, quantised, hp);
+    if (st) return st;
+  }
+  return FAAR_OK;
+}
+
+int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* pos, bool quantised, float beta,
+            bool keep, uint8_t* arena, void* Z, void* Hout, void* ws) {
+  const Sizes s = sizes(m, batch, seq);
+  const Arena A(s, m->n_layers, keep);
+  const int T = (int)s.T;
+  auto part = [&](int l) { return arena + (keep ? l : l % (int)A.parts) * A.b.bytes; };
+  uint8_t* const tmp = arena + A.tmp;
+  uint8_t* p = part(0);
+  int e = faar_launch_embedding(ctx, T, s.d, m->vocab, m->embed, s.d, tokens, p + A.b.x_in, s.d);
+  if (!e)
+    e = faar_launch_rmsnorm(ctx, T, s.d, p + A.b.x_in, s.d, nullptr, 0, nullptr, 0, m->blocks[0].attn_norm, m->eps, p + A.b.hn, s.d,
+                            reinterpret_cast<float*>(p + A.b.rstd1));
+  for (int l = 0; l < m->n_layers && !e; ++l) {
+    const faar_block& b = m->blocks[l];
+    p = part(l);
+    __nv_bfloat16* const qkv = reinterpret_cast<__nv_bfloat16*>(p + A.b.qkv);
+    e = group_forward(ctx, b.qkv, s.T, s.d, p + A.b.hn, quantised, beta, qkv, ws);
+    // q and k lie side by side: their heads turn in one launch
+    if (!e) e = faar_launch_rope(ctx, T, m->n_heads + m->n_kv_heads, m->head_dim, qkv, s.qkv, pos, m->theta, 0, qkv, s.qkv);
+    if (!e)
+      e = faar_launch_attention_fwd(ctx, batch, seq, m->n_heads, m->n_kv_heads, m->head_dim, qkv, s.qkv, qkv + s.qd, qkv + s.qd + s.kvd,
+                                    s.qkv, p + A.b.a, s.qd, reinterpret_cast<float*>(p + A.b.lse));
+    if (!e) e = group_forward(ctx, b.o, s.T, s.qd, p + A.b.a, quantised, beta, tmp, ws);
+    // residual connection and the MLP's norm in one pass
+    if (!e)
+      e = faar_launch_rmsnorm(ctx, T, s.d, p + A.b.x_in, s.d, tmp, s.d, p + A.b.x_mid, s.d, b.mlp_norm, m->eps, p + A.b.mn, s.d,
+                              reinterpret_cast<float*>(p + A.b.rstd2));
+    __nv_bfloat16* const gu = reinterpret_cast<__nv_bfloat16*>(p + A.b.gu);
+    if (!e) e = group_forward(ctx, b.gate_up, s.T, s.d, p + A.b.mn, quantised, beta, gu, ws);
+    if (!e) e = faar_launch_silu_mul(ctx, T, s.f, gu, 2 * s.f, gu + s.f, 2 * s.f, p + A.b.act, s.f);
+    if (!e) e = group_forward(ctx, b.down, s.T, s.f, p + A.b.act, quantised, beta, tmp, ws);
+    if (e) break;
+    // residual connection and the next block's attention norm (after the last block: the final norm)
+    const bool last = l + 1 == m->n_layers;
+    uint8_t* const n = last ? nullptr : part(l + 1);
+    e = faar_launch_rmsnorm(ctx, T, s.d, p + A.b.x_mid, s.d, tmp, s.d, last ? arena + A.x_last : n + A.b.x_in, s.d,
+                            last ? m->final_norm : m->blocks[l + 1].attn_norm, m->eps, last ? Hout : n + A.b.hn, s.d,
+                            reinterpret_cast<float*>(last ? arena + A.rstd_f : n + A.b.rstd1));
+  }
+  if (!e) e = product(ctx, s.T, m->vocab, s.d, Hout, s.d, m->lm_head, s.d, false, Z, m->vocab, ws);
+  return e;
+}
+
+int backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* pos, const faar_hparams* hp, uint8_t* arena,
+             const void* dZ, int64_t ldz, const void* dH, uint8_t* scratch, void* ws) {
+  const Sizes s = sizes(m, batch, seq);
+  const Arena A(s, m->n_layers, true);
+  const Scratch S(s);
+  const int T = (int)s.T;
+  uint8_t* const dx = scratch + S.dx;
+  // LM head (frozen): dH += dZ W_lm, then the final norm
+  int e = product(ctx, s.T, s.d, m->vocab, dZ, ldz, m->lm_head_t, m->ld_lm_head_t, false, scratch + S.dhz, s.d, ws);
+  if (!e)
+    e = faar_launch_rmsnorm_bwd(ctx, T, s.d, scratch + S.dhz, dH, nullptr, s.d, arena + A.x_last, s.d, m->final_norm,
+                                reinterpret_cast<const float*>(arena + A.rstd_f), nullptr, 0, dx, s.d);
+  for (int l = m->n_layers - 1; l >= 0 && !e; --l) {
+    const faar_block& b = m->blocks[l];
+    uint8_t* const p = arena + (size_t)l * A.b.bytes;
+    const __nv_bfloat16* const gu = reinterpret_cast<const __nv_bfloat16*>(p + A.b.gu);
+    __nv_bfloat16* const dgu = reinterpret_cast<__nv_bfloat16*>(scratch + S.dgu);
+    // MLP branch: x = x_mid + act W_down^T
+    e = group_backward(ctx, b.down, s.T, s.f, dx, p + A.b.act, hp, scratch + S.dact, ws);
+    if (!e)
+      e = faar_launch_silu_mul_bwd(ctx, T, s.f, scratch + S.dact, s.f, gu, 2 * s.f, gu + s.f, 2 * s.f, dgu, 2 * s.f, dgu + s.f, 2 * s.f);
+    if (!e) e = group_backward(ctx, b.gate_up, s.T, s.d, dgu, p + A.b.mn, hp, scratch + S.dn, ws);
+    if (!e)
+      e = faar_launch_rmsnorm_bwd(ctx, T, s.d, scratch + S.dn, nullptr, nullptr, s.d, p + A.b.x_mid, s.d, b.mlp_norm,
+                                  reinterpret_cast<const float*>(p + A.b.rstd2), dx, s.d, dx, s.d);
+    // attention branch: x_mid = x_in + a W_o^T
+    if (!e) e = group_backward(ctx, b.o, s.T, s.qd, dx, p + A.b.a, hp, scratch + S.da, ws);
+    const __nv_bfloat16* const qkv = reinterpret_cast<const __nv_bfloat16*>(p + A.b.qkv);
+    __nv_bfloat16* const dqkv = reinterpret_cast<__nv_bfloat16*>(scratch + S.dqkv);
+    if (!e)
+      e = faar_launch_attention_bwd(ctx, batch, seq, m->n_heads, m->n_kv_heads, m->head_dim, qkv, s.qkv, qkv + s.qd, qkv + s.qd + s.kvd,
+                                    s.qkv, p + A.b.a, scratch + S.da, s.qd, reinterpret_cast<const float*>(p + A.b.lse),
+                                    reinterpret_cast<float*>(scratch + S.dsum), dqkv, dqkv + s.qd, dqkv + s.qd + s.kvd);
+    if (!e) e = faar_launch_rope(ctx, T, m->n_heads + m->n_kv_heads, m->head_dim, dqkv, s.qkv, pos, m->theta, 1, dqkv, s.qkv);
+    if (!e) e = group_backward(ctx, b.qkv, s.T, s.d, dqkv, p + A.b.hn, hp, scratch + S.dn, ws);
+    if (!e)
+      e = faar_launch_rmsnorm_bwd(ctx, T, s.d, scratch + S.dn, nullptr, nullptr, s.d, p + A.b.x_in, s.d, b.attn_norm,
+                                  reinterpret_cast<const float*>(p + A.b.rstd1), dx, s.d, dx, s.d);
+  }
+  return e;
+}
+
+// The context's device is current for the duration of a call.
+struct Device {
+  int prev = -1, err = 0;
+  explicit Device(int dev) {
+    cudaError_t e = cudaGetDevice(&prev);
+    if (e == cudaSuccess && prev != dev) e = cudaSetDevice(dev); else if (e == cudaSuccess) prev = -1;
+    if (e != cudaSuccess) { err = (int)e; prev = -1; }
+  }
+  ~Device() { if (prev >= 0) (void)cudaSetDevice(prev); }
+};
+int status(faar_ctx* ctx, int e) {
+  if (e == 0) return FAAR_OK;
+  ctx->last_cuda_error = e;
+  return FAAR_ERR_CUDA;
+}
+
+}  // namespace
+
+extern "C" {
+
+int faar_model_sizes(const faar_model* m, int batch, int seq, int keep, size_t* arena_bytes, size_t* scratch_bytes) {
+  if (!m || !arena_bytes || !scratch_bytes) return FAAR_ERR_INVALID_ARG;
+  if (batch <= 0 || seq <= 0 || m->n_layers <= 0 || m->hidden <= 0 || m->ffn <= 0 || m->n_heads <= 0 || m->n_kv_heads <= 0 || m->head_dim <= 0)
+    return FAAR_ERR_SHAPE;
+  const Sizes s = sizes(m, batch, seq);
+  *arena_bytes = Arena(s, m->n_layers, keep != 0).total;
+  *scratch_bytes = Scratch(s).total;
+  return FAAR_OK;
+}
+
+int faar_model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, int quantised,
+                       float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, void* workspace,
+                       size_t workspace_bytes) {
+  int st = check_model(ctx, m, batch, seq, quantised != 0, nullptr, workspace, workspace_bytes);
+  if (st) return st;
+  if (!tokens || !positions || !arena || !Z || !H) return FAAR_ERR_INVALID_ARG;
+  if (quantised && !(beta > 0.f)) return FAAR_ERR_INVALID_ARG;
+  if (!aligned(Z) || !aligned(H) || (reinterpret_cast<uintptr_t>(arena) & 255u)) return FAAR_ERR_ALIGN;
+  size_t need = 0, scratch = 0;
+  if ((st = faar_model_sizes(m, batch, seq, keep, &need, &scratch))) return st;
+  if (arena_bytes < need) return FAAR_ERR_WORKSPACE;
+  Device dev(ctx->device);
+  if (dev.err) return status(ctx, dev.err);
+  return status(ctx, forward(ctx, m, batch, seq, tokens, positions, quantised != 0, beta, keep != 0, reinterpret_cast<uint8_t*>(arena), Z, H,
+                             workspace));
+}
+
+int faar_model_backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* positions, const faar_hparams* hp,
+                        void* arena, size_t arena_bytes, const void* dZ, int64_t ldz, const void* dH, void* scratch,
+                        size_t scratch_bytes, void* workspace, size_t workspace_bytes) {
+  int st = faar_check_hparams(hp, true);
+  if (st) return st;
+  st = check_model(ctx, m, batch, seq, true, hp, workspace, workspace_bytes);
+  if (st) return st;
+  if (!positions || !arena || !dZ || !dH || !scratch || !m->lm_head_t) return FAAR_ERR_INVALID_ARG;
+  if (ldz < m->vocab || m->ld_lm_head_t < m->vocab) return FAAR_ERR_SHAPE;
+  if (!aligned(dZ) || !aligned(dH) || ldz % 8 || m->ld_lm_head_t % 8 || (reinterpret_cast<uintptr_t>(arena) & 255u) ||
+      (reinterpret_cast<uintptr_t>(scratch) & 255u))
+    return FAAR_ERR_ALIGN;
+  size_t need = 0, need_s = 0;
+  if ((st = faar_model_sizes(m, batch, seq, 1, &need, &need_s))) return st;
+  if (arena_bytes < need || scratch_bytes < need_s) return FAAR_ERR_WORKSPACE;
+  Device dev(ctx->device);
+  if (dev.err) return status(ctx, dev.err);
+  if (ctx->wsoft_ws == workspace) ctx->wsoft_ws = nullptr;
+  return status(ctx, backward(ctx, m, batch, seq, positions, hp, reinterpret_cast<uint8_t*>(arena), dZ, ldz, dH,
+                              reinterpret_cast<uint8_t*>(scratch), workspace));
+}
+
+}  // extern "C"

@@ -74,6 +74,9 @@ SIGNATURES = {
     "faar_tune_wide_tiles": (_I, [_P, _I]),
     "faar_attention_fwd": (_I, [_P, _I, _I, _I, _I, _I, _P, _L, _P, _P, _L, _P, _L, _P]),
     "faar_attention_bwd": (_I, [_P, _I, _I, _I, _I, _I, _P, _L, _P, _P, _L, _P, _P, _L, _P, _P, _P, _P, _P]),
+    "faar_model_sizes": (_I, [_P, _I, _I, _I, _P, _P]),
+    "faar_model_forward": (_I, [_P, _P, _I, _I, _P, _P, _I, _F, _I, _P, _Z, _P, _P, _P, _Z]),
+    "faar_model_backward": (_I, [_P, _P, _I, _I, _P, _P, _P, _Z, _P, _L, _P, _P, _Z, _P, _Z]),
     "faar_nvfp4_gemm": (_I, [_P, _I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _L, _P, _Z]),
 }
 EXPORTS = list(SIGNATURES)
@@ -89,6 +92,26 @@ class Shape(C.Structure):
     _fields_ = [("O", C.c_int), ("K", C.c_int), ("T", C.c_int), ("ldw", C.c_int64), ("ldx", C.c_int64),
                 ("ldxt", C.c_int64), ("ldy", C.c_int64), ("w_dtype", C.c_int), ("yref_dtype", C.c_int),
                 ("yref_transposed", C.c_int)]
+
+
+class Linear(C.Structure):
+    _fields_ = [("rows", C.c_int), ("V", _P), ("code", _P), ("scales", _P), ("s_global", _P), ("adam_m", _P), ("adam_u", _P),
+                ("dV", _P)]
+
+
+class LinearGroup(C.Structure):
+    _fields_ = [("n", C.c_int), ("W", _P), ("Wsoft", _P), ("lin", Linear * 3)]
+
+
+class Block(C.Structure):
+    _fields_ = [("qkv", LinearGroup), ("o", LinearGroup), ("gate_up", LinearGroup), ("down", LinearGroup), ("attn_norm", _P),
+                ("mlp_norm", _P)]
+
+
+class Model(C.Structure):
+    _fields_ = [("vocab", C.c_int), ("hidden", C.c_int), ("n_layers", C.c_int), ("n_heads", C.c_int), ("n_kv_heads", C.c_int),
+                ("head_dim", C.c_int), ("ffn", C.c_int), ("eps", C.c_float), ("theta", C.c_float), ("embed", _P), ("lm_head", _P),
+                ("lm_head_t", _P), ("ld_lm_head_t", C.c_int64), ("final_norm", _P), ("blocks", _P)]
 
 
 class FaarError(RuntimeError):
@@ -352,6 +375,23 @@ def attention_bwd(ctx, batch, seq, n_heads, n_kv_heads, head_dim, q, ldq, k, v, 
 def nvfp4_gemm(ctx, M, N, K, A_packed, A_scales_tiled, A_s_global, B_packed, B_scales_tiled, B_s_global, C, ldc, ws):
     _check(_fast().faar_nvfp4_gemm(ctx._n, M, N, K, A_packed, A_scales_tiled, A_s_global, B_packed, B_scales_tiled,
            B_s_global, C, ldc, ws, ws.numel()), "faar_nvfp4_gemm")
+
+
+def model_sizes(model: Model, batch: int, seq: int, keep: int) -> tuple[int, int]:
+    """(arena bytes, scratch bytes) of a pass over the model."""
+    a, b = C.c_size_t(0), C.c_size_t(0)
+    _check(lib().faar_model_sizes(C.byref(model), batch, seq, keep, C.byref(a), C.byref(b)), "faar_model_sizes")
+    return a.value, b.value
+
+
+def model_forward(ctx, model, batch, seq, tokens, positions, quantised, beta, keep, arena, Z, H, ws):
+    _check(_fast().faar_model_forward(ctx._n, model, batch, seq, tokens, positions, int(quantised), beta, int(keep), arena,
+                                      arena.numel(), Z, H, ws, ws.numel()), "faar_model_forward")
+
+
+def model_backward(ctx, model, batch, seq, positions, hp, arena, dZ, ldz, dH, scratch, ws):
+    _check(_fast().faar_model_backward(ctx._n, model, batch, seq, positions, hp, arena, arena.numel(), dZ, ldz, dH, scratch,
+                                       scratch.numel(), ws, ws.numel()), "faar_model_backward")
 
 
 def transpose_bf16(ctx, rows, cols, inp, ld_in, out, ld_out):

@@ -1,19 +1,21 @@
 """Stage-2 driver: full-model alignment (Eq. 6, Procedure steps 15-24) of a Llama-style decoder model whose
-linears all carry their own rounding tensor V.  Host loop and buffer management only: every arithmetic step --
-embedding, norms, rotary embedding, attention, the gated MLP, every matrix product, the loss with its gradients,
-the chain rule into V, the optimiser update -- is a call into the CUDA library through `faar`.
+linears all carry their own rounding tensor V.  Buffer management only: every arithmetic step -- embedding, norms, rotary
+embedding, attention, the gated MLP, every matrix product, the loss with its gradients, the chain rule into V, the
+optimiser update -- is done by the CUDA library, whose faar_model_forward / faar_model_backward enqueue a whole pass.
 
 One step (`Stage2Model.step`):
   frozen model forward (BF16 weights)                      -> Z_fp, H_fp            Procedure 16
   quantised model forward (Eq. 2 soft weights of every V)  -> Z_q, H_q, activations Procedure 17
   faar_align_loss                                          -> L_KL, L_MSE, dZ_q, dH_q   Procedure 18-20, Eq. 6
-  backward through the quantised model; per linear: input gradient dX = dY W_soft (faar_layer_dx_operand on the
-  forward pass's soft weights, i.e. at the pre-update V), then dW GEMM + chain rule + Round Loss gradient + optimiser update + clip (faar_layer_bwd)
+  backward through the quantised model; per group of linears with a common input: input gradient dX = dY W_soft on the
+  forward pass's soft weights, i.e. at the pre-update V, then dW GEMM + chain rule + Round Loss gradient + optimiser
+  update + clip
                                                                                      Procedure 21-23
 Embedding, norms and LM head are frozen and stay in BF16 / FP32; the seven linears of every block are quantised.
 """
 from __future__ import annotations
 
+import ctypes
 from dataclasses import dataclass
 
 import torch
@@ -102,146 +104,81 @@ class Stage2Model:
         self.aws = torch.empty(faar.align_loss_workspace_size(T, c.vocab), dtype=torch.uint8, device=dev)
         faar.workspace_init(ctx, self.aws)
         self.loss = torch.zeros(2, dtype=torch.float32, device=dev)
-        self.ldt = (T + 7) // 8 * 8
-        self.dsum = torch.empty((batch, c.n_heads, seq), dtype=torch.float32, device=dev)
         self.step_count = 0
+        self._addresses, self._model, self._blocks = None, None, None
+        table = self._table()
+        self.arena_bytes = {bool(k): faar.model_sizes(table, batch, seq, k)[0] for k in (0, 1)}
+        self.scratch_bytes = faar.model_sizes(table, batch, seq, 1)[1]
 
     # ---- helpers ------------------------------------------------------------------------------------
     def _new(self, cols, dtype=torch.bfloat16):
         return torch.empty((self.T, cols), dtype=dtype, device=self.dev)
 
-    def _matmul(self, X, W):
-        """Y[T, O] = X[T, K] W[O, K]^T on the tensor cores (the frozen-target GEMM)."""
-        O, K = W.shape
-        Y = self._new(O)
-        faar.layer_ref(self.ctx, faar.make_shape(O, K, self.T), X, W, Y, self.ws)
-        return Y
+    def _groups(self, l):
+        """(field, names, frozen weights, soft weights) of a block's groups of linears with a common input."""
+        lin, wg, wsg = self.lin[l], self.w_group[l], self.wsoft_group[l]
+        return (("qkv", GROUPS["qkv"], wg["qkv"], wsg["qkv"]), ("o", ("o_proj",), lin["o_proj"].W, lin["o_proj"].Wsoft),
+                ("gate_up", GROUPS["gate_up"], wg["gate_up"], wsg["gate_up"]),
+                ("down", ("down_proj",), lin["down_proj"].W, lin["down_proj"].Wsoft))
 
-    def _linear_group(self, l, group, X, quantised, beta):
-        """The linears of one group on their common input: one product with the stacked weights.  Returns the
-        [T, sum of widths] result; each linear's output is a column range of it."""
-        if not quantised:
-            return self._matmul(X, self.w_group[l][group])
-        for n in GROUPS[group]:
-            lin = self.lin[l][n]
-            faar.softquant_eval(self.ctx, faar.make_shape(lin.O, lin.K, self.T), lin.V, lin.code, lin.scales, lin.s_global,
-                                beta, None, None, lin.Wsoft)
-        return self._matmul(X, self.wsoft_group[l][group])
-
-    def _linear(self, l, name, X, quantised, beta):
-        lin = self.lin[l][name]
-        if not quantised:
-            return self._matmul(X, lin.W)
-        faar.softquant_eval(self.ctx, faar.make_shape(lin.O, lin.K, self.T), lin.V, lin.code, lin.scales, lin.s_global, beta,
-                            None, None, lin.Wsoft)
-        return self._matmul(X, lin.Wsoft)
+    def _table(self) -> faar.Model:
+        """The model as the library takes it: addresses of the tensors that the attributes hold now, read on every call
+        (the structure is only rebuilt if one of them has moved)."""
+        p = self.params
+        held = [p["embed"], p["lm_head"], p["final_norm"], self.lm_head_t]
+        for l, lins in enumerate(self.lin):
+            held += (p[f"attn_norm.{l}"], p[f"mlp_norm.{l}"], *self.w_group[l].values(), *self.wsoft_group[l].values())
+            for x in lins.values():
+                held += (x.W, x.Wsoft, x.V, x.code, x.scales, x.s_global, x.m, x.u)
+        addresses = [0 if t is None else t.data_ptr() for t in held]
+        if addresses == self._addresses:
+            return self._model
+        assert all(t is None or t.is_cuda for t in held), "device tensors only"
+        c, ptr = self.cfg, lambda t: None if t is None else t.data_ptr()
+        blocks = (faar.Block * c.n_layers)()
+        for l in range(c.n_layers):
+            for field, names, W, Wsoft in self._groups(l):
+                g = getattr(blocks[l], field)
+                g.n, g.W, g.Wsoft = len(names), ptr(W), ptr(Wsoft)
+                for i, n in enumerate(names):
+                    x = self.lin[l][n]
+                    g.lin[i] = faar.Linear(x.O, ptr(x.V), ptr(x.code), ptr(x.scales), ptr(x.s_global), ptr(x.m), ptr(x.u), None)
+            blocks[l].attn_norm, blocks[l].mlp_norm = ptr(p[f"attn_norm.{l}"]), ptr(p[f"mlp_norm.{l}"])
+        self._blocks, self._addresses = blocks, addresses
+        self._model = faar.Model(c.vocab, c.hidden, c.n_layers, c.n_heads, c.n_kv_heads, c.head_dim, c.ffn, c.eps, c.theta,
+                                 ptr(p["embed"]), ptr(p["lm_head"]), ptr(self.lm_head_t), self.lm_head_t.shape[1],
+                                 ptr(p["final_norm"]), ctypes.addressof(blocks))
+        return self._model
 
     # ---- forward -------------------------------------------------------------------------------------
     def forward(self, tokens: torch.Tensor, quantised: bool, beta: float = 4.0, keep: bool = False):
-        """tokens: [batch*seq] int32 on the device.  Returns (Z [T, vocab], H [T, hidden], cache or None)."""
-        c, ctx, T = self.cfg, self.ctx, self.T
-        d, qd, kvd, f = c.hidden, c.n_heads * c.head_dim, c.n_kv_heads * c.head_dim, c.ffn
-        x = self._new(d)
-        faar.embedding(ctx, T, d, c.vocab, self.params["embed"], d, tokens, x, d)
-        cache = []
-        hn, rstd1 = self._new(d), torch.empty(T, dtype=torch.float32, device=self.dev)
-        faar.rmsnorm(ctx, T, d, x, d, self.params["attn_norm.0"], c.eps, hn, d, rstd1)
-        for l in range(c.n_layers):
-            s = {"x_in": x, "rstd1": rstd1}
-            qkv = self._linear_group(l, "qkv", hn, quantised, beta)
-            ldp = qkv.shape[1]
-            q, k, v = qkv[:, :qd], qkv[:, qd:qd + kvd], qkv[:, qd + kvd:]
-            faar.rope(ctx, T, c.n_heads, c.head_dim, q, ldp, self.pos, c.theta, 0, q, ldp)
-            faar.rope(ctx, T, c.n_kv_heads, c.head_dim, k, ldp, self.pos, c.theta, 0, k, ldp)
-            a = self._new(qd)
-            lse = torch.empty((self.batch, c.n_heads, self.seq), dtype=torch.float32, device=self.dev)
-            faar.attention_fwd(ctx, self.batch, self.seq, c.n_heads, c.n_kv_heads, c.head_dim, q, ldp, k, v, ldp, a, qd, lse)
-            o = self._linear(l, "o_proj", a, quantised, beta)
-            # residual connection and the MLP's norm in one pass
-            x_mid, mn, s["rstd2"] = self._new(d), self._new(d), torch.empty(T, dtype=torch.float32, device=self.dev)
-            faar.add_rmsnorm(ctx, T, d, x, d, o, d, x_mid, d, self.params[f"mlp_norm.{l}"], c.eps, mn, d, s["rstd2"])
-            gu = self._linear_group(l, "gate_up", mn, quantised, beta)
-            g, u = gu[:, :f], gu[:, f:]
-            act = self._new(f)
-            faar.silu_mul(ctx, T, f, g, 2 * f, u, 2 * f, act, f)
-            dn = self._linear(l, "down_proj", act, quantised, beta)
-            if keep:
-                s.update(hn=hn, q=q, k=k, v=v, a=a, lse=lse, x_mid=x_mid, mn=mn, g=g, u=u, act=act)
-                cache.append(s)
-            # residual connection and the next block's attention norm (after the last block: the final norm)
-            g_next = self.params[f"attn_norm.{l + 1}"] if l + 1 < c.n_layers else self.params["final_norm"]
-            x, hn, rstd1 = self._new(d), self._new(d), torch.empty(T, dtype=torch.float32, device=self.dev)
-            faar.add_rmsnorm(ctx, T, d, x_mid, d, dn, d, x, d, g_next, c.eps, hn, d, rstd1)
-        H, rstd_f = hn, rstd1
-        Z = self._matmul(H, self.params["lm_head"])
-        return Z, H, ((cache, x, rstd_f) if keep else None)
+        """tokens: [batch*seq] int32 on the device.  Returns (Z [T, vocab], H [T, hidden], activations or None)."""
+        model = self._table()
+        arena = torch.empty(self.arena_bytes[bool(keep)], dtype=torch.uint8, device=self.dev)
+        Z, H = self._new(self.cfg.vocab), self._new(self.cfg.hidden)
+        faar.model_forward(self.ctx, model, self.batch, self.seq, tokens, self.pos, quantised, beta, keep, arena, Z, H, self.ws)
+        return Z, H, (arena if keep else None)
 
     # ---- backward ------------------------------------------------------------------------------------
-    def _update(self, l, name, dY, ldy, X, hp, want_dv):
-        """dW GEMM of one quantised linear with the chain rule into V, the Round Loss gradient, the optimiser update
-        and the clip.  dY [T, O] (row stride ldy) and X [T, K] as the backward pass holds them: no transposed
-        copies.  Returns dV or None."""
-        lin = self.lin[l][name]
-        shape = faar.make_shape(lin.O, lin.K, self.T, ldxt=self.ldt, ldy=ldy)
-        dV = torch.empty((lin.O, lin.K), dtype=torch.float32, device=self.dev) if want_dv else None
-        faar.layer_bwd_rowmajor(self.ctx, shape, hp, dY, X, lin.V, lin.code, lin.scales, lin.s_global, lin.m, lin.u, dV, self.ws)
-        return dV
-
-    def _linear_bwd(self, l, name, dY, X, hp, want_dv):
-        """One quantised linear: dX = dY W_soft at the pre-update V, then its update.  Returns (dX, dV or None)."""
-        lin = self.lin[l][name]
-        dX = self._new(lin.K)
-        # lin.Wsoft still holds this step's soft weights: V changes only in the update below
-        faar.layer_dx_operand(self.ctx, faar.make_shape(lin.O, lin.K, self.T), dY, lin.Wsoft, dX, self.ws)
-        return dX, self._update(l, name, dY, lin.O, X, hp, want_dv)
-
-    def _group_bwd(self, l, group, dY, X, hp, want_dv, grads):
-        """The linears of one group: the gradient towards their common input is one product of the stacked output
-        gradients dY [T, sum of widths] with the stacked soft weights (the sum over the linears is the contraction),
-        then each linear's update from its column range of dY."""
-        K = self.lin[l][GROUPS[group][0]].K
-        dX = self._new(K)
-        faar.layer_dx_operand(self.ctx, faar.make_shape(dY.shape[1], K, self.T), dY, self.wsoft_group[l][group], dX, self.ws)
-        c0 = 0
-        for n in GROUPS[group]:
-            O = self.lin[l][n].O
-            grads[(l, n)] = self._update(l, n, dY[:, c0:c0 + O], dY.shape[1], X, hp, want_dv)
-            c0 += O
-        return dX
-
     def backward(self, dZ, dH, saved, hp, want_dv=False):
         """From the loss gradients at the logits and at the last hidden state back to every V (updated in place).
         Follows the quantised forward pass of the same step: every linear's Wsoft buffer is read as that pass left it.
         Returns {(l, name): dV} if want_dv."""
-        c, ctx, T = self.cfg, self.ctx, self.T
-        d, qd, kvd, f = c.hidden, c.n_heads * c.head_dim, c.n_kv_heads * c.head_dim, c.ffn
-        cache, x_last, rstd_f = saved
+        model = self._table()
         grads = {}
-        # LM head (frozen): dH += dZ W_lm, then the final norm
-        dHz = self._new(d)
-        faar.layer_ref(ctx, faar.make_shape(d, self.lm_head_t.shape[1], T, ldw=self.lm_head_t.shape[1], ldx=dZ.shape[1]), dZ,
-                       self.lm_head_t, dHz, self.ws)
-        dx = self._new(d)
-        faar.rmsnorm_bwd_sum(ctx, T, d, dHz, dH, None, d, x_last, d, self.params["final_norm"], rstd_f, None, d, dx, d)
-        for l in reversed(range(c.n_layers)):
-            s = cache[l]
-            # MLP branch: x = x_mid + act W_down^T
-            dact, grads[(l, "down_proj")] = self._linear_bwd(l, "down_proj", dx, s["act"], hp, want_dv)
-            dgu = self._new(2 * f)
-            faar.silu_mul_bwd(ctx, T, f, dact, f, s["g"], 2 * f, s["u"], 2 * f, dgu[:, :f], 2 * f, dgu[:, f:], 2 * f)
-            dmn = self._group_bwd(l, "gate_up", dgu, s["mn"], hp, want_dv, grads)
-            faar.rmsnorm_bwd(ctx, T, d, dmn, d, s["x_mid"], d, self.params[f"mlp_norm.{l}"], s["rstd2"], dx, d, dx, d)
-            # attention branch: x_mid = x_in + a W_o^T
-            da, grads[(l, "o_proj")] = self._linear_bwd(l, "o_proj", dx, s["a"], hp, want_dv)
-            dqkv = self._new(qd + 2 * kvd)
-            ldp = qd + 2 * kvd
-            dq, dk, dv = dqkv[:, :qd], dqkv[:, qd:qd + kvd], dqkv[:, qd + kvd:]
-            faar.attention_bwd(ctx, self.batch, self.seq, c.n_heads, c.n_kv_heads, c.head_dim, s["q"], ldp, s["k"], s["v"], ldp,
-                               s["a"], da, qd, s["lse"], self.dsum, dq, dk, dv)
-            faar.rope(ctx, T, c.n_heads, c.head_dim, dq, ldp, self.pos, c.theta, 1, dq, ldp)
-            faar.rope(ctx, T, c.n_kv_heads, c.head_dim, dk, ldp, self.pos, c.theta, 1, dk, ldp)
-            dhn = self._group_bwd(l, "qkv", dqkv, s["hn"], hp, want_dv, grads)
-            faar.rmsnorm_bwd(ctx, T, d, dhn, d, s["x_in"], d, self.params[f"attn_norm.{l}"], s["rstd1"], dx, d, dx, d)
+        if want_dv:
+            for l in range(self.cfg.n_layers):
+                for field, names, _, _ in self._groups(l):
+                    for i, n in enumerate(names):
+                        x = self.lin[l][n]
+                        grads[(l, n)] = torch.empty((x.O, x.K), dtype=torch.float32, device=self.dev)
+                        getattr(self._blocks[l], field).lin[i].dV = grads[(l, n)].data_ptr()
+        scratch = torch.empty(self.scratch_bytes, dtype=torch.uint8, device=self.dev)
+        try:
+            faar.model_backward(self.ctx, model, self.batch, self.seq, self.pos, hp, saved, dZ, dZ.shape[1], dH, scratch, self.ws)
+        finally:
+            if want_dv:
+                self._addresses = None               # the structure holds the gradients' addresses: build it anew
         return grads if want_dv else None
 
     # ---- one step of Eq. 6 -----------------------------------------------------------------------------
