@@ -838,6 +838,11 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (col_begin + 16 * q < col_end) { yraw[2 * q] = y4[2 * q]; yraw[2 * q + 1] = y4[2 * q + 1]; }
         }
       }
+      // FWD otherwise: the target values of the warp's first 16 columns (the others one chunk ahead of their use)
+      float ynext[MODE == FAAR_GEMM_FWD ? 16 : 1];
+      if constexpr (MODE == FAAR_GEMM_FWD) {
+        if (!yvec && col_begin < col_end && n0 + col_begin < p.N) load_yref(p, o, n0 + col_begin, ynext);
+      }
       const int k_end = min(p.N, n0 + TW);               // BWD: columns of this tile that exist
       // the linear this warp's 8 rows belong to (several only with both operands row-major)
       const int o_warp = m0 + quarter * 32 + 8 * (ew >> 2);
@@ -917,7 +922,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (n0 + c >= p.N) break;                    // warp-uniform
             uint32_t r[16];
             tmem_ld16(trow + (uint32_t)c, r);
-            if (MODE == FAAR_GEMM_REF) {
+            if constexpr (MODE == FAAR_GEMM_REF) {
               const bool second = c + 16 < col_end && n0 + c + 16 < p.N;
               uint32_t r2[16];
               if (second) tmem_ld16(trow + (uint32_t)(c + 16), r2);
@@ -925,9 +930,11 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               epi_ref(p, o, n0 + c, r);
               if (second) epi_ref(p, o, n0 + c + 16, r2);
             } else {
-              tmem_ld_wait();
               float yr[16];
-              load_yref(p, o, n0 + c, yr);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) yr[j] = ynext[j];
+              if (c + 16 < col_end && n0 + c + 16 < p.N) load_yref(p, o, n0 + c + 16, ynext);
+              tmem_ld_wait();
               warp_acc += epi_fwd(p, o, n0 + c, r, yr);
             }
           }
@@ -963,9 +970,9 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       if (threadIdx.x == 0) {
         __threadfence();                                     // this CTA's partials, ordered by the barrier above
         int last = 0;
-        // after a wait that gave up the partials are incomplete: no final sums (the caller re-initialises
-        // the workspace, which also clears this counter)
-        if (*reinterpret_cast<volatile uint32_t*>(p.status) == 0u) {
+        // after a wait that gave up this CTA's partials are incomplete: it does not count, so nobody forms final sums
+        // (the caller re-initialises the workspace, which also clears this counter)
+        if (!*abort_flag) {
           const uint32_t prev = atomicAdd(p.fin_counter, 1u);
           last = prev == gridDim.x - 1;
           if (last) *p.fin_counter = 0u;                     // ready for the next launch
@@ -1050,14 +1057,15 @@ int make_map_mn(faar_ctx* ctx, CUtensorMap* map, const void* ptr, int kc_rows, i
 // width.  A smaller problem is a matter of latency: its tiles run at once, each brings its share of the epilogue, and
 // narrower tiles spread that over more SMs.
 // REF, FWD: the width with the smallest estimated time of the busiest pair (microseconds).  A k block costs the ring's
-// latency, or what the L2 needs for all pairs' operands (about 10 TB/s); the epilogue 0.4 / 0.6 per 64 columns.
+// latency, or what the L2 needs for all pairs' operands (about 14 TB/s); the epilogue per 64 columns 0.4 (REF), 0.6 (FWD with
+// a transposed BF16 target) or 1.5 (FWD otherwise); a further wave of tiles 1.
 // Measured (width before -> after): product [260, 1024] over 512 8.8 -> 6.2 us (128 -> 32), forward kernel of a
 // 128 x 256 layer at 1024 tokens 12.8 -> 10.7 us, input gradient [192, 128] over 384 11.1 -> 8.9 us.
 // BWD: its per-weight epilogue is bound by instruction issue and a tile of it has a fixed cost of several microseconds,
 // so only 128-wide tiles (cut into halves of 64 by pick_full while pairs are idle) while fewer than half of the
 // pairs would have a 256-wide one; 32-wide tiles: dW kernel of a 128 x 256 layer 19.2 -> 18.8 us, of a 1024 x 3600 layer
 // 33.6 -> 51 us.
-int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs, bool b_mn) {
+int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs, bool b_mn, bool fwd_vec) {
   if (ctx->tune_bn >= 128 && ctx->tune_bn <= BN_MAX && ctx->tune_bn % 16 == 0)
     return b_mn ? (ctx->tune_bn + 31) / 32 * 32 : ctx->tune_bn;      // a CTA's first column of an N-contiguous B: 32-byte aligned
   const long long m_tiles = (M + 2 * BM - 1) / (2 * BM);
@@ -1067,16 +1075,16 @@ int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs
   }
   const int widest = N > 128 ? (N < BN_MAX ? (N + 31) / 32 * 32 : BN_MAX) : (N > 64 ? 128 : (N > 32 ? 64 : 32));
   if (m_tiles * ((N + widest - 1) / widest) >= pairs) return widest;
-  const double epi64 = mode == FAAR_GEMM_FWD ? 0.6 : 0.4;
+  const double epi64 = mode == FAAR_GEMM_FWD ? (fwd_vec ? 0.6 : 1.5) : 0.4;
   int best = widest;
   double best_cost = 1e30;
   for (int bn = widest; bn >= 32; bn = bn > 128 ? 128 : bn / 2) {
     const long long tiles = m_tiles * ((N + bn - 1) / bn);
     const long long waves = (tiles + pairs - 1) / pairs, active = tiles < pairs ? tiles : pairs;
-    const double l2 = 2.0 * active * (BM + bn / 2) * BK * 2 / 1e7;
+    const double l2 = 2.0 * active * (BM + bn / 2) * BK * 2 / 1.4e7;
     const double latency = bn > 128 ? 0.22 : (bn > 64 ? 0.19 : 0.16);
     const double loop = k_blocks * (l2 > latency ? l2 : latency), epi = epi64 * bn / 64.0;
-    const double cost = waves * loop + epi + (waves - 1) * (epi > loop ? epi - loop : 0.0);
+    const double cost = waves * loop + epi + (waves - 1) * (1.0 + (epi > loop ? epi - loop : 0.0));
     if (cost < best_cost - 1e-9) { best_cost = cost; best = bn; }
   }
   return best;
@@ -1118,15 +1126,19 @@ int pick_full(faar_ctx* ctx, int mode, int m_tiles, int n_main, int narrow, int 
   return best_full;
 }
 
-// Whether a launch takes 256 x 512 tiles (see Cfg): only on request (ctx->tune_wide == 1) and where the shape
-// allows.  Measured: on a down_proj-shaped layer (2048 x 8192, 4096 tokens) in a short job at full clocks the
-// forward GEMM gains 1-4 % (64 tiles in one wave instead of 128 in two unequal ones), but in the long,
-// power-capped jobs of whole decoder blocks the same launch and the q / o projections lose 6-10 %; the dW GEMM
-// loses 29 % (its long epilogue is no longer hidden) and the plain product loses whenever it needs more than
-// one wave.  No rule was found that wins consistently, so the default never takes them.
-bool pick_wide(const faar_ctx* ctx, int mode, int M, int N, int bn) {
-  const int tokens = mode == FAAR_GEMM_REF && M > N ? M : N;           // REF may have the tokens as its rows
-  return ctx->tune_wide == 1 && bn == BN_MAX && tokens > BN_MAX;
+// Whether a launch takes 256 x 512 tiles (see Cfg): on request (ctx->tune_wide == 1) wherever the shape allows;
+// otherwise, for plain products and the forward product, where they turn two waves of 256-wide tiles into one of twice
+// the width, which pulls a quarter less operand data through the SMs and leaves fewer of them idle: forward kernel of a
+// 2048 x 8192 layer at 4096 tokens (128 tiles on 74 pairs -> 64) 137 -> 123 us, product [2000, 4096] over 2048 37 -> 32 us.
+// With more waves their epilogue, which nothing overlaps, costs more than that: gate/up at 8192 tokens 406 -> 477 us, the
+// forward kernel of an 8192 x 2048 layer 143 -> 168 us; the dW product's epilogue always does (173 -> 198 us).  The second
+// half's epilogue has to be earned by the main loop: the forward kernel of a 2048 x 2048 layer (32 k blocks) 40 -> 45 us.
+bool pick_wide(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int pairs) {
+  if (bn != BN_MAX || ctx->tune_wide == 0) return false;
+  if (ctx->tune_wide == 1) return (mode == FAAR_GEMM_REF && M > N ? M : N) > BN_MAX;    // REF may have the tokens as its rows
+  const long long m_tiles = (M + 2 * BM - 1) / (2 * BM);
+  return (mode == FAAR_GEMM_FWD ? k_blocks >= 64 : mode == FAAR_GEMM_REF && k_blocks >= 24) && N > BN_MAX && ctx->tune_tail < 0 && ctx->tune_bn == 0 && m_tiles * ((N + BN_MAX - 1) / BN_MAX) > pairs &&
+         m_tiles * ((N + WIDE_BN - 1) / WIDE_BN) <= pairs;
 }
 
 template <int MODE, int OPT, bool WIDE, int MN>
@@ -1196,7 +1208,8 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
   const int e = faar_allow_smem(ctx, (const void*)kern, C::SMEM_BYTES);
   if (e) return e;
   const int max_pairs = faar_max_pairs(ctx, MODE == FAAR_GEMM_BWD ? 2 + OPT : MODE, (const void*)kern, &cfg);
-  const int bn = pick_bn(ctx, MODE, a->M, a->N, (a->Kc + BK - 1) / BK, max_pairs, a->b_mn != 0);
+  const int bn = pick_bn(ctx, MODE, a->M, a->N, (a->Kc + BK - 1) / BK, max_pairs, a->b_mn != 0,
+                          a->yref_t && a->yref_dtype == FAAR_BF16 && !a->Yout);
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
   // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient), the dW
   // product with B or with both untransposed
@@ -1208,7 +1221,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
     if (mn == 3) return launch_variant<MODE, OPT, false, 3>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   }
   if (mn != 0) return (int)cudaErrorInvalidValue;
-  if (pick_wide(ctx, MODE, a->M, a->N, bn)) return launch_variant<MODE, OPT, true, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+  if (pick_wide(ctx, MODE, a->M, a->N, (a->Kc + BK - 1) / BK, bn, max_pairs)) return launch_variant<MODE, OPT, true, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   return launch_variant<MODE, OPT, false, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
 }
 

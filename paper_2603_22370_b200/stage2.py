@@ -153,7 +153,9 @@ class Stage2Model:
     # ---- forward -------------------------------------------------------------------------------------
     def forward(self, tokens: torch.Tensor, quantised: bool, beta: float = 4.0, keep: bool = False):
         """tokens: [batch*seq] int32 on the device.  Returns (Z [T, vocab], H [T, hidden], activations or None)."""
-        model = self._table()
+        return self._forward(self._table(), tokens, quantised, beta, keep)
+
+    def _forward(self, model: faar.Model, tokens, quantised, beta=4.0, keep=False):
         arena = torch.empty(self.arena_bytes[bool(keep)], dtype=torch.uint8, device=self.dev)
         Z, H = self._new(self.cfg.vocab), self._new(self.cfg.hidden)
         faar.model_forward(self.ctx, model, self.batch, self.seq, tokens, self.pos, quantised, beta, keep, arena, Z, H, self.ws)
@@ -164,7 +166,9 @@ class Stage2Model:
         """From the loss gradients at the logits and at the last hidden state back to every V (updated in place).
         Follows the quantised forward pass of the same step: every linear's Wsoft buffer is read as that pass left it.
         Returns {(l, name): dV} if want_dv."""
-        model = self._table()
+        return self._backward(self._table(), dZ, dH, saved, hp, want_dv)
+
+    def _backward(self, model: faar.Model, dZ, dH, saved, hp, want_dv):
         grads = {}
         if want_dv:
             for l in range(self.cfg.n_layers):
@@ -188,14 +192,15 @@ class Stage2Model:
         self.loss (device).  fp_outputs = (Z_fp, H_fp) reuses a frozen-model forward of the same batch.  want_dv: also
         return the quantised model's outputs, the loss gradients and every linear's dV (for inspection)."""
         self.step_count += 1
-        Z_fp, H_fp = fp_outputs if fp_outputs is not None else self.forward(tokens, quantised=False)[:2]
-        Z_q, H_q, saved = self.forward(tokens, quantised=True, beta=beta, keep=True)
+        model = self._table()
+        Z_fp, H_fp = fp_outputs if fp_outputs is not None else self._forward(model, tokens, quantised=False)[:2]
+        Z_q, H_q, saved = self._forward(model, tokens, quantised=True, beta=beta, keep=True)
         c, T = self.cfg, self.T
         dZ, dH = torch.empty_like(Z_q), torch.empty_like(H_q)
         faar.align_loss(self.ctx, T, c.vocab, c.hidden, Z_fp, Z_q, Z_q.shape[1], H_fp, H_q, c.hidden, tau, lambda_kl, dZ, dH,
                         self.loss, self.aws)
         hp = faar.make_hparams(beta=beta, lambda_round=lambda_round, opt=self.opt, lr=lr, step=self.step_count)
-        grads = self.backward(dZ, dH, saved, hp, want_dv)
+        grads = self._backward(model, dZ, dH, saved, hp, want_dv)
         return {"Z_q": Z_q, "H_q": H_q, "dZ": dZ, "dH": dH, "dV": grads} if want_dv else None
 
     def round_loss_sum(self) -> float:
