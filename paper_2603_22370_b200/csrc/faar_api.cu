@@ -237,17 +237,18 @@ int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes) {
   return (int)e;
 }
 
-int faar_max_pairs(faar_ctx* c, int slot, const void* kernel, cudaLaunchConfig_t* cfg) {
+int faar_max_clusters(faar_ctx* c, int slot, int size, const void* kernel, cudaLaunchConfig_t* cfg) {
   constexpr int DEVICES = 64;
-  static std::atomic<int> known[DEVICES][FAAR_PAIR_KERNELS];       // 0 = not asked yet
+  static std::atomic<int> known[DEVICES][FAAR_PAIR_KERNELS][FAAR_CLUSTER_SIZES];       // 0 = not asked yet
   const bool keep = c->device < DEVICES;
-  int n = keep ? known[c->device][slot].load(std::memory_order_relaxed) : 0;
+  int n = keep ? known[c->device][slot][size].load(std::memory_order_relaxed) : 0;
   if (n) return n;
-  cfg->gridDim = dim3(2 * (c->num_sms / 2), 1, 1);
+  const int ctas = 2 << size, most = c->num_sms / ctas;
+  cfg->gridDim = dim3(ctas * most, 1, 1);
   const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kernel, cfg);
-  if (e != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = c->num_sms / 2; }
-  if (n > c->num_sms / 2) n = c->num_sms / 2;
-  if (keep) known[c->device][slot].store(n, std::memory_order_relaxed);
+  if (e != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = size ? 1 : most; }
+  if (n > most) n = most;
+  if (keep) known[c->device][slot][size].store(n, std::memory_order_relaxed);
   return n;
 }
 

@@ -391,7 +391,7 @@ int launch4(faar_ctx* ctx, const uint8_t* A, const uint8_t* sfa, const uint8_t* 
   cfg.numAttrs = 2;
   int e = faar_allow_smem(ctx, (const void*)kern, C4::SMEM);
   if (e) return e;
-  const int max_pairs = faar_max_pairs(ctx, FAAR_GEMM_VARIANTS + (BN == 256), (const void*)kern, &cfg);
+  const int max_pairs = faar_max_clusters(ctx, FAAR_GEMM_VARIANTS + (BN == 256), 0, (const void*)kern, &cfg);
   CUtensorMap tmA, tmB, tmSA, tmSB;
   e = byte_map(ctx, &tmA, A, p.M, p.K, TM);
   if (!e) e = byte_map(ctx, &tmB, B, p.N, p.K, BN / 2);

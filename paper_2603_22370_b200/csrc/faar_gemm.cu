@@ -13,6 +13,10 @@
 //                                "empty" / "accumulator full" barriers of both CTAs)
 //   warps 2..   : epilogue      (tcgen05.ld; two accumulator buffers, so the epilogue of one tile
 //                                overlaps the main loop of the next)
+// A launch with few tiles and a long contraction splits it (p.splits = 2 or 4): the pairs of a cluster of 4 or 8 CTAs take
+// a part of the k blocks of the SAME tile each, then every CTA sends the accumulator columns that are another pair's
+// to finish to that pair's CTA of the same rows (distributed shared memory, into the idle operand ring) and finishes its
+// own share of the columns, adding the parts in a fixed order (see exchange_parts).
 // The three epilogues are the operations of the layer step:
 //   REF : Y_fp = X W^T                                   (Procedure step 8)
 //   FWD : r = Y_q - Y_ref, sum r^2, dY = 2c r -> dY^T     (steps 9-10, Eq. 5 first term)
@@ -98,6 +102,16 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
+// the same with what the arriving threads of other CTAs wrote before visible here
+__device__ __forceinline__ uint32_t mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+  return done;
+}
 __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t done;
   asm volatile(
@@ -137,6 +151,24 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, const
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const AbortCtl& ac, uint32_t code) {
   if (mbar_try_wait(bar, parity)) return true;
   return mbar_wait_slow(bar, parity, ac, code);
+}
+
+__device__ __noinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, const AbortCtl& ac, uint32_t code) {
+  const unsigned long long t0 = global_ns();
+  for (uint32_t spin = 1;; ++spin) {
+    if (mbar_try_wait_cluster(bar, parity)) return true;
+    if ((spin & 0xFF) == 0) {
+      if (*ac.flag) return false;
+      if (global_ns() - t0 > ac.limit_ns) {
+        atomicCAS(ac.status, 0u, code);
+        *ac.flag = 1;
+        return false;
+      }
+    }
+  }
+}
+__device__ __forceinline__ void sts128_cluster(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
 // 2-D tiled TMA load into this CTA's shared memory; the byte count is credited to `bar`, which may be
@@ -181,9 +213,10 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// When all MMAs issued so far have completed, arrive on the barrier at offset `bar` in both CTAs.
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
-  const uint16_t mask = 3;
+// When all MMAs issued so far have completed, arrive on the barrier at offset `bar` in both CTAs of the pair whose leader
+// has cluster rank `leader`.
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint32_t leader) {
+  const uint16_t mask = (uint16_t)(3u << leader);
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(bar), "h"(mask) : "memory");
 }
@@ -259,6 +292,7 @@ struct KParams {
   int M, N, Kc;
   int bn;                 // tile width
   int stages, stage_bytes;   // ring depth, bytes of a stage (both CTAs alike)
+  int splits;             // CTA pairs that share a tile's contraction: 1, or 2 / 4 (one tile per cluster then)
   int n_main;             // tile columns of bn; a last column with at most bn/2 columns of the matrix (narrow) is extra
   int narrow;             // 1: there is such a column; its tiles are bn/2 wide
   int n_full;             // the first n_full tiles of the main columns are bn wide, the others come as two halves (tail split)
@@ -639,14 +673,69 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, const Segment& s
   return n_el - tt;                                               // sum of 1 - (2 v - 1)^2
 }
 
+// ---- split contraction -----------------------------------------------------------------------
+// What arrives from the other pairs lies in the operand ring as [part][4 columns][row] of 16 bytes: a warp, one row per
+// lane, reads and writes consecutive 16-byte units.
+__device__ __forceinline__ uint32_t part_unit(uint32_t ring, int slot, int cols, int unit, int row) {
+  return ring + (uint32_t)(((slot * (cols >> 2) + unit) * BM + row) << 4);
+}
+// One epilogue warp's share of the exchange: `trow` is the warp's lane quarter of the tile's accumulator, `cols` the
+// columns each pair finishes.  False: a wait gave up.  Barriers: `bar_free`, the other pairs' CTAs have nothing in flight
+// into (or out of) their rings any more; `bar_recv`, their parts have arrived here.
+__device__ __forceinline__ bool exchange_parts(uint32_t trow, int cols, int splits, int split, uint32_t prank, uint32_t ring,
+                                               uint32_t bar_free, uint32_t bar_recv, int quarter, int cg, int groups, int ew, int lane,
+                                               const AbortCtl& ac) {
+  if (ew == 0 && lane < splits && lane != split) mbar_arrive_cluster(map_to_cta(bar_free, 2u * (uint32_t)lane + prank));
+  bool ok = mbar_wait_cluster(bar_free, 0u, ac, 0x800u);
+  if (!__all_sync(0xffffffffu, ok)) return false;
+  const int chunks = cols / 16, row = quarter * 32 + lane;
+  int i = 0;
+  for (int d = 0; d < splits; ++d) {
+    if (d == split) continue;
+    const int slot = split < d ? split : split - 1;
+    for (int c = 0; c < chunks; ++c, ++i) {
+      if (i % groups != cg) continue;
+      uint32_t r[16];
+      tmem_ld16(trow + (uint32_t)(d * cols + 16 * c), r);
+      tmem_ld_wait();
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        sts128_cluster(map_to_cta(part_unit(ring, slot, cols, 4 * c + u, row), 2u * (uint32_t)d + prank), r[4 * u], r[4 * u + 1],
+                       r[4 * u + 2], r[4 * u + 3]);
+    }
+  }
+  asm volatile("fence.acq_rel.cluster;" ::: "memory");
+  __syncwarp();
+  if (lane < splits && lane != split) mbar_arrive_cluster(map_to_cta(bar_recv, 2u * (uint32_t)lane + prank));
+  ok = mbar_wait_cluster(bar_recv, 0u, ac, 0x810u);
+  return __all_sync(0xffffffffu, ok);
+}
+// r += what the other pairs sent for the 16 columns from `c` (of this pair's share) of this lane's row
+__device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t ring, int splits, int cols, int c, int row) {
+  for (int slot = 0; slot + 1 < splits; ++slot) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float4 v = lds128(part_unit(ring, slot, cols, (c >> 2) + u, row));
+      r[4 * u] = __float_as_uint(__uint_as_float(r[4 * u]) + v.x);
+      r[4 * u + 1] = __float_as_uint(__uint_as_float(r[4 * u + 1]) + v.y);
+      r[4 * u + 2] = __float_as_uint(__uint_as_float(r[4 * u + 2]) + v.z);
+      r[4 * u + 3] = __float_as_uint(__uint_as_float(r[4 * u + 3]) + v.w);
+    }
+  }
+}
+
 // ---- the kernel ------------------------------------------------------------------------------
-// Launched as clusters of two CTAs along x: CTAs 2c and 2c+1 form pair c.
+// Launched as clusters of 2 * splits CTAs along x; CTAs 2c and 2c+1 form a pair.
 // MN: bit 0 = the A operand, bit 1 = the B operand is stored with its M / N index contiguous (KParams.a_mn / b_mn);
 // a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.
-template <int MODE, int OPT, bool WIDE, int MN>
-__global__ void __launch_bounds__(Cfg<MODE, WIDE>::THREADS, 1)
+// SHAPE: 0 = tiles of up to 256 columns, WIDE_TILES, SPLIT_TILES; at compile time for the same reason.
+constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2;
+constexpr int MIN_SPLIT_BLOCKS = 24;            // contractions of fewer k blocks stay whole (see pick_splits)
+template <int MODE, int OPT, int SHAPE, int MN>
+__global__ void __launch_bounds__(Cfg<MODE, SHAPE == WIDE_TILES>::THREADS, 1)
 faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ KParams p) {
+  constexpr bool WIDE = SHAPE == WIDE_TILES, SPLIT = SHAPE == SPLIT_TILES;
   using C = Cfg<MODE, WIDE>;
   constexpr bool A_MN = (MN & 1) != 0, B_MN = (MN & 2) != 0;
   const int BN = p.bn;
@@ -669,12 +758,17 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const AbortCtl ac{abort_flag, p.status};
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();             // 0 = leader of the pair
-  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int splits = SPLIT ? p.splits : 1;
+  const uint32_t crank = cluster_ctarank();
+  const uint32_t rank = SPLIT ? crank & 1u : crank, leader = SPLIT ? crank & ~1u : 0u;   // rank 0 = leader of the pair
+  const int split = SPLIT ? (int)(crank >> 1) : 0;     // this pair's part of the contraction
+  const int pair = blockIdx.x / (2 * splits), n_pairs = gridDim.x / (2 * splits);      // (clusters, with splits > 1)
   const int m_tiles = (p.M + 2 * BM - 1) / (2 * BM);
   // WIDE: tiles of 512 columns, numbered row block fastest; no tail split
   const int total_tiles = WIDE ? m_tiles * ((p.N + WIDE_BN - 1) / WIDE_BN) : tile_count(p, m_tiles);
   const int k_blocks = (p.Kc + BK - 1) / BK;
+  const int kb0 = SPLIT ? k_blocks * split / splits : 0, kb1 = SPLIT ? k_blocks * (split + 1) / splits : k_blocks;
+  const uint32_t bar_free = ctl_u32 + 208u, bar_recv = ctl_u32 + 216u;                  // SPLIT: see exchange_parts
 
   if (threadIdx.x == 64) {                             // the copies' descriptors, fetched during the set-up
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
@@ -684,6 +778,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     // accumulator-empty barriers are used in the leader only: every epilogue warp of both CTAs arrives there
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 2 * C::EPI_WARPS); }
+    if (SPLIT) { mbar_init(bar_free, splits - 1); mbar_init(bar_recv, (splits - 1) * C::EPI_WARPS); }
     for (int q = 0; q < 8; ++q) mbar_init(ctl_u32 + 256u + 8u * q, 4);   // panel staged / panel consumed, per lane quarter
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -716,7 +811,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int m0 = tc.m0 + (int)rank * BM;
         const int n0 = tc.n0 + (int)rank * (tc.w / 2);
         const CUtensorMap* mapB = tc.w == BN ? &tmB : &tmBh;      // box of w/2 rows
-        for (int kb = 0; kb < k_blocks; ++kb) {
+        for (int kb = kb0; kb < kb1; ++kb) {
           ok = mbar_wait(empty_bar(stage), phase ^ 1u, ac, 0x100u | stage);
           if (!ok) break;
           const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + C::A_BYTES;
@@ -724,7 +819,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           if (rank == 0)
             mbar_expect_tx(full_bar(stage), WIDE ? 2u * (uint32_t)(C::A_BYTES + C::B_BYTES)
                                                  : 2u * (uint32_t)(C::A_BYTES + (B_MN ? mn_boxes(tc.w / 2) * MN_BOX : tc.w / 2) * BK * 2));
-          const uint32_t leader_full = map_to_cta(full_bar(stage), 0);
+          const uint32_t leader_full = map_to_cta(full_bar(stage), leader);
           if (A_MN) {                                          // two boxes of 64 rows of A, each [64 k][64 m]
             tma_load_2d(sa, &tmA, m0, kb * BK, leader_full, keep);
             tma_load_2d(sa + MN_BOX_BYTES, &tmA, m0 + MN_BOX, kb * BK, leader_full, keep);
@@ -765,7 +860,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + acc * BN_MAX;
         const uint32_t idesc = make_idesc(WIDE ? BN_MAX : tile_coord(p, tile, m_tiles).w, A_MN ? 1 : 0, B_MN ? 1 : 0);
-        for (int kb = 0; kb < k_blocks; ++kb) {
+        for (int kb = kb0; kb < kb1; ++kb) {
           ok = __all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, ac, 0x300u | stage));
           if (!ok) break;
           tc_fence_after();
@@ -778,19 +873,19 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             for (int k = 0; k < BK / UMMA_K; ++k) {
               // advancing 16 bf16 = 32 bytes inside the swizzled row: +2 in the 16-byte address field
               // (MN-major: 16 rows of 128 bytes further on)
-              tc_mma_bf16(tmem_d, da + ka * k, db + kbs * k, idesc, (kb | k) != 0 ? 1u : 0u);
+              tc_mma_bf16(tmem_d, da + ka * k, db + kbs * k, idesc, (SPLIT ? kb != kb0 || k != 0 : (kb | k) != 0) ? 1u : 0u);
               if (WIDE)
                 tc_mma_bf16(tmem_d + BN_MAX, da + 2u * k, make_smem_desc(sb + C::BH_BYTES) + 2u * k, idesc,
-                            (kb | k) != 0 ? 1u : 0u);
+                            (SPLIT ? kb != kb0 || k != 0 : (kb | k) != 0) ? 1u : 0u);
             }
-            tc_commit_pair(empty_bar(stage));          // frees this stage in both CTAs
+            tc_commit_pair(empty_bar(stage), leader);          // frees this stage in both CTAs
           }
           __syncwarp();
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (ok && faar_elect_one()) {
-          tc_commit_pair(tfull_bar(acc));              // accumulator ready in both CTAs
-          if (WIDE) tc_commit_pair(tfull_bar(1));
+          tc_commit_pair(tfull_bar(acc), leader);              // accumulator ready in both CTAs
+          if (WIDE) tc_commit_pair(tfull_bar(1), leader);
         }
         __syncwarp();
       }
@@ -819,7 +914,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       TileCoord tc;
       if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * WIDE_BN + acc * BN_MAX; tc.w = BN_MAX; }
       else tc = tile_coord(p, tile, m_tiles);
-      const int m0 = tc.m0 + (int)rank * BM, n0 = tc.n0, TW = tc.w;
+      // the columns of the tile that this pair finishes: with a split contraction its share
+      const int TW = tc.w / splits, m0 = tc.m0 + (int)rank * BM, n0 = tc.n0 + split * TW;
       const int cols_per_warp = ((TW / C::COL_GROUPS + 15) / 16) * 16;
       const int col_begin = cg * cols_per_warp;
       const int col_end = min(col_begin + cols_per_warp, TW);
@@ -855,7 +951,13 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t trow = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN_MAX);
+      const uint32_t ttile = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN_MAX);
+      const uint32_t trow = ttile + (uint32_t)(split * TW);
+      if (SPLIT) {
+        ok = exchange_parts(ttile, TW, splits, split, rank, base, bar_free, bar_recv, quarter, ew >> 2, C::COL_GROUPS, ew, lane, ac);
+        if (!ok) break;
+        tc_fence_after();
+      }
       if constexpr (MODE == FAAR_GEMM_BWD) {
         // PW-column panels, staged by the four warps of this lane quarter together (see epi_bwd_rows)
         const int sub = ew >> 2;
@@ -875,6 +977,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             uint32_t r[16];
             tmem_ld16(trow + (uint32_t)c, r);
             tmem_ld_wait();
+            if (SPLIT) add_parts(r, base, splits, TW, c, quarter * 32 + lane);
 #pragma unroll
             for (int u = 0; u < 4; ++u)
               sts128(panel + (uint32_t)lane * (4u * PW) + (uint32_t)(((4 * sub + u) ^ (lane & 7)) << 4), r[4 * u],
@@ -885,7 +988,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           if (pc + PW >= TW || n0 + pc + PW >= p.N) {    // this warp's last read of the accumulator
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), 0));
+            if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), leader));
             released = true;
           }
           okp = mbar_wait(pfull, pn & 1u, ac, 0x600u | quarter);
@@ -899,7 +1002,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (!released) {
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), 0));
+          if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), leader));
         }
         continue;
       } else {
@@ -911,6 +1014,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               uint32_t r[16];
               tmem_ld16(trow + (uint32_t)c, r);
               tmem_ld_wait();
+              if (SPLIT) add_parts(r, base, splits, TW, c, quarter * 32 + lane);
               warp_acc += epi_fwd_vec(p, o, n0 + c, r, yraw[2 * q], yraw[2 * q + 1]);
             }
           }
@@ -927,6 +1031,10 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               uint32_t r2[16];
               if (second) tmem_ld16(trow + (uint32_t)(c + 16), r2);
               tmem_ld_wait();
+              if (SPLIT) {
+                add_parts(r, base, splits, TW, c, quarter * 32 + lane);
+                if (second) add_parts(r2, base, splits, TW, c + 16, quarter * 32 + lane);
+              }
               epi_ref(p, o, n0 + c, r);
               if (second) epi_ref(p, o, n0 + c + 16, r2);
             } else {
@@ -935,6 +1043,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               for (int j = 0; j < 16; ++j) yr[j] = ynext[j];
               if (c + 16 < col_end && n0 + c + 16 < p.N) load_yref(p, o, n0 + c + 16, ynext);
               tmem_ld_wait();
+              if (SPLIT) add_parts(r, base, splits, TW, c, quarter * 32 + lane);
               warp_acc += epi_fwd(p, o, n0 + c, r, yr);
             }
           }
@@ -942,7 +1051,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), 0));
+      if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), leader));
     }
     if (MODE != FAAR_GEMM_REF) {
       warp_acc = faar_warp_sum(warp_acc);
@@ -1090,6 +1199,28 @@ int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs
   return best;
 }
 
+// Over how many CTA pairs a tile's contraction is split, and how wide the tiles are then.  With few tiles the time is that
+// of one pair's main loop, 0.18 us per k block whatever the tile's width (a block's latency through the ring), while other
+// pairs idle; parts of the contraction run at once, for an exchange of about 2 us.  That is paid back from 24 k blocks on
+// (1536; with halves of 128-wide tiles from 28), and the more parts, and the narrower the tiles, the better while the
+// device holds a cluster for every tile: 64-wide tiles have the smaller exchange and epilogue, 256-wide ones never won.
+// Measured, whole tiles -> split (parts x width), us: forward kernel and soft weights of 128 x 8192 at 512 tokens 35.2 ->
+// 18.4 (4 x 64), 700 x 4096 at 300 tokens 24.8 -> 17.5 (4 x 64), 256 x 2048 at 2000 tokens 16.5 -> 14.9 (2 x 64); product
+// [83, 1024] over 3600 16.2 -> 10.9 (4 x 128); dW kernel of 170 x 496 at 3881 tokens 20.1 -> 13.0 (4 x 64), of 128 x 256 at
+// 1536 tokens 11.9 -> 10.7 (4 x 64), at 1024 tokens (16 k blocks) 10.2 -> 11.1 (2 x 128), which stays whole.
+// The choice depends on the problem and the device alone, not on forced tile shapes or operand layouts, because it is part
+// of the order in which an output element is summed.
+int pick_splits(int M, int N, int k_blocks, const int (&clusters)[FAAR_CLUSTER_SIZES], int* bn_out) {
+  const long long m_tiles = (M + 2 * BM - 1) / (2 * BM);
+  for (int i = 2; i >= 1; --i)
+    for (int bn = 64; bn <= 128; bn *= 2) {
+      if (m_tiles * ((N + bn - 1) / bn) > clusters[i] || k_blocks < (i == 1 && bn == 128 ? 28 : MIN_SPLIT_BLOCKS)) continue;
+      *bn_out = bn;
+      return 1 << i;
+    }
+  return 1;
+}
+
 // How many tiles of the raster stay whole.  Tiles go to CTA pairs round-robin, all whole tiles first.  A half tile costs
 // 0.75 of a whole one (its A rows are loaded all the same), and the epilogue of a pair's last tile is not overlapped by
 // anything (0.4 of that tile's cost).  Returns the number that minimises the busiest pair's time (ties: fewer halves).
@@ -1141,14 +1272,15 @@ bool pick_wide(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn
          m_tiles * ((N + WIDE_BN - 1) / WIDE_BN) <= pairs;
 }
 
-template <int MODE, int OPT, bool WIDE, int MN>
+template <int MODE, int OPT, int SHAPE, int MN>
 int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_out, int bn, int max_pairs,
                    const cudaLaunchConfig_t& base_cfg) {
+  constexpr bool WIDE = SHAPE == WIDE_TILES;
   using C = Cfg<MODE, WIDE>;
   static_assert(C::MIN_STAGES >= 3, "ring too short");
   static_assert(C::SMEM_BYTES <= SMEM_LIMIT, "shared memory budget");
   static_assert(C::EPI_WARPS <= MAX_EPI_WARPS, "partials budget");
-  auto kern = faar_gemm_kernel<MODE, OPT, WIDE, MN>;
+  auto kern = faar_gemm_kernel<MODE, OPT, SHAPE, MN>;
   int e = faar_allow_smem(ctx, (const void*)kern, C::SMEM_BYTES);
   if (e) return e;
   cudaLaunchConfig_t cfg = base_cfg;
@@ -1157,9 +1289,9 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   kp.stage_bytes = WIDE ? C::STAGE_BYTES : C::A_BYTES + (a->b_mn ? mn_boxes(bn / 2) * MN_BOX_BYTES : (int)faar_align_up((size_t)(bn / 2) * BK * 2, 1024));   // whole swizzle atoms
   kp.stages = C::RING_BYTES / kp.stage_bytes < MAX_STAGES ? C::RING_BYTES / kp.stage_bytes : MAX_STAGES;
   const int m_tiles = (a->M + 2 * BM - 1) / (2 * BM), n_cols = (a->N + bn - 1) / bn;
-  kp.narrow = !WIDE && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
+  kp.narrow = SHAPE == PLAIN_TILES && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
   kp.n_main = n_cols - kp.narrow;
-  kp.n_full = WIDE ? 0 : pick_full(ctx, MODE, m_tiles, kp.n_main, kp.narrow, bn, max_pairs);
+  kp.n_full = WIDE ? 0 : (SHAPE == SPLIT_TILES ? m_tiles * kp.n_main : pick_full(ctx, MODE, m_tiles, kp.n_main, kp.narrow, bn, max_pairs));
   CUtensorMap tmA, tmB, tmBh;
   e = a->a_mn ? make_map_mn(ctx, &tmA, a->A, a->Kc, a->M, a->lda) : make_map(ctx, &tmA, a->A, a->M, a->Kc, a->lda, BM);
   if (e) return e;
@@ -1175,7 +1307,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   if (e) return e;
   const long long tiles = WIDE ? (long long)m_tiles * ((a->N + WIDE_BN - 1) / WIDE_BN)
                                : 2ll * m_tiles * kp.n_main - kp.n_full + (kp.narrow ? m_tiles : 0);
-  const int pairs = (int)(tiles < max_pairs ? tiles : max_pairs);
+  const int pairs = SHAPE == SPLIT_TILES ? (int)tiles * kp.splits : (int)(tiles < max_pairs ? tiles : max_pairs);
   cfg.gridDim = dim3(2 * pairs, 1, 1);
   if (n_partials_out) *n_partials_out = 2 * pairs * C::EPI_WARPS;
   ctx->last_gemm_bn = WIDE ? WIDE_BN : bn;
@@ -1186,6 +1318,12 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   cudaError_t ce = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmBh, kp);
   if (ce != cudaSuccess) return (int)ce;
   return (int)cudaGetLastError();
+}
+
+template <int MODE, int OPT, int MN>
+int launch_tiles(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_out, int bn, int max_pairs, const cudaLaunchConfig_t& cfg) {
+  return kp.splits > 1 ? launch_variant<MODE, OPT, SPLIT_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg)
+                       : launch_variant<MODE, OPT, PLAIN_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
 }
 
 template <int MODE, int OPT = 0>
@@ -1204,25 +1342,40 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
   cfg.stream = ctx->stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  auto kern = faar_gemm_kernel<MODE, OPT, false, 0>;               // every variant takes one CTA per SM
+  auto kern = faar_gemm_kernel<MODE, OPT, PLAIN_TILES, 0>;               // every variant takes one CTA per SM
   const int e = faar_allow_smem(ctx, (const void*)kern, C::SMEM_BYTES);
   if (e) return e;
-  const int max_pairs = faar_max_pairs(ctx, MODE == FAAR_GEMM_BWD ? 2 + OPT : MODE, (const void*)kern, &cfg);
-  const int bn = pick_bn(ctx, MODE, a->M, a->N, (a->Kc + BK - 1) / BK, max_pairs, a->b_mn != 0,
-                          a->yref_t && a->yref_dtype == FAAR_BF16 && !a->Yout);
+  const int slot = MODE == FAAR_GEMM_BWD ? 2 + OPT : MODE;
+  const int max_pairs = faar_max_clusters(ctx, slot, 0, (const void*)kern, &cfg);
+  const int k_blocks = (a->Kc + BK - 1) / BK;
+  kp.splits = 1;
+  int split_bn = BN_MAX;
+  if (k_blocks >= MIN_SPLIT_BLOCKS) {
+    int clusters[FAAR_CLUSTER_SIZES] = {max_pairs};
+    for (int i = 1; i < FAAR_CLUSTER_SIZES; ++i) {
+      attr[0].val.clusterDim.x = 2u << i;
+      clusters[i] = faar_max_clusters(ctx, slot, i, (const void*)kern, &cfg);
+    }
+    kp.splits = pick_splits(a->M, a->N, k_blocks, clusters, &split_bn);
+    attr[0].val.clusterDim.x = 2u * (unsigned)kp.splits;
+  }
+  int bn = pick_bn(ctx, MODE, a->M, a->N, k_blocks, max_pairs, a->b_mn != 0,
+                   a->yref_t && a->yref_dtype == FAAR_BF16 && !a->Yout);
+  // a forced width is kept if every pair's share of it is a multiple of 16 columns and the tiles find clusters
+  if (kp.splits > 1 && (ctx->tune_bn == 0 || bn % (32 * kp.splits) != 0)) bn = split_bn;
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
   // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient), the dW
   // product with B or with both untransposed
   if constexpr (MODE == FAAR_GEMM_REF) {
-    if (mn == 2) return launch_variant<MODE, OPT, false, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
-  }
-  if constexpr (MODE == FAAR_GEMM_BWD) {
-    if (mn == 2) return launch_variant<MODE, OPT, false, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
-    if (mn == 3) return launch_variant<MODE, OPT, false, 3>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+    if (mn == 2) return launch_tiles<MODE, OPT, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+  } else if constexpr (MODE == FAAR_GEMM_BWD) {
+    if (mn == 2) return launch_tiles<MODE, OPT, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+    if (mn == 3) return launch_tiles<MODE, OPT, 3>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   }
   if (mn != 0) return (int)cudaErrorInvalidValue;
-  if (pick_wide(ctx, MODE, a->M, a->N, (a->Kc + BK - 1) / BK, bn, max_pairs)) return launch_variant<MODE, OPT, true, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
-  return launch_variant<MODE, OPT, false, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+  if (kp.splits == 1 && pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs))
+    return launch_variant<MODE, OPT, WIDE_TILES, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+  return launch_tiles<MODE, OPT, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
 }
 
 }  // namespace

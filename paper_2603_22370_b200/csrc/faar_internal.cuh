@@ -55,9 +55,10 @@ struct faar_prof_scope {
 // Raises a kernel's dynamic shared-memory limit, once per context (the call costs about as much host time as a launch's
 // argument checks and every launch of a small layer would pay it).  The context's device is current.
 int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes);
-// How many CTA pairs of `kernel` (launched as *cfg, a cluster of two, its grid ignored) the context's device holds at once:
-// a fact of device and kernel (a GPC with an odd SM count strands one SM), asked once per device and process.
-int faar_max_pairs(faar_ctx* c, int slot, const void* kernel, cudaLaunchConfig_t* cfg);
+// How many clusters of `kernel` (launched as *cfg, which says their size 2 << size; its grid ignored) the context's device
+// holds at once: a fact of device and kernel (a GPC with an odd SM count strands one SM), asked once per device and process.
+constexpr int FAAR_CLUSTER_SIZES = 3;     // 2, 4, 8 CTAs
+int faar_max_clusters(faar_ctx* c, int slot, int size, const void* kernel, cudaLaunchConfig_t* cfg);
 
 // Launch with stream serialisation relaxed (programmatic dependent launch): the kernel's CTAs may be scheduled while the
 // kernel before it drains; the kernel itself waits (faar_pdl_sync) before it touches global memory.

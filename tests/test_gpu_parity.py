@@ -779,6 +779,41 @@ def test_wide_tiles_give_the_same_step(ctx, O, K, T):
     assert np.all(np.abs(out[0][6] - out[1][6]) <= 1e-5 * np.abs(out[0][6]))
 
 
+@pytest.mark.parametrize("O,K,T,split", [
+    (40, 1552, 72, "fwd"),           # four parts of 6 or 7 k blocks, one 64-wide tile column and a bit
+    (300, 1808, 700, "fwd"),         # several row blocks; last block of the contraction ragged
+    (520, 1808, 1300, "fwd"),        # two parts only
+    (130, 208, 1552, "bwd"),         # the dW product: shares of 16 columns of each tile
+    (300, 1040, 1800, "bwd"),
+    (1552, 80, 72, "dx"),            # the input gradient contracts over O
+])
+def test_contractions_split_over_several_cta_pairs(ctx, O, K, T, split):
+    """Few tiles and a long contraction: the pairs of a cluster take a part of it each and exchange partial sums.  Only the
+    order of the FP32 additions differs from a whole contraction, which the bounds of the tests called here allow for."""
+    tiles = {"fwd": (O, T), "bwd": (O, K), "dx": (T, K)}[split]
+
+    def was_split():
+        bn, pairs = faar.last_gemm_config(ctx)[:2]
+        return pairs > min(-(-m // 256) * -(-n // bn) for m, n in (tiles, tiles[::-1]))
+
+    if split == "fwd":
+        for yref_dtype in (faar.BF16, faar.F32):
+            test_layer_ref(ctx, O, K, T, yref_dtype)
+            assert was_split()
+        test_layer_fwd(ctx, O, K, T)
+        assert was_split()
+        test_transposed_target_layout_gives_the_same_results(ctx, O, K, T, faar.BF16)
+    elif split == "bwd":
+        for opt in (1, 0):
+            test_layer_bwd(ctx, O, K, T, opt)
+            assert was_split()
+            test_backward_on_row_major_operands_gives_the_same_bits(ctx, O, K, T, opt)
+            assert was_split()
+    else:
+        test_layer_dx(ctx, O, K, T)
+        assert was_split()
+
+
 @pytest.mark.parametrize("opt", [0, 1])
 @pytest.mark.parametrize("O,K,T", [(300, 1040, 600), (520, 784, 1300), (64, 128, 72), (1024, 512, 2048)])
 def test_backward_on_row_major_operands_gives_the_same_bits(ctx, O, K, T, opt):
