@@ -2,10 +2,9 @@
 // bracket, V_init), the FP32 soft-weight view, the BF16 soft-weight operand,
 // Round Loss reduction, hardening + packing, and a BF16 transpose.
 //
-// Work decomposition used by all per-weight kernels: one thread owns 8
-// consecutive weights of a row (half a scale block), so V moves as two float4,
-// the code as one 32-bit word and BF16 data as one 16-byte vector; the two
-// threads of a block exchange their maxima with one shuffle.
+// Work decomposition: the quantising kernels give a thread one scale block of 16 values, the other per-weight kernels 8
+// consecutive weights of a row, so that V moves as two float4, the code as one 32-bit word and BF16 data as one 16-byte
+// vector.
 #include "faar_internal.cuh"
 
 #include <atomic>
@@ -14,61 +13,77 @@ namespace {
 
 constexpr int EW_THREADS = 256;
 
-// Element offset in W of 8-element group g.  Dense rows (ldw == K) need no division; otherwise the
-// row comes from a 32-bit division (the host checks that the group count fits).
-__device__ __forceinline__ int64_t w_offset(int64_t g, uint32_t groups_per_row, int64_t ldw, bool dense) {
-  if (dense) return g * 8;
-  const uint32_t row = (uint32_t)g / groups_per_row;
-  return (int64_t)row * ldw + (int64_t)((uint32_t)g - row * groups_per_row) * 8;
+// ---- 32-byte global accesses: one instruction per scale block of BF16 values ------------------------------
+__device__ __forceinline__ bool aligned32(const void* p, int64_t row_bytes) {
+  return ((reinterpret_cast<uintptr_t>(p) | (uintptr_t)row_bytes) & 31) == 0;
+}
+__device__ __forceinline__ void ldg32(const void* p, bool wide, uint32_t* r) {
+  if (wide) {
+    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "l"(p));
+  } else {
+    const uint4 a = reinterpret_cast<const uint4*>(p)[0], b = reinterpret_cast<const uint4*>(p)[1];
+    r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w;
+    r[4] = b.x; r[5] = b.y; r[6] = b.z; r[7] = b.w;
+  }
+}
+__device__ __forceinline__ void stg32(void* p, bool wide, const uint32_t* r) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]),
+                 "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+  } else {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(r[0], r[1], r[2], r[3]);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(r[4], r[5], r[6], r[7]);
+  }
+}
+// The 16 values of a block as loaded: 32 bytes of BF16 (in r[0..7]) or 64 bytes of FP32.
+struct block_raw {
+  uint32_t r[16];
+};
+template <bool BF16IN>
+__device__ __forceinline__ block_raw load_block(const void* W, int64_t idx, bool wide) {
+  block_raw raw;
+  if (BF16IN) {
+    ldg32(reinterpret_cast<const __nv_bfloat16*>(W) + idx, wide, raw.r);
+  } else {
+    ldg32(reinterpret_cast<const float*>(W) + idx, wide, raw.r);
+    ldg32(reinterpret_cast<const float*>(W) + idx + 8, wide, raw.r + 8);
+  }
+  return raw;
 }
 
 // ---- pass 1: max |W| over the tensor -----------------------------------------
-// One thread takes 8-value groups g, g + stride, ...; eight 16-byte loads (FP32: sixteen) are in flight per
-// thread and iteration, the ragged end re-reads the last group instead of branching.  BF16 values are
-// compared as packed pairs.
+// One thread takes 32-byte units (16 BF16 or 8 FP32 values) u, u + stride, ...; four of them are in flight per thread and
+// iteration, the ragged end re-reads the last unit instead of branching.  BF16 values are compared as packed pairs.
+// Every CTA takes one contiguous piece of 32 KB and leaves: [16384, 8192] 55 -> 52 us (268 MB), [4096, 8192] 16.5 -> 15.7
+// against resident CTAs that stride over the tensor with 16-byte loads.
 template <bool BF16IN>
 __global__ void __launch_bounds__(EW_THREADS)
 amax_kernel(const void* __restrict__ W, int O, int K, int64_t ldw, unsigned long long* amax_word, uint32_t epoch) {
   faar_pdl_sync();
-  const uint32_t groups_per_row = K / 8;
-  const int64_t total = (int64_t)O * groups_per_row;
-  const bool dense = ldw == K;
+  constexpr int ES = BF16IN ? 2 : 4, DEPTH = 4;
+  const uint32_t units_per_row = K * ES / 32;
+  const int64_t total = (int64_t)O * units_per_row;
+  const uint8_t* base = reinterpret_cast<const uint8_t*>(W);
+  const bool dense = ldw == K, wide = aligned32(W, ldw * ES);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  constexpr int DEPTH = 8;
   float amax = 0.f;
   __nv_bfloat162 mx2 = __float2bfloat162_rn(0.f);
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += DEPTH * stride) {
-    if (BF16IN) {
-      uint4 raw[DEPTH];
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x * DEPTH + threadIdx.x; u < total; u += DEPTH * stride) {
+    block_raw raw[DEPTH];
 #pragma unroll
-      for (int j = 0; j < DEPTH; ++j) {
-        const int64_t gj = min(g + j * stride, total - 1);
-        raw[j] = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(W) +
-                                                 w_offset(gj, groups_per_row, ldw, dense));
-      }
-#pragma unroll
-      for (int j = 0; j < DEPTH; ++j) {
-        const uint32_t r[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) mx2 = __hmax2(mx2, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&r[i])));
-      }
-    } else {
-      float4 raw[DEPTH][2];
-#pragma unroll
-      for (int j = 0; j < DEPTH; ++j) {
-        const int64_t gj = min(g + j * stride, total - 1);
-        const float4* p = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(W) +
-                                                          w_offset(gj, groups_per_row, ldw, dense));
-        raw[j][0] = p[0];
-        raw[j][1] = p[1];
-      }
-#pragma unroll
-      for (int j = 0; j < DEPTH; ++j)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-          amax = fmaxf(fmaxf(amax, fabsf(raw[j][h].x)),
-                       fmaxf(fmaxf(fabsf(raw[j][h].y), fabsf(raw[j][h].z)), fabsf(raw[j][h].w)));
+    for (int j = 0; j < DEPTH; ++j) {
+      const int64_t uj = min(u + j * EW_THREADS, total - 1);
+      const uint32_t row = dense ? 0u : (uint32_t)uj / units_per_row;
+      ldg32(base + (dense ? uj * 32 : (int64_t)row * ldw * ES + (int64_t)((uint32_t)uj - row * units_per_row) * 32), wide, raw[j].r);
     }
+#pragma unroll
+    for (int j = 0; j < DEPTH; ++j)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (BF16IN) mx2 = __hmax2(mx2, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&raw[j].r[i])));
+        else amax = fmaxf(amax, fabsf(__uint_as_float(raw[j].r[i])));
+      }
   }
   if (BF16IN) amax = fmaxf(__low2float(mx2), __high2float(mx2));
 #pragma unroll
@@ -88,8 +103,7 @@ amax_kernel(const void* __restrict__ W, int O, int K, int64_t ldw, unsigned long
 // ---- one thread, one 16-element scale block -----------------------------------------------------
 // The set-up and activation kernels give each thread a whole scale block: the block maximum needs no
 // exchange, the E4M3 scale is formed once per 16 values, and all 16 quotients w / s share one
-// reciprocal.  Outputs wider than the input (V: 64 bytes per thread) pass through shared memory so that
-// every global store instruction of a warp covers one contiguous run.
+// reciprocal.
 //
 // These kernels are bound by the SM's integer/logic pipe (compares, selects, min/max, shifts and
 // bit operations issue at half the rate of FP32 multiply-add), so the per-value work is phrased in
@@ -97,29 +111,6 @@ amax_kernel(const void* __restrict__ W, int O, int K, int64_t ldw, unsigned long
 // saturating multiply-adds, floor() from an addition that rounds down, the nibbles of eight values
 // are summed as small integers in FP32.  Every such operation is exact, so the results equal those
 // of the compare-and-select formulation bit for bit.
-
-// The 16 values of a block as loaded: 32 bytes of BF16 (in r[0..7]) or 64 bytes of FP32.
-struct block_raw {
-  uint32_t r[16];
-};
-template <bool BF16IN>
-__device__ __forceinline__ block_raw load_block(const void* W, int64_t idx) {
-  block_raw raw;
-  if (BF16IN) {
-    const uint4* p = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(W) + idx);
-    const uint4 r0 = p[0], r1 = p[1];
-    raw.r[0] = r0.x; raw.r[1] = r0.y; raw.r[2] = r0.z; raw.r[3] = r0.w;
-    raw.r[4] = r1.x; raw.r[5] = r1.y; raw.r[6] = r1.z; raw.r[7] = r1.w;
-  } else {
-    const uint4* p = reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(W) + idx);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint4 r = p[j];
-      raw.r[4 * j] = r.x; raw.r[4 * j + 1] = r.y; raw.r[4 * j + 2] = r.z; raw.r[4 * j + 3] = r.w;
-    }
-  }
-  return raw;
-}
 
 // Values as binary32, the block maximum of |w|, and whether some magnitude is below 2^-80 (zero included):
 // such a block takes the division instruction instead of the shared reciprocal (see block_quotients).
@@ -228,28 +219,6 @@ __device__ __forceinline__ uint32_t pack_nibbles(const float (&n)[8]) {
   return __byte_perm(__float_as_uint(__fadd_rn(lo, 0x1p23f)), __float_as_uint(__fadd_rn(hi, 0x1p23f)), 0x5410);
 }
 
-// A warp's threads each hold CH 16-byte chunks that are consecutive in the output (thread t: chunks
-// t*CH .. t*CH+CH-1 of the warp's run).  Pass them through the warp's slice of shared memory so that
-// store instruction i writes chunks 32 i .. 32 i + 31.  The chunk position inside a thread's group is
-// XOR-ed with a few bits of the thread index: without it the 8 threads of a quarter-warp, CH chunks
-// apart, would fall on the same banks.
-template <int CH>
-__device__ __forceinline__ void warp_store_chunks(uint4* stage_warp, const uint4 (&mine)[CH], uint4* out_warp,
-                                                  int valid_threads) {
-  const int lane = threadIdx.x & 31;
-  constexpr int G = 8 / CH;
-#pragma unroll
-  for (int j = 0; j < CH; ++j) stage_warp[lane * CH + (j ^ ((lane / G) & (CH - 1)))] = mine[j];
-  __syncwarp();
-#pragma unroll
-  for (int i = 0; i < CH; ++i) {
-    const int c = i * 32 + lane, t = c / CH, j = c % CH;
-    const uint4 x = stage_warp[t * CH + (j ^ ((t / G) & (CH - 1)))];
-    if (t < valid_threads) out_warp[c] = x;
-  }
-  __syncwarp();
-}
-
 // Element offset in a row-major tensor of 16-element block b.
 __device__ __forceinline__ int64_t block_offset(int64_t b, uint32_t blocks_per_row, int64_t ld, bool dense) {
   if (dense) return b * 16;
@@ -257,14 +226,30 @@ __device__ __forceinline__ int64_t block_offset(int64_t b, uint32_t blocks_per_r
   return (int64_t)row * ld + (int64_t)((uint32_t)b - row * blocks_per_row) * 16;
 }
 
+__device__ __forceinline__ float scale_of_maximum(float amax) { return amax == 0.f ? 1.0f : __fdiv_rn(amax, 2688.0f); }
 __device__ __forceinline__ float tensor_scale(float s_global_in, const unsigned long long* amax_word) {
   if (s_global_in > 0.f) return s_global_in;
-  const float amax_t = __uint_as_float((uint32_t)*amax_word);      // low half: the maximum's bits
-  return amax_t == 0.f ? 1.0f : __fdiv_rn(amax_t, 2688.0f);
+  return scale_of_maximum(__uint_as_float((uint32_t)*amax_word));  // low half: the maximum's bits
 }
 
 __device__ __forceinline__ bool fast_division_ok(float s, float amax, bool has_minute) {
   return s >= 0x1p-40f && s <= 0x1p40f && amax <= 0x1p40f && !has_minute;
+}
+
+// The block's E4M3 scale: amax / d rounded to nearest in binary32, then to E4M3.  The divisor is the same for the whole
+// tensor, so its correctly rounded reciprocal `r` (0 where d is out of the range that block_quotients needs) serves every
+// block, by the same two corrections.
+__device__ __forceinline__ float divisor_reciprocal(float d) { return d >= 0x1p-40f && d <= 0x1p40f ? __frcp_rn(d) : 0.f; }
+__device__ __forceinline__ uint32_t block_scale(float amax, float d, float r) {
+  float q;
+  if (r != 0.f && amax <= 0x1p40f && (amax >= 0x1p-80f || amax == 0.f)) {
+    q = __fmul_rn(amax, r);
+    q = __fmaf_rn(__fmaf_rn(-q, d, amax), r, q);
+    q = __fmaf_rn(__fmaf_rn(-q, d, amax), r, q);
+  } else {
+    q = __fdiv_rn(amax, d);
+  }
+  return faar_float_to_e4m3(q);
 }
 
 // ---- pass 2: block scales, bracket, V_init -------------------------------------
@@ -286,52 +271,42 @@ __device__ __forceinline__ void bracket_block(const float (&w)[16], float s, flo
   }
 }
 
+// A block's input and output move as 32-byte accesses, which are whole sectors per thread, so nothing passes through shared
+// memory; bound by instruction issue (about 20 per value).  [8192, 2048] 21.7 -> 20.2 us, with the maximum 31.0 -> 28.4.
 template <bool BF16IN>
 __global__ void __launch_bounds__(EW_THREADS, 3)
 softquant_init_kernel(const void* __restrict__ W, int O, int K, int64_t ldw,
                       float s_global_in, const unsigned long long* __restrict__ amax_word,
                       uint8_t* __restrict__ scales, float* __restrict__ s_global_out,
                       uint8_t* __restrict__ code, float* __restrict__ V) {
-  __shared__ uint4 stage[EW_THREADS * 4];
   faar_pdl_sync();                                        // the maximum (and W itself) may come from the kernel before
   const float s_global = tensor_scale(s_global_in, amax_word);
   if (blockIdx.x == 0 && threadIdx.x == 0) *s_global_out = s_global;
-  const float d = __fmul_rn(s_global, 6.0f);
-
+  const float d = __fmul_rn(s_global, 6.0f), rd = divisor_reciprocal(d);
   const uint32_t blocks_per_row = K / 16;
   const int64_t total = (int64_t)O * blocks_per_row;
-  const bool dense = ldw == K;
+  const bool dense = ldw == K, wide_in = aligned32(W, ldw * (BF16IN ? 2 : 4)), wide_out = aligned32(V, 0);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  uint4* stage_warp = stage + (threadIdx.x & ~31) * 4;
-  int64_t b0 = (int64_t)blockIdx.x * blockDim.x;
-  if (b0 >= total) return;
+  int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= total) return;
   // the next block's values are requested before this block's arithmetic starts
-  block_raw next = load_block<BF16IN>(W, block_offset(min(b0 + threadIdx.x, total - 1), blocks_per_row, ldw, dense));
-  for (; b0 < total; b0 += stride) {
-    const int64_t b = b0 + threadIdx.x;
-    const bool valid = b < total;
+  block_raw next = load_block<BF16IN>(W, block_offset(b, blocks_per_row, ldw, dense), wide_in);
+  for (; b < total; b += stride) {
     const block_raw raw = next;
-    if (b0 + stride < total)
-      next = load_block<BF16IN>(W, block_offset(min(b + stride, total - 1), blocks_per_row, ldw, dense));
+    if (b + stride < total) next = load_block<BF16IN>(W, block_offset(b + stride, blocks_per_row, ldw, dense), wide_in);
     float w[16];
     bool has_minute;
     const float amax = unpack_block<BF16IN>(raw, w, &has_minute);
-    const uint32_t sb = faar_float_to_e4m3(__fdiv_rn(amax, d));
+    const uint32_t sb = block_scale(amax, d, rd);
     const float s = __fmul_rn(faar_e4m3_to_float(sb), s_global);
-    uint32_t cw[2];
-    uint4 vq[4];
+    uint32_t cw[2], vq[16];
     float(&v)[16] = *reinterpret_cast<float(*)[16]>(vq);
     if (fast_division_ok(s, amax, has_minute)) bracket_block<true>(w, s, v, cw);
     else bracket_block<false>(w, s, v, cw);
-    const int64_t warp_first = b0 + (threadIdx.x & ~31);
-    if (warp_first < total) {
-      const int64_t left = total - warp_first;
-      warp_store_chunks<4>(stage_warp, vq, reinterpret_cast<uint4*>(V + warp_first * 16), left < 32 ? (int)left : 32);
-    }
-    if (valid) {
-      *reinterpret_cast<uint2*>(code + b * 8) = make_uint2(cw[0], cw[1]);
-      scales[b] = (uint8_t)sb;
-    }
+    stg32(V + b * 16, wide_out, vq);
+    stg32(V + b * 16 + 8, wide_out, vq + 8);
+    *reinterpret_cast<uint2*>(code + b * 8) = make_uint2(cw[0], cw[1]);
+    scales[b] = (uint8_t)sb;
   }
 }
 
@@ -345,7 +320,7 @@ softquant_init_kernel(const void* __restrict__ W, int O, int K, int64_t ldw,
 // bit clear, so a quotient on a midpoint moves above it, and one below a midpoint stays below.  The codes convert back
 // to F16 pairs (nodes exactly); shifting the magnitude bits right by three makes them BF16 values scaled by 2^-112 (the
 // difference of the exponent biases), which the block scale times 2^112 undoes in one exact packed product.
-// 42 -> 14 thread instructions per value: [4096, 8192] 54 -> 29 us (153 MB; the maximum pass excluded), now bound by HBM.
+// [4096, 8192] 54 -> 27.7 us, [16384, 8192] 103 us (611 MB; the maximum pass excluded): bound by HBM.
 __device__ __forceinline__ uint32_t to_e2m1x2(float lo, float hi) {             // one byte: lo in bits 3:0
   uint32_t r;
   asm("{\n\t.reg .b8 b;\n\tcvt.rn.satfinite.e2m1x2.f32 b, %1, %2;\n\tcvt.u32.u8 %0, b;\n\t}" : "=r"(r) : "f"(hi), "f"(lo));
@@ -373,64 +348,111 @@ __device__ __forceinline__ void nearest_block(const float (&q)[16], float sg, ui
   cw[1] = __byte_perm(__byte_perm(by[4], by[5], 0x0040), __byte_perm(by[6], by[7], 0x0040), 0x5410);
 }
 
-__global__ void __launch_bounds__(EW_THREADS, 3)
+// One scale block: its values in BF16 (o), its codes (cw); returns its E4M3 scale.
+__device__ __forceinline__ uint32_t fakequant_block(const block_raw& raw, float s_global, float d, float rd, uint32_t (&o)[8], uint32_t (&cw)[2]) {
+      float w[16];
+      bool has_minute;
+      const float amax = unpack_block<true>(raw, w, &has_minute);
+      const uint32_t sb = block_scale(amax, d, rd);
+      const float sg = faar_e4m3_to_float(sb);
+      const float s = __fmul_rn(sg, s_global);
+          float q[16];
+      // a quotient far below the smallest midpoint need not be exact, so minute values take the fast path here (and -0.0
+      // becomes +0.0 in its residual corrections)
+      if (fast_division_ok(s, amax, false)) {
+        block_quotients<true>(w, s, q);
+      } else {
+        block_quotients<false>(w, s, q);
+  #pragma unroll
+        for (int i = 0; i < 16; ++i) q[i] = copysignf(q[i], w[i] < 0.f ? -1.0f : 1.0f);
+      }
+      nearest_block(q, sg, o, cw);
+  return sb;
+}
+
+__global__ void __launch_bounds__(EW_THREADS, 4)
 act_fakequant_kernel(const __nv_bfloat16* __restrict__ X, int T, int K, int64_t ldx, float s_global_in,
                      const unsigned long long* __restrict__ amax_word, __nv_bfloat16* __restrict__ Xq, int64_t ldq,
                      float* __restrict__ s_global_out, uint8_t* __restrict__ packed, uint8_t* __restrict__ scales) {
-  __shared__ uint4 stage[EW_THREADS * 2];
   faar_pdl_sync();
   const float s_global = tensor_scale(s_global_in, amax_word);
   if (blockIdx.x == 0 && threadIdx.x == 0) *s_global_out = s_global;
-  const float d = __fmul_rn(s_global, 6.0f);
+  const float d = __fmul_rn(s_global, 6.0f), rd = divisor_reciprocal(d);
   const uint32_t blocks_per_row = K / 16;
   const int64_t total = (int64_t)T * blocks_per_row;
-  const bool dense_in = ldx == K, dense_out = ldq == K;
-  uint4* stage_warp = stage + (threadIdx.x & ~31) * 2;
+  const bool dense_in = ldx == K, dense_out = ldq == K, wide_in = aligned32(X, ldx * 2), wide_out = aligned32(Xq, ldq * 2);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  int64_t b0 = (int64_t)blockIdx.x * blockDim.x;
-  if (b0 >= total) return;
-  block_raw next = load_block<true>(X, block_offset(min(b0 + threadIdx.x, total - 1), blocks_per_row, ldx, dense_in));
-  for (; b0 < total; b0 += stride) {
-    const int64_t b = b0 + threadIdx.x;
-    const bool valid = b < total;
+  int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= total) return;
+  block_raw next = load_block<true>(X, block_offset(b, blocks_per_row, ldx, dense_in), wide_in);
+  for (; b < total; b += stride) {
     const block_raw raw = next;
-    if (b0 + stride < total)
-      next = load_block<true>(X, block_offset(min(b + stride, total - 1), blocks_per_row, ldx, dense_in));
-    float w[16];
-    bool has_minute;
-    const float amax = unpack_block<true>(raw, w, &has_minute);
-    const uint32_t sb = faar_float_to_e4m3(__fdiv_rn(amax, d));
-    const float sg = faar_e4m3_to_float(sb);
-    const float s = __fmul_rn(sg, s_global);
-    uint32_t cw[2];
-    uint4 oq[2];
-    uint32_t(&o)[8] = *reinterpret_cast<uint32_t(*)[8]>(oq);
-    float q[16];
-    // a quotient far below the smallest midpoint need not be exact, so minute values take the fast path here (and -0.0
-    // becomes +0.0 in its residual corrections)
-    if (fast_division_ok(s, amax, false)) {
-      block_quotients<true>(w, s, q);
-    } else {
-      block_quotients<false>(w, s, q);
+    if (b + stride < total) next = load_block<true>(X, block_offset(b + stride, blocks_per_row, ldx, dense_in), wide_in);
+    uint32_t cw[2], o[8];
+    const uint32_t sb = fakequant_block(raw, s_global, d, rd, o, cw);
+    stg32(Xq + block_offset(b, blocks_per_row, ldq, dense_out), wide_out, o);
+    if (packed) *reinterpret_cast<uint2*>(packed + b * 8) = make_uint2(cw[0], cw[1]);
+    if (scales) scales[b] = (uint8_t)sb;
+  }
+}
+
+// A few rows: maximum and quantisation in one launch of one cluster, a scale block or two per thread, which stay in
+// registers while the CTAs exchange their maxima through distributed shared memory.  Bound by latency: [8, 2048] 5.6 -> 3.8
+// us, and one launch less for the host.  Eight CTAs (the largest portable cluster) of 512 threads hold two blocks a thread,
+// 131072 values; beyond, the two passes over the whole chip are the faster form ([128, 2048] 5.8 us).
+constexpr int SMALL_CTAS = 8, SMALL_MAX_THREADS = 512;
+template <int R>
+__global__ void __launch_bounds__(SMALL_MAX_THREADS)
+act_fakequant_small_kernel(const __nv_bfloat16* __restrict__ X, int T, int K, int64_t ldx, __nv_bfloat16* __restrict__ Xq, int64_t ldq,
+                           float* __restrict__ s_global_out, uint8_t* __restrict__ packed, uint8_t* __restrict__ scales) {
+  __shared__ float warp_max[SMALL_MAX_THREADS / 32];
+  __shared__ float cta_max[SMALL_CTAS];
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");     // with the wait below: every CTA has started
+  faar_pdl_sync();
+  const uint32_t blocks_per_row = K / 16;
+  const int total = T * (int)blocks_per_row, lane = threadIdx.x & 31;
+  const bool dense_in = ldx == K, dense_out = ldq == K, wide_in = aligned32(X, ldx * 2), wide_out = aligned32(Xq, ldq * 2);
+  const int b0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  block_raw raw[R];
+  __nv_bfloat162 mx = __float2bfloat162_rn(0.f);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) q[i] = copysignf(q[i], w[i] < 0.f ? -1.0f : 1.0f);
+  for (int j = 0; j < R; ++j)
+    if (b0 + j * step < total) raw[j] = load_block<true>(X, block_offset(b0 + j * step, blocks_per_row, ldx, dense_in), wide_in);
+#pragma unroll
+  for (int j = 0; j < R; ++j)
+    if (b0 + j * step < total) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) mx = __hmax2(mx, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&raw[j].r[i])));
     }
-    nearest_block(q, sg, o, cw);
-    if (dense_out) {
-      const int64_t warp_first = b0 + (threadIdx.x & ~31);
-      if (warp_first < total) {
-        const int64_t left = total - warp_first;
-        warp_store_chunks<2>(stage_warp, oq, reinterpret_cast<uint4*>(Xq + warp_first * 16), left < 32 ? (int)left : 32);
-      }
-    } else if (valid) {
-      uint4* p = reinterpret_cast<uint4*>(Xq + block_offset(b, blocks_per_row, ldq, false));
-      p[0] = oq[0];
-      p[1] = oq[1];
-    }
-    if (valid) {
-      if (packed) *reinterpret_cast<uint2*>(packed + b * 8) = make_uint2(cw[0], cw[1]);
-      if (scales) scales[b] = (uint8_t)sb;
-    }
+  float m = fmaxf(__low2float(mx), __high2float(mx));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) warp_max[threadIdx.x >> 5] = m;
+  __syncthreads();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (threadIdx.x < gridDim.x) {                       // thread c: this CTA's maximum to CTA c
+    m = 0.f;
+    for (int i = 0; i < (int)blockDim.x / 32; ++i) m = fmaxf(m, warp_max[i]);
+    uint32_t dst = (uint32_t)__cvta_generic_to_shared(&cta_max[blockIdx.x]);
+    asm volatile("mapa.shared::cluster.u32 %0, %0, %1;" : "+r"(dst) : "r"(threadIdx.x));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(m) : "memory");
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  m = 0.f;
+  for (int c = 0; c < (int)gridDim.x; ++c) m = fmaxf(m, cta_max[c]);
+  const float s_global = scale_of_maximum(m);
+  if (b0 == 0) *s_global_out = s_global;
+  const float d = __fmul_rn(s_global, 6.0f), rd = divisor_reciprocal(d);
+#pragma unroll
+  for (int j = 0; j < R; ++j) {
+    const int b = b0 + j * step;
+    if (b >= total) break;
+    uint32_t cw[2], o[8];
+    const uint32_t sb = fakequant_block(raw[j], s_global, d, rd, o, cw);
+    stg32(Xq + block_offset(b, blocks_per_row, ldq, dense_out), wide_out, o);
+    if (packed) *reinterpret_cast<uint2*>(packed + (int64_t)b * 8) = make_uint2(cw[0], cw[1]);
+    if (scales) scales[b] = (uint8_t)sb;
   }
 }
 
@@ -816,9 +838,9 @@ static int launch_amax(faar_ctx* ctx, bool bf16, const void* W, int rows, int K,
     if (e != cudaSuccess) return (int)e;
     epoch = ++g_amax_epoch;
   }
-  const int64_t groups = (int64_t)rows * (K / 8);
+  const int64_t units = (int64_t)rows * (K / (bf16 ? 16 : 8));
   faar_prof_scope ps(ctx, FAAR_K_AMAX);
-  const int grid = grid_for(ctx, (groups + 7) / 8, 8);
+  const int grid = grid_for(ctx, (units + 3) / 4, 100000);
   const cudaError_t e = faar_launch_pdl(ctx, bf16 ? amax_kernel<true> : amax_kernel<false>, dim3(grid), dim3(EW_THREADS), 0, W, rows,
                                         K, ld, amax_word, epoch);
   return e != cudaSuccess ? (int)e : (int)cudaGetLastError();
@@ -844,12 +866,35 @@ int faar_launch_act_fakequant(faar_ctx* ctx, int T, int K, const void* X, int64_
                               int64_t ldq, float* s_global_out, uint8_t* packed, uint8_t* scales,
                               unsigned long long* amax_word) {
   const int64_t blocks = (int64_t)T * (K / 16);
+  if (!(s_global_in > 0.f) && blocks <= 2 * SMALL_CTAS * SMALL_MAX_THREADS) {
+    faar_prof_scope ps(ctx, FAAR_K_ACT_FAKEQUANT);
+    int threads = 128;
+    while (threads < SMALL_MAX_THREADS && blocks > SMALL_CTAS * threads) threads *= 2;
+    int ctas = 1;
+    while (ctas < SMALL_CTAS && blocks > ctas * threads) ctas *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = ctx->stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, blocks > ctas * threads ? act_fakequant_small_kernel<2> : act_fakequant_small_kernel<1>,
+                                             reinterpret_cast<const __nv_bfloat16*>(X), T, K, ldx, reinterpret_cast<__nv_bfloat16*>(Xq),
+                                             ldq, s_global_out, packed, scales);
+    return e != cudaSuccess ? (int)e : (int)cudaGetLastError();
+  }
   if (!(s_global_in > 0.f)) {
     int e = launch_amax(ctx, true, X, T, K, ldx, amax_word);
     if (e) return e;
   }
   faar_prof_scope ps(ctx, FAAR_K_ACT_FAKEQUANT);
-  cudaError_t e = faar_launch_pdl(ctx, act_fakequant_kernel, dim3(grid_for(ctx, blocks, 3)), dim3(EW_THREADS), 0,
+  cudaError_t e = faar_launch_pdl(ctx, act_fakequant_kernel, dim3(grid_for(ctx, blocks, 4)), dim3(EW_THREADS), 0,
                                  reinterpret_cast<const __nv_bfloat16*>(X), T, K, ldx, s_global_in,
                                  (const unsigned long long*)amax_word, reinterpret_cast<__nv_bfloat16*>(Xq), ldq,
                                  s_global_out, packed, scales);

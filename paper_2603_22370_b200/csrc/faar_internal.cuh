@@ -233,26 +233,16 @@ __device__ __forceinline__ float faar_width(int k) { return k < 4 ? 0.5f : (k < 
 
 // FP8 E4M3 byte -> float (finite codes only).
 __device__ __forceinline__ float faar_e4m3_to_float(uint32_t b) {
-  uint32_t e = (b >> 3) & 0xF, m = b & 7;
-  float sub = (float)m * 0.001953125f;  // m * 2^-9
-  float nor = __uint_as_float(((e + 120u) << 23) | (m << 20));
-  return e == 0 ? sub : nor;
+  uint32_t h;                                   // exact: E4M3 is a subset of F16
+  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h) : "h"((uint16_t)(b & 0x7Fu)));
+  return __low2float(*reinterpret_cast<const __half2*>(&h));
 }
 
-// Non-negative finite float -> nearest finite E4M3 byte, ties to even, saturating at 448.
+// Non-negative float -> nearest finite E4M3 byte, ties to even, saturating at 448 (also from infinity and NaN).
 __device__ __forceinline__ uint32_t faar_float_to_e4m3(float q) {
-  if (!(q < 448.0f)) return 0x7Eu;
-  if (q < 0.015625f) {                       // below 2^-6: fixed quantum 2^-9
-    return (uint32_t)__float2int_rn(q * 512.0f);   // 0..8; 8 is the smallest normal
-  }
-  uint32_t bits = __float_as_uint(q);
-  uint32_t lsb = (bits >> 20) & 1u;
-  bits += 0x7FFFFu + lsb;                    // round to nearest even at bit 20
-  bits &= 0xFFF00000u;
-  if (bits > 0x43E00000u) return 0x7Eu;      // above 448
-  uint32_t e = (bits >> 23) - 120u;
-  uint32_t m = (bits >> 20) & 7u;
-  return (e << 3) | m;
+  uint16_t r;
+  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(0.f), "f"(fminf(q, 448.0f)));
+  return r;
 }
 
 // Eq. 3 in FP32 with a relative error of a few 1e-7 over the whole range of h, also where h is tiny.

@@ -63,6 +63,33 @@ def test_act_fakequant_bit_exact(ctx, T, K, ldx, sg_in):
     assert torch.equal(Xq, Xq2)
 
 
+@pytest.mark.parametrize("T,K,pad,shift", [
+    (1, 16, 0, 0), (8, 2048, 0, 0), (9, 1040, 8, 0),          # one block; one cluster; rows off 32 bytes
+    (32, 2048, 0, 0), (33, 2048, 0, 0), (64, 2048, 16, 0),    # one and two blocks per thread, the largest single launch
+    (65, 2048, 0, 0), (1025, 1040, 0, 8)])                    # maximum and quantisation apart; base off 32 bytes
+def test_act_fakequant_in_one_launch_and_in_two(ctx, T, K, pad, shift):
+    """Bit for bit against the oracle on both sides of the size up to which one cluster does both passes; the largest
+    value sits in the last block."""
+    rng = np.random.default_rng(T + K)
+    X = (rng.standard_normal((T, K)) * 2.0 ** rng.integers(-6, 3, (T, K))).astype(np.float32)
+    X[-1, -1] = -300.0
+    ld = K + pad
+    buf = torch.full((T * ld + shift,), 1e4, dtype=torch.bfloat16, device=DEV)
+    Xd = buf[shift:].view(T, ld)
+    Xd[:, :K] = dev_bf16(X)
+    ws = ctx.workspace(faar.make_shape(16, 16, 8))
+    Xq = torch.zeros((T, K), dtype=torch.bfloat16, device=DEV)
+    sx = torch.zeros(1, dtype=torch.float32, device=DEV)
+    packed = torch.zeros((T, K // 2), dtype=torch.uint8, device=DEV)
+    scales = torch.zeros((T, K // 16), dtype=torch.uint8, device=DEV)
+    faar.act_fakequant(ctx, T, K, Xd, ld, 0.0, Xq, K, sx, packed, scales, ws)
+    units, sg, packed_o, scales_o = fo.act_fake_quant(host(dev_bf16(X)), 0.0)
+    assert host(sx)[0] == sg
+    assert np.array_equal(host(scales), scales_o)
+    assert np.array_equal(host(packed), packed_o)
+    assert np.array_equal(host(Xq).astype(np.float64), units)
+
+
 @pytest.mark.parametrize("sg_in", [0.0, 2.0 ** -7, 0.013])
 @pytest.mark.parametrize("spread", [4, 24, 120])
 def test_act_fakequant_over_the_bf16_range(ctx, sg_in, spread):
