@@ -122,12 +122,11 @@ void set_update(faar_gemm_args* a, const faar_hparams* hp) {
 
 int bwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const void* dYt, const void* Xt,
              float* V, const uint8_t* code, const uint8_t* scales, const float* s_global, float* adam_m,
-             float* adam_u, float* dV, uint8_t* ws, const faar_ws_layout& l, int* n_partials,
-             float* loss_out2 = nullptr, int n_mse_partials = 0, int row_major = 0) {
+             float* adam_u, float* dV, uint8_t* ws, const faar_ws_layout& l, float* loss_out2 = nullptr, int n_mse_partials = 0, int row_major = 0) {
   faar_gemm_args a = {};
   if (loss_out2) {
-    // the kernel's last CTA sums the forward's MSE partials and its own Round Loss partials
-    a.fin_counter = reinterpret_cast<uint32_t*>(ws) + 2;
+    // the kernel's last CTA forms both values from the forward's MSE partials and its CTAs' Round Loss sums
+    a.fin_word = reinterpret_cast<unsigned long long*>(ws) + 1;
     a.fin_mse_partials = reinterpret_cast<const float*>(ws + l.off_mse_partials);
     a.fin_n_mse = n_mse_partials;
     a.fin_scale_mse = hp->mse_scale;
@@ -147,7 +146,6 @@ int bwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const v
     a.B = Xt; a.ldb = s->ldxt;
   }
   a.status = reinterpret_cast<uint32_t*>(ws);
-  a.partials = reinterpret_cast<float*>(ws + l.off_round_partials);
   a.n_seg = 1;
   a.seg[0] = {V, code, scales, s_global, adam_m, adam_u, dV, (float)((double)hp->lambda_round / ((double)s->O * (double)s->K)), s->O};
   if (hp->beta_next > 0.f) {
@@ -160,7 +158,7 @@ int bwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const v
   }
   a.act_scale = hp->act_scale > 0.f ? hp->act_scale : 1.0f;
   set_update(&a, hp);
-  return faar_launch_gemm(ctx, &a, n_partials);
+  return faar_launch_gemm(ctx, &a, nullptr);
 }
 
 int check_gemm_operands(const faar_shape* s, bool need_x, bool need_xt) {
@@ -223,7 +221,6 @@ int faar_bwd_group(faar_ctx* ctx, int n_seg, faar_bwd_state* seg, int T, int K, 
   a.A = dY; a.lda = ldy; a.a_mn = 1;
   a.B = X; a.ldb = ldx; a.b_mn = 1;
   a.status = reinterpret_cast<uint32_t*>(ws);
-  a.partials = reinterpret_cast<float*>(ws + FAAR_WS_HEADER) + FAAR_MAX_PARTIALS;
   a.act_scale = hp->act_scale > 0.f ? hp->act_scale : 1.0f;
   set_update(&a, hp);
   return faar_launch_gemm(ctx, &a, nullptr);
@@ -708,7 +705,7 @@ int faar_layer_bwd(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, c
   FAAR_DEVICE_GUARD(ctx);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const faar_ws_layout l = faar_ws_plan(s);
-  return cuda_fail(ctx, bwd_impl(ctx, s, hp, dYt, Xt, V, code, scales, s_global, adam_m, adam_u, dV, ws, l, nullptr));
+  return cuda_fail(ctx, bwd_impl(ctx, s, hp, dYt, Xt, V, code, scales, s_global, adam_m, adam_u, dV, ws, l));
 }
 
 int faar_layer_bwd_rowmajor(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const void* dY, const void* X,
@@ -728,8 +725,7 @@ int faar_layer_bwd_rowmajor(faar_ctx* ctx, const faar_shape* s, const faar_hpara
   FAAR_DEVICE_GUARD(ctx);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const faar_ws_layout l = faar_ws_plan(s);
-  return cuda_fail(ctx, bwd_impl(ctx, s, hp, dY, X, V, code, scales, s_global, adam_m, adam_u, dV, ws, l, nullptr, nullptr, 0,
-                                 1));
+  return cuda_fail(ctx, bwd_impl(ctx, s, hp, dY, X, V, code, scales, s_global, adam_m, adam_u, dV, ws, l, nullptr, 0, 1));
 }
 
 int faar_layer_step(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const void* X, const void* Xt,
@@ -742,11 +738,10 @@ int faar_layer_step(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, 
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const faar_ws_layout l = faar_ws_plan(s);
   void* dYt = ws + l.off_dyt;
-  int np_mse = 0, np_round = 0;
+  int np_mse = 0;
   int e = fwd_impl(ctx, s, hp, X, Y_ref, V, code, scales, s_global, dYt, nullptr, ws, l, &np_mse);
   if (e) return cuda_fail(ctx, e);
-  e = bwd_impl(ctx, s, hp, dYt, Xt, V, code, scales, s_global, adam_m, adam_u, nullptr, ws, l, &np_round, loss_out2,
-               np_mse);
+  e = bwd_impl(ctx, s, hp, dYt, Xt, V, code, scales, s_global, adam_m, adam_u, nullptr, ws, l, loss_out2, np_mse);
   return cuda_fail(ctx, e);
 }
 
@@ -820,10 +815,10 @@ int faar_layer_step_host_nvfp4(faar_ctx* ctx, const faar_shape* s, const faar_hp
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const faar_ws_layout l = faar_ws_plan(s);
   void* dYt = ws + l.off_dyt;
-  int np_mse = 0, np_round = 0;
+  int np_mse = 0;
   le = fwd_impl(ctx, s, hp, Xq_dev, Yref_dev, V, code, scales, s_global, dYt, nullptr, ws, l, &np_mse);
   if (le) return cuda_fail(ctx, le);
-  le = bwd_impl(ctx, s, hp, dYt, Xq_dev, V, code, scales, s_global, adam_m, adam_u, nullptr, ws, l, &np_round, loss_dev2,
+  le = bwd_impl(ctx, s, hp, dYt, Xq_dev, V, code, scales, s_global, adam_m, adam_u, nullptr, ws, l, loss_dev2,
                 np_mse, 2);
   if (le) return cuda_fail(ctx, le);
   e = cudaMemcpyAsync(loss_host2, loss_dev2, 2 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream);

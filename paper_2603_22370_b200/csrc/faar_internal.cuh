@@ -78,8 +78,8 @@ static inline cudaError_t faar_launch_pdl(faar_ctx* ctx, void (*kernel)(KArgs...
 }
 
 // ---- workspace layout -------------------------------------------------------
-// [0, 256)            header: word 0 = status (0 = ok), word 2 = count of dW-GEMM
-//                     CTAs that have finished (zero between launches), bytes 16..23 = tensor maximum of
+// [0, 256)            header: word 0 = status (0 = ok), bytes 8..15 = the final sums of a
+//                     dW launch while its CTAs finish (zero between launches), bytes 16..23 = tensor maximum of
 //                     the last set-up pass (high word: the pass's serial number, low word: max |W| bits)
 // [256, 256+P)        loss partials (float): MSE region then Round region
 // [..]                W_soft bf16 [O,K]
@@ -202,17 +202,17 @@ struct faar_gemm_args {
   __nv_bfloat16* dYt; int64_t ld_dyt;          // FWD: [M(O), ld_dyt]
   float mse2c;                                 // FWD: 2 * mse_scale
   float act_scale;                             // FWD, BWD: tensor scale of quantised activations (1 = none)
-  float* partials;                             // FWD: sum r^2 partials; BWD: Round Loss partials
+  float* partials;                             // FWD: sum r^2 partials
   // BWD: M = O, N = K
   int n_seg; faar_bwd_state seg[FAAR_MAX_SEGMENTS];
   float beta, lr, b1, b2, eps, inv_bc1, inv_bc2; int opt;
   // BWD, optional: also write the next step's BF16 operand W_soft(V', beta_next) (null = not wanted)
   __nv_bfloat16* wsoft_next; float beta_next;
   // BWD, optional: final loss sums by the last CTA (fin_out2 null = not wanted)
-  uint32_t* fin_counter; const float* fin_mse_partials; int fin_n_mse; float fin_scale_mse, fin_scale_round;
+  unsigned long long* fin_word; const float* fin_mse_partials; int fin_n_mse; float fin_scale_mse, fin_scale_round;
   float* fin_out2;
 };
-// n_partials_out: number of floats written to args.partials
+// n_partials_out: number of floats a FWD launch writes to args.partials
 int faar_launch_gemm(faar_ctx*, const faar_gemm_args*, int* n_partials_out);
 int faar_gemm_max_partials(const faar_ctx*, int M, int N);
 int faar_launch_wait_selftest(faar_ctx*, uint32_t* status, unsigned long long limit_ns);
