@@ -285,6 +285,8 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     int it = 0;
     for (int t = pair; t < tiles; t += n_pairs, ++it) {
       const int acc = it & 1;
+      // whether a later tile waits for the shared columns, for this accumulator: else their release is not sent
+      const bool next = t + n_pairs < tiles, again = t + 2 * n_pairs < tiles;
       bool ok = bar_wait(tfull(acc), (uint32_t)((it >> 1) & 1), ab, 0xC00u | acc);
       if (!__all_sync(0xffffffffu, ok)) break;
       fence_after();
@@ -302,7 +304,7 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if (owner && i == C4::OVERLAP / 16 - 1) {
           fence_before();
           __syncwarp();
-          if (lane == 0) bar_arrive_cluster(map_to_leader(shared_free));
+          if (next && lane == 0) bar_arrive_cluster(map_to_leader(shared_free));
         }
         if (row < p.M && col < p.N) {
           __nv_bfloat16* out = p.C + (long long)row * p.ldc + col;
@@ -313,8 +315,13 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(r[2 * q]) * alpha, __uint_as_float(r[2 * q + 1]) * alpha);
               o[q] = *reinterpret_cast<uint32_t*>(&v);
             }
-            reinterpret_cast<uint4*>(out)[0] = make_uint4(o[0], o[1], o[2], o[3]);
-            reinterpret_cast<uint4*>(out)[1] = make_uint4(o[4], o[5], o[6], o[7]);
+            if ((reinterpret_cast<uintptr_t>(out) & 31) == 0) {
+              asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(out), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]),
+                           "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
+            } else {
+              reinterpret_cast<uint4*>(out)[0] = make_uint4(o[0], o[1], o[2], o[3]);
+              reinterpret_cast<uint4*>(out)[1] = make_uint4(o[4], o[5], o[6], o[7]);
+            }
           } else {
 #pragma unroll
             for (int q = 0; q < 16; ++q)
@@ -324,12 +331,19 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       }
       fence_before();
       __syncwarp();
-      if (lane == 0) bar_arrive_cluster(map_to_leader(tempty(acc)));
+      if (again && lane == 0) bar_arrive_cluster(map_to_leader(tempty(acc)));
     }
   }
   __syncwarp();
+  // Neither CTA leaves while the other can still use its memory or arrive on its barriers; all of that has been waited for
+  // by now, so a relaxed arrival does, which does not wait for this CTA's results to reach L2.  After a wait that gave up
+  // it may still be on its way: then the full form, and some time.
   fence_before();
-  cluster_sync_all();              // neither CTA leaves while the other can still arrive on its barriers or use its memory
+  __syncthreads();
+  if (*abort_flag) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  else asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (*abort_flag) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
   if (warp == 1) {
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS) : "memory");
