@@ -15,7 +15,7 @@
 //                                overlaps the main loop of the next)
 // A launch with few tiles and a long contraction splits it (p.splits = 2 or 4): the pairs of a cluster of 4 or 8 CTAs take
 // a part of the k blocks of the SAME tile each, then every CTA sends the accumulator columns that are another pair's
-// to finish to that pair's CTA of the same rows (distributed shared memory, into the idle operand ring) and finishes its
+// to finish to that pair's CTA of the same rows (distributed shared memory) and finishes its
 // own share of the columns, adding the parts in a fixed order (see exchange_parts).
 // The three epilogues are the operations of the layer step:
 //   REF : Y_fp = X W^T                                   (Procedure step 8)
@@ -169,8 +169,10 @@ __device__ __noinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, co
     }
   }
 }
-__device__ __forceinline__ void sts128_cluster(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared::cluster.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+// 16 bytes into another CTA's shared memory, credited there to its barrier `bar`
+__device__ __forceinline__ void st_async128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1,%2,%3,%4}, [%5];"
+               ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar) : "memory");
 }
 
 // 2-D tiled TMA load into this CTA's shared memory; the byte count is credited to `bar`, which may be
@@ -677,52 +679,55 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, const Segment& s
 }
 
 // ---- split contraction -----------------------------------------------------------------------
-// What arrives from the other pairs lies in the operand ring as [part][4 columns][row] of 16 bytes: a warp, one row per
-// lane, reads and writes consecutive 16-byte units.
-__device__ __forceinline__ uint32_t part_unit(uint32_t ring, int slot, int cols, int unit, int row) {
-  return ring + (uint32_t)(((slot * (cols >> 2) + unit) * BM + row) << 4);
+// The pairs of a cluster finish consecutive shares of the tile's columns, in whole chunks of 16: pair d those from
+// share_begin(w, splits, d) on.  What arrives from the other pairs lies behind the operand ring as
+// [part][4 columns][row] of 16 bytes: a warp, one row per lane, reads and writes consecutive 16-byte units.
+__host__ __device__ constexpr int share_begin(int w, int splits, int d) { return 16 * ((w / 16) * d / splits); }
+constexpr int parts_bytes(int splits, int w) { return (splits - 1) * 16 * ((w / 16 + splits - 1) / splits) * BM * 4; }     // the largest share
+__device__ __forceinline__ uint32_t part_unit(uint32_t parts, int slot, int cols, int unit, int row) {
+  return parts + (uint32_t)(((slot * (cols >> 2) + unit) * BM + row) << 4);
 }
-// One epilogue warp's share of the exchange: `trow` is the warp's lane quarter of the tile's accumulator, `cols` the
-// columns each pair finishes.  False: a wait gave up.  Barriers: `bar_free`, the other pairs' CTAs have nothing in flight
-// into (or out of) their rings any more; `bar_recv`, their parts have arrived here.
-__device__ __forceinline__ bool exchange_parts(uint32_t trow, int cols, int splits, int split, uint32_t prank, uint32_t ring,
-                                               uint32_t bar_free, uint32_t bar_recv, int quarter, int cg, int groups, int ew, int lane,
-                                               const AbortCtl& ac) {
-  if (ew == 0 && lane < splits && lane != split) mbar_arrive_cluster(map_to_cta(bar_free, 2u * (uint32_t)lane + prank));
-  bool ok = mbar_wait_cluster(bar_free, 0u, ac, 0x800u);
-  if (!__all_sync(0xffffffffu, ok)) return false;
-  const int chunks = cols / 16, row = quarter * 32 + lane;
+// One epilogue warp's share of the exchange: `trow` is the warp's lane quarter of the tile's accumulator, w columns wide.
+// Nobody waits before sending: the room is used once and for this alone, and the stores themselves complete the
+// receiver's barrier (a handshake, fences and arrivals around plain stores took 1.4 us more).  False: the wait for the
+// others' parts gave up.
+__device__ __forceinline__ bool exchange_parts(uint32_t trow, int w, int splits, int split, uint32_t prank, uint32_t parts,
+                                               uint32_t bar_recv, int quarter, int cg, int groups, int lane, const AbortCtl& ac) {
+  const int row = quarter * 32 + lane;
   int i = 0;
   for (int d = 0; d < splits; ++d) {
     if (d == split) continue;
-    const int slot = split < d ? split : split - 1;
-    for (int c = 0; c < chunks; ++c, ++i) {
+    const int slot = split < d ? split : split - 1, c0 = share_begin(w, splits, d), cols = share_begin(w, splits, d + 1) - c0;
+    const uint32_t dst = 2u * (uint32_t)d + prank, bar = map_to_cta(bar_recv, dst);
+    for (int c = 0; c < cols; c += 16, ++i) {
       if (i % groups != cg) continue;
       uint32_t r[16];
-      tmem_ld16(trow + (uint32_t)(d * cols + 16 * c), r);
+      tmem_ld16(trow + (uint32_t)(c0 + c), r);
       tmem_ld_wait();
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        sts128_cluster(map_to_cta(part_unit(ring, slot, cols, 4 * c + u, row), 2u * (uint32_t)d + prank), r[4 * u], r[4 * u + 1],
-                       r[4 * u + 2], r[4 * u + 3]);
+        st_async128(map_to_cta(part_unit(parts, slot, cols, (c >> 2) + u, row), dst), r[4 * u], r[4 * u + 1], r[4 * u + 2], r[4 * u + 3], bar);
     }
   }
-  asm volatile("fence.acq_rel.cluster;" ::: "memory");
-  __syncwarp();
-  if (lane < splits && lane != split) mbar_arrive_cluster(map_to_cta(bar_recv, 2u * (uint32_t)lane + prank));
-  ok = mbar_wait_cluster(bar_recv, 0u, ac, 0x810u);
-  return __all_sync(0xffffffffu, ok);
+  return __all_sync(0xffffffffu, mbar_wait_cluster(bar_recv, 0u, ac, 0x800u));
 }
-// r += what the other pairs sent for the 16 columns from `c` (of this pair's share) of this lane's row
-__device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t ring, int splits, int cols, int c, int row) {
-  for (int slot = 0; slot + 1 < splits; ++slot) {
+// r += what the other pairs sent for the 16 columns from `c` (of this pair's share, `cols` wide) of this lane's row; four
+// parts as (0 + 1) + (2 + 3), which is the same sum whichever of them is the own one.
+__device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t parts, int splits, int split, int cols, int c, int row) {
+  auto slot = [&](int j) { return j < split ? j : j - 1; };
+  const int other = (split ^ 2) & 2;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float4 v = lds128(part_unit(ring, slot, cols, (c >> 2) + u, row));
-      r[4 * u] = __float_as_uint(__uint_as_float(r[4 * u]) + v.x);
-      r[4 * u + 1] = __float_as_uint(__uint_as_float(r[4 * u + 1]) + v.y);
-      r[4 * u + 2] = __float_as_uint(__uint_as_float(r[4 * u + 2]) + v.z);
-      r[4 * u + 3] = __float_as_uint(__uint_as_float(r[4 * u + 3]) + v.w);
+  for (int u = 0; u < 4; ++u) {
+    const float4 v = lds128(part_unit(parts, slot(split ^ 1), cols, (c >> 2) + u, row));
+    const float p[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) r[4 * u + j] = __float_as_uint(__uint_as_float(r[4 * u + j]) + p[j]);
+    if (splits == 4) {
+      const float4 x = lds128(part_unit(parts, slot(other), cols, (c >> 2) + u, row));
+      const float4 y = lds128(part_unit(parts, slot(other + 1), cols, (c >> 2) + u, row));
+      const float q[4] = {x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) r[4 * u + j] = __float_as_uint(__uint_as_float(r[4 * u + j]) + q[j]);
     }
   }
 }
@@ -733,7 +738,7 @@ __device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t ring, int 
 // a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.
 // SHAPE: 0 = tiles of up to 256 columns, WIDE_TILES, SPLIT_TILES; at compile time for the same reason.
 constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2;
-constexpr int MIN_SPLIT_BLOCKS = 24;            // contractions of fewer k blocks stay whole (see pick_splits)
+constexpr int MIN_SPLIT_BLOCKS = 12;            // contractions of fewer k blocks stay whole (see pick_splits)
 template <int MODE, int OPT, int SHAPE, int MN>
 __global__ void __launch_bounds__(Cfg<MODE, SHAPE == WIDE_TILES>::THREADS, 1)
 faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -773,7 +778,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int total_tiles = WIDE ? m_tiles * ((p.N + WIDE_BN - 1) / WIDE_BN) : tile_count(p, m_tiles);
   const int k_blocks = (p.Kc + BK - 1) / BK;
   const int kb0 = SPLIT ? k_blocks * split / splits : 0, kb1 = SPLIT ? k_blocks * (split + 1) / splits : k_blocks;
-  const uint32_t bar_free = ctl_u32 + 208u, bar_recv = ctl_u32 + 216u;                  // SPLIT: see exchange_parts
+  const uint32_t bar_recv = ctl_u32 + 208u, parts = base + (uint32_t)STAGES * STAGE_BYTES;   // SPLIT: see exchange_parts
 
   if (threadIdx.x == 64) {                             // the copies' descriptors, fetched during the set-up
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
@@ -783,7 +788,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     // accumulator-empty barriers are used in the leader only: every epilogue warp of both CTAs arrives there
     for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 2 * C::EPI_WARPS); }
-    if (SPLIT) { mbar_init(bar_free, splits - 1); mbar_init(bar_recv, (splits - 1) * C::EPI_WARPS); }
+    if (SPLIT) { mbar_init(bar_recv, 1); mbar_expect_tx(bar_recv, (uint32_t)((splits - 1) * (share_begin(BN, splits, split + 1) - share_begin(BN, splits, split)) * BM * 4)); }
     for (int q = 0; q < 8; ++q) mbar_init(ctl_u32 + 256u + 8u * q, 4);   // panel staged / panel consumed, per lane quarter
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -934,7 +939,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * WIDE_BN + acc * BN_MAX; tc.w = BN_MAX; }
       else tc = tile_coord(p, tile, m_tiles);
       // the columns of the tile that this pair finishes: with a split contraction its share
-      const int TW = tc.w / splits, m0 = tc.m0 + (int)rank * BM, n0 = tc.n0 + split * TW;
+      const int share0 = SPLIT ? share_begin(tc.w, splits, split) : 0;
+      const int TW = SPLIT ? share_begin(tc.w, splits, split + 1) - share0 : tc.w, m0 = tc.m0 + (int)rank * BM, n0 = tc.n0 + share0;
       const int cols_per_warp = ((TW / C::COL_GROUPS + 15) / 16) * 16;
       const int col_begin = cg * cols_per_warp;
       const int col_end = min(col_begin + cols_per_warp, TW);
@@ -971,9 +977,9 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       if (!ok) break;
       tc_fence_after();
       const uint32_t ttile = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN_MAX);
-      const uint32_t trow = ttile + (uint32_t)(split * TW);
+      const uint32_t trow = ttile + (uint32_t)share0;
       if (SPLIT) {
-        ok = exchange_parts(ttile, TW, splits, split, rank, base, bar_free, bar_recv, quarter, ew >> 2, C::COL_GROUPS, ew, lane, ac);
+        ok = exchange_parts(ttile, tc.w, splits, split, rank, parts, bar_recv, quarter, ew >> 2, C::COL_GROUPS, lane, ac);
         if (!ok) break;
         tc_fence_after();
       }
@@ -996,7 +1002,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             uint32_t r[16];
             tmem_ld16(trow + (uint32_t)c, r);
             tmem_ld_wait();
-            if (SPLIT) add_parts(r, base, splits, TW, c, quarter * 32 + lane);
+            if (SPLIT) add_parts(r, parts, splits, split, TW, c, quarter * 32 + lane);
 #pragma unroll
             for (int u = 0; u < 4; ++u)
               sts128(panel + (uint32_t)lane * (4u * PW) + (uint32_t)(((4 * sub + u) ^ (lane & 7)) << 4), r[4 * u],
@@ -1033,7 +1039,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               uint32_t r[16];
               tmem_ld16(trow + (uint32_t)c, r);
               tmem_ld_wait();
-              if (SPLIT) add_parts(r, base, splits, TW, c, quarter * 32 + lane);
+              if (SPLIT) add_parts(r, parts, splits, split, TW, c, quarter * 32 + lane);
               warp_acc += epi_fwd_vec(p, o, n0 + c, r, yraw[2 * q], yraw[2 * q + 1]);
             }
           }
@@ -1051,8 +1057,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               if (second) tmem_ld16(trow + (uint32_t)(c + 16), r2);
               tmem_ld_wait();
               if (SPLIT) {
-                add_parts(r, base, splits, TW, c, quarter * 32 + lane);
-                if (second) add_parts(r2, base, splits, TW, c + 16, quarter * 32 + lane);
+                add_parts(r, parts, splits, split, TW, c, quarter * 32 + lane);
+                if (second) add_parts(r2, parts, splits, split, TW, c + 16, quarter * 32 + lane);
               }
               epi_ref(p, o, n0 + c, r);
               if (second) epi_ref(p, o, n0 + c + 16, r2);
@@ -1062,7 +1068,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               for (int j = 0; j < 16; ++j) yr[j] = ynext[j];
               if (c + 16 < col_end && n0 + c + 16 < p.N) load_yref(p, o, n0 + c + 16, ynext);
               tmem_ld_wait();
-              if (SPLIT) add_parts(r, base, splits, TW, c, quarter * 32 + lane);
+              if (SPLIT) add_parts(r, parts, splits, split, TW, c, quarter * 32 + lane);
               warp_acc += epi_fwd(p, o, n0 + c, r, yr);
             }
           }
@@ -1215,23 +1221,28 @@ int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs
 
 // Over how many CTA pairs a tile's contraction is split, and how wide the tiles are then.  With few tiles the time is that
 // of one pair's main loop, 0.18 us per k block whatever the tile's width (a block's latency through the ring), while other
-// pairs idle; parts of the contraction run at once, for an exchange of about 2 us.  That is paid back from 24 k blocks on
-// (1536; with halves of 128-wide tiles from 28), and the more parts, and the narrower the tiles, the better while the
-// device holds a cluster for every tile: 64-wide tiles have the smaller exchange and epilogue, 256-wide ones never won.
-// Measured, whole tiles -> split (parts x width), us: forward kernel and soft weights of 128 x 8192 at 512 tokens 35.2 ->
-// 18.4 (4 x 64), 700 x 4096 at 300 tokens 24.8 -> 17.5 (4 x 64), 256 x 2048 at 2000 tokens 16.5 -> 14.9 (2 x 64); product
-// [83, 1024] over 3600 16.2 -> 10.9 (4 x 128); dW kernel of 170 x 496 at 3881 tokens 20.1 -> 13.0 (4 x 64), of 128 x 256 at
-// 1536 tokens 11.9 -> 10.7 (4 x 64), at 1024 tokens (16 k blocks) 10.2 -> 11.1 (2 x 128), which stays whole.
-// The choice depends on the problem and the device alone, not on forced tile shapes or operand layouts, because it is part
-// of the order in which an output element is summed.
-int pick_splits(int M, int N, int k_blocks, const int (&clusters)[FAAR_CLUSTER_SIZES], int* bn_out) {
-  const long long m_tiles = (M + 2 * BM - 1) / (2 * BM);
-  for (int i = 2; i >= 1; --i)
-    for (int bn = 64; bn <= 128; bn *= 2) {
-      if (m_tiles * ((N + bn - 1) / bn) > clusters[i] || k_blocks < (i == 1 && bn == 128 ? 28 : MIN_SPLIT_BLOCKS)) continue;
-      *bn_out = bn;
-      return 1 << i;
-    }
+// pairs idle; parts of the contraction run at once, for an exchange of about 1 us.  Two or four parts, tiles of 64 or 128
+// columns (wider ones never won: more to exchange, more to finish), as long as the device holds a cluster for every tile;
+// 64-wide tiles are paid back from 12 k blocks on (two parts of them from 14), 128-wide ones, with twice the exchange,
+// from 20, and from 40 four parts of those are better than two of 64.
+// Measured, whole tiles -> split (parts x width), us: whole step of 640 x 640 at 640 tokens (10 k blocks) 16.6 -> 17.0
+// (2 x 64), of 512 x 768 at 768 tokens (12) 19.3 -> 19.9 (2 x 64), of 128 x 768 at 768 17.4 -> 16.6 (4 x 64); 256 x 1024 at 1024 tokens (16) forward 11.4 -> 10.6 and dW 10.0 -> 9.2 (2 x 64),
+// 11.2 and 10.0 (4 x 128), 10.9 and 10.3 (2 x 128); 128 x 1536 at 1536 tokens (24) 13.6 -> 11.3 and 11.8 -> 10.2 (2 x 64);
+// 300 x 2048 at 2048 tokens 16.2 -> 14.3 and 14.0 -> 12.7 (2 x 128); whole step of 128 x 8192 at 512 tokens 48.3 -> 27.2.
+// The choice depends on the problem and the device alone, not on forced tile widths or operand layouts, because it is part
+// of the order in which an output element is summed (for the plain product it is the same with M and N exchanged).
+int pick_splits(int mode, int M, int N, int k_blocks, const int (&clusters)[FAAR_CLUSTER_SIZES], int* bn_out) {
+  auto tiles = [](int m, int n, int bn) { return (long long)((m + 2 * BM - 1) / (2 * BM)) * ((n + bn - 1) / bn); };
+  struct Form { int size, bn, least; };
+  const Form four64 = {2, 64, MIN_SPLIT_BLOCKS}, two64 = {1, 64, 14}, four128 = {2, 128, 20}, two128 = {1, 128, 20};
+  const bool lots = k_blocks >= 40;
+  for (const Form& f : {four64, lots ? four128 : two64, lots ? two64 : four128, two128}) {
+    long long n = tiles(M, N, f.bn);
+    if (mode == FAAR_GEMM_REF && tiles(N, M, f.bn) > n) n = tiles(N, M, f.bn);
+    if (n > clusters[f.size] || k_blocks < f.least) continue;
+    *bn_out = f.bn;
+    return 1 << f.size;
+  }
   return 1;
 }
 
@@ -1301,7 +1312,8 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   cfg.dynamicSmemBytes = C::SMEM_BYTES;
   kp.bn = bn;
   kp.stage_bytes = WIDE ? C::STAGE_BYTES : C::A_BYTES + (a->b_mn ? mn_boxes(bn / 2) * MN_BOX_BYTES : (int)faar_align_up((size_t)(bn / 2) * BK * 2, 1024));   // whole swizzle atoms
-  kp.stages = C::RING_BYTES / kp.stage_bytes < MAX_STAGES ? C::RING_BYTES / kp.stage_bytes : MAX_STAGES;
+  const int ring = (C::RING_BYTES - (SHAPE == SPLIT_TILES ? parts_bytes(kp.splits, bn) : 0)) / kp.stage_bytes;
+  kp.stages = ring < MAX_STAGES ? ring : MAX_STAGES;
   const int m_tiles = (a->M + 2 * BM - 1) / (2 * BM), n_cols = (a->N + bn - 1) / bn;
   kp.narrow = SHAPE == PLAIN_TILES && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
   kp.n_main = n_cols - kp.narrow;
@@ -1364,19 +1376,19 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
   const int k_blocks = (a->Kc + BK - 1) / BK;
   kp.splits = 1;
   int split_bn = BN_MAX;
-  if (k_blocks >= MIN_SPLIT_BLOCKS) {
+  // (forced tail splits and wide tiles compare forms of the whole contraction)
+  if (k_blocks >= MIN_SPLIT_BLOCKS && ctx->tune_tail < 0 && ctx->tune_wide < 0) {
     int clusters[FAAR_CLUSTER_SIZES] = {max_pairs};
     for (int i = 1; i < FAAR_CLUSTER_SIZES; ++i) {
       attr[0].val.clusterDim.x = 2u << i;
       clusters[i] = faar_max_clusters(ctx, slot, i, (const void*)kern, &cfg);
     }
-    kp.splits = pick_splits(a->M, a->N, k_blocks, clusters, &split_bn);
+    kp.splits = pick_splits(MODE, a->M, a->N, k_blocks, clusters, &split_bn);
     attr[0].val.clusterDim.x = 2u * (unsigned)kp.splits;
   }
   int bn = pick_bn(ctx, MODE, a->M, a->N, k_blocks, max_pairs, a->b_mn != 0,
                    a->yref_t && a->yref_dtype == FAAR_BF16 && !a->Yout);
-  // a forced width is kept if every pair's share of it is a multiple of 16 columns and the tiles find clusters
-  if (kp.splits > 1 && (ctx->tune_bn == 0 || bn % (32 * kp.splits) != 0)) bn = split_bn;
+  if (kp.splits > 1 && ctx->tune_bn == 0) bn = split_bn;
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
   // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient), the dW
   // product with B or with both untransposed
