@@ -448,34 +448,67 @@ __device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const
 }
 
 // FWD: residual, sum of squares, dY^T.
-// Y_ref[t0..t0+15, o] for this lane's output feature o.
-__device__ __forceinline__ void load_yref(const KParams& p, int o, int t0, float (&yr)[16]) {
+// Y_ref[t0..t0+15, o] for this lane's output feature o, as it is in memory: anything done to a value here (widening BF16, a
+// select at the matrix edge) would wait for it here, one latency per chunk of 16 columns.  Forward kernel, row-major target,
+// before -> after: 4096 x 2048 at 2048 tokens BF16 90 -> 45, FP32 51 -> 46 us (transposed BF16: 40); 5312 x 304 at 1504
+// tokens 74 -> 27 and 32 -> 26.
+__device__ __forceinline__ void load_yref(const KParams& p, int o, int t0, uint32_t (&yr)[16]) {
   if (o >= p.M) return;
+  const bool bf16 = p.yref_dtype == FAAR_BF16;
   if (p.yref_t) {
-    if (p.yref_dtype == FAAR_BF16) {
+    if (bf16) {
       const uint4* y4 = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.Yref) + (long long)o * p.ldy + t0);
       const uint4 a = y4[0], b = y4[1];
-      const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        yr[2 * i] = __uint_as_float(w[i] << 16);
-        yr[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-      }
+      yr[0] = a.x; yr[1] = a.y; yr[2] = a.z; yr[3] = a.w;
+      yr[4] = b.x; yr[5] = b.y; yr[6] = b.z; yr[7] = b.w;
     } else {
-      const float4* y4 = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p.Yref) + (long long)o * p.ldy + t0);
+      const uint4* y4 = reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(p.Yref) + (long long)o * p.ldy + t0);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) { const float4 v = y4[q]; yr[4 * q] = v.x; yr[4 * q + 1] = v.y; yr[4 * q + 2] = v.z; yr[4 * q + 3] = v.w; }
+      for (int q = 0; q < 4; ++q) { const uint4 v = y4[q]; yr[4 * q] = v.x; yr[4 * q + 1] = v.y; yr[4 * q + 2] = v.z; yr[4 * q + 3] = v.w; }
     }
-    return;
-  }
-  if (p.yref_dtype == FAAR_BF16) {
-    const __nv_bfloat16* y = reinterpret_cast<const __nv_bfloat16*>(p.Yref);
+  } else if (bf16) {
+    const uint16_t* y = reinterpret_cast<const uint16_t*>(p.Yref);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) yr[j] = (t0 + j < p.N) ? __bfloat162float(y[(long long)(t0 + j) * p.ldy + o]) : 0.f;
+    for (int j = 0; j < 16; ++j)
+      if (t0 + j < p.N) asm volatile("ld.global.u16 %0, [%1];" : "=r"(yr[j]) : "l"(y + (long long)(t0 + j) * p.ldy + o));
   } else {
-    const float* y = reinterpret_cast<const float*>(p.Yref);
+    const uint32_t* y = reinterpret_cast<const uint32_t*>(p.Yref);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) yr[j] = (t0 + j < p.N) ? y[(long long)(t0 + j) * p.ldy + o] : 0.f;
+    for (int j = 0; j < 16; ++j)
+      if (t0 + j < p.N) asm volatile("ld.global.b32 %0, [%1];" : "=r"(yr[j]) : "l"(y + (long long)(t0 + j) * p.ldy + o));
+  }
+}
+// the same as numbers (columns beyond the matrix: anything)
+__device__ __forceinline__ void yref_values(const KParams& p, const uint32_t (&raw)[16], float (&yr)[16]) {
+  const int shift = p.yref_dtype == FAAR_BF16 ? 16 : 0;
+  const bool pairs = p.yref_t && shift;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const uint32_t pair = j & 1 ? raw[j >> 1] & 0xFFFF0000u : raw[j >> 1] << 16;
+    yr[j] = __uint_as_float(pairs ? pair : raw[j] << shift);
+  }
+}
+
+// Asks L2 for a warp's part of a row-major target: 32 rows of the accumulator from o_first, columns [t0, t1), one line per
+// column (two where the row's start makes its values span two).
+__device__ __forceinline__ void prefetch_yref(const KParams& p, int lane, int o_first, int t0, int t1) {
+  if (o_first >= p.M) return;
+  const long long es = p.yref_dtype == FAAR_BF16 ? 2 : 4;
+  const int last = min(o_first + 31, p.M - 1);
+  for (int t = t0 + lane; t < min(t1, p.N); t += 32) {
+    const char* row = reinterpret_cast<const char*>(p.Yref) + (long long)t * p.ldy * es;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(row + o_first * es) : "memory");
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(row + last * es) : "memory");
+  }
+}
+// 16 BF16 values of a row of dY^T: one 32-byte store where the row allows it (any token count that rounds up to 16)
+__device__ __forceinline__ void store_row16(__nv_bfloat16* out, const uint32_t (&d)[8]) {
+  if ((reinterpret_cast<uintptr_t>(out) & 31) == 0) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(out), "r"(d[0]), "r"(d[1]), "r"(d[2]), "r"(d[3]), "r"(d[4]),
+                 "r"(d[5]), "r"(d[6]), "r"(d[7]) : "memory");
+  } else {
+    reinterpret_cast<uint4*>(out)[0] = make_uint4(d[0], d[1], d[2], d[3]);
+    reinterpret_cast<uint4*>(out)[1] = make_uint4(d[4], d[5], d[6], d[7]);
   }
 }
 
@@ -493,9 +526,10 @@ __device__ __forceinline__ float epi_fwd(const KParams& p, int o, int t0, const 
   __nv_bfloat16* drow = p.dYt + (long long)o * p.ld_dyt + t0;
   if (!FAAR_DBG_OK(p, drow, 2 * (t0 + 16 <= p.N ? 16 : p.N - t0), p.dYt, p.ext_dyt, 2u)) return ss;
   if (t0 + 16 <= p.N) {
-    uint4* d4 = reinterpret_cast<uint4*>(drow);
-    d4[0] = make_uint4(pack_bf16x2(dy[0], dy[1]), pack_bf16x2(dy[2], dy[3]), pack_bf16x2(dy[4], dy[5]), pack_bf16x2(dy[6], dy[7]));
-    d4[1] = make_uint4(pack_bf16x2(dy[8], dy[9]), pack_bf16x2(dy[10], dy[11]), pack_bf16x2(dy[12], dy[13]), pack_bf16x2(dy[14], dy[15]));
+    uint32_t d[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) d[i] = pack_bf16x2(dy[2 * i], dy[2 * i + 1]);
+    store_row16(drow, d);
   } else {
 #pragma unroll
     for (int j = 0; j < 16; ++j)
@@ -528,10 +562,9 @@ __device__ __forceinline__ float epi_fwd_vec(const KParams& p, int o, int t0, co
     ss = fmaf(r1, r1, ss);
     d[i] = pack_bf16x2(p.mse2c * r0, p.mse2c * r1);
   }
-  uint4* d4 = reinterpret_cast<uint4*>(p.dYt + (long long)o * p.ld_dyt + t0);
-  if (!FAAR_DBG_OK(p, d4, 32, p.dYt, p.ext_dyt, 2u)) return ss;
-  d4[0] = make_uint4(d[0], d[1], d[2], d[3]);
-  d4[1] = make_uint4(d[4], d[5], d[6], d[7]);
+  __nv_bfloat16* drow = p.dYt + (long long)o * p.ld_dyt + t0;
+  if (!FAAR_DBG_OK(p, drow, 32, p.dYt, p.ext_dyt, 2u)) return ss;
+  store_row16(drow, d);
   return ss;
 }
 
@@ -960,9 +993,12 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
       }
       // FWD otherwise: the target values of the warp's first 16 columns (the others one chunk ahead of their use)
-      float ynext[MODE == FAAR_GEMM_FWD ? 16 : 1];
+      uint32_t ynext[MODE == FAAR_GEMM_FWD ? 16 : 1];
       if constexpr (MODE == FAAR_GEMM_FWD) {
         if (!yvec && col_begin < col_end && n0 + col_begin < p.N) load_yref(p, o, n0 + col_begin, ynext);
+        // the others of a row-major target into L2 (5312 x 304 at 1504 tokens, tiles of 256: 27.9 -> 26.1 us; 64-wide tiles
+        // have one chunk more only and lose 0.2 us by asking)
+        if (!p.yref_t && col_end - col_begin > 32) prefetch_yref(p, lane, m0 + quarter * 32, n0 + col_begin + 16, n0 + col_end);
       }
       const int k_end = min(p.N, n0 + TW);               // BWD: columns of this tile that exist
       // the linear this warp's 8 rows belong to (several only with both operands row-major)
@@ -1064,8 +1100,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               if (second) epi_ref(p, o, n0 + c + 16, r2);
             } else {
               float yr[16];
-#pragma unroll
-              for (int j = 0; j < 16; ++j) yr[j] = ynext[j];
+              yref_values(p, ynext, yr);
               if (c + 16 < col_end && n0 + c + 16 < p.N) load_yref(p, o, n0 + c + 16, ynext);
               tmem_ld_wait();
               if (SPLIT) add_parts(r, parts, splits, split, TW, c, quarter * 32 + lane);
@@ -1187,7 +1222,7 @@ int make_map_mn(faar_ctx* ctx, CUtensorMap* map, const void* ptr, int kc_rows, i
 // narrower tiles spread that over more SMs.
 // REF, FWD: the width with the smallest estimated time of the busiest pair (microseconds).  A k block costs the ring's
 // latency, or what the L2 needs for all pairs' operands (about 14 TB/s); the epilogue per 64 columns 0.4 (REF), 0.6 (FWD with
-// a transposed BF16 target) or 1.5 (FWD otherwise); a further wave of tiles 1.
+// a transposed BF16 target) or 0.9 (FWD otherwise); a further wave of tiles 1.
 // Measured (width before -> after): product [260, 1024] over 512 8.8 -> 6.2 us (128 -> 32), forward kernel of a
 // 128 x 256 layer at 1024 tokens 12.8 -> 10.7 us, input gradient [192, 128] over 384 11.1 -> 8.9 us.
 // BWD: its per-weight epilogue is bound by instruction issue and a tile of it has a fixed cost of several microseconds,
@@ -1204,7 +1239,7 @@ int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs
   }
   const int widest = N > 128 ? (N < BN_MAX ? (N + 31) / 32 * 32 : BN_MAX) : (N > 64 ? 128 : (N > 32 ? 64 : 32));
   if (m_tiles * ((N + widest - 1) / widest) >= pairs) return widest;
-  const double epi64 = mode == FAAR_GEMM_FWD ? (fwd_vec ? 0.6 : 1.5) : 0.4;
+  const double epi64 = mode == FAAR_GEMM_FWD ? (fwd_vec ? 0.6 : 0.9) : 0.4;
   int best = widest;
   double best_cost = 1e30;
   for (int bn = widest; bn >= 32; bn = bn > 128 ? 128 : bn / 2) {
