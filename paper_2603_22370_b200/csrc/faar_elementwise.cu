@@ -562,13 +562,11 @@ softquant_eval_kernel(const float* __restrict__ V, const uint8_t* __restrict__ c
   }
 }
 
-// The BF16 operand alone, for up to three linears whose output rows are stacked in `out`: one launch for the linears of a
-// decoder block that share an input.  Each segment's bases are moved back by its first group, so that groups of the
-// launch index them; a segment starts at a multiple of eight rows.
-struct SoftSegment { const float* V; const uint8_t* code; const uint8_t* scales; const float* s_global; };
-struct SoftGroup { SoftSegment seg[FAAR_MAX_SEGMENTS]; int64_t end[FAAR_MAX_SEGMENTS - 1]; };
+// The BF16 operand alone, for many linears in one launch, each with its own output.  A CTA takes 256 groups of eight
+// weights of one linear at a time; the linears' pieces are numbered through.
+struct SoftWeights { faar_soft_item item[FAAR_MAX_SOFT_ITEMS]; int first[FAAR_MAX_SOFT_ITEMS + 1]; int n; float beta; };
 __global__ void __launch_bounds__(EW_THREADS)
-soft_weights_group_kernel(const __grid_constant__ SoftGroup sg, float beta, int64_t n_groups, __nv_bfloat16* __restrict__ out) {
+soft_weights_kernel(const __grid_constant__ SoftWeights p) {
   __shared__ float2 lut[16];
   if (threadIdx.x < 16) {
     const int k = threadIdx.x & 7;
@@ -578,17 +576,18 @@ soft_weights_group_kernel(const __grid_constant__ SoftGroup sg, float beta, int6
   __syncthreads();
   faar_pdl_sync();
   float nbl, hbl;
-  faar_operand_consts(beta, &nbl, &hbl);
-  const float sg0 = *sg.seg[0].s_global, sg1 = *sg.seg[1].s_global, sg2 = *sg.seg[2].s_global;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n_groups; g += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (g >= sg.end[0]) + (g >= sg.end[1]);
-    const SoftSegment& s = sg.seg[i];
-    const int64_t e = g * 8;
+  faar_operand_consts(p.beta, &nbl, &hbl);
+  int i = 0;
+  for (int piece = blockIdx.x; piece < p.first[p.n]; piece += gridDim.x) {
+    while (piece >= p.first[i + 1]) ++i;
+    const faar_soft_item& s = p.item[i];
+    const int64_t g = (int64_t)(piece - p.first[i]) * EW_THREADS + threadIdx.x, e = g * 8;
+    if (e >= s.weights) continue;
     const float4* vp = reinterpret_cast<const float4*>(s.V + e);
     const float4 a = vp[0], b = vp[1];
     const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     const uint32_t cw = *reinterpret_cast<const uint32_t*>(s.code + e / 2);
-    const float sc = __fmul_rn(faar_e4m3_to_float(s.scales[e / 16]), i == 0 ? sg0 : (i == 1 ? sg1 : sg2));
+    const float sc = __fmul_rn(faar_e4m3_to_float(s.scales[e / 16]), *s.s_global);
     uint32_t o[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -601,7 +600,7 @@ soft_weights_group_kernel(const __grid_constant__ SoftGroup sg, float beta, int6
       const __nv_bfloat162 p2 = __floats2bfloat162_rn(w[0], w[1]);
       o[j] = *reinterpret_cast<const uint32_t*>(&p2);
     }
-    *reinterpret_cast<uint4*>(out + e) = make_uint4(o[0], o[1], o[2], o[3]);
+    *reinterpret_cast<uint4*>(s.out + e) = make_uint4(o[0], o[1], o[2], o[3]);
   }
 }
 
@@ -922,20 +921,17 @@ int faar_launch_softquant_eval(faar_ctx* ctx, const faar_shape* s, const float* 
   return (int)cudaGetLastError();
 }
 
-int faar_launch_soft_weights_group(faar_ctx* ctx, int n_seg, const faar_bwd_state* seg, int K, float beta, __nv_bfloat16* out) {
-  SoftGroup g = {};
-  int64_t row0 = 0;
-  for (int i = 0; i < FAAR_MAX_SEGMENTS; ++i) {
-    if (i) g.end[i - 1] = i < n_seg ? row0 * (K / 8) : INT64_MAX;
-    const faar_bwd_state& b = seg[i < n_seg ? i : 0];
-    const int64_t e0 = i < n_seg ? row0 * K : 0;
-    g.seg[i] = {b.V - e0, b.code - e0 / 2, b.scales - e0 / 16, b.s_global};
-    if (i < n_seg) row0 += b.rows;
+int faar_launch_soft_weights(faar_ctx* ctx, int n, const faar_soft_item* item, float beta) {
+  SoftWeights p = {};
+  p.n = n;
+  p.beta = beta;
+  for (int i = 0; i < n; ++i) {
+    p.item[i] = item[i];
+    p.first[i + 1] = p.first[i] + (int)((item[i].weights / 8 + EW_THREADS - 1) / EW_THREADS);
   }
-  const int64_t groups = row0 * (K / 8);
+  const int64_t pieces = p.first[n], resident = (int64_t)ctx->num_sms * 8;
   faar_prof_scope ps(ctx, FAAR_K_SOFT_WEIGHTS);
-  const cudaError_t e = faar_launch_pdl(ctx, soft_weights_group_kernel, dim3(grid_for(ctx, groups, 8)), dim3(EW_THREADS), 0, g, beta,
-                                        groups, out);
+  const cudaError_t e = faar_launch_pdl(ctx, soft_weights_kernel, dim3((unsigned)(pieces < resident ? pieces : resident)), dim3(EW_THREADS), 0, p);
   return e != cudaSuccess ? (int)e : (int)cudaGetLastError();
 }
 

@@ -139,7 +139,10 @@ int faar_launch_softquant_eval(faar_ctx*, const faar_shape*, const float* V, con
                                float* W_soft, float* h, __nv_bfloat16* W_soft_bf16,
                                float* W_operand_f32 = nullptr);
 // BF16 soft weights of up to three linears stacked by output rows (seg: V, code, scales, s_global, rows)
-int faar_launch_soft_weights_group(faar_ctx*, int n_seg, const faar_bwd_state* seg, int K, float beta, __nv_bfloat16* out);
+// BF16 soft weights of several linears (1 .. FAAR_MAX_SOFT_ITEMS), `weights` (a multiple of 16, below 2^40) each
+constexpr int FAAR_MAX_SOFT_ITEMS = 28;
+struct faar_soft_item { const float* V; const uint8_t* code; const uint8_t* scales; const float* s_global; __nv_bfloat16* out; int64_t weights; };
+int faar_launch_soft_weights(faar_ctx*, int n, const faar_soft_item* item, float beta);
 int faar_launch_act_fakequant(faar_ctx*, int T, int K, const void* X, int64_t ldx, float s_global_in, void* Xq,
                               int64_t ldq, float* s_global_out, uint8_t* packed, uint8_t* scales,
                               unsigned long long* amax_word);

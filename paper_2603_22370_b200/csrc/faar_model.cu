@@ -86,16 +86,46 @@ int segments(const faar_linear_group& g, faar_bwd_state (&seg)[FAAR_MAX_SEGMENTS
   }
   return g.n;
 }
-// A group's forward product: frozen weights, or soft weights formed first.
-int group_forward(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* X, bool quantised, float beta, void* Y, void* ws) {
+// A group's soft weights as items of a launch; returns how many.
+int soft_items(const faar_linear_group& g, int K, faar_soft_item* item) {
+  __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(g.Wsoft);
+  for (int i = 0; i < g.n; ++i) {
+    const faar_linear& l = g.lin[i];
+    item[i] = {l.V, l.code, l.scales, l.s_global, out, (int64_t)l.rows * K};
+    out += (int64_t)l.rows * K;
+  }
+  return g.n;
+}
+// Soft weights of the blocks from l on in one launch, as many whole blocks as SOFT_AHEAD weights allow; returns their
+// number in *n.  0: the next block is larger than that, and its groups' soft weights are formed just before their products,
+// which then find them in L2.  A small model is a chain of launches of a few microseconds: an alignment step of two 128-wide
+// blocks 321 -> 310 us.
+constexpr int64_t SOFT_AHEAD = 16 << 20;        // 32 MB of BF16, which stays in L2 until used
+int soft_blocks(faar_ctx* ctx, const faar_model* m, const Sizes& s, int l, float beta, int* n) {
+  const int64_t per_block = (int64_t)s.d * (s.qkv + s.qd + 3 * (int64_t)s.f);
+  constexpr int PER_BLOCK = 7;
+  faar_soft_item item[FAAR_MAX_SOFT_ITEMS];
+  int items = 0;
+  for (*n = 0; l + *n < m->n_layers && items + PER_BLOCK <= FAAR_MAX_SOFT_ITEMS && (*n + 1) * per_block <= SOFT_AHEAD; ++*n) {
+    const faar_block& b = m->blocks[l + *n];
+    items += soft_items(b.qkv, s.d, item + items);
+    items += soft_items(b.o, s.qd, item + items);
+    items += soft_items(b.gate_up, s.d, item + items);
+    items += soft_items(b.down, s.f, item + items);
+  }
+  return items ? faar_launch_soft_weights(ctx, items, item, beta) : 0;
+}
+// A group's forward product with frozen weights, with soft weights (formed already), or with soft weights formed first.
+enum Weights { FROZEN, SOFT, FORM_SOFT };
+int group_forward(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* X, Weights weights, float beta, void* Y, void* ws) {
   const int rows = group_rows(g);
-  if (quantised) {
-    faar_bwd_state seg[FAAR_MAX_SEGMENTS];
-    const int n = segments(g, seg);
-    const int e = faar_launch_soft_weights_group(ctx, n, seg, K, beta, reinterpret_cast<__nv_bfloat16*>(g.Wsoft));
+  if (weights == FORM_SOFT) {
+    faar_soft_item item[FAAR_MAX_SEGMENTS];
+    const int n = soft_items(g, K, item);
+    const int e = faar_launch_soft_weights(ctx, n, item, beta);
     if (e) return e;
   }
-  return product(ctx, T, rows, K, X, K, quantised ? g.Wsoft : g.W, K, false, Y, rows, ws);
+  return product(ctx, T, rows, K, X, K, weights == FROZEN ? g.W : g.Wsoft, K, false, Y, rows, ws);
 }
 // A group's backward: the gradient towards the common input, then the update of every V (at the pre-update soft weights).
 int group_backward(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp,
@@ -160,25 +190,33 @@ int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* t
   if (!e)
     e = faar_launch_rmsnorm(ctx, T, s.d, p + A.b.x_in, s.d, nullptr, 0, nullptr, 0, m->blocks[0].attn_norm, m->eps, p + A.b.hn, s.d,
                             reinterpret_cast<float*>(p + A.b.rstd1));
+  int soft_end = 0;                              // blocks below this have their soft weights
   for (int l = 0; l < m->n_layers && !e; ++l) {
     const faar_block& b = m->blocks[l];
     p = part(l);
+    if (quantised && l >= soft_end) {
+      int n = 0;
+      e = soft_blocks(ctx, m, s, l, beta, &n);
+      if (e) break;
+      soft_end = l + n;
+    }
+    const Weights w = !quantised ? FROZEN : (l < soft_end ? SOFT : FORM_SOFT);
     __nv_bfloat16* const qkv = reinterpret_cast<__nv_bfloat16*>(p + A.b.qkv);
-    e = group_forward(ctx, b.qkv, s.T, s.d, p + A.b.hn, quantised, beta, qkv, ws);
+    e = group_forward(ctx, b.qkv, s.T, s.d, p + A.b.hn, w, beta, qkv, ws);
     // q and k lie side by side: their heads turn in one launch
     if (!e) e = faar_launch_rope(ctx, T, m->n_heads + m->n_kv_heads, m->head_dim, qkv, s.qkv, pos, m->theta, 0, qkv, s.qkv);
     if (!e)
       e = faar_launch_attention_fwd(ctx, batch, seq, m->n_heads, m->n_kv_heads, m->head_dim, qkv, s.qkv, qkv + s.qd, qkv + s.qd + s.kvd,
                                     s.qkv, p + A.b.a, s.qd, reinterpret_cast<float*>(p + A.b.lse));
-    if (!e) e = group_forward(ctx, b.o, s.T, s.qd, p + A.b.a, quantised, beta, tmp, ws);
+    if (!e) e = group_forward(ctx, b.o, s.T, s.qd, p + A.b.a, w, beta, tmp, ws);
     // residual connection and the MLP's norm in one pass
     if (!e)
       e = faar_launch_rmsnorm(ctx, T, s.d, p + A.b.x_in, s.d, tmp, s.d, p + A.b.x_mid, s.d, b.mlp_norm, m->eps, p + A.b.mn, s.d,
                               reinterpret_cast<float*>(p + A.b.rstd2));
     __nv_bfloat16* const gu = reinterpret_cast<__nv_bfloat16*>(p + A.b.gu);
-    if (!e) e = group_forward(ctx, b.gate_up, s.T, s.d, p + A.b.mn, quantised, beta, gu, ws);
+    if (!e) e = group_forward(ctx, b.gate_up, s.T, s.d, p + A.b.mn, w, beta, gu, ws);
     if (!e) e = faar_launch_silu_mul(ctx, T, s.f, gu, 2 * s.f, gu + s.f, 2 * s.f, p + A.b.act, s.f);
-    if (!e) e = group_forward(ctx, b.down, s.T, s.f, p + A.b.act, quantised, beta, tmp, ws);
+    if (!e) e = group_forward(ctx, b.down, s.T, s.f, p + A.b.act, w, beta, tmp, ws);
     if (e) break;
     // residual connection and the next block's attention norm (after the last block: the final norm)
     const bool last = l + 1 == m->n_layers;

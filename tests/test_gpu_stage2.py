@@ -132,3 +132,28 @@ def test_stage2_steps_reduce_the_alignment_loss(ctx):
             lin = model.lin[l][n]
             p_o, _, _ = fo.harden_pack(host(lin.V), host(lin.code), host(lin.scales), host(lin.s_global)[0])
             assert np.array_equal(host(packed[l][n]), p_o)
+
+
+@pytest.mark.parametrize("hidden,heads,kv_heads,ffn,layers", [
+    (128, 2, 1, 256, 5),          # four blocks in one launch, then one
+    (2048, 32, 8, 2048, 1)])      # a block above the limit: group by group
+def test_soft_weights_of_a_model_are_those_of_its_linears(ctx, hidden, heads, kv_heads, ffn, layers):
+    """The forward pass forms the BF16 soft weights of many linears per launch: bit for bit what each linear's own
+    evaluation gives."""
+    gen = torch.Generator(device=DEV).manual_seed(3)
+    cfg = stage2.ModelConfig(vocab=64, hidden=hidden, n_layers=layers, n_heads=heads, n_kv_heads=kv_heads, head_dim=64, ffn=ffn)
+    rand = lambda *s: (0.05 * torch.randn(s, device=DEV, generator=gen)).to(torch.bfloat16)
+    params = {"embed": rand(64, hidden), "lm_head": rand(64, hidden), "final_norm": torch.ones(hidden, device=DEV)}
+    for l in range(layers):
+        params[f"attn_norm.{l}"] = params[f"mlp_norm.{l}"] = torch.ones(hidden, device=DEV)
+    weights = [{n: rand(*s) for n, s in cfg.linear_shapes().items()} for _ in range(layers)]
+    model = stage2.Stage2Model(ctx, cfg, params, weights, 1, 16)
+    for lins in model.lin:
+        for x in lins.values():
+            x.V.uniform_(0, 1, generator=gen)
+    model.forward(torch.arange(16, dtype=torch.int32, device=DEV), quantised=True, beta=5.0)
+    for lins in model.lin:
+        for x in lins.values():
+            alone = torch.empty_like(x.Wsoft)
+            faar.softquant_eval(ctx, faar.make_shape(x.O, x.K, 16), x.V, x.code, x.scales, x.s_global, 5.0, None, None, alone)
+            assert torch.equal(x.Wsoft, alone)
