@@ -592,6 +592,14 @@ FAAR_API int faar_model_sizes(const faar_model* model, int batch, int seq, int k
 FAAR_API int faar_model_forward(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* tokens, const int* positions,
                                 int quantised, float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H,
                                 void* workspace, size_t workspace_bytes);
+/* The two forward passes of an alignment step (frozen, without keeping activations; quantised, keeping them) in one call:
+ * the frozen one runs on a stream of the context's own and is joined to the context's stream before the call returns, so
+ * that what is enqueued there next finds both done.  Same results as two calls of faar_model_forward; both arenas are in
+ * use at once.  faar_model_overlap: 1 if the model and batch are small enough to gain from it. */
+FAAR_API int faar_model_overlap(const faar_model* model, int batch, int seq, int* overlap);
+FAAR_API int faar_model_forward_both(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* tokens, const int* positions,
+                                     float beta, void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp, void* arena,
+                                     size_t arena_bytes, void* Z, void* H, void* workspace, size_t workspace_bytes);
 /* From the loss gradients at the logits (dZ, row stride ldz) and at the last hidden state (dH) back to every V, which is
  * updated in place.  arena: of the quantised forward pass with keep != 0 of the same step. */
 FAAR_API int faar_model_backward(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* positions,

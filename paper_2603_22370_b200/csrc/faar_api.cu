@@ -318,6 +318,8 @@ int faar_create(faar_ctx** out, int device, void* stream) {
   c->ev_done[0] = c->ev_done[1] = nullptr;
   c->host_calls = 0;
   c->last_staging = nullptr;
+  c->side_stream = nullptr;
+  c->ev_fork = c->ev_join = nullptr;
   c->last_gemm_bn = 0;
   c->last_gemm_pairs = 0;
   c->prof_on = false;
@@ -339,6 +341,9 @@ int faar_destroy(faar_ctx* ctx) {
     for (int i = 0; i < 2; ++i)
       if (ctx->ev_done[i]) cudaEventDestroy(ctx->ev_done[i]);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
+    if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
+    if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+    if (ctx->side_stream) cudaStreamDestroy(ctx->side_stream);
   }
   delete ctx;
   return FAAR_OK;

@@ -37,6 +37,9 @@ struct faar_ctx {
   cudaEvent_t ev_copied, ev_done[2];
   unsigned long long host_calls;
   const void* last_staging;
+  // faar_model_forward_both: the frozen pass runs on its own stream
+  cudaStream_t side_stream;
+  cudaEvent_t ev_fork, ev_join;
   // per-kernel timing (faar_profile_begin / faar_profile_end)
   bool prof_on;
   int prof_used;                          // event pairs used since faar_profile_begin

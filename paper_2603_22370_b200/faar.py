@@ -76,6 +76,8 @@ SIGNATURES = {
     "faar_attention_bwd": (_I, [_P, _I, _I, _I, _I, _I, _P, _L, _P, _P, _L, _P, _P, _L, _P, _P, _P, _P, _P]),
     "faar_model_sizes": (_I, [_P, _I, _I, _I, _P, _P]),
     "faar_model_forward": (_I, [_P, _P, _I, _I, _P, _P, _I, _F, _I, _P, _Z, _P, _P, _P, _Z]),
+    "faar_model_overlap": (_I, [_P, _I, _I, _P]),
+    "faar_model_forward_both": (_I, [_P, _P, _I, _I, _P, _P, _F, _P, _Z, _P, _P, _P, _Z, _P, _P, _P, _Z]),
     "faar_model_backward": (_I, [_P, _P, _I, _I, _P, _P, _P, _Z, _P, _L, _P, _P, _Z, _P, _Z]),
     "faar_nvfp4_gemm": (_I, [_P, _I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _L, _P, _Z]),
 }
@@ -387,6 +389,18 @@ def model_sizes(model: Model, batch: int, seq: int, keep: int) -> tuple[int, int
 def model_forward(ctx, model, batch, seq, tokens, positions, quantised, beta, keep, arena, Z, H, ws):
     _check(_fast().faar_model_forward(ctx._n, model, batch, seq, tokens, positions, int(quantised), beta, int(keep), arena,
                                       arena.numel(), Z, H, ws, ws.numel()), "faar_model_forward")
+
+
+def model_overlap(model: Model, batch: int, seq: int) -> bool:
+    """Whether the two forward passes of a step gain from running at once (model_forward_both)."""
+    n = C.c_int(0)
+    _check(lib().faar_model_overlap(C.byref(model), batch, seq, C.byref(n)), "faar_model_overlap")
+    return bool(n.value)
+
+
+def model_forward_both(ctx, model, batch, seq, tokens, positions, beta, arena_fp, Z_fp, H_fp, arena, Z, H, ws):
+    _check(_fast().faar_model_forward_both(ctx._n, model, batch, seq, tokens, positions, beta, arena_fp, arena_fp.numel(), Z_fp, H_fp,
+                                           arena, arena.numel(), Z, H, ws, ws.numel()), "faar_model_forward_both")
 
 
 def model_backward(ctx, model, batch, seq, positions, hp, arena, dZ, ldz, dH, scratch, ws):

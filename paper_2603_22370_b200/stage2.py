@@ -109,6 +109,7 @@ class Stage2Model:
         table = self._table()
         self.arena_bytes = {bool(k): faar.model_sizes(table, batch, seq, k)[0] for k in (0, 1)}
         self.scratch_bytes = faar.model_sizes(table, batch, seq, 1)[1]
+        self.overlap = faar.model_overlap(table, batch, seq)
 
     # ---- helpers ------------------------------------------------------------------------------------
     def _new(self, cols, dtype=torch.bfloat16):
@@ -161,6 +162,12 @@ class Stage2Model:
         faar.model_forward(self.ctx, model, self.batch, self.seq, tokens, self.pos, quantised, beta, keep, arena, Z, H, self.ws)
         return Z, H, (arena if keep else None)
 
+    def _forward_both(self, model: faar.Model, tokens, beta):
+        fp, q = (torch.empty(self.arena_bytes[k], dtype=torch.uint8, device=self.dev) for k in (False, True))
+        Z_fp, H_fp, Z, H = self._new(self.cfg.vocab), self._new(self.cfg.hidden), self._new(self.cfg.vocab), self._new(self.cfg.hidden)
+        faar.model_forward_both(self.ctx, model, self.batch, self.seq, tokens, self.pos, beta, fp, Z_fp, H_fp, q, Z, H, self.ws)
+        return Z_fp, H_fp, Z, H, q
+
     # ---- backward ------------------------------------------------------------------------------------
     def backward(self, dZ, dH, saved, hp, want_dv=False):
         """From the loss gradients at the logits and at the last hidden state back to every V (updated in place).
@@ -193,8 +200,11 @@ class Stage2Model:
         return the quantised model's outputs, the loss gradients and every linear's dV (for inspection)."""
         self.step_count += 1
         model = self._table()
-        Z_fp, H_fp = fp_outputs if fp_outputs is not None else self._forward(model, tokens, quantised=False)[:2]
-        Z_q, H_q, saved = self._forward(model, tokens, quantised=True, beta=beta, keep=True)
+        if fp_outputs is None and self.overlap:
+            Z_fp, H_fp, Z_q, H_q, saved = self._forward_both(model, tokens, beta)
+        else:
+            Z_fp, H_fp = fp_outputs if fp_outputs is not None else self._forward(model, tokens, quantised=False)[:2]
+            Z_q, H_q, saved = self._forward(model, tokens, quantised=True, beta=beta, keep=True)
         c, T = self.cfg, self.T
         dZ, dH = torch.empty_like(Z_q), torch.empty_like(H_q)
         faar.align_loss(self.ctx, T, c.vocab, c.hidden, Z_fp, Z_q, Z_q.shape[1], H_fp, H_q, c.hidden, tau, lambda_kl, dZ, dH,

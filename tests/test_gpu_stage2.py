@@ -157,3 +157,35 @@ def test_soft_weights_of_a_model_are_those_of_its_linears(ctx, hidden, heads, kv
             alone = torch.empty_like(x.Wsoft)
             faar.softquant_eval(ctx, faar.make_shape(x.O, x.K, 16), x.V, x.code, x.scales, x.s_global, 5.0, None, None, alone)
             assert torch.equal(x.Wsoft, alone)
+
+
+def test_both_forward_passes_at_once_give_the_same_step(ctx):
+    """The frozen pass on the context's side stream next to the quantised one: losses and every V bit for bit those of one
+    pass after the other, over several steps enqueued without a synchronisation, also on a stream of the caller's."""
+    cfg, _, params, W_fp, _, tokens = small_model(1)
+    B, S = tokens.shape
+    dparams = {k: (dev_bf16(v) if k in ("embed", "lm_head") else dev_f32(v)) for k, v in params.items()}
+    dweights = [{n: dev_bf16(W_fp[l][n]) for n in so.LINEARS} for l in range(cfg["n_layers"])]
+    tok = torch.from_numpy(tokens.reshape(-1).astype(np.int32)).to(DEV)
+    own = torch.cuda.Stream()
+    runs = []
+    try:
+        for stream, overlap in ((torch.cuda.current_stream(), False), (torch.cuda.current_stream(), True), (own, True)):
+            torch.cuda.synchronize()
+            ctx.set_stream(stream)
+            with torch.cuda.stream(stream):
+                model = stage2.Stage2Model(ctx, stage2.ModelConfig(**cfg), dparams, dweights, B, S)
+                assert model.overlap
+                model.overlap = overlap
+                losses = []
+                for _ in range(4):
+                    model.step(tok, beta=4.0)
+                    losses.append(model.loss.clone())
+                torch.cuda.synchronize()
+                faar.check_status(ctx, model.ws)
+                runs.append(losses + [x.V for lins in model.lin for x in lins.values()])
+    finally:
+        torch.cuda.synchronize()
+        ctx.set_stream(torch.cuda.current_stream())
+    for other in runs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(runs[0], other))
