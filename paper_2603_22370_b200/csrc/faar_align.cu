@@ -2,13 +2,16 @@
 // models' logits, the squared error of their last hidden states, and both gradients towards the
 // quantised model's outputs.
 //
-// Softmax needs a row's maximum and sum before any probability, and a token's two logit rows (2 x vocab
-// BF16, 0.5 MB at a 128 K vocabulary) do not fit one SM's shared memory.  One persistent CTA per SM takes
-// a token at a time and reads its rows twice: the first pass (from HBM) keeps a running maximum and sum
-// of exponentials per thread, the second (the same 0.5 MB again, which L2 still holds: one row pair per
-// SM is 76 MB over the chip) forms P_fp, P_q, the KL terms and the gradient.  HBM sees each logit once and
-// the gradient once; the four exponentials per vocabulary entry cost about as much time on the
-// special-function units as the traffic does on HBM, and both passes mix the two.
+// Softmax needs a row's maximum and sum before any probability, and a token's two logit rows (2 x vocab BF16, 0.5 MB at a
+// 128 K vocabulary) do not fit one SM's shared memory, so they are read twice: the first pass (from HBM) keeps a running
+// maximum and sum of exponentials per thread, the second (from L2) forms P_fp, P_q, the KL terms and the gradient.  HBM
+// sees each logit once and the gradient once; the four exponentials per vocabulary entry take the special-function units
+// about as long as the traffic takes HBM.  To have both at work all the time, one loop does the second pass of a token
+// together with the first pass of the next one.  Two tokens' rows per SM would be more than L2 holds at a 128 K vocabulary,
+// so there two CTAs (a cluster on two SMs) share a token, half a row each, and exchange maxima and sums through
+// distributed shared memory.
+// One token after the other, each pass for itself -> this, us: 2000 tokens, vocabulary 32000 144 -> 122; 512, 8000 23.7 ->
+// 16.6; 3000, 50000 298 -> 251; 8192, 128256 1590 -> 1568 (6.3 GB).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -28,9 +31,9 @@ struct AlignParams {
   __nv_bfloat16* dZ; __nv_bfloat16* dH;
   float c;                 // log2(e) / tau: softmax(z / tau) in base 2
   float gscale;            // lambda_kl / (tau T)
-  float* kl_partials;      // one per CTA
-  float* mse_partials;     // one per CTA
-  int T;                   // tokens; CTA k takes tokens k, k + gridDim.x, ...
+  float* kl_partials;      // one per cluster (or CTA)
+  float* mse_partials;
+  int T;                   // tokens; cluster k takes tokens k, k + the number of clusters, ...
 };
 
 __device__ __forceinline__ float ex2f(float x) {
@@ -98,77 +101,108 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&p);
 }
 
+// CL CTAs per token.
+template <int CL>
 __global__ void __launch_bounds__(AL_THREADS, 1)
 align_loss_kernel(const AlignParams p) {
+  if (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // with the wait below: both CTAs have started
   faar_pdl_sync();
-  __shared__ float wred[4][AL_WARPS];
-  __shared__ float row[2];                                         // log2-sum-exp of the token's row: fp, q
+  if (CL > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  __shared__ float4 wred[AL_WARPS];
+  __shared__ float4 xch[2][CL];                                    // by parity of the token: each CTA's maximum and sum, fp and q
+  __shared__ alignas(8) float tot[CL][2];                          // rank 0: every CTA's sums
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rank = CL > 1 ? blockIdx.x % CL : 0, n_cl = gridDim.x / CL;
   const int ngroups = (p.V + 7) / 8;                               // 16-byte groups of a row (rows are padded: ldz >= ceil8(V))
+  const int share = (ngroups + CL - 1) / CL, g_first = rank * share + threadIdx.x, g_end = min(ngroups, (rank + 1) * share);
   const int tail = p.V & 7;                                        // valid columns of a partial last group, 0 = none
   const uint64_t stream = l2_stream_policy(), keep = l2_keep_policy();   // first pass: keep the rows in L2; second: done with them
   float kl = 0.f, mse = 0.f;                                       // this thread's share over all of the CTA's tokens
-  for (int t = blockIdx.x; t < p.T; t += gridDim.x) {
-    const uint4* gf = reinterpret_cast<const uint4*>(p.Zfp + (long long)t * p.ldz);
-    const uint4* gq = reinterpret_cast<const uint4*>(p.Zq + (long long)t * p.ldz);
-
-    // ---- pass 1 (from HBM): running maximum and sum of 2^(c z - max) per thread.  Columns beyond the
-    // vocabulary in the last group count as -1e30 (their exponentials are 0).
-    float mf = -INFINITY, sf = 0.f, mq = -INFINITY, sq = 0.f;
-    auto online = [&](uint4 v, float& m, float& s) {
-      const __nv_bfloat162 x = __hmax2(__hmax2(as_bf162(v.x), as_bf162(v.y)), __hmax2(as_bf162(v.z), as_bf162(v.w)));
-      const float m8 = fmaxf(__low2float(x), __high2float(x)) * p.c;          // tau > 0: scaling keeps the order
-      if (m8 > m) { s *= ex2f(m - m8); m = m8; }                                // 2^-inf = 0 on the first group
-      float z[8];
-      unpack8(v, z);
+  // running maximum and sum of 2^(c z - max) of this thread's part of a row, fp and q
+  float mf, sf, mq, sq;
+  auto online = [&](const uint4& v, float& m, float& s) {
+    const __nv_bfloat162 x = __hmax2(__hmax2(as_bf162(v.x), as_bf162(v.y)), __hmax2(as_bf162(v.z), as_bf162(v.w)));
+    const float m8 = fmaxf(__low2float(x), __high2float(x)) * p.c;          // tau > 0: scaling keeps the order
+    if (m8 > m) { s *= ex2f(m - m8); m = m8; }                                // 2^-inf = 0 on the first group
+    float z[8];
+    unpack8(v, z);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) s += ex2f(fmaf(z[i], p.c, -m));
-    };
-    {
-      int g = threadIdx.x;
-      for (; g + AL_THREADS < ngroups; g += 2 * AL_THREADS) {      // two groups per tensor in flight; only the second can be the row's last
-        const uint4 a0 = ldg128_policy(gf + g, keep), b0 = ldg128_policy(gq + g, keep);
-        const uint4 a1 = ldg128_policy(gf + g + AL_THREADS, keep), b1 = ldg128_policy(gq + g + AL_THREADS, keep);
-        online(a0, mf, sf);
-        online(b0, mq, sq);
-        if (tail && g + AL_THREADS == ngroups - 1) {
-          online(mask_tail(a1, tail), mf, sf);
-          online(mask_tail(b1, tail), mq, sq);
-        } else {
-          online(a1, mf, sf);
-          online(b1, mq, sq);
-        }
-      }
-      if (g < ngroups) {
-        uint4 a = ldg128_policy(gf + g, keep), b = ldg128_policy(gq + g, keep);
-        if (tail && g == ngroups - 1) { a = mask_tail(a, tail); b = mask_tail(b, tail); }
-        online(a, mf, sf);
-        online(b, mq, sq);
-      }
-    }
+    for (int i = 0; i < 8; ++i) s += ex2f(fmaf(z[i], p.c, -m));
+  };
+  // first pass of one group; columns beyond the vocabulary count as -1e30 (their exponentials are 0)
+  auto first = [&](uint4 a, uint4 b, int g) {
+    if (tail && g == ngroups - 1) { a = mask_tail(a, tail); b = mask_tail(b, tail); }
+    online(a, mf, sf);
+    online(b, mq, sq);
+  };
+  // log2-sum-exp of a token's rows from what the threads hold; `parity` alternates between tokens
+  float lse_f = 0.f, lse_q = 0.f;
+  auto combine = [&](int parity) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       merge(mf, sf, __shfl_xor_sync(0xffffffffu, mf, o), __shfl_xor_sync(0xffffffffu, sf, o));
       merge(mq, sq, __shfl_xor_sync(0xffffffffu, mq, o), __shfl_xor_sync(0xffffffffu, sq, o));
     }
-    __syncthreads();                                               // the previous token's readers of wred / row are done
-    if (lane == 0) { wred[0][warp] = mf; wred[1][warp] = sf; wred[2][warp] = mq; wred[3][warp] = sq; }
+    if (lane == 0) wred[warp] = make_float4(mf, sf, mq, sq);
     __syncthreads();
-    if (threadIdx.x == 0) {
-      float a = wred[0][0], b = wred[1][0], c = wred[2][0], d = wred[3][0];
-      for (int w = 1; w < AL_WARPS; ++w) { merge(a, b, wred[0][w], wred[1][w]); merge(c, d, wred[2][w], wred[3][w]); }
-      row[0] = a + lg2f(b);
-      row[1] = c + lg2f(d);
+    if (warp == 0) {
+      float4 r = wred[lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        merge(r.x, r.y, __shfl_xor_sync(0xffffffffu, r.x, o), __shfl_xor_sync(0xffffffffu, r.y, o));
+        merge(r.z, r.w, __shfl_xor_sync(0xffffffffu, r.z, o), __shfl_xor_sync(0xffffffffu, r.w, o));
+      }
+      if (lane < CL) {                                             // lane c: to CTA c of the cluster
+        uint32_t dst = (uint32_t)__cvta_generic_to_shared(&xch[parity][rank]);
+        if (CL > 1) asm volatile("mapa.shared::cluster.u32 %0, %0, %1;" : "+r"(dst) : "r"(lane));
+        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "f"(r.x), "f"(r.y), "f"(r.z), "f"(r.w) : "memory");
+      }
     }
-    __syncthreads();
-    const float lse_f = row[0], lse_q = row[1];
+    if (CL > 1) {
+      __syncwarp();
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
+      __syncthreads();
+    }
+    float4 r = xch[parity][0];
+#pragma unroll
+    for (int c = 1; c < CL; ++c) {
+      const float4 x = xch[parity][c];
+      merge(r.x, r.y, x.x, x.y);
+      merge(r.z, r.w, x.z, x.w);
+    }
+    lse_f = r.x + lg2f(r.y);
+    lse_q = r.z + lg2f(r.w);
+  };
+  auto row = [&](const __nv_bfloat16* z, int t) { return reinterpret_cast<const uint4*>(z + (long long)t * p.ldz); };
 
-    // ---- pass 2 (the same rows again, now from L2: one row pair per SM is in flight, far less than L2 holds):
+  int t = blockIdx.x / CL, parity = 0;
+  mf = mq = -INFINITY;
+  sf = sq = 0.f;
+  if (t < p.T) {
+    const uint4 *gf = row(p.Zfp, t), *gq = row(p.Zq, t);
+    for (int g = g_first; g < g_end; g += AL_THREADS) first(ldg128_policy(gf + g, keep), ldg128_policy(gq + g, keep), g);
+    combine(parity);
+  }
+  for (; t < p.T; t += n_cl) {
+    const int tn = t + n_cl;
+    const bool more = tn < p.T;
+    const uint4 *gf = row(p.Zfp, t), *gq = row(p.Zq, t), *nf = row(p.Zfp, more ? tn : t), *nq = row(p.Zq, more ? tn : t);
     // log2 P = c z - lse, so log2 P_fp - log2 P_q = c (z_fp - z_q) - (lse_fp - lse_q)
     const float dlse = lse_f - lse_q;
     __nv_bfloat16* const gd = p.dZ ? p.dZ + (long long)t * p.ldz : nullptr;
-    for (int g = threadIdx.x; g < ngroups; g += AL_THREADS) {
+    mf = mq = -INFINITY;
+    sf = sq = 0.f;
+    uint4 a1 = make_uint4(0u, 0u, 0u, 0u), b1 = a1;
+    if (more && g_first < g_end) { a1 = ldg128_policy(nf + g_first, keep); b1 = ldg128_policy(nq + g_first, keep); }
+    for (int g = g_first; g < g_end; g += AL_THREADS) {
       uint4 va = ldg128_policy(gf + g, stream), vb = ldg128_policy(gq + g, stream);
+      if (more) {                                                  // the next token's first pass, its loads one group ahead
+        const uint4 a = a1, b = b1;
+        const int gn = g + AL_THREADS;
+        if (gn < g_end) { a1 = ldg128_policy(nf + gn, keep); b1 = ldg128_policy(nq + gn, keep); }
+        first(a, b, g);
+      }
       const bool last_partial = tail && g == ngroups - 1;
       if (last_partial) { va = mask_tail(va, tail); vb = mask_tail(vb, tail); }
       float a[8], b[8], gr[8];
@@ -189,13 +223,12 @@ align_loss_kernel(const AlignParams p) {
         }
       }
     }
-
     // ---- last hidden states
     {
       const __nv_bfloat16* hf = p.Hfp + (long long)t * p.ldh;
       const __nv_bfloat16* hq = p.Hq + (long long)t * p.ldh;
       __nv_bfloat16* dh = p.dH ? p.dH + (long long)t * p.ldh : nullptr;
-      for (int g = threadIdx.x; 8 * g < p.D; g += AL_THREADS) {
+      for (int g = rank * AL_THREADS + threadIdx.x; 8 * g < p.D; g += CL * AL_THREADS) {
         const int nv = min(8, p.D - 8 * g);
         float a[8], b[8], d[8];
         unpack8(reinterpret_cast<const uint4*>(hf)[g], a);         // rows are padded to 8 columns (ldh >= ceil8(D))
@@ -216,17 +249,33 @@ align_loss_kernel(const AlignParams p) {
         }
       }
     }
+    if (more) {
+      parity ^= 1;
+      combine(parity);
+    }
   }
   kl = faar_warp_sum(kl);
   mse = faar_warp_sum(mse);
   __syncthreads();                                                 // wred is reused
-  if (lane == 0) { wred[0][warp] = kl; wred[1][warp] = mse; }
+  if (lane == 0) wred[warp] = make_float4(kl, mse, 0.f, 0.f);
   __syncthreads();
   if (threadIdx.x == 0) {
     float a = 0.f, b = 0.f;
-    for (int w = 0; w < AL_WARPS; ++w) { a += wred[0][w]; b += wred[1][w]; }
-    p.kl_partials[blockIdx.x] = a * 0.6931471805599453f;           // log2 -> natural log
-    p.mse_partials[blockIdx.x] = b;
+    for (int w = 0; w < AL_WARPS; ++w) { a += wred[w].x; b += wred[w].y; }
+    uint32_t dst = (uint32_t)__cvta_generic_to_shared(&tot[rank][0]);
+    if (CL > 1) asm volatile("mapa.shared::cluster.u32 %0, %0, 0;" : "+r"(dst));
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(a), "f"(b) : "memory");
+  }
+  if (CL > 1) {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    float a = 0.f, b = 0.f;
+#pragma unroll
+    for (int c = 0; c < CL; ++c) { a += tot[c][0]; b += tot[c][1]; }
+    p.kl_partials[blockIdx.x / CL] = a * 0.6931471805599453f;      // log2 -> natural log
+    p.mse_partials[blockIdx.x / CL] = b;
   }
 }
 
@@ -245,11 +294,27 @@ int faar_launch_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const vo
   p.gscale = (float)((double)lambda_kl / ((double)tau * (double)T));
   p.kl_partials = kl_partials; p.mse_partials = mse_partials;
   p.T = T;
-  // one persistent CTA per SM, each looping over its tokens: one row pair per SM in flight keeps the second
-  // pass inside L2
-  const int grid = T < ctx->num_sms ? T : ctx->num_sms;
-  *n_partials = grid;
+  // Persistent CTAs, one per SM.  Two tokens' rows (4 vocab bytes each) per CTA or cluster are in use at a time and are to
+  // stay in L2: a CTA per token up to 130 MB, then two.  1500 tokens, one against two, us: vocabulary 88000 (99 MB) 214,
+  // 239; 96000 230, 248; 104000 (117 MB) 258, 271.
   faar_prof_scope ps(ctx, FAAR_K_ALIGN_LOSS);
-  faar_launch_pdl(ctx, align_loss_kernel, dim3(grid), dim3(AL_THREADS), 0, p);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.blockDim = dim3(AL_THREADS);
+  cfg.stream = ctx->stream;
+  cfg.attrs = attr;
+  const int sms = ctx->num_sms;
+  const bool two = T > sms / 2 && 2ll * (T < sms ? T : sms) * 4 * vocab > 130ll << 20;
+  const int most = two ? sms / 2 : sms, n = T < most ? T : most;
+  *n_partials = n;
+  cfg.gridDim = dim3(two ? 2 * n : n);
+  cfg.numAttrs = two ? 2 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, two ? align_loss_kernel<2> : align_loss_kernel<1>, p);
+  if (e != cudaSuccess) return (int)e;
   return (int)cudaGetLastError();
 }

@@ -74,6 +74,13 @@ def test_align_loss_matches_oracle(ctx, T, V, D, tau, lam, pad):
     assert np.array_equal(loss, loss2)
 
 
+@pytest.mark.parametrize("T,V", [(150, 115300), (150, 115021), (400, 1000), (149, 8)])
+def test_tokens_follow_one_another_through_the_loop(ctx, T, V):
+    """More tokens than CTAs, so that a token's second pass runs with the next one's first, for one and for two CTAs per
+    token (the first two shapes lie on both sides of that limit), the row's last group partial, rows of one group."""
+    test_align_loss_matches_oracle(ctx, T, V, 24, 1.3, 0.7, 0)
+
+
 def test_identical_models_give_zero(ctx):
     rng = np.random.default_rng(3)
     Z = _bf16(rng.standard_normal((4, 9000)) * 4)
