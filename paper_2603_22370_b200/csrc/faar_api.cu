@@ -295,14 +295,16 @@ const char* faar_status_string(int status) {
 int faar_create(faar_ctx** out, int device, void* stream) {
   if (!out) return FAAR_ERR_INVALID_ARG;
   *out = nullptr;
-  cudaDeviceProp prop;
-  cudaError_t e = cudaGetDeviceProperties(&prop, device);
+  // single attributes: the whole property structure takes milliseconds of driver queries, for every context
+  int major = 0, sms = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   if (e != cudaSuccess) return FAAR_ERR_CUDA;
-  if (prop.major != 10) return FAAR_ERR_ARCH;
+  if (major != 10) return FAAR_ERR_ARCH;
   faar_ctx* c = new (std::nothrow) faar_ctx();
   if (!c) return FAAR_ERR_INVALID_ARG;
   c->device = device;
-  c->num_sms = prop.multiProcessorCount;
+  c->num_sms = sms;
   c->stream = reinterpret_cast<cudaStream_t>(stream);
   c->last_cuda_error = 0;
   c->encode_tiled = nullptr;
