@@ -137,16 +137,17 @@ FAAR_API const char* faar_status_string(int status);
 FAAR_API int faar_last_cuda_error(const faar_ctx* ctx);
 
 /* ---- GEMM tiling (no counterpart in the paper: tuning and introspection of this library) -------
- * The tensor-core kernels cover the output with 256-row tiles whose width is chosen per launch (a
- * multiple of 16 in [128, 256]): the widest unless the problem is too small to give every CTA pair a
- * tile.  faar_tune_tile_n forces a width for the following launches on this context
+ * The tensor-core kernels cover the output with 256-row tiles whose width is chosen per launch: 256 columns unless
+ * the problem is too small to give every CTA pair a tile, then down to 32.  With few tiles and a long contraction
+ * two or four CTA pairs share a tile's contraction; whether they do depends on the problem and the device alone.
+ * faar_tune_tile_n forces a width (a multiple of 16 in [128, 256]) for the following launches on this context
  * (0 = automatic again).  faar_last_gemm_config reports the width and the number of CTA pairs of the
  * most recent GEMM launch (host out-pointers). */
 FAAR_API int faar_tune_tile_n(faar_ctx* ctx, int bn);
-/* The last, partly empty wave of tiles: the trailing tile columns can be cut into half-width tiles so
- * that more CTA pairs share it and the final, un-overlapped epilogue is half as long.  The number of
- * columns cut is chosen per launch from a cost model; faar_tune_tail_split forces it (-1 = automatic,
- * 0 = none).  faar_last_tail_split reports what the most recent GEMM launch used. */
+/* The last, partly empty wave of tiles: trailing tiles can be cut into half-width tiles so that more CTA pairs
+ * share it and the final, un-overlapped epilogue is half as long.  How many is chosen per launch from a cost model;
+ * faar_tune_tail_split forces a number of whole tile columns (-1 = automatic, 0 = none) and keeps contractions
+ * whole.  faar_last_tail_split reports what the most recent GEMM launch used, rounded up to tile columns. */
 FAAR_API int faar_tune_tail_split(faar_ctx* ctx, int columns);
 FAAR_API int faar_last_tail_split(const faar_ctx* ctx, int* columns);
 FAAR_API int faar_last_gemm_config(const faar_ctx* ctx, int* bn, int* cta_pairs);
@@ -154,8 +155,8 @@ FAAR_API int faar_last_gemm_config(const faar_ctx* ctx, int* bn, int* cta_pairs)
  * traffic per flop, no overlap of a tile's epilogue with the next tile's main loop, no tail split.
  * mode: 1 = whenever the output has more than 256 columns and 256-wide tiles would have been used; 0 = never;
  * -1 (the default) = for plain and forward products where they need one wave of tiles instead of two.
- * faar_last_gemm_config reports bn = 512 for such a launch.  The per-weight results (dW, V, moments) do not depend
- * on the tile shape. */
+ * faar_last_gemm_config reports bn = 512 for such a launch.  0 and 1 also keep contractions whole.  The per-weight
+ * results (dW, V, moments) do not depend on the tile shape. */
 FAAR_API int faar_tune_wide_tiles(faar_ctx* ctx, int mode);
 
 /* Bytes of workspace that any call on this shape needs (host out-pointer).

@@ -211,3 +211,8 @@ def test_glue_argument_checks(ctx):
         with pytest.raises(faar.FaarError) as e:
             call()
         assert e.value.status == status
+
+
+@pytest.mark.parametrize("rows,cols,ld", [(33, 512, 512), (34, 520, 528), (2500, 1000, 1000)])
+def test_rmsnorm_backward_at_the_limits_of_its_register_forms(ctx, rows, cols, ld):
+    test_rmsnorm_forward_and_backward(ctx, rows, cols, ld)

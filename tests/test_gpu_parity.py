@@ -1037,3 +1037,69 @@ def test_chaining_arguments_are_checked(ctx):
         with pytest.raises(faar.FaarError):
             lay.step(faar.make_hparams(beta_next=bad))
     lay.check()
+
+
+# ---- which kernel form a launch takes ---------------------------------------------------------------------------
+@pytest.mark.parametrize("O,K,T", [(2048, 4096, 2560), (2000, 4096, 2570)])
+def test_wide_tiles_chosen_automatically_give_the_same_bits(ctx, O, K, T):
+    """80 tiles of 256 x 256 are two waves of the CTA pairs, 40 of 256 x 512 one: the forward and the plain product take
+    those by themselves, and every output element is the same sum in the same order."""
+    gen = torch.Generator(device=DEV).manual_seed(1)
+    T16 = (T + 15) // 16 * 16
+    shape = faar.make_shape(O, K, T, ldy=T16, yref_transposed=1)
+    rand = lambda *s: torch.randn(s, device=DEV, generator=gen).to(torch.bfloat16)
+    W, X, Yref = 0.02 * rand(O, K), rand(T, K), rand(O, T16)
+    ws = torch.empty(faar.workspace_size(shape), dtype=torch.uint8, device=DEV)
+    faar.workspace_init(ctx, ws)
+    scales, code = (torch.empty((O, K // n), dtype=torch.uint8, device=DEV) for n in (16, 2))
+    sg, V = torch.empty(1, device=DEV), torch.empty((O, K), device=DEV)
+    faar.softquant_init(ctx, shape, W, 0.0, scales, sg, code, V, ws)
+    hp, _ = f32hp(beta=6.0, step=1)
+    out = []
+    try:
+        for wide in (-1, 0):
+            faar.tune_wide_tiles(ctx, wide)
+            Y = torch.zeros((O, T16), dtype=torch.bfloat16, device=DEV)
+            dYt, loss = torch.zeros((O, (T + 7) // 8 * 8), dtype=torch.bfloat16, device=DEV), torch.zeros(1, device=DEV)
+            faar.layer_ref(ctx, shape, X, W, Y, ws)
+            assert faar.last_gemm_config(ctx)[0] == (512 if wide else 256)
+            faar.layer_fwd(ctx, shape, hp, X, Yref, V, code, scales, sg, dYt, loss, None, ws)
+            assert faar.last_gemm_config(ctx)[0] == (512 if wide else 256)
+            out.append((Y[:, :T].clone(), dYt[:, :T].clone()))
+    finally:
+        faar.tune_wide_tiles(ctx, -1)
+    faar.check_status(ctx, ws)
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("yref_dtype", [faar.BF16, faar.F32])
+@pytest.mark.parametrize("O,ldy,offset", [(200, 208, 0), (200, 204, 0), (200, 201, 0), (33, 40, 0), (200, 208, 8), (77, 77, 1)])
+def test_plain_product_rows_of_any_alignment(ctx, O, ldy, offset, yref_dtype):
+    """The result's rows leave as 32-byte, 16-byte or single-value stores depending on where they lie, for narrow tiles too;
+    nothing beyond a row's O values is written.  FP32 sums of 64 products: K 2^-24 of the sum of magnitudes."""
+    K, T = 64, 70
+    gen = torch.Generator(device=DEV).manual_seed(O)
+    W, X = (torch.randn(n, K, device=DEV, generator=gen).to(torch.bfloat16) for n in (O, T))
+    dt = torch.bfloat16 if yref_dtype == faar.BF16 else torch.float32
+    buf = torch.full((offset + T * ldy,), 7.0, dtype=dt, device=DEV)
+    Y = buf[offset:].view(T, ldy)
+    shape = faar.make_shape(O, K, T, ldy=ldy, yref_dtype=yref_dtype)
+    ws = torch.empty(faar.workspace_size(shape), dtype=torch.uint8, device=DEV)
+    faar.workspace_init(ctx, ws)
+    faar.layer_ref(ctx, shape, X, W, Y, ws)
+    faar.check_status(ctx, ws)
+    ref, mag = X.double() @ W.double().T, X.double().abs() @ W.double().abs().T
+    tol = K * 2.0 ** -24 * mag + (2.0 ** -8 * ref.abs() if yref_dtype == faar.BF16 else 0.0)
+    assert torch.all((Y[:, :O].double() - ref).abs() <= tol)
+    assert torch.all(Y[:, O:] == 7.0) and torch.all(buf[:offset] == 7.0)
+
+
+def test_the_native_marshalling_refuses_what_it_cannot_pass_on(ctx):
+    x = torch.zeros((4, 16), dtype=torch.bfloat16, device=DEV)
+    with pytest.raises(AssertionError):
+        faar.add(ctx, 4, 16, x, 16, x.cpu(), 16, x, 16)                    # a host tensor
+    with pytest.raises(TypeError):
+        faar._fast().faar_add(ctx._n, 4, 16, x, 16, x, 16, x)             # an argument short
+    with pytest.raises(TypeError):
+        faar.add(ctx, 4, "16", x, 16, x, 16, x, 16)
+    faar.add(ctx, 4, 16, x, 16, x, 16, x, 16)
