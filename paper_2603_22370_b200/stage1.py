@@ -45,13 +45,16 @@ def optimise_layer(ctx: faar.Context, W: torch.Tensor, X: torch.Tensor, steps: i
     code = torch.empty((O, K // 2), dtype=torch.uint8, device=dev)
     s_global = torch.empty(1, dtype=torch.float32, device=dev)
     V = torch.empty((O, K), dtype=torch.float32, device=dev)
+    # the GPU starts on the set-up while the host allocates the rest; only rows with padding need zeros in it
+    faar.softquant_init(ctx, shape, W, s_global_in, scales, s_global, code, V, ws)
+    padded = torch.empty if T % 16 == 0 else torch.zeros
+    Yref = padded((O, shape.ldy), dtype=torch.bfloat16, device=dev)
+    faar.layer_ref(ctx, shape, X, W, Yref, ws)
+    Xt = padded((K, ldt), dtype=torch.bfloat16, device=dev)
     m = torch.zeros((O, K), dtype=torch.float32, device=dev) if opt == 1 else None
     u = torch.zeros((O, K), dtype=torch.float32, device=dev) if opt == 1 else None
-    Yref = torch.zeros((O, shape.ldy), dtype=torch.bfloat16, device=dev)
     loss = torch.zeros(2, dtype=torch.float32, device=dev)
 
-    faar.softquant_init(ctx, shape, W, s_global_in, scales, s_global, code, V, ws)
-    faar.layer_ref(ctx, shape, X, W, Yref, ws)
     act_scale = 0.0
     Xg = X
     if quantise_activations:
@@ -59,7 +62,6 @@ def optimise_layer(ctx: faar.Context, W: torch.Tensor, X: torch.Tensor, steps: i
         sx = torch.empty(1, dtype=torch.float32, device=dev)
         faar.act_fakequant(ctx, T, K, X, K, 0.0, Xg, K, sx, None, None, ws)
         act_scale = float(sx.item())                     # one read-back at set-up
-    Xt = torch.zeros((K, ldt), dtype=torch.bfloat16, device=dev)
     faar.transpose_bf16(ctx, T, K, Xg, K, Xt, ldt)
 
     history = []
