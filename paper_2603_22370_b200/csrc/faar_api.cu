@@ -587,6 +587,8 @@ int faar_layer_ref(faar_ctx* ctx, const faar_shape* s, const void* X, const void
   FAAR_DEVICE_GUARD(ctx);
   faar_gemm_args a = {};
   a.mode = FAAR_GEMM_REF;
+  // steps take differences against it: its sums keep one order, as the forward product's do
+  a.whole = 1;
   a.Kc = s->K;
   if (s->yref_transposed) {                // Y^T[O, T]: one row per output feature
     a.M = s->O; a.N = s->T;

@@ -1075,7 +1075,6 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               uint32_t r[16];
               tmem_ld16(trow + (uint32_t)c, r);
               tmem_ld_wait();
-              if (SPLIT) add_parts(r, parts, splits, split, TW, c, quarter * 32 + lane);
               warp_acc += epi_fwd_vec(p, o, n0 + c, r, yraw[2 * q], yraw[2 * q + 1]);
             }
           }
@@ -1103,7 +1102,6 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               yref_values(p, ynext, yr);
               if (c + 16 < col_end && n0 + c + 16 < p.N) load_yref(p, o, n0 + c + 16, ynext);
               tmem_ld_wait();
-              if (SPLIT) add_parts(r, parts, splits, split, TW, c, quarter * 32 + lane);
               warp_acc += epi_fwd(p, o, n0 + c, r, yr);
             }
           }
@@ -1260,12 +1258,15 @@ int pick_bn(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int pairs
 // columns (wider ones never won: more to exchange, more to finish), as long as the device holds a cluster for every tile;
 // 64-wide tiles are paid back from 12 k blocks on (two parts of them from 14), 128-wide ones, with twice the exchange,
 // from 20, and from 40 four parts of those are better than two of 64.
-// Measured, whole tiles -> split (parts x width), us: whole step of 640 x 640 at 640 tokens (10 k blocks) 16.6 -> 17.0
-// (2 x 64), of 512 x 768 at 768 tokens (12) 19.3 -> 19.9 (2 x 64), of 128 x 768 at 768 17.4 -> 16.6 (4 x 64); 256 x 1024 at 1024 tokens (16) forward 11.4 -> 10.6 and dW 10.0 -> 9.2 (2 x 64),
-// 11.2 and 10.0 (4 x 128), 10.9 and 10.3 (2 x 128); 128 x 1536 at 1536 tokens (24) 13.6 -> 11.3 and 11.8 -> 10.2 (2 x 64);
-// 300 x 2048 at 2048 tokens 16.2 -> 14.3 and 14.0 -> 12.7 (2 x 128); whole step of 128 x 8192 at 512 tokens 48.3 -> 27.2.
+// Measured, whole tiles -> split (parts x width), us: dW kernel of 256 x 1024 at 1024 tokens (16 k blocks) 10.0 -> 9.2
+// (2 x 64), 10.0 (4 x 128), 10.3 (2 x 128); 128 x 256 at 1024 9.8 -> 8.5 (4 x 64); 128 x 1536 at 1536 (24) 11.8 -> 10.2
+// (2 x 64); 300 x 2048 at 2048 14.0 -> 12.7 (2 x 128); product [128, 768] over 768 (12) 6.1 -> 5.5 (4 x 64), [1024, 83] over
+// 3600 16.2 -> 9.6.
+// The forward product and the frozen target are never split: their difference, the residual, is rounded to BF16, and
+// it is small against either, so that another order of the sums (with the target, another rounding to BF16) moves single
+// entries of the first moments by as much as their mean size.  In the dW and plain products it moves results by 1e-5.
 // The choice depends on the problem and the device alone, not on forced tile widths or operand layouts, because it is part
-// of the order in which an output element is summed (for the plain product it is the same with M and N exchanged).
+// of the order in which an output element is summed (with M and N exchanged a plain product is split alike).
 int pick_splits(int mode, int M, int N, int k_blocks, const int (&clusters)[FAAR_CLUSTER_SIZES], int* bn_out) {
   auto tiles = [](int m, int n, int bn) { return (long long)((m + 2 * BM - 1) / (2 * BM)) * ((n + bn - 1) / bn); };
   struct Form { int size, bn, least; };
@@ -1383,8 +1384,10 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
 
 template <int MODE, int OPT, int MN>
 int launch_tiles(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_out, int bn, int max_pairs, const cudaLaunchConfig_t& cfg) {
-  return kp.splits > 1 ? launch_variant<MODE, OPT, SPLIT_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg)
-                       : launch_variant<MODE, OPT, PLAIN_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+  if constexpr (MODE != FAAR_GEMM_FWD) {
+    if (kp.splits > 1) return launch_variant<MODE, OPT, SPLIT_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+  }
+  return launch_variant<MODE, OPT, PLAIN_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
 }
 
 template <int MODE, int OPT = 0>
@@ -1412,7 +1415,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
   kp.splits = 1;
   int split_bn = BN_MAX;
   // (forced tail splits and wide tiles compare forms of the whole contraction)
-  if (k_blocks >= MIN_SPLIT_BLOCKS && ctx->tune_tail < 0 && ctx->tune_wide < 0) {
+  if (MODE != FAAR_GEMM_FWD && k_blocks >= MIN_SPLIT_BLOCKS && !a->whole && ctx->tune_tail < 0 && ctx->tune_wide < 0) {
     int clusters[FAAR_CLUSTER_SIZES] = {max_pairs};
     for (int i = 1; i < FAAR_CLUSTER_SIZES; ++i) {
       attr[0].val.clusterDim.x = 2u << i;

@@ -24,8 +24,8 @@ def ctx():
     c.close()
 
 
-def small_model(seed=0):
-    cfg = dict(vocab=512, hidden=128, n_layers=2, n_heads=2, n_kv_heads=1, head_dim=64, ffn=256)
+def small_model(seed=0, vocab=512):
+    cfg = dict(vocab=vocab, hidden=128, n_layers=2, n_heads=2, n_kv_heads=1, head_dim=64, ffn=256)
     rng = np.random.default_rng(seed)
     bf = inputs.to_bf16_f32
     params = {"embed": bf(rng.standard_normal((cfg["vocab"], cfg["hidden"]))),
@@ -189,3 +189,10 @@ def test_both_forward_passes_at_once_give_the_same_step(ctx):
         ctx.set_stream(torch.cuda.current_stream())
     for other in runs[1:]:
         assert all(torch.equal(a, b) for a, b in zip(runs[0], other))
+
+
+def test_stage2_step_with_a_split_lm_head_gradient_matches_the_oracle(ctx, monkeypatch):
+    """A vocabulary long enough for the last hidden state's gradient, which contracts over it, to be split over CTA pairs."""
+    build = small_model
+    monkeypatch.setitem(globals(), "small_model", lambda seed=0: build(seed, vocab=1600))
+    test_stage2_step_matches_the_oracle(ctx)
