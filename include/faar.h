@@ -139,7 +139,8 @@ FAAR_API int faar_last_cuda_error(const faar_ctx* ctx);
 /* ---- GEMM tiling (no counterpart in the paper: tuning and introspection of this library) -------
  * The tensor-core kernels cover the output with 256-row tiles whose width is chosen per launch: 256 columns unless
  * the problem is too small to give every CTA pair a tile, then down to 32.  With few tiles and a long contraction
- * two or four CTA pairs share a tile's contraction; whether they do depends on the problem and the device alone.
+ * two or four CTA pairs share a tile's contraction in the dW product, input gradients and a model's products; whether
+ * they do depends on the problem and the device alone.
  * faar_tune_tile_n forces a width (a multiple of 16 in [128, 256]) for the following launches on this context
  * (0 = automatic again).  faar_last_gemm_config reports the width and the number of CTA pairs of the
  * most recent GEMM launch (host out-pointers). */
