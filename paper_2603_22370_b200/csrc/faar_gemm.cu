@@ -13,7 +13,7 @@
 //                                "empty" / "accumulator full" barriers of both CTAs)
 //   warps 2..   : epilogue      (tcgen05.ld; two accumulator buffers, so the epilogue of one tile
 //                                overlaps the main loop of the next)
-// A launch with few tiles and a long contraction splits it (p.splits = 2 or 4): the pairs of a cluster of 4 or 8 CTAs take
+// A REF or BWD launch with few tiles and a long contraction splits it (p.splits = 2 or 4): the pairs of a cluster of 4 or 8 CTAs take
 // a part of the k blocks of the SAME tile each, then every CTA sends the accumulator columns that are another pair's
 // to finish to that pair's CTA of the same rows (distributed shared memory) and finishes its
 // own share of the columns, adding the parts in a fixed order (see exchange_parts).
