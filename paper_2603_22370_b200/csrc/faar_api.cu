@@ -127,6 +127,8 @@ int bwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const v
   if (loss_out2) {
     // the kernel's last CTA forms both values from the forward's MSE partials and its CTAs' Round Loss sums
     a.fin_word = reinterpret_cast<unsigned long long*>(ws) + 1;
+    a.fin_far = reinterpret_cast<unsigned long long*>(ws) + 8;
+    a.fin_far_sums = reinterpret_cast<double*>(ws + l.off_round_partials);
     a.fin_mse_partials = reinterpret_cast<const float*>(ws + l.off_mse_partials);
     a.fin_n_mse = n_mse_partials;
     a.fin_scale_mse = hp->mse_scale;

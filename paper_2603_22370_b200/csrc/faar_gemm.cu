@@ -328,6 +328,8 @@ struct KParams {
   // BWD, optional: the CTA that finishes last also forms the step's two loss values (see the end of the kernel)
   unsigned long long* fin_word;     // workspace word, zero between launches
   double fin_unit, fin_inv_unit;    // fixed-point units per 1 of the Round Loss sum, a power of two; its inverse
+  unsigned long long* fin_far;      // workspace: one bit per CTA whose sum does not fit the fixed-point field (zero between launches)
+  double* fin_far_sums;             // and those sums, by CTA
   const float* fin_mse_partials; int fin_n_mse; float fin_scale_mse;
   float fin_scale_round; float* fin_out2;   // {L_MSE, L_round}; null = no final sums here
 };
@@ -1142,24 +1144,42 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
   if constexpr (MODE == FAAR_GEMM_BWD) {
     // Final loss sums by whichever CTA finishes last.  Each adds its Round Loss sum to one word, as a fixed-point number
-    // above nine bits that count the CTAs and nine that count sums that are not numbers: the addition is exact, so neither
-    // the order nor which CTA is last matters, and the last one has the total from that one atomic (a small layer's step
-    // 18.1 -> 17.2 us, of 1000 x 1040 24.5 -> 22.6 against partials in memory that it had to read back).  After a wait that gave up this CTA's sums are incomplete: it does not count, so nobody forms
-    // final sums (the caller re-initialises the workspace, which also clears the word).
+    // above nine bits that count the CTAs and nine that count sums kept elsewhere.  A sum is rounded to the field's unit
+    // (2^-20 for 16 M weights); the addition is exact, so neither the order nor which CTA is last matters, and the last one
+    // has the total from that one atomic (a small layer's step 18.1 -> 17.2 us, of 1000 x 1040 24.5 -> 22.6 against partials
+    // in memory that it had to read back).  The field has room for one per weight of every CTA's tiles, which is what v in
+    // [0, 1] can give.  A sum beyond that (v outside, infinite or not a number) goes to the CTA's slot in memory with a bit
+    // that says so; the last CTA adds those in the order of the CTAs.  After a wait that gave up this CTA's sums are
+    // incomplete: it does not count, so nobody forms final sums (the caller re-initialises the workspace, which also clears
+    // the word and the bits).
     if (p.fin_out2 != nullptr && threadIdx.x == 0 && !*abort_flag) {
       double rnd = 0.0;
 #pragma unroll
       for (int w = 0; w < C::EPI_WARPS; ++w) rnd += (double)fin_warp[w];
       constexpr uint32_t COUNT = (1u << FIN_COUNT_BITS) - 1u;
-      unsigned long long mine = 1ull + (1ull << FIN_COUNT_BITS);                  // not a number
-      if (rnd == rnd) mine = ((unsigned long long)__double2ll_rn(rnd * p.fin_unit) << (2 * FIN_COUNT_BITS)) + 1ull;
+      const int columns = SPLIT ? share_begin(BN, splits, split + 1) - share_begin(BN, splits, split) : (WIDE ? WIDE_BN : BN);
+      const double room = (double)((total_tiles - pair + n_pairs - 1) / n_pairs) * (double)(BM * columns);
+      unsigned long long mine;
+      if (fabs(rnd) <= room) {
+        mine = ((unsigned long long)__double2ll_rn(rnd * p.fin_unit) << (2 * FIN_COUNT_BITS)) + 1ull;
+      } else {
+        p.fin_far_sums[blockIdx.x] = rnd;
+        atomicOr(p.fin_far + (blockIdx.x >> 6), 1ull << (blockIdx.x & 63));
+        __threadfence();
+        mine = 1ull + (1ull << FIN_COUNT_BITS);
+      }
       const unsigned long long sum = atomicAdd(p.fin_word, mine) + mine;
       if (((uint32_t)sum & COUNT) == gridDim.x) {
         *p.fin_word = 0ull;                                  // ready for the next launch
+        double total = (double)((long long)sum >> (2 * FIN_COUNT_BITS)) * p.fin_inv_unit;
+        if (((uint32_t)sum >> FIN_COUNT_BITS & COUNT) != 0u) {
+          __threadfence();
+          for (uint32_t c = 0; c < gridDim.x; ++c)
+            if (__ldcg(p.fin_far + (c >> 6)) >> (c & 63) & 1ull) total += __ldcg(p.fin_far_sums + c);
+          for (uint32_t i = 0; i <= (gridDim.x - 1) >> 6; ++i) p.fin_far[i] = 0ull;
+        }
         p.fin_out2[0] = (float)(*fin_mse * (double)p.fin_scale_mse);
-        p.fin_out2[1] = ((uint32_t)sum >> FIN_COUNT_BITS & COUNT) != 0u
-                            ? __uint_as_float(0x7FC00000u)
-                            : (float)((double)((long long)sum >> (2 * FIN_COUNT_BITS)) * p.fin_inv_unit * (double)p.fin_scale_round);
+        p.fin_out2[1] = (float)(total * (double)p.fin_scale_round);
       }
     }
   }
@@ -1353,6 +1373,14 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   const int m_tiles = (a->M + 2 * BM - 1) / (2 * BM), n_cols = (a->N + bn - 1) / bn;
   kp.narrow = SHAPE == PLAIN_TILES && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
   kp.n_main = n_cols - kp.narrow;
+  if (MODE == FAAR_GEMM_BWD) {
+    // the widest unit at which the Round Loss field holds one per weight of the tiles (half tiles counted as whole: twice
+    // that) with its sign
+    const long long area = (long long)m_tiles * 2 * BM * (WIDE ? (a->N + WIDE_BN - 1) / WIDE_BN * (long long)WIDE_BN : (long long)n_cols * bn);
+    int int_bits = 1;
+    while (area >> int_bits) ++int_bits;
+    kp.fin_unit = ldexp(1.0, 62 - 2 * FIN_COUNT_BITS - int_bits); kp.fin_inv_unit = 1.0 / kp.fin_unit;
+  }
   kp.n_full = WIDE ? 0 : (SHAPE == SPLIT_TILES ? m_tiles * kp.n_main : pick_full(ctx, MODE, m_tiles, kp.n_main, kp.narrow, bn, max_pairs));
   CUtensorMap tmA, tmB, tmBh;
   e = a->a_mn ? make_map_mn(ctx, &tmA, a->A, a->Kc, a->M, a->lda) : make_map(ctx, &tmA, a->A, a->M, a->Kc, a->lda, BM);
@@ -1496,10 +1524,7 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* a, int* n_partials_out
   kp.nbl_next = -(a->beta_next * 1.4426950408889634f); kp.hbl_next = -0.5f * kp.nbl_next;
   kp.wsoft_next = a->wsoft_next;
   kp.fin_word = a->fin_word;
-  // the sum is at most M N: the widest fixed-point field that holds it with its sign
-  int int_bits = 1;
-  while (((long long)a->M * a->N) >> int_bits) ++int_bits;
-  kp.fin_unit = ldexp(1.0, 62 - 2 * FIN_COUNT_BITS - int_bits); kp.fin_inv_unit = 1.0 / kp.fin_unit;
+  kp.fin_far = a->fin_far; kp.fin_far_sums = a->fin_far_sums;
   if (a->fin_out2 && ctx->num_sms >= 1 << FIN_COUNT_BITS) return (int)cudaErrorInvalidValue;
   kp.fin_mse_partials = a->fin_mse_partials; kp.fin_n_mse = a->fin_n_mse;
   kp.fin_scale_mse = a->fin_scale_mse; kp.fin_scale_round = a->fin_scale_round; kp.fin_out2 = a->fin_out2;

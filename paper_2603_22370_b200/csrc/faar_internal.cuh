@@ -83,7 +83,9 @@ static inline cudaError_t faar_launch_pdl(faar_ctx* ctx, void (*kernel)(KArgs...
 // ---- workspace layout -------------------------------------------------------
 // [0, 256)            header: word 0 = status (0 = ok), bytes 8..15 = the final sums of a
 //                     dW launch while its CTAs finish (zero between launches), bytes 16..23 = tensor maximum of
-//                     the last set-up pass (high word: the pass's serial number, low word: max |W| bits)
+//                     the last set-up pass (high word: the pass's serial number, low word: max |W| bits),
+//                     bytes 64..127 = a bit per CTA of a dW launch whose Round Loss sum lies in the Round region
+//                     (zero between launches)
 // [256, 256+P)        loss partials (float): MSE region then Round region
 // [..]                W_soft bf16 [O,K]
 // [..]                dYt bf16 [O, ceil8(T)]
@@ -216,7 +218,7 @@ struct faar_gemm_args {
   // BWD, optional: also write the next step's BF16 operand W_soft(V', beta_next) (null = not wanted)
   __nv_bfloat16* wsoft_next; float beta_next;
   // BWD, optional: final loss sums by the last CTA (fin_out2 null = not wanted)
-  unsigned long long* fin_word; const float* fin_mse_partials; int fin_n_mse; float fin_scale_mse, fin_scale_round;
+  unsigned long long* fin_word; unsigned long long* fin_far; double* fin_far_sums; const float* fin_mse_partials; int fin_n_mse; float fin_scale_mse, fin_scale_round;
   float* fin_out2;
 };
 // n_partials_out: number of floats a FWD launch writes to args.partials

@@ -880,6 +880,34 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_survives(ctx):
     assert rel_l2(host(lay.V), Vo) <= 2e-3
 
 
+@pytest.mark.parametrize("O,K,T", [(128, 256, 256), (1000, 1040, 203)])      # split contraction; half-width tiles
+@pytest.mark.parametrize("opt", [0, 1])
+def test_round_loss_of_a_step_for_any_v(ctx, O, K, T, opt):
+    """V is the caller's: values outside [0, 1], infinities and NaN count in the first step's Round Loss as its definition
+    says, mean(1 - (2v - 1)^2), and leave nothing behind for the next step's (V is clipped by then).  FP32 terms summed per
+    thread: 2^-16 of the terms' magnitudes."""
+    W, X, Yref = _problem(O, K, T, seed=3)
+    lay = GpuLayer(ctx, W, X)
+    lay.init()
+    lay.set_yref(Yref)
+    V0 = host(lay.V).copy()
+    one = np.zeros(V0.shape, bool)
+    one.flat[V0.size // 3] = True
+    for v in (V0, np.full_like(V0, 2.0), np.full_like(V0, -1.0), np.full_like(V0, 1.5), np.full_like(V0, 1e3),
+              np.where(one, np.float32(1e10), V0), np.where(one, np.float32(np.inf), V0), np.where(one, np.float32(-np.inf), V0),
+              np.where(one, np.float32(np.nan), V0)):
+        lay.set_state(V=v, m=np.zeros_like(V0), u=np.zeros_like(V0))
+        for step in (1, 2):
+            t2 = (2.0 * host(lay.V).astype(np.float64) - 1.0) ** 2
+            lay.step(f32hp(beta=4.0, step=step, opt=opt)[0])
+            lay.check()
+            want, got = np.mean(1.0 - t2), float(host(lay.loss)[1])
+            if np.isfinite(want):
+                assert abs(got - want) <= 2.0 ** -16 * np.mean(1.0 + t2), (float(v.flat[0]), step, got, want)
+            else:
+                assert np.isnan(got) if np.isnan(want) else got == want, (step, got, want)
+
+
 def test_outputs_stay_inside_their_buffers(ctx):
     """Canaries around every buffer a step writes (dY^T, V, Adam moments, dV, losses) and around the packed
     output: a ragged shape, so that partial tiles, partial panels and partial vectors all occur."""
