@@ -350,23 +350,25 @@ __device__ __forceinline__ void nearest_block(const float (&q)[16], float sg, ui
 
 // One scale block: its values in BF16 (o), its codes (cw); returns its E4M3 scale.
 __device__ __forceinline__ uint32_t fakequant_block(const block_raw& raw, float s_global, float d, float rd, uint32_t (&o)[8], uint32_t (&cw)[2]) {
-      float w[16];
-      bool has_minute;
-      const float amax = unpack_block<true>(raw, w, &has_minute);
-      const uint32_t sb = block_scale(amax, d, rd);
-      const float sg = faar_e4m3_to_float(sb);
-      const float s = __fmul_rn(sg, s_global);
-          float q[16];
-      // a quotient far below the smallest midpoint need not be exact, so minute values take the fast path here (and -0.0
-      // becomes +0.0 in its residual corrections)
-      if (fast_division_ok(s, amax, false)) {
-        block_quotients<true>(w, s, q);
-      } else {
-        block_quotients<false>(w, s, q);
-  #pragma unroll
-        for (int i = 0; i < 16; ++i) q[i] = copysignf(q[i], w[i] < 0.f ? -1.0f : 1.0f);
-      }
-      nearest_block(q, sg, o, cw);
+  float w[16];
+  bool has_minute;
+  const float amax = unpack_block<true>(raw, w, &has_minute);
+  const uint32_t sb = block_scale(amax, d, rd);
+  const float sg = faar_e4m3_to_float(sb);
+  const float s = __fmul_rn(sg, s_global);
+  float q[16];
+  // a quotient far below the smallest midpoint need not be exact, so minute values take the fast path here (and -0.0
+  // becomes +0.0 in its residual corrections)
+  if (fast_division_ok(s, amax, false)) {
+    block_quotients<true>(w, s, q);
+  } else {
+    block_quotients<false>(w, s, q);
+    // infinite quotients (and inf / inf) are the largest node with the value's sign: setting the lowest bit of an infinity
+    // would make it a NaN, which the conversion takes for +6
+#pragma unroll
+    for (int i = 0; i < 16; ++i) q[i] = copysignf(fminf(fabsf(q[i]), 6.0f), w[i] < 0.f ? -1.0f : 1.0f);
+  }
+  nearest_block(q, sg, o, cw);
   return sb;
 }
 

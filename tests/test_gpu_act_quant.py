@@ -107,6 +107,22 @@ def test_act_fakequant_over_the_bf16_range(ctx, sg_in, spread):
     assert np.array_equal(host(Xq).astype(np.float64), units)
 
 
+@pytest.mark.parametrize("sg_in", [0.0, 0.013, 2.0 ** -100])
+@pytest.mark.parametrize("T,K", [(3, 48), (65, 2048)])                  # one launch, two launches
+def test_act_fakequant_of_infinite_values(ctx, T, K, sg_in):
+    """An infinite value, or one whose quotient overflows, is the largest node with its own sign."""
+    rng = np.random.default_rng(T)
+    X = rng.standard_normal((T, K)).astype(np.float32)
+    X[0, 0], X[0, 17], X[1, 20], X[2, 47] = -np.inf, np.inf, -np.float32(2.0 ** 127), np.float32(2.0 ** 127)
+    Xq, _, packed, scales = _quantise(ctx, X, sg_in)
+    codes = host(packed)
+    nibble = lambda r, c: int(codes[r, c // 2]) >> (4 * (c & 1)) & 15
+    big = [(0, 0, -1), (0, 17, 1)] + ([(1, 20, -1), (2, 47, 1)] if sg_in else [])
+    for r, c, sign in big:
+        assert nibble(r, c) == (15 if sign < 0 else 7), (r, c)
+        assert host(scales)[r, c // 16] == 0x7E and host(Xq)[r, c] == sign * 6 * 448.0
+
+
 @pytest.mark.parametrize("O,K,T", [(300, 1040, 600), (128, 256, 1024)])
 def test_layer_step_on_quantised_activations(ctx, O, K, T):
     W, X = inputs.config2(9, O, K, T)
