@@ -15,8 +15,9 @@
 // converged warp: fwd 145.5 -> 140.6 us, bwd 385 -> 354 us at 4 x 2048 tokens, 32 heads, against a lane-0 branch); the
 // scores have two buffers in tensor memory, so S of tile j + 1 is formed while the warps work on tile j, and two
 // CTAs per SM overlap what remains serial (softmax -> P V).
-// Rows of a query tile beyond the sequence end compute on whatever rows follow in memory (or zeros past the
-// tensor) and are not stored; keys beyond the end are masked.
+// Rows of a tile beyond the sequence end arrive as zeros (the copies' maps have the sequence as a dimension of its own): a
+// probability of 0 for a masked key would not keep an infinity or NaN of the next sequence's rows out of a product.  Query
+// rows beyond the end are not stored; keys beyond it are masked.
 // Every barrier wait is bounded; a wait that gives up records a code in a status word of this module (read by
 // faar_attention_status), raises the CTA's abort flag and all roles leave.
 #include <cuda.h>
@@ -89,9 +90,9 @@ __device__ __noinline__ bool bar_wait_slow(uint32_t b, uint32_t parity, volatile
 __device__ __forceinline__ bool bar_wait(uint32_t b, uint32_t parity, volatile int* abort_flag, uint32_t code) {
   return bar_try(b, parity) ? true : bar_wait_slow(b, parity, abort_flag, code);
 }
-__device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-               ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
+__device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+  asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+               ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -196,11 +197,11 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// NP boxes of 64 columns
+// NP boxes of 64 columns, rows from `row` of sequence b (rows beyond the sequence arrive as zeros)
 template <int HD>
-__device__ __forceinline__ void tma_head(uint32_t dst, uint32_t panel, const CUtensorMap* map, int x, int y, uint32_t bar) {
+__device__ __forceinline__ void tma_head(uint32_t dst, uint32_t panel, const CUtensorMap* map, int x, int row, int b, uint32_t bar) {
 #pragma unroll
-  for (int c = 0; c < HD / 64; ++c) tma_2d(dst + c * panel, map, x + 64 * c, y, bar);
+  for (int c = 0; c < HD / 64; ++c) tma_3d(dst + c * panel, map, x + 64 * c, row, b, bar);
 }
 
 template <int HD>
@@ -262,16 +263,16 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
     };
     auto load_k = [&](int j) {
-      if (lead) { bar_expect(kfull(j & 1), KV_BYTES); tma_head<HD>(sK(j & 1), KV_PANEL, &tmK, g * HD, (int)(seq0 + (long long)j * KT), kfull(j & 1)); }
+      if (lead) { bar_expect(kfull(j & 1), KV_BYTES); tma_head<HD>(sK(j & 1), KV_PANEL, &tmK, g * HD, j * KT, b, kfull(j & 1)); }
       __syncwarp();
     };
     auto load_v = [&](int j) {
-      if (lead) { bar_expect(vfull(j & 1), KV_BYTES); tma_head<HD>(sV(j & 1), KV_PANEL, &tmV, g * HD, (int)(seq0 + (long long)j * KT), vfull(j & 1)); }
+      if (lead) { bar_expect(vfull(j & 1), KV_BYTES); tma_head<HD>(sV(j & 1), KV_PANEL, &tmV, g * HD, j * KT, b, vfull(j & 1)); }
       __syncwarp();
     };
     if (lead) {
       bar_expect(bar_q, Q_BYTES);
-      tma_head<HD>(sQ, Q_PANEL, &tmQ, h * HD, (int)(seq0 + q0), bar_q);
+      tma_head<HD>(sQ, Q_PANEL, &tmQ, h * HD, q0, b, bar_q);
     }
     load_k(0); load_v(0);
     if (n_kt > 1) { load_k(1); load_v(1); }
@@ -536,15 +537,15 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       const int st = j % C::STAGES;
       if (lead) {
         bar_expect(kvfull(st), 2 * KV_BYTES);
-        tma_head<HD>(sK(st), KV_PANEL, &tmK, g * HD, (int)(seq0 + (long long)j * KT), kvfull(st));
-        tma_head<HD>(sV(st), KV_PANEL, &tmV, g * HD, (int)(seq0 + (long long)j * KT), kvfull(st));
+        tma_head<HD>(sK(st), KV_PANEL, &tmK, g * HD, j * KT, b, kvfull(st));
+        tma_head<HD>(sV(st), KV_PANEL, &tmV, g * HD, j * KT, b, kvfull(st));
       }
       __syncwarp();
     };
     if (lead) {
       bar_expect(bar_qd, 2 * Q_BYTES);
-      tma_head<HD>(sQ, Q_PANEL, &tmQ, h * HD, (int)(seq0 + q0), bar_qd);
-      tma_head<HD>(sDO, Q_PANEL, &tmDO, h * HD, (int)(seq0 + q0), bar_qd);
+      tma_head<HD>(sQ, Q_PANEL, &tmQ, h * HD, q0, b, bar_qd);
+      tma_head<HD>(sDO, Q_PANEL, &tmDO, h * HD, q0, b, bar_qd);
     }
     load_kv(0);
     if (n_kt > 1) load_kv(1);
@@ -702,7 +703,7 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 // chain (score products -> rows -> accumulating products -> next item's score products, which overwrite P^T / dS^T
 // and so wait for the accumulating products).  Q / dO tiles come through four TMA stages (requested three items
 // ahead), lse and delta of a tile's 64 queries are staged in shared memory by the row threads themselves.  Queries
-// beyond the sequence end are masked (their rows hold the next sequence's data).
+// beyond the sequence end are masked.
 // head_dim 128: dV and dK take 256 columns and the operands 162 KB, so one CTA per SM with all 512 columns: two S^T and two
 // dP^T buffers, the score products of item i + 1 run while the rows work on item i; three stages.
 template <int HD> struct Dkv {
@@ -788,15 +789,15 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const int st = i % C::STAGES;
       if (lead) {
         bar_expect(qfull(st), 2 * C::QD_BYTES);
-        tma_head<HD>(sQ(st), KV_PANEL, &tmQ, head_of(i) * HD, (int)(seq0 + q0_of(i)), qfull(st));
-        tma_head<HD>(sDO(st), KV_PANEL, &tmDO, head_of(i) * HD, (int)(seq0 + q0_of(i)), qfull(st));
+        tma_head<HD>(sQ(st), KV_PANEL, &tmQ, head_of(i) * HD, q0_of(i), b, qfull(st));
+        tma_head<HD>(sDO(st), KV_PANEL, &tmDO, head_of(i) * HD, q0_of(i), b, qfull(st));
       }
       __syncwarp();
     };
     if (lead) {
       bar_expect(bar_kv, 2 * C::KEY_BYTES);
-      tma_head<HD>(sKt, Q_PANEL, &tmK, g * HD, (int)(seq0 + k0), bar_kv);
-      tma_head<HD>(sVt, Q_PANEL, &tmV, g * HD, (int)(seq0 + k0), bar_kv);
+      tma_head<HD>(sKt, Q_PANEL, &tmK, g * HD, k0, b, bar_kv);
+      tma_head<HD>(sVt, Q_PANEL, &tmV, g * HD, k0, b, bar_kv);
     }
     load_item(0);
     if (n_it > 1) load_item(1);
@@ -971,13 +972,13 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// [rows, cols] BF16, row stride ld elements: boxes of 64 columns x box_rows rows, 128-byte swizzle
-int head_map(faar_ctx* ctx, CUtensorMap* map, const void* ptr, long long rows, int cols, long long ld, int box_rows) {
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
-  cuuint32_t es[2] = {1, 1};
-  CUresult r = reinterpret_cast<EncodeFn>(ctx->encode_tiled)(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims,
+// B sequences of [S, cols] BF16, row stride ld elements: boxes of 64 columns x box_rows rows of one sequence, 128-byte swizzle
+int head_map(faar_ctx* ctx, CUtensorMap* map, const void* ptr, int B, int S, int cols, long long ld, int box_rows) {
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)S, (cuuint64_t)B};
+  cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)S * (cuuint64_t)ld * 2};
+  cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  CUresult r = reinterpret_cast<EncodeFn>(ctx->encode_tiled)(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims,
                                                              strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                                                              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -988,11 +989,10 @@ template <int HD>
 int launch_fwd(faar_ctx* ctx, const TcParams& p, const void* q, int64_t ldq, const void* k, const void* v, int64_t ldk) {
   using F = Fwd<HD>;
   static_assert(2 * (F::SMEM + 1024) <= 228 * 1024, "two CTAs per SM");
-  const long long T = (long long)p.B * p.S;
   CUtensorMap tmQ, tmK, tmV;
-  int e = head_map(ctx, &tmQ, q, T, p.H * HD, ldq, QT);
-  if (!e) e = head_map(ctx, &tmK, k, T, p.Hkv * HD, ldk, KT);
-  if (!e) e = head_map(ctx, &tmV, v, T, p.Hkv * HD, ldk, KT);
+  int e = head_map(ctx, &tmQ, q, p.B, p.S, p.H * HD, ldq, QT);
+  if (!e) e = head_map(ctx, &tmK, k, p.B, p.S, p.Hkv * HD, ldk, KT);
+  if (!e) e = head_map(ctx, &tmV, v, p.B, p.S, p.Hkv * HD, ldk, KT);
   if (!e) e = faar_allow_smem(ctx, (const void*)attn_fwd_tc_kernel<HD>, F::SMEM);
   if (e) return e;
   faar_launch_pdl(ctx, attn_fwd_tc_kernel<HD>, dim3(((p.S + QT - 1) / QT) * p.H * p.B, 1, 1), dim3(THREADS), F::SMEM, tmQ, tmK, tmV, p);
@@ -1002,16 +1002,15 @@ int launch_fwd(faar_ctx* ctx, const TcParams& p, const void* q, int64_t ldq, con
 template <int HD>
 int launch_bwd(faar_ctx* ctx, const TcBwdParams& p, const void* q, int64_t ldq, const void* k, const void* v, int64_t ldk,
                const void* dout, int64_t ldo) {
-  const long long T = (long long)p.B * p.S;
   CUtensorMap tmQ, tmDO, tmK, tmV, tmQk, tmDOk, tmKk, tmVk;      // boxes of 128 rows / of 64 rows
-  int e = head_map(ctx, &tmQ, q, T, p.H * HD, ldq, QT);
-  if (!e) e = head_map(ctx, &tmDO, dout, T, p.H * HD, ldo, QT);
-  if (!e) e = head_map(ctx, &tmK, k, T, p.Hkv * HD, ldk, QT);
-  if (!e) e = head_map(ctx, &tmV, v, T, p.Hkv * HD, ldk, QT);
-  if (!e) e = head_map(ctx, &tmQk, q, T, p.H * HD, ldq, KT);
-  if (!e) e = head_map(ctx, &tmDOk, dout, T, p.H * HD, ldo, KT);
-  if (!e) e = head_map(ctx, &tmKk, k, T, p.Hkv * HD, ldk, KT);
-  if (!e) e = head_map(ctx, &tmVk, v, T, p.Hkv * HD, ldk, KT);
+  int e = head_map(ctx, &tmQ, q, p.B, p.S, p.H * HD, ldq, QT);
+  if (!e) e = head_map(ctx, &tmDO, dout, p.B, p.S, p.H * HD, ldo, QT);
+  if (!e) e = head_map(ctx, &tmK, k, p.B, p.S, p.Hkv * HD, ldk, QT);
+  if (!e) e = head_map(ctx, &tmV, v, p.B, p.S, p.Hkv * HD, ldk, QT);
+  if (!e) e = head_map(ctx, &tmQk, q, p.B, p.S, p.H * HD, ldq, KT);
+  if (!e) e = head_map(ctx, &tmDOk, dout, p.B, p.S, p.H * HD, ldo, KT);
+  if (!e) e = head_map(ctx, &tmKk, k, p.B, p.S, p.Hkv * HD, ldk, KT);
+  if (!e) e = head_map(ctx, &tmVk, v, p.B, p.S, p.Hkv * HD, ldk, KT);
   if (!e) e = faar_allow_smem(ctx, (const void*)attn_dkv_tc_kernel<HD>, Dkv<HD>::SMEM);
   if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_tc_kernel<HD>, Dq<HD>::SMEM);
   if (e) return e;

@@ -164,6 +164,31 @@ def test_attention_at_the_alignment_benchmark_size_on_sampled_head_groups(ctx, f
         assert abs(float(lse[b, h, S - 1]) - ref) <= 1e-3 * max(1.0, abs(ref))
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("S", [7, 65, 100, 190])                        # rows of a 64-key and of a 128-query tile beyond the end
+def test_a_sequence_does_not_see_the_next_ones_values(ctx, S, D):
+    """Infinities and NaN in the second sequence: every output of the first is bit for bit what it is without them."""
+    H, HKV, B = 4, 2, 2
+    gen = torch.Generator(device=DEV).manual_seed(S + D)
+    rand = lambda h: torch.randn((B * S, h * D), device=DEV, generator=gen).to(torch.bfloat16)
+    q, k, v, do = rand(H), rand(HKV), rand(HKV), rand(H)
+    outs = []
+    for poke in (False, True):
+        if poke:
+            for t, x in ((q, float("inf")), (k, float("nan")), (v, float("-inf")), (do, float("nan"))):
+                t[S:] = x
+        o, dq, dk, dv = (torch.zeros_like(t) for t in (q, q, k, v))
+        lse = torch.zeros((B, H, S), dtype=torch.float32, device=DEV)
+        dsum = torch.zeros_like(lse)
+        faar.attention_fwd(ctx, B, S, H, HKV, D, q, H * D, k, v, HKV * D, o, H * D, lse)
+        faar.attention_bwd(ctx, B, S, H, HKV, D, q, H * D, k, v, HKV * D, o, do, H * D, lse, dsum, dq, dk, dv)
+        torch.cuda.synchronize()
+        faar.attention_status(ctx)
+        outs.append([t[:S].clone() for t in (o, dq, dk, dv)] + [lse[0].clone()])
+    assert all(torch.isfinite(t).all() for t in outs[0])
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+
+
 def test_attention_argument_checks(ctx):
     x = torch.zeros((64, 128), dtype=torch.bfloat16, device=DEV)
     lse = torch.zeros(128, dtype=torch.float32, device=DEV)
