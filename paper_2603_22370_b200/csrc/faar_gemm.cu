@@ -305,9 +305,9 @@ struct KParams {
   // REF / FWD
   void* Yout; int yout_dtype; long long ldy;
   const void* Yref; int yref_dtype;
-  int yref_t;             // FWD: Y_ref / Y_q stored transposed, [O, ldy] with ldy >= T rounded up to 16
-  int y_store;            // REF: rows of Yout take 16 columns as 3: one 32-byte store, padded (columns beyond N are written as 0),
-                          // 2: one 32-byte store, 1: 16-byte stores, 0: single values
+  int yref_t;             // FWD: Y_ref / Y_q stored transposed, [O, ldy] with ldy >= T rounded up to 16; REF: rows of Yout are
+                          // padded like that, columns beyond N up to the next multiple of 16 are written as 0
+  int y_store;            // REF: rows of Yout take 2: 32-byte stores, 1: 16-byte stores, 0: single values
   __nv_bfloat16* dYt; long long ld_dyt;
   float mse2c;
   float act_scale;        // FWD: Y_q = act_scale * acc; BWD: G = act_scale * acc
@@ -398,11 +398,16 @@ __device__ __forceinline__ void stg256(void* ptr, const uint32_t (&w)[8]) {
 // REF: write acc to row `row`, columns c0..c0+15 of Y.  A whole 32-byte sector per lane and instruction: with the output
 // feature in the lane and the token in the column (2-byte stores, 64 bytes per warp instruction) the epilogue of a
 // 256-wide tile took 7.4-9 us, most of it after the last product of a launch.
+__device__ __forceinline__ void store_units(void* y, const uint32_t (&w)[8], bool wide) {      // 32 bytes
+  if (wide) { stg256(y, w); return; }
+  reinterpret_cast<uint4*>(y)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+  reinterpret_cast<uint4*>(y)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+}
 __device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const uint32_t (&acc)[16]) {
   if (row >= p.M) return;
   const long long off = (long long)row * p.ldy + c0;
-  if (p.y_store >= 2 && (p.y_store == 3 || c0 + 16 <= p.N)) {
-    const bool whole = c0 + 16 <= p.N;
+  const bool whole = c0 + 16 <= p.N, wide = p.y_store == 2;
+  if (p.y_store && (whole || p.yref_t)) {
     if (p.yout_dtype == FAAR_BF16) {
       __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + off;
       uint32_t w[8];
@@ -410,7 +415,7 @@ __device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const
       for (int j = 0; j < 8; ++j)
         w[j] = pack_bf16x2(whole || c0 + 2 * j < p.N ? __uint_as_float(acc[2 * j]) : 0.f,
                            whole || c0 + 2 * j + 1 < p.N ? __uint_as_float(acc[2 * j + 1]) : 0.f);
-      if (FAAR_DBG_OK(p, y, 32, p.Yout, p.ext_yout, 1u)) stg256(y, w);
+      if (FAAR_DBG_OK(p, y, 32, p.Yout, p.ext_yout, 1u)) store_units(y, w, wide);
     } else {
       float* y = reinterpret_cast<float*>(p.Yout) + off;
       if (!FAAR_DBG_OK(p, y, 64, p.Yout, p.ext_yout, 1u)) return;
@@ -419,7 +424,7 @@ __device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const
         uint32_t w[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) w[j] = whole || c0 + 8 * h + j < p.N ? acc[8 * h + j] : 0u;
-        stg256(y + 8 * h, w);
+        store_units(y + 8 * h, w, wide);
       }
     }
     return;
@@ -427,17 +432,6 @@ __device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const
   const int n = min(16, p.N - c0);
   if (p.yout_dtype == FAAR_BF16) {
     __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + off;
-    if (p.y_store && n == 16) {
-      if (!FAAR_DBG_OK(p, y, 32, p.Yout, p.ext_yout, 1u)) return;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = pack_bf16x2(__uint_as_float(acc[8 * h + 2 * j]), __uint_as_float(acc[8 * h + 2 * j + 1]));
-        reinterpret_cast<uint4*>(y)[h] = make_uint4(w[0], w[1], w[2], w[3]);
-      }
-      return;
-    }
 #pragma unroll
     for (int j = 0; j < 16; ++j)
       if (j < n && FAAR_DBG_OK(p, y + j, 2, p.Yout, p.ext_yout, 1u)) y[j] = __float2bfloat16_rn(__uint_as_float(acc[j]));
@@ -1490,7 +1484,7 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* a, int* n_partials_out
                                     : ((long long)(a->N - 1) * a->ldy + a->M)) * ysz : 0;
     const bool al32 = a->ldy * ysz % 32 == 0 && (reinterpret_cast<uintptr_t>(a->Yout) & 31) == 0;
     const bool al16 = a->ldy * ysz % 16 == 0 && (reinterpret_cast<uintptr_t>(a->Yout) & 15) == 0;
-    kp.y_store = al32 ? (a->yref_t ? 3 : 2) : (al16 ? 1 : 0);
+    kp.y_store = al32 ? 2 : (al16 ? 1 : 0);
     kp.ext_dyt = a->dYt ? ((long long)(a->M - 1) * a->ld_dyt + a->N) * 2 : 0;
     kp.ext_state = (long long)a->M * a->N * 4;
     kp.ext_wsoft = (long long)a->M * a->N * 2;

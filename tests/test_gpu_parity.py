@@ -1114,6 +1114,27 @@ def test_plain_product_rows_of_any_alignment(ctx, O, ldy, offset, yref_dtype):
     assert torch.all(Y[:, O:] == 7.0) and torch.all(buf[:offset] == 7.0)
 
 
+@pytest.mark.parametrize("yref_dtype", [faar.BF16, faar.F32])
+@pytest.mark.parametrize("T,ldy,offset", [(20, 32, 0), (20, 40, 0), (16, 24, 0), (203, 216, 0), (20, 32, 8), (9, 16, 8)])
+def test_padding_of_a_transposed_target_is_written_as_zeros(ctx, T, ldy, offset, yref_dtype):
+    """Rows that start on 32 and on 16 bytes: the values, then zeros up to the next multiple of 16 columns, then nothing."""
+    O, K = 130, 64
+    gen = torch.Generator(device=DEV).manual_seed(T)
+    W, X = (torch.randn(n, K, device=DEV, generator=gen).to(torch.bfloat16) for n in (O, T))
+    dt = torch.bfloat16 if yref_dtype == faar.BF16 else torch.float32
+    off = offset if yref_dtype == faar.BF16 else offset // 2                # 16 bytes
+    Y = torch.full((off + O * ldy,), 7.0, dtype=dt, device=DEV)[off:].view(O, ldy)
+    shape = faar.make_shape(O, K, T, ldy=ldy, yref_dtype=yref_dtype, yref_transposed=1)
+    ws = torch.empty(faar.workspace_size(shape), dtype=torch.uint8, device=DEV)
+    faar.workspace_init(ctx, ws)
+    faar.layer_ref(ctx, shape, X, W, Y, ws)
+    faar.check_status(ctx, ws)
+    plain = torch.empty((T, O), dtype=dt, device=DEV)
+    faar.layer_ref(ctx, faar.make_shape(O, K, T, yref_dtype=yref_dtype), X, W, plain, ws)
+    T16 = (T + 15) // 16 * 16
+    assert torch.equal(Y[:, :T], plain.t()) and torch.all(Y[:, T:T16] == 0.0) and torch.all(Y[:, T16:] == 7.0)
+
+
 def test_the_native_marshalling_refuses_what_it_cannot_pass_on(ctx):
     x = torch.zeros((4, 16), dtype=torch.bfloat16, device=DEV)
     with pytest.raises(AssertionError):
