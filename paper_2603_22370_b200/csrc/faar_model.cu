@@ -5,6 +5,8 @@
 // they cost 7.5 us of host time each, more than the kernels of a small model take: an alignment step of two 128-wide blocks
 // on 192 tokens took 770 us for 500 us of device time.  Activations live in one caller-owned arena per pass at
 // offsets that depend on the sizes alone.
+#include <math.h>
+
 #include "faar_internal.cuh"
 
 namespace {
@@ -142,6 +144,14 @@ constexpr size_t OVERLAP_LIMIT = 28 << 20;     // see faar_model_overlap
 
 bool aligned(const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// The checks of the single entry points (faar_embedding, faar_rmsnorm, faar_rope, faar_layer_ref, faar_layer_bwd_rowmajor
+// and so on) for everything that a pass hands to their kernels.
+bool sizes_ok(const faar_model* m) {
+  if (m->n_layers <= 0 || m->hidden <= 0 || m->ffn <= 0 || m->n_heads <= 0 || m->n_kv_heads <= 0 || m->head_dim <= 0) return false;
+  // widths are held as int, and the dW epilogue counts up to 7 rows of V in 32 bits
+  const long long q = (long long)m->n_heads * m->head_dim, kv = (long long)m->n_kv_heads * m->head_dim;
+  return q + 2 * kv <= 0x7FFFFFFFll && 8 * q <= 0x7FFFFFFFll && 8ll * m->ffn <= 0x7FFFFFFFll && 8ll * m->hidden <= 0x7FFFFFFFll;
+}
 int check_group(const faar_linear_group& g, int n, const int* rows, bool quantised, const faar_hparams* hp) {
   if (g.n != n) return FAAR_ERR_INVALID_ARG;
   if (quantised ? !aligned(g.Wsoft) : !aligned(g.W)) return g.W || g.Wsoft ? FAAR_ERR_ALIGN : FAAR_ERR_INVALID_ARG;
@@ -160,10 +170,12 @@ int check_group(const faar_linear_group& g, int n, const int* rows, bool quantis
 int check_model(const faar_ctx* ctx, const faar_model* m, int batch, int seq, bool quantised, const faar_hparams* hp, const void* ws,
                 size_t ws_bytes) {
   if (!ctx || !m || !m->blocks || !m->embed || !m->lm_head || !m->final_norm) return FAAR_ERR_INVALID_ARG;
-  if (batch <= 0 || seq <= 0 || (long long)batch * seq > 0x7FFFFFFFll || m->n_layers <= 0 || m->n_heads <= 0 || m->n_kv_heads <= 0 ||
-      m->n_heads % m->n_kv_heads || (m->head_dim != 64 && m->head_dim != 128))
+  if (!(m->eps >= 0.f) || !isfinite(m->eps) || !(m->theta > 1.f) || !isfinite(m->theta)) return FAAR_ERR_INVALID_ARG;
+  if (batch <= 0 || seq <= 0 || (long long)batch * seq > 0x7FFFFFFFll || !sizes_ok(m) || m->n_heads % m->n_kv_heads ||
+      (m->head_dim != 64 && m->head_dim != 128))
     return FAAR_ERR_SHAPE;
-  if (m->vocab <= 0 || m->vocab % 16 || m->hidden <= 0 || m->hidden % 16 || m->ffn <= 0 || m->ffn % 16) return FAAR_ERR_SHAPE;
+  if (m->vocab <= 0 || m->vocab % 16 || m->hidden % 16 || m->ffn % 16) return FAAR_ERR_SHAPE;
+  if (!aligned(m->embed) || !aligned(m->lm_head) || !aligned(m->final_norm)) return FAAR_ERR_ALIGN;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < FAAR_WS_HEADER + 2 * sizeof(float) * FAAR_MAX_PARTIALS)
     return FAAR_ERR_WORKSPACE;
   const int qd = m->n_heads * m->head_dim, kvd = m->n_kv_heads * m->head_dim;
@@ -171,6 +183,7 @@ int check_model(const faar_ctx* ctx, const faar_model* m, int batch, int seq, bo
   for (int l = 0; l < m->n_layers; ++l) {
     const faar_block& b = m->blocks[l];
     if (!b.attn_norm || !b.mlp_norm) return FAAR_ERR_INVALID_ARG;
+    if (!aligned(b.attn_norm) || !aligned(b.mlp_norm)) return FAAR_ERR_ALIGN;
     int st = check_group(b.qkv, 3, qkv, quantised, hp);
     if (!st) st = check_group(b.o, 1, one, quantised, hp);
     if (!st) st = check_group(b.gate_up, 2, gu, quantised, hp);
@@ -317,8 +330,7 @@ extern "C" {
 
 int faar_model_sizes(const faar_model* m, int batch, int seq, int keep, size_t* arena_bytes, size_t* scratch_bytes) {
   if (!m || !arena_bytes || !scratch_bytes) return FAAR_ERR_INVALID_ARG;
-  if (batch <= 0 || seq <= 0 || m->n_layers <= 0 || m->hidden <= 0 || m->ffn <= 0 || m->n_heads <= 0 || m->n_kv_heads <= 0 || m->head_dim <= 0)
-    return FAAR_ERR_SHAPE;
+  if (batch <= 0 || seq <= 0 || !sizes_ok(m)) return FAAR_ERR_SHAPE;
   const Sizes s = sizes(m, batch, seq);
   *arena_bytes = Arena(s, m->n_layers, keep != 0).total;
   *scratch_bytes = Scratch(s).total;
@@ -331,7 +343,7 @@ int faar_model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, c
   int st = check_model(ctx, m, batch, seq, quantised != 0, nullptr, workspace, workspace_bytes);
   if (st) return st;
   if (!tokens || !positions || !arena || !Z || !H) return FAAR_ERR_INVALID_ARG;
-  if (quantised && !(beta > 0.f)) return FAAR_ERR_INVALID_ARG;
+  if (quantised && (!(beta > 0.f) || !isfinite(beta))) return FAAR_ERR_INVALID_ARG;
   if (!aligned(Z) || !aligned(H) || (reinterpret_cast<uintptr_t>(arena) & 255u)) return FAAR_ERR_ALIGN;
   size_t need = 0, scratch = 0;
   if ((st = faar_model_sizes(m, batch, seq, keep, &need, &scratch))) return st;
@@ -348,7 +360,7 @@ int faar_model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, c
 // fills the GPU (and both arenas at once are gigabytes).
 int faar_model_overlap(const faar_model* m, int batch, int seq, int* overlap) {
   if (!m || !overlap) return FAAR_ERR_INVALID_ARG;
-  if (batch <= 0 || seq <= 0) return FAAR_ERR_SHAPE;
+  if (batch <= 0 || seq <= 0 || !sizes_ok(m)) return FAAR_ERR_SHAPE;
   const Sizes s = sizes(m, batch, seq);
   const size_t widest = s.qkv > 2 * s.f ? s.qkv : 2 * s.f;
   *overlap = s.T * widest <= OVERLAP_LIMIT;
@@ -361,7 +373,7 @@ int faar_model_forward_both(faar_ctx* ctx, const faar_model* m, int batch, int s
   int st = check_model(ctx, m, batch, seq, false, nullptr, workspace, workspace_bytes);
   if (!st) st = check_model(ctx, m, batch, seq, true, nullptr, workspace, workspace_bytes);
   if (st) return st;
-  if (!tokens || !positions || !arena_fp || !Z_fp || !H_fp || !arena || !Z || !H || !(beta > 0.f)) return FAAR_ERR_INVALID_ARG;
+  if (!tokens || !positions || !arena_fp || !Z_fp || !H_fp || !arena || !Z || !H || !(beta > 0.f) || !isfinite(beta)) return FAAR_ERR_INVALID_ARG;
   if (!aligned(Z_fp) || !aligned(H_fp) || !aligned(Z) || !aligned(H) || (reinterpret_cast<uintptr_t>(arena) & 255u) ||
       (reinterpret_cast<uintptr_t>(arena_fp) & 255u))
     return FAAR_ERR_ALIGN;
@@ -384,7 +396,7 @@ int faar_model_backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, 
   if (st) return st;
   if (!positions || !arena || !dZ || !dH || !scratch || !m->lm_head_t) return FAAR_ERR_INVALID_ARG;
   if (ldz < m->vocab || m->ld_lm_head_t < m->vocab) return FAAR_ERR_SHAPE;
-  if (!aligned(dZ) || !aligned(dH) || ldz % 8 || m->ld_lm_head_t % 8 || (reinterpret_cast<uintptr_t>(arena) & 255u) ||
+  if (!aligned(dZ) || !aligned(dH) || !aligned(m->lm_head_t) || ldz % 8 || m->ld_lm_head_t % 8 || (reinterpret_cast<uintptr_t>(arena) & 255u) ||
       (reinterpret_cast<uintptr_t>(scratch) & 255u))
     return FAAR_ERR_ALIGN;
   size_t need = 0, need_s = 0;

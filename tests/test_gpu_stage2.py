@@ -196,3 +196,71 @@ def test_stage2_step_with_a_split_lm_head_gradient_matches_the_oracle(ctx, monke
     build = small_model
     monkeypatch.setitem(globals(), "small_model", lambda seed=0: build(seed, vocab=1600))
     test_stage2_step_matches_the_oracle(ctx)
+
+
+def test_the_passes_of_a_model_refuse_what_their_kernels_cannot_take(ctx):
+    """Every refusal comes from a comparison on the host: nothing is launched."""
+    cfg, _, params, W_fp, _, tokens = small_model(2)
+    B, S = tokens.shape
+    dparams = {k: (dev_bf16(v) if k in ("embed", "lm_head") else dev_f32(v)) for k, v in params.items()}
+    dweights = [{n: dev_bf16(W_fp[l][n]) for n in so.LINEARS} for l in range(cfg["n_layers"])]
+    model = stage2.Stage2Model(ctx, stage2.ModelConfig(**cfg), dparams, dweights, B, S)
+    T, tok = B * S, torch.from_numpy(tokens.reshape(-1).astype(np.int32)).to(DEV)
+    arenas = {k: torch.empty(n, dtype=torch.uint8, device=DEV) for k, n in model.arena_bytes.items()}
+    scratch = torch.empty(model.scratch_bytes, dtype=torch.uint8, device=DEV)
+    Z, dZ = (torch.zeros((T, cfg["vocab"]), dtype=torch.bfloat16, device=DEV) for _ in range(2))
+    H, dH = (torch.zeros((T, cfg["hidden"]), dtype=torch.bfloat16, device=DEV) for _ in range(2))
+    hp = faar.make_hparams(beta=4.0, step=1)
+
+    def refused(status, calls="fqbp", block=None, beta=4.0, shape=(B, S), arena=None, **fields):
+        m = faar.Model.from_buffer_copy(model._table())
+        blocks = (faar.Block * cfg["n_layers"]).from_buffer_copy(model._blocks)
+        for k, v in fields.items():
+            setattr(m, k, v(getattr(m, k)) if callable(v) else v)
+        if block:
+            block(blocks[1])
+        m.blocks = stage2.ctypes.addressof(blocks)
+        big, small = arena if arena is not None else (arenas[True], arenas[False])
+        run = {"f": lambda: faar.model_forward(ctx, m, *shape, tok, model.pos, 0, beta, 0, small, Z, H, model.ws),
+               "q": lambda: faar.model_forward(ctx, m, *shape, tok, model.pos, 1, beta, 1, big, Z, H, model.ws),
+               "p": lambda: faar.model_forward_both(ctx, m, *shape, tok, model.pos, beta, small, Z, H, big, Z, H, model.ws),
+               "b": lambda: faar.model_backward(ctx, m, *shape, model.pos, hp, big, dZ, cfg["vocab"], dH, scratch, model.ws),
+               "s": lambda: faar.model_sizes(m, *shape, 1), "o": lambda: faar.model_overlap(m, *shape)}
+        for c in calls:
+            with pytest.raises(faar.FaarError) as e:
+                run[c]()
+            assert e.value.status == status, (c, fields, e.value.status)
+
+    off = lambda n: lambda p: p + n
+    for name, n in (("embed", 2), ("lm_head", 8), ("final_norm", 4)):
+        refused(faar.ERR_ALIGN, **{name: off(n)})
+        refused(faar.ERR_INVALID_ARG, **{name: None})
+    refused(faar.ERR_ALIGN, "b", lm_head_t=off(2))
+    refused(faar.ERR_INVALID_ARG, "b", lm_head_t=None)
+    for eps in (-1e-5, float("nan"), float("inf")):
+        refused(faar.ERR_INVALID_ARG, eps=eps)
+    for theta in (1.0, 0.5, float("nan"), float("inf")):
+        refused(faar.ERR_INVALID_ARG, theta=theta)
+    for beta in (0.0, float("nan"), float("inf")):
+        refused(faar.ERR_INVALID_ARG, "qp", beta=beta)
+    for field in ("attn_norm", "mlp_norm"):
+        refused(faar.ERR_ALIGN, block=lambda b: setattr(b, field, getattr(b, field) + 4))
+        refused(faar.ERR_INVALID_ARG, block=lambda b: setattr(b, field, None))
+    refused(faar.ERR_ALIGN, "f", block=lambda b: setattr(b.o, "W", b.o.W + 2))
+    refused(faar.ERR_ALIGN, "qbp", block=lambda b: setattr(b.o, "Wsoft", b.o.Wsoft + 2))
+    refused(faar.ERR_ALIGN, "qbp", block=lambda b: setattr(b.qkv.lin[2], "V", b.qkv.lin[2].V + 4))
+    refused(faar.ERR_ALIGN, "qbp", block=lambda b: setattr(b.down.lin[0], "code", b.down.lin[0].code + 1))
+    refused(faar.ERR_INVALID_ARG, "qbp", block=lambda b: setattr(b.down.lin[0], "scales", None))
+    refused(faar.ERR_INVALID_ARG, "b", block=lambda b: setattr(b.gate_up.lin[1], "adam_u", None))
+    refused(faar.ERR_INVALID_ARG, block=lambda b: setattr(b.gate_up, "n", 1))
+    refused(faar.ERR_SHAPE, block=lambda b: setattr(b.gate_up.lin[0], "rows", 240))
+    refused(faar.ERR_SHAPE, "fqbpso", shape=(0, S))
+    refused(faar.ERR_SHAPE, shape=(65536, 65536))
+    refused(faar.ERR_SHAPE, "fqbpso", n_heads=1 << 25)
+    refused(faar.ERR_SHAPE, "fqbpso", hidden=1 << 29)
+    refused(faar.ERR_SHAPE, head_dim=32)
+    refused(faar.ERR_SHAPE, vocab=cfg["vocab"] + 8)
+    refused(faar.ERR_WORKSPACE, arena=(arenas[True][:-256], arenas[False][:-256]))
+    refused(faar.ERR_ALIGN, arena=(arenas[True][16:], arenas[False][16:]))
+    torch.cuda.synchronize()
+    faar.check_status(ctx, model.ws)
