@@ -178,19 +178,26 @@ class Stage2Model:
     def _backward(self, model: faar.Model, dZ, dH, saved, hp, want_dv):
         grads = {}
         if want_dv:
-            for l in range(self.cfg.n_layers):
-                for field, names, _, _ in self._groups(l):
-                    for i, n in enumerate(names):
-                        x = self.lin[l][n]
-                        grads[(l, n)] = torch.empty((x.O, x.K), dtype=torch.float32, device=self.dev)
-                        getattr(self._blocks[l], field).lin[i].dV = grads[(l, n)].data_ptr()
+            grads = {(l, n): torch.empty((x.O, x.K), dtype=torch.float32, device=self.dev)
+                     for l, lins in enumerate(self.lin) for n, x in lins.items()}
         scratch = torch.empty(self.scratch_bytes, dtype=torch.uint8, device=self.dev)
+        if not want_dv:
+            faar.model_backward(self.ctx, model, self.batch, self.seq, self.pos, hp, saved, dZ, dZ.shape[1], dH, scratch, self.ws)
+            return None
+        # the gradients' addresses are in the structure for this call alone
+        self._set_dv(grads)
         try:
             faar.model_backward(self.ctx, model, self.batch, self.seq, self.pos, hp, saved, dZ, dZ.shape[1], dH, scratch, self.ws)
         finally:
-            if want_dv:
-                self._addresses = None               # the structure holds the gradients' addresses: build it anew
-        return grads if want_dv else None
+            self._set_dv({})
+        return grads
+
+    def _set_dv(self, grads):
+        for l in range(self.cfg.n_layers):
+            for field, names, _, _ in self._groups(l):
+                for i, n in enumerate(names):
+                    g = grads.get((l, n))
+                    getattr(self._blocks[l], field).lin[i].dV = None if g is None else g.data_ptr()
 
     # ---- one step of Eq. 6 -----------------------------------------------------------------------------
     def step(self, tokens: torch.Tensor, beta: float, tau: float = 1.0, lambda_kl: float = 1.0, lambda_round: float = 1.0,

@@ -198,6 +198,39 @@ def test_stage2_step_with_a_split_lm_head_gradient_matches_the_oracle(ctx, monke
     test_stage2_step_matches_the_oracle(ctx)
 
 
+def test_gradients_of_a_step_that_failed_are_not_written_later(ctx, monkeypatch):
+    """A step that wanted dV and ran out of memory between its allocations leaves no address of a freed gradient behind."""
+    cfg, _, params, W_fp, _, tokens = small_model(1)
+    B, S = tokens.shape
+    dparams = {k: (dev_bf16(v) if k in ("embed", "lm_head") else dev_f32(v)) for k, v in params.items()}
+    dweights = [{n: dev_bf16(W_fp[l][n]) for n in so.LINEARS} for l in range(cfg["n_layers"])]
+    model = stage2.Stage2Model(ctx, stage2.ModelConfig(**cfg), dparams, dweights, B, S)
+    tok = torch.from_numpy(tokens.reshape(-1).astype(np.int32)).to(DEV)
+    held = lambda: [getattr(b, g).lin[i].dV for b in model._blocks for g in ("qkv", "o", "gate_up", "down") for i in range(3)]
+    assert len(model.step(tok, beta=4.0, want_dv=True)["dV"]) == 7 * cfg["n_layers"] and not any(held())
+    real, left = torch.empty, [0]
+
+    def empty(size, *a, **kw):
+        if kw.get("dtype") == torch.float32 and len(size) == 2:              # a gradient
+            left[0] -= 1
+            if left[0] < 0:
+                raise torch.cuda.OutOfMemoryError("no room")
+        return real(size, *a, **kw)
+
+    for n in (0, 5):
+        left[0] = n
+        with monkeypatch.context() as m:
+            m.setattr(stage2.torch, "empty", empty)
+            with pytest.raises(torch.cuda.OutOfMemoryError):
+                model.step(tok, beta=4.0, want_dv=True)
+        assert not any(held())
+    with pytest.raises(faar.FaarError):                                      # refused by the call itself
+        model.backward(torch.zeros((B * S, 8), dtype=torch.bfloat16, device=DEV), model.pos, real(256, dtype=torch.uint8, device=DEV),
+                       faar.make_hparams(beta=4.0, step=1), want_dv=True)
+    assert not any(held())
+    torch.cuda.synchronize()
+
+
 def test_the_passes_of_a_model_refuse_what_their_kernels_cannot_take(ctx):
     """Every refusal comes from a comparison on the host: nothing is launched."""
     cfg, _, params, W_fp, _, tokens = small_model(2)
