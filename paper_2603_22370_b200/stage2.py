@@ -105,7 +105,7 @@ class Stage2Model:
         faar.workspace_init(ctx, self.aws)
         self.loss = torch.zeros(2, dtype=torch.float32, device=dev)
         self.step_count = 0
-        self._addresses, self._model, self._blocks = None, None, None
+        self._held, self._model, self._blocks = None, None, None
         table = self._table()
         self.arena_bytes = {bool(k): faar.model_sizes(table, batch, seq, k)[0] for k in (0, 1)}
         self.scratch_bytes = faar.model_sizes(table, batch, seq, 1)[1]
@@ -123,19 +123,20 @@ class Stage2Model:
                 ("down", ("down_proj",), lin["down_proj"].W, lin["down_proj"].Wsoft))
 
     def _table(self) -> faar.Model:
-        """The model as the library takes it: addresses of the tensors that the attributes hold now, read on every call
-        (the structure is only rebuilt if one of them has moved)."""
-        p = self.params
+        """The model as the library takes it: the configuration's values and the addresses of the tensors that the attributes
+        hold now, read on every call (the structure is only rebuilt if one of them has changed)."""
+        p, c = self.params, self.cfg
         held = [p["embed"], p["lm_head"], p["final_norm"], self.lm_head_t]
         for l, lins in enumerate(self.lin):
             held += (p[f"attn_norm.{l}"], p[f"mlp_norm.{l}"], *self.w_group[l].values(), *self.wsoft_group[l].values())
             for x in lins.values():
                 held += (x.W, x.Wsoft, x.V, x.code, x.scales, x.s_global, x.m, x.u)
-        addresses = [0 if t is None else t.data_ptr() for t in held]
-        if addresses == self._addresses:
+        now = [c.vocab, c.hidden, c.n_layers, c.n_heads, c.n_kv_heads, c.head_dim, c.ffn, c.eps, c.theta]
+        now += [0 if t is None else t.data_ptr() for t in held]
+        if now == self._held:
             return self._model
         assert all(t is None or t.is_cuda for t in held), "device tensors only"
-        c, ptr = self.cfg, lambda t: None if t is None else t.data_ptr()
+        ptr = lambda t: None if t is None else t.data_ptr()
         blocks = (faar.Block * c.n_layers)()
         for l in range(c.n_layers):
             for field, names, W, Wsoft in self._groups(l):
@@ -145,7 +146,7 @@ class Stage2Model:
                     x = self.lin[l][n]
                     g.lin[i] = faar.Linear(x.O, ptr(x.V), ptr(x.code), ptr(x.scales), ptr(x.s_global), ptr(x.m), ptr(x.u), None)
             blocks[l].attn_norm, blocks[l].mlp_norm = ptr(p[f"attn_norm.{l}"]), ptr(p[f"mlp_norm.{l}"])
-        self._blocks, self._addresses = blocks, addresses
+        self._blocks, self._held = blocks, now
         self._model = faar.Model(c.vocab, c.hidden, c.n_layers, c.n_heads, c.n_kv_heads, c.head_dim, c.ffn, c.eps, c.theta,
                                  ptr(p["embed"]), ptr(p["lm_head"]), ptr(self.lm_head_t), self.lm_head_t.shape[1],
                                  ptr(p["final_norm"]), ctypes.addressof(blocks))

@@ -198,6 +198,20 @@ def test_stage2_step_with_a_split_lm_head_gradient_matches_the_oracle(ctx, monke
     test_stage2_step_matches_the_oracle(ctx)
 
 
+def test_a_changed_configuration_counts_from_the_next_pass_on(ctx):
+    cfg, _, params, W_fp, _, tokens = small_model(1)
+    B, S = tokens.shape
+    dparams = {k: (dev_bf16(v) if k in ("embed", "lm_head") else dev_f32(v)) for k, v in params.items()}
+    dweights = [{n: dev_bf16(W_fp[l][n]) for n in so.LINEARS} for l in range(cfg["n_layers"])]
+    tok = torch.from_numpy(tokens.reshape(-1).astype(np.int32)).to(DEV)
+    new = lambda **kw: stage2.Stage2Model(ctx, stage2.ModelConfig(**cfg, **kw), dparams, dweights, B, S)
+    model, want = new(), new(eps=0.5, theta=100.0)
+    before = model.forward(tok, quantised=True)[0]
+    model.cfg.eps, model.cfg.theta = 0.5, 100.0
+    after = model.forward(tok, quantised=True)[0]
+    assert torch.equal(after, want.forward(tok, quantised=True)[0]) and not torch.equal(after, before)
+
+
 def test_gradients_of_a_step_that_failed_are_not_written_later(ctx, monkeypatch):
     """A step that wanted dV and ran out of memory between its allocations leaves no address of a freed gradient behind."""
     cfg, _, params, W_fp, _, tokens = small_model(1)
