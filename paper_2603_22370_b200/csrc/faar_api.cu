@@ -238,16 +238,17 @@ int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes) {
 
 int faar_max_clusters(faar_ctx* c, int slot, int size, const void* kernel, cudaLaunchConfig_t* cfg) {
   constexpr int DEVICES = 64;
-  static std::atomic<int> known[DEVICES][FAAR_PAIR_KERNELS][FAAR_CLUSTER_SIZES];       // 0 = not asked yet
+  static std::atomic<int> known[DEVICES][FAAR_PAIR_KERNELS][FAAR_CLUSTER_SIZES];       // number + 1; 0 = not asked yet
   const bool keep = c->device < DEVICES;
-  int n = keep ? known[c->device][slot][size].load(std::memory_order_relaxed) : 0;
-  if (n) return n;
+  int n = keep ? known[c->device][slot][size].load(std::memory_order_relaxed) - 1 : -1;
+  if (n >= 0) return n;
   const int ctas = 2 << size, most = c->num_sms / ctas;
   cfg->gridDim = dim3(ctas * most, 1, 1);
+  n = 0;
   const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kernel, cfg);
-  if (e != cudaSuccess || n <= 0) { (void)cudaGetLastError(); n = size ? 1 : most; }
-  if (n > most) n = most;
-  if (keep) known[c->device][slot][size].store(n, std::memory_order_relaxed);
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  n = faar_cluster_count(e == cudaSuccess, n, size, most);
+  if (keep) known[c->device][slot][size].store(n + 1, std::memory_order_relaxed);
   return n;
 }
 

@@ -62,6 +62,12 @@ int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes);
 // holds at once: a fact of device and kernel (a GPC with an odd SM count strands one SM), asked once per device and process.
 constexpr int FAAR_CLUSTER_SIZES = 3;     // 2, 4, 8 CTAs
 int faar_max_clusters(faar_ctx* c, int slot, int size, const void* kernel, cudaLaunchConfig_t* cfg);
+// The number from the query's answer; `most` is what the SM count allows.  Without an answer every SM is counted for pairs,
+// which every launch needs, and no larger cluster: a contraction is then not split over one that the device may refuse.
+inline int faar_cluster_count(bool answered, int n, int size, int most) {
+  if (!answered || n <= 0) return size ? 0 : most;
+  return n < most ? n : most;
+}
 
 // Launch with stream serialisation relaxed (programmatic dependent launch): the kernel's CTAs may be scheduled while the
 // kernel before it drains; the kernel itself waits (faar_pdl_sync) before it touches global memory.

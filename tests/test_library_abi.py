@@ -3,6 +3,7 @@ entry point that include/faar.h declares.  No compute call is made here."""
 import ctypes as C
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -88,3 +89,22 @@ def test_debug_build_exports_the_same_symbols():
     dbg = C.CDLL(path)
     for n in declared_symbols():
         assert hasattr(dbg, n), n
+
+
+def test_no_cluster_is_assumed_that_the_device_did_not_confirm(tmp_path):
+    """Without an answer to the occupancy query a launch counts on pairs of CTAs, which it needs, and on no larger cluster."""
+    src = tmp_path / "clusters.cu"
+    src.write_text('#include <cstdio>\n#include "faar_internal.cuh"\n'
+                   "int main() {\n  for (int size = 0; size < FAAR_CLUSTER_SIZES; ++size)\n"
+                   '    for (int n : {-1, 0, 5, 200}) printf("%d %d ", faar_cluster_count(false, n, size, 74 >> size), '
+                   "faar_cluster_count(true, n, size, 74 >> size));\n}\n")
+    exe = str(tmp_path / "clusters")
+    subprocess.run([faar_build._nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-I", os.path.join(ROOT, "include"),
+                    "-I", faar_build.CSRC, str(src), "-o", exe], check=True, capture_output=True)
+    got = [int(x) for x in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()]
+    want = []
+    for size in range(3):
+        most = 74 >> size
+        fallback = 0 if size else most
+        want += [fallback, fallback, fallback, fallback, fallback, min(5, most), fallback, most]
+    assert got == want
