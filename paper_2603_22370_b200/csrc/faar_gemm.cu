@@ -794,6 +794,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   volatile int* abort_flag = reinterpret_cast<volatile int*>(ctl + 8 * (2 * MAX_STAGES + 4) + 4);
   double* fin_mse = reinterpret_cast<double*>(ctl + 320);            // BWD with final sums: L_MSE's sum
   float* fin_warp = reinterpret_cast<float*>(ctl + 328);             // and the epilogue warps' Round Loss sums
+  volatile int* fin_flags = reinterpret_cast<volatile int*>(ctl + 392);   // 0: a warp's sum is out of range; 1: no final sums
   const AbortCtl ac{abort_flag, p.status};
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -820,6 +821,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     if (SPLIT) { mbar_init(bar_recv, 1); mbar_expect_tx(bar_recv, (uint32_t)((splits - 1) * (share_begin(BN, splits, split + 1) - share_begin(BN, splits, split)) * BM * 4)); }
     for (int q = 0; q < 8; ++q) mbar_init(ctl_u32 + 256u + 8u * q, 4);   // panel staged / panel consumed, per lane quarter
     *abort_flag = 0;
+    if (MODE == FAAR_GEMM_BWD) fin_flags[0] = fin_flags[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -886,6 +888,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       // the forward's share of the loss values, under the epilogue: strided double accumulation, then a tree over lanes
       if (p.fin_out2 != nullptr) {
         __syncwarp();
+        if (lane == 0 && __ldcg(p.status) != 0u) fin_flags[1] = 1;
         double mse = 0.0;
 #pragma unroll 8
         for (int i = lane; i < p.fin_n_mse; i += 32) mse += (double)__ldcg(p.fin_mse_partials + i);
@@ -956,7 +959,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const bool yvec_ok = MODE == FAAR_GEMM_FWD && p.yref_t && p.yref_dtype == FAAR_BF16 && p.Yout == nullptr;
     bool dead = false;
     // One pass per accumulator buffer that fills: a tile, or (WIDE) a 256-column half of a tile.
-    for (int vt = 0;; ++vt) {
+    int vt = 0;
+    for (;; ++vt) {
       const int it = WIDE ? vt >> 1 : vt;
       const int tile = pair + it * n_pairs;
       if (tile >= total_tiles) break;
@@ -1111,7 +1115,12 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       warp_acc = faar_warp_sum(warp_acc);
       if (lane == 0) {
         if (MODE == FAAR_GEMM_FWD) p.partials[blockIdx.x * C::EPI_WARPS + ew] = warp_acc;
-        else fin_warp[ew] = warp_acc;
+        else {
+          fin_warp[ew] = warp_acc;
+          // one per weight that the warp may have had
+          const int columns = SPLIT ? share_begin(BN, splits, split + 1) - share_begin(BN, splits, split) : BN;
+          if (!(fabsf(warp_acc) <= (float)(vt * (BM * columns / C::EPI_WARPS)))) fin_flags[0] = 1;
+        }
       }
     }
   }
@@ -1145,18 +1154,14 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // [0, 1] can give.  A sum beyond that (v outside, infinite or not a number) goes to the CTA's slot in memory with a bit
     // that says so; the last CTA adds those in the order of the CTAs.  After a wait that gave up this CTA's sums are
     // incomplete: it does not count, so nobody forms final sums (the caller re-initialises the workspace, which also clears
-    // the word and the bits).
-    if (p.fin_out2 != nullptr && threadIdx.x == 0 && !*abort_flag) {
+    // the word and the bits).  Nor does anybody if an earlier launch's status is set: the forward's sums may be incomplete.
+    if (p.fin_out2 != nullptr && threadIdx.x == 0 && !*abort_flag && !fin_flags[1]) {
       double rnd = 0.0;
 #pragma unroll
       for (int w = 0; w < C::EPI_WARPS; ++w) rnd += (double)fin_warp[w];
       constexpr uint32_t COUNT = (1u << FIN_COUNT_BITS) - 1u;
-      const int columns = SPLIT ? share_begin(BN, splits, split + 1) - share_begin(BN, splits, split) : (WIDE ? WIDE_BN : BN);
-      const double room = (double)((total_tiles - pair + n_pairs - 1) / n_pairs) * (double)(BM * columns);
-      unsigned long long mine;
-      if (fabs(rnd) <= room) {
-        mine = ((unsigned long long)__double2ll_rn(rnd * p.fin_unit) << (2 * FIN_COUNT_BITS)) + 1ull;
-      } else {
+      unsigned long long mine = ((unsigned long long)__double2ll_rn(rnd * p.fin_unit) << (2 * FIN_COUNT_BITS)) + 1ull;
+      if (fin_flags[0]) {
         p.fin_far_sums[blockIdx.x] = rnd;
         atomicOr(p.fin_far + (blockIdx.x >> 6), 1ull << (blockIdx.x & 63));
         __threadfence();

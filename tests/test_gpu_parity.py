@@ -908,6 +908,31 @@ def test_round_loss_of_a_step_for_any_v(ctx, O, K, T, opt):
                 assert np.isnan(got) if np.isnan(want) else got == want, (step, got, want)
 
 
+def test_no_losses_are_written_after_a_wait_that_ran_out(ctx):
+    """The status word of an earlier launch stands: the sums that the losses are formed from may be incomplete, so a step
+    leaves the caller's two values alone until the workspace has been initialised again."""
+    W, X, Yref = _problem(128, 256, 256)
+    lay = GpuLayer(ctx, W, X)
+    lay.init()
+    lay.set_yref(Yref)
+    hp, _ = f32hp()
+    lay.step(hp)
+    lay.check()
+    first = host(lay.loss).copy()
+    faar.selftest_wait_timeout(ctx, lay.ws, 1000)
+    lay.loss.fill_(123.0)
+    lay.step(hp)
+    with pytest.raises(faar.FaarError):
+        faar.check_status(ctx, lay.ws)
+    assert np.all(host(lay.loss) == 123.0)
+    faar.workspace_init(ctx, lay.ws)
+    lay.init()
+    lay.set_state(m=np.zeros(W.shape), u=np.zeros(W.shape))
+    lay.step(hp)
+    lay.check()
+    assert np.array_equal(host(lay.loss), first)
+
+
 def test_outputs_stay_inside_their_buffers(ctx):
     """Canaries around every buffer a step writes (dY^T, V, Adam moments, dV, losses) and around the packed
     output: a ragged shape, so that partial tiles, partial panels and partial vectors all occur."""
