@@ -22,7 +22,8 @@
 //   FWD : r = Y_q - Y_ref, sum r^2, dY = 2c r -> dY^T     (steps 9-10, Eq. 5 first term)
 //   BWD : G = dY^T X -> dV -> optimiser update + clip     (step 13, Eq. 5, with Eq. 2/3 chain rule)
 // In FWD and BWD the accumulator row (TMEM lane) is the output feature o.  In REF it is a row of the result as it lies in
-// memory (a token, or an output feature if the target is wanted transposed), so that a lane's 16 columns are contiguous.
+// memory (a token, or an output feature if the target is wanted transposed), so that a lane's 16 columns are contiguous, or
+// a column of it where rows are few or off 16 bytes (see result_columns).
 //
 // Every wait on an mbarrier is bounded: after about two seconds the waiting thread records a code in
 // the status word, raises a CTA-wide abort flag and every role leaves its loop; both CTAs then meet at
@@ -305,6 +306,7 @@ struct KParams {
   // REF / FWD
   void* Yout; int yout_dtype; long long ldy;
   const void* Yref; int yref_dtype;
+  int columns;            // REF: Yout is [N, ldy], the accumulator's rows are its columns (compiled in: COLUMNS)
   int yref_t;             // FWD: Y_ref / Y_q stored transposed, [O, ldy] with ldy >= T rounded up to 16; REF: rows of Yout are
                           // padded like that, columns beyond N up to the next multiple of 16 are written as 0
   int y_store;            // REF: rows of Yout take 2: 32-byte stores, 1: 16-byte stores, 0: single values
@@ -402,6 +404,22 @@ __device__ __forceinline__ void store_units(void* y, const uint32_t (&w)[8], boo
   if (wide) { stg256(y, w); return; }
   reinterpret_cast<uint4*>(y)[0] = make_uint4(w[0], w[1], w[2], w[3]);
   reinterpret_cast<uint4*>(y)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+}
+// The accumulator's rows as columns of Y: neighbouring lanes write neighbouring values, whatever the alignment of a row of Y.
+__device__ __forceinline__ void epi_ref_columns(const KParams& p, int col, int r0, const uint32_t (&acc)[16]) {
+  if (col >= p.M) return;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    if (r0 + j >= p.N) continue;
+    const long long off = (long long)(r0 + j) * p.ldy + col;
+    if (p.yout_dtype == FAAR_BF16) {
+      __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + off;
+      if (FAAR_DBG_OK(p, y, 2, p.Yout, p.ext_yout, 1u)) *y = __float2bfloat16_rn(__uint_as_float(acc[j]));
+    } else {
+      float* y = reinterpret_cast<float*>(p.Yout) + off;
+      if (FAAR_DBG_OK(p, y, 4, p.Yout, p.ext_yout, 1u)) *y = __uint_as_float(acc[j]);
+    }
+  }
 }
 __device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const uint32_t (&acc)[16]) {
   if (row >= p.M) return;
@@ -764,7 +782,8 @@ __device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t parts, int
 // ---- the kernel ------------------------------------------------------------------------------
 // Launched as clusters of 2 * splits CTAs along x; CTAs 2c and 2c+1 form a pair.
 // MN: bit 0 = the A operand, bit 1 = the B operand is stored with its M / N index contiguous (KParams.a_mn / b_mn);
-// a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.
+// a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.  Bit 2 (REF): the
+// accumulator's rows are the result's columns; compiled in as well (as a branch it cost 0.1 us in every small product).
 // SHAPE: 0 = tiles of up to 256 columns, WIDE_TILES, SPLIT_TILES; at compile time for the same reason.
 constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2;
 constexpr int MIN_SPLIT_BLOCKS = 12;            // contractions of fewer k blocks stay whole (see pick_splits)
@@ -774,7 +793,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                  const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ KParams p) {
   constexpr bool WIDE = SHAPE == WIDE_TILES, SPLIT = SHAPE == SPLIT_TILES;
   using C = Cfg<MODE, WIDE>;
-  constexpr bool A_MN = (MN & 1) != 0, B_MN = (MN & 2) != 0;
+  constexpr bool A_MN = (MN & 1) != 0, B_MN = (MN & 2) != 0, COLUMNS = (MN & 4) != 0;
   const int BN = p.bn;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -1095,8 +1114,13 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 add_parts(r, parts, splits, split, TW, c, quarter * 32 + lane);
                 if (second) add_parts(r2, parts, splits, split, TW, c + 16, quarter * 32 + lane);
               }
-              epi_ref(p, o, n0 + c, r);
-              if (second) epi_ref(p, o, n0 + c + 16, r2);
+              if (COLUMNS) {
+                epi_ref_columns(p, o, n0 + c, r);
+                if (second) epi_ref_columns(p, o, n0 + c + 16, r2);
+              } else {
+                epi_ref(p, o, n0 + c, r);
+                if (second) epi_ref(p, o, n0 + c + 16, r2);
+              }
             } else {
               float yr[16];
               yref_values(p, ynext, yr);
@@ -1455,9 +1479,15 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
                    a->yref_t && a->yref_dtype == FAAR_BF16 && !a->Yout);
   if (kp.splits > 1 && ctx->tune_bn == 0) bn = split_bn;
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
-  // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient), the dW
-  // product with B or with both untransposed
+  // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient; A, if the
+  // accumulator's rows are the result's columns), the dW product with B or with both untransposed
   if constexpr (MODE == FAAR_GEMM_REF) {
+    if (kp.columns && mn == 0) {
+      if (kp.splits == 1 && pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs))
+        return launch_variant<MODE, OPT, WIDE_TILES, 4>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+      return launch_tiles<MODE, OPT, 4>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+    }
+    if (kp.columns && mn == 1) return launch_tiles<MODE, OPT, 5>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
     if (mn == 2) return launch_tiles<MODE, OPT, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   } else if constexpr (MODE == FAAR_GEMM_BWD) {
     if (mn == 2) return launch_tiles<MODE, OPT, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
@@ -1471,6 +1501,17 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
 
 }  // namespace
 
+// Which index of a plain product Y[M, N] lies on the accumulator's rows.  N (Y's columns) where Y's rows are not 16-byte
+// aligned, because neighbouring lanes then write neighbouring values instead of one lane a row of single ones: [1000, 5000]
+// over 2048 with 5003 values a row 106 -> 28 us.  And N up to 128 rows of Y, which is half a tile: the tile's other half
+// would be padding that is staged all the same.  M on the accumulator's rows -> N, us: 1 row of 8192 over 2048 15.1 -> 10.6,
+// 64 rows 12.8 -> 12.0, 128 rows 13.1 -> 12.2, 160 rows 13.1 -> 13.8; input gradient of 8 rows of 8192 over 2048 14.5 -> 11.9.
+static bool result_columns(const faar_gemm_args* a) {
+  if (a->yref_t) return false;
+  const long long row = a->ldy * (a->yout_dtype == FAAR_BF16 ? 2 : 4);
+  return a->M <= BM || row % 16 != 0 || (reinterpret_cast<uintptr_t>(a->Yout) & 15) != 0;
+}
+
 int faar_launch_wait_selftest(faar_ctx* ctx, uint32_t* status, unsigned long long limit_ns) {
   wait_selftest_kernel<<<1, 64, 0, ctx->stream>>>(status, limit_ns);
   return (int)cudaGetLastError();
@@ -1478,13 +1519,23 @@ int faar_launch_wait_selftest(faar_ctx* ctx, uint32_t* status, unsigned long lon
 
 int faar_gemm_max_partials(const faar_ctx* ctx, int, int) { return ctx->num_sms * MAX_EPI_WARPS; }
 
-int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* a, int* n_partials_out) {
+int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_out) {
+  faar_gemm_args swapped;
+  const faar_gemm_args* a = args;
   KParams kp;
+  kp.columns = args->mode == FAAR_GEMM_REF && result_columns(args);
+  if (kp.columns) {
+    swapped = *args;
+    swapped.M = args->N; swapped.N = args->M;
+    swapped.A = args->B; swapped.lda = args->ldb; swapped.a_mn = args->b_mn;
+    swapped.B = args->A; swapped.ldb = args->lda; swapped.b_mn = args->a_mn;
+    a = &swapped;
+  }
   kp.M = a->M; kp.N = a->N; kp.Kc = a->Kc; kp.bn = BN_MAX; kp.n_main = kp.narrow = kp.n_full = 0; kp.status = a->status;
   {
     const long long ysz = a->yout_dtype == FAAR_BF16 ? 2 : 4;
     // the last row ends after its last valid (or padded) column; REF and the transposed FWD layout: [M, ldy], else [N(T), ldy]
-    const bool rows_m = a->mode == FAAR_GEMM_REF || a->yref_t;
+    const bool rows_m = (a->mode == FAAR_GEMM_REF && !kp.columns) || a->yref_t;
     kp.ext_yout = a->Yout ? (rows_m ? ((long long)(a->M - 1) * a->ldy + (a->yref_t ? (a->N + 15) / 16 * 16 : a->N))
                                     : ((long long)(a->N - 1) * a->ldy + a->M)) * ysz : 0;
     const bool al32 = a->ldy * ysz % 32 == 0 && (reinterpret_cast<uintptr_t>(a->Yout) & 31) == 0;

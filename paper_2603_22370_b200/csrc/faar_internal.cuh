@@ -204,7 +204,7 @@ enum { FAAR_GEMM_REF = 0, FAAR_GEMM_FWD = 1, FAAR_GEMM_BWD = 2 };
 
 struct faar_gemm_args {
   int mode;
-  int M, N, Kc;           // C[M,N] = A[M,Kc] * B[N,Kc]^T, both operands bf16 with Kc contiguous
+  int M, N, Kc;           // C[M,N] = A[M,Kc] * B[N,Kc]^T, both operands bf16 with Kc contiguous (REF: the launch may exchange them)
   const void* A; int64_t lda;
   const void* B; int64_t ldb;
   int whole;              // 1: the contraction is not split over CTA pairs (the order of its sums is that of one pair)

@@ -1140,6 +1140,48 @@ def test_plain_product_rows_of_any_alignment(ctx, O, ldy, offset, yref_dtype):
 
 
 @pytest.mark.parametrize("yref_dtype", [faar.BF16, faar.F32])
+@pytest.mark.parametrize("O,pad,offset", [(208, 0, 0), (200, 4, 0), (200, 0, 0), (201, 0, 0), (300, 4, 8), (77, 0, 1)])
+@pytest.mark.parametrize("T", [1, 17, 128, 129, 300])
+def test_plain_product_with_either_index_on_the_accumulator_rows(ctx, T, O, pad, offset, yref_dtype):
+    """Up to 128 rows, or rows off 16 bytes, put the result's columns on the accumulator's rows.  All alignments of a row on
+    both sides of that line; nothing beyond a row's O values is written.  FP32 sums of 80 products: K 2^-24 of the sum of
+    magnitudes."""
+    K, ldy = 80, O + pad
+    gen = torch.Generator(device=DEV).manual_seed(T + O)
+    W, X = (torch.randn(n, K, device=DEV, generator=gen).to(torch.bfloat16) for n in (O, T))
+    dt = torch.bfloat16 if yref_dtype == faar.BF16 else torch.float32
+    buf = torch.full((offset + T * ldy + 16,), 7.0, dtype=dt, device=DEV)
+    Y = buf[offset:offset + T * ldy].view(T, ldy)
+    shape = faar.make_shape(O, K, T, ldy=ldy, yref_dtype=yref_dtype)
+    ws = torch.empty(faar.workspace_size(shape), dtype=torch.uint8, device=DEV)
+    faar.workspace_init(ctx, ws)
+    faar.layer_ref(ctx, shape, X, W, Y, ws)
+    faar.check_status(ctx, ws)
+    ref, mag = X.double() @ W.double().T, X.double().abs() @ W.double().abs().T
+    tol = K * 2.0 ** -24 * mag + (2.0 ** -8 * ref.abs() if yref_dtype == faar.BF16 else 0.0)
+    assert torch.all((Y[:, :O].double() - ref).abs() <= tol)
+    assert torch.all(Y[:, O:] == 7.0) and torch.all(buf[:offset] == 7.0) and torch.all(buf[offset + T * ldy:] == 7.0)
+
+
+@pytest.mark.parametrize("O", [80, 1600])                                     # a whole contraction; a split one
+@pytest.mark.parametrize("T,K,ldx,ldy", [(1, 80, 80, 0), (17, 272, 280, 8), (128, 80, 88, 0), (129, 80, 80, 8), (300, 272, 280, 0)])
+def test_input_gradient_with_either_index_on_the_accumulator_rows(ctx, O, T, K, ldx, ldy):
+    """The same for dX = dY W_soft, whose weights are read as they are (contraction index as the row) on either side."""
+    gen = torch.Generator(device=DEV).manual_seed(T + O)
+    ldy += O
+    dY, Ws = (torch.randn(*s, device=DEV, generator=gen).to(torch.bfloat16) for s in ((T, ldy), (O, K)))
+    dX = torch.full((T, ldx), 7.0, dtype=torch.bfloat16, device=DEV)
+    shape = faar.make_shape(O, K, T, ldx=ldx, ldy=ldy)
+    ws = torch.empty(faar.workspace_size(shape), dtype=torch.uint8, device=DEV)
+    faar.workspace_init(ctx, ws)
+    faar.layer_dx_operand(ctx, shape, dY, Ws, dX, ws)
+    faar.check_status(ctx, ws)
+    ref, mag = dY[:, :O].double() @ Ws.double(), dY[:, :O].double().abs() @ Ws.double().abs()
+    assert torch.all((dX[:, :K].double() - ref).abs() <= O * 2.0 ** -24 * mag + 2.0 ** -8 * ref.abs())
+    assert torch.all(dX[:, K:] == 7.0)
+
+
+@pytest.mark.parametrize("yref_dtype", [faar.BF16, faar.F32])
 @pytest.mark.parametrize("T,ldy,offset", [(20, 32, 0), (20, 40, 0), (16, 24, 0), (203, 216, 0), (20, 32, 8), (9, 16, 8)])
 def test_padding_of_a_transposed_target_is_written_as_zeros(ctx, T, ldy, offset, yref_dtype):
     """Rows that start on 32 and on 16 bytes: the values, then zeros up to the next multiple of 16 columns, then nothing."""
