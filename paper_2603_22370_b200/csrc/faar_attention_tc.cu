@@ -257,20 +257,20 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   auto sV = [&](int s) { return base + OFF_V + (uint32_t)s * KV_BYTES; };
 
   if (warp == 4) {
-    // ---------------- copies and MMAs: one lane of this warp, which stays converged (see faar_elect_one) ----------
-    const bool lead = lane == 0;
+    // ---------------- copies and MMAs: one lane of this warp, which stays converged (see faar_elect_one; copies issued under
+    // `if (lane == 0)` cost the 64-element heads' backward pass 3 %) ----------
     auto wait = [&](uint32_t bar, uint32_t parity, uint32_t code) {
       return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
     };
     auto load_k = [&](int j) {
-      if (lead) { bar_expect(kfull(j & 1), KV_BYTES); tma_head<HD>(sK(j & 1), KV_PANEL, &tmK, g * HD, j * KT, b, kfull(j & 1)); }
+      if (faar_elect_one()) { bar_expect(kfull(j & 1), KV_BYTES); tma_head<HD>(sK(j & 1), KV_PANEL, &tmK, g * HD, j * KT, b, kfull(j & 1)); }
       __syncwarp();
     };
     auto load_v = [&](int j) {
-      if (lead) { bar_expect(vfull(j & 1), KV_BYTES); tma_head<HD>(sV(j & 1), KV_PANEL, &tmV, g * HD, j * KT, b, vfull(j & 1)); }
+      if (faar_elect_one()) { bar_expect(vfull(j & 1), KV_BYTES); tma_head<HD>(sV(j & 1), KV_PANEL, &tmV, g * HD, j * KT, b, vfull(j & 1)); }
       __syncwarp();
     };
-    if (lead) {
+    if (faar_elect_one()) {
       bar_expect(bar_q, Q_BYTES);
       tma_head<HD>(sQ, Q_PANEL, &tmQ, h * HD, q0, b, bar_q);
     }
@@ -529,20 +529,19 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   auto col_ds = [&](int j, int step) { return C::TWO ? col_s(j) + (uint32_t)(32 * (step >> 1) + 8 * (step & 1)) : 192u + 8u * (uint32_t)step; };
 
   if (warp == 8) {
-    const bool lead = lane == 0;
     auto wait = [&](uint32_t bar, uint32_t parity, uint32_t code) {
       return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
     };
     auto load_kv = [&](int j) {
       const int st = j % C::STAGES;
-      if (lead) {
+      if (faar_elect_one()) {
         bar_expect(kvfull(st), 2 * KV_BYTES);
         tma_head<HD>(sK(st), KV_PANEL, &tmK, g * HD, j * KT, b, kvfull(st));
         tma_head<HD>(sV(st), KV_PANEL, &tmV, g * HD, j * KT, b, kvfull(st));
       }
       __syncwarp();
     };
-    if (lead) {
+    if (faar_elect_one()) {
       bar_expect(bar_qd, 2 * Q_BYTES);
       tma_head<HD>(sQ, Q_PANEL, &tmQ, h * HD, q0, b, bar_qd);
       tma_head<HD>(sDO, Q_PANEL, &tmDO, h * HD, q0, b, bar_qd);
@@ -781,20 +780,19 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   auto q0_of = [&](int i) { return (qt0 + i % per_head) * KT; };
 
   if (warp == 8) {
-    const bool lead = lane == 0;
     auto wait = [&](uint32_t bar, uint32_t parity, uint32_t code) {
       return __all_sync(0xffffffffu, bar_wait(bar, parity, abort_flag, code)) != 0;
     };
     auto load_item = [&](int i) {
       const int st = i % C::STAGES;
-      if (lead) {
+      if (faar_elect_one()) {
         bar_expect(qfull(st), 2 * C::QD_BYTES);
         tma_head<HD>(sQ(st), KV_PANEL, &tmQ, head_of(i) * HD, q0_of(i), b, qfull(st));
         tma_head<HD>(sDO(st), KV_PANEL, &tmDO, head_of(i) * HD, q0_of(i), b, qfull(st));
       }
       __syncwarp();
     };
-    if (lead) {
+    if (faar_elect_one()) {
       bar_expect(bar_kv, 2 * C::KEY_BYTES);
       tma_head<HD>(sKt, Q_PANEL, &tmK, g * HD, k0, b, bar_kv);
       tma_head<HD>(sVt, Q_PANEL, &tmV, g * HD, k0, b, bar_kv);
