@@ -1361,19 +1361,19 @@ int pick_full(faar_ctx* ctx, int mode, int m_tiles, int n_main, int narrow, int 
   return best_full;
 }
 
-// Whether a launch takes 256 x 512 tiles (see Cfg): on request (ctx->tune_wide == 1) wherever the shape allows;
-// otherwise, for plain products and the forward product, where they turn two waves of 256-wide tiles into one of twice
-// the width, which pulls a quarter less operand data through the SMs and leaves fewer of them idle: forward kernel of a
-// 2048 x 8192 layer at 4096 tokens (128 tiles on 74 pairs -> 64) 137 -> 123 us, product [2000, 4096] over 2048 37 -> 32 us.
-// With more waves their epilogue, which nothing overlaps, costs more than that: gate/up at 8192 tokens 406 -> 477 us, the
-// forward kernel of an 8192 x 2048 layer 143 -> 168 us; the dW product's epilogue always does (173 -> 198 us).  The second
-// half's epilogue has to be earned by the main loop: the forward kernel of a 2048 x 2048 layer (32 k blocks) 40 -> 45 us.
-bool pick_wide(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int pairs) {
+// Whether a launch takes 256 x 512 tiles (see Cfg): on request (ctx->tune_wide == 1) wherever the shape allows.  They move a
+// quarter less operand data, but nothing overlaps their epilogue, and they give a wave of tiles no halves to even it out.
+// Plain product of 256-wide tiles -> 512-wide, us: 80 tiles (40 wide ones) over 2048 21.6 -> 30.0; 128 over 2048 34.0 -> 38.4,
+// over 4096 58.0 -> 62.4, over 8192 97 -> 99; 144 over 8192 101.3 -> 100.8; forward kernel and soft weights of 2048 x 4096 at
+// 4096 tokens 72.3 -> 74.2, with an FP32 target of 2048 x 8192 152 -> 164.  By themselves therefore only for a forward product
+// with a transposed BF16 target and 8192 or more contraction elements, where they take one wave that fills six of seven CTA
+// pairs: step of 2048 x 8192 at 4096 tokens 303 -> 298, its operands coming from HBM.
+bool pick_wide(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int pairs, bool fwd_vec) {
   if (bn != BN_MAX || ctx->tune_wide == 0) return false;
-  if (ctx->tune_wide == 1) return (mode == FAAR_GEMM_REF && M > N ? M : N) > BN_MAX;    // REF may have the tokens as its rows
-  const long long m_tiles = (M + 2 * BM - 1) / (2 * BM);
-  return (mode == FAAR_GEMM_FWD ? k_blocks >= 64 : mode == FAAR_GEMM_REF && k_blocks >= 24) && N > BN_MAX && ctx->tune_tail < 0 && ctx->tune_bn == 0 && m_tiles * ((N + BN_MAX - 1) / BN_MAX) > pairs &&
-         m_tiles * ((N + WIDE_BN - 1) / WIDE_BN) <= pairs;
+  if (ctx->tune_wide == 1) return (mode == FAAR_GEMM_REF && M > N ? M : N) > BN_MAX;    // REF may have either index as its rows
+  const long long wide = (long long)((M + 2 * BM - 1) / (2 * BM)) * ((N + WIDE_BN - 1) / WIDE_BN);
+  return mode == FAAR_GEMM_FWD && fwd_vec && k_blocks >= 128 && N > BN_MAX && ctx->tune_tail < 0 && ctx->tune_bn == 0 && wide <= pairs &&
+         7 * wide >= 6 * pairs;
 }
 
 template <int MODE, int OPT, int SHAPE, int MN>
@@ -1475,15 +1475,15 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
     kp.splits = pick_splits(MODE, a->M, a->N, k_blocks, clusters, &split_bn);
     attr[0].val.clusterDim.x = 2u * (unsigned)kp.splits;
   }
-  int bn = pick_bn(ctx, MODE, a->M, a->N, k_blocks, max_pairs, a->b_mn != 0,
-                   a->yref_t && a->yref_dtype == FAAR_BF16 && !a->Yout);
+  const bool fwd_vec = a->yref_t && a->yref_dtype == FAAR_BF16 && !a->Yout;
+  int bn = pick_bn(ctx, MODE, a->M, a->N, k_blocks, max_pairs, a->b_mn != 0, fwd_vec);
   if (kp.splits > 1 && ctx->tune_bn == 0) bn = split_bn;
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
   // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient; A, if the
   // accumulator's rows are the result's columns), the dW product with B or with both untransposed
   if constexpr (MODE == FAAR_GEMM_REF) {
     if (kp.columns && mn == 0) {
-      if (kp.splits == 1 && pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs))
+      if (kp.splits == 1 && pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs, fwd_vec))
         return launch_variant<MODE, OPT, WIDE_TILES, 4>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
       return launch_tiles<MODE, OPT, 4>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
     }
@@ -1494,7 +1494,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
     if (mn == 3) return launch_tiles<MODE, OPT, 3>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   }
   if (mn != 0) return (int)cudaErrorInvalidValue;
-  if (kp.splits == 1 && pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs))
+  if (kp.splits == 1 && pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs, fwd_vec))
     return launch_variant<MODE, OPT, WIDE_TILES, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   return launch_tiles<MODE, OPT, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
 }

@@ -23,7 +23,7 @@ struct faar_ctx {
   void* encode_tiled;  // cuTensorMapEncodeTiled, resolved through the runtime
   int tune_bn;                            // 0 = choose the GEMM tile width automatically
   int tune_tail;                          // -1 = choose the tail split automatically, else columns to split
-  int tune_wide;                          // 256 x 512 GEMM tiles: 1 = wherever the shape allows, 0 = never, -1 (default) = where they save a wave
+  int tune_wide;                          // 256 x 512 GEMM tiles: 1 = wherever the shape allows, 0 = never, -1 (default) = pick_wide's rule; 0 and 1 keep contractions whole
   int tune_attention_fragments;           // attention: 0 = tcgen05 kernels, 2 = mma.sync kernels (head_dim 64), 1 = the shared-memory fragment kernels
   int last_gemm_bn, last_gemm_pairs, last_gemm_split;   // what the last GEMM launch used
   std::vector<const void*> smem_set;      // kernels whose dynamic shared-memory limit has been raised on this device

@@ -348,7 +348,8 @@ def add(ctx, rows, cols, a, lda, b, ldb, out, ldo):
 
 
 def tune_wide_tiles(ctx, mode: int):
-    """1: 256 x 512 GEMM tiles whenever the shape allows; 0: never; -1 (the default): where they save a wave of tiles."""
+    """1: 256 x 512 GEMM tiles whenever the shape allows; 0: never; -1 (the default): for long forward products that
+    fill a wave of them.  0 and 1 keep contractions whole."""
     _check(lib().faar_tune_wide_tiles(ctx._h, mode), "faar_tune_wide_tiles")
 
 

@@ -1085,10 +1085,11 @@ def test_chaining_arguments_are_checked(ctx):
 
 
 # ---- which kernel form a launch takes ---------------------------------------------------------------------------
-@pytest.mark.parametrize("O,K,T", [(2048, 4096, 2560), (2000, 4096, 2570)])
-def test_wide_tiles_chosen_automatically_give_the_same_bits(ctx, O, K, T):
-    """80 tiles of 256 x 256 are two waves of the CTA pairs, 40 of 256 x 512 one: the forward and the plain product take
-    those by themselves, and every output element is the same sum in the same order."""
+@pytest.mark.parametrize("O,K,T,auto", [(2048, 4096, 2560, 256), (2000, 4096, 2570, 256), (2000, 8192, 4090, 512)])
+def test_wide_tiles_give_the_same_bits_and_are_taken_where_they_fill_a_wave(ctx, O, K, T, auto):
+    """80 tiles of 256 x 256 are two waves of the CTA pairs, 40 of 256 x 512 one, which takes longer all the same; 64 of
+    those with a long contraction the forward product takes by itself.  Every output element is the same sum in the same
+    order."""
     gen = torch.Generator(device=DEV).manual_seed(1)
     T16 = (T + 15) // 16 * 16
     shape = faar.make_shape(O, K, T, ldy=T16, yref_transposed=1)
@@ -1102,19 +1103,20 @@ def test_wide_tiles_chosen_automatically_give_the_same_bits(ctx, O, K, T):
     hp, _ = f32hp(beta=6.0, step=1)
     out = []
     try:
-        for wide in (-1, 0):
+        for wide in (1, 0, -1):
             faar.tune_wide_tiles(ctx, wide)
             Y = torch.zeros((O, T16), dtype=torch.bfloat16, device=DEV)
             dYt, loss = torch.zeros((O, (T + 7) // 8 * 8), dtype=torch.bfloat16, device=DEV), torch.zeros(1, device=DEV)
             faar.layer_ref(ctx, shape, X, W, Y, ws)
-            assert faar.last_gemm_config(ctx)[0] == (512 if wide else 256)
+            assert faar.last_gemm_config(ctx)[0] == {1: 512, 0: 256, -1: 256}[wide]
             faar.layer_fwd(ctx, shape, hp, X, Yref, V, code, scales, sg, dYt, loss, None, ws)
-            assert faar.last_gemm_config(ctx)[0] == (512 if wide else 256)
+            assert faar.last_gemm_config(ctx)[0] == {1: 512, 0: 256, -1: auto}[wide]
             out.append((Y[:, :T].clone(), dYt[:, :T].clone()))
     finally:
         faar.tune_wide_tiles(ctx, -1)
     faar.check_status(ctx, ws)
-    assert all(torch.equal(a, b) for a, b in zip(*out))
+    for other in out[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(out[0], other))
 
 
 @pytest.mark.parametrize("yref_dtype", [faar.BF16, faar.F32])
