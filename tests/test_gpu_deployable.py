@@ -159,6 +159,31 @@ def test_own_nvfp4_gemm_agrees_with_the_layer_path(ctx):
     assert rel_l2(a, b) <= 6e-3
 
 
+@pytest.mark.parametrize("M,N", [(130, 300), (1, 17), (2100, 2311)])
+def test_nvfp4_gemm_rows_of_any_alignment(ctx, M, N):
+    """Rows on 32, 16, 8, 4 and 2 bytes: the same bits, and nothing beyond a row's N values."""
+    K = 96
+    gen = torch.Generator(device=DEV).manual_seed(M)
+    u8 = lambda hi, *s: torch.randint(0, hi, s, device=DEV, generator=gen, dtype=torch.int32).to(torch.uint8)
+    a, b, sa, sb = u8(256, M, K // 2), u8(256, N, K // 2), u8(127, M, K // 16), u8(127, N, K // 16)
+    tiled = [torch.zeros((n + 127) // 128 * ((K // 16 + 3) // 4) * 512, dtype=torch.uint8, device=DEV) for n in (M, N)]
+    faar.swizzle_scales(ctx, M, K // 16, sa, tiled[0])
+    faar.swizzle_scales(ctx, N, K // 16, sb, tiled[1])
+    one = torch.full((1,), 0.125, device=DEV)
+    ws = ctx.workspace(faar.make_shape(16, 16, 8))
+    ref = None
+    for ldc, off in (((N + 15) // 16 * 16, 0), ((N + 15) // 16 * 16, 8), ((N + 7) // 8 * 8 + 4, 4), (N + 1 + N % 2, 0), (N + 1 + N % 2, 2),
+                     (N + N % 2, 1), (N + 2 + N % 2, 2), (N, 0)):
+        buf = torch.full((off + M * ldc + 16,), 7.0, dtype=torch.bfloat16, device=DEV)
+        faar.nvfp4_gemm(ctx, M, N, K, a, tiled[0], one, b, tiled[1], one, buf[off:], ldc, ws)
+        torch.cuda.synchronize()
+        faar.check_status(ctx, ws)
+        C = buf[off:off + M * ldc].view(M, ldc)
+        ref = C[:, :N].clone() if ref is None else ref
+        assert torch.equal(C[:, :N], ref), (ldc, off)
+        assert torch.all(C[:, N:] == 7.0) and torch.all(buf[:off] == 7.0) and torch.all(buf[off + M * ldc:] == 7.0)
+
+
 def test_nvfp4_gemm_argument_checks(ctx):
     lay, (px, _, sxt, sx), (pw, _, swt, sw) = _deployable_operands(ctx, 128, 64, 128, 3)
     Y = torch.empty((128, 128), dtype=torch.bfloat16, device=DEV)
