@@ -178,7 +178,11 @@ rmsnorm_kernel(const __nv_bfloat16* x, int64_t ldx, const __nv_bfloat16* b, int6
 // Backward of RMSNorm towards x (the norm weights are frozen): with xh = x * rstd and w = g * dy,
 // dx = rstd * (w - xh * mean(w * xh)), optionally added to `add` (the residual branch's gradient).  dy is the
 // FP32 sum of up to three BF16 tensors (the gradients of the linears that read the norm's output).  One warp
-// per row; the row is read twice (the dot product, then the result), the second time from L1 / L2.
+// per row; the row is read twice (the dot product, then the result), the second time from L1 / L2.  NG groups of a row are
+// requested at a time: two for long rows and where few rows leave a warp alone with its loads' latency, else one, which
+// leaves room for more warps.  Two gradients, one group -> two, us: 2000 x 2048 12.5 -> 10.5, 300 x 2048 8.1 -> 7.6,
+// 8192 x 4096 81 -> 72; 4000 x 2048 15.5 -> 17.0, 8192 x 1024 12.5 -> 14.1, 20000 x 64 8.2 -> 10.3.
+template <int NG>
 __global__ void __launch_bounds__(GL_THREADS)
 rmsnorm_bwd_kernel(const __nv_bfloat16* dy, const __nv_bfloat16* dy2, const __nv_bfloat16* dy3, int64_t lddy,
                    const __nv_bfloat16* x, int64_t ldx, const float* __restrict__ g, const float* __restrict__ rstd_in,
@@ -188,21 +192,39 @@ rmsnorm_bwd_kernel(const __nv_bfloat16* dy, const __nv_bfloat16* dy2, const __nv
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int n_groups = cols / 8;
   for (int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < rows; row += warps) {
-    const __nv_bfloat16* xr = x + (int64_t)row * ldx;
     const int64_t doff = (int64_t)row * lddy;
+    const uint4* xr = reinterpret_cast<const uint4*>(x + (int64_t)row * ldx);
+    const uint4* d1 = reinterpret_cast<const uint4*>(dy + doff);
+    const uint4* d2 = reinterpret_cast<const uint4*>(dy2 ? dy2 + doff : nullptr);
+    const uint4* d3 = reinterpret_cast<const uint4*>(dy3 ? dy3 + doff : nullptr);
+    const uint4* ar = reinterpret_cast<const uint4*>(add ? add + (int64_t)row * ldadd : nullptr);
+    uint4* out = reinterpret_cast<uint4*>(dx + (int64_t)row * lddx);
     const float rstd = rstd_in[row];
-    // w = g * (dy + dy2 + dy3) of one group
-    auto load_w = [&](int c, float (&w)[8]) {
-      unpack8(*reinterpret_cast<const uint4*>(dy + doff + 8 * c), w);
-      if (dy2) {
+    uint4 xv[NG], v1[NG], v2[NG], v3[NG];
+    auto request = [&](int c0) {
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        const int c = c0 + 32 * k;
+        if (c < n_groups) {
+          xv[k] = xr[c];
+          v1[k] = d1[c];
+          if (d2) v2[k] = d2[c];
+          if (d3) v3[k] = d3[c];
+        }
+      }
+    };
+    // w = g * (dy + dy2 + dy3) of the k-th requested group
+    auto weigh = [&](int k, int c, float (&w)[8]) {
+      unpack8(v1[k], w);
+      if (d2) {
         float t[8];
-        unpack8(*reinterpret_cast<const uint4*>(dy2 + doff + 8 * c), t);
+        unpack8(v2[k], t);
 #pragma unroll
         for (int i = 0; i < 8; ++i) w[i] += t[i];
       }
-      if (dy3) {
+      if (d3) {
         float t[8];
-        unpack8(*reinterpret_cast<const uint4*>(dy3 + doff + 8 * c), t);
+        unpack8(v3[k], t);
 #pragma unroll
         for (int i = 0; i < 8; ++i) w[i] += t[i];
       }
@@ -212,27 +234,45 @@ rmsnorm_bwd_kernel(const __nv_bfloat16* dy, const __nv_bfloat16* dy2, const __nv
       for (int i = 0; i < 8; ++i) w[i] *= gg[i];
     };
     float dot = 0.f;
-    for (int c = lane; c < n_groups; c += 32) {
-      float a[8], w[8];
-      unpack8(*reinterpret_cast<const uint4*>(xr + 8 * c), a);
-      load_w(c, w);
+    for (int c0 = lane; c0 < n_groups; c0 += 32 * NG) {
+      request(c0);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) dot = fmaf(w[i], a[i] * rstd, dot);
+      for (int k = 0; k < NG; ++k) {
+        const int c = c0 + 32 * k;
+        if (c < n_groups) {
+          float a[8], w[8];
+          unpack8(xv[k], a);
+          weigh(k, c, w);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) dot = fmaf(w[i], a[i] * rstd, dot);
+        }
+      }
     }
     dot = faar_warp_sum(dot) / (float)cols;
-    for (int c = lane; c < n_groups; c += 32) {
-      float a[8], w[8], o[8];
-      unpack8(*reinterpret_cast<const uint4*>(xr + 8 * c), a);
-      load_w(c, w);
+    for (int c0 = lane; c0 < n_groups; c0 += 32 * NG) {
+      request(c0);
+      uint4 av[NG];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) o[i] = rstd * fmaf(-(a[i] * rstd), dot, w[i]);
-      if (add) {
-        float r[8];
-        unpack8(*reinterpret_cast<const uint4*>(add + (int64_t)row * ldadd + 8 * c), r);
+      for (int k = 0; k < NG; ++k)
+        if (ar && c0 + 32 * k < n_groups) av[k] = ar[c0 + 32 * k];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] += r[i];
+      for (int k = 0; k < NG; ++k) {
+        const int c = c0 + 32 * k;
+        if (c < n_groups) {
+          float a[8], w[8], o[8];
+          unpack8(xv[k], a);
+          weigh(k, c, w);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) o[i] = rstd * fmaf(-(a[i] * rstd), dot, w[i]);
+          if (ar) {
+            float r[8];
+            unpack8(av[k], r);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[i] += r[i];
+          }
+          out[c] = pack8(o);
+        }
       }
-      *reinterpret_cast<uint4*>(dx + (int64_t)row * lddx + 8 * c) = pack8(o);
     }
   }
 }
@@ -482,7 +522,7 @@ int faar_launch_rmsnorm_bwd(faar_ctx* ctx, int rows, int cols, const void* dy, c
     faar_launch_pdl(ctx, cols <= 8 * 32 * 2 ? rmsnorm_bwd_row_kernel<2> : rmsnorm_bwd_row_kernel<8>, dim3(grid), dim3(GL_THREADS), 0, d1, lddy,
                     xp, ldx, g, rstd, ap, ldadd, op, lddx, rows, cols);
   else
-    faar_launch_pdl(ctx, rmsnorm_bwd_kernel, dim3(grid), dim3(GL_THREADS), 0, d1, d2, d3, lddy, xp, ldx, g, rstd, ap, ldadd, op, lddx, rows, cols);
+    faar_launch_pdl(ctx, cols > 8 * 32 * 8 || (cols > 8 * 32 * 4 && rows <= 16 * ctx->num_sms) ? rmsnorm_bwd_kernel<2> : rmsnorm_bwd_kernel<1>, dim3(grid), dim3(GL_THREADS), 0, d1, d2, d3, lddy, xp, ldx, g, rstd, ap, ldadd, op, lddx, rows, cols);
   return (int)cudaGetLastError();
 }
 

@@ -73,9 +73,10 @@ def test_rmsnorm_forward_and_backward(ctx, rows, cols, ld):
     assert torch.equal(R[:, :cols], DX[:, :cols])
 
 
-@pytest.mark.parametrize("rows,cols,ld", [(77, 136, 144), (40, 2048, 2048), (9, 2056, 2064), (3, 4096, 4096)])
+@pytest.mark.parametrize("rows,cols,ld", [(77, 136, 144), (40, 2048, 2048), (9, 2056, 2064), (3, 4096, 4096), (5, 1032, 1032), (2400, 1032, 1040)])
 def test_residual_add_fused_with_the_norm_and_gradient_sums_inside_its_backward(ctx, rows, cols, ld):
-    """Rows of up to 2048 elements stay in registers, longer ones are read twice: both forms, ragged widths."""
+    """Rows of up to 2048 elements stay in registers, longer ones (and several gradients) are read twice, one or two groups at
+    a time: all forms, ragged widths."""
     rng = np.random.default_rng(cols + rows)
     a = inputs.to_bf16_f32(rng.standard_normal((rows, cols)) * 2)
     b = inputs.to_bf16_f32(rng.standard_normal((rows, cols)))
