@@ -149,7 +149,6 @@ int faar_launch_softquant_eval(faar_ctx*, const faar_shape*, const float* V, con
                                const uint8_t* scales, const float* s_global, float beta,
                                float* W_soft, float* h, __nv_bfloat16* W_soft_bf16,
                                float* W_operand_f32 = nullptr);
-// BF16 soft weights of up to three linears stacked by output rows (seg: V, code, scales, s_global, rows)
 // BF16 soft weights of several linears (1 .. FAAR_MAX_SOFT_ITEMS), `weights` (a multiple of 16, below 2^40) each
 constexpr int FAAR_MAX_SOFT_ITEMS = 28;
 struct faar_soft_item { const float* V; const uint8_t* code; const uint8_t* scales; const float* s_global; __nv_bfloat16* out; int64_t weights; };

@@ -33,11 +33,11 @@ def padded(a, ld, fill=9.0):
 @pytest.mark.parametrize("B,S,H,HKV,D", [(2, 100, 4, 2, 64), (1, 64, 2, 2, 64), (3, 7, 2, 1, 64), (1, 200, 4, 1, 128),
                                          (2, 129, 8, 2, 64), (1, 321, 4, 4, 64)])
 def test_attention_forward_and_backward_match_the_oracle(ctx, B, S, H, HKV, D, fragments):
-    """fragments = 0: the default kernels (head_dim 64: forward and backward on tcgen05); 2: head_dim 64 with scores
-    in registers (mma.sync) forward and backward; 1: head_dim 64 through the shared-memory fragment kernels that
-    head_dim 128 always uses."""
+    """fragments = 0: the default kernels (forward and backward on tcgen05); 2: head_dim 64 with scores in registers
+    (mma.sync) forward and backward; 1: head_dim 64 through the shared-memory fragment kernels (128-element heads have a
+    test of their own)."""
     if fragments and D != 64:
-        pytest.skip("head_dim 128 has one kind of kernel")
+        pytest.skip("covered by test_attention_of_128_element_heads")
     faar.tune_attention(ctx, fragments)
     try:
         _attention_case(ctx, B, S, H, HKV, D)

@@ -779,32 +779,36 @@ def test_wide_tiles_give_the_same_step(ctx, O, K, T):
     assert np.all(np.abs(out[0][6] - out[1][6]) <= 1e-5 * np.abs(out[0][6]))
 
 
-@pytest.mark.parametrize("O,K,T,split", [
-    (300, 80, 752, "bwd"),           # the shortest: twelve k blocks, the last one ragged, parts of three
-    (40, 80, 1552, "bwd"),           # four parts of 6 or 7 k blocks, one 64-wide tile column and a bit
-    (520, 1312, 1808, "bwd"),        # two parts only
-    (130, 208, 1552, "bwd"),         # the dW product: shares of 16 columns of each tile
-    (300, 1040, 1800, "bwd"),
-    (1552, 80, 72, "dx"),            # the input gradient contracts over O
+@pytest.mark.parametrize("O,K,T,split,form", [
+    (300, 80, 752, "bwd", (64, 4)),        # the shortest: twelve k blocks, the last one ragged, parts of three
+    (40, 80, 1552, "bwd", (64, 4)),        # four parts of 6 or 7 k blocks, one 64-wide tile column and a bit
+    (520, 1312, 1808, "bwd", (128, 2)),    # two parts only
+    (130, 208, 1552, "bwd", (64, 4)),      # the dW product: shares of 16 columns of each tile
+    (300, 1040, 1800, "bwd", (128, 2)),
+    (256, 1536, 1536, "bwd", (64, 2)),     # shares of 32 columns
+    (300, 656, 2600, "bwd", (128, 4)),     # over 40 k blocks: three incoming parts, shares of two chunks
+    (1552, 80, 72, "dx", (64, 4)),         # the input gradient contracts over O
+    (2600, 1008, 100, "dx", (128, 4)),
 ])
-def test_contractions_split_over_several_cta_pairs(ctx, O, K, T, split):
+def test_contractions_split_over_several_cta_pairs(ctx, O, K, T, split, form):
     """Few tiles and a long contraction: the pairs of a cluster take a part of it each and exchange partial sums.  Only the
-    order of the FP32 additions differs from a whole contraction, which the bounds of the tests called here allow for."""
-    tiles = {"bwd": (O, K), "dx": (T, K)}[split]
+    order of the FP32 additions differs from a whole contraction, which the bounds of the tests called here allow for.
+    form: width of the tiles and parts of the contraction on a whole B200."""
+    M, N = (O, K) if split == "bwd" else ((K, T) if T <= 128 else (T, K))
 
-    def was_split():
+    def taken():
         bn, pairs = faar.last_gemm_config(ctx)[:2]
-        return pairs > min(-(-m // 256) * -(-n // bn) for m, n in (tiles, tiles[::-1]))
+        return bn, pairs // (-(-M // 256) * -(-N // bn))
 
     if split == "bwd":
         for opt in (1, 0):
             test_layer_bwd(ctx, O, K, T, opt)
-            assert was_split()
+            assert taken() == form
             test_backward_on_row_major_operands_gives_the_same_bits(ctx, O, K, T, opt)
-            assert was_split()
+            assert taken() == form
     else:
         test_layer_dx(ctx, O, K, T)
-        assert was_split()
+        assert taken() == form
 
 
 @pytest.mark.parametrize("opt", [0, 1])

@@ -192,7 +192,16 @@ def test_both_forward_passes_at_once_give_the_same_step(ctx):
 
 
 def test_stage2_step_with_a_split_lm_head_gradient_matches_the_oracle(ctx, monkeypatch):
-    """A vocabulary long enough for the last hidden state's gradient, which contracts over it, to be split over CTA pairs."""
+    """A vocabulary long enough for the last hidden state's gradient, which contracts over it, to be split over CTA pairs: a
+    product of the same sizes, on which alone the choice depends, says so."""
+    T, hidden, vocab = 2 * 96, 128, 1600
+    shape = faar.make_shape(vocab, hidden, T)
+    ws = torch.empty(faar.workspace_size(shape), dtype=torch.uint8, device=DEV)
+    faar.workspace_init(ctx, ws)
+    dY, Ws, dX = (torch.zeros(s, dtype=torch.bfloat16, device=DEV) for s in ((T, vocab), (vocab, hidden), (T, hidden)))
+    faar.layer_dx_operand(ctx, shape, dY, Ws, dX, ws)
+    bn, pairs = faar.last_gemm_config(ctx)[:2]
+    assert (bn, pairs) == (64, 4 * 2)
     build = small_model
     monkeypatch.setitem(globals(), "small_model", lambda seed=0: build(seed, vocab=1600))
     test_stage2_step_matches_the_oracle(ctx)
