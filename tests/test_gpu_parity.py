@@ -786,7 +786,7 @@ def test_wide_tiles_give_the_same_step(ctx, O, K, T):
     (130, 208, 1552, "bwd", (64, 4)),      # the dW product: shares of 16 columns of each tile
     (300, 1040, 1800, "bwd", (128, 2)),
     (256, 1536, 1536, "bwd", (64, 2)),     # shares of 32 columns
-    (300, 656, 2600, "bwd", (128, 4)),     # over 40 k blocks: three incoming parts, shares of two chunks
+    (300, 464, 2600, "bwd", (128, 4)),     # over 40 k blocks: three incoming parts, shares of two chunks
     (1552, 80, 72, "dx", (64, 4)),         # the input gradient contracts over O
     (2600, 1008, 100, "dx", (128, 4)),
 ])
