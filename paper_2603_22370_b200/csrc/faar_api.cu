@@ -228,10 +228,11 @@ int faar_bwd_group(faar_ctx* ctx, int n_seg, faar_bwd_state* seg, int T, int K, 
   return faar_launch_gemm(ctx, &a, nullptr);
 }
 
-int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes) {
+int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes, int carveout) {
   for (const void* k : c->smem_set)
     if (k == kernel) return 0;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && carveout >= 0) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
   if (e == cudaSuccess) c->smem_set.push_back(kernel);
   return (int)e;
 }

@@ -55,18 +55,36 @@ constexpr int BN_MAX = 256;
 // bounds these kernels; the price is that the epilogue of a tile no longer overlaps the next tile's main loop
 // (the two halves drain one after the other while the issuer waits).
 constexpr int WIDE_BN = 2 * BN_MAX;
-template <int MODE, bool WIDE = false> struct Cfg {
+// The tile forms of a launch, chosen at compile time (as run-time options of one kernel they cost the others time): tiles of
+// up to 256 columns, 256 x 512, a contraction split over the pairs of a cluster, or (BWD) 256-wide tiles of a short contraction.
+//
+// SHORT_TILES: a dW launch of few k blocks is bound by its epilogue's state traffic.  What limits that is the L1 cache: a
+// load in flight holds its L1 lines, and with all of an SM's 256 KB but 28 taken as shared memory, loads beyond about 24 KB
+// wait to be issued (1000 clocks per instruction of 4 weights a lane).  So a short contraction gives up one stage of the ring,
+// the next smaller carve-out leaves 60 KB of L1, and a lane requests 8 weights at a time, in 32-byte accesses.
+// dW kernel of 8192 x 2048, us: 64 tokens 93.3 -> 75.9 (4.5 -> 5.4 TB/s of state), 1024 95.3 -> 82.1, 2048 100.8 -> 93.8, 3000
+// 130.0 -> 128.9, 4096 134 -> 137; of 12288 x 2048 at 2000 149 -> 143.  With the carve-out but 4 weights at a time 64 tokens
+// take 91.8, with 8 at a time but no carve-out 97.6; without another stage (92 KB of L1) nothing changes but 2000 tokens, 148.
+// Above SHORT_BLOCKS the main loop needs the stage: operands and state together then take all the 64 bytes a clock that an
+// SM draws from L2.
+constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2, SHORT_TILES = 3;
+constexpr int SHORT_BLOCKS = 40;
+constexpr int SHORT_SMEM = 387 * 512;          // with the system's 1 KB below the 196 KB carve-out
+constexpr int SHORT_CARVEOUT = 85;             // percent of the 228 KB: 196 KB
+template <int MODE, int SHAPE = PLAIN_TILES> struct Cfg {
+  static constexpr bool WIDE = SHAPE == WIDE_TILES, SHORT = SHAPE == SHORT_TILES;
   static constexpr int EPI_WARPS = MODE == FAAR_GEMM_BWD ? 16 : 8;
   static constexpr int THREADS = 32 * (2 + EPI_WARPS);
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int BH_BYTES = (BN_MAX / 2) * BK * 2;       // this CTA's 128 rows of one 256-column B tile
   static constexpr int B_BYTES = WIDE ? 2 * BH_BYTES : BH_BYTES;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr int LANE_WEIGHTS = SHORT ? 8 : 4;             // BWD: weights of one instruction's state per lane
   static constexpr int EPI_BYTES = MODE == FAAR_GEMM_BWD ? 4 * PANEL_BYTES : 0;
   // The ring: as many stages of the launch's tile width as fit (a stage is the A rows plus bn / 2 rows of B: 32 KB for
   // 256 columns, 18 KB for 32), at most MAX_STAGES.  A small launch's main loop runs at stages / latency, so narrow
   // tiles get the deeper ring.
-  static constexpr int RING_BYTES = (SMEM_LIMIT - 1024 - CTL_BYTES - EPI_BYTES) / 1024 * 1024;
+  static constexpr int RING_BYTES = ((SHORT ? SHORT_SMEM : SMEM_LIMIT) - 1024 - CTL_BYTES - EPI_BYTES) / 1024 * 1024;
   static constexpr int MIN_STAGES = RING_BYTES / STAGE_BYTES;
   static constexpr int TMEM_COLS = 2 * BN_MAX;                 // two accumulator buffers
   static constexpr int COL_GROUPS = EPI_WARPS / 4;             // warps sharing one TMEM lane quarter
@@ -197,14 +215,36 @@ __device__ __forceinline__ uint64_t l2_policy_stream() {
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-__device__ __forceinline__ float4 ldg128_stream(const float* ptr, uint64_t pol) {
-  float4 v;
-  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(ptr), "l"(pol));
-  return v;
+// Four or eight consecutive values of the per-weight state: one access of 16 or 32 bytes, or (`wide` false: a base that is
+// off 32 bytes) two of 16.
+__device__ __forceinline__ void ldg_state(const float* ptr, bool wide, uint64_t pol, float (&v)[8]) {
+  if (wide) {
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], %9;"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(ptr), "l"(pol));
+  } else {
+#pragma unroll
+    for (int h = 0; h < 8; h += 4)
+      asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
+                   : "=f"(v[h]), "=f"(v[h + 1]), "=f"(v[h + 2]), "=f"(v[h + 3]) : "l"(ptr + h), "l"(pol));
+  }
 }
-__device__ __forceinline__ void stg128_stream(float* ptr, float a, float b, float c, float d, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(ptr), "f"(a), "f"(b), "f"(c), "f"(d), "l"(pol)
+__device__ __forceinline__ void ldg_state(const float* ptr, bool, uint64_t pol, float (&v)[4]) {
+  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(ptr), "l"(pol));
+}
+__device__ __forceinline__ void stg_state(float* ptr, bool wide, uint64_t pol, const float (&v)[8]) {
+  if (wide) {
+    asm volatile("st.global.L2::cache_hint.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8}, %9;" ::"l"(ptr), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "l"(pol) : "memory");
+  } else {
+#pragma unroll
+    for (int h = 0; h < 8; h += 4)
+      asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(ptr + h), "f"(v[h]), "f"(v[h + 1]), "f"(v[h + 2]),
+                   "f"(v[h + 3]), "l"(pol) : "memory");
+  }
+}
+__device__ __forceinline__ void stg_state(float* ptr, bool, uint64_t pol, const float (&v)[4]) {
+  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(ptr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "l"(pol)
                : "memory");
 }
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
@@ -291,6 +331,7 @@ struct Segment {
   float* V; const uint8_t* code; const uint8_t* scales; const float* s_global;
   float* adam_m; float* adam_u; float* dV;
   float lam4;                       // -4 lambda / N: (lambda / N) (4 - 8 v) = lam4 (2 v - 1)
+  int wide;                         // V, m, u and dV all lie on 32-byte boundaries (a row is a multiple of 64 bytes)
 };
 
 struct KParams {
@@ -600,10 +641,10 @@ __device__ __forceinline__ float rcp_approx(float x) {
 }
 
 // The four epilogue warps that share a TMEM lane quarter stage a 32-row x PW-column panel of G in
-// shared memory (row r at panel + 4 PW r, its 16-byte units XOR-swizzled by (r & 7)); then warp `sub`
-// of the quarter takes rows 8 sub .. 8 sub + 7, LPR = PW / 4 lanes per row and lane l the columns
-// 4 (l % LPR)..+3, so that one warp instruction moves 512 bytes of V / m / u as 32 / LPR row pieces of
-// 4 PW contiguous bytes each: whole lines as 16-byte vectors.  (A panel of 128 columns gives one 512-byte
+// shared memory (row r at panel + 4 PW r, its 16-byte units swizzled: panel_unit); then warp `sub`
+// of the quarter takes rows 8 sub .. 8 sub + 7, LPR = PW / LW lanes per row and lane l the columns
+// LW (l % LPR) and on, so that one warp instruction moves 128 LW bytes of V / m / u as 32 / LPR row pieces of
+// 4 PW contiguous bytes each: whole lines as 16- or 32-byte vectors.  (A panel of 128 columns gives one 512-byte
 // piece per instruction but leaves room for five TMA stages only; the sixth stage is worth more.)
 // The per-weight state of the next instruction is requested before the current one's is computed, and a panel's first
 // before the panel is staged (a tile's first before its accumulator is ready): a request takes 600-800 clocks, the
@@ -611,116 +652,127 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // o_first: output feature of panel row 0; k_first: input feature of panel column 0; k_end: first
 // input feature beyond the tile (or the matrix).
 // Returns the Round Loss contribution of the pre-update v's.
-constexpr int LPR = PW / 4;                     // lanes per panel row
-constexpr int RPI = 32 / LPR;                   // rows per warp instruction
-constexpr int ITS = 8 / RPI;                    // instructions per warp and panel
-struct RowState { float4 v, m, u; uint32_t cw, sb; };
-// State of this lane's four weights of instruction `it` of the panel whose row 0 / column 0 is (o_first, k_first), or
+// LW is 4, or 8 in launches of short contractions (Cfg::LANE_WEIGHTS).
+// 16-byte unit `u` of row `row` of a panel: the row moves its units around so that a column of rows does not collide, and with
+// eight columns a lane even units lie in a row's first half, odd ones in its second, so that its lanes read consecutive units.
+template <int LW> __device__ __forceinline__ uint32_t panel_unit(uint32_t panel, int row, int u) {
+  return panel + (uint32_t)row * (4u * PW) + (uint32_t)((LW == 4 ? u ^ (row & 7) : ((u >> 1) ^ (row & 7)) | (u & 1) << 3) << 4);
+}
+template <int LW> struct RowState { float v[LW], m[LW], u[LW]; uint32_t cw, sb; };
+// State of this lane's LW weights of instruction `it` of the panel whose row 0 / column 0 is (o_first, k_first), or
 // nothing if they lie outside the matrix or at or beyond column k_end.
-template <int OPT>
+template <int OPT, int LW>
 __device__ __forceinline__ bool load_row_state(const KParams& p, const Segment& g, int lane, int sub, int o_first, int k_first, int k_end, int it,
-                                               uint64_t stream, RowState& st) {
-  const int row = o_first + 8 * sub + lane / LPR + RPI * it, col = k_first + 4 * (lane % LPR);
+                                               uint64_t stream, RowState<LW>& st) {
+  constexpr int LPR = PW / LW, RPI = 32 / LPR;                     // lanes per panel row; rows per warp instruction
+  const int row = o_first + 8 * sub + lane / LPR + RPI * it, col = k_first + LW * (lane % LPR);
   const bool ok = row < p.M && col < k_end;
   if (ok) {
     const long long e = (long long)row * p.N + col;
-    st.v = ldg128_stream(g.V + e, stream);
-    st.cw = *reinterpret_cast<const uint16_t*>(g.code + (e >> 1));
+    ldg_state(g.V + e, g.wide, stream, st.v);
+    if (LW == 4) st.cw = *reinterpret_cast<const uint16_t*>(g.code + (e >> 1));
+    else st.cw = *reinterpret_cast<const uint32_t*>(g.code + (e >> 1));
     st.sb = g.scales[e >> 4];
     if (OPT & 1) {
-      st.m = ldg128_stream(g.adam_m + e, stream);
-      st.u = ldg128_stream(g.adam_u + e, stream);
+      ldg_state(g.adam_m + e, g.wide, stream, st.m);
+      ldg_state(g.adam_u + e, g.wide, stream, st.u);
     }
   }
   return ok;
 }
 // `st` / `st_ok` hold the state of instruction 0 on entry; on return those of instruction 0 of the panel at column
 // k_next (unless k_next >= k_end).
-template <int OPT>
+template <int OPT, int LW>
 __device__ __forceinline__ float epi_bwd_rows(const KParams& p, const Segment& sg, uint32_t panel, int lane, int sub, int o_first,
-                                              int k_first, int k_next, int k_end, float s_global, RowState& st, bool& st_ok) {
-  const int cu = lane % LPR;                                       // 16-byte unit of the row
+                                              int k_first, int k_next, int k_end, float s_global, RowState<LW>& st, bool& st_ok) {
+  constexpr int LPR = PW / LW, RPI = 32 / LPR, ITS = 8 / RPI;      // ITS: instructions per warp and panel
+  const int cu = lane % LPR;                                       // LW columns of the row
   const int r0 = 8 * sub + lane / LPR;                             // this lane's row in the first instruction
-  const long long e0 = (long long)(o_first + r0) * p.N + k_first + 4 * cu;         // row r0 element of this lane
+  const long long e0 = (long long)(o_first + r0) * p.N + k_first + LW * cu;        // row r0 element of this lane
   const uint64_t stream = l2_policy_stream();
   const uint64_t vkeep = l2_policy_keep();       // the updated V is the next kernel's input (soft weights)
   float tt = 0.f, n_el = 0.f;                                     // sum of (2 v - 1)^2, elements seen
 #pragma unroll
   for (int it = 0; it < ITS; ++it) {
-    const RowState cur = st;
+    RowState<LW> cur = st;
     const bool ok = st_ok;
     st_ok = it + 1 < ITS ? load_row_state<OPT>(p, sg, lane, sub, o_first, k_first, k_end, it + 1, stream, st)
                          : load_row_state<OPT>(p, sg, lane, sub, o_first, k_next, k_end, 0, stream, st);
-    {
-      if (ok) {
-        const int row = r0 + RPI * it;
-        const long long e = e0 + (long long)(RPI * it) * p.N;
-        const float4 g4 = lds128(panel + (uint32_t)row * (4u * PW) + (uint32_t)((cu ^ (row & 7)) << 4));
-        const float G[4] = {g4.x, g4.y, g4.z, g4.w};
-        const float vv[4] = {cur.v.x, cur.v.y, cur.v.z, cur.v.w};
-        const float sc = __fmul_rn(faar_e4m3_to_float(cur.sb), s_global);
-        const float sbh = sc * p.sbeta;
-        // byte j: log2 of (interval width / 0.5) of element j, looked up by its interval index k (0 0 0 0 1 1 2)
-        const uint32_t ksel = cur.cw & 0x7777u;
-        const uint32_t wlog = __byte_perm(0u, 0x00020101u, ksel);
-        // OPT & 2: bytes 3 and 2 of the lower node's float (0 .5 1 1.5 2 3 4) by the same look-up
-        uint32_t lo_hi = 0u, lo_lo = 0u;
-        if (OPT & 2) {
-          lo_hi = __byte_perm(0x3F3F3F00u, 0x00404040u, ksel);
-          lo_lo = __byte_perm(0xC0800000u, 0x00804000u, ksel);
-        }
-        float wn[4];
-        float g[4], vn[4], mn[4], un[4];
-        float mm[4], uu[4];
-        if (OPT & 1) {
-          mm[0] = cur.m.x; mm[1] = cur.m.y; mm[2] = cur.m.z; mm[3] = cur.m.w;
-          uu[0] = cur.u.x; uu[1] = cur.u.y; uu[2] = cur.u.z; uu[3] = cur.u.w;
-        }
+    if (!ok) continue;
+    const int row = r0 + RPI * it;
+    const long long e = e0 + (long long)(RPI * it) * p.N;
+    const float sc = __fmul_rn(faar_e4m3_to_float(cur.sb), s_global);
+    const float sbh = sc * p.sbeta;
+    float g[LW];
+    uint32_t wn[LW / 2];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float ex = ex2_approx(-fabsf(fmaf(p.bl, vv[j], p.hbl)));         // e^-|beta (v - 0.5)|
-          const float hs = rcp_approx(1.0f + ex);
-          const float dh = ex * hs * hs;                                     // h (1 - h)
-          // dh times the width factor by an add to its exponent field (a dh flushed to 0 becomes ~1e-38), then
-          // the sign of w from bit 3 of the nibble
-          const uint32_t wexp = (j < 3 ? wlog << (23 - 8 * j) : wlog >> 1) & 0x01800000u;
-          const uint32_t sgn = (cur.cw << (28 - 4 * j)) & 0x80000000u;
-          float chain = sbh * __uint_as_float(__float_as_uint(dh) + wexp);
-          chain = __uint_as_float(__float_as_uint(chain) ^ sgn);
-          const float t = fmaf(2.f, vv[j], -1.f);
-          g[j] = fmaf(G[j], chain, sg.lam4 * t);
-          tt = fmaf(t, t, tt);
-          if (OPT & 1) {
-            mn[j] = fmaf(p.b1, mm[j], p.c1 * g[j]);
-            un[j] = fmaf(p.b2, uu[j], p.c2 * g[j] * g[j]);
-            const float den = fmaf(sqrt_approx(un[j]), p.rbc2, p.eps);
-            vn[j] = __saturatef(fmaf(p.nstep, mn[j] * rcp_approx(den), vv[j]));   // clip to [0, 1]
-          } else {
-            vn[j] = __saturatef(fmaf(p.nstep, g[j], vv[j]));
-          }
-          if (OPT & 2) {
-            // Eq. 2 / Eq. 3 at the updated v with the next step's beta: (lo + h width) s with the sign of w, in
-            // the soft-weights kernel's operations, so that the BF16 operand is the same bit for bit
-            const float lo = __uint_as_float(__byte_perm(lo_hi, lo_lo, (uint32_t)((j << 12) | ((4 + j) << 8))) & 0xFFFF0000u);
-            const float wd = __uint_as_float(0x3F000000u + wexp);
-            const float mag = faar_operand_weight(faar_sigmoid_operand(p.nbl_next, p.hbl_next, vn[j]), lo, wd, sc);
-            wn[j] = __uint_as_float(__float_as_uint(mag) ^ sgn);
-          }
-        }
-        // one check covers the five stores below: they share the element offset e
-        if (!FAAR_DBG_OK(p, sg.V + e, 16, sg.V, p.ext_state, 3u)) continue;
-        if ((OPT & 2) && !FAAR_DBG_OK(p, p.wsoft_next + e, 8, p.wsoft_next, p.ext_wsoft, 4u)) continue;
-        if (OPT & 2)
-          *reinterpret_cast<uint2*>(p.wsoft_next + e) = make_uint2(pack_bf16x2(wn[0], wn[1]), pack_bf16x2(wn[2], wn[3]));
-        if (sg.dV) stg128_stream(sg.dV + e, g[0], g[1], g[2], g[3], stream);
+    for (int h = 0; h < LW / 4; ++h) {
+      const float4 g4 = lds128(panel_unit<LW>(panel, row, LW / 4 * cu + h));
+      const float G[4] = {g4.x, g4.y, g4.z, g4.w};
+      const uint32_t cw = h ? cur.cw >> 16 : cur.cw;
+      // byte j: log2 of (interval width / 0.5) of element j, looked up by its interval index k (0 0 0 0 1 1 2)
+      const uint32_t ksel = cw & 0x7777u;
+      const uint32_t wlog = __byte_perm(0u, 0x00020101u, ksel);
+      // OPT & 2: bytes 3 and 2 of the lower node's float (0 .5 1 1.5 2 3 4) by the same look-up
+      uint32_t lo_hi = 0u, lo_lo = 0u;
+      if (OPT & 2) {
+        lo_hi = __byte_perm(0x3F3F3F00u, 0x00404040u, ksel);
+        lo_lo = __byte_perm(0xC0800000u, 0x00804000u, ksel);
+      }
+      float w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float& v = cur.v[4 * h + j];
+        const float ex = ex2_approx(-fabsf(fmaf(p.bl, v, p.hbl)));         // e^-|beta (v - 0.5)|
+        const float hs = rcp_approx(1.0f + ex);
+        const float dh = ex * hs * hs;                                     // h (1 - h)
+        // dh times the width factor by an add to its exponent field (a dh flushed to 0 becomes ~1e-38), then
+        // the sign of w from bit 3 of the nibble
+        const uint32_t wexp = (j < 3 ? wlog << (23 - 8 * j) : wlog >> 1) & 0x01800000u;
+        const uint32_t sgn = (cw << (28 - 4 * j)) & 0x80000000u;
+        float chain = sbh * __uint_as_float(__float_as_uint(dh) + wexp);
+        chain = __uint_as_float(__float_as_uint(chain) ^ sgn);
+        const float t = fmaf(2.f, v, -1.f);
+        const float gj = fmaf(G[j], chain, sg.lam4 * t);
+        g[4 * h + j] = gj;
+        tt = fmaf(t, t, tt);
         if (OPT & 1) {
-          stg128_stream(sg.adam_m + e, mn[0], mn[1], mn[2], mn[3], stream);
-          stg128_stream(sg.adam_u + e, un[0], un[1], un[2], un[3], stream);
+          float &m = cur.m[4 * h + j], &u = cur.u[4 * h + j];
+          m = fmaf(p.b1, m, p.c1 * gj);
+          u = fmaf(p.b2, u, p.c2 * gj * gj);
+          const float den = fmaf(sqrt_approx(u), p.rbc2, p.eps);
+          v = __saturatef(fmaf(p.nstep, m * rcp_approx(den), v));           // clip to [0, 1]
+        } else {
+          v = __saturatef(fmaf(p.nstep, gj, v));
         }
-        stg128_stream(sg.V + e, vn[0], vn[1], vn[2], vn[3], vkeep);
-        n_el += 4.f;
+        if (OPT & 2) {
+          // Eq. 2 / Eq. 3 at the updated v with the next step's beta: (lo + h width) s with the sign of w, in
+          // the soft-weights kernel's operations, so that the BF16 operand is the same bit for bit
+          const float lo = __uint_as_float(__byte_perm(lo_hi, lo_lo, (uint32_t)((j << 12) | ((4 + j) << 8))) & 0xFFFF0000u);
+          const float wd = __uint_as_float(0x3F000000u + wexp);
+          const float mag = faar_operand_weight(faar_sigmoid_operand(p.nbl_next, p.hbl_next, v), lo, wd, sc);
+          w[j] = __uint_as_float(__float_as_uint(mag) ^ sgn);
+        }
+      }
+      if (OPT & 2) {
+        wn[2 * h] = pack_bf16x2(w[0], w[1]);
+        wn[2 * h + 1] = pack_bf16x2(w[2], w[3]);
       }
     }
+    // one check covers the five stores below: they share the element offset e
+    if (!FAAR_DBG_OK(p, sg.V + e, 4 * LW, sg.V, p.ext_state, 3u)) continue;
+    if ((OPT & 2) && !FAAR_DBG_OK(p, p.wsoft_next + e, 2 * LW, p.wsoft_next, p.ext_wsoft, 4u)) continue;
+    if (OPT & 2) {
+      if constexpr (LW == 4) *reinterpret_cast<uint2*>(p.wsoft_next + e) = make_uint2(wn[0], wn[1]);
+      else *reinterpret_cast<uint4*>(p.wsoft_next + e) = make_uint4(wn[0], wn[1], wn[2], wn[3]);
+    }
+    if (sg.dV) stg_state(sg.dV + e, sg.wide, stream, g);
+    if (OPT & 1) {
+      stg_state(sg.adam_m + e, sg.wide, stream, cur.m);
+      stg_state(sg.adam_u + e, sg.wide, stream, cur.u);
+    }
+    stg_state(sg.V + e, sg.wide, vkeep, cur.v);
+    n_el += (float)LW;
   }
   return n_el - tt;                                               // sum of 1 - (2 v - 1)^2
 }
@@ -784,15 +836,15 @@ __device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t parts, int
 // MN: bit 0 = the A operand, bit 1 = the B operand is stored with its M / N index contiguous (KParams.a_mn / b_mn);
 // a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.  Bit 2 (REF): the
 // accumulator's rows are the result's columns; compiled in as well (as a branch it cost 0.1 us in every small product).
-// SHAPE: 0 = tiles of up to 256 columns, WIDE_TILES, SPLIT_TILES; at compile time for the same reason.
-constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2;
+// SHAPE: PLAIN_TILES, WIDE_TILES, SPLIT_TILES, SHORT_TILES (see Cfg).
 constexpr int MIN_SPLIT_BLOCKS = 12;            // contractions of fewer k blocks stay whole (see pick_splits)
 template <int MODE, int OPT, int SHAPE, int MN>
-__global__ void __launch_bounds__(Cfg<MODE, SHAPE == WIDE_TILES>::THREADS, 1)
+__global__ void __launch_bounds__(Cfg<MODE, SHAPE>::THREADS, 1)
 faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ KParams p) {
   constexpr bool WIDE = SHAPE == WIDE_TILES, SPLIT = SHAPE == SPLIT_TILES;
-  using C = Cfg<MODE, WIDE>;
+  using C = Cfg<MODE, SHAPE>;
+  constexpr int LW = C::LANE_WEIGHTS;
   constexpr bool A_MN = (MN & 1) != 0, B_MN = (MN & 2) != 0, COLUMNS = (MN & 4) != 0;
   const int BN = p.bn;
   extern __shared__ uint8_t smem_raw[];
@@ -973,7 +1025,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     float s_global = 0.f;
     if (MODE == FAAR_GEMM_BWD) s_global = *p.seg[0].s_global;
     uint32_t pn = 0;                                   // panels this quarter has staged so far
-    RowState row_state;                                // BWD: state requested ahead
+    RowState<LW> row_state;                               // BWD: state requested ahead
     bool row_ok = false;
     const bool yvec_ok = MODE == FAAR_GEMM_FWD && p.yref_t && p.yref_dtype == FAAR_BF16 && p.Yout == nullptr;
     bool dead = false;
@@ -1060,8 +1112,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (SPLIT) add_parts(r, parts, splits, split, TW, c, quarter * 32 + lane);
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-              sts128(panel + (uint32_t)lane * (4u * PW) + (uint32_t)(((4 * sub + u) ^ (lane & 7)) << 4), r[4 * u],
-                     r[4 * u + 1], r[4 * u + 2], r[4 * u + 3]);
+              sts128(panel_unit<LW>(panel, lane, 4 * sub + u), r[4 * u], r[4 * u + 1], r[4 * u + 2], r[4 * u + 3]);
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(pfull);
@@ -1380,12 +1431,12 @@ template <int MODE, int OPT, int SHAPE, int MN>
 int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_out, int bn, int max_pairs,
                    const cudaLaunchConfig_t& base_cfg) {
   constexpr bool WIDE = SHAPE == WIDE_TILES;
-  using C = Cfg<MODE, WIDE>;
+  using C = Cfg<MODE, SHAPE>;
   static_assert(C::MIN_STAGES >= 3, "ring too short");
   static_assert(C::SMEM_BYTES <= SMEM_LIMIT, "shared memory budget");
   static_assert(C::EPI_WARPS <= MAX_EPI_WARPS, "partials budget");
   auto kern = faar_gemm_kernel<MODE, OPT, SHAPE, MN>;
-  int e = faar_allow_smem(ctx, (const void*)kern, C::SMEM_BYTES);
+  int e = faar_allow_smem(ctx, (const void*)kern, C::SMEM_BYTES, C::SHORT ? SHORT_CARVEOUT : -1);
   if (e) return e;
   cudaLaunchConfig_t cfg = base_cfg;
   cfg.dynamicSmemBytes = C::SMEM_BYTES;
@@ -1437,6 +1488,10 @@ template <int MODE, int OPT, int MN>
 int launch_tiles(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_out, int bn, int max_pairs, const cudaLaunchConfig_t& cfg) {
   if constexpr (MODE != FAAR_GEMM_FWD) {
     if (kp.splits > 1) return launch_variant<MODE, OPT, SPLIT_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+  }
+  if constexpr (MODE == FAAR_GEMM_BWD) {
+    if (bn == BN_MAX && (a->Kc + BK - 1) / BK <= SHORT_BLOCKS)
+      return launch_variant<MODE, OPT, SHORT_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   }
   return launch_variant<MODE, OPT, PLAIN_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
 }
@@ -1563,6 +1618,8 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
       k.V = g.V - e0; k.code = g.code - e0 / 2; k.scales = g.scales - e0 / 16; k.s_global = g.s_global;
       k.adam_m = g.adam_m ? g.adam_m - e0 : nullptr; k.adam_u = g.adam_u ? g.adam_u - e0 : nullptr; k.dV = g.dV ? g.dV - e0 : nullptr;
       k.lam4 = -4.f * g.lam_over_n;
+      k.wide = ((reinterpret_cast<uintptr_t>(g.V) | reinterpret_cast<uintptr_t>(g.adam_m) | reinterpret_cast<uintptr_t>(g.adam_u) |
+                 reinterpret_cast<uintptr_t>(g.dV)) & 31) == 0;
       row0 += g.rows;
     }
   }

@@ -57,7 +57,8 @@ struct faar_prof_scope {
 
 // Raises a kernel's dynamic shared-memory limit, once per context (the call costs about as much host time as a launch's
 // argument checks and every launch of a small layer would pay it).  The context's device is current.
-int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes);
+// carveout: the part of the SM's memory that is preferred as shared memory, in percent; -1 leaves it to the driver.
+int faar_allow_smem(faar_ctx* c, const void* kernel, int bytes, int carveout = -1);
 // How many clusters of `kernel` (launched as *cfg, which says their size 2 << size; its grid ignored) the context's device
 // holds at once: a fact of device and kernel (a GPC with an odd SM count strands one SM), asked once per device and process.
 constexpr int FAAR_CLUSTER_SIZES = 3;     // 2, 4, 8 CTAs
