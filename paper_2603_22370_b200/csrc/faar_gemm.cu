@@ -447,20 +447,41 @@ __device__ __forceinline__ void store_units(void* y, const uint32_t (&w)[8], boo
   reinterpret_cast<uint4*>(y)[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 // The accumulator's rows as columns of Y: neighbouring lanes write neighbouring values, whatever the alignment of a row of Y.
+template <typename T>
+__device__ __forceinline__ void store_columns(const KParams& p, int col, int r0, const uint32_t (&acc)[16]) {
+  T* y = reinterpret_cast<T*>(p.Yout) + (long long)r0 * p.ldy + col;
+  auto store = [&](int j) {
+    if (!FAAR_DBG_OK(p, y + j * p.ldy, (int)sizeof(T), p.Yout, p.ext_yout, 1u)) return;
+    if constexpr (sizeof(T) == 2) y[j * p.ldy] = __float2bfloat16_rn(__uint_as_float(acc[j]));
+    else y[j * p.ldy] = __uint_as_float(acc[j]);
+  };
+  if (r0 + 16 <= p.N) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) store(j);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (r0 + j < p.N) store(j);
+  }
+}
 __device__ __forceinline__ void epi_ref_columns(const KParams& p, int col, int r0, const uint32_t (&acc)[16]) {
   if (col >= p.M) return;
+  if (p.yout_dtype == FAAR_BF16) store_columns<__nv_bfloat16>(p, col, r0, acc);
+  else store_columns<float>(p, col, r0, acc);
+}
+// 16 columns as BF16 pairs, those beyond the matrix as 0.  One test for all of them: `whole || column < N` for each became 16
+// branches, 600 clocks per 16 columns and most of a 256-wide tile's epilogue, which nothing hides for a pair's last tile:
+// products over 2048, us: [2000, 2048] 18.1 -> 16.8, [2000, 4096] 28.5 -> 27.1; [2000, 2048] over 6144 38.7 -> 37.3.
+__device__ __forceinline__ void pack_ref(const KParams& p, int c0, const uint32_t (&acc)[16], uint32_t (&w)[8]) {
+  if (c0 + 16 <= p.N) {
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    if (r0 + j >= p.N) continue;
-    const long long off = (long long)(r0 + j) * p.ldy + col;
-    if (p.yout_dtype == FAAR_BF16) {
-      __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + off;
-      if (FAAR_DBG_OK(p, y, 2, p.Yout, p.ext_yout, 1u)) *y = __float2bfloat16_rn(__uint_as_float(acc[j]));
-    } else {
-      float* y = reinterpret_cast<float*>(p.Yout) + off;
-      if (FAAR_DBG_OK(p, y, 4, p.Yout, p.ext_yout, 1u)) *y = __uint_as_float(acc[j]);
-    }
+    for (int j = 0; j < 8; ++j) w[j] = pack_bf16x2(__uint_as_float(acc[2 * j]), __uint_as_float(acc[2 * j + 1]));
+    return;
   }
+  const uint32_t valid = (1u << max(p.N - c0, 0)) - 1u;
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    w[j] = pack_bf16x2(valid >> (2 * j) & 1u ? __uint_as_float(acc[2 * j]) : 0.f, valid >> (2 * j + 1) & 1u ? __uint_as_float(acc[2 * j + 1]) : 0.f);
 }
 __device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const uint32_t (&acc)[16]) {
   if (row >= p.M) return;
@@ -470,19 +491,17 @@ __device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const
     if (p.yout_dtype == FAAR_BF16) {
       __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + off;
       uint32_t w[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        w[j] = pack_bf16x2(whole || c0 + 2 * j < p.N ? __uint_as_float(acc[2 * j]) : 0.f,
-                           whole || c0 + 2 * j + 1 < p.N ? __uint_as_float(acc[2 * j + 1]) : 0.f);
+      pack_ref(p, c0, acc, w);
       if (FAAR_DBG_OK(p, y, 32, p.Yout, p.ext_yout, 1u)) store_units(y, w, wide);
     } else {
       float* y = reinterpret_cast<float*>(p.Yout) + off;
       if (!FAAR_DBG_OK(p, y, 64, p.Yout, p.ext_yout, 1u)) return;
+      const uint32_t valid = whole ? 0xFFFFu : (1u << max(p.N - c0, 0)) - 1u;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         uint32_t w[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) w[j] = whole || c0 + 8 * h + j < p.N ? acc[8 * h + j] : 0u;
+        for (int j = 0; j < 8; ++j) w[j] = valid >> (8 * h + j) & 1u ? acc[8 * h + j] : 0u;
         store_units(y + 8 * h, w, wide);
       }
     }
@@ -1445,7 +1464,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   const int ring = (C::RING_BYTES - (SHAPE == SPLIT_TILES ? parts_bytes(kp.splits, bn) : 0)) / kp.stage_bytes;
   kp.stages = ring < MAX_STAGES ? ring : MAX_STAGES;
   const int m_tiles = (a->M + 2 * BM - 1) / (2 * BM), n_cols = (a->N + bn - 1) / bn;
-  kp.narrow = SHAPE == PLAIN_TILES && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
+  kp.narrow = (SHAPE == PLAIN_TILES || SHAPE == SHORT_TILES) && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
   kp.n_main = n_cols - kp.narrow;
   if (MODE == FAAR_GEMM_BWD) {
     // the widest unit at which the Round Loss field holds one per weight of the tiles (half tiles counted as whole: twice
