@@ -49,8 +49,8 @@ constexpr int FIN_COUNT_BITS = 9;              // CTAs of a launch: below 512
 // The tile width bn (accumulator columns, a multiple of 16 up to 256) is a launch parameter chosen by
 // the host (pick_bn).  Shared memory and tensor memory are laid out for the widest tile.
 constexpr int BN_MAX = 256;
-// WIDE: the pair's tile is 256 x 512, the whole of tensor memory as ONE accumulator (two column halves of 256,
-// each fed by its own MMA from the same A stage).  A stage then holds this CTA's 128 rows of both B halves.
+// WIDE: the pair's tile is 256 x (257 .. 512), the whole of tensor memory as ONE accumulator (column halves of 256 and of
+// the rest, each fed by its own MMA from the same A stage).  A stage then holds this CTA's rows of both B halves.
 // Per flop the tile pulls a quarter less operand data through the SM than a 256 x 256 tile, which is what
 // bounds these kernels; the price is that the epilogue of a tile no longer overlaps the next tile's main loop
 // (the two halves drain one after the other while the issuer waits).
@@ -339,7 +339,8 @@ struct KParams {
   int bn;                 // tile width
   int stages, stage_bytes;   // ring depth, bytes of a stage (both CTAs alike)
   int splits;             // CTA pairs that share a tile's contraction: 1, or 2 / 4 (one tile per cluster then)
-  int n_main;             // tile columns of bn; a last column with at most bn/2 columns of the matrix (narrow) is extra
+  int n_main;             // WIDE: columns of the second accumulator half (the first has 256); otherwise
+                          // tile columns of bn; a last column with at most bn/2 columns of the matrix (narrow) is extra
   int narrow;             // 1: there is such a column; its tiles are bn/2 wide
   int n_full;             // the first n_full tiles of the main columns are bn wide, the others come as two halves (tail split)
   uint32_t* status;
@@ -551,6 +552,12 @@ __device__ __forceinline__ void load_yref(const KParams& p, int o, int t0, uint3
     for (int j = 0; j < 16; ++j)
       if (t0 + j < p.N) asm volatile("ld.global.b32 %0, [%1];" : "=r"(yr[j]) : "l"(y + (long long)(t0 + j) * p.ldy + o));
   }
+}
+// 16 of a lane's target values as BF16 pairs (transposed target): columns 16 q .. of `columns` from n_first on
+__device__ __forceinline__ void request_yref(const KParams& p, int o, int n_first, int q, int columns, uint4 (&y)[16]) {
+  if (o >= p.M || 16 * q >= columns) return;
+  const uint4* y4 = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.Yref) + (long long)o * p.ldy + n_first);
+  y[2 * q] = y4[2 * q]; y[2 * q + 1] = y4[2 * q + 1];
 }
 // the same as numbers (columns beyond the matrix: anything)
 __device__ __forceinline__ void yref_values(const KParams& p, const uint32_t (&raw)[16], float (&yr)[16]) {
@@ -894,8 +901,9 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int split = SPLIT ? (int)(crank >> 1) : 0;     // this pair's part of the contraction
   const int pair = blockIdx.x / (2 * splits), n_pairs = gridDim.x / (2 * splits);      // (clusters, with splits > 1)
   const int m_tiles = (p.M + 2 * BM - 1) / (2 * BM);
-  // WIDE: tiles of 512 columns, numbered row block fastest; no tail split
-  const int total_tiles = WIDE ? m_tiles * ((p.N + WIDE_BN - 1) / WIDE_BN) : tile_count(p, m_tiles);
+  // WIDE: tiles of 256 + n_main columns, numbered row block fastest; no tail split
+  const int wide_w = BN_MAX + p.n_main;
+  const int total_tiles = WIDE ? m_tiles * ((p.N + wide_w - 1) / wide_w) : tile_count(p, m_tiles);
   const int k_blocks = (p.Kc + BK - 1) / BK;
   const int kb0 = SPLIT ? k_blocks * split / splits : 0, kb1 = SPLIT ? k_blocks * (split + 1) / splits : k_blocks;
   const uint32_t bar_recv = ctl_u32 + 208u, parts = base + (uint32_t)STAGES * STAGE_BYTES;   // SPLIT: see exchange_parts
@@ -933,7 +941,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       bool ok = true;
       auto coords = [&](int tile) {
         TileCoord tc;
-        if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * WIDE_BN; tc.w = BN_MAX; }
+        if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * wide_w; tc.w = BN_MAX; }
         else tc = tile_coord(p, tile, m_tiles);
         return tc;
       };
@@ -948,7 +956,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + C::A_BYTES;
           // the leader's barrier collects the bytes of both CTAs' copies
           if (rank == 0)
-            mbar_expect_tx(full_bar(stage), WIDE ? 2u * (uint32_t)(C::A_BYTES + C::B_BYTES)
+            mbar_expect_tx(full_bar(stage), WIDE ? 2u * (uint32_t)(C::A_BYTES + wide_w / 2 * BK * 2)
                                                  : 2u * (uint32_t)(C::A_BYTES + (B_MN ? mn_boxes(tc.w / 2) * MN_BOX : tc.w / 2) * BK * 2));
           const uint32_t leader_full = map_to_cta(full_bar(stage), leader);
           if (A_MN) {                                          // two boxes of 64 rows of A, each [64 k][64 m]
@@ -964,7 +972,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             tma_load_2d(sb, mapB, kb * BK, n0, leader_full, keep);
           }
           // second column half (rows beyond the matrix arrive as zeros)
-          if (WIDE) tma_load_2d(sb + C::BH_BYTES, &tmB, kb * BK, n0 + BN_MAX, leader_full, keep);
+          if (WIDE) tma_load_2d(sb + C::BH_BYTES, &tmBh, kb * BK, tc.n0 + BN_MAX + (int)rank * (p.n_main / 2), leader_full, keep);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
@@ -1003,6 +1011,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (!ok) break;
         tc_fence_after();
         const uint32_t tmem_d = tmem_base + acc * BN_MAX;
+        const uint32_t idesc1 = WIDE ? make_idesc(p.n_main) : 0u;
         const uint32_t idesc = make_idesc(WIDE ? BN_MAX : tile_coord(p, tile, m_tiles).w, A_MN ? 1 : 0, B_MN ? 1 : 0);
         for (int kb = kb0; kb < kb1; ++kb) {
           ok = __all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, ac, 0x300u | stage));
@@ -1019,7 +1028,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               // (MN-major: 16 rows of 128 bytes further on)
               tc_mma_bf16(tmem_d, da + ka * k, db + kbs * k, idesc, (SPLIT ? kb != kb0 || k != 0 : (kb | k) != 0) ? 1u : 0u);
               if (WIDE)
-                tc_mma_bf16(tmem_d + BN_MAX, da + 2u * k, make_smem_desc(sb + C::BH_BYTES) + 2u * k, idesc,
+                tc_mma_bf16(tmem_d + BN_MAX, da + 2u * k, make_smem_desc(sb + C::BH_BYTES) + 2u * k, idesc1,
                             (SPLIT ? kb != kb0 || k != 0 : (kb | k) != 0) ? 1u : 0u);
             }
             tc_commit_pair(empty_bar(stage), leader);          // frees this stage in both CTAs
@@ -1048,6 +1057,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     bool row_ok = false;
     const bool yvec_ok = MODE == FAAR_GEMM_FWD && p.yref_t && p.yref_dtype == FAAR_BF16 && p.Yout == nullptr;
     bool dead = false;
+    uint4 ywide[MODE == FAAR_GEMM_FWD && WIDE ? 16 : 1];
     // One pass per accumulator buffer that fills: a tile, or (WIDE) a 256-column half of a tile.
     int vt = 0;
     for (;; ++vt) {
@@ -1059,7 +1069,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       // whether a later tile takes this accumulator buffer: else nobody waits for its release
       const bool again = tile + (WIDE ? 1 : 2) * n_pairs < total_tiles;
       TileCoord tc;
-      if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * WIDE_BN + acc * BN_MAX; tc.w = BN_MAX; }
+      if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * wide_w + acc * BN_MAX; tc.w = acc ? p.n_main : BN_MAX; }
       else tc = tile_coord(p, tile, m_tiles);
       // the columns of the tile that this pair finishes: with a split contraction its share
       const int share0 = SPLIT ? share_begin(tc.w, splits, split) : 0;
@@ -1072,7 +1082,12 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       // 16-byte loads) are requested before the wait for the accumulator, so their latency lies under the main loop
       const bool yvec = yvec_ok && n0 + col_end <= p.N;
       uint4 yraw[MODE == FAAR_GEMM_FWD ? 16 : 1];
-      if constexpr (MODE == FAAR_GEMM_FWD) {
+      if constexpr (MODE == FAAR_GEMM_FWD && WIDE) {
+        if (yvec && acc == 0) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) request_yref(p, o, n0 + col_begin, q, col_end - col_begin, ywide);
+        }
+      } else if constexpr (MODE == FAAR_GEMM_FWD) {
         static_assert(BN_MAX / C::COL_GROUPS == 128, "a warp's columns of the widest tile");
         if (yvec && o < p.M) {
           const uint4* y4 = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.Yref) +
@@ -1164,7 +1179,14 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               uint32_t r[16];
               tmem_ld16(trow + (uint32_t)c, r);
               tmem_ld_wait();
-              warp_acc += epi_fwd_vec(p, o, n0 + c, r, yraw[2 * q], yraw[2 * q + 1]);
+              if constexpr (WIDE) warp_acc += epi_fwd_vec(p, o, n0 + c, r, ywide[2 * q], ywide[2 * q + 1]);
+              else warp_acc += epi_fwd_vec(p, o, n0 + c, r, yraw[2 * q], yraw[2 * q + 1]);
+            }
+            if constexpr (MODE == FAAR_GEMM_FWD && WIDE) {
+              // the second half's values, as the registers of the first half's come free: asked for after the first half's
+              // stores they took 6 k clocks
+              const int w2 = (p.n_main / C::COL_GROUPS + 15) / 16 * 16, begin2 = cg * w2, end2 = min(begin2 + w2, p.n_main);
+              if (acc == 0 && tc.n0 + BN_MAX + end2 <= p.N) request_yref(p, o, tc.n0 + BN_MAX + begin2, q, end2 - begin2, ywide);
             }
           }
         } else {
@@ -1431,19 +1453,27 @@ int pick_full(faar_ctx* ctx, int mode, int m_tiles, int n_main, int narrow, int 
   return best_full;
 }
 
-// Whether a launch takes 256 x 512 tiles (see Cfg): on request (ctx->tune_wide == 1) wherever the shape allows.  They move a
-// quarter less operand data, but nothing overlaps their epilogue, and they give a wave of tiles no halves to even it out.
-// Plain product of 256-wide tiles -> 512-wide, us: 80 tiles (40 wide ones) over 2048 21.6 -> 30.0; 128 over 2048 34.0 -> 38.4,
-// over 4096 58.0 -> 62.4, over 8192 97 -> 99; 144 over 8192 101.3 -> 100.8; forward kernel and soft weights of 2048 x 4096 at
-// 4096 tokens 72.3 -> 74.2, with an FP32 target of 2048 x 8192 152 -> 164.  By themselves therefore only for a forward product
-// with a transposed BF16 target and 8192 or more contraction elements, where they take one wave that fills six of seven CTA
-// pairs: step of 2048 x 8192 at 4096 tokens 303 -> 298, its operands coming from HBM.
-bool pick_wide(const faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int pairs, bool fwd_vec) {
-  if (bn != BN_MAX || ctx->tune_wide == 0) return false;
-  if (ctx->tune_wide == 1) return (mode == FAAR_GEMM_REF && M > N ? M : N) > BN_MAX;    // REF may have either index as its rows
-  const long long wide = (long long)((M + 2 * BM - 1) / (2 * BM)) * ((N + WIDE_BN - 1) / WIDE_BN);
-  return mode == FAAR_GEMM_FWD && fwd_vec && k_blocks >= 128 && N > BN_MAX && ctx->tune_tail < 0 && ctx->tune_bn == 0 && wide <= pairs &&
-         7 * wide >= 6 * pairs;
+// The width of a launch's 256 x (257 .. 512) tiles (see Cfg), 0 for none.  512 on request (ctx->tune_wide == 1) wherever the
+// shape allows.  They move up to a quarter less operand data, but nothing overlaps their epilogue, and they give a wave of tiles no
+// halves to even it out.  Plain product of 256-wide tiles -> 512-wide, us: 80 tiles (40 wide ones) over 2048 21.6 -> 30.0; 128
+// over 2048 34.0 -> 38.4, over 4096 58.0 -> 62.4, over 8192 97 -> 99; 144 over 8192 101.3 -> 100.8; forward kernel and soft
+// weights of 2048 x 4096 at 4096 tokens 72.3 -> 74.2, with an FP32 target of 2048 x 8192 152 -> 164.  By themselves therefore
+// only for a forward product with a transposed BF16 target and 8192 or more contraction elements, where the least width
+// that gives one wave (a multiple of 16) is at most 512 and takes less main loop than the waves of 256-wide tiles.  Forward
+// kernel and soft weights of 2048 x 8192, us: 4096 tokens (512 -> 464 columns, 64 -> 72 of 74 pairs) 118 -> 112, 2500 tokens (256 ->
+// 288) 98.2 -> 86.0.
+int pick_wide(faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int pairs, bool fwd_vec) {
+  if (bn != BN_MAX || ctx->tune_wide == 0) return 0;
+  if (ctx->tune_wide == 1) return (mode == FAAR_GEMM_REF && M > N ? M : N) > BN_MAX ? WIDE_BN : 0;    // REF may have either index as its rows
+  if (mode != FAAR_GEMM_FWD || !fwd_vec || k_blocks < 128 || N <= BN_MAX || ctx->tune_tail >= 0 || ctx->tune_bn != 0) return 0;
+  const int m_tiles = (M + 2 * BM - 1) / (2 * BM), cols = pairs / m_tiles;
+  if (cols == 0) return 0;
+  const int w = ((N + cols - 1) / cols + 15) / 16 * 16;
+  if (w <= BN_MAX || w > WIDE_BN) return 0;
+  // 256-wide tiles: whole waves, and a last one of up to half the pairs cut into half tiles, which cost 0.75 (pick_full)
+  const int tiles = m_tiles * ((N + BN_MAX - 1) / BN_MAX), rest = tiles % pairs;
+  const double plain = tiles / pairs + (rest == 0 ? 0.0 : (2 * rest <= pairs ? 0.75 : 1.0));
+  return w <= plain * BN_MAX ? w : 0;
 }
 
 template <int MODE, int OPT, int SHAPE, int MN>
@@ -1464,12 +1494,13 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   const int ring = (C::RING_BYTES - (SHAPE == SPLIT_TILES ? parts_bytes(kp.splits, bn) : 0)) / kp.stage_bytes;
   kp.stages = ring < MAX_STAGES ? ring : MAX_STAGES;
   const int m_tiles = (a->M + 2 * BM - 1) / (2 * BM), n_cols = (a->N + bn - 1) / bn;
+  const int wide_w1 = kp.n_main, wide_w = BN_MAX + wide_w1, wide_cols = (a->N + wide_w - 1) / wide_w;
   kp.narrow = (SHAPE == PLAIN_TILES || SHAPE == SHORT_TILES) && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
-  kp.n_main = n_cols - kp.narrow;
+  kp.n_main = WIDE ? wide_w1 : n_cols - kp.narrow;
   if (MODE == FAAR_GEMM_BWD) {
     // the widest unit at which the Round Loss field holds one per weight of the tiles (half tiles counted as whole: twice
     // that) with its sign
-    const long long area = (long long)m_tiles * 2 * BM * (WIDE ? (a->N + WIDE_BN - 1) / WIDE_BN * (long long)WIDE_BN : (long long)n_cols * bn);
+    const long long area = (long long)m_tiles * 2 * BM * (WIDE ? wide_cols * (long long)wide_w : (long long)n_cols * bn);
     int int_bits = 1;
     while (area >> int_bits) ++int_bits;
     kp.fin_unit = ldexp(1.0, 62 - 2 * FIN_COUNT_BITS - int_bits); kp.fin_inv_unit = 1.0 / kp.fin_unit;
@@ -1484,16 +1515,17 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   } else {
     e = make_map(ctx, &tmB, a->B, a->N, a->Kc, a->ldb, bn / 2);
     if (e) return e;
-    if (kp.narrow || kp.n_full < m_tiles * kp.n_main) e = make_map(ctx, &tmBh, a->B, a->N, a->Kc, a->ldb, bn % 32 == 0 ? bn / 4 : bn / 2);   // half-width tiles
+    if (WIDE) e = make_map(ctx, &tmBh, a->B, a->N, a->Kc, a->ldb, wide_w1 / 2);           // the second half's
+    else if (kp.narrow || kp.n_full < m_tiles * kp.n_main) e = make_map(ctx, &tmBh, a->B, a->N, a->Kc, a->ldb, bn % 32 == 0 ? bn / 4 : bn / 2);   // half-width tiles
     else tmBh = tmB;
   }
   if (e) return e;
-  const long long tiles = WIDE ? (long long)m_tiles * ((a->N + WIDE_BN - 1) / WIDE_BN)
+  const long long tiles = WIDE ? (long long)m_tiles * wide_cols
                                : 2ll * m_tiles * kp.n_main - kp.n_full + (kp.narrow ? m_tiles : 0);
   const int pairs = SHAPE == SPLIT_TILES ? (int)tiles * kp.splits : (int)(tiles < max_pairs ? tiles : max_pairs);
   cfg.gridDim = dim3(2 * pairs, 1, 1);
   if (n_partials_out) *n_partials_out = 2 * pairs * C::EPI_WARPS;
-  ctx->last_gemm_bn = WIDE ? WIDE_BN : bn;
+  ctx->last_gemm_bn = WIDE ? WIDE_BN : bn;                   // (the form; a tile may have fewer columns)
   ctx->last_gemm_pairs = pairs;
   // in columns' worth of tiles
   ctx->last_gemm_split = WIDE ? 0 : kp.narrow + (m_tiles * kp.n_main - kp.n_full + m_tiles - 1) / m_tiles;
@@ -1552,12 +1584,14 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
   const bool fwd_vec = a->yref_t && a->yref_dtype == FAAR_BF16 && !a->Yout;
   int bn = pick_bn(ctx, MODE, a->M, a->N, k_blocks, max_pairs, a->b_mn != 0, fwd_vec);
   if (kp.splits > 1 && ctx->tune_bn == 0) bn = split_bn;
+  const int wide = pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs, fwd_vec);
+  kp.n_main = wide > BN_MAX ? wide - BN_MAX : BN_MAX;
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
   // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient; A, if the
   // accumulator's rows are the result's columns), the dW product with B or with both untransposed
   if constexpr (MODE == FAAR_GEMM_REF) {
     if (kp.columns && mn == 0) {
-      if (kp.splits == 1 && pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs, fwd_vec))
+      if (kp.splits == 1 && wide)
         return launch_variant<MODE, OPT, WIDE_TILES, 4>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
       return launch_tiles<MODE, OPT, 4>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
     }
@@ -1568,7 +1602,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
     if (mn == 3) return launch_tiles<MODE, OPT, 3>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   }
   if (mn != 0) return (int)cudaErrorInvalidValue;
-  if (kp.splits == 1 && pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs, fwd_vec))
+  if (kp.splits == 1 && wide)
     return launch_variant<MODE, OPT, WIDE_TILES, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   return launch_tiles<MODE, OPT, 0>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
 }
