@@ -67,12 +67,17 @@ constexpr int WIDE_BN = 2 * BN_MAX;
 // take 91.8, with 8 at a time but no carve-out 97.6; without another stage (92 KB of L1) nothing changes but 2000 tokens, 148.
 // Above SHORT_BLOCKS the main loop needs the stage: operands and state together then take all the 64 bytes a clock that an
 // SM draws from L2.
-constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2, SHORT_TILES = 3;
+//
+// SPLIT_NARROW: a split contraction that leaves a CTA at most 32 columns to finish, of a dW launch.  The lanes of its epilogue then
+// cover 16 or 32 columns of a row instead of 64, most of which there would be none of: a small layer's epilogue executed the
+// instructions of four times its weights.  Step of 128 x 256 at 1024 tokens (16 columns) 14.7 -> 13.6 us.  (As a choice inside
+// SPLIT_TILES it cost shares of 64 columns 2 %.)
+constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2, SHORT_TILES = 3, SPLIT_NARROW = 4;
 constexpr int SHORT_BLOCKS = 40;
 constexpr int SHORT_SMEM = 387 * 512;          // with the system's 1 KB below the 196 KB carve-out
 constexpr int SHORT_CARVEOUT = 85;             // percent of the 228 KB: 196 KB
 template <int MODE, int SHAPE = PLAIN_TILES> struct Cfg {
-  static constexpr bool WIDE = SHAPE == WIDE_TILES, SHORT = SHAPE == SHORT_TILES;
+  static constexpr bool WIDE = SHAPE == WIDE_TILES, SHORT = SHAPE == SHORT_TILES, SPLIT = SHAPE == SPLIT_TILES || SHAPE == SPLIT_NARROW;
   static constexpr int EPI_WARPS = MODE == FAAR_GEMM_BWD ? 16 : 8;
   static constexpr int THREADS = 32 * (2 + EPI_WARPS);
   static constexpr int A_BYTES = BM * BK * 2;
@@ -668,7 +673,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
 
 // The four epilogue warps that share a TMEM lane quarter stage a 32-row x PW-column panel of G in
 // shared memory (row r at panel + 4 PW r, its 16-byte units swizzled: panel_unit); then warp `sub`
-// of the quarter takes rows 8 sub .. 8 sub + 7, LPR = PW / LW lanes per row and lane l the columns
+// of the quarter takes rows 8 sub .. 8 sub + 7, LPR = PX / LW lanes per row and lane l the columns
 // LW (l % LPR) and on, so that one warp instruction moves 128 LW bytes of V / m / u as 32 / LPR row pieces of
 // 4 PW contiguous bytes each: whole lines as 16- or 32-byte vectors.  (A panel of 128 columns gives one 512-byte
 // piece per instruction but leaves room for five TMA stages only; the sixth stage is worth more.)
@@ -678,7 +683,8 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // o_first: output feature of panel row 0; k_first: input feature of panel column 0; k_end: first
 // input feature beyond the tile (or the matrix).
 // Returns the Round Loss contribution of the pre-update v's.
-// LW is 4, or 8 in launches of short contractions (Cfg::LANE_WEIGHTS).
+// LW is 4, or 8 in launches of short contractions (Cfg::LANE_WEIGHTS); PX the columns that the lanes of a row cover: PW, or 16
+// or 32 (SPLIT_NARROW).
 // 16-byte unit `u` of row `row` of a panel: the row moves its units around so that a column of rows does not collide, and with
 // eight columns a lane even units lie in a row's first half, odd ones in its second, so that its lanes read consecutive units.
 template <int LW> __device__ __forceinline__ uint32_t panel_unit(uint32_t panel, int row, int u) {
@@ -687,10 +693,10 @@ template <int LW> __device__ __forceinline__ uint32_t panel_unit(uint32_t panel,
 template <int LW> struct RowState { float v[LW], m[LW], u[LW]; uint32_t cw, sb; };
 // State of this lane's LW weights of instruction `it` of the panel whose row 0 / column 0 is (o_first, k_first), or
 // nothing if they lie outside the matrix or at or beyond column k_end.
-template <int OPT, int LW>
+template <int OPT, int LW, int PX>
 __device__ __forceinline__ bool load_row_state(const KParams& p, const Segment& g, int lane, int sub, int o_first, int k_first, int k_end, int it,
                                                uint64_t stream, RowState<LW>& st) {
-  constexpr int LPR = PW / LW, RPI = 32 / LPR;                     // lanes per panel row; rows per warp instruction
+  constexpr int LPR = PX / LW, RPI = 32 / LPR;                     // lanes per panel row; rows per warp instruction
   const int row = o_first + 8 * sub + lane / LPR + RPI * it, col = k_first + LW * (lane % LPR);
   const bool ok = row < p.M && col < k_end;
   if (ok) {
@@ -708,10 +714,10 @@ __device__ __forceinline__ bool load_row_state(const KParams& p, const Segment& 
 }
 // `st` / `st_ok` hold the state of instruction 0 on entry; on return those of instruction 0 of the panel at column
 // k_next (unless k_next >= k_end).
-template <int OPT, int LW>
+template <int OPT, int LW, int PX>
 __device__ __forceinline__ float epi_bwd_rows(const KParams& p, const Segment& sg, uint32_t panel, int lane, int sub, int o_first,
                                               int k_first, int k_next, int k_end, float s_global, RowState<LW>& st, bool& st_ok) {
-  constexpr int LPR = PW / LW, RPI = 32 / LPR, ITS = 8 / RPI;      // ITS: instructions per warp and panel
+  constexpr int LPR = PX / LW, RPI = 32 / LPR, ITS = 8 / RPI;      // ITS: instructions per warp and panel
   const int cu = lane % LPR;                                       // LW columns of the row
   const int r0 = 8 * sub + lane / LPR;                             // this lane's row in the first instruction
   const long long e0 = (long long)(o_first + r0) * p.N + k_first + LW * cu;        // row r0 element of this lane
@@ -722,8 +728,8 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, const Segment& s
   for (int it = 0; it < ITS; ++it) {
     RowState<LW> cur = st;
     const bool ok = st_ok;
-    st_ok = it + 1 < ITS ? load_row_state<OPT>(p, sg, lane, sub, o_first, k_first, k_end, it + 1, stream, st)
-                         : load_row_state<OPT>(p, sg, lane, sub, o_first, k_next, k_end, 0, stream, st);
+    st_ok = it + 1 < ITS ? load_row_state<OPT, LW, PX>(p, sg, lane, sub, o_first, k_first, k_end, it + 1, stream, st)
+                         : load_row_state<OPT, LW, PX>(p, sg, lane, sub, o_first, k_next, k_end, 0, stream, st);
     if (!ok) continue;
     const int row = r0 + RPI * it;
     const long long e = e0 + (long long)(RPI * it) * p.N;
@@ -808,7 +814,8 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, const Segment& s
 // share_begin(w, splits, d) on.  What arrives from the other pairs lies behind the operand ring as
 // [part][4 columns][row] of 16 bytes: a warp, one row per lane, reads and writes consecutive 16-byte units.
 __host__ __device__ constexpr int share_begin(int w, int splits, int d) { return 16 * ((w / 16) * d / splits); }
-constexpr int parts_bytes(int splits, int w) { return (splits - 1) * 16 * ((w / 16 + splits - 1) / splits) * BM * 4; }     // the largest share
+constexpr int largest_share(int w, int splits) { return 16 * ((w / 16 + splits - 1) / splits); }
+constexpr int parts_bytes(int splits, int w) { return (splits - 1) * largest_share(w, splits) * BM * 4; }
 __device__ __forceinline__ uint32_t part_unit(uint32_t parts, int slot, int cols, int unit, int row) {
   return parts + (uint32_t)(((slot * (cols >> 2) + unit) * BM + row) << 4);
 }
@@ -862,13 +869,13 @@ __device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t parts, int
 // MN: bit 0 = the A operand, bit 1 = the B operand is stored with its M / N index contiguous (KParams.a_mn / b_mn);
 // a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.  Bit 2 (REF): the
 // accumulator's rows are the result's columns; compiled in as well (as a branch it cost 0.1 us in every small product).
-// SHAPE: PLAIN_TILES, WIDE_TILES, SPLIT_TILES, SHORT_TILES (see Cfg).
+// SHAPE: one of the tile forms (see Cfg).
 constexpr int MIN_SPLIT_BLOCKS = 12;            // contractions of fewer k blocks stay whole (see pick_splits)
 template <int MODE, int OPT, int SHAPE, int MN>
 __global__ void __launch_bounds__(Cfg<MODE, SHAPE>::THREADS, 1)
 faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ KParams p) {
-  constexpr bool WIDE = SHAPE == WIDE_TILES, SPLIT = SHAPE == SPLIT_TILES;
+  constexpr bool WIDE = SHAPE == WIDE_TILES, SPLIT = Cfg<MODE, SHAPE>::SPLIT;
   using C = Cfg<MODE, SHAPE>;
   constexpr int LW = C::LANE_WEIGHTS;
   constexpr bool A_MN = (MN & 1) != 0, B_MN = (MN & 2) != 0, COLUMNS = (MN & 4) != 0;
@@ -1111,7 +1118,12 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const Segment& seg = p.seg[MODE == FAAR_GEMM_BWD && MN == 3 ? (o_warp >= p.seg_end[0]) + (o_warp >= p.seg_end[1]) : 0];
       if constexpr (MODE == FAAR_GEMM_BWD) {
         if (MN == 3) s_global = *seg.s_global;
-        row_ok = load_row_state<OPT>(p, seg, lane, ew >> 2, m0 + quarter * 32, n0, k_end, 0, l2_policy_stream(), row_state);
+        const int o0 = m0 + quarter * 32;
+        if constexpr (SHAPE == SPLIT_NARROW)
+          row_ok = TW <= 16 ? load_row_state<OPT, LW, 16>(p, seg, lane, ew >> 2, o0, n0, k_end, 0, l2_policy_stream(), row_state)
+                            : load_row_state<OPT, LW, 32>(p, seg, lane, ew >> 2, o0, n0, k_end, 0, l2_policy_stream(), row_state);
+        else
+          row_ok = load_row_state<OPT, LW, PW>(p, seg, lane, ew >> 2, o0, n0, k_end, 0, l2_policy_stream(), row_state);
       }
       bool ok = mbar_wait(tfull_bar(acc), acc_phase, ac, 0x400u | acc);
       ok = __all_sync(0xffffffffu, ok);
@@ -1158,7 +1170,12 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
           okp = mbar_wait(pfull, pn & 1u, ac, 0x600u | quarter);
           if (!__all_sync(0xffffffffu, okp)) { dead = true; break; }
-          warp_acc += epi_bwd_rows<OPT>(p, seg, panel, lane, sub, o_first, n0 + pc, n0 + pc + PW, k_end, s_global, row_state, row_ok);
+          const int k0 = n0 + pc, k1 = k0 + PW;            // SPLIT_NARROW: one panel
+          if constexpr (SHAPE == SPLIT_NARROW)
+            warp_acc += TW <= 16 ? epi_bwd_rows<OPT, LW, 16>(p, seg, panel, lane, sub, o_first, k0, k1, k_end, s_global, row_state, row_ok)
+                                 : epi_bwd_rows<OPT, LW, 32>(p, seg, panel, lane, sub, o_first, k0, k1, k_end, s_global, row_state, row_ok);
+          else
+            warp_acc += epi_bwd_rows<OPT, LW, PW>(p, seg, panel, lane, sub, o_first, k0, k1, k_end, s_global, row_state, row_ok);
           __syncwarp();
           if (lane == 0) mbar_arrive(pdone);
           ++pn;
@@ -1479,8 +1496,8 @@ int pick_wide(faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int p
 template <int MODE, int OPT, int SHAPE, int MN>
 int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_out, int bn, int max_pairs,
                    const cudaLaunchConfig_t& base_cfg) {
-  constexpr bool WIDE = SHAPE == WIDE_TILES;
   using C = Cfg<MODE, SHAPE>;
+  constexpr bool WIDE = C::WIDE, SPLIT = C::SPLIT;
   static_assert(C::MIN_STAGES >= 3, "ring too short");
   static_assert(C::SMEM_BYTES <= SMEM_LIMIT, "shared memory budget");
   static_assert(C::EPI_WARPS <= MAX_EPI_WARPS, "partials budget");
@@ -1491,7 +1508,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   cfg.dynamicSmemBytes = C::SMEM_BYTES;
   kp.bn = bn;
   kp.stage_bytes = WIDE ? C::STAGE_BYTES : C::A_BYTES + (a->b_mn ? mn_boxes(bn / 2) * MN_BOX_BYTES : (int)faar_align_up((size_t)(bn / 2) * BK * 2, 1024));   // whole swizzle atoms
-  const int ring = (C::RING_BYTES - (SHAPE == SPLIT_TILES ? parts_bytes(kp.splits, bn) : 0)) / kp.stage_bytes;
+  const int ring = (C::RING_BYTES - (SPLIT ? parts_bytes(kp.splits, bn) : 0)) / kp.stage_bytes;
   kp.stages = ring < MAX_STAGES ? ring : MAX_STAGES;
   const int m_tiles = (a->M + 2 * BM - 1) / (2 * BM), n_cols = (a->N + bn - 1) / bn;
   const int wide_w1 = kp.n_main, wide_w = BN_MAX + wide_w1, wide_cols = (a->N + wide_w - 1) / wide_w;
@@ -1505,7 +1522,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
     while (area >> int_bits) ++int_bits;
     kp.fin_unit = ldexp(1.0, 62 - 2 * FIN_COUNT_BITS - int_bits); kp.fin_inv_unit = 1.0 / kp.fin_unit;
   }
-  kp.n_full = WIDE ? 0 : (SHAPE == SPLIT_TILES ? m_tiles * kp.n_main : pick_full(ctx, MODE, m_tiles, kp.n_main, kp.narrow, bn, max_pairs));
+  kp.n_full = WIDE ? 0 : (SPLIT ? m_tiles * kp.n_main : pick_full(ctx, MODE, m_tiles, kp.n_main, kp.narrow, bn, max_pairs));
   CUtensorMap tmA, tmB, tmBh;
   e = a->a_mn ? make_map_mn(ctx, &tmA, a->A, a->Kc, a->M, a->lda) : make_map(ctx, &tmA, a->A, a->M, a->Kc, a->lda, BM);
   if (e) return e;
@@ -1522,7 +1539,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   if (e) return e;
   const long long tiles = WIDE ? (long long)m_tiles * wide_cols
                                : 2ll * m_tiles * kp.n_main - kp.n_full + (kp.narrow ? m_tiles : 0);
-  const int pairs = SHAPE == SPLIT_TILES ? (int)tiles * kp.splits : (int)(tiles < max_pairs ? tiles : max_pairs);
+  const int pairs = SPLIT ? (int)tiles * kp.splits : (int)(tiles < max_pairs ? tiles : max_pairs);
   cfg.gridDim = dim3(2 * pairs, 1, 1);
   if (n_partials_out) *n_partials_out = 2 * pairs * C::EPI_WARPS;
   ctx->last_gemm_bn = WIDE ? WIDE_BN : bn;                   // (the form; a tile may have fewer columns)
@@ -1538,6 +1555,10 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
 template <int MODE, int OPT, int MN>
 int launch_tiles(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_out, int bn, int max_pairs, const cudaLaunchConfig_t& cfg) {
   if constexpr (MODE != FAAR_GEMM_FWD) {
+    if constexpr (MODE == FAAR_GEMM_BWD) {
+      if (kp.splits > 1 && largest_share(bn, kp.splits) <= 32)
+        return launch_variant<MODE, OPT, SPLIT_NARROW, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+    }
     if (kp.splits > 1) return launch_variant<MODE, OPT, SPLIT_TILES, MN>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   }
   if constexpr (MODE == FAAR_GEMM_BWD) {
