@@ -49,12 +49,13 @@ constexpr int FIN_COUNT_BITS = 9;              // CTAs of a launch: below 512
 // The tile width bn (accumulator columns, a multiple of 16 up to 256) is a launch parameter chosen by
 // the host (pick_bn).  Shared memory and tensor memory are laid out for the widest tile.
 constexpr int BN_MAX = 256;
-// WIDE: the pair's tile is 256 x (257 .. 512), the whole of tensor memory as ONE accumulator (column halves of 256 and of
-// the rest, each fed by its own MMA from the same A stage).  A stage then holds this CTA's rows of both B halves.
+// WIDE: the pair's tile is 256 x (288 .. 512), the whole of tensor memory as ONE accumulator (column halves of 256 and of
+// the rest, at least 32, each fed by its own MMA from the same A stage).  A stage then holds this CTA's rows of both B halves.
 // Per flop the tile pulls a quarter less operand data through the SM than a 256 x 256 tile, which is what
 // bounds these kernels; the price is that the epilogue of a tile no longer overlaps the next tile's main loop
 // (the two halves drain one after the other while the issuer waits).
 constexpr int WIDE_BN = 2 * BN_MAX;
+constexpr int WIDE_BN_MIN = BN_MAX + 32;       // no other launch gives a pair of CTAs an MMA of fewer than 32 columns either
 // The tile forms of a launch, chosen at compile time (as run-time options of one kernel they cost the others time): tiles of
 // up to 256 columns, 256 x 512, a contraction split over the pairs of a cluster, or (BWD) 256-wide tiles of a short contraction.
 //
@@ -1470,7 +1471,7 @@ int pick_full(faar_ctx* ctx, int mode, int m_tiles, int n_main, int narrow, int 
   return best_full;
 }
 
-// The width of a launch's 256 x (257 .. 512) tiles (see Cfg), 0 for none.  512 on request (ctx->tune_wide == 1) wherever the
+// The width of a launch's 256 x (288 .. 512) tiles (see Cfg), 0 for none.  512 on request (ctx->tune_wide == 1) wherever the
 // shape allows.  They move up to a quarter less operand data, but nothing overlaps their epilogue, and they give a wave of tiles no
 // halves to even it out.  Plain product of 256-wide tiles -> 512-wide, us: 80 tiles (40 wide ones) over 2048 21.6 -> 30.0; 128
 // over 2048 34.0 -> 38.4, over 4096 58.0 -> 62.4, over 8192 97 -> 99; 144 over 8192 101.3 -> 100.8; forward kernel and soft
@@ -1485,8 +1486,9 @@ int pick_wide(faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int p
   if (mode != FAAR_GEMM_FWD || !fwd_vec || k_blocks < 128 || N <= BN_MAX || ctx->tune_tail >= 0 || ctx->tune_bn != 0) return 0;
   const int m_tiles = (M + 2 * BM - 1) / (2 * BM), cols = pairs / m_tiles;
   if (cols == 0) return 0;
-  const int w = ((N + cols - 1) / cols + 15) / 16 * 16;
+  int w = ((N + cols - 1) / cols + 15) / 16 * 16;
   if (w <= BN_MAX || w > WIDE_BN) return 0;
+  if (w < WIDE_BN_MIN) w = WIDE_BN_MIN;
   // 256-wide tiles: whole waves, and a last one of up to half the pairs cut into half tiles, which cost 0.75 (pick_full)
   const int tiles = m_tiles * ((N + BN_MAX - 1) / BN_MAX), rest = tiles % pairs;
   const double plain = tiles / pairs + (rest == 0 ? 0.0 : (2 * rest <= pairs ? 0.75 : 1.0));

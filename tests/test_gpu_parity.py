@@ -1089,11 +1089,15 @@ def test_chaining_arguments_are_checked(ctx):
 
 
 # ---- which kernel form a launch takes ---------------------------------------------------------------------------
-@pytest.mark.parametrize("O,K,T,auto", [(2048, 4096, 2560, 256), (2000, 4096, 2570, 256), (2000, 8192, 4090, 512)])
-def test_wide_tiles_give_the_same_bits_and_are_taken_where_they_fill_a_wave(ctx, O, K, T, auto):
-    """80 tiles of 256 x 256 are two waves of the CTA pairs, 40 of 256 x 512 one, which takes longer all the same; 64 of
-    those with a long contraction the forward product takes by itself.  Every output element is the same sum in the same
-    order."""
+@pytest.mark.parametrize("O,K,T,auto,pairs", [
+    (2048, 4096, 2560, 256, 74), (2000, 4096, 2570, 256, 74),
+    (2000, 8192, 4090, 512, 72),       # 464 columns: 9 x 8 tiles
+    (1500, 8192, 3100, 512, 66),       # 259 columns would do for 12 x 6 tiles; the narrowest form has 288: 11 x 6
+])
+def test_wide_tiles_give_the_same_bits_and_are_taken_where_they_fill_a_wave(ctx, O, K, T, auto, pairs):
+    """80 tiles of 256 x 256 are two waves of the CTA pairs, 40 of 256 x 512 one, which takes longer all the same; with a long
+    contraction the forward product takes tiles of the least width, from 288 columns on, that gives one wave.  Every output
+    element is the same sum in the same order.  pairs: on a whole B200."""
     gen = torch.Generator(device=DEV).manual_seed(1)
     T16 = (T + 15) // 16 * 16
     shape = faar.make_shape(O, K, T, ldy=T16, yref_transposed=1)
@@ -1115,6 +1119,7 @@ def test_wide_tiles_give_the_same_bits_and_are_taken_where_they_fill_a_wave(ctx,
             assert faar.last_gemm_config(ctx)[0] == {1: 512, 0: 256, -1: 256}[wide]
             faar.layer_fwd(ctx, shape, hp, X, Yref, V, code, scales, sg, dYt, loss, None, ws)
             assert faar.last_gemm_config(ctx)[0] == {1: 512, 0: 256, -1: auto}[wide]
+            assert wide >= 0 or faar.last_gemm_config(ctx)[1] == pairs
             out.append((Y[:, :T].clone(), dYt[:, :T].clone()))
     finally:
         faar.tune_wide_tiles(ctx, -1)
