@@ -559,12 +559,6 @@ __device__ __forceinline__ void load_yref(const KParams& p, int o, int t0, uint3
       if (t0 + j < p.N) asm volatile("ld.global.b32 %0, [%1];" : "=r"(yr[j]) : "l"(y + (long long)(t0 + j) * p.ldy + o));
   }
 }
-// 16 of a lane's target values as BF16 pairs (transposed target): columns 16 q .. of `columns` from n_first on
-__device__ __forceinline__ void request_yref(const KParams& p, int o, int n_first, int q, int columns, uint4 (&y)[16]) {
-  if (o >= p.M || 16 * q >= columns) return;
-  const uint4* y4 = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.Yref) + (long long)o * p.ldy + n_first);
-  y[2 * q] = y4[2 * q]; y[2 * q + 1] = y4[2 * q + 1];
-}
 // the same as numbers (columns beyond the matrix: anything)
 __device__ __forceinline__ void yref_values(const KParams& p, const uint32_t (&raw)[16], float (&yr)[16]) {
   const int shift = p.yref_dtype == FAAR_BF16 ? 16 : 0;
@@ -1065,7 +1059,6 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     bool row_ok = false;
     const bool yvec_ok = MODE == FAAR_GEMM_FWD && p.yref_t && p.yref_dtype == FAAR_BF16 && p.Yout == nullptr;
     bool dead = false;
-    uint4 ywide[MODE == FAAR_GEMM_FWD && WIDE ? 16 : 1];
     // One pass per accumulator buffer that fills: a tile, or (WIDE) a 256-column half of a tile.
     int vt = 0;
     for (;; ++vt) {
@@ -1087,15 +1080,13 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int col_end = min(col_begin + cols_per_warp, TW);
       const int o = m0 + quarter * 32 + lane;
       // FWD with a transposed BF16 target, columns inside the matrix: this lane's target values (128 at most, sixteen
-      // 16-byte loads) are requested before the wait for the accumulator, so their latency lies under the main loop
+      // 16-byte loads) are requested before the wait for the accumulator, so their latency lies under the main loop (of a
+      // wide tile's second half: behind the first half's stores.  Asked for between those stores, the forward kernel and soft
+      // weights of 2048 x 8192 take, us, at 4608 tokens 121.5 -> 122.3, at 4096 112.3 -> 112.9, of 4096 x 8192 at 2048 135.3 -> 136.3;
+      // both halves' before the main loop, in 64 more registers, spill: 123.0, 113.7, 136.5)
       const bool yvec = yvec_ok && n0 + col_end <= p.N;
       uint4 yraw[MODE == FAAR_GEMM_FWD ? 16 : 1];
-      if constexpr (MODE == FAAR_GEMM_FWD && WIDE) {
-        if (yvec && acc == 0) {
-#pragma unroll
-          for (int q = 0; q < 8; ++q) request_yref(p, o, n0 + col_begin, q, col_end - col_begin, ywide);
-        }
-      } else if constexpr (MODE == FAAR_GEMM_FWD) {
+      if constexpr (MODE == FAAR_GEMM_FWD) {
         static_assert(BN_MAX / C::COL_GROUPS == 128, "a warp's columns of the widest tile");
         if (yvec && o < p.M) {
           const uint4* y4 = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.Yref) +
@@ -1197,14 +1188,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               uint32_t r[16];
               tmem_ld16(trow + (uint32_t)c, r);
               tmem_ld_wait();
-              if constexpr (WIDE) warp_acc += epi_fwd_vec(p, o, n0 + c, r, ywide[2 * q], ywide[2 * q + 1]);
-              else warp_acc += epi_fwd_vec(p, o, n0 + c, r, yraw[2 * q], yraw[2 * q + 1]);
-            }
-            if constexpr (MODE == FAAR_GEMM_FWD && WIDE) {
-              // the second half's values, as the registers of the first half's come free: asked for after the first half's
-              // stores they took 6 k clocks
-              const int w2 = (p.n_main / C::COL_GROUPS + 15) / 16 * 16, begin2 = cg * w2, end2 = min(begin2 + w2, p.n_main);
-              if (acc == 0 && tc.n0 + BN_MAX + end2 <= p.N) request_yref(p, o, tc.n0 + BN_MAX + begin2, q, end2 - begin2, ywide);
+              warp_acc += epi_fwd_vec(p, o, n0 + c, r, yraw[2 * q], yraw[2 * q + 1]);
             }
           }
         } else {
