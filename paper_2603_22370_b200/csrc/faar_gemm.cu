@@ -1461,9 +1461,11 @@ int pick_full(faar_ctx* ctx, int mode, int m_tiles, int n_main, int narrow, int 
 // over 2048 34.0 -> 38.4, over 4096 58.0 -> 62.4, over 8192 97 -> 99; 144 over 8192 101.3 -> 100.8; forward kernel and soft
 // weights of 2048 x 4096 at 4096 tokens 72.3 -> 74.2, with an FP32 target of 2048 x 8192 152 -> 164.  By themselves therefore
 // only for a forward product with a transposed BF16 target and 8192 or more contraction elements, where the least width
-// that gives one wave (a multiple of 16) is at most 512 and takes less main loop than the waves of 256-wide tiles.  Forward
-// kernel and soft weights of 2048 x 8192, us: 4096 tokens (512 -> 464 columns, 64 -> 72 of 74 pairs) 118 -> 112, 2500 tokens (256 ->
-// 288) 98.2 -> 86.0.
+// that gives one wave (a multiple of 16) is at most 512 and takes less main loop than the waves of 256-wide tiles: a
+// sixteenth less if it leaves more than a seventh of the pairs idle, as a thin second wave of 256-wide tiles has the L2 to itself.
+// Forward kernel and soft weights over 8192, 256-wide -> this, us: 2048 outputs, 4096 tokens (464 columns, 72 of 74 pairs) 116.2 ->
+// 112.3, 2500 (288) 98.4 -> 87.4, 4600 (512) 124.1 -> 122.6; 7680 outputs (60 pairs), 900 tokens (464) 167.0 -> 164.3; but
+// 1024 (512) 167.4 -> 170.5, and 4864 outputs (57), 1410 (480 for two waves) 139.4 -> 141.5, 1320 (448 for 1.75) 132.6 -> 135.5.
 int pick_wide(faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int pairs, bool fwd_vec) {
   if (bn != BN_MAX || ctx->tune_wide == 0) return 0;
   if (ctx->tune_wide == 1) return (mode == FAAR_GEMM_REF && M > N ? M : N) > BN_MAX ? WIDE_BN : 0;    // REF may have either index as its rows
@@ -1473,10 +1475,14 @@ int pick_wide(faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int p
   int w = ((N + cols - 1) / cols + 15) / 16 * 16;
   if (w <= BN_MAX || w > WIDE_BN) return 0;
   if (w < WIDE_BN_MIN) w = WIDE_BN_MIN;
-  // 256-wide tiles: whole waves, and a last one of up to half the pairs cut into half tiles, which cost 0.75 (pick_full)
-  const int tiles = m_tiles * ((N + BN_MAX - 1) / BN_MAX), rest = tiles % pairs;
-  const double plain = tiles / pairs + (rest == 0 ? 0.0 : (2 * rest <= pairs ? 0.75 : 1.0));
-  return w <= plain * BN_MAX ? w : 0;
+  // 256-wide tiles: waves of whole ones, and a last wave, of half tiles (0.75 each, pick_full) where the pairs suffice for
+  // them; a last column of up to 128 comes as half tiles anyway
+  const int whole = m_tiles * (N / BN_MAX + (N % BN_MAX > BN_MAX / 2)), narrow = N % BN_MAX != 0 && N % BN_MAX <= BN_MAX / 2 ? m_tiles : 0;
+  const int rest = whole % pairs;
+  const double last = rest + narrow == 0 ? 0.0 : (2 * rest + narrow <= pairs ? 0.75 : (rest + narrow <= pairs ? 1.0 : 1.75));
+  const double limit = (whole / pairs + last) * BN_MAX;
+  const int wide_cols = (N + w - 1) / w;
+  return 7 * m_tiles * wide_cols >= 6 * pairs ? (w <= limit ? w : 0) : (w < limit * 15 / 16 ? w : 0);
 }
 
 template <int MODE, int OPT, int SHAPE, int MN>

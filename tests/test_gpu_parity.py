@@ -1093,6 +1093,8 @@ def test_chaining_arguments_are_checked(ctx):
     (2048, 4096, 2560, 256, 74), (2000, 4096, 2570, 256, 74),
     (2000, 8192, 4090, 512, 72),       # 464 columns: 9 x 8 tiles
     (1500, 8192, 3100, 512, 66),       # 259 columns would do for 12 x 6 tiles; the narrowest form has 288: 11 x 6
+    (7680, 8192, 1024, 256, 74),       # 2 x 30 tiles of 512 columns would save no main loop and leave 14 pairs idle
+    (4864, 8192, 1320, 256, 74),       # the last of six columns of tiles is 40 wide: half tiles, 1.75 waves
 ])
 def test_wide_tiles_give_the_same_bits_and_are_taken_where_they_fill_a_wave(ctx, O, K, T, auto, pairs):
     """80 tiles of 256 x 256 are two waves of the CTA pairs, 40 of 256 x 512 one, which takes longer all the same; with a long
