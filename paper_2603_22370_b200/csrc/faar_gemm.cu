@@ -454,15 +454,22 @@ __device__ __forceinline__ void store_units(void* y, const uint32_t (&w)[8], boo
   reinterpret_cast<uint4*>(y)[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 // The accumulator's rows as columns of Y: neighbouring lanes write neighbouring values, whatever the alignment of a row of Y.
+// A chunk's 16 stores go out together, which shortens an epilogue that nothing hides.  apart: BF16 values one after the other,
+// each behind its own test, where the next tile's main loop is long enough to hide that: back to back these stores of 64 bytes
+// of a row get in the way of its operands.  Products with 3 values of padding a row, us, together -> apart: [4000, 12288] over
+// 2048 144.6 -> 141.2 (one by one everywhere, as before: 141.3), [8192, 4096] over 3072 141.1 -> 135.0 (139.0), over 1536 75.4 -> 72.7
+// (75.9); over 1280 64.6 -> 64.5 (67.8) and [3000, 8192] over 1024, where every tile's stores go out together, 43.1 (50.1).  FP32
+// values, whose stores fill 128 bytes, cost the same either way.
+constexpr int APART_BLOCKS = 24;
 template <typename T>
-__device__ __forceinline__ void store_columns(const KParams& p, int col, int r0, const uint32_t (&acc)[16]) {
+__device__ __forceinline__ void store_columns(const KParams& p, int col, int r0, const uint32_t (&acc)[16], bool apart) {
   T* y = reinterpret_cast<T*>(p.Yout) + (long long)r0 * p.ldy + col;
   auto store = [&](int j) {
     if (!FAAR_DBG_OK(p, y + j * p.ldy, (int)sizeof(T), p.Yout, p.ext_yout, 1u)) return;
     if constexpr (sizeof(T) == 2) y[j * p.ldy] = __float2bfloat16_rn(__uint_as_float(acc[j]));
     else y[j * p.ldy] = __uint_as_float(acc[j]);
   };
-  if (r0 + 16 <= p.N) {
+  if (r0 + 16 <= p.N && !apart) {
 #pragma unroll
     for (int j = 0; j < 16; ++j) store(j);
   } else {
@@ -471,10 +478,10 @@ __device__ __forceinline__ void store_columns(const KParams& p, int col, int r0,
       if (r0 + j < p.N) store(j);
   }
 }
-__device__ __forceinline__ void epi_ref_columns(const KParams& p, int col, int r0, const uint32_t (&acc)[16]) {
+__device__ __forceinline__ void epi_ref_columns(const KParams& p, int col, int r0, const uint32_t (&acc)[16], bool apart) {
   if (col >= p.M) return;
-  if (p.yout_dtype == FAAR_BF16) store_columns<__nv_bfloat16>(p, col, r0, acc);
-  else store_columns<float>(p, col, r0, acc);
+  if (p.yout_dtype == FAAR_BF16) store_columns<__nv_bfloat16>(p, col, r0, acc, apart);
+  else store_columns<float>(p, col, r0, acc, false);
 }
 // 16 columns as BF16 pairs, those beyond the matrix as 0.  One test for all of them: `whole || column < N` for each became 16
 // branches, 600 clocks per 16 columns and most of a 256-wide tile's epilogue, which nothing hides for a pair's last tile:
@@ -1194,6 +1201,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         } else {
           // REF: two chunks' accumulators in flight (a warp's column count is a multiple of 16: the second may be absent)
           constexpr int STEP = MODE == FAAR_GEMM_REF ? 32 : 16;
+          const bool apart = COLUMNS && k_blocks >= APART_BLOCKS && tile + n_pairs < total_tiles;
 #pragma unroll 1
           for (int c = col_begin; c < col_end; c += STEP) {
             if (n0 + c >= p.N) break;                    // warp-uniform
@@ -1209,8 +1217,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if (second) add_parts(r2, parts, splits, split, TW, c + 16, quarter * 32 + lane);
               }
               if (COLUMNS) {
-                epi_ref_columns(p, o, n0 + c, r);
-                if (second) epi_ref_columns(p, o, n0 + c + 16, r2);
+                epi_ref_columns(p, o, n0 + c, r, apart);
+                if (second) epi_ref_columns(p, o, n0 + c + 16, r2, apart);
               } else {
                 epi_ref(p, o, n0 + c, r);
                 if (second) epi_ref(p, o, n0 + c + 16, r2);

@@ -47,6 +47,25 @@ def test_plain_product_at_the_edges_of_tiles(ctx, O, T, pad, transposed, width):
     assert torch.all(Y[:, cols:written] == 0.0) and torch.all(Y[:, written:] == 7.0)
 
 
+@pytest.mark.parametrize("T", [2300, 2317])                                # whole and cut last chunks of 16 rows
+@pytest.mark.parametrize("K", [1472, 1488, 1536])                           # 23 k blocks; 24, the last one ragged; 24
+@pytest.mark.parametrize("yref_dtype", [faar.BF16, faar.F32])
+def test_plain_product_with_unaligned_rows_over_several_waves(ctx, T, K, yref_dtype):
+    """99 to 110 tiles, more than there are pairs: a pair's tiles but its last store their chunks' rows one by one from 24 k blocks on."""
+    O, pad = 2603, 2
+    X, W = _rand(6, T, K), _rand(7, O, K)
+    shape = faar.make_shape(O, K, T, ldy=O + pad, yref_dtype=yref_dtype)
+    ws = ctx.workspace(shape)
+    Y = torch.full((T, O + pad), 7.0, dtype=torch.bfloat16 if yref_dtype == faar.BF16 else torch.float32, device=DEV)
+    faar.layer_ref(ctx, shape, X, W, Y, ws)
+    assert faar.last_gemm_config(ctx)[:2] == (256, 74)
+    faar.check_status(ctx, ws)
+    ref, mag = X.double() @ W.double().T, X.double().abs() @ W.double().abs().T
+    eps = 2.0 ** -8 if yref_dtype == faar.BF16 else 0.0
+    assert torch.all((Y[:, :O].double() - ref).abs() <= K * 2.0 ** -24 * mag + eps * ref.abs())
+    assert torch.all(Y[:, O:] == 7.0)
+
+
 @pytest.mark.parametrize("target", ["transposed", "transposed f32", "rows"])
 @pytest.mark.parametrize("O,K,T,width", [(256, 96, 256, 256), (300, 96, 200, 128), (300, 96, 1030, 256), (100, 96, 1040, 512), (600, 96, 3000, 512),
                                          (2048, 8192, 2600, 0), (2000, 8192, 4090, 0)])
