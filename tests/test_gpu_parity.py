@@ -884,12 +884,17 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_survives(ctx):
     assert rel_l2(host(lay.V), Vo) <= 2e-3
 
 
-@pytest.mark.parametrize("O,K,T", [(128, 256, 256), (1000, 1040, 203)])      # split contraction; half-width tiles
+@pytest.mark.parametrize("O,K,T,form", [
+    (128, 256, 256, (128, 4)),         # whole contractions, half-width tiles
+    (1000, 1040, 203, (128, 68)),
+    (128, 256, 1024, (64, 16)),        # four parts of a contraction each: shares of 16 columns
+    (512, 512, 800, (128, 16)),        # two parts: shares of 64
+])
 @pytest.mark.parametrize("opt", [0, 1])
-def test_round_loss_of_a_step_for_any_v(ctx, O, K, T, opt):
+def test_round_loss_of_a_step_for_any_v(ctx, O, K, T, form, opt):
     """V is the caller's: values outside [0, 1], infinities and NaN count in the first step's Round Loss as its definition
     says, mean(1 - (2v - 1)^2), and leave nothing behind for the next step's (V is clipped by then).  FP32 terms summed per
-    thread: 2^-16 of the terms' magnitudes."""
+    thread: 2^-16 of the terms' magnitudes.  form: width of the dW tiles and CTA pairs on a whole B200."""
     W, X, Yref = _problem(O, K, T, seed=3)
     lay = GpuLayer(ctx, W, X)
     lay.init()
@@ -905,6 +910,7 @@ def test_round_loss_of_a_step_for_any_v(ctx, O, K, T, opt):
             t2 = (2.0 * host(lay.V).astype(np.float64) - 1.0) ** 2
             lay.step(f32hp(beta=4.0, step=step, opt=opt)[0])
             lay.check()
+            assert faar.last_gemm_config(ctx) == form
             want, got = np.mean(1.0 - t2), float(host(lay.loss)[1])
             if np.isfinite(want):
                 assert abs(got - want) <= 2.0 ** -16 * np.mean(1.0 + t2), (float(v.flat[0]), step, got, want)

@@ -35,10 +35,12 @@ def test_plain_product_at_the_edges_of_tiles(ctx, O, T, pad, transposed, width):
             faar.tune_wide_tiles(ctx, 1)
         faar.tune_tile_n(ctx, min(width, 256))
         faar.layer_ref(ctx, shape, X, W, Y, ws)
+        taken = faar.last_gemm_config(ctx)[0]
     finally:
         faar.tune_tile_n(ctx, 0)
         faar.tune_wide_tiles(ctx, -1)
     faar.check_status(ctx, ws)
+    assert width == 0 or taken == (512 if width == 512 and max(O, T) > 256 else min(width, 256))
     ref, mag = X.double() @ W.double().T, X.double().abs() @ W.double().abs().T
     if transposed:
         ref, mag = ref.T, mag.T
@@ -68,7 +70,8 @@ def test_plain_product_with_unaligned_rows_over_several_waves(ctx, T, K, yref_dt
 
 @pytest.mark.parametrize("target", ["transposed", "transposed f32", "rows"])
 @pytest.mark.parametrize("O,K,T,width", [(256, 96, 256, 256), (300, 96, 200, 128), (300, 96, 1030, 256), (100, 96, 1040, 512), (600, 96, 3000, 512),
-                                         (2048, 8192, 2600, 0), (2000, 8192, 4090, 0)])
+                                         # tiles of 288, 304 and 464 columns for a transposed BF16 target, of 256 otherwise
+                                         (2048, 8192, 2400, 0), (2048, 8192, 2600, 0), (2000, 8192, 4090, 0)])
 def test_forward_product_at_the_edges_of_tiles(ctx, O, K, T, width, target):
     """dY = 2 (Y_q - Y_ref) in BF16, Y_q in FP32 from the soft weights' BF16 operand; nothing beyond a row's T values."""
     f32, trans = target.endswith("f32"), target.startswith("transposed")
@@ -89,10 +92,13 @@ def test_forward_product_at_the_edges_of_tiles(ctx, O, K, T, width, target):
             faar.tune_wide_tiles(ctx, 1)
         faar.tune_tile_n(ctx, min(width, 256))
         faar.layer_fwd(ctx, shape, faar.make_hparams(beta=6.0), X, Yref, V, code, scales, s_global, dYt, loss, None, ws)
+        taken = faar.last_gemm_config(ctx)
     finally:
         faar.tune_tile_n(ctx, 0)
         faar.tune_wide_tiles(ctx, -1)
     faar.check_status(ctx, ws)
+    # one wave of 9 x 8 fitted tiles on a whole B200
+    assert taken == ((512, 72) if target == "transposed" else (256, 74)) if width == 0 else taken[0] == width
     r = Wb.double() @ X.double().T - (Yref[:, :T] if trans else Yref[:, :O].T).double()
     err = K * 2.0 ** -24 * (Wb.double().abs() @ X.double().abs().T) + 2.0 ** -23 * r.abs()
     assert torch.all((dYt[:, :T].double() - 2.0 * r).abs() <= 2.0 * err + 2.0 ** -8 * (2.0 * r).abs())
