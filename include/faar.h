@@ -152,11 +152,11 @@ FAAR_API int faar_tune_tile_n(faar_ctx* ctx, int bn);
 FAAR_API int faar_tune_tail_split(faar_ctx* ctx, int columns);
 FAAR_API int faar_last_tail_split(const faar_ctx* ctx, int* columns);
 FAAR_API int faar_last_gemm_config(const faar_ctx* ctx, int* bn, int* cta_pairs);
-/* A launch can take 256 x 512 tiles: the pair's whole tensor memory as one accumulator, a quarter less operand
- * traffic per flop, no overlap of a tile's epilogue with the next tile's main loop, no tail split.
- * mode: 1 = whenever the output has more than 256 columns and 256-wide tiles would have been used; 0 = never; -1 (the
+/* A launch can take tiles of 256 x (288 .. 512): the pair's whole tensor memory as one accumulator, up to a quarter less
+ * operand traffic per flop, no overlap of a tile's epilogue with the next tile's main loop, no tail split.
+ * mode: 1 = of 512, whenever the output has more than 256 columns and 256-wide tiles would have been used; 0 = never; -1 (the
  * default) = for a forward product with a transposed BF16 target and a contraction of 8192 or more that tiles of 288 to 512
- * columns finish in one wave: with the least such width.  faar_last_gemm_config reports bn = 512 for any of them.
+ * columns finish in one wave, in less main loop than 256-wide ones: with the least such width.  faar_last_gemm_config reports bn = 512 for any of them.
  * 0 and 1 also keep contractions whole.  The per-weight
  * results (dW, V, moments) do not depend on the tile shape. */
 FAAR_API int faar_tune_wide_tiles(faar_ctx* ctx, int mode);

@@ -320,7 +320,8 @@ softquant_init_kernel(const void* __restrict__ W, int O, int K, int64_t ldw,
 // bit clear, so a quotient on a midpoint moves above it, and one below a midpoint stays below.  The codes convert back
 // to F16 pairs (nodes exactly); shifting the magnitude bits right by three makes them BF16 values scaled by 2^-112 (the
 // difference of the exponent biases), which the block scale times 2^112 undoes in one exact packed product.
-// [4096, 8192] 54 -> 27.7 us, [16384, 8192] 103 us (611 MB; the maximum pass excluded): bound by HBM.
+// [4096, 8192] 54 -> 28.2 us, [16384, 8192] 103 us (153 and 611 MB: 23.4 and 94 us of HBM; the maximum pass excluded).  Bound by
+// instruction issue, 18 a value, next to HBM: without the packed copy, an eighth of the bytes, 27.5 and 99.7, and from L2 no faster.
 __device__ __forceinline__ uint32_t to_e2m1x2(float lo, float hi) {             // one byte: lo in bits 3:0
   uint32_t r;
   asm("{\n\t.reg .b8 b;\n\tcvt.rn.satfinite.e2m1x2.f32 b, %1, %2;\n\tcvt.u32.u8 %0, b;\n\t}" : "=r"(r) : "f"(hi), "f"(lo));

@@ -57,7 +57,7 @@ constexpr int BN_MAX = 256;
 constexpr int WIDE_BN = 2 * BN_MAX;
 constexpr int WIDE_BN_MIN = BN_MAX + 32;       // no other launch gives a pair of CTAs an MMA of fewer than 32 columns either
 // The tile forms of a launch, chosen at compile time (as run-time options of one kernel they cost the others time): tiles of
-// up to 256 columns, 256 x 512, a contraction split over the pairs of a cluster, or (BWD) 256-wide tiles of a short contraction.
+// up to 256 columns, 256 x (288 .. 512), a contraction split over the pairs of a cluster, or (BWD) 256-wide tiles of a short contraction.
 //
 // SHORT_TILES: a dW launch of few k blocks is bound by its epilogue's state traffic.  What limits that is the L1 cache: a
 // load in flight holds its L1 lines, and with all of an SM's 256 KB but 28 taken as shared memory, loads beyond about 24 KB
@@ -67,16 +67,18 @@ constexpr int WIDE_BN_MIN = BN_MAX + 32;       // no other launch gives a pair o
 // 130.0 -> 128.9, 4096 134 -> 137; of 12288 x 2048 at 2000 149 -> 143.  With the carve-out but 4 weights at a time 64 tokens
 // take 91.8, with 8 at a time but no carve-out 97.6; without another stage (92 KB of L1) nothing changes but 2000 tokens, 148.
 // Above SHORT_BLOCKS the main loop needs the stage: operands and state together then take all the 64 bytes a clock that an
-// SM draws from L2.
+// SM draws from L2.  The line is the same for plain gradient descent, a third of the state, us: 64 tokens 51.9 -> 38.9, 1024
+// 58.2 -> 46.0, 2048 67.9 -> 62.4, 2560 74.9 -> 73.1 (Adam 107.0 -> 104.7, writing the next operand too 116.3 -> 115.4).
 //
 // SPLIT_NARROW: a split contraction that leaves a CTA at most 32 columns to finish, of a dW launch.  The lanes of its epilogue then
 // cover 16 or 32 columns of a row instead of 64, most of which there would be none of: a small layer's epilogue executed the
-// instructions of four times its weights.  Step of 128 x 256 at 1024 tokens (16 columns) 14.7 -> 13.6 us.  (As a choice inside
-// SPLIT_TILES it cost shares of 64 columns 2 %.)
+// instructions of four times its weights.  Step of 128 x 256 at 1024 tokens (16 columns) 14.75 -> 12.6 us; dW kernel (shares of 16
+// columns) of 256 x 256 at 1024 tokens 9.7 -> 7.9, 128 x 256 at 4096 12.3 -> 10.7, 256 x 1024 at 1024 10.0 -> 8.9, (of 32) 128 x 1536 at 1536
+// 11.1 -> 10.0, 300 x 464 at 2600 12.6 -> 11.6.  (As a choice inside SPLIT_TILES it cost shares of 64 columns 2 %.)
 constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2, SHORT_TILES = 3, SPLIT_NARROW = 4;
 constexpr int SHORT_BLOCKS = 40;
 constexpr int SHORT_SMEM = 387 * 512;          // with the system's 1 KB below the 196 KB carve-out
-constexpr int SHORT_CARVEOUT = 85;             // percent of the 228 KB: 196 KB
+constexpr int SHORT_CARVEOUT = 85;             // percent of the 228 KB: 193.8, which is rounded up to the size on offer, 196 KB
 template <int MODE, int SHAPE = PLAIN_TILES> struct Cfg {
   static constexpr bool WIDE = SHAPE == WIDE_TILES, SHORT = SHAPE == SHORT_TILES, SPLIT = SHAPE == SPLIT_TILES || SHAPE == SPLIT_NARROW;
   static constexpr int EPI_WARPS = MODE == FAAR_GEMM_BWD ? 16 : 8;
@@ -677,7 +679,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // shared memory (row r at panel + 4 PW r, its 16-byte units swizzled: panel_unit); then warp `sub`
 // of the quarter takes rows 8 sub .. 8 sub + 7, LPR = PX / LW lanes per row and lane l the columns
 // LW (l % LPR) and on, so that one warp instruction moves 128 LW bytes of V / m / u as 32 / LPR row pieces of
-// 4 PW contiguous bytes each: whole lines as 16- or 32-byte vectors.  (A panel of 128 columns gives one 512-byte
+// 4 PX contiguous bytes each, as 16- or 32-byte vectors: two lines (half a line or one where PX is 16 or 32).  (A panel of 128 columns gives one 512-byte
 // piece per instruction but leaves room for five TMA stages only; the sixth stage is worth more.)
 // The per-weight state of the next instruction is requested before the current one's is computed, and a panel's first
 // before the panel is staged (a tile's first before its accumulator is ready): a request takes 600-800 clocks, the

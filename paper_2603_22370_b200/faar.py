@@ -349,7 +349,7 @@ def add(ctx, rows, cols, a, lda, b, ldb, out, ldo):
 
 def tune_wide_tiles(ctx, mode: int):
     """1: 256 x 512 GEMM tiles whenever the shape allows; 0: never; -1 (the default): for long forward products that
-    fill a wave of them.  0 and 1 keep contractions whole."""
+    tiles of 288 to 512 columns finish in one wave, of the least such width.  0 and 1 keep contractions whole."""
     _check(lib().faar_tune_wide_tiles(ctx._h, mode), "faar_tune_wide_tiles")
 
 
