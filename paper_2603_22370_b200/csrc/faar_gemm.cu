@@ -456,12 +456,13 @@ __device__ __forceinline__ void store_units(void* y, const uint32_t (&w)[8], boo
   reinterpret_cast<uint4*>(y)[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 // The accumulator's rows as columns of Y: neighbouring lanes write neighbouring values, whatever the alignment of a row of Y.
-// A chunk's 16 stores go out together, which shortens an epilogue that nothing hides.  apart: BF16 values one after the other,
-// each behind its own test, where the next tile's main loop is long enough to hide that: back to back these stores of 64 bytes
-// of a row get in the way of its operands.  Products with 3 values of padding a row, us, together -> apart: [4000, 12288] over
+// A chunk's 16 stores go out together, which shortens an epilogue that nothing hides.  apart: one after the other, each behind
+// its own test, where the next tile's main loop is long enough to hide that: back to back these stores of 64 bytes of a row (FP32:
+// 128) get in the way of its operands.  BF16 products with 3 values of padding a row, us, together -> apart: [4000, 12288] over
 // 2048 144.6 -> 141.2 (one by one everywhere, as before: 141.3), [8192, 4096] over 3072 141.1 -> 135.0 (139.0), over 1536 75.4 -> 72.7
 // (75.9); over 1280 64.6 -> 64.5 (67.8) and [3000, 8192] over 1024, where every tile's stores go out together, 43.1 (50.1).  FP32
-// values, whose stores fill 128 bytes, cost the same either way.
+// [4000, 12288] over 1536 123.1 -> 122.0 (122.0), over 2048 154.6 either way.  Tiles of up to 128 columns gain nothing ([128,
+// 128256] over 2048 87.4 -> 87.6).
 constexpr int APART_BLOCKS = 24;
 template <typename T>
 __device__ __forceinline__ void store_columns(const KParams& p, int col, int r0, const uint32_t (&acc)[16], bool apart) {
@@ -483,7 +484,7 @@ __device__ __forceinline__ void store_columns(const KParams& p, int col, int r0,
 __device__ __forceinline__ void epi_ref_columns(const KParams& p, int col, int r0, const uint32_t (&acc)[16], bool apart) {
   if (col >= p.M) return;
   if (p.yout_dtype == FAAR_BF16) store_columns<__nv_bfloat16>(p, col, r0, acc, apart);
-  else store_columns<float>(p, col, r0, acc, false);
+  else store_columns<float>(p, col, r0, acc, apart);
 }
 // 16 columns as BF16 pairs, those beyond the matrix as 0.  One test for all of them: `whole || column < N` for each became 16
 // branches, 600 clocks per 16 columns and most of a 256-wide tile's epilogue, which nothing hides for a pair's last tile:
@@ -1203,7 +1204,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         } else {
           // REF: two chunks' accumulators in flight (a warp's column count is a multiple of 16: the second may be absent)
           constexpr int STEP = MODE == FAAR_GEMM_REF ? 32 : 16;
-          const bool apart = COLUMNS && k_blocks >= APART_BLOCKS && tile + n_pairs < total_tiles;
+          const bool apart = COLUMNS && BN > 128 && k_blocks >= APART_BLOCKS && tile + n_pairs < total_tiles;
 #pragma unroll 1
           for (int c = col_begin; c < col_end; c += STEP) {
             if (n0 + c >= p.N) break;                    // warp-uniform
