@@ -79,16 +79,18 @@ constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2, SHORT_TILES = 3,
 constexpr int SHORT_BLOCKS = 40;
 constexpr int SHORT_SMEM = 387 * 512;          // with the system's 1 KB below the 196 KB carve-out
 constexpr int SHORT_CARVEOUT = 85;             // percent of the 228 KB: 193.8, which is rounded up to the size on offer, 196 KB
-template <int MODE, int SHAPE = PLAIN_TILES> struct Cfg {
+constexpr int GATED_FWD = 8, GATED_BWD = 10;   // MN (see the kernel) of the gated product's launches
+constexpr int GATE_COLS = 32, GATE_PANEL = 32 * GATE_COLS * 2;        // backward: a warp's 32 rows x 32 columns in BF16
+template <int MODE, int SHAPE = PLAIN_TILES, int MN = 0> struct Cfg {
   static constexpr bool WIDE = SHAPE == WIDE_TILES, SHORT = SHAPE == SHORT_TILES, SPLIT = SHAPE == SPLIT_TILES || SHAPE == SPLIT_NARROW;
-  static constexpr int EPI_WARPS = MODE == FAAR_GEMM_BWD ? 16 : 8;
+  static constexpr int EPI_WARPS = MODE == FAAR_GEMM_BWD || MN == GATED_BWD ? 16 : 8;
   static constexpr int THREADS = 32 * (2 + EPI_WARPS);
   static constexpr int A_BYTES = BM * BK * 2;
   static constexpr int BH_BYTES = (BN_MAX / 2) * BK * 2;       // this CTA's 128 rows of one 256-column B tile
   static constexpr int B_BYTES = WIDE ? 2 * BH_BYTES : BH_BYTES;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int LANE_WEIGHTS = SHORT ? 8 : 4;             // BWD: weights of one instruction's state per lane
-  static constexpr int EPI_BYTES = MODE == FAAR_GEMM_BWD ? 4 * PANEL_BYTES : 0;
+  static constexpr int EPI_BYTES = MODE == FAAR_GEMM_BWD ? 4 * PANEL_BYTES : (MN == GATED_BWD ? EPI_WARPS * GATE_PANEL : 0);
   // The ring: as many stages of the launch's tile width as fit (a stage is the A rows plus bn / 2 rows of B: 32 KB for
   // 256 columns, 18 KB for 32), at most MAX_STAGES.  A small launch's main loop runs at stages / latency, so narrow
   // tiles get the deeper ring.
@@ -538,6 +540,72 @@ __device__ __forceinline__ void epi_ref(const KParams& p, int row, int c0, const
   }
 }
 
+// REF of a decoder block's gate and up projections (weights stacked, N = 2 f): a tile holds w / 2 columns of the gate and the
+// same w / 2 of up, since either half of a tile's B rows is loaded by one CTA of the pair and the second one's start f rows
+// further on.  A lane then has both values of its 16 features and writes act = silu(gate) up (p.dYt, rows of p.ld_dyt) next
+// to them, or, where nobody reads them again (p.Yout null), instead of them: the values that a product rounded to BF16 and
+// faar_silu_mul give, without that call's pass over 3 f values a token.  The main loop hides it.  Product and call -> this, us:
+// 8192 tokens, f 8192 over 2048 338 + 59 -> 336 (with gate and up written too 348); 2000, 6144 over 2048 69.5 + 13.2 -> 70 (72).
+// The contraction is never split here: that would part a feature's two columns.
+__device__ __forceinline__ void epi_gated_fwd(const KParams& p, int row, int c0, const uint32_t (&gate)[16], const uint32_t (&up)[16]) {
+  if (row >= p.M) return;
+  uint32_t g[8], u[8], a[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    g[j] = pack_bf16x2(__uint_as_float(gate[2 * j]), __uint_as_float(gate[2 * j + 1]));
+    u[j] = pack_bf16x2(__uint_as_float(up[2 * j]), __uint_as_float(up[2 * j + 1]));
+    a[j] = pack_bf16x2(faar_silu_mul(__uint_as_float(g[j] << 16), __uint_as_float(u[j] << 16)),
+                       faar_silu_mul(__uint_as_float(g[j] & 0xFFFF0000u), __uint_as_float(u[j] & 0xFFFF0000u)));
+  }
+  __nv_bfloat16* act = p.dYt + (long long)row * p.ld_dyt + c0;
+  if (FAAR_DBG_OK(p, act, 32, p.dYt, p.ext_dyt, 2u)) stg256(act, a);
+  if (!p.Yout) return;
+  __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + (long long)row * p.ldy + c0;
+  if (FAAR_DBG_OK(p, y, 32, p.Yout, p.ext_yout, 1u)) stg256(y, g);
+  if (FAAR_DBG_OK(p, y + p.N / 2, 32, p.Yout, p.ext_yout, 1u)) stg256(y + p.N / 2, u);
+}
+// REF of the input gradient of a block's down projection (N = f): the accumulator is the gradient towards act; from it and the
+// gate and up values of the forward pass (p.Yref, rows as Yout's: gate, then up) come the gradients of both (p.Yout).
+//
+// Gate and up come in (and both gradients leave) as 16 bytes a lane, a row of 32 columns in four neighbouring lanes, the
+// accumulator's columns passing through the warp's panel of shared memory for it, which fits next to the ring's six stages: a
+// lane reading its own row's 32 bytes holds a line of L1 for each, and 28 KB of L1 then keep too few bytes in flight.  Sixteen
+// warps, because a warp's loads, arithmetic and stores do not overlap.  Input gradient and element-wise call -> this, us: 8192
+// tokens, f 8192 over 2048 167 + 108 -> 204 (lanes reading their own rows 250; eight warps of 64 columns 224); 2000, 6144 over
+// 2048 40.5 + 18.6 -> 49.  More L1 for a stage of the ring (as SHORT_TILES): 212.
+struct GateUp { uint4 g, u; };
+struct GateRows {                                // which of the warp's 32 rows and 16-byte units a lane takes in step `it` of a panel
+  int log_units;                                 // 2 or 4 units a row
+  __device__ __forceinline__ int steps() const { return 1 << log_units; }
+  __device__ __forceinline__ int row(int lane, int it) const { return (it << (5 - log_units)) + (lane >> log_units); }
+  __device__ __forceinline__ int unit(int lane) const { return lane & ((1 << log_units) - 1); }
+};
+__device__ __forceinline__ uint32_t gate_unit(uint32_t panel, int row, int u) { return panel + (uint32_t)(row * 64 + ((u ^ (row >> 1 & 3)) << 4)); }
+__device__ __forceinline__ void load_gate_up(const KParams& p, int row, int col, int col_end, GateUp& v) {
+  if (row >= p.M || col >= col_end) return;
+  const __nv_bfloat16* y = reinterpret_cast<const __nv_bfloat16*>(p.Yref) + (long long)row * p.ldy + col;
+  v.g = *reinterpret_cast<const uint4*>(y);
+  v.u = *reinterpret_cast<const uint4*>(y + p.N);
+}
+__device__ __forceinline__ void epi_gated_bwd(const KParams& p, int row, int col, int col_end, uint32_t staged, const GateUp& v) {
+  if (row >= p.M || col >= col_end) return;
+  const float4 raw = lds128(staged);
+  const uint32_t d[4] = {__float_as_uint(raw.x), __float_as_uint(raw.y), __float_as_uint(raw.z), __float_as_uint(raw.w)};
+  const uint32_t g[4] = {v.g.x, v.g.y, v.g.z, v.g.w}, u[4] = {v.u.x, v.u.y, v.u.z, v.u.w};
+  uint32_t dg[4], du[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float g0, g1, u0, u1;
+    faar_silu_mul_bwd(__uint_as_float(d[j] << 16), __uint_as_float(g[j] << 16), __uint_as_float(u[j] << 16), g0, u0);
+    faar_silu_mul_bwd(__uint_as_float(d[j] & 0xFFFF0000u), __uint_as_float(g[j] & 0xFFFF0000u), __uint_as_float(u[j] & 0xFFFF0000u), g1, u1);
+    dg[j] = pack_bf16x2(g0, g1);
+    du[j] = pack_bf16x2(u0, u1);
+  }
+  __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + (long long)row * p.ldy + col;
+  if (FAAR_DBG_OK(p, y, 16, p.Yout, p.ext_yout, 1u)) *reinterpret_cast<uint4*>(y) = make_uint4(dg[0], dg[1], dg[2], dg[3]);
+  if (FAAR_DBG_OK(p, y + p.N, 16, p.Yout, p.ext_yout, 1u)) *reinterpret_cast<uint4*>(y + p.N) = make_uint4(du[0], du[1], du[2], du[3]);
+}
+
 // FWD: residual, sum of squares, dY^T.
 // Y_ref[t0..t0+15, o] for this lane's output feature o, as it is in memory: anything done to a value here (widening BF16, a
 // select at the matrix edge) would wait for it here, one latency per chunk of 16 columns.  Forward kernel, row-major target,
@@ -873,17 +941,18 @@ __device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t parts, int
 // Launched as clusters of 2 * splits CTAs along x; CTAs 2c and 2c+1 form a pair.
 // MN: bit 0 = the A operand, bit 1 = the B operand is stored with its M / N index contiguous (KParams.a_mn / b_mn);
 // a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.  Bit 2 (REF): the
-// accumulator's rows are the result's columns; compiled in as well (as a branch it cost 0.1 us in every small product).
+// accumulator's rows are the result's columns; compiled in as well (as a branch it cost 0.1 us in every small product).  Bit 3
+// (REF): the gated product's epilogue, forward, or backward where B is N-contiguous.
 // SHAPE: one of the tile forms (see Cfg).
 constexpr int MIN_SPLIT_BLOCKS = 12;            // contractions of fewer k blocks stay whole (see pick_splits)
 template <int MODE, int OPT, int SHAPE, int MN>
-__global__ void __launch_bounds__(Cfg<MODE, SHAPE>::THREADS, 1)
+__global__ void __launch_bounds__(Cfg<MODE, SHAPE, MN>::THREADS, 1)
 faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ KParams p) {
-  constexpr bool WIDE = SHAPE == WIDE_TILES, SPLIT = Cfg<MODE, SHAPE>::SPLIT;
-  using C = Cfg<MODE, SHAPE>;
+  using C = Cfg<MODE, SHAPE, MN>;
+  constexpr bool WIDE = C::WIDE, SPLIT = C::SPLIT;
   constexpr int LW = C::LANE_WEIGHTS;
-  constexpr bool A_MN = (MN & 1) != 0, B_MN = (MN & 2) != 0, COLUMNS = (MN & 4) != 0;
+  constexpr bool A_MN = (MN & 1) != 0, B_MN = (MN & 2) != 0, COLUMNS = (MN & 4) != 0, GATED = MN == GATED_FWD, GATED_B = MN == GATED_BWD;
   const int BN = p.bn;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -960,7 +1029,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       for (int tile = pair; tile < total_tiles && ok; tile += n_pairs) {
         const TileCoord tc = coords(tile);
         const int m0 = tc.m0 + (int)rank * BM;
-        const int n0 = tc.n0 + (int)rank * (tc.w / 2);
+        const int n0 = GATED ? tc.n0 / 2 + (int)rank * (p.N / 2) : tc.n0 + (int)rank * (tc.w / 2);
         const CUtensorMap* mapB = tc.w == BN ? &tmB : &tmBh;      // box of w/2 rows
         for (int kb = kb0; kb < kb1; ++kb) {
           ok = mbar_wait(empty_bar(stage), phase ^ 1u, ac, 0x100u | stage);
@@ -1127,6 +1196,15 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         else
           row_ok = load_row_state<OPT, LW, PW>(p, seg, lane, ew >> 2, o0, n0, k_end, 0, l2_policy_stream(), row_state);
       }
+      // backward of the gated product: gate and up values of the warp's first 32 columns
+      GateUp ahead[GATED_B ? 4 : 1];
+      const GateRows gr = {cols_per_warp <= 16 ? 1 : 2};
+      const int o_quarter = m0 + quarter * 32, gate_end = min(n0 + col_end, p.N);
+      if constexpr (GATED_B) {
+#pragma unroll
+        for (int it = 0; it < 4; ++it)
+          if (it < gr.steps()) load_gate_up(p, o_quarter + gr.row(lane, it), n0 + col_begin + 8 * gr.unit(lane), gate_end, ahead[it]);
+      }
       bool ok = mbar_wait(tfull_bar(acc), acc_phase, ac, 0x400u | acc);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -1189,6 +1267,49 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           if (again && lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar(acc), leader));
         }
         continue;
+      } else if constexpr (GATED_B) {
+        const uint32_t panel = epi_u32 + (uint32_t)(ew * GATE_PANEL);
+#pragma unroll 1
+        for (int c0 = col_begin; c0 < col_end && n0 + c0 < p.N; c0 += GATE_COLS) {
+#pragma unroll
+          for (int q = 0; q < GATE_COLS / 16; ++q) {
+            const int c = c0 + 16 * q;
+            if (c < col_end) {                           // warp-uniform
+              uint32_t r[16];
+              tmem_ld16(trow + (uint32_t)c, r);
+              tmem_ld_wait();
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                uint32_t w[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) w[j] = pack_bf16x2(__uint_as_float(r[8 * h + 2 * j]), __uint_as_float(r[8 * h + 2 * j + 1]));
+                sts128(gate_unit(panel, lane, 2 * q + h), w[0], w[1], w[2], w[3]);
+              }
+            }
+          }
+          __syncwarp();
+          const int col = n0 + c0 + 8 * gr.unit(lane);
+#pragma unroll
+          for (int it = 0; it < 4; ++it) {
+            if (it < gr.steps()) {
+              const int row = o_quarter + gr.row(lane, it);
+              epi_gated_bwd(p, row, col, gate_end, gate_unit(panel, gr.row(lane, it), gr.unit(lane)), ahead[it]);
+              load_gate_up(p, row, col + GATE_COLS, gate_end, ahead[it]);
+            }
+          }
+          __syncwarp();
+        }
+      } else if constexpr (GATED) {
+        // the warps of a lane quarter take 16 features of the tile in turn
+        const int half = tc.w / 2, f0 = n0 / 2;
+#pragma unroll 1
+        for (int c = 16 * cg; c < half && f0 + c < p.N / 2; c += 16 * C::COL_GROUPS) {
+          uint32_t r[16], r2[16];
+          tmem_ld16(trow + (uint32_t)c, r);
+          tmem_ld16(trow + (uint32_t)(half + c), r2);
+          tmem_ld_wait();
+          epi_gated_fwd(p, o, f0 + c, r, r2);
+        }
       } else {
         if (MODE == FAAR_GEMM_FWD && yvec) {
 #pragma unroll
@@ -1499,7 +1620,7 @@ int pick_wide(faar_ctx* ctx, int mode, int M, int N, int k_blocks, int bn, int p
 template <int MODE, int OPT, int SHAPE, int MN>
 int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_out, int bn, int max_pairs,
                    const cudaLaunchConfig_t& base_cfg) {
-  using C = Cfg<MODE, SHAPE>;
+  using C = Cfg<MODE, SHAPE, MN>;
   constexpr bool WIDE = C::WIDE, SPLIT = C::SPLIT;
   static_assert(C::MIN_STAGES >= 3, "ring too short");
   static_assert(C::SMEM_BYTES <= SMEM_LIMIT, "shared memory budget");
@@ -1509,6 +1630,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   if (e) return e;
   cudaLaunchConfig_t cfg = base_cfg;
   cfg.dynamicSmemBytes = C::SMEM_BYTES;
+  cfg.blockDim = dim3(C::THREADS, 1, 1);
   kp.bn = bn;
   kp.stage_bytes = WIDE ? C::STAGE_BYTES : C::A_BYTES + (a->b_mn ? mn_boxes(bn / 2) * MN_BOX_BYTES : (int)faar_align_up((size_t)(bn / 2) * BK * 2, 1024));   // whole swizzle atoms
   const int ring = (C::RING_BYTES - (SPLIT ? parts_bytes(kp.splits, bn) : 0)) / kp.stage_bytes;
@@ -1611,6 +1733,13 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
   const int wide = pick_wide(ctx, MODE, a->M, a->N, k_blocks, bn, max_pairs, fwd_vec);
   kp.n_main = wide > BN_MAX ? wide - BN_MAX : BN_MAX;
   const int mn = (a->a_mn ? 1 : 0) | (a->b_mn ? 2 : 0);
+  if constexpr (MODE == FAAR_GEMM_REF) {
+    if (a->gated == FAAR_GATED_FWD) {                   // either half of a whole or half-width tile is a multiple of 16
+      if (bn != 32) bn = (bn + 63) / 64 * 64;
+      return launch_variant<MODE, OPT, PLAIN_TILES, GATED_FWD>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+    }
+    if (a->gated == FAAR_GATED_BWD) return launch_variant<MODE, OPT, PLAIN_TILES, GATED_BWD>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+  }
   // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient; A, if the
   // accumulator's rows are the result's columns), the dW product with B or with both untransposed
   if constexpr (MODE == FAAR_GEMM_REF) {
@@ -1639,7 +1768,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
 // would be padding that is staged all the same.  M on the accumulator's rows -> N, us: 1 row of 8192 over 2048 15.1 -> 10.6,
 // 64 rows 12.8 -> 12.0, 128 rows 13.1 -> 12.2, 160 rows 13.1 -> 13.8; input gradient of 8 rows of 8192 over 2048 14.5 -> 11.9.
 static bool result_columns(const faar_gemm_args* a) {
-  if (a->yref_t) return false;
+  if (a->yref_t || a->gated) return false;
   const long long row = a->ldy * (a->yout_dtype == FAAR_BF16 ? 2 : 4);
   return a->M <= BM || row % 16 != 0 || (reinterpret_cast<uintptr_t>(a->Yout) & 15) != 0;
 }
@@ -1663,6 +1792,13 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
     swapped.B = args->A; swapped.ldb = args->lda; swapped.b_mn = args->a_mn;
     a = &swapped;
   }
+  if (a->gated) {                                      // unsplit, f a multiple of 16, every row on 32 bytes
+    const int f = a->gated == FAAR_GATED_FWD ? a->N / 2 : a->N;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(a->Yout) | reinterpret_cast<uintptr_t>(a->act) | reinterpret_cast<uintptr_t>(a->gate_up);
+    if (a->mode != FAAR_GEMM_REF || !a->whole || f % 16 || a->ldy % 16 || at & 31 || a->a_mn || (a->b_mn != 0) != (a->gated == FAAR_GATED_BWD) ||
+        a->yout_dtype != FAAR_BF16 || (a->gated == FAAR_GATED_FWD ? !a->act || a->N % 2 : !a->Yout || !a->gate_up))
+      return (int)cudaErrorInvalidValue;
+  }
   kp.M = a->M; kp.N = a->N; kp.Kc = a->Kc; kp.bn = BN_MAX; kp.n_main = kp.narrow = kp.n_full = 0; kp.status = a->status;
   {
     const long long ysz = a->yout_dtype == FAAR_BF16 ? 2 : 4;
@@ -1680,6 +1816,13 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
   kp.Yout = a->Yout; kp.yout_dtype = a->yout_dtype; kp.ldy = a->ldy;
   kp.Yref = a->Yref; kp.yref_dtype = a->yref_dtype; kp.yref_t = a->yref_t;
   kp.dYt = a->dYt; kp.ld_dyt = a->ld_dyt; kp.mse2c = a->mse2c; kp.act_scale = a->act_scale; kp.partials = a->partials;
+  if (a->gated == FAAR_GATED_FWD) {
+    kp.dYt = reinterpret_cast<__nv_bfloat16*>(a->act); kp.ld_dyt = a->N / 2;
+    kp.ext_dyt = (long long)a->M * a->N;
+  } else if (a->gated == FAAR_GATED_BWD) {
+    kp.Yref = a->gate_up;
+    kp.ext_yout = ((long long)(a->M - 1) * a->ldy + 2ll * a->N) * 2;
+  }
   if (a->mode == FAAR_GEMM_BWD) {
     long long row0 = 0;
     for (int i = 0; i < FAAR_MAX_SEGMENTS; ++i) {

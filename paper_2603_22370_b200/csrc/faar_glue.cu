@@ -28,14 +28,6 @@ __device__ __forceinline__ uint4 pack8(const float (&x)[8]) {
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// sigmoid(x) in FP32: 1 / (1 + e^-x) with the library exponential (relative error ~1e-7) and the hardware
-// reciprocal (rcp.approx: relative error below 2^-22); e^-x overflowing to +inf gives 0, the limit.
-__device__ __forceinline__ float sigmoid_f32(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + expf(-x)));
-  return r;
-}
-
 // Work split of the [rows, 8-element groups] kernels: threadIdx.x / blockIdx.x run over the groups of a row,
 // threadIdx.y / blockIdx.y over rows (grid-stride), so no thread divides its index by the row length.
 struct Split { dim3 grid, block; };
@@ -64,12 +56,12 @@ silu_mul_kernel(const __nv_bfloat16* gate, int64_t ldg, const __nv_bfloat16* up,
     float a[8], b[8], y[8];
     unpack8(ga, a); unpack8(ua, b);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = a[i] * sigmoid_f32(a[i]) * b[i];
+    for (int i = 0; i < 8; ++i) y[i] = faar_silu_mul(a[i], b[i]);
     *reinterpret_cast<uint4*>(out + (int64_t)row * ldo + col) = pack8(y);
     if (two) {
       unpack8(gb, a); unpack8(ub, b);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) y[i] = a[i] * sigmoid_f32(a[i]) * b[i];
+      for (int i = 0; i < 8; ++i) y[i] = faar_silu_mul(a[i], b[i]);
       *reinterpret_cast<uint4*>(out + (int64_t)row1 * ldo + col) = pack8(y);
     }
   }
@@ -395,7 +387,7 @@ rope_kernel(const __nv_bfloat16* x, int64_t ldx, const int* __restrict__ pos, __
   }
 }
 
-// ---- backward of the gated product: with s = sigmoid(g),  dg = d u s (1 + g (1 - s)),  du = d g s -----
+// ---- backward of the gated product ----------------------------------------------------------------
 __global__ void __launch_bounds__(GL_THREADS)
 silu_mul_bwd_kernel(const __nv_bfloat16* dout, int64_t ldd, const __nv_bfloat16* gate, int64_t ldg, const __nv_bfloat16* up,
                     int64_t ldu, __nv_bfloat16* dgate, int64_t lddg, __nv_bfloat16* dup, int64_t lddu, int rows, int groups) {
@@ -409,11 +401,7 @@ silu_mul_bwd_kernel(const __nv_bfloat16* dout, int64_t ldd, const __nv_bfloat16*
     unpack8(*reinterpret_cast<const uint4*>(gate + (int64_t)row * ldg + col), g);
     unpack8(*reinterpret_cast<const uint4*>(up + (int64_t)row * ldu + col), u);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float sg = sigmoid_f32(g[i]);
-      og[i] = d[i] * u[i] * sg * fmaf(g[i], 1.0f - sg, 1.0f);
-      ou[i] = d[i] * g[i] * sg;
-    }
+    for (int i = 0; i < 8; ++i) faar_silu_mul_bwd(d[i], g[i], u[i], og[i], ou[i]);
     *reinterpret_cast<uint4*>(dgate + (int64_t)row * lddg + col) = pack8(og);
     *reinterpret_cast<uint4*>(dup + (int64_t)row * lddu + col) = pack8(ou);
   }

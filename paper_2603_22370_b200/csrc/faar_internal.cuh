@@ -200,6 +200,7 @@ int faar_bwd_group(faar_ctx*, int n_seg, faar_bwd_state* seg, int T, int K, cons
                    const void* X, int64_t ldx, void* workspace);
 int faar_check_hparams(const faar_hparams* hp, bool need_opt);
 
+enum { FAAR_GATED_FWD = 1, FAAR_GATED_BWD = 2 };
 enum { FAAR_GEMM_REF = 0, FAAR_GEMM_FWD = 1, FAAR_GEMM_BWD = 2 };
 
 struct faar_gemm_args {
@@ -214,6 +215,8 @@ struct faar_gemm_args {
   void* Yout; int yout_dtype; int64_t ldy;     // REF: [M, ldy]; FWD: [N(T), M(O)] written transposed, nullable
   const void* Yref; int yref_dtype;            // FWD
   int yref_t;                                  // FWD: Y stored transposed [O, ldy]; REF: rows of Yout padded to 16 columns
+  int gated;                                   // REF: an epilogue of the gated product, FAAR_GATED_FWD or FAAR_GATED_BWD (0: plain)
+  void* act; const void* gate_up;              // and its further tensors (see faar_gemm.cu)
   __nv_bfloat16* dYt; int64_t ld_dyt;          // FWD: [M(O), ld_dyt]
   float mse2c;                                 // FWD: 2 * mse_scale
   float act_scale;                             // FWD, BWD: tensor scale of quantised activations (1 = none)
@@ -328,6 +331,21 @@ __device__ __forceinline__ bool faar_elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
   return p != 0;
+}
+
+// sigmoid(x) in FP32: 1 / (1 + e^-x) with the library exponential (relative error ~1e-7) and the hardware
+// reciprocal (rcp.approx: relative error below 2^-22); e^-x overflowing to +inf gives 0, the limit.
+__device__ __forceinline__ float faar_sigmoid(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + expf(-x)));
+  return r;
+}
+// The gated product silu(g) u and its backward: with s = sigmoid(g),  dg = d u s (1 + g (1 - s)),  du = d g s.
+__device__ __forceinline__ float faar_silu_mul(float g, float u) { return g * faar_sigmoid(g) * u; }
+__device__ __forceinline__ void faar_silu_mul_bwd(float d, float g, float u, float& dg, float& du) {
+  const float s = faar_sigmoid(g);
+  dg = d * u * s * fmaf(g, 1.0f - s, 1.0f);
+  du = d * g * s;
 }
 
 __device__ __forceinline__ float faar_warp_sum(float v) {

@@ -30,13 +30,13 @@ Sizes sizes(const faar_model* m, int batch, int seq) {
 // Byte offsets of a block's saved activations inside its part of the arena.
 struct BlockLayout {
   size_t x_in, hn, rstd1, qkv, a, lse, x_mid, rstd2, mn, gu, act, bytes;
-  explicit BlockLayout(const Sizes& s) {
+  BlockLayout(const Sizes& s, bool keep) {
     size_t o = 0;
     auto take = [&](size_t n) { const size_t at = o; o += align256(n); return at; };
     x_in = take(s.T * s.d * 2); hn = take(s.T * s.d * 2); rstd1 = take(s.T * 4);
     qkv = take(s.T * s.qkv * 2); a = take(s.T * s.qd * 2); lse = take(s.seq_rows * 4);
     x_mid = take(s.T * s.d * 2); rstd2 = take(s.T * 4); mn = take(s.T * s.d * 2);
-    gu = take(s.T * 2 * s.f * 2); act = take(s.T * s.f * 2);
+    gu = take(keep ? s.T * 2 * s.f * 2 : 0); act = take(s.T * s.f * 2);      // gate and up: for a backward pass alone
     bytes = o;
   }
 };
@@ -44,7 +44,7 @@ struct BlockLayout {
 struct Arena {
   BlockLayout b;
   size_t parts, x_last, rstd_f, tmp, total;
-  Arena(const Sizes& s, int n_layers, bool keep) : b(s) {
+  Arena(const Sizes& s, int n_layers, bool keep) : b(s, keep) {
     parts = keep ? n_layers : (n_layers < 2 ? n_layers : 2);
     x_last = parts * b.bytes;
     rstd_f = x_last + align256(s.T * s.d * 2);
@@ -53,11 +53,11 @@ struct Arena {
   }
 };
 struct Scratch {
-  size_t dhz, dx, dact, dgu, dn, da, dqkv, dsum, total;
+  size_t dhz, dx, dgu, dn, da, dqkv, dsum, total;
   explicit Scratch(const Sizes& s) {
     size_t o = 0;
     auto take = [&](size_t n) { const size_t at = o; o += align256(n); return at; };
-    dhz = take(s.T * s.d * 2); dx = take(s.T * s.d * 2); dact = take(s.T * s.f * 2); dgu = take(s.T * 2 * s.f * 2);
+    dhz = take(s.T * s.d * 2); dx = take(s.T * s.d * 2); dgu = take(s.T * 2 * s.f * 2);
     dn = take(s.T * s.d * 2); da = take(s.T * s.qd * 2); dqkv = take(s.T * s.qkv * 2); dsum = take(s.seq_rows * 4);
     total = o;
   }
@@ -73,6 +73,33 @@ int product(faar_ctx* ctx, size_t T, int O, int K, const void* X, int64_t ldx, c
   a.B = W; a.ldb = ldw; a.b_mn = w_rows_contract;
   a.status = reinterpret_cast<uint32_t*>(ws);
   a.Yout = Y; a.yout_dtype = FAAR_BF16; a.ldy = ldy;
+  return faar_launch_gemm(ctx, &a, nullptr);
+}
+
+// [gate | up] = X W^T over the stacked weights and act = silu(gate) up; gu null: act alone
+int product_gated(faar_ctx* ctx, size_t T, int f, int K, const void* X, const void* W, void* gu, void* act, void* ws) {
+  faar_gemm_args a = {};
+  a.mode = FAAR_GEMM_REF;
+  a.M = (int)T; a.N = 2 * f; a.Kc = K;
+  a.A = X; a.lda = K;
+  a.B = W; a.ldb = K;
+  a.whole = 1;
+  a.status = reinterpret_cast<uint32_t*>(ws);
+  a.Yout = gu; a.yout_dtype = FAAR_BF16; a.ldy = 2 * f;
+  a.gated = FAAR_GATED_FWD; a.act = act;
+  return faar_launch_gemm(ctx, &a, nullptr);
+}
+// [d gate | d up] of act = silu(gate) up from d act = dY[T, K] W[K, f] (which is not kept) and the forward pass's [gate | up]
+int product_gated_bwd(faar_ctx* ctx, size_t T, int f, int K, const void* dY, const void* W, const void* gu, void* dgu, void* ws) {
+  faar_gemm_args a = {};
+  a.mode = FAAR_GEMM_REF;
+  a.M = (int)T; a.N = f; a.Kc = K;
+  a.A = dY; a.lda = K;
+  a.B = W; a.ldb = f; a.b_mn = 1;
+  a.whole = 1;
+  a.status = reinterpret_cast<uint32_t*>(ws);
+  a.Yout = dgu; a.yout_dtype = FAAR_BF16; a.ldy = 2 * f;
+  a.gated = FAAR_GATED_BWD; a.gate_up = gu;
   return faar_launch_gemm(ctx, &a, nullptr);
 }
 
@@ -117,24 +144,31 @@ int soft_blocks(faar_ctx* ctx, const faar_model* m, const Sizes& s, int l, float
   }
   return items ? faar_launch_soft_weights(ctx, items, item, beta) : 0;
 }
-// A group's forward product with frozen weights, with soft weights (formed already), or with soft weights formed first.
+// A group's operand: frozen weights, soft weights (formed already), or soft weights formed first.
 enum Weights { FROZEN, SOFT, FORM_SOFT };
+int group_operand(faar_ctx* ctx, const faar_linear_group& g, int K, Weights weights, float beta, const void** W) {
+  *W = weights == FROZEN ? g.W : g.Wsoft;
+  if (weights != FORM_SOFT) return 0;
+  faar_soft_item item[FAAR_MAX_SEGMENTS];
+  const int n = soft_items(g, K, item);
+  return faar_launch_soft_weights(ctx, n, item, beta);
+}
 int group_forward(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* X, Weights weights, float beta, void* Y, void* ws) {
   const int rows = group_rows(g);
-  if (weights == FORM_SOFT) {
-    faar_soft_item item[FAAR_MAX_SEGMENTS];
-    const int n = soft_items(g, K, item);
-    const int e = faar_launch_soft_weights(ctx, n, item, beta);
-    if (e) return e;
-  }
-  return product(ctx, T, rows, K, X, K, weights == FROZEN ? g.W : g.Wsoft, K, false, Y, rows, ws);
+  const void* W;
+  const int e = group_operand(ctx, g, K, weights, beta, &W);
+  return e ? e : product(ctx, T, rows, K, X, K, W, K, false, Y, rows, ws);
 }
 // A group's backward: the gradient towards the common input, then the update of every V (at the pre-update soft weights).
+int group_update(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp, void* ws);
 int group_backward(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp,
                    void* dX, void* ws) {
   const int rows = group_rows(g);
-  int e = product(ctx, T, K, rows, dY, rows, g.Wsoft, K, true, dX, K, ws);
-  if (e) return e;
+  const int e = product(ctx, T, K, rows, dY, rows, g.Wsoft, K, true, dX, K, ws);
+  return e ? e : group_update(ctx, g, T, K, dY, X, hp, ws);
+}
+int group_update(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp, void* ws) {
+  const int rows = group_rows(g);
   faar_bwd_state seg[FAAR_MAX_SEGMENTS];
   const int n = segments(g, seg);
   return faar_bwd_group(ctx, n, seg, (int)T, K, hp, dY, rows, X, K, ws);
@@ -229,8 +263,10 @@ int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* t
       e = faar_launch_rmsnorm(ctx, T, s.d, p + A.b.x_in, s.d, tmp, s.d, p + A.b.x_mid, s.d, b.mlp_norm, m->eps, p + A.b.mn, s.d,
                               reinterpret_cast<float*>(p + A.b.rstd2));
     __nv_bfloat16* const gu = reinterpret_cast<__nv_bfloat16*>(p + A.b.gu);
-    if (!e) e = group_forward(ctx, b.gate_up, s.T, s.d, p + A.b.mn, w, beta, gu, ws);
-    if (!e) e = faar_launch_silu_mul(ctx, T, s.f, gu, 2 * s.f, gu + s.f, 2 * s.f, p + A.b.act, s.f);
+    // act = silu(gate) up leaves with the product; gate and up themselves only where a backward pass will read them
+    const void* Wgu = nullptr;
+    if (!e) e = group_operand(ctx, b.gate_up, s.d, w, beta, &Wgu);
+    if (!e) e = product_gated(ctx, s.T, s.f, s.d, p + A.b.mn, Wgu, keep ? gu : nullptr, p + A.b.act, ws);
     if (!e) e = group_forward(ctx, b.down, s.T, s.f, p + A.b.act, w, beta, tmp, ws);
     if (e) break;
     // residual connection and the next block's attention norm (after the last block: the final norm)
@@ -262,9 +298,8 @@ int backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* 
     const __nv_bfloat16* const gu = reinterpret_cast<const __nv_bfloat16*>(p + A.b.gu);
     __nv_bfloat16* const dgu = reinterpret_cast<__nv_bfloat16*>(scratch + S.dgu);
     // MLP branch: x = x_mid + act W_down^T
-    e = group_backward(ctx, b.down, s.T, s.f, dx, p + A.b.act, hp, scratch + S.dact, ws);
-    if (!e)
-      e = faar_launch_silu_mul_bwd(ctx, T, s.f, scratch + S.dact, s.f, gu, 2 * s.f, gu + s.f, 2 * s.f, dgu, 2 * s.f, dgu + s.f, 2 * s.f);
+    e = product_gated_bwd(ctx, s.T, s.f, s.d, dx, b.down.Wsoft, gu, dgu, ws);
+    if (!e) e = group_update(ctx, b.down, s.T, s.f, dx, p + A.b.act, hp, ws);
     if (!e) e = group_backward(ctx, b.gate_up, s.T, s.d, dgu, p + A.b.mn, hp, scratch + S.dn, ws);
     if (!e)
       e = faar_launch_rmsnorm_bwd(ctx, T, s.d, scratch + S.dn, nullptr, nullptr, s.d, p + A.b.x_mid, s.d, b.mlp_norm,
