@@ -210,10 +210,11 @@ faar_prof_scope::faar_prof_scope(faar_ctx* ctx, int kernel_id) : c(ctx), pair(-1
 int faar_check_hparams(const faar_hparams* hp, bool need_opt) { return check_hp(hp, need_opt); }
 
 int faar_bwd_group(faar_ctx* ctx, int n_seg, faar_bwd_state* seg, int T, int K, const faar_hparams* hp, const void* dY, int64_t ldy,
-                   const void* X, int64_t ldx, void* workspace) {
+                   const void* X, int64_t ldx, void* workspace, bool beside) {
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   faar_gemm_args a = {};
   a.mode = FAAR_GEMM_BWD;
+  a.beside = beside;
   for (int i = 0; i < n_seg; ++i) {
     seg[i].lam_over_n = (float)((double)hp->lambda_round / ((double)seg[i].rows * (double)K));
     a.seg[i] = seg[i];

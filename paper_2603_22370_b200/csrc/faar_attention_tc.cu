@@ -519,7 +519,7 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;                         // head_dim 64: S in columns 0..63, dP: 64..127, dQ: 128..191, dS (BF16 pairs): 192..223
-  faar_pdl_sync();                                          // set-up done; now wait for the previous kernel's data
+  faar_pdl_launch();                                        // needs nothing of the dK / dV kernel, next to which it runs
   const uint32_t sQ = base, sDO = base + C::OFF_DO;
   auto sK = [&](int s) { return base + C::OFF_KV + (uint32_t)s * C::STAGE; };
   auto sV = [&](int s) { return sK(s) + KV_BYTES; };
@@ -688,6 +688,7 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C::TMEM) : "memory");
   }
+  if (threadIdx.x == 0) faar_pdl_join();
 }
 
 // ---- backward, dK and dV: one CTA per 128 keys of a key / value head ------------------------------------------
@@ -770,7 +771,7 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
-  faar_pdl_sync();                                          // set-up done; now wait for the previous kernel's data
+  faar_pdl_wait_first();                                    // set-up done; now wait for the previous kernel's data, then let dQ's start
   const uint32_t sKt = base, sVt = base + C::OFF_V;
   auto sQ = [&](int s) { return base + C::OFF_QD + (uint32_t)s * C::STAGE; };
   auto sDO = [&](int s) { return sQ(s) + C::QD_BYTES; };

@@ -358,7 +358,7 @@ struct KParams {
   // REF / FWD
   void* Yout; int yout_dtype; long long ldy;
   const void* Yref; int yref_dtype;
-  int columns;            // REF: Yout is [N, ldy], the accumulator's rows are its columns (compiled in: COLUMNS)
+  int columns;            // REF: Yout is [N, ldy], the accumulator's rows are its columns (compiled in: COLUMNS); BWD: beside
   int yref_t;             // FWD: Y_ref / Y_q stored transposed, [O, ldy] with ldy >= T rounded up to 16; REF: rows of Yout are
                           // padded like that, columns beyond N up to the next multiple of 16 are written as 0
   int y_store;            // REF: rows of Yout take 2: 32-byte stores, 1: 16-byte stores, 0: single values
@@ -1011,7 +1011,10 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   tc_fence_before();
   cluster_sync_all();                                  // barriers of both CTAs are initialised
   tc_fence_after();
-  faar_pdl_sync();                                     // set-up done; now wait for the previous kernel's data
+  // set-up done; now wait for the previous kernel's data
+  if (MODE == FAAR_GEMM_REF) faar_pdl_wait_first();
+  else if (MODE == FAAR_GEMM_BWD && p.columns) faar_pdl_launch();
+  else faar_pdl_sync();
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
@@ -1396,6 +1399,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   }
 
   if constexpr (MODE == FAAR_GEMM_BWD) {
+    if (p.columns && threadIdx.x == 0) faar_pdl_join();
     // Final loss sums by whichever CTA finishes last.  Each adds its Round Loss sum to one word, as a fixed-point number
     // above nine bits that count the CTAs and nine that count sums kept elsewhere.  A sum is rounded to the field's unit
     // (2^-20 for 16 M weights); the addition is exact, so neither the order nor which CTA is last matters, and the last one
@@ -1784,8 +1788,8 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
   faar_gemm_args swapped;
   const faar_gemm_args* a = args;
   KParams kp;
-  kp.columns = args->mode == FAAR_GEMM_REF && result_columns(args);
-  if (kp.columns) {
+  kp.columns = args->mode == FAAR_GEMM_REF ? result_columns(args) : args->mode == FAAR_GEMM_BWD && args->beside;
+  if (args->mode == FAAR_GEMM_REF && kp.columns) {
     swapped = *args;
     swapped.M = args->N; swapped.N = args->M;
     swapped.A = args->B; swapped.lda = args->ldb; swapped.a_mn = args->b_mn;

@@ -196,8 +196,9 @@ int faar_launch_harden_pack(faar_ctx*, const faar_shape*, const float* V, const 
 
 // dW products with chain rule and update on row-major operands dY [T, ldy], X [T, ldx]; the segments' rows stacked in dY's
 // columns.  hp has been checked.
+// beside: the launch before it on the stream is the input gradient of the same dY (a plain product), which it runs next to
 int faar_bwd_group(faar_ctx*, int n_seg, faar_bwd_state* seg, int T, int K, const faar_hparams* hp, const void* dY, int64_t ldy,
-                   const void* X, int64_t ldx, void* workspace);
+                   const void* X, int64_t ldx, void* workspace, bool beside = false);
 int faar_check_hparams(const faar_hparams* hp, bool need_opt);
 
 enum { FAAR_GATED_FWD = 1, FAAR_GATED_BWD = 2 };
@@ -208,6 +209,7 @@ struct faar_gemm_args {
   int M, N, Kc;           // C[M,N] = A[M,Kc] * B[N,Kc]^T, both operands bf16 with Kc contiguous (REF: the launch may exchange them)
   const void* A; int64_t lda;
   const void* B; int64_t ldb;
+  int beside;             // BWD: 1: needs nothing of the launch before it, a plain product (see faar_pdl_wait_first)
   int whole;              // 1: the contraction is not split over CTA pairs (the order of its sums is that of one pair)
   int a_mn, b_mn;         // 1: the operand is stored with M (N) contiguous instead: A[Kc, M] (lda), B[Kc, N] (ldb)
   uint32_t* status;       // workspace status word
@@ -322,6 +324,19 @@ __device__ __forceinline__ void faar_pdl_sync() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+
+// The other order, for a kernel that the next one may run next to (an input gradient and the dW product of the same dY): once
+// every CTA is past its wait, all that came before is complete, so a dependent that needs nothing of THIS kernel starts at
+// once, on the SMs that are free or become so, and only has to wait (faar_pdl_join) before it ends: what follows it then
+// finds both complete.  The dW products of a backward pass next to the input gradients and dQ next to dK / dV, alignment step,
+// us: four 128-wide blocks on 1200 tokens 531 -> 459, two of 512 on 400 357 -> 318, two of 2048 / 8192 on 700 1832 -> 1803, two
+// of 2048 / 6144 on 500 1350 -> 1323, on 2000 2985 -> 2968.
+__device__ __forceinline__ void faar_pdl_wait_first() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void faar_pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void faar_pdl_join() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // One lane of a converged warp.  A warp that issues tensor-core instructions runs its loop with all lanes and guards
 // only those instructions with this, so that the descriptors stay in uniform registers; under `if (lane == 0)` every

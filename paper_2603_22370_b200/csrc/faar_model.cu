@@ -171,7 +171,7 @@ int group_update(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, con
   const int rows = group_rows(g);
   faar_bwd_state seg[FAAR_MAX_SEGMENTS];
   const int n = segments(g, seg);
-  return faar_bwd_group(ctx, n, seg, (int)T, K, hp, dY, rows, X, K, ws);
+  return faar_bwd_group(ctx, n, seg, (int)T, K, hp, dY, rows, X, K, ws, true);
 }
 
 constexpr size_t OVERLAP_LIMIT = 28 << 20;     // see faar_model_overlap
