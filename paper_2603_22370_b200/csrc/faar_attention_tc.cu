@@ -468,6 +468,7 @@ struct TcBwdParams {
   long long ldq, ldk;
   int B, S, H, Hkv;
   float scale_log2, inv_sqrt_d;
+  int apart;                       // dQ: its memory may hold what the dK / dV kernel reads, so it waits for that one
 };
 
 template <int HD>
@@ -519,7 +520,8 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;                         // head_dim 64: S in columns 0..63, dP: 64..127, dQ: 128..191, dS (BF16 pairs): 192..223
-  faar_pdl_launch();                                        // needs nothing of the dK / dV kernel, next to which it runs
+  if (p.apart) faar_pdl_sync();
+  else faar_pdl_launch();                                   // needs nothing of the dK / dV kernel, next to which it runs
   const uint32_t sQ = base, sDO = base + C::OFF_DO;
   auto sK = [&](int s) { return base + C::OFF_KV + (uint32_t)s * C::STAGE; };
   auto sV = [&](int s) { return sK(s) + KV_BYTES; };
@@ -1041,6 +1043,12 @@ int faar_launch_attention_bwd_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, in
   p.dq = reinterpret_cast<__nv_bfloat16*>(dq); p.dk = reinterpret_cast<__nv_bfloat16*>(dk); p.dv = reinterpret_cast<__nv_bfloat16*>(dv);
   p.ldq = ldq; p.ldk = ldk; p.B = B; p.S = S; p.H = H; p.Hkv = Hkv; p.scale_log2 = scale_log2;
   p.inv_sqrt_d = scale_log2 / 1.4426950408889634f;
+  const uintptr_t dq0 = reinterpret_cast<uintptr_t>(dq), rows = (uintptr_t)B * S - 1, dq1 = dq0 + (rows * ldq + (uintptr_t)H * D) * 2;
+  auto meets = [&](const void* a, int64_t ld, int heads) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a);
+    return x < dq1 && dq0 < x + (rows * ld + (uintptr_t)heads * D) * 2;
+  };
+  p.apart = meets(q, ldq, H) || meets(dout, ldo, H) || meets(k, ldk, Hkv) || meets(v, ldk, Hkv);
   return D == 64 ? launch_bwd<64>(ctx, p, q, ldq, k, v, ldk, dout, ldo) : launch_bwd<128>(ctx, p, q, ldq, k, v, ldk, dout, ldo);
 }
 
