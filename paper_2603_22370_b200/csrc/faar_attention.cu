@@ -862,7 +862,7 @@ int launch_fwd(faar_ctx* ctx, const AttnParams& p) {
 }
 
 template <int D>
-int launch_bwd(faar_ctx* ctx, const AttnParams& p, float* dsum) {
+int launch_bwd(faar_ctx* ctx, const AttnParams& p, float* dsum, const float2* rope) {
   faar_prof_scope ps(ctx, FAAR_K_ATTENTION);
   long long rows = (long long)p.B * p.H * ((p.S + 256 / D - 1) / (256 / D));      // warp passes of the row-sum kernel
   long long blocks = (rows + 3) / 4;
@@ -871,7 +871,8 @@ int launch_bwd(faar_ctx* ctx, const AttnParams& p, float* dsum) {
   const int tiles = (p.S + AT - 1) / AT;
   if (ctx->tune_attention_fragments == 0)
     return faar_launch_attention_bwd_tc(ctx, p.B, p.S, p.H, p.Hkv, D, p.q, p.ldq, p.k, p.v, p.ldk, p.dout, p.ldo, p.lse, dsum,
-                                        p.dq, p.dk, p.dv, p.scale_log2);
+                                        p.dq, p.dk, p.dv, p.scale_log2, rope);
+  if (rope) return (int)cudaErrorInvalidValue;
   if (D == HD && ctx->tune_attention_fragments == 2) {
     int e = faar_allow_smem(ctx, (const void*)attn_dkv64_kernel, BWD64_SMEM);
     if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq64_kernel, BWD64_SMEM);
@@ -902,7 +903,7 @@ int faar_launch_attention_fwd(faar_ctx* ctx, int B, int S, int H, int Hkv, int D
 
 int faar_launch_attention_bwd(faar_ctx* ctx, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                               const void* v, int64_t ldk, const void* out, const void* dout, int64_t ldo, const float* lse,
-                              float* dsum, void* dq, void* dk, void* dv) {
+                              float* dsum, void* dq, void* dk, void* dv, const float2* rope) {
   AttnParams p = {};
   p.q = reinterpret_cast<const __nv_bfloat16*>(q); p.k = reinterpret_cast<const __nv_bfloat16*>(k);
   p.v = reinterpret_cast<const __nv_bfloat16*>(v);
@@ -911,5 +912,5 @@ int faar_launch_attention_bwd(faar_ctx* ctx, int B, int S, int H, int Hkv, int D
   p.dq = reinterpret_cast<__nv_bfloat16*>(dq); p.dk = reinterpret_cast<__nv_bfloat16*>(dk); p.dv = reinterpret_cast<__nv_bfloat16*>(dv);
   p.ldq = ldq; p.ldk = ldk; p.ldo = ldo; p.B = B; p.S = S; p.H = H; p.Hkv = Hkv;
   p.scale_log2 = LOG2E / sqrtf((float)D);
-  return D == 64 ? launch_bwd<64>(ctx, p, dsum) : launch_bwd<128>(ctx, p, dsum);
+  return D == 64 ? launch_bwd<64>(ctx, p, dsum, rope) : launch_bwd<128>(ctx, p, dsum, rope);
 }

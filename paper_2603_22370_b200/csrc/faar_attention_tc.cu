@@ -146,6 +146,19 @@ __device__ __forceinline__ void ld32x2(uint32_t ta, uint32_t tb, float (&a)[32],
 #pragma unroll
   for (int i = 0; i < 32; ++i) { a[i] = __uint_as_float(u[i]); b[i] = __uint_as_float(v[i]); }
 }
+__device__ __forceinline__ void ld16x2(uint32_t ta, uint32_t tb, float (&a)[16], float (&b)[16]) {
+  uint32_t u[16], v[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]), "=r"(u[9]), "=r"(u[10]),
+        "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]), "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
+        "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(ta), "r"(tb) : "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) { a[i] = __uint_as_float(u[i]); b[i] = __uint_as_float(v[i]); }
+}
 // 32 consecutive 32-bit columns of this thread's tensor-memory lane, written (BF16 pairs of an A operand)
 __device__ __forceinline__ void st32(uint32_t taddr, const uint32_t (&u)[32]) {
   asm volatile(
@@ -468,8 +481,39 @@ struct TcBwdParams {
   long long ldq, ldk;
   int B, S, H, Hkv;
   float scale_log2, inv_sqrt_d;
+  const float2* rope;              // dq and dk turn back by their row's angles (null: not)
   int apart;                       // dQ: its memory may hold what the dK / dV kernel reads, so it waits for that one
 };
+
+// A gradient's row towards a head before the rotary embedding: this thread's HD / 4 pairs (elements i and i + HD / 2, from
+// i = HD / 4 * half on), turned back from FP32 accumulators in tensor memory (`t`: the head's first column) by the row's `angles`.
+// 4 x 2048 tokens, 32 / 8 heads of 64, us: dK / dV 217 and a pass over dq and dk 17.4 more -> 218.5, dQ 157 -> 160; 2 x 1000, 16 / 8
+// heads of 128: 49.5 + 8.3 -> 51.3, 28.2 -> 30.  (Sines and cosines formed here: dQ 174 and 37; a row's angles side by side: 168, 33.)
+// The first 16 angles are requested before the last product is waited for.
+struct Angles { float2 sc[16]; };
+__device__ __forceinline__ void load_angles(const float2* angles, long long tokens, int c, Angles& v) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v.sc[j] = angles[(c + j) * tokens];
+}
+template <int HD>
+__device__ __forceinline__ void turn_back(const float2* angles, long long tokens, Angles& v, uint32_t t, int half, bool valid, __nv_bfloat16* row) {
+#pragma unroll
+  for (int c = HD / 4 * half; c < HD / 4 * (half + 1); c += 16) {
+    float a[16], b[16];
+    ld16x2(t + (uint32_t)c, t + (uint32_t)(c + HD / 2), a, b);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) faar_rope_turn(a[j], b[j], -v.sc[j].x, v.sc[j].y);
+    if (c + 16 < HD / 4 * (half + 1) && valid) load_angles(angles, tokens, c + 16, v);
+    if (!valid) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      reinterpret_cast<uint4*>(row + c)[h] = make_uint4(pack2(a[8 * h], a[8 * h + 1]), pack2(a[8 * h + 2], a[8 * h + 3]),
+                                                        pack2(a[8 * h + 4], a[8 * h + 5]), pack2(a[8 * h + 6], a[8 * h + 7]));
+      reinterpret_cast<uint4*>(row + HD / 2 + c)[h] = make_uint4(pack2(b[8 * h], b[8 * h + 1]), pack2(b[8 * h + 2], b[8 * h + 3]),
+                                                                 pack2(b[8 * h + 4], b[8 * h + 5]), pack2(b[8 * h + 6], b[8 * h + 7]));
+    }
+  }
+}
 
 template <int HD>
 __global__ void __launch_bounds__(BWD_THREADS, Dq<HD>::CTAS)
@@ -662,6 +706,10 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
       fence_before();
       bar_arrive(bar_ds(j));
     }
+    const long long tokens = (long long)p.B * p.S;
+    const float2* const angles = p.rope ? p.rope + seq0 + qi : nullptr;
+    Angles first;
+    if (angles && qi < p.S) load_angles(angles, tokens, HD / 4 * half, first);
     if (ok) {
       ok = bar_wait(bar_done(n_kt - 1), parity(n_kt - 1), abort_flag, 0xD30u);
       ok = __all_sync(0xffffffffu, ok);
@@ -669,6 +717,8 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (ok) {
       fence_after();
       uint4* dst = reinterpret_cast<uint4*>(p.dq + (seq0 + qi) * p.ldq + h * HD);
+      if (angles) turn_back<HD>(angles, tokens, first, t_lane + (uint32_t)C::COL_DQ, half, qi < p.S, reinterpret_cast<__nv_bfloat16*>(dst));
+      else
 #pragma unroll
       for (int q = 0; q < C::NP; ++q) {                       // this thread's half of the row
         float t[32];
@@ -936,6 +986,10 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       fence_before();
       bar_arrive(bar_pds(i & 1));
     }
+    const long long tokens = (long long)p.B * p.S;
+    const float2* const angles = p.rope ? p.rope + seq0 + kj : nullptr;
+    Angles first;
+    if (angles && kj < p.S) load_angles(angles, tokens, HD / 4 * half, first);
     if (ok) {
       ok = bar_wait(bar_done((n_it - 1) & 1), (uint32_t)(((n_it - 1) >> 1) & 1), abort_flag, 0xF30u);
       ok = __all_sync(0xffffffffu, ok);
@@ -945,6 +999,10 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 #pragma unroll
       for (int which = 0; which < 2; ++which) {
         uint4* dst = reinterpret_cast<uint4*>((which ? p.dk : p.dv) + (seq0 + kj) * p.ldk + g * HD);
+        if (which && angles) {
+          turn_back<HD>(angles, tokens, first, t_lane + (uint32_t)C::COL_DK, half, kj < p.S, reinterpret_cast<__nv_bfloat16*>(dst));
+          break;
+        }
 #pragma unroll
         for (int q = 0; q < C::NP; ++q) {                      // this thread's half of the row
           float t[32];
@@ -1036,9 +1094,10 @@ int faar_launch_attention_fwd_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, in
 
 int faar_launch_attention_bwd_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                                  const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
-                                 const float* dsum, void* dq, void* dk, void* dv, float scale_log2) {
+                                 const float* dsum, void* dq, void* dk, void* dv, float scale_log2, const float2* rope) {
   if ((long long)B * S > 0x7FFFFFFFll) return (int)cudaErrorInvalidValue;
   TcBwdParams p = {};
+  p.rope = rope;
   p.lse = lse; p.dsum = dsum;
   p.dq = reinterpret_cast<__nv_bfloat16*>(dq); p.dk = reinterpret_cast<__nv_bfloat16*>(dk); p.dv = reinterpret_cast<__nv_bfloat16*>(dv);
   p.ldq = ldq; p.ldk = ldk; p.B = B; p.S = S; p.H = H; p.Hkv = Hkv; p.scale_log2 = scale_log2;

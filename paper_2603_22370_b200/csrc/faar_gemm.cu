@@ -79,7 +79,7 @@ constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2, SHORT_TILES = 3,
 constexpr int SHORT_BLOCKS = 40;
 constexpr int SHORT_SMEM = 387 * 512;          // with the system's 1 KB below the 196 KB carve-out
 constexpr int SHORT_CARVEOUT = 85;             // percent of the 228 KB: 193.8, which is rounded up to the size on offer, 196 KB
-constexpr int GATED_FWD = 8, GATED_BWD = 10;   // MN (see the kernel) of the gated product's launches
+constexpr int GATED_FWD = 8, GATED_BWD = 10, ROPE = 16;   // MN (see the kernel) of the gated product's launches and of q / k / v's
 constexpr int GATE_COLS = 32, GATE_PANEL = 32 * GATE_COLS * 2;        // backward: a warp's 32 rows x 32 columns in BF16
 template <int MODE, int SHAPE = PLAIN_TILES, int MN = 0> struct Cfg {
   static constexpr bool WIDE = SHAPE == WIDE_TILES, SHORT = SHAPE == SHORT_TILES, SPLIT = SHAPE == SPLIT_TILES || SHAPE == SPLIT_NARROW;
@@ -606,6 +606,57 @@ __device__ __forceinline__ void epi_gated_bwd(const KParams& p, int row, int col
   if (FAAR_DBG_OK(p, y + p.N, 16, p.Yout, p.ext_yout, 1u)) *reinterpret_cast<uint4*>(y + p.N) = make_uint4(du[0], du[1], du[2], du[3]);
 }
 
+// REF of a block's q / k / v projections: the heads of q and k leave turned by their row's angles (p.Yref: [head_dim / 2, M]
+// sines and cosines, p.yref_dtype: head_dim, p.ld_dyt: columns of q and k; tiles are whole heads).  A warp takes 16 of a head's
+// head_dim / 2 angles at a time, which serve all heads of the tile; the first 16 are requested before the accumulator is
+// ready.  The values of the product rounded to BF16 and faar_rope.  Product and call -> this, us:
+// [8192, 3072] over 2048 69.6 + 17.4 -> 70.2, [2000, 4096] over 2048 28.9 + 8.3 -> 29.8.  (Sines and cosines formed here: 70.8 and
+// 34.0; angles of a row side by side, a line of L1 per lane: 30.6.)
+__device__ __forceinline__ void load_angles(const KParams& p, int row, int c, float2 (&sc)[16]) {
+  if (row >= p.M || c >= p.yref_dtype / 2) return;
+  const float2* t = reinterpret_cast<const float2*>(p.Yref) + (long long)c * p.M + row;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) sc[j] = t[(long long)j * p.M];
+}
+__device__ __forceinline__ void store_row(const KParams& p, int row, int c0, const uint32_t (&w)[8]) {
+  __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Yout) + (long long)row * p.ldy + c0;
+  if (FAAR_DBG_OK(p, y, 32, p.Yout, p.ext_yout, 1u)) stg256(y, w);
+}
+__device__ __forceinline__ void epi_rope(const KParams& p, uint32_t trow, int row, int n0, int width, int cg, int groups, float2 (&sc)[16]) {
+  const int hd = p.yref_dtype, turning = (int)p.ld_dyt - n0, end = min(width, p.N - n0);
+#pragma unroll 1
+  for (int c = 16 * cg; c < hd / 2; c += 16 * groups) {
+    if (c >= 16 * groups) load_angles(p, row, c, sc);
+#pragma unroll 1
+    for (int h = 0; h < end; h += hd) {
+      uint32_t a[16], b[16], lo[8], hi[8];
+      tmem_ld16(trow + (uint32_t)(h + c), a);
+      tmem_ld16(trow + (uint32_t)(h + hd / 2 + c), b);
+      tmem_ld_wait();
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        lo[j] = pack_bf16x2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1]));
+        hi[j] = pack_bf16x2(__uint_as_float(b[2 * j]), __uint_as_float(b[2 * j + 1]));
+      }
+      if (h < turning) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          float x0 = __uint_as_float(lo[j] << 16), x1 = __uint_as_float(lo[j] & 0xFFFF0000u);
+          float y0 = __uint_as_float(hi[j] << 16), y1 = __uint_as_float(hi[j] & 0xFFFF0000u);
+          faar_rope_turn(x0, y0, sc[2 * j].x, sc[2 * j].y);
+          faar_rope_turn(x1, y1, sc[2 * j + 1].x, sc[2 * j + 1].y);
+          lo[j] = pack_bf16x2(x0, x1);
+          hi[j] = pack_bf16x2(y0, y1);
+        }
+      }
+      if (row < p.M) {
+        store_row(p, row, n0 + h + c, lo);
+        store_row(p, row, n0 + h + hd / 2 + c, hi);
+      }
+    }
+  }
+}
+
 // FWD: residual, sum of squares, dY^T.
 // Y_ref[t0..t0+15, o] for this lane's output feature o, as it is in memory: anything done to a value here (widening BF16, a
 // select at the matrix edge) would wait for it here, one latency per chunk of 16 columns.  Forward kernel, row-major target,
@@ -942,7 +993,7 @@ __device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t parts, int
 // MN: bit 0 = the A operand, bit 1 = the B operand is stored with its M / N index contiguous (KParams.a_mn / b_mn);
 // a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.  Bit 2 (REF): the
 // accumulator's rows are the result's columns; compiled in as well (as a branch it cost 0.1 us in every small product).  Bit 3
-// (REF): the gated product's epilogue, forward, or backward where B is N-contiguous.
+// (REF): the gated product's epilogue, forward, or backward where B is N-contiguous.  Bit 4 (REF): heads turn by their position.
 // SHAPE: one of the tile forms (see Cfg).
 constexpr int MIN_SPLIT_BLOCKS = 12;            // contractions of fewer k blocks stay whole (see pick_splits)
 template <int MODE, int OPT, int SHAPE, int MN>
@@ -1208,6 +1259,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int it = 0; it < 4; ++it)
           if (it < gr.steps()) load_gate_up(p, o_quarter + gr.row(lane, it), n0 + col_begin + 8 * gr.unit(lane), gate_end, ahead[it]);
       }
+      float2 angles[MN == ROPE ? 16 : 1];
+      if constexpr (MN == ROPE) load_angles(p, o, 16 * cg, angles);
       bool ok = mbar_wait(tfull_bar(acc), acc_phase, ac, 0x400u | acc);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -1302,6 +1355,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
           __syncwarp();
         }
+      } else if constexpr (MN == ROPE) {
+        epi_rope(p, trow, o, n0, tc.w, cg, C::COL_GROUPS, angles);
       } else if constexpr (GATED) {
         // the warps of a lane quarter take 16 features of the tile in turn
         const int half = tc.w / 2, f0 = n0 / 2;
@@ -1641,7 +1696,8 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   kp.stages = ring < MAX_STAGES ? ring : MAX_STAGES;
   const int m_tiles = (a->M + 2 * BM - 1) / (2 * BM), n_cols = (a->N + bn - 1) / bn;
   const int wide_w1 = kp.n_main, wide_w = BN_MAX + wide_w1, wide_cols = (a->N + wide_w - 1) / wide_w;
-  kp.narrow = (SHAPE == PLAIN_TILES || SHAPE == SHORT_TILES) && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
+  const bool halves = MN != ROPE || bn / 2 % a->head_dim == 0;       // a half-width tile, too, is whole heads
+  kp.narrow = (SHAPE == PLAIN_TILES || SHAPE == SHORT_TILES) && halves && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
   kp.n_main = WIDE ? wide_w1 : n_cols - kp.narrow;
   if (MODE == FAAR_GEMM_BWD) {
     // the widest unit at which the Round Loss field holds one per weight of the tiles (half tiles counted as whole: twice
@@ -1651,7 +1707,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
     while (area >> int_bits) ++int_bits;
     kp.fin_unit = ldexp(1.0, 62 - 2 * FIN_COUNT_BITS - int_bits); kp.fin_inv_unit = 1.0 / kp.fin_unit;
   }
-  kp.n_full = WIDE ? 0 : (SPLIT ? m_tiles * kp.n_main : pick_full(ctx, MODE, m_tiles, kp.n_main, kp.narrow, bn, max_pairs));
+  kp.n_full = WIDE ? 0 : (SPLIT || !halves ? m_tiles * kp.n_main : pick_full(ctx, MODE, m_tiles, kp.n_main, kp.narrow, bn, max_pairs));
   CUtensorMap tmA, tmB, tmBh;
   e = a->a_mn ? make_map_mn(ctx, &tmA, a->A, a->Kc, a->M, a->lda) : make_map(ctx, &tmA, a->A, a->M, a->Kc, a->lda, BM);
   if (e) return e;
@@ -1742,6 +1798,10 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
       if (bn != 32) bn = (bn + 63) / 64 * 64;
       return launch_variant<MODE, OPT, PLAIN_TILES, GATED_FWD>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
     }
+    if (a->rope) {                                  // whole heads
+      bn = (bn + a->head_dim - 1) / a->head_dim * a->head_dim;
+      return launch_variant<MODE, OPT, PLAIN_TILES, ROPE>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+    }
     if (a->gated == FAAR_GATED_BWD) return launch_variant<MODE, OPT, PLAIN_TILES, GATED_BWD>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   }
   // which operand layouts a mode is ever launched with: the plain product with B untransposed (input gradient; A, if the
@@ -1772,7 +1832,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
 // would be padding that is staged all the same.  M on the accumulator's rows -> N, us: 1 row of 8192 over 2048 15.1 -> 10.6,
 // 64 rows 12.8 -> 12.0, 128 rows 13.1 -> 12.2, 160 rows 13.1 -> 13.8; input gradient of 8 rows of 8192 over 2048 14.5 -> 11.9.
 static bool result_columns(const faar_gemm_args* a) {
-  if (a->yref_t || a->gated) return false;
+  if (a->yref_t || a->gated || a->rope) return false;
   const long long row = a->ldy * (a->yout_dtype == FAAR_BF16 ? 2 : 4);
   return a->M <= BM || row % 16 != 0 || (reinterpret_cast<uintptr_t>(a->Yout) & 15) != 0;
 }
@@ -1803,6 +1863,10 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
         a->yout_dtype != FAAR_BF16 || (a->gated == FAAR_GATED_FWD ? !a->act || a->N % 2 : !a->Yout || !a->gate_up))
       return (int)cudaErrorInvalidValue;
   }
+  if (a->rope && (a->mode != FAAR_GEMM_REF || !a->whole || a->a_mn || a->b_mn || a->gated || (a->head_dim != 64 && a->head_dim != 128) ||
+                      a->N % a->head_dim || (reinterpret_cast<uintptr_t>(a->rope) & 7) || a->rope_cols % a->head_dim || a->ldy % 16 || (reinterpret_cast<uintptr_t>(a->Yout) & 31) ||
+                      a->yout_dtype != FAAR_BF16))
+    return (int)cudaErrorInvalidValue;
   kp.M = a->M; kp.N = a->N; kp.Kc = a->Kc; kp.bn = BN_MAX; kp.n_main = kp.narrow = kp.n_full = 0; kp.status = a->status;
   {
     const long long ysz = a->yout_dtype == FAAR_BF16 ? 2 : 4;
@@ -1820,6 +1884,9 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
   kp.Yout = a->Yout; kp.yout_dtype = a->yout_dtype; kp.ldy = a->ldy;
   kp.Yref = a->Yref; kp.yref_dtype = a->yref_dtype; kp.yref_t = a->yref_t;
   kp.dYt = a->dYt; kp.ld_dyt = a->ld_dyt; kp.mse2c = a->mse2c; kp.act_scale = a->act_scale; kp.partials = a->partials;
+  if (a->rope) {
+    kp.Yref = a->rope; kp.yref_dtype = a->head_dim; kp.ld_dyt = a->rope_cols;
+  }
   if (a->gated == FAAR_GATED_FWD) {
     kp.dYt = reinterpret_cast<__nv_bfloat16*>(a->act); kp.ld_dyt = a->N / 2;
     kp.ext_dyt = (long long)a->M * a->N;

@@ -354,7 +354,7 @@ rope_kernel(const __nv_bfloat16* x, int64_t ldx, const int* __restrict__ pos, __
   const int64_t off = (int64_t)chunk * HPT * head_dim + 8 * gi;
   float inv_freq[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) inv_freq[i] = exp2f(-2.0f * (float)(8 * gi + i) / (float)head_dim * log2_theta);
+  for (int i = 0; i < 8; ++i) inv_freq[i] = faar_rope_frequency(8 * gi + i, head_dim, log2_theta);
   for (int row = split_row0(); row < rows; row += split_row_step()) {
     const __nv_bfloat16* xr = x + (int64_t)row * ldx + off;
     __nv_bfloat16* yr = y + (int64_t)row * ldy + off;
@@ -373,16 +373,13 @@ rope_kernel(const __nv_bfloat16* x, int64_t ldx, const int* __restrict__ pos, __
     }
 #pragma unroll
     for (int h = 0; h < HPT; ++h) {
-      float a[8], b[8], oa[8], ob[8];
+      float a[8], b[8];
       unpack8(ra[h], a);
       unpack8(rb[h], b);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        oa[i] = a[i] * cs[i] - b[i] * sn[i];
-        ob[i] = b[i] * cs[i] + a[i] * sn[i];
-      }
-      *reinterpret_cast<uint4*>(yr + h * head_dim) = pack8(oa);
-      *reinterpret_cast<uint4*>(yr + h * head_dim + half) = pack8(ob);
+      for (int i = 0; i < 8; ++i) faar_rope_turn(a[i], b[i], sn[i], cs[i]);
+      *reinterpret_cast<uint4*>(yr + h * head_dim) = pack8(a);
+      *reinterpret_cast<uint4*>(yr + h * head_dim + half) = pack8(b);
     }
   }
 }
@@ -408,11 +405,25 @@ silu_mul_bwd_kernel(const __nv_bfloat16* dout, int64_t ldd, const __nv_bfloat16*
 }
 
 // ---- embedding: out[t, :] = table[tokens[t], :]; a token outside [0, vocab) gives a row of zeros --------
+// A model's pass starts with it, so it also leaves the rotary angles of every row (an angle's rows side by side), which all blocks' products and attention
+// kernels read: one sine and cosine per token and angle instead of one per token, angle and few heads.
 __global__ void __launch_bounds__(GL_THREADS)
 embedding_kernel(const __nv_bfloat16* __restrict__ table, int64_t ldt, const int* __restrict__ tokens, int vocab,
-                 __nv_bfloat16* __restrict__ out, int64_t ldo, int rows, int groups) {
+                 __nv_bfloat16* __restrict__ out, int64_t ldo, int rows, int groups, const int* __restrict__ pos, int head_dim,
+                 float log2_theta, float2* __restrict__ rope) {
   faar_pdl_sync();
   const int cg = split_group();
+  if (rope) {
+    // threads side by side take neighbouring rows, as the rows' lanes will read them
+    const int threads = blockDim.x * blockDim.y, id = threadIdx.y * blockDim.x + threadIdx.x;
+    const int64_t all = (int64_t)rows * (head_dim / 2), step = (int64_t)gridDim.x * gridDim.y * threads;
+    for (int64_t k = (int64_t)(blockIdx.y * gridDim.x + blockIdx.x) * threads + id; k < all; k += step) {
+      const int i = (int)(k / rows), row = (int)(k - (int64_t)i * rows);
+      float2 sc;
+      sincosf((float)pos[row] * faar_rope_frequency(i, head_dim, log2_theta), &sc.x, &sc.y);
+      rope[k] = sc;
+    }
+  }
   if (cg >= groups) return;
   const int col = 8 * cg;
   for (int row = split_row0(); row < rows; row += split_row_step()) {
@@ -541,12 +552,12 @@ int faar_launch_silu_mul_bwd(faar_ctx* ctx, int rows, int cols, const void* dout
 }
 
 int faar_launch_embedding(faar_ctx* ctx, int rows, int cols, int vocab, const void* table, int64_t ldt, const int* tokens,
-                          void* out, int64_t ldo) {
+                          void* out, int64_t ldo, const int* pos, int head_dim, float theta, float2* rope) {
   faar_prof_scope ps(ctx, FAAR_K_GLUE);
   const Split sp = glue_split(ctx, rows, cols / 8);
   faar_launch_pdl(ctx, embedding_kernel, sp.grid, sp.block, 0, 
       reinterpret_cast<const __nv_bfloat16*>(table), ldt, tokens, vocab, reinterpret_cast<__nv_bfloat16*>(out), ldo, rows,
-      cols / 8);
+      cols / 8, pos, head_dim, rope ? log2f(theta) : 0.f, rope);
   return (int)cudaGetLastError();
 }
 

@@ -142,9 +142,10 @@ int faar_launch_nvfp4_expand(faar_ctx*, int rows, int K, const uint8_t* packed, 
 // head_dim D = 64 or 128 on the tcgen05 tensor cores
 int faar_launch_attention_fwd_tc(faar_ctx*, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                                  const void* v, int64_t ldk, void* out, int64_t ldo, float* lse, float scale_log2);
+// rope: dq and dk turn back by their row's angles, [D / 2, B S] sines and cosines, on the way out (null: they don't)
 int faar_launch_attention_bwd_tc(faar_ctx*, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                                  const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
-                                 const float* dsum, void* dq, void* dk, void* dv, float scale_log2);
+                                 const float* dsum, void* dq, void* dk, void* dv, float scale_log2, const float2* rope);
 int faar_attention_tc_status(uint32_t* code_out);
 int faar_launch_softquant_eval(faar_ctx*, const faar_shape*, const float* V, const uint8_t* code,
                                const uint8_t* scales, const float* s_global, float beta,
@@ -175,15 +176,16 @@ int faar_launch_rope(faar_ctx*, int rows, int n_heads, int head_dim, const void*
                      int inverse, void* y, int64_t ldy);
 int faar_launch_silu_mul_bwd(faar_ctx*, int rows, int cols, const void* dout, int64_t ldd, const void* gate, int64_t ldg,
                              const void* up, int64_t ldu, void* dgate, int64_t lddg, void* dup, int64_t lddu);
+// rope (nullable): also the sine and cosine of every row's head_dim / 2 rotary angles, [head_dim / 2, rows]
 int faar_launch_embedding(faar_ctx*, int rows, int cols, int vocab, const void* table, int64_t ldt, const int* tokens,
-                          void* out, int64_t ldo);
+                          void* out, int64_t ldo, const int* pos = nullptr, int head_dim = 0, float theta = 0.f, float2* rope = nullptr);
 int faar_launch_add(faar_ctx*, int rows, int cols, const void* a, int64_t lda, const void* b, int64_t ldb, void* out,
                     int64_t ldo);
 int faar_launch_attention_fwd(faar_ctx*, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                               const void* v, int64_t ldk, void* out, int64_t ldo, float* lse);
 int faar_launch_attention_bwd(faar_ctx*, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                               const void* v, int64_t ldk, const void* out, const void* dout, int64_t ldo, const float* lse,
-                              float* dsum, void* dq, void* dk, void* dv);
+                              float* dsum, void* dq, void* dk, void* dv, const float2* rope = nullptr);
 int faar_launch_nvfp4_gemm(faar_ctx*, int M, int N, int K, const uint8_t* A, const uint8_t* sfa, const float* sa,
                            const uint8_t* B, const uint8_t* sfb, const float* sb, void* C, int64_t ldc, uint32_t* status);
 int faar_launch_round_partials(faar_ctx*, const float* V, int64_t N, float* partials, int* n_partials);
@@ -219,6 +221,8 @@ struct faar_gemm_args {
   int yref_t;                                  // FWD: Y stored transposed [O, ldy]; REF: rows of Yout padded to 16 columns
   int gated;                                   // REF: an epilogue of the gated product, FAAR_GATED_FWD or FAAR_GATED_BWD (0: plain)
   void* act; const void* gate_up;              // and its further tensors (see faar_gemm.cu)
+  const float2* rope;                          // REF: the first rope_cols columns of the result are heads that turn by their row's
+  int rope_cols, head_dim;                     // angles, [head_dim / 2, M] sines and cosines (null: none do)
   __nv_bfloat16* dYt; int64_t ld_dyt;          // FWD: [M(O), ld_dyt]
   float mse2c;                                 // FWD: 2 * mse_scale
   float act_scale;                             // FWD, BWD: tensor scale of quantised activations (1 = none)
@@ -361,6 +365,17 @@ __device__ __forceinline__ void faar_silu_mul_bwd(float d, float g, float u, flo
   const float s = faar_sigmoid(g);
   dg = d * u * s * fmaf(g, 1.0f - s, 1.0f);
   du = d * g * s;
+}
+
+// Rotary position embedding, half-split pairing: element i (i < head_dim / 2) of a head and element i + head_dim / 2 turn by
+// pos theta^(-2 i / head_dim); the backward pass of an orthogonal map is the rotation by the negative angle.
+__device__ __forceinline__ float faar_rope_frequency(int i, int head_dim, float log2_theta) {
+  return exp2f(-2.0f * (float)i / (float)head_dim * log2_theta);
+}
+__device__ __forceinline__ void faar_rope_turn(float& a, float& b, float sn, float cs) {
+  const float x = fmaf(a, cs, -(b * sn)), y = fmaf(b, cs, a * sn);
+  a = x;
+  b = y;
 }
 
 __device__ __forceinline__ float faar_warp_sum(float v) {

@@ -15,14 +15,14 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 struct Sizes {
   size_t T;
-  int d, qd, kvd, qkv, f, H;
+  int d, qd, kvd, qkv, f, H, hd;
   size_t seq_rows;                            // floats of one lse array
 };
 Sizes sizes(const faar_model* m, int batch, int seq) {
   Sizes s;
   s.T = (size_t)batch * seq;
   s.d = m->hidden; s.qd = m->n_heads * m->head_dim; s.kvd = m->n_kv_heads * m->head_dim; s.qkv = s.qd + 2 * s.kvd; s.f = m->ffn;
-  s.H = m->n_heads;
+  s.H = m->n_heads; s.hd = m->head_dim;
   s.seq_rows = s.T * m->n_heads;
   return s;
 }
@@ -40,16 +40,17 @@ struct BlockLayout {
     bytes = o;
   }
 };
-// keep: one part per block, then the final norm's input and rstd, then the temporary; otherwise two parts used in turn.
+// keep: one part per block, then the final norm's input and rstd, the temporary and the rotary angles; otherwise two parts used in turn.
 struct Arena {
   BlockLayout b;
-  size_t parts, x_last, rstd_f, tmp, total;
+  size_t parts, x_last, rstd_f, tmp, rope, total;
   Arena(const Sizes& s, int n_layers, bool keep) : b(s, keep) {
     parts = keep ? n_layers : (n_layers < 2 ? n_layers : 2);
     x_last = parts * b.bytes;
     rstd_f = x_last + align256(s.T * s.d * 2);
     tmp = rstd_f + align256(s.T * 4);
-    total = tmp + align256(s.T * s.d * 2);
+    rope = tmp + align256(s.T * s.d * 2);
+    total = rope + align256(s.T * s.hd / 2 * sizeof(float2));
   }
 };
 struct Scratch {
@@ -87,6 +88,19 @@ int product_gated(faar_ctx* ctx, size_t T, int f, int K, const void* X, const vo
   a.status = reinterpret_cast<uint32_t*>(ws);
   a.Yout = gu; a.yout_dtype = FAAR_BF16; a.ldy = 2 * f;
   a.gated = FAAR_GATED_FWD; a.act = act;
+  return faar_launch_gemm(ctx, &a, nullptr);
+}
+// [q | k | v] = X W^T over the stacked weights, the heads of q and k turned by their row's angles
+int product_rope(faar_ctx* ctx, const faar_model* m, const Sizes& s, const void* X, const void* W, const float2* rope, void* qkv, void* ws) {
+  faar_gemm_args a = {};
+  a.mode = FAAR_GEMM_REF;
+  a.M = (int)s.T; a.N = s.qkv; a.Kc = s.d;
+  a.A = X; a.lda = s.d;
+  a.B = W; a.ldb = s.d;
+  a.whole = 1;
+  a.status = reinterpret_cast<uint32_t*>(ws);
+  a.Yout = qkv; a.yout_dtype = FAAR_BF16; a.ldy = s.qkv;
+  a.rope = rope; a.rope_cols = s.qd + s.kvd; a.head_dim = m->head_dim;
   return faar_launch_gemm(ctx, &a, nullptr);
 }
 // [d gate | d up] of act = silu(gate) up from d act = dY[T, K] W[K, f] (which is not kept) and the forward pass's [gate | up]
@@ -235,7 +249,8 @@ int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* t
   auto part = [&](int l) { return arena + (keep ? l : l % (int)A.parts) * A.b.bytes; };
   uint8_t* const tmp = arena + A.tmp;
   uint8_t* p = part(0);
-  int e = faar_launch_embedding(ctx, T, s.d, m->vocab, m->embed, s.d, tokens, p + A.b.x_in, s.d);
+  float2* const rope = reinterpret_cast<float2*>(arena + A.rope);
+  int e = faar_launch_embedding(ctx, T, s.d, m->vocab, m->embed, s.d, tokens, p + A.b.x_in, s.d, pos, s.hd, m->theta, rope);
   if (!e)
     e = faar_launch_rmsnorm(ctx, T, s.d, p + A.b.x_in, s.d, nullptr, 0, nullptr, 0, m->blocks[0].attn_norm, m->eps, p + A.b.hn, s.d,
                             reinterpret_cast<float*>(p + A.b.rstd1));
@@ -251,9 +266,9 @@ int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* t
     }
     const Weights w = !quantised ? FROZEN : (l < soft_end ? SOFT : FORM_SOFT);
     __nv_bfloat16* const qkv = reinterpret_cast<__nv_bfloat16*>(p + A.b.qkv);
-    e = group_forward(ctx, b.qkv, s.T, s.d, p + A.b.hn, w, beta, qkv, ws);
-    // q and k lie side by side: their heads turn in one launch
-    if (!e) e = faar_launch_rope(ctx, T, m->n_heads + m->n_kv_heads, m->head_dim, qkv, s.qkv, pos, m->theta, 0, qkv, s.qkv);
+    const void *Wqkv = nullptr, *Wgu = nullptr;
+    e = group_operand(ctx, b.qkv, s.d, w, beta, &Wqkv);
+    if (!e) e = product_rope(ctx, m, s, p + A.b.hn, Wqkv, rope, qkv, ws);
     if (!e)
       e = faar_launch_attention_fwd(ctx, batch, seq, m->n_heads, m->n_kv_heads, m->head_dim, qkv, s.qkv, qkv + s.qd, qkv + s.qd + s.kvd,
                                     s.qkv, p + A.b.a, s.qd, reinterpret_cast<float*>(p + A.b.lse));
@@ -264,7 +279,6 @@ int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* t
                               reinterpret_cast<float*>(p + A.b.rstd2));
     __nv_bfloat16* const gu = reinterpret_cast<__nv_bfloat16*>(p + A.b.gu);
     // act = silu(gate) up leaves with the product; gate and up themselves only where a backward pass will read them
-    const void* Wgu = nullptr;
     if (!e) e = group_operand(ctx, b.gate_up, s.d, w, beta, &Wgu);
     if (!e) e = product_gated(ctx, s.T, s.f, s.d, p + A.b.mn, Wgu, keep ? gu : nullptr, p + A.b.act, ws);
     if (!e) e = group_forward(ctx, b.down, s.T, s.f, p + A.b.act, w, beta, tmp, ws);
@@ -308,11 +322,14 @@ int backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* 
     if (!e) e = group_backward(ctx, b.o, s.T, s.qd, dx, p + A.b.a, hp, scratch + S.da, ws);
     const __nv_bfloat16* const qkv = reinterpret_cast<const __nv_bfloat16*>(p + A.b.qkv);
     __nv_bfloat16* const dqkv = reinterpret_cast<__nv_bfloat16*>(scratch + S.dqkv);
+    // the tcgen05 kernels turn dq and dk back on the way out; the others leave that to a pass over both, which lie side by side
+    const bool turned = ctx->tune_attention_fragments == 0;
     if (!e)
       e = faar_launch_attention_bwd(ctx, batch, seq, m->n_heads, m->n_kv_heads, m->head_dim, qkv, s.qkv, qkv + s.qd, qkv + s.qd + s.kvd,
                                     s.qkv, p + A.b.a, scratch + S.da, s.qd, reinterpret_cast<const float*>(p + A.b.lse),
-                                    reinterpret_cast<float*>(scratch + S.dsum), dqkv, dqkv + s.qd, dqkv + s.qd + s.kvd);
-    if (!e) e = faar_launch_rope(ctx, T, m->n_heads + m->n_kv_heads, m->head_dim, dqkv, s.qkv, pos, m->theta, 1, dqkv, s.qkv);
+                                    reinterpret_cast<float*>(scratch + S.dsum), dqkv, dqkv + s.qd, dqkv + s.qd + s.kvd,
+                                    turned ? reinterpret_cast<const float2*>(arena + A.rope) : nullptr);
+    if (!e && !turned) e = faar_launch_rope(ctx, T, m->n_heads + m->n_kv_heads, m->head_dim, dqkv, s.qkv, pos, m->theta, 1, dqkv, s.qkv);
     if (!e) e = group_backward(ctx, b.qkv, s.T, s.d, dqkv, p + A.b.hn, hp, scratch + S.dn, ws);
     if (!e)
       e = faar_launch_rmsnorm_bwd(ctx, T, s.d, scratch + S.dn, nullptr, nullptr, s.d, p + A.b.x_in, s.d, b.attn_norm,

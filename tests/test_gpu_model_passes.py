@@ -1,5 +1,5 @@
 """The passes of a model against the same passes strung together from the library's single calls: what a pass's products do
-in their epilogues (the gated product and its backward) has to give the values of the element-wise calls, over token counts and
+in their epilogues (the gated product and its backward, rotary embedding) has to give the values of the element-wise calls, over token counts and
 widths that fill no tile, one tile, several, and over the width choices of the launches."""
 import pytest
 import torch
@@ -169,4 +169,7 @@ def test_a_models_passes_are_those_of_its_single_calls(ctx, batch, seq, hidden, 
         faar.tune_wide_tiles(ctx, -1)
     assert torch.equal(H_fp, Hr_fp) and torch.equal(Z_fp, Zr_fp) and torch.equal(H, Hr) and torch.equal(Z, Zr)
     worst = max(rel(got[k], want[k]) for k in want)
-    assert worst <= 1e-5, worst            # the dW products' FP32 sums may be split differently
+    # dq and dk turn back before their rounding to BF16, the single calls round before and after: up to 2^-9 of an element, and as
+    # much again wherever one of the gradients formed from them (of the norm, gate / up, the attention output) rounds differently
+    assert worst <= 4 * 2.0**-9, worst
+    assert max(rel(got[1, n], want[1, n]) for n in ("o_proj", "gate_proj", "up_proj", "down_proj")) <= 1e-5      # (before any attention gradient)
