@@ -332,9 +332,10 @@ __device__ __forceinline__ void faar_pdl_sync() {
 // The other order, for a kernel that the next one may run next to (an input gradient and the dW product of the same dY): once
 // every CTA is past its wait, all that came before is complete, so a dependent that needs nothing of THIS kernel starts at
 // once, on the SMs that are free or become so, and only has to wait (faar_pdl_join) before it ends: what follows it then
-// finds both complete.  The dW products of a backward pass next to the input gradients and dQ next to dK / dV, alignment step,
-// us: four 128-wide blocks on 1200 tokens 531 -> 459, two of 512 on 400 357 -> 318, two of 2048 / 8192 on 700 1832 -> 1803, two
-// of 2048 / 6144 on 500 1350 -> 1323, on 2000 2985 -> 2968.
+// finds both complete.  Several may follow one another like this.  The dW products of a backward pass next to the input
+// gradients and dQ next to dK / dV, alignment step, us: four 128-wide blocks on 1200 tokens 531 -> 459, two of 512 on 400 357 -> 318,
+// two of 2048 / 8192 on 700 1832 -> 1803, two of 2048 / 6144 on 500 1350 -> 1323; with two dW products next to gate / up's input
+// gradient, and the output projection's next to dQ, 436 -> 403, 306 -> 283, 1775 -> 1770 and 1303 -> 1291.
 __device__ __forceinline__ void faar_pdl_wait_first() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -174,18 +174,20 @@ int group_forward(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, co
   return e ? e : product(ctx, T, rows, K, X, K, W, K, false, Y, rows, ws);
 }
 // A group's backward: the gradient towards the common input, then the update of every V (at the pre-update soft weights).
-int group_update(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp, void* ws);
+int group_update(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp, void* ws,
+                 bool beside = true);
 int group_backward(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp,
                    void* dX, void* ws) {
   const int rows = group_rows(g);
   const int e = product(ctx, T, K, rows, dY, rows, g.Wsoft, K, true, dX, K, ws);
   return e ? e : group_update(ctx, g, T, K, dY, X, hp, ws);
 }
-int group_update(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp, void* ws) {
+int group_update(faar_ctx* ctx, const faar_linear_group& g, size_t T, int K, const void* dY, const void* X, const faar_hparams* hp, void* ws,
+                 bool beside) {
   const int rows = group_rows(g);
   faar_bwd_state seg[FAAR_MAX_SEGMENTS];
   const int n = segments(g, seg);
-  return faar_bwd_group(ctx, n, seg, (int)T, K, hp, dY, rows, X, K, ws, true);
+  return faar_bwd_group(ctx, n, seg, (int)T, K, hp, dY, rows, X, K, ws, beside);
 }
 
 constexpr size_t OVERLAP_LIMIT = 28 << 20;     // see faar_model_overlap
@@ -313,13 +315,13 @@ int backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* 
     __nv_bfloat16* const dgu = reinterpret_cast<__nv_bfloat16*>(scratch + S.dgu);
     // MLP branch: x = x_mid + act W_down^T
     e = product_gated_bwd(ctx, s.T, s.f, s.d, dx, b.down.Wsoft, gu, dgu, ws);
-    if (!e) e = group_update(ctx, b.down, s.T, s.f, dx, p + A.b.act, hp, ws);
     if (!e) e = group_backward(ctx, b.gate_up, s.T, s.d, dgu, p + A.b.mn, hp, scratch + S.dn, ws);
+    if (!e) e = group_update(ctx, b.down, s.T, s.f, dx, p + A.b.act, hp, ws);       // next to the two before it
     if (!e)
       e = faar_launch_rmsnorm_bwd(ctx, T, s.d, scratch + S.dn, nullptr, nullptr, s.d, p + A.b.x_mid, s.d, b.mlp_norm,
                                   reinterpret_cast<const float*>(p + A.b.rstd2), dx, s.d, dx, s.d);
     // attention branch: x_mid = x_in + a W_o^T
-    if (!e) e = group_backward(ctx, b.o, s.T, s.qd, dx, p + A.b.a, hp, scratch + S.da, ws);
+    if (!e) e = product(ctx, s.T, s.qd, s.d, dx, s.d, b.o.Wsoft, s.qd, true, scratch + S.da, s.qd, ws);
     const __nv_bfloat16* const qkv = reinterpret_cast<const __nv_bfloat16*>(p + A.b.qkv);
     __nv_bfloat16* const dqkv = reinterpret_cast<__nv_bfloat16*>(scratch + S.dqkv);
     // the tcgen05 kernels turn dq and dk back on the way out; the others leave that to a pass over both, which lie side by side
@@ -329,6 +331,8 @@ int backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* 
                                     s.qkv, p + A.b.a, scratch + S.da, s.qd, reinterpret_cast<const float*>(p + A.b.lse),
                                     reinterpret_cast<float*>(scratch + S.dsum), dqkv, dqkv + s.qd, dqkv + s.qd + s.kvd,
                                     turned ? reinterpret_cast<const float2*>(arena + A.rope) : nullptr);
+    if (!e && turned) e = group_update(ctx, b.o, s.T, s.qd, dx, p + A.b.a, hp, ws);          // next to dQ (and so to dK / dV)
+    if (!e && !turned) e = group_update(ctx, b.o, s.T, s.qd, dx, p + A.b.a, hp, ws, false);
     if (!e && !turned) e = faar_launch_rope(ctx, T, m->n_heads + m->n_kv_heads, m->head_dim, dqkv, s.qkv, pos, m->theta, 1, dqkv, s.qkv);
     if (!e) e = group_backward(ctx, b.qkv, s.T, s.d, dqkv, p + A.b.hn, hp, scratch + S.dn, ws);
     if (!e)
