@@ -33,6 +33,9 @@ struct AlignParams {
   float gscale;            // lambda_kl / (tau T)
   float* kl_partials;      // one per cluster (or CTA)
   float* mse_partials;
+  float* loss_out2;        // {KL / T, MSE}: written by the cluster that finishes last
+  uint32_t* finished;      // workspace: clusters that have, zero between launches
+  float kl_scale;
   int T;                   // tokens; cluster k takes tokens k, k + the number of clusters, ...
 };
 
@@ -270,12 +273,34 @@ align_loss_kernel(const AlignParams p) {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
-  if (rank == 0 && threadIdx.x == 0) {
-    float a = 0.f, b = 0.f;
+  // The two loss values, in a fixed order in double, by whichever cluster finishes last: a launch of its own for a few hundred
+  // sums cost a small model's step as much as any other.
+  if (rank == 0 && warp == 0) {
+    uint32_t done = 0u;
+    if (lane == 0) {
+      float a = 0.f, b = 0.f;
 #pragma unroll
-    for (int c = 0; c < CL; ++c) { a += tot[c][0]; b += tot[c][1]; }
-    p.kl_partials[blockIdx.x / CL] = a * 0.6931471805599453f;      // log2 -> natural log
-    p.mse_partials[blockIdx.x / CL] = b;
+      for (int c = 0; c < CL; ++c) { a += tot[c][0]; b += tot[c][1]; }
+      p.kl_partials[blockIdx.x / CL] = a * 0.6931471805599453f;    // log2 -> natural log
+      p.mse_partials[blockIdx.x / CL] = b;
+      __threadfence();
+      done = atomicAdd(p.finished, 1u) + 1u;
+    }
+    if (__shfl_sync(0xffffffffu, done, 0) == (uint32_t)n_cl) {
+      __threadfence();
+      double kl_sum = 0.0, mse_sum = 0.0;
+      for (int c = lane; c < n_cl; c += 32) { kl_sum += (double)__ldcg(p.kl_partials + c); mse_sum += (double)__ldcg(p.mse_partials + c); }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        kl_sum += __shfl_xor_sync(0xffffffffu, kl_sum, o);
+        mse_sum += __shfl_xor_sync(0xffffffffu, mse_sum, o);
+      }
+      if (lane == 0) {
+        p.loss_out2[0] = (float)(kl_sum * (double)p.kl_scale);
+        p.loss_out2[1] = (float)mse_sum;
+        *p.finished = 0u;                                          // ready for the next launch
+      }
+    }
   }
 }
 
@@ -283,7 +308,7 @@ align_loss_kernel(const AlignParams p) {
 
 int faar_launch_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
                            const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, void* dZ_q,
-                           void* dH_q, float* kl_partials, float* mse_partials, int* n_partials) {
+                           void* dH_q, float* kl_partials, float* mse_partials, uint32_t* finished, float* loss_out2) {
   AlignParams p;
   p.Zfp = reinterpret_cast<const __nv_bfloat16*>(Z_fp); p.Zq = reinterpret_cast<const __nv_bfloat16*>(Z_q);
   p.ldz = ldz; p.V = vocab;
@@ -293,6 +318,7 @@ int faar_launch_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const vo
   p.c = (float)(1.4426950408889634 / (double)tau);
   p.gscale = (float)((double)lambda_kl / ((double)tau * (double)T));
   p.kl_partials = kl_partials; p.mse_partials = mse_partials;
+  p.loss_out2 = loss_out2; p.finished = finished; p.kl_scale = (float)(1.0 / (double)T);
   p.T = T;
   // Persistent CTAs, one per SM.  Two tokens' rows (4 vocab bytes each) per CTA or cluster are in use at a time and are to
   // stay in L2: a CTA per token up to 130 MB, then two.  1500 tokens, one against two, us: vocabulary 88000 (99 MB) 214,
@@ -311,7 +337,6 @@ int faar_launch_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const vo
   const int sms = ctx->num_sms;
   const bool two = T > sms / 2 && 2ll * (T < sms ? T : sms) * 4 * vocab > 130ll << 20;
   const int most = two ? sms / 2 : sms, n = T < most ? T : most;
-  *n_partials = n;
   cfg.gridDim = dim3(two ? 2 * n : n);
   cfg.numAttrs = two ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, two ? align_loss_kernel<2> : align_loss_kernel<1>, p);

@@ -1049,12 +1049,8 @@ int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_f
   FAAR_DEVICE_GUARD(ctx);
   float* kl_p = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace) + FAAR_WS_HEADER);
   float* mse_p = kl_p + (size_t)T;
-  int np = 0;
-  int e = faar_launch_align_loss(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, dZ_q, dH_q, kl_p,
-                                 mse_p, &np);
-  if (e) return cuda_fail(ctx, e);
-  e = faar_launch_finalize(ctx, kl_p, np, (float)(1.0 / (double)T), loss_out2, mse_p, np, 1.0f, loss_out2 + 1);
-  return cuda_fail(ctx, e);
+  return cuda_fail(ctx, faar_launch_align_loss(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, dZ_q, dH_q, kl_p,
+                                               mse_p, reinterpret_cast<uint32_t*>(workspace) + 6, loss_out2));
 }
 
 int faar_harden_pack(faar_ctx* ctx, const faar_shape* s, const float* V, const uint8_t* code, const uint8_t* scales,

@@ -91,6 +91,7 @@ static inline cudaError_t faar_launch_pdl(faar_ctx* ctx, void (*kernel)(KArgs...
 // [0, 256)            header: word 0 = status (0 = ok), bytes 8..15 = the final sums of a
 //                     dW launch while its CTAs finish (zero between launches), bytes 16..23 = tensor maximum of
 //                     the last set-up pass (high word: the pass's serial number, low word: max |W| bits),
+//                     bytes 24..27 = clusters of an alignment-loss launch that have finished (zero between launches),
 //                     bytes 64..127 = a bit per CTA of a dW launch whose Round Loss sum lies in the Round region
 //                     (zero between launches)
 // [256, 256+P)        loss partials (float): MSE region then Round region
@@ -161,10 +162,10 @@ int faar_launch_act_fakequant(faar_ctx*, int T, int K, const void* X, int64_t ld
 int faar_launch_transpose_bf16(faar_ctx*, int rows, int cols, const void* in, int64_t ld_in, void* out,
                                int64_t ld_out);
 int faar_launch_swizzle_scales(faar_ctx*, int rows, int cols, const uint8_t* in, uint8_t* out);
-// Eq. 6's data terms: one partial per CTA, at most one CTA per token
+// Eq. 6's data terms: one partial of each per CTA or cluster, at most one per token; `finished` is zero between launches
 int faar_launch_align_loss(faar_ctx*, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
                            const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, void* dZ_q,
-                           void* dH_q, float* kl_partials, float* mse_partials, int* n_partials);
+                           void* dH_q, float* kl_partials, float* mse_partials, uint32_t* finished, float* loss_out2);
 int faar_launch_silu_mul(faar_ctx*, int rows, int cols, const void* gate, int64_t ldg, const void* up, int64_t ldu,
                          void* out, int64_t ldo);
 int faar_launch_rmsnorm(faar_ctx*, int rows, int cols, const void* x, int64_t ldx, const void* b, int64_t ldb,
@@ -176,9 +177,12 @@ int faar_launch_rope(faar_ctx*, int rows, int n_heads, int head_dim, const void*
                      int inverse, void* y, int64_t ldy);
 int faar_launch_silu_mul_bwd(faar_ctx*, int rows, int cols, const void* dout, int64_t ldd, const void* gate, int64_t ldg,
                              const void* up, int64_t ldu, void* dgate, int64_t lddg, void* dup, int64_t lddu);
-// rope (nullable): also the sine and cosine of every row's head_dim / 2 rotary angles, [head_dim / 2, rows]
 int faar_launch_embedding(faar_ctx*, int rows, int cols, int vocab, const void* table, int64_t ldt, const int* tokens,
-                          void* out, int64_t ldo, const int* pos = nullptr, int head_dim = 0, float theta = 0.f, float2* rope = nullptr);
+                          void* out, int64_t ldo);
+// How a model's pass begins: x = the tokens' rows of the table, y = rmsnorm(x), and every row's rotary angles, [head_dim / 2,
+// rows] sines and cosines
+int faar_launch_embed_rmsnorm(faar_ctx*, int rows, int cols, int vocab, const void* table, const int* tokens, void* x, const float* g,
+                              float eps, void* y, float* rstd, const int* pos, int head_dim, float theta, float2* rope);
 int faar_launch_add(faar_ctx*, int rows, int cols, const void* a, int64_t lda, const void* b, int64_t ldb, void* out,
                     int64_t ldo);
 int faar_launch_attention_fwd(faar_ctx*, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,

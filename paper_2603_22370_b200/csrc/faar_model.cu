@@ -243,19 +243,26 @@ int check_model(const faar_ctx* ctx, const faar_model* m, int batch, int seq, bo
   return FAAR_OK;
 }
 
-int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* pos, bool quantised, float beta,
-            bool keep, uint8_t* arena, void* Z, void* Hout, void* ws) {
+// The first block's input and norm and the rotary angles, into the arena of a pass.
+int begin(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* pos, bool keep, uint8_t* arena) {
+  const Sizes s = sizes(m, batch, seq);
+  const Arena A(s, m->n_layers, keep);
+  return faar_launch_embed_rmsnorm(ctx, (int)s.T, s.d, m->vocab, m->embed, tokens, arena + A.b.x_in, m->blocks[0].attn_norm, m->eps,
+                                   arena + A.b.hn, reinterpret_cast<float*>(arena + A.b.rstd1), pos, s.hd, m->theta,
+                                   reinterpret_cast<float2*>(arena + A.rope));
+}
+// The blocks, the final norm and the LM head.  begun: the arena that begin() has filled, this pass's or that of another pass
+// (which keeps its activations) on the same tokens.
+int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, bool quantised, float beta, bool keep, uint8_t* arena,
+            const uint8_t* begun, void* Z, void* Hout, void* ws) {
   const Sizes s = sizes(m, batch, seq);
   const Arena A(s, m->n_layers, keep);
   const int T = (int)s.T;
   auto part = [&](int l) { return arena + (keep ? l : l % (int)A.parts) * A.b.bytes; };
   uint8_t* const tmp = arena + A.tmp;
-  uint8_t* p = part(0);
-  float2* const rope = reinterpret_cast<float2*>(arena + A.rope);
-  int e = faar_launch_embedding(ctx, T, s.d, m->vocab, m->embed, s.d, tokens, p + A.b.x_in, s.d, pos, s.hd, m->theta, rope);
-  if (!e)
-    e = faar_launch_rmsnorm(ctx, T, s.d, p + A.b.x_in, s.d, nullptr, 0, nullptr, 0, m->blocks[0].attn_norm, m->eps, p + A.b.hn, s.d,
-                            reinterpret_cast<float*>(p + A.b.rstd1));
+  uint8_t* p = nullptr;
+  const float2* const rope = reinterpret_cast<const float2*>(begun + Arena(s, m->n_layers, keep || begun != arena).rope);
+  int e = 0;
   int soft_end = 0;                              // blocks below this have their soft weights
   for (int l = 0; l < m->n_layers && !e; ++l) {
     const faar_block& b = m->blocks[l];
@@ -270,14 +277,15 @@ int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* t
     __nv_bfloat16* const qkv = reinterpret_cast<__nv_bfloat16*>(p + A.b.qkv);
     const void *Wqkv = nullptr, *Wgu = nullptr;
     e = group_operand(ctx, b.qkv, s.d, w, beta, &Wqkv);
-    if (!e) e = product_rope(ctx, m, s, p + A.b.hn, Wqkv, rope, qkv, ws);
+    const uint8_t* const in = l == 0 ? begun : p;          // x_in and hn lie first in either form of the arena
+    if (!e) e = product_rope(ctx, m, s, in + A.b.hn, Wqkv, rope, qkv, ws);
     if (!e)
       e = faar_launch_attention_fwd(ctx, batch, seq, m->n_heads, m->n_kv_heads, m->head_dim, qkv, s.qkv, qkv + s.qd, qkv + s.qd + s.kvd,
                                     s.qkv, p + A.b.a, s.qd, reinterpret_cast<float*>(p + A.b.lse));
     if (!e) e = group_forward(ctx, b.o, s.T, s.qd, p + A.b.a, w, beta, tmp, ws);
     // residual connection and the MLP's norm in one pass
     if (!e)
-      e = faar_launch_rmsnorm(ctx, T, s.d, p + A.b.x_in, s.d, tmp, s.d, p + A.b.x_mid, s.d, b.mlp_norm, m->eps, p + A.b.mn, s.d,
+      e = faar_launch_rmsnorm(ctx, T, s.d, in + A.b.x_in, s.d, tmp, s.d, p + A.b.x_mid, s.d, b.mlp_norm, m->eps, p + A.b.mn, s.d,
                               reinterpret_cast<float*>(p + A.b.rstd2));
     __nv_bfloat16* const gu = reinterpret_cast<__nv_bfloat16*>(p + A.b.gu);
     // act = silu(gate) up leaves with the product; gate and up themselves only where a backward pass will read them
@@ -342,24 +350,27 @@ int backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* 
   return e;
 }
 
-// Both forward passes at once: the frozen one on the context's side stream, between two events.  The products of either
-// use nothing of the workspace but its status word.
+// Both forward passes at once: the frozen one on the context's side stream, between two events, behind the first block's
+// input and norm, which they share.  The products of either use nothing of the workspace but its status word.
 int forward_both(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* pos, float beta, uint8_t* arena_fp,
                  void* Z_fp, void* H_fp, uint8_t* arena, void* Z, void* H, void* ws) {
   cudaError_t ce = cudaSuccess;
   if (!ctx->side_stream) ce = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
   if (ce == cudaSuccess && !ctx->ev_fork) ce = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
   if (ce == cudaSuccess && !ctx->ev_join) ce = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
+  if (ce != cudaSuccess) return (int)ce;
+  int e = begin(ctx, m, batch, seq, tokens, pos, true, arena);
+  if (e) return e;
   const cudaStream_t main = ctx->stream;
-  if (ce == cudaSuccess) ce = cudaEventRecord(ctx->ev_fork, main);
+  ce = cudaEventRecord(ctx->ev_fork, main);
   if (ce == cudaSuccess) ce = cudaStreamWaitEvent(ctx->side_stream, ctx->ev_fork, 0);
   if (ce != cudaSuccess) return (int)ce;
   ctx->stream = ctx->side_stream;
-  int e = forward(ctx, m, batch, seq, tokens, pos, false, beta, false, arena_fp, Z_fp, H_fp, ws);
+  e = forward(ctx, m, batch, seq, false, beta, false, arena_fp, arena, Z_fp, H_fp, ws);
   ctx->stream = main;
   // joined whatever happened, so that the caller's stream orders everything that was enqueued
   ce = cudaEventRecord(ctx->ev_join, ctx->side_stream);
-  if (!e) e = forward(ctx, m, batch, seq, tokens, pos, true, beta, true, arena, Z, H, ws);
+  if (!e) e = forward(ctx, m, batch, seq, true, beta, true, arena, arena, Z, H, ws);
   if (ce == cudaSuccess) ce = cudaStreamWaitEvent(main, ctx->ev_join, 0);
   return e ? e : (int)ce;
 }
@@ -406,8 +417,9 @@ int faar_model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, c
   if (arena_bytes < need) return FAAR_ERR_WORKSPACE;
   Device dev(ctx->device);
   if (dev.err) return status(ctx, dev.err);
-  return status(ctx, forward(ctx, m, batch, seq, tokens, positions, quantised != 0, beta, keep != 0, reinterpret_cast<uint8_t*>(arena), Z, H,
-                             workspace));
+  uint8_t* const at = reinterpret_cast<uint8_t*>(arena);
+  const int e = begin(ctx, m, batch, seq, tokens, positions, keep != 0, at);
+  return status(ctx, e ? e : forward(ctx, m, batch, seq, quantised != 0, beta, keep != 0, at, at, Z, H, workspace));
 }
 
 // Overlap pays while the passes are chains of launches that leave much of the GPU idle.  Whole alignment step, one pass after

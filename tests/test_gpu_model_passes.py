@@ -147,6 +147,7 @@ def rel(a, b):
 def test_a_models_passes_are_those_of_its_single_calls(ctx, batch, seq, hidden, heads, kv_heads, head_dim, ffn, width):
     m, tokens, gen = make_model(ctx, batch, seq, vocab=528, hidden=hidden, n_layers=2, n_heads=heads, n_kv_heads=kv_heads, head_dim=head_dim,
                                 ffn=ffn)
+    tokens[1], tokens[-1] = 528, -1        # outside the table: rows of zeros
     faar.tune_tile_n(ctx, width)
     faar.tune_wide_tiles(ctx, 0)           # every contraction whole, as faar_layer_ref has it: one order of every sum
     try:
