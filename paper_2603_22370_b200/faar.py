@@ -387,6 +387,18 @@ def model_sizes(model: Model, batch: int, seq: int, keep: int) -> tuple[int, int
     return a.value, b.value
 
 
+class Region(int):
+    """Device memory by its address, `bytes` long: stands for a tensor in the calls of a model's passes."""
+
+    def __new__(cls, address: int, bytes: int):
+        r = int.__new__(cls, address)
+        r.bytes = bytes
+        return r
+
+    def numel(self) -> int:
+        return self.bytes
+
+
 def model_forward(ctx, model, batch, seq, tokens, positions, quantised, beta, keep, arena, Z, H, ws):
     _check(_fast().faar_model_forward(ctx._n, model, batch, seq, tokens, positions, int(quantised), beta, int(keep), arena,
                                       arena.numel(), Z, H, ws, ws.numel()), "faar_model_forward")

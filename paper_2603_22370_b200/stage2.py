@@ -16,6 +16,7 @@ Embedding, norms and LM head are frozen and stay in BF16 / FP32; the seven linea
 from __future__ import annotations
 
 import ctypes
+import operator
 from dataclasses import dataclass
 
 import torch
@@ -110,10 +111,21 @@ class Stage2Model:
         self.arena_bytes = {bool(k): faar.model_sizes(table, batch, seq, k)[0] for k in (0, 1)}
         self.scratch_bytes = faar.model_sizes(table, batch, seq, 1)[1]
         self.overlap = faar.model_overlap(table, batch, seq)
+        self._regions, self._regions_of = None, None
 
     # ---- helpers ------------------------------------------------------------------------------------
     def _new(self, cols, dtype=torch.bfloat16):
         return torch.empty((self.T, cols), dtype=dtype, device=self.dev)
+
+    def _plan_regions(self):
+        """Where the buffers of a small model's step lie in its one allocation: (name, first byte, bytes)."""
+        z, h = 2 * self.T * self.cfg.vocab, 2 * self.T * self.cfg.hidden
+        self._regions, at = [], 0
+        for name, n in (("fp", self.arena_bytes[False]), ("q", self.arena_bytes[True]), ("scratch", self.scratch_bytes), ("Z_fp", z),
+                        ("H_fp", h), ("Z_q", z), ("H_q", h), ("dZ", z), ("dH", h)):
+            self._regions.append((name, at, n))
+            at += (n + 255) // 256 * 256
+        self._region_bytes, self._regions_of = at, (self.cfg.vocab, self.cfg.hidden)
 
     def _groups(self, l):
         """(field, names, frozen weights, soft weights) of a block's groups of linears with a common input."""
@@ -121,6 +133,8 @@ class Stage2Model:
         return (("qkv", GROUPS["qkv"], wg["qkv"], wsg["qkv"]), ("o", ("o_proj",), lin["o_proj"].W, lin["o_proj"].Wsoft),
                 ("gate_up", GROUPS["gate_up"], wg["gate_up"], wsg["gate_up"]),
                 ("down", ("down_proj",), lin["down_proj"].W, lin["down_proj"].Wsoft))
+
+    _STATE = operator.attrgetter("W", "Wsoft", "V", "code", "scales", "s_global", "m", "u")
 
     def _table(self) -> faar.Model:
         """The model as the library takes it: the configuration's values and the addresses of the tensors that the attributes
@@ -130,7 +144,7 @@ class Stage2Model:
         for l, lins in enumerate(self.lin):
             held += (p[f"attn_norm.{l}"], p[f"mlp_norm.{l}"], *self.w_group[l].values(), *self.wsoft_group[l].values())
             for x in lins.values():
-                held += (x.W, x.Wsoft, x.V, x.code, x.scales, x.s_global, x.m, x.u)
+                held += self._STATE(x)
         now = [c.vocab, c.hidden, c.n_layers, c.n_heads, c.n_kv_heads, c.head_dim, c.ffn, c.eps, c.theta]
         now += [0 if t is None else t.data_ptr() for t in held]
         if now == self._held:
@@ -208,6 +222,21 @@ class Stage2Model:
         return the quantised model's outputs, the loss gradients and every linear's dV (for inspection)."""
         self.step_count += 1
         model = self._table()
+        hp = faar.make_hparams(beta=beta, lambda_round=lambda_round, opt=self.opt, lr=lr, step=self.step_count)
+        if fp_outputs is None and self.overlap and not want_dv:
+            # nothing of the passes is handed out: one allocation and addresses in it instead of nine tensors
+            c = self.cfg
+            if self._regions_of != (c.vocab, c.hidden):
+                self._plan_regions()
+            memory = torch.empty(self._region_bytes, dtype=torch.uint8, device=self.dev)
+            base = memory.data_ptr()
+            r = {name: faar.Region(base + at, n) for name, at, n in self._regions}
+            faar.model_forward_both(self.ctx, model, self.batch, self.seq, tokens, self.pos, beta, r["fp"], r["Z_fp"], r["H_fp"], r["q"], r["Z_q"],
+                                    r["H_q"], self.ws)
+            faar.align_loss(self.ctx, self.T, c.vocab, c.hidden, r["Z_fp"], r["Z_q"], c.vocab, r["H_fp"], r["H_q"], c.hidden, tau, lambda_kl,
+                            r["dZ"], r["dH"], self.loss, self.aws)
+            faar.model_backward(self.ctx, model, self.batch, self.seq, self.pos, hp, r["q"], r["dZ"], c.vocab, r["dH"], r["scratch"], self.ws)
+            return None
         if fp_outputs is None and self.overlap:
             Z_fp, H_fp, Z_q, H_q, saved = self._forward_both(model, tokens, beta)
         else:
@@ -217,7 +246,6 @@ class Stage2Model:
         dZ, dH = torch.empty_like(Z_q), torch.empty_like(H_q)
         faar.align_loss(self.ctx, T, c.vocab, c.hidden, Z_fp, Z_q, Z_q.shape[1], H_fp, H_q, c.hidden, tau, lambda_kl, dZ, dH,
                         self.loss, self.aws)
-        hp = faar.make_hparams(beta=beta, lambda_round=lambda_round, opt=self.opt, lr=lr, step=self.step_count)
         grads = self._backward(model, dZ, dH, saved, hp, want_dv)
         return {"Z_q": Z_q, "H_q": H_q, "dZ": dZ, "dH": dH, "dV": grads} if want_dv else None
 
