@@ -146,6 +146,17 @@ __device__ __forceinline__ void ld32x2(uint32_t ta, uint32_t tb, float (&a)[32],
 #pragma unroll
   for (int i = 0; i < 32; ++i) { a[i] = __uint_as_float(u[i]); b[i] = __uint_as_float(v[i]); }
 }
+__device__ __forceinline__ void ld16(uint32_t ta, float (&a)[16]) {
+  uint32_t u[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]), "=r"(u[9]), "=r"(u[10]),
+        "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+      : "r"(ta) : "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) a[i] = __uint_as_float(u[i]);
+}
 __device__ __forceinline__ void ld16x2(uint32_t ta, uint32_t tb, float (&a)[16], float (&b)[16]) {
   uint32_t u[16], v[16];
   asm volatile(
@@ -482,6 +493,7 @@ struct TcBwdParams {
   int B, S, H, Hkv;
   float scale_log2, inv_sqrt_d;
   const float2* rope;              // dq and dk turn back by their row's angles (null: not)
+  int parts;                       // dK / dV: CTAs of a cluster that share a key tile's items (1, 2 or 4)
   int apart;                       // dQ: its memory may hold what the dK / dV kernel reads, so it waits for that one
 };
 
@@ -773,7 +785,79 @@ template <int HD> struct Dkv {
   static_assert(CTAS * (SMEM + 1024) <= 228 * 1024, "shared memory budget");
 };
 
+// Few key tiles leave SMs idle while one CTA sweeps every query tile of every head of its group, so the items of a key tile are
+// then dealt over the CTAs of a cluster.  Each ends with partial dV and dK; of their 2 HD columns each CTA finishes a part:
+// the others' values for it come through distributed shared memory, over the operands, which all have been read by then.
+// A part is 16-column chunks from the lower half of dV's (or dK's) columns and their partners HD / 2 further on, which the
+// rotary embedding pairs.  Values lie in 16-byte units, [sender][chunk][4 columns][row].
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 template <int HD>
+__device__ __noinline__ void finish_parts(uint32_t base, uint32_t t_acc, int row, int half, int parts, int rank, bool has, bool valid,
+                                          __nv_bfloat16* dk, __nv_bfloat16* dv, const float2* angles, long long tokens) {
+  const int per = parts / 2, pairs = HD / 32 / per;             // CTAs for each of dV and dK; pairs of chunks a CTA finishes
+  auto column = [&](int owner, int pair, int partner) {         // of the accumulators, dV's columns first
+    return (owner >= per ? HD : 0) + 16 * ((owner % per) * pairs + pair) + partner * (HD / 2);
+  };
+  auto unit = [&](int sender, int pair, int partner, int u) {
+    return base + (uint32_t)(((((sender * pairs + pair) * 2 + partner) * 4 + u) * QT + row) << 4);
+  };
+  cluster_sync();                                               // nobody's operands are read any more
+  for (int d = 1; d < parts; ++d) {
+    const int owner = (rank + d) % parts, slot = rank < owner ? rank : rank - 1;
+    for (int pair = half; pair < pairs * 2; pair += 2) {        // (pair, partner) one after the other
+      float v[16];
+      ld16(t_acc + (uint32_t)column(owner, pair >> 1, pair & 1), v);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        uint32_t dst;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(unit(slot, pair >> 1, pair & 1, u)), "r"(owner));
+        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "f"(has ? v[4 * u] : 0.f), "f"(has ? v[4 * u + 1] : 0.f),
+                     "f"(has ? v[4 * u + 2] : 0.f), "f"(has ? v[4 * u + 3] : 0.f) : "memory");
+      }
+    }
+  }
+  cluster_sync();
+  const bool is_k = rank >= per;
+  __nv_bfloat16* const out = is_k ? dk : dv;
+  for (int pair = half; pair < pairs; pair += 2) {
+    float v[2][16];
+#pragma unroll
+    for (int partner = 0; partner < 2; ++partner) {
+      ld16(t_acc + (uint32_t)column(rank, pair, partner), v[partner]);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[partner][j] = has ? v[partner][j] : 0.f;
+      for (int sender = 0; sender < parts - 1; ++sender) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          float4 x;
+          asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(unit(sender, pair, partner, u)) : "memory");
+          v[partner][4 * u] += x.x; v[partner][4 * u + 1] += x.y; v[partner][4 * u + 2] += x.z; v[partner][4 * u + 3] += x.w;
+        }
+      }
+    }
+    const int c = column(rank, pair, 0) - (is_k ? HD : 0);
+    if (!valid) continue;
+    if (is_k && angles) {
+      Angles a;
+      load_angles(angles, tokens, c, a);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) faar_rope_turn(v[0][j], v[1][j], -a.sc[j].x, a.sc[j].y);
+    }
+#pragma unroll
+    for (int partner = 0; partner < 2; ++partner) {
+      uint4* dst = reinterpret_cast<uint4*>(out + c + partner * (HD / 2));
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        dst[q] = make_uint4(pack2(v[partner][8 * q], v[partner][8 * q + 1]), pack2(v[partner][8 * q + 2], v[partner][8 * q + 3]),
+                            pack2(v[partner][8 * q + 4], v[partner][8 * q + 5]), pack2(v[partner][8 * q + 6], v[partner][8 * q + 7]));
+    }
+  }
+}
+
+// DEALT: p.parts CTAs share a key tile (compiled in: as a choice at run time it cost whole key tiles 1 %)
+template <int HD, bool DEALT>
 __global__ void __launch_bounds__(BWD_THREADS, Dkv<HD>::CTAS)
 attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
                      const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const TcBwdParams p) {
@@ -795,14 +879,15 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   // one-dimensional grid, key tile slowest: CTAs start in order of decreasing work (the first key tiles see the
   // most queries), so the short ones fill the end of the launch
   const int groups = p.Hkv * p.B;
-  const int kt = blockIdx.x / groups, g = (blockIdx.x % groups) % p.Hkv, b = (blockIdx.x % groups) / p.Hkv;
+  const int parts = DEALT ? p.parts : 1, rank = (int)(blockIdx.x % (unsigned)parts), tile = (int)(blockIdx.x / (unsigned)parts);
+  const int kt = tile / groups, g = (tile % groups) % p.Hkv, b = (tile % groups) / p.Hkv;
   const int rep = p.H / p.Hkv;
   const long long seq0 = (long long)b * p.S;
   const int k0 = kt * QT;
   const int n_qt = (p.S + KT - 1) / KT;
   const int qt0 = k0 / KT;                                         // first query tile that sees a key of this tile
   const int per_head = n_qt - qt0;
-  const int n_it = rep * per_head;
+  const int n_all = rep * per_head, n_it = n_all > rank ? (n_all - rank + parts - 1) / parts : 0;      // this CTA's: rank, rank + parts, ...
 
   if (threadIdx.x == 0) {
     bar_init(bar_kv, 1);
@@ -829,8 +914,8 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   auto sDO = [&](int s) { return sQ(s) + C::QD_BYTES; };
   auto col_s = [&](int i) { return C::TWO ? 64u * (uint32_t)(i & 1) : 0u; };
   auto col_dp = [&](int i) { return (uint32_t)C::COL_DP + col_s(i); };
-  auto head_of = [&](int i) { return g * rep + i / per_head; };
-  auto q0_of = [&](int i) { return (qt0 + i % per_head) * KT; };
+  auto head_of = [&](int i) { return g * rep + (i * parts + rank) / per_head; };
+  auto q0_of = [&](int i) { return (qt0 + (i * parts + rank) % per_head) * KT; };
 
   if (warp == 8) {
     auto wait = [&](uint32_t bar, uint32_t parity, uint32_t code) {
@@ -845,15 +930,15 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       }
       __syncwarp();
     };
-    if (faar_elect_one()) {
+    if (n_it > 0 && faar_elect_one()) {
       bar_expect(bar_kv, 2 * C::KEY_BYTES);
       tma_head<HD>(sKt, Q_PANEL, &tmK, g * HD, k0, b, bar_kv);
       tma_head<HD>(sVt, Q_PANEL, &tmV, g * HD, k0, b, bar_kv);
     }
-    load_item(0);
+    if (n_it > 0) load_item(0);
     if (n_it > 1) load_item(1);
     if (n_it > 2) load_item(2);
-    bool ok = wait(bar_kv, 0u, 0xE01u);
+    bool ok = n_it > 0 && wait(bar_kv, 0u, 0xE01u);
     constexpr uint32_t id_k = idesc(KT, 0), id_n = idesc(HD, 1);
     auto issue_s = [&](int i) {                                // S^T and dP^T of item i
       const int st = i % C::STAGES;
@@ -916,7 +1001,9 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         }
       }
     }
-    if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
+    if (!ok && n_it > 0) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
+    __syncwarp();
+    if (DEALT) { cluster_sync(); cluster_sync(); }      // the row warps' (finish_parts)
   } else {
     const int row = 32 * (warp & 3) + lane, half = warp >> 2;    // this thread: queries 32 half .. 32 half + 31 of an item
     const int kj = k0 + row;
@@ -931,7 +1018,7 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       if (q >= p.S) return 0.f;
       return row < KT ? p.lse[ro + q] : -p.dsum[ro + q] * p.inv_sqrt_d;
     };
-    float rv_next = half == 0 ? row_value(0) : 0.f;
+    float rv_next = half == 0 && n_it > 0 ? row_value(0) : 0.f;
     for (int i = 0; i < n_it; ++i) {
       const int q0 = q0_of(i);
       float* rowv = rowv_all + (i & 1) * 2 * KT;
@@ -989,12 +1076,16 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const long long tokens = (long long)p.B * p.S;
     const float2* const angles = p.rope ? p.rope + seq0 + kj : nullptr;
     Angles first;
-    if (angles && kj < p.S) load_angles(angles, tokens, HD / 4 * half, first);
-    if (ok) {
+    if (angles && kj < p.S && !DEALT) load_angles(angles, tokens, HD / 4 * half, first);
+    if (ok && n_it > 0) {
       ok = bar_wait(bar_done((n_it - 1) & 1), (uint32_t)(((n_it - 1) >> 1) & 1), abort_flag, 0xF30u);
       ok = __all_sync(0xffffffffu, ok);
     }
-    if (ok) {
+    if constexpr (DEALT) {
+      fence_after();
+      const long long at = (seq0 + kj) * p.ldk + g * HD;
+      finish_parts<HD>(base, t_lane + (uint32_t)C::COL_DV, row, half, parts, rank, n_it > 0, kj < p.S, p.dk + at, p.dv + at, angles, tokens);
+    } else if (ok) {
       fence_after();
 #pragma unroll
       for (int which = 0; which < 2; ++which) {
@@ -1058,8 +1149,18 @@ int launch_fwd(faar_ctx* ctx, const TcParams& p, const void* q, int64_t ldq, con
   return (int)cudaGetLastError();
 }
 
+// Over how many CTAs the items of a key tile are dealt: as many as the device holds twice over (dQ fills what is left), while
+// the first key tile leaves each two items.  Backward call, one CTA a key tile -> two -> four, us: 32 / 8 heads of 64, 2 x 1000
+// tokens (128 key tiles) 112 -> 73 -> 70, 1 x 300 36 -> 24.6 -> 19, 4 x 2048 (512; one) 338 -> 361 -> 408; 16 / 8 heads of 128, 2 x
+// 1000 (128; two) 64 -> 62.4 -> 81, 3 x 2048 (384; one) 250 -> 275 -> 343.
+int pick_parts(int slots, int tiles, int longest) {
+  int parts = 1;
+  while (parts < 4 && 2 * parts * tiles <= 2 * slots && longest >= 4 * parts) parts *= 2;
+  return parts;
+}
+
 template <int HD>
-int launch_bwd(faar_ctx* ctx, const TcBwdParams& p, const void* q, int64_t ldq, const void* k, const void* v, int64_t ldk,
+int launch_bwd(faar_ctx* ctx, TcBwdParams& p, const void* q, int64_t ldq, const void* k, const void* v, int64_t ldk,
                const void* dout, int64_t ldo) {
   CUtensorMap tmQ, tmDO, tmK, tmV, tmQk, tmDOk, tmKk, tmVk;      // boxes of 128 rows / of 64 rows
   int e = head_map(ctx, &tmQ, q, p.B, p.S, p.H * HD, ldq, QT);
@@ -1070,12 +1171,27 @@ int launch_bwd(faar_ctx* ctx, const TcBwdParams& p, const void* q, int64_t ldq, 
   if (!e) e = head_map(ctx, &tmDOk, dout, p.B, p.S, p.H * HD, ldo, KT);
   if (!e) e = head_map(ctx, &tmKk, k, p.B, p.S, p.Hkv * HD, ldk, KT);
   if (!e) e = head_map(ctx, &tmVk, v, p.B, p.S, p.Hkv * HD, ldk, KT);
-  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dkv_tc_kernel<HD>, Dkv<HD>::SMEM);
+  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dkv_tc_kernel<HD, false>, Dkv<HD>::SMEM);
+  if (!e) e = faar_allow_smem(ctx, (const void*)attn_dkv_tc_kernel<HD, true>, Dkv<HD>::SMEM);
   if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_tc_kernel<HD>, Dq<HD>::SMEM);
   if (e) return e;
   const int tiles = (p.S + QT - 1) / QT;
-  faar_launch_pdl(ctx, attn_dkv_tc_kernel<HD>, dim3(tiles * p.Hkv * p.B, 1, 1), dim3(BWD_THREADS), Dkv<HD>::SMEM, tmQk, tmDOk, tmK, tmV, p);
-  e = (int)cudaGetLastError();
+  p.parts = pick_parts(ctx->num_sms * Dkv<HD>::CTAS, tiles * p.Hkv * p.B, p.H / p.Hkv * ((p.S + KT - 1) / KT));
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = p.parts;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(tiles * p.Hkv * p.B * p.parts);
+  cfg.blockDim = dim3(BWD_THREADS);
+  cfg.dynamicSmemBytes = Dkv<HD>::SMEM;
+  cfg.stream = ctx->stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = p.parts > 1 ? 2 : 1;
+  e = (int)cudaLaunchKernelEx(&cfg, p.parts > 1 ? attn_dkv_tc_kernel<HD, true> : attn_dkv_tc_kernel<HD, false>, tmQk, tmDOk, tmK, tmV, p);
+  if (!e) e = (int)cudaGetLastError();
   if (e) return e;
   faar_launch_pdl(ctx, attn_dq_tc_kernel<HD>, dim3(tiles * p.H * p.B, 1, 1), dim3(BWD_THREADS), Dq<HD>::SMEM, tmQ, tmDO, tmKk, tmVk, p);
   return (int)cudaGetLastError();
