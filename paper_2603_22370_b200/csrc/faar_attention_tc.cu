@@ -1149,13 +1149,14 @@ int launch_fwd(faar_ctx* ctx, const TcParams& p, const void* q, int64_t ldq, con
   return (int)cudaGetLastError();
 }
 
-// Over how many CTAs the items of a key tile are dealt: as many as the device holds twice over (dQ fills what is left), while
-// the first key tile leaves each two items.  Backward call, one CTA a key tile -> two -> four, us: 32 / 8 heads of 64, 2 x 1000
-// tokens (128 key tiles) 112 -> 73 -> 70, 1 x 300 36 -> 24.6 -> 19, 4 x 2048 (512; one) 338 -> 361 -> 408; 16 / 8 heads of 128, 2 x
-// 1000 (128; two) 64 -> 62.4 -> 81, 3 x 2048 (384; one) 250 -> 275 -> 343.
-int pick_parts(int slots, int tiles, int longest) {
+// Over how many CTAs the items of a key tile are dealt: up to `most` CTAs in all (four an SM with heads of 64, of which two run at
+// a time; one with heads of 128, where dQ next to this kernel has use for what is left), while the first key tile leaves each two
+// items.  Backward call, one CTA a key tile -> two -> four, us: 32 / 8 heads of 64, 2 x 1000 tokens (128 key tiles) 112 -> 73 -> 70,
+// 1 x 300 36 -> 24.6 -> 19, 4 x 2048 (512; one) 338 -> 361 -> 408; 16 / 8 heads of 128, 2 x 1000 (128; one) 64 -> 62.4 -> 81, in an
+// alignment step 2882 -> 2905 with two; 3 x 2048 (384; one) 250 -> 275 -> 343.
+int pick_parts(int most, int tiles, int longest) {
   int parts = 1;
-  while (parts < 4 && 2 * parts * tiles <= 2 * slots && longest >= 4 * parts) parts *= 2;
+  while (parts < 4 && 2 * parts * tiles <= most && longest >= 4 * parts) parts *= 2;
   return parts;
 }
 
@@ -1176,7 +1177,7 @@ int launch_bwd(faar_ctx* ctx, TcBwdParams& p, const void* q, int64_t ldq, const 
   if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_tc_kernel<HD>, Dq<HD>::SMEM);
   if (e) return e;
   const int tiles = (p.S + QT - 1) / QT;
-  p.parts = pick_parts(ctx->num_sms * Dkv<HD>::CTAS, tiles * p.Hkv * p.B, p.H / p.Hkv * ((p.S + KT - 1) / KT));
+  p.parts = pick_parts(ctx->num_sms * Dkv<HD>::CTAS * Dkv<HD>::CTAS, tiles * p.Hkv * p.B, p.H / p.Hkv * ((p.S + KT - 1) / KT));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
