@@ -211,25 +211,28 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      int stage = 0; uint32_t phase = 0; bool ok = true;
-      for (int t = pair; t < tiles && ok; t += n_pairs) {
-        const int mt = t % m_tiles, nt = t / m_tiles;
-        for (int ks = 0; ks < k_stages; ++ks) {
-          ok = bar_wait(empty(stage), phase ^ 1u, ab, 0x900u | stage);
-          if (!ok) break;
-          const uint32_t sa = base + stage * C4::STAGE, sb = sa + C4::A_BYTES, sfa = sb + C4::B_BYTES, sfb = sfa + C4::SFA_BYTES;
+    // the whole warp, converged (see faar_elect_one): four copies a stage under `if (lane == 0)` took about 400 of the 512 clocks
+    // that a stage's MMAs take, and a few stages' worth of a short contraction's whole time
+    int stage = 0; uint32_t phase = 0; bool ok = true;
+    for (int t = pair; t < tiles && ok; t += n_pairs) {
+      const int mt = t % m_tiles, nt = t / m_tiles;
+      for (int ks = 0; ks < k_stages; ++ks) {
+        ok = __all_sync(0xffffffffu, bar_wait(empty(stage), phase ^ 1u, ab, 0x900u | stage));
+        if (!ok) break;
+        const uint32_t sa = base + stage * C4::STAGE, sb = sa + C4::A_BYTES, sfa = sb + C4::B_BYTES, sfb = sfa + C4::SFA_BYTES;
+        const uint32_t bar = map_to_leader(full(stage));
+        if (faar_elect_one()) {
           if (rank == 0) bar_expect(full(stage), 2u * (uint32_t)C4::STAGE);
-          const uint32_t bar = map_to_leader(full(stage));
           tma_2d(sa, &tmA, ks * ROW_BYTES, mt * 2 * TM + (int)rank * TM, bar);
           tma_2d(sb, &tmB, ks * ROW_BYTES, nt * BN + (int)rank * (BN / 2), bar);
           tma_3d(sfa, &tmSA, 0, 4 * ks, 2 * mt + (int)rank, bar);
           tma_3d(sfb, &tmSB, 0, 4 * ks, nt * C4::N_SFB, bar);
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
+        __syncwarp();
+        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
     }
+    if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
   } else if (warp == 1) {
     if (rank == 0) {                                         // the whole warp, converged (see faar_elect_one)
       int stage = 0; uint32_t phase = 0; int it = 0; bool ok = true;

@@ -1069,31 +1069,31 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    // ---------------- TMA producer (both CTAs) ----------------
-    if (lane == 0) {
-      const uint64_t keep = l2_policy_keep();
-      int stage = 0; uint32_t phase = 0;
-      bool ok = true;
-      auto coords = [&](int tile) {
-        TileCoord tc;
-        if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * wide_w; tc.w = BN_MAX; }
-        else tc = tile_coord(p, tile, m_tiles);
-        return tc;
-      };
-      for (int tile = pair; tile < total_tiles && ok; tile += n_pairs) {
-        const TileCoord tc = coords(tile);
-        const int m0 = tc.m0 + (int)rank * BM;
-        const int n0 = GATED ? tc.n0 / 2 + (int)rank * (p.N / 2) : tc.n0 + (int)rank * (tc.w / 2);
-        const CUtensorMap* mapB = tc.w == BN ? &tmB : &tmBh;      // box of w/2 rows
-        for (int kb = kb0; kb < kb1; ++kb) {
-          ok = mbar_wait(empty_bar(stage), phase ^ 1u, ac, 0x100u | stage);
-          if (!ok) break;
-          const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + C::A_BYTES;
+    // ---------------- TMA producer (both CTAs; the whole warp, converged: see faar_elect_one) ----------------
+    const uint64_t keep = l2_policy_keep();
+    int stage = 0; uint32_t phase = 0;
+    bool ok = true;
+    auto coords = [&](int tile) {
+      TileCoord tc;
+      if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * wide_w; tc.w = BN_MAX; }
+      else tc = tile_coord(p, tile, m_tiles);
+      return tc;
+    };
+    for (int tile = pair; tile < total_tiles && ok; tile += n_pairs) {
+      const TileCoord tc = coords(tile);
+      const int m0 = tc.m0 + (int)rank * BM;
+      const int n0 = GATED ? tc.n0 / 2 + (int)rank * (p.N / 2) : tc.n0 + (int)rank * (tc.w / 2);
+      const CUtensorMap* mapB = tc.w == BN ? &tmB : &tmBh;      // box of w/2 rows
+      for (int kb = kb0; kb < kb1; ++kb) {
+        ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, ac, 0x100u | stage));
+        if (!ok) break;
+        const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + C::A_BYTES;
+        const uint32_t leader_full = map_to_cta(full_bar(stage), leader);
+        if (faar_elect_one()) {
           // the leader's barrier collects the bytes of both CTAs' copies
           if (rank == 0)
             mbar_expect_tx(full_bar(stage), WIDE ? 2u * (uint32_t)(C::A_BYTES + wide_w / 2 * BK * 2)
                                                  : 2u * (uint32_t)(C::A_BYTES + (B_MN ? mn_boxes(tc.w / 2) * MN_BOX : tc.w / 2) * BK * 2));
-          const uint32_t leader_full = map_to_cta(full_bar(stage), leader);
           if (A_MN) {                                          // two boxes of 64 rows of A, each [64 k][64 m]
             tma_load_2d(sa, &tmA, m0, kb * BK, leader_full, keep);
             tma_load_2d(sa + MN_BOX_BYTES, &tmA, m0 + MN_BOX, kb * BK, leader_full, keep);
@@ -1108,14 +1108,15 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
           // second column half (rows beyond the matrix arrive as zeros)
           if (WIDE) tma_load_2d(sb + C::BH_BYTES, &tmBh, kb * BK, tc.n0 + BN_MAX + (int)rank * (p.n_main / 2), leader_full, keep);
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
+        __syncwarp();
+        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) {
-        // give copies already in flight a bounded chance to land before the CTA exits
-        const unsigned long long t0 = global_ns();
-        while (global_ns() - t0 < 2000000ull) {}
-      }
+    }
+    if (!ok) {
+      // give copies already in flight a bounded chance to land before the CTA exits
+      const unsigned long long t0 = global_ns();
+      while (global_ns() - t0 < 2000000ull) {}
     }
     if constexpr (MODE == FAAR_GEMM_BWD) {
       // the forward's share of the loss values, under the epilogue: strided double accumulation, then a tree over lanes

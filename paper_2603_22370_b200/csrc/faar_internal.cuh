@@ -350,7 +350,10 @@ __device__ __forceinline__ void faar_pdl_join() { asm volatile("griddepcontrol.w
 // One lane of a converged warp.  A warp that issues tensor-core instructions runs its loop with all lanes and guards
 // only those instructions with this, so that the descriptors stay in uniform registers; under `if (lane == 0)` every
 // operand is moved there first, about 65 clocks per instruction, and the issuing thread becomes the bottleneck
-// (NVFP4 GEMM, C[4096, 2048], K = 8192: 71 us against 33.8 us).
+// (NVFP4 GEMM, C[4096, 2048], K = 8192: 71 us against 33.8 us).  The same for a warp that issues copies: two or four a stage and
+// their barrier took most of what a stage of a narrow tile lasts.  Step of 64 x 8192 at 300 tokens 44.6 -> 42.6 us, 512 x 2048 at 4096 30.2
+// -> 29.3, 512 x 512 at 512 16.9 -> 16.1, 128 x 256 at 1024 12.8 -> 12.5; alignment step of two 512-wide blocks on 400 tokens 270.6 ->
+// 262.6; NVFP4 product of 8 tokens, 2048 x 8192, with its quantiser 18.5 -> 16.5, of 1000 tokens, 2048 x 4096, 9.1 -> 8.4.
 __device__ __forceinline__ bool faar_elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
