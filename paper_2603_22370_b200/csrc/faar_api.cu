@@ -97,6 +97,7 @@ int fwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const v
   }
   faar_gemm_args a = {};
   a.mode = FAAR_GEMM_FWD;
+  a.ahead = !hp->wsoft_ready;              // the launch before it wrote the soft weights and nothing else
   a.M = s->O; a.N = s->T; a.Kc = s->K;
   a.A = wsoft; a.lda = s->K;
   a.B = X; a.ldb = s->ldx;
@@ -136,6 +137,7 @@ int bwd_impl(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const v
     a.fin_out2 = loss_out2;
   }
   a.mode = FAAR_GEMM_BWD;
+  a.ahead = loss_out2 != nullptr;          // a whole step: the launch before it is the forward product, which wrote dY^T (and loss sums)
   a.M = s->O; a.N = s->K; a.Kc = s->T;
   if (row_major == 1) {                    // dY [T, ldy] and X [T, ldx] as they are: token index = contraction row
     a.A = dYt; a.lda = s->ldy; a.a_mn = 1;

@@ -510,7 +510,7 @@ softquant_eval_kernel(const float* __restrict__ V, const uint8_t* __restrict__ c
     lut[threadIdx.x] = make_float2(sgn * faar_node(k), sgn * faar_width(k));
   }
   __syncthreads();
-  faar_pdl_sync();                                   // V comes from the previous step's backward kernel
+  faar_pdl_wait_first();                             // V comes from the previous step's backward kernel; the product after this one starts ahead
   const float s_global = *s_global_p;
   float nbl, hbl;
   faar_operand_consts(beta, &nbl, &hbl);

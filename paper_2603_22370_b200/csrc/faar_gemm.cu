@@ -344,6 +344,13 @@ struct Segment {
   int wide;                         // V, m, u and dV all lie on 32-byte boundaries (a row is a multiple of 64 bytes)
 };
 
+// What a launch needs of the one before it on the stream: everything (0), nothing (BESIDE, see faar_pdl_wait_first), or the A
+// operand alone (AHEAD): the first ring of the B operand and what the epilogue asks for ahead (target values, optimiser state) then
+// come in under the end of that launch.  Step, us: 128 x 256 at 1024 tokens 12.5 -> 12.0, 512 x 512 at 512 16.1 -> 15.7, 256 x 1024 at 1024
+// 16.0 -> 15.6, 64 x 8192 at 300 42.8 -> 41.7, 1000 x 1040 at 777 20.35 -> 20.15, 2048 x 2048 at 1024 40.4 -> 39.9; 512 x 2048 at 4096 29.26 ->
+// 29.38, larger ones the same.
+constexpr int BESIDE = 1, AHEAD = 2;
+
 struct KParams {
   int M, N, Kc;
   int bn;                 // tile width
@@ -358,7 +365,7 @@ struct KParams {
   // REF / FWD
   void* Yout; int yout_dtype; long long ldy;
   const void* Yref; int yref_dtype;
-  int columns;            // REF: Yout is [N, ldy], the accumulator's rows are its columns (compiled in: COLUMNS); BWD: beside
+  int columns;            // REF: Yout is [N, ldy], the accumulator's rows are its columns (compiled in: COLUMNS); FWD, BWD: 0, BESIDE or AHEAD
   int yref_t;             // FWD: Y_ref / Y_q stored transposed, [O, ldy] with ldy >= T rounded up to 16; REF: rows of Yout are
                           // padded like that, columns beyond N up to the next multiple of 16 are written as 0
   int y_store;            // REF: rows of Yout take 2: 32-byte stores, 1: 16-byte stores, 0: single values
@@ -1062,52 +1069,62 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   tc_fence_before();
   cluster_sync_all();                                  // barriers of both CTAs are initialised
   tc_fence_after();
-  // set-up done; now wait for the previous kernel's data
-  if (MODE == FAAR_GEMM_REF) faar_pdl_wait_first();
-  else if (MODE == FAAR_GEMM_BWD && p.columns) faar_pdl_launch();
+  // set-up done; now wait for the previous kernel's data: all of it, or (AHEAD) only the producer for the A operand
+  if (MODE != FAAR_GEMM_REF && p.columns != 0) faar_pdl_launch();
+  else if (MODE != FAAR_GEMM_BWD) faar_pdl_wait_first();
   else faar_pdl_sync();
   const uint32_t tmem_base = *tmem_slot;
 
+  const uint64_t keep = l2_policy_keep();
+  // one stage's B operand (this CTA's half); the leader's barrier collects the bytes of both CTAs' copies of A and B
+  auto load_b = [&](const TileCoord& tc, int kb, int stage) {
+    const int n0 = GATED ? tc.n0 / 2 + (int)rank * (p.N / 2) : tc.n0 + (int)rank * (tc.w / 2);
+    const uint32_t sb = base + stage * STAGE_BYTES + C::A_BYTES, leader_full = map_to_cta(full_bar(stage), leader);
+    if (rank == 0)
+      mbar_expect_tx(full_bar(stage), WIDE ? 2u * (uint32_t)(C::A_BYTES + wide_w / 2 * BK * 2)
+                                           : 2u * (uint32_t)(C::A_BYTES + (B_MN ? mn_boxes(tc.w / 2) * MN_BOX : tc.w / 2) * BK * 2));
+    if (B_MN) {                                            // this CTA's w / 2 columns of B, in boxes of 64
+      tma_load_2d(sb, &tmB, n0, kb * BK, leader_full, keep);
+      if (tc.w / 2 > MN_BOX) tma_load_2d(sb + MN_BOX_BYTES, &tmB, n0 + MN_BOX, kb * BK, leader_full, keep);
+    } else {
+      tma_load_2d(sb, tc.w == BN ? &tmB : &tmBh, kb * BK, n0, leader_full, keep);      // box of w / 2 rows
+    }
+    // second column half (rows beyond the matrix arrive as zeros)
+    if (WIDE) tma_load_2d(sb + C::BH_BYTES, &tmBh, kb * BK, tc.n0 + BN_MAX + (int)rank * (p.n_main / 2), leader_full, keep);
+  };
+  auto coords = [&](int tile) {
+    TileCoord tc;
+    if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * wide_w; tc.w = BN; }
+    else tc = tile_coord(p, tile, m_tiles);
+    return tc;
+  };
+  const bool b_ahead = MODE != FAAR_GEMM_REF && p.columns == AHEAD;      // the first ring of B is warp 1's to ask for, under the
+                                                                          // end of the kernel before
+
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs; the whole warp, converged: see faar_elect_one) ----------------
-    const uint64_t keep = l2_policy_keep();
+    int loaded = b_ahead ? min(STAGES, kb1 - kb0) : 0;
+    if (b_ahead) faar_pdl_join();
     int stage = 0; uint32_t phase = 0;
     bool ok = true;
-    auto coords = [&](int tile) {
-      TileCoord tc;
-      if (WIDE) { tc.m0 = (tile % m_tiles) * (2 * BM); tc.n0 = (tile / m_tiles) * wide_w; tc.w = BN_MAX; }
-      else tc = tile_coord(p, tile, m_tiles);
-      return tc;
-    };
     for (int tile = pair; tile < total_tiles && ok; tile += n_pairs) {
       const TileCoord tc = coords(tile);
       const int m0 = tc.m0 + (int)rank * BM;
-      const int n0 = GATED ? tc.n0 / 2 + (int)rank * (p.N / 2) : tc.n0 + (int)rank * (tc.w / 2);
-      const CUtensorMap* mapB = tc.w == BN ? &tmB : &tmBh;      // box of w/2 rows
       for (int kb = kb0; kb < kb1; ++kb) {
         ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, ac, 0x100u | stage));
         if (!ok) break;
-        const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + C::A_BYTES;
+        const uint32_t sa = base + stage * STAGE_BYTES;
         const uint32_t leader_full = map_to_cta(full_bar(stage), leader);
+        const bool with_b = loaded == 0;
+        if (!with_b) --loaded;
         if (faar_elect_one()) {
-          // the leader's barrier collects the bytes of both CTAs' copies
-          if (rank == 0)
-            mbar_expect_tx(full_bar(stage), WIDE ? 2u * (uint32_t)(C::A_BYTES + wide_w / 2 * BK * 2)
-                                                 : 2u * (uint32_t)(C::A_BYTES + (B_MN ? mn_boxes(tc.w / 2) * MN_BOX : tc.w / 2) * BK * 2));
+          if (with_b) load_b(tc, kb, stage);
           if (A_MN) {                                          // two boxes of 64 rows of A, each [64 k][64 m]
             tma_load_2d(sa, &tmA, m0, kb * BK, leader_full, keep);
             tma_load_2d(sa + MN_BOX_BYTES, &tmA, m0 + MN_BOX, kb * BK, leader_full, keep);
           } else {
             tma_load_2d(sa, &tmA, kb * BK, m0, leader_full, keep);
           }
-          if (B_MN) {                                          // this CTA's w / 2 columns of B, in boxes of 64
-            tma_load_2d(sb, &tmB, n0, kb * BK, leader_full, keep);
-            if (tc.w / 2 > MN_BOX) tma_load_2d(sb + MN_BOX_BYTES, &tmB, n0 + MN_BOX, kb * BK, leader_full, keep);
-          } else {
-            tma_load_2d(sb, mapB, kb * BK, n0, leader_full, keep);
-          }
-          // second column half (rows beyond the matrix arrive as zeros)
-          if (WIDE) tma_load_2d(sb + C::BH_BYTES, &tmBh, kb * BK, tc.n0 + BN_MAX + (int)rank * (p.n_main / 2), leader_full, keep);
         }
         __syncwarp();
         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -1133,6 +1150,15 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (leader CTA only; the whole warp, converged: see faar_elect_one) ----------------
+    // (AHEAD, both CTAs: first the B ring.  By the producer itself, in front of its wait, it held up the A operand of CTAs that
+    // start late: step of 512 x 2048 at 4096 tokens 30.2 -> 32.2 us)
+    if (b_ahead) {
+      const TileCoord tc = coords(pair);
+      for (int i = 0; i < min(STAGES, kb1 - kb0); ++i) {
+        if (faar_elect_one()) load_b(tc, kb0 + i, i);
+        __syncwarp();
+      }
+    }
     if (rank == 0) {
       int stage = 0; uint32_t phase = 0;
       int it = 0;
@@ -1455,7 +1481,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   }
 
   if constexpr (MODE == FAAR_GEMM_BWD) {
-    if (p.columns && threadIdx.x == 0) faar_pdl_join();
+    if (p.columns == BESIDE && threadIdx.x == 0) faar_pdl_join();
     // Final loss sums by whichever CTA finishes last.  Each adds its Round Loss sum to one word, as a fixed-point number
     // above nine bits that count the CTAs and nine that count sums kept elsewhere.  A sum is rounded to the field's unit
     // (2^-20 for 16 M weights); the addition is exact, so neither the order nor which CTA is last matters, and the last one
@@ -1849,7 +1875,7 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
   faar_gemm_args swapped;
   const faar_gemm_args* a = args;
   KParams kp;
-  kp.columns = args->mode == FAAR_GEMM_REF ? result_columns(args) : args->mode == FAAR_GEMM_BWD && args->beside;
+  kp.columns = args->mode == FAAR_GEMM_REF ? result_columns(args) : (args->beside ? BESIDE : (args->ahead ? AHEAD : 0));
   if (args->mode == FAAR_GEMM_REF && kp.columns) {
     swapped = *args;
     swapped.M = args->N; swapped.N = args->M;

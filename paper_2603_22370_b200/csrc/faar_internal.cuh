@@ -216,6 +216,8 @@ struct faar_gemm_args {
   const void* A; int64_t lda;
   const void* B; int64_t ldb;
   int beside;             // BWD: 1: needs nothing of the launch before it, a plain product (see faar_pdl_wait_first)
+  int ahead;              // FWD, BWD: 1: of what the launch before it on the stream writes it needs the A operand alone, and that launch lets
+                          // it start once all before is complete (faar_pdl_wait_first)
   int whole;              // 1: the contraction is not split over CTA pairs (the order of its sums is that of one pair)
   int a_mn, b_mn;         // 1: the operand is stored with M (N) contiguous instead: A[Kc, M] (lda), B[Kc, N] (ldb)
   uint32_t* status;       // workspace status word
