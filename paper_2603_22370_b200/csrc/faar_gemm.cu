@@ -347,8 +347,9 @@ struct Segment {
 // What a launch needs of the one before it on the stream: everything (0), nothing (BESIDE, see faar_pdl_wait_first), or the A
 // operand alone (AHEAD): the first ring of the B operand and what the epilogue asks for ahead (target values, optimiser state) then
 // come in under the end of that launch.  Step, us: 128 x 256 at 1024 tokens 12.5 -> 12.0, 512 x 512 at 512 16.1 -> 15.7, 256 x 1024 at 1024
-// 16.0 -> 15.6, 64 x 8192 at 300 42.8 -> 41.7, 1000 x 1040 at 777 20.35 -> 20.15, 2048 x 2048 at 1024 40.4 -> 39.9; 512 x 2048 at 4096 29.26 ->
-// 29.38, larger ones the same.
+// 16.0 -> 15.6, 64 x 8192 at 300 42.8 -> 41.7, 1000 x 1040 at 777 20.35 -> 20.15, 2048 x 2048 at 2048 53.3 -> 52.2, 4096 x 2048 at 2000 90.1 ->
+// 88.0, 3000 x 2000 at 3000 98.7 -> 96.3; 512 x 2048 at 4096 29.26 -> 29.38.  Not wide tiles (2048 x 8192 at 4096 247.2 -> 248.6, at 2500
+// 200.3 -> 201.6; their dW launch alone 199.8).
 constexpr int BESIDE = 1, AHEAD = 2;
 
 struct KParams {
@@ -1070,7 +1071,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   cluster_sync_all();                                  // barriers of both CTAs are initialised
   tc_fence_after();
   // set-up done; now wait for the previous kernel's data: all of it, or (AHEAD) only the producer for the A operand
-  if (MODE != FAAR_GEMM_REF && p.columns != 0) faar_pdl_launch();
+  if (MODE != FAAR_GEMM_REF && !WIDE && p.columns != 0) faar_pdl_launch();
   else if (MODE != FAAR_GEMM_BWD) faar_pdl_wait_first();
   else faar_pdl_sync();
   const uint32_t tmem_base = *tmem_slot;
@@ -1098,7 +1099,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     else tc = tile_coord(p, tile, m_tiles);
     return tc;
   };
-  const bool b_ahead = MODE != FAAR_GEMM_REF && p.columns == AHEAD;      // the first ring of B is warp 1's to ask for, under the
+  const bool b_ahead = MODE != FAAR_GEMM_REF && !WIDE && p.columns == AHEAD;      // the first ring of B is warp 1's to ask for, under the
                                                                           // end of the kernel before
 
   if (warp == 0) {
