@@ -459,6 +459,15 @@ FAAR_API int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const 
                              int64_t ldz, const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl,
                              void* dZ_q, void* dH_q, float* loss_out2, void* workspace, size_t workspace_bytes);
 
+/* The same loss from softmax statistics that the logits' products left behind (faar_model_forward_stats,
+ * faar_model_forward_both_stats, at the same tau): stats_fp, stats_q, of the size that faar_logit_stats_size
+ * gives (0: the product is too small for them to pay, and the forward calls refuse to take them), 16-byte aligned.
+ * The logits are then read once instead of twice. */
+FAAR_API int faar_logit_stats_size(faar_ctx* ctx, int T, int vocab, size_t* bytes);
+FAAR_API int faar_align_loss_stats(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
+                                   const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, const void* stats_fp,
+                                   const void* stats_q, void* dZ_q, void* dH_q, float* loss_out2, void* workspace, size_t workspace_bytes);
+
 /* ---- deployable scale-factor layout ---------------------------------------
  * "Hardening and Inference": the final weights are "directly deployable on NVFP4
  * hardware".  Block-scaled tensor-core GEMMs read the E4M3 block scales not
@@ -603,6 +612,14 @@ FAAR_API int faar_model_overlap(const faar_model* model, int batch, int seq, int
 FAAR_API int faar_model_forward_both(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* tokens, const int* positions,
                                      float beta, void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp, void* arena,
                                      size_t arena_bytes, void* Z, void* H, void* workspace, size_t workspace_bytes);
+/* Both with the logits' softmax statistics at temperature tau (see faar_align_loss_stats). */
+FAAR_API int faar_model_forward_stats(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* tokens, const int* positions,
+                                      int quantised, float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, float tau,
+                                      void* stats, void* workspace, size_t workspace_bytes);
+FAAR_API int faar_model_forward_both_stats(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* tokens,
+                                           const int* positions, float beta, void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp,
+                                           void* arena, size_t arena_bytes, void* Z, void* H, float tau, void* stats_fp, void* stats,
+                                           void* workspace, size_t workspace_bytes);
 /* From the loss gradients at the logits (dZ, row stride ldz) and at the last hidden state (dH) back to every V, which is
  * updated in place.  arena: of the quantised forward pass with keep != 0 of the same step. */
 FAAR_API int faar_model_backward(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* positions,

@@ -22,8 +22,7 @@
 
 namespace {
 
-constexpr int AL_THREADS = 1024;
-constexpr int AL_WARPS = AL_THREADS / 32;
+constexpr int AL_THREADS = 1024, AL_STATS_THREADS = 256;      // one CTA per SM; with the products' statistics several
 
 struct AlignParams {
   const __nv_bfloat16* Zfp; const __nv_bfloat16* Zq; long long ldz; int V;
@@ -36,6 +35,7 @@ struct AlignParams {
   float* loss_out2;        // {KL / T, MSE}: written by the cluster that finishes last
   uint32_t* finished;      // workspace: clusters that have, zero between launches
   float kl_scale;
+  const float2* stats_fp; const float2* stats_q; int slots;      // STATS: [T, slots] (maximum, sum) of 128 columns each
   int T;                   // tokens; cluster k takes tokens k, k + the number of clusters, ...
 };
 
@@ -104,14 +104,18 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&p);
 }
 
-// CL CTAs per token.
-template <int CL>
-__global__ void __launch_bounds__(AL_THREADS, 1)
+// CL CTAs per token.  STATS: maxima and sums of the rows' parts come from the products that wrote the logits, so the first pass is
+// over those, a thirtieth of the bytes, and the logits are read once; half the exponentials, too.  Four CTAs of 256 threads an SM, because
+// a token's pass ends in a reduction that one CTA alone would wait for.  Two passes -> this, us: 8192 tokens, vocabulary 128256 1597 ->
+// 1103 (6.3 GB; 1140 with one CTA an SM, 1121 with two), 2000 tokens, vocabulary 32000 120 -> 76 (92, 78).
+template <int CL, bool STATS>
+__global__ void __launch_bounds__(STATS ? AL_STATS_THREADS : AL_THREADS, STATS ? AL_THREADS / AL_STATS_THREADS : 1)
 align_loss_kernel(const AlignParams p) {
+  constexpr int THREADS = STATS ? AL_STATS_THREADS : AL_THREADS, WARPS = THREADS / 32;
   if (CL > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // with the wait below: both CTAs have started
   faar_pdl_sync();
   if (CL > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  __shared__ float4 wred[AL_WARPS];
+  __shared__ float4 wred[WARPS];
   __shared__ float4 xch[2][CL];                                    // by parity of the token: each CTA's maximum and sum, fp and q
   __shared__ alignas(8) float tot[CL][2];                          // rank 0: every CTA's sums
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -149,7 +153,7 @@ align_loss_kernel(const AlignParams p) {
     if (lane == 0) wred[warp] = make_float4(mf, sf, mq, sq);
     __syncthreads();
     if (warp == 0) {
-      float4 r = wred[lane];
+      float4 r = lane < WARPS ? wred[lane] : make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         merge(r.x, r.y, __shfl_xor_sync(0xffffffffu, r.x, o), __shfl_xor_sync(0xffffffffu, r.y, o));
@@ -177,6 +181,15 @@ align_loss_kernel(const AlignParams p) {
     lse_f = r.x + lg2f(r.y);
     lse_q = r.z + lg2f(r.w);
   };
+  // STATS: this thread's part of a token's statistics instead of its first pass
+  auto first_of_stats = [&](int t) {
+    const float2 *f = p.stats_fp + (long long)t * p.slots, *q = p.stats_q + (long long)t * p.slots;
+    for (int i = threadIdx.x; i < p.slots; i += THREADS) {
+      const float2 a = f[i], b = q[i];
+      merge(mf, sf, a.x, a.y);
+      merge(mq, sq, b.x, b.y);
+    }
+  };
   auto row = [&](const __nv_bfloat16* z, int t) { return reinterpret_cast<const uint4*>(z + (long long)t * p.ldz); };
 
   int t = blockIdx.x / CL, parity = 0;
@@ -184,7 +197,9 @@ align_loss_kernel(const AlignParams p) {
   sf = sq = 0.f;
   if (t < p.T) {
     const uint4 *gf = row(p.Zfp, t), *gq = row(p.Zq, t);
-    for (int g = g_first; g < g_end; g += AL_THREADS) first(ldg128_policy(gf + g, keep), ldg128_policy(gq + g, keep), g);
+    if (STATS) first_of_stats(t);
+    else
+      for (int g = g_first; g < g_end; g += THREADS) first(ldg128_policy(gf + g, keep), ldg128_policy(gq + g, keep), g);
     combine(parity);
   }
   for (; t < p.T; t += n_cl) {
@@ -197,12 +212,22 @@ align_loss_kernel(const AlignParams p) {
     mf = mq = -INFINITY;
     sf = sq = 0.f;
     uint4 a1 = make_uint4(0u, 0u, 0u, 0u), b1 = a1;
-    if (more && g_first < g_end) { a1 = ldg128_policy(nf + g_first, keep); b1 = ldg128_policy(nq + g_first, keep); }
-    for (int g = g_first; g < g_end; g += AL_THREADS) {
-      uint4 va = ldg128_policy(gf + g, stream), vb = ldg128_policy(gq + g, stream);
-      if (more) {                                                  // the next token's first pass, its loads one group ahead
+    if (STATS) {
+      if (more) first_of_stats(tn);
+      if (g_first < g_end) { a1 = ldg128_policy(gf + g_first, stream); b1 = ldg128_policy(gq + g_first, stream); }
+    } else if (more && g_first < g_end) { a1 = ldg128_policy(nf + g_first, keep); b1 = ldg128_policy(nq + g_first, keep); }
+    for (int g = g_first; g < g_end; g += THREADS) {
+      uint4 va, vb;
+      if (STATS) {                                                 // the row itself, its loads one group ahead
+        va = a1; vb = b1;
+        const int gn = g + THREADS;
+        if (gn < g_end) { a1 = ldg128_policy(gf + gn, stream); b1 = ldg128_policy(gq + gn, stream); }
+      } else {
+        va = ldg128_policy(gf + g, stream); vb = ldg128_policy(gq + g, stream);
+      }
+      if (!STATS && more) {                                                  // the next token's first pass, its loads one group ahead
         const uint4 a = a1, b = b1;
-        const int gn = g + AL_THREADS;
+        const int gn = g + THREADS;
         if (gn < g_end) { a1 = ldg128_policy(nf + gn, keep); b1 = ldg128_policy(nq + gn, keep); }
         first(a, b, g);
       }
@@ -231,7 +256,7 @@ align_loss_kernel(const AlignParams p) {
       const __nv_bfloat16* hf = p.Hfp + (long long)t * p.ldh;
       const __nv_bfloat16* hq = p.Hq + (long long)t * p.ldh;
       __nv_bfloat16* dh = p.dH ? p.dH + (long long)t * p.ldh : nullptr;
-      for (int g = rank * AL_THREADS + threadIdx.x; 8 * g < p.D; g += CL * AL_THREADS) {
+      for (int g = rank * THREADS + threadIdx.x; 8 * g < p.D; g += CL * THREADS) {
         const int nv = min(8, p.D - 8 * g);
         float a[8], b[8], d[8];
         unpack8(reinterpret_cast<const uint4*>(hf)[g], a);         // rows are padded to 8 columns (ldh >= ceil8(D))
@@ -264,7 +289,7 @@ align_loss_kernel(const AlignParams p) {
   __syncthreads();
   if (threadIdx.x == 0) {
     float a = 0.f, b = 0.f;
-    for (int w = 0; w < AL_WARPS; ++w) { a += wred[w].x; b += wred[w].y; }
+    for (int w = 0; w < WARPS; ++w) { a += wred[w].x; b += wred[w].y; }
     uint32_t dst = (uint32_t)__cvta_generic_to_shared(&tot[rank][0]);
     if (CL > 1) asm volatile("mapa.shared::cluster.u32 %0, %0, 0;" : "+r"(dst));
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(a), "f"(b) : "memory");
@@ -308,7 +333,8 @@ align_loss_kernel(const AlignParams p) {
 
 int faar_launch_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
                            const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, void* dZ_q,
-                           void* dH_q, float* kl_partials, float* mse_partials, uint32_t* finished, float* loss_out2) {
+                           void* dH_q, float* kl_partials, float* mse_partials, uint32_t* finished, float* loss_out2, const float2* stats_fp,
+                           const float2* stats_q) {
   AlignParams p;
   p.Zfp = reinterpret_cast<const __nv_bfloat16*>(Z_fp); p.Zq = reinterpret_cast<const __nv_bfloat16*>(Z_q);
   p.ldz = ldz; p.V = vocab;
@@ -331,15 +357,17 @@ int faar_launch_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const vo
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = 2;
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-  cfg.blockDim = dim3(AL_THREADS);
   cfg.stream = ctx->stream;
   cfg.attrs = attr;
   const int sms = ctx->num_sms;
-  const bool two = T > sms / 2 && 2ll * (T < sms ? T : sms) * 4 * vocab > 130ll << 20;
-  const int most = two ? sms / 2 : sms, n = T < most ? T : most;
+  const bool given = stats_fp && stats_q;
+  p.stats_fp = stats_fp; p.stats_q = stats_q; p.slots = (vocab + 127) / 128;
+  cfg.blockDim = dim3(given ? AL_STATS_THREADS : AL_THREADS);
+  const bool two = !given && T > sms / 2 && 2ll * (T < sms ? T : sms) * 4 * vocab > 130ll << 20;
+  const int most = given ? sms * (AL_THREADS / AL_STATS_THREADS) : (two ? sms / 2 : sms), n = T < most ? T : most;
   cfg.gridDim = dim3(two ? 2 * n : n);
   cfg.numAttrs = two ? 2 : 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, two ? align_loss_kernel<2> : align_loss_kernel<1>, p);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, given ? align_loss_kernel<1, true> : (two ? align_loss_kernel<2, false> : align_loss_kernel<1, false>), p);
   if (e != cudaSuccess) return (int)e;
   return (int)cudaGetLastError();
 }

@@ -1033,9 +1033,9 @@ int faar_align_loss_workspace_size(int T, int vocab, size_t* bytes) {
   return FAAR_OK;
 }
 
-int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
-                    const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, void* dZ_q, void* dH_q,
-                    float* loss_out2, void* workspace, size_t workspace_bytes) {
+static int align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz, const void* H_fp,
+                      const void* H_q, int64_t ldh, float tau, float lambda_kl, const void* stats_fp, const void* stats_q, void* dZ_q,
+                      void* dH_q, float* loss_out2, void* workspace, size_t workspace_bytes) {
   if (!ctx || !Z_fp || !Z_q || !H_fp || !H_q || !loss_out2) return FAAR_ERR_INVALID_ARG;
   if (!(tau > 0.f) || !isfinite(tau) || !isfinite(lambda_kl)) return FAAR_ERR_INVALID_ARG;
   if (T <= 0 || vocab <= 0 || hidden <= 0) return FAAR_ERR_SHAPE;
@@ -1052,7 +1052,31 @@ int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_f
   float* kl_p = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(workspace) + FAAR_WS_HEADER);
   float* mse_p = kl_p + (size_t)T;
   return cuda_fail(ctx, faar_launch_align_loss(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, dZ_q, dH_q, kl_p,
-                                               mse_p, reinterpret_cast<uint32_t*>(workspace) + 6, loss_out2));
+                                               mse_p, reinterpret_cast<uint32_t*>(workspace) + 6, loss_out2,
+                                               reinterpret_cast<const float2*>(stats_fp), reinterpret_cast<const float2*>(stats_q)));
+}
+
+int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
+                    const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, void* dZ_q, void* dH_q,
+                    float* loss_out2, void* workspace, size_t workspace_bytes) {
+  return align_loss(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, nullptr, nullptr, dZ_q, dH_q, loss_out2, workspace,
+                    workspace_bytes);
+}
+
+int faar_align_loss_stats(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz, const void* H_fp,
+                          const void* H_q, int64_t ldh, float tau, float lambda_kl, const void* stats_fp, const void* stats_q, void* dZ_q,
+                          void* dH_q, float* loss_out2, void* workspace, size_t workspace_bytes) {
+  if (!stats_fp || !stats_q) return FAAR_ERR_INVALID_ARG;
+  if (!aligned16(stats_fp) || !aligned16(stats_q)) return FAAR_ERR_ALIGN;
+  return align_loss(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, stats_fp, stats_q, dZ_q, dH_q, loss_out2, workspace,
+                    workspace_bytes);
+}
+
+int faar_logit_stats_size(faar_ctx* ctx, int T, int vocab, size_t* bytes) {
+  if (!ctx || !bytes) return FAAR_ERR_INVALID_ARG;
+  if (T <= 0 || vocab <= 0) return FAAR_ERR_SHAPE;
+  *bytes = vocab % 16 == 0 && faar_logit_stats_pay(ctx, T, vocab) ? (size_t)T * (size_t)((vocab + 127) / 128) * sizeof(float2) : 0;
+  return FAAR_OK;
 }
 
 int faar_harden_pack(faar_ctx* ctx, const faar_shape* s, const float* V, const uint8_t* code, const uint8_t* scales,

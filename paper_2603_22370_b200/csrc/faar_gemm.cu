@@ -79,7 +79,7 @@ constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2, SHORT_TILES = 3,
 constexpr int SHORT_BLOCKS = 40;
 constexpr int SHORT_SMEM = 387 * 512;          // with the system's 1 KB below the 196 KB carve-out
 constexpr int SHORT_CARVEOUT = 85;             // percent of the 228 KB: 193.8, which is rounded up to the size on offer, 196 KB
-constexpr int GATED_FWD = 8, GATED_BWD = 10, ROPE = 16;   // MN (see the kernel) of the gated product's launches and of q / k / v's
+constexpr int GATED_FWD = 8, GATED_BWD = 10, ROPE = 16, STATS = 32;   // MN (see the kernel) of the gated product's launches, of q / k / v's, of logits'
 constexpr int GATE_COLS = 32, GATE_PANEL = 32 * GATE_COLS * 2;        // backward: a warp's 32 rows x 32 columns in BF16
 template <int MODE, int SHAPE = PLAIN_TILES, int MN = 0> struct Cfg {
   static constexpr bool WIDE = SHAPE == WIDE_TILES, SHORT = SHAPE == SHORT_TILES, SPLIT = SHAPE == SPLIT_TILES || SHAPE == SPLIT_NARROW;
@@ -431,6 +431,11 @@ __device__ __forceinline__ int tile_count(const KParams& p, int m_tiles) {
   return 2 * m_tiles * p.n_main - p.n_full + (p.narrow ? m_tiles : 0);
 }
 
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&p);
@@ -665,6 +670,25 @@ __device__ __forceinline__ void epi_rope(const KParams& p, uint32_t trow, int ro
   }
 }
 
+// REF of an LM head's logits (whole 256-wide tiles): with the BF16 values go, per row and 128 columns, the maximum m of y = c z and the
+// sum of 2^(y - m) (p.partials: [M, slots] pairs; p.mse2c: c), from which the alignment loss has a row's log-sum-exp without a pass
+// of its own over the logits.  A warp's 128 columns are one slot; its lanes keep (m, s) of their rows over the 32 columns in
+// registers.  Under the main loop: [8192, 128256] over 2048 2.85 ms either way, [2000, 32000] 150 us.
+__device__ __forceinline__ void stats_update(const KParams& p, const uint32_t (&acc)[16], float& m, float& s) {
+  float y[16], mx = -INFINITY;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint32_t w = pack_bf16x2(__uint_as_float(acc[2 * j]), __uint_as_float(acc[2 * j + 1]));
+    y[2 * j] = __uint_as_float(w << 16);
+    y[2 * j + 1] = __uint_as_float(w & 0xFFFF0000u);
+    mx = fmaxf(mx, fmaxf(y[2 * j], y[2 * j + 1]));
+  }
+  mx *= p.mse2c;                                        // c > 0: scaling keeps the order
+  if (mx > m) { s *= ex2_approx(m - mx); m = mx; }      // 2^-inf = 0 on the first chunk
+#pragma unroll
+  for (int j = 0; j < 16; ++j) s += ex2_approx(fmaf(y[j], p.mse2c, -m));
+}
+
 // FWD: residual, sum of squares, dY^T.
 // Y_ref[t0..t0+15, o] for this lane's output feature o, as it is in memory: anything done to a value here (widening BF16, a
 // select at the matrix edge) would wait for it here, one latency per chunk of 16 columns.  Forward kernel, row-major target,
@@ -790,11 +814,6 @@ __device__ __forceinline__ float epi_fwd_vec(const KParams& p, int o, int t0, co
 __device__ __forceinline__ float sqrt_approx(float x) {       // sqrt(0) = 0, about 1 ulp
   float y;
   asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -1001,7 +1020,8 @@ __device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t parts, int
 // MN: bit 0 = the A operand, bit 1 = the B operand is stored with its M / N index contiguous (KParams.a_mn / b_mn);
 // a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.  Bit 2 (REF): the
 // accumulator's rows are the result's columns; compiled in as well (as a branch it cost 0.1 us in every small product).  Bit 3
-// (REF): the gated product's epilogue, forward, or backward where B is N-contiguous.  Bit 4 (REF): heads turn by their position.
+// (REF): the gated product's epilogue, forward, or backward where B is N-contiguous.  Bit 4 (REF): heads turn by their position.  Bit 5
+// (REF): each row's softmax statistics leave with it.
 // SHAPE: one of the tile forms (see Cfg).
 constexpr int MIN_SPLIT_BLOCKS = 12;            // contractions of fewer k blocks stay whole (see pick_splits)
 template <int MODE, int OPT, int SHAPE, int MN>
@@ -1411,6 +1431,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         } else {
           // REF: two chunks' accumulators in flight (a warp's column count is a multiple of 16: the second may be absent)
           constexpr int STEP = MODE == FAAR_GEMM_REF ? 32 : 16;
+          float sm = -INFINITY, ssum = 0.f;              // STATS
           const bool apart = COLUMNS && BN > 128 && k_blocks >= APART_BLOCKS && tile + n_pairs < total_tiles;
 #pragma unroll 1
           for (int c = col_begin; c < col_end; c += STEP) {
@@ -1432,6 +1453,10 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               } else {
                 epi_ref(p, o, n0 + c, r);
                 if (second) epi_ref(p, o, n0 + c + 16, r2);
+                if constexpr (MN == STATS) {
+                  stats_update(p, r, sm, ssum);
+                  if (second) stats_update(p, r2, sm, ssum);
+                }
               }
             } else {
               float yr[16];
@@ -1440,6 +1465,10 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               tmem_ld_wait();
               warp_acc += epi_fwd(p, o, n0 + c, r, yr);
             }
+          }
+          if constexpr (MN == STATS) {
+            const int slots = (p.N + 127) / 128, slot = (n0 + col_begin) / 128;
+            if (o < p.M && n0 + col_begin < p.N) reinterpret_cast<float2*>(p.partials)[(long long)o * slots + slot] = make_float2(sm, ssum);
           }
         }
       }
@@ -1724,7 +1753,7 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
   kp.stages = ring < MAX_STAGES ? ring : MAX_STAGES;
   const int m_tiles = (a->M + 2 * BM - 1) / (2 * BM), n_cols = (a->N + bn - 1) / bn;
   const int wide_w1 = kp.n_main, wide_w = BN_MAX + wide_w1, wide_cols = (a->N + wide_w - 1) / wide_w;
-  const bool halves = MN != ROPE || bn / 2 % a->head_dim == 0;       // a half-width tile, too, is whole heads
+  const bool halves = MN != STATS && (MN != ROPE || bn / 2 % a->head_dim == 0);       // a half-width tile, too, is whole heads
   kp.narrow = (SHAPE == PLAIN_TILES || SHAPE == SHORT_TILES) && halves && bn % 32 == 0 && bn > 32 && a->N - (n_cols - 1) * bn <= bn / 2;
   kp.n_main = WIDE ? wide_w1 : n_cols - kp.narrow;
   if (MODE == FAAR_GEMM_BWD) {
@@ -1826,6 +1855,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
       if (bn != 32) bn = (bn + 63) / 64 * 64;
       return launch_variant<MODE, OPT, PLAIN_TILES, GATED_FWD>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
     }
+    if (a->stats) return launch_variant<MODE, OPT, PLAIN_TILES, STATS>(ctx, a, kp, n_partials_out, BN_MAX, max_pairs, cfg);
     if (a->rope) {                                  // whole heads
       bn = (bn + a->head_dim - 1) / a->head_dim * a->head_dim;
       return launch_variant<MODE, OPT, PLAIN_TILES, ROPE>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
@@ -1860,9 +1890,16 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
 // would be padding that is staged all the same.  M on the accumulator's rows -> N, us: 1 row of 8192 over 2048 15.1 -> 10.6,
 // 64 rows 12.8 -> 12.0, 128 rows 13.1 -> 12.2, 160 rows 13.1 -> 13.8; input gradient of 8 rows of 8192 over 2048 14.5 -> 11.9.
 static bool result_columns(const faar_gemm_args* a) {
-  if (a->yref_t || a->gated || a->rope) return false;
+  if (a->yref_t || a->gated || a->rope || a->stats) return false;
   const long long row = a->ldy * (a->yout_dtype == FAAR_BF16 ? 2 : 4);
   return a->M <= BM || row % 16 != 0 || (reinterpret_cast<uintptr_t>(a->Yout) & 15) != 0;
+}
+
+// Whether the logits' statistics are worth taking: where every CTA pair has 256-wide tiles anyway (and more than a half-empty row
+// block); a smaller product is better cut into narrower ones.
+bool faar_logit_stats_pay(const faar_ctx* ctx, int T, int vocab) {
+  const long long tiles = (long long)((T + 2 * BM - 1) / (2 * BM)) * ((vocab + BN_MAX - 1) / BN_MAX);
+  return T > BM && tiles >= ctx->num_sms / 2;
 }
 
 int faar_launch_wait_selftest(faar_ctx* ctx, uint32_t* status, unsigned long long limit_ns) {
@@ -1891,6 +1928,9 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
         a->yout_dtype != FAAR_BF16 || (a->gated == FAAR_GATED_FWD ? !a->act || a->N % 2 : !a->Yout || !a->gate_up))
       return (int)cudaErrorInvalidValue;
   }
+  if (a->stats && (a->mode != FAAR_GEMM_REF || !a->whole || a->a_mn || a->b_mn || a->gated || a->rope || a->yref_t || a->N % 16 || a->ldy % 8 ||
+                   (reinterpret_cast<uintptr_t>(a->Yout) & 15) || (reinterpret_cast<uintptr_t>(a->stats) & 7) || a->yout_dtype != FAAR_BF16))
+    return (int)cudaErrorInvalidValue;
   if (a->rope && (a->mode != FAAR_GEMM_REF || !a->whole || a->a_mn || a->b_mn || a->gated || (a->head_dim != 64 && a->head_dim != 128) ||
                       a->N % a->head_dim || (reinterpret_cast<uintptr_t>(a->rope) & 7) || a->rope_cols % a->head_dim || a->ldy % 16 || (reinterpret_cast<uintptr_t>(a->Yout) & 31) ||
                       a->yout_dtype != FAAR_BF16))
@@ -1912,6 +1952,7 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
   kp.Yout = a->Yout; kp.yout_dtype = a->yout_dtype; kp.ldy = a->ldy;
   kp.Yref = a->Yref; kp.yref_dtype = a->yref_dtype; kp.yref_t = a->yref_t;
   kp.dYt = a->dYt; kp.ld_dyt = a->ld_dyt; kp.mse2c = a->mse2c; kp.act_scale = a->act_scale; kp.partials = a->partials;
+  if (a->stats) { kp.partials = reinterpret_cast<float*>(a->stats); kp.mse2c = a->stats_c; }
   if (a->rope) {
     kp.Yref = a->rope; kp.yref_dtype = a->head_dim; kp.ld_dyt = a->rope_cols;
   }

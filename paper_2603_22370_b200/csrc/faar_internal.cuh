@@ -165,7 +165,8 @@ int faar_launch_swizzle_scales(faar_ctx*, int rows, int cols, const uint8_t* in,
 // Eq. 6's data terms: one partial of each per CTA or cluster, at most one per token; `finished` is zero between launches
 int faar_launch_align_loss(faar_ctx*, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
                            const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, void* dZ_q,
-                           void* dH_q, float* kl_partials, float* mse_partials, uint32_t* finished, float* loss_out2);
+                           void* dH_q, float* kl_partials, float* mse_partials, uint32_t* finished, float* loss_out2,
+                           const float2* stats_fp = nullptr, const float2* stats_q = nullptr);      // of the logits' products, both or none
 int faar_launch_silu_mul(faar_ctx*, int rows, int cols, const void* gate, int64_t ldg, const void* up, int64_t ldu,
                          void* out, int64_t ldo);
 int faar_launch_rmsnorm(faar_ctx*, int rows, int cols, const void* x, int64_t ldx, const void* b, int64_t ldb,
@@ -227,6 +228,7 @@ struct faar_gemm_args {
   int yref_t;                                  // FWD: Y stored transposed [O, ldy]; REF: rows of Yout padded to 16 columns
   int gated;                                   // REF: an epilogue of the gated product, FAAR_GATED_FWD or FAAR_GATED_BWD (0: plain)
   void* act; const void* gate_up;              // and its further tensors (see faar_gemm.cu)
+  float2* stats; float stats_c;                // REF: softmax statistics of every row, [M, ceil(N / 128)] (null: not wanted)
   const float2* rope;                          // REF: the first rope_cols columns of the result are heads that turn by their row's
   int rope_cols, head_dim;                     // angles, [head_dim / 2, M] sines and cosines (null: none do)
   __nv_bfloat16* dYt; int64_t ld_dyt;          // FWD: [M(O), ld_dyt]
@@ -244,6 +246,7 @@ struct faar_gemm_args {
 };
 // n_partials_out: number of floats a FWD launch writes to args.partials
 int faar_launch_gemm(faar_ctx*, const faar_gemm_args*, int* n_partials_out);
+bool faar_logit_stats_pay(const faar_ctx*, int T, int vocab);
 int faar_gemm_max_partials(const faar_ctx*, int M, int N);
 int faar_launch_wait_selftest(faar_ctx*, uint32_t* status, unsigned long long limit_ns);
 

@@ -117,6 +117,23 @@ int product_gated_bwd(faar_ctx* ctx, size_t T, int f, int K, const void* dY, con
   return faar_launch_gemm(ctx, &a, nullptr);
 }
 
+// Logits and, if wanted, their rows' softmax statistics at temperature tau
+struct Stats { float tau; void* out; };
+int product_logits(faar_ctx* ctx, const faar_model* m, size_t T, const void* H, void* Z, const Stats& st, void* ws) {
+  if (!st.out) return product(ctx, T, m->vocab, m->hidden, H, m->hidden, m->lm_head, m->hidden, false, Z, m->vocab, ws);
+  faar_gemm_args a = {};
+  a.mode = FAAR_GEMM_REF;
+  a.M = (int)T; a.N = m->vocab; a.Kc = m->hidden;
+  a.A = H; a.lda = m->hidden;
+  a.B = m->lm_head; a.ldb = m->hidden;
+  a.whole = 1;
+  a.status = reinterpret_cast<uint32_t*>(ws);
+  a.Yout = Z; a.yout_dtype = FAAR_BF16; a.ldy = m->vocab;
+  a.stats = reinterpret_cast<float2*>(st.out);
+  a.stats_c = (float)(1.4426950408889634 / (double)st.tau);
+  return faar_launch_gemm(ctx, &a, nullptr);
+}
+
 int group_rows(const faar_linear_group& g) {
   int r = 0;
   for (int i = 0; i < g.n; ++i) r += g.lin[i].rows;
@@ -254,7 +271,7 @@ int begin(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tok
 // The blocks, the final norm and the LM head.  begun: the arena that begin() has filled, this pass's or that of another pass
 // (which keeps its activations) on the same tokens.
 int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, bool quantised, float beta, bool keep, uint8_t* arena,
-            const uint8_t* begun, void* Z, void* Hout, void* ws) {
+            const uint8_t* begun, void* Z, void* Hout, const Stats& stats, void* ws) {
   const Sizes s = sizes(m, batch, seq);
   const Arena A(s, m->n_layers, keep);
   const int T = (int)s.T;
@@ -300,8 +317,7 @@ int forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, bool quantis
                             last ? m->final_norm : m->blocks[l + 1].attn_norm, m->eps, last ? Hout : n + A.b.hn, s.d,
                             reinterpret_cast<float*>(last ? arena + A.rstd_f : n + A.b.rstd1));
   }
-  if (!e) e = product(ctx, s.T, m->vocab, s.d, Hout, s.d, m->lm_head, s.d, false, Z, m->vocab, ws);
-  return e;
+  return e ? e : product_logits(ctx, m, s.T, Hout, Z, stats, ws);
 }
 
 int backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* pos, const faar_hparams* hp, uint8_t* arena,
@@ -353,7 +369,7 @@ int backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* 
 // Both forward passes at once: the frozen one on the context's side stream, between two events, behind the first block's
 // input and norm, which they share.  The products of either use nothing of the workspace but its status word.
 int forward_both(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* pos, float beta, uint8_t* arena_fp,
-                 void* Z_fp, void* H_fp, uint8_t* arena, void* Z, void* H, void* ws) {
+                 void* Z_fp, void* H_fp, uint8_t* arena, void* Z, void* H, const Stats& stats_fp, const Stats& stats, void* ws) {
   cudaError_t ce = cudaSuccess;
   if (!ctx->side_stream) ce = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
   if (ce == cudaSuccess && !ctx->ev_fork) ce = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
@@ -366,11 +382,11 @@ int forward_both(faar_ctx* ctx, const faar_model* m, int batch, int seq, const i
   if (ce == cudaSuccess) ce = cudaStreamWaitEvent(ctx->side_stream, ctx->ev_fork, 0);
   if (ce != cudaSuccess) return (int)ce;
   ctx->stream = ctx->side_stream;
-  e = forward(ctx, m, batch, seq, false, beta, false, arena_fp, arena, Z_fp, H_fp, ws);
+  e = forward(ctx, m, batch, seq, false, beta, false, arena_fp, arena, Z_fp, H_fp, stats_fp, ws);
   ctx->stream = main;
   // joined whatever happened, so that the caller's stream orders everything that was enqueued
   ce = cudaEventRecord(ctx->ev_join, ctx->side_stream);
-  if (!e) e = forward(ctx, m, batch, seq, true, beta, true, arena, arena, Z, H, ws);
+  if (!e) e = forward(ctx, m, batch, seq, true, beta, true, arena, arena, Z, H, stats, ws);
   if (ce == cudaSuccess) ce = cudaStreamWaitEvent(main, ctx->ev_join, 0);
   return e ? e : (int)ce;
 }
@@ -404,9 +420,15 @@ int faar_model_sizes(const faar_model* m, int batch, int seq, int keep, size_t* 
   return FAAR_OK;
 }
 
-int faar_model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, int quantised,
-                       float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, void* workspace,
-                       size_t workspace_bytes) {
+static int check_stats(faar_ctx* ctx, const faar_model* m, int batch, int seq, const Stats& st) {
+  if (!st.out) return FAAR_OK;
+  if (!(st.tau > 0.f) || !isfinite(st.tau)) return FAAR_ERR_INVALID_ARG;
+  if (!aligned(st.out)) return FAAR_ERR_ALIGN;
+  return faar_logit_stats_pay(ctx, batch * seq, m->vocab) ? FAAR_OK : FAAR_ERR_SHAPE;
+}
+static int model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, int quantised,
+                         float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, const Stats& stats, void* workspace,
+                         size_t workspace_bytes) {
   int st = check_model(ctx, m, batch, seq, quantised != 0, nullptr, workspace, workspace_bytes);
   if (st) return st;
   if (!tokens || !positions || !arena || !Z || !H) return FAAR_ERR_INVALID_ARG;
@@ -415,11 +437,25 @@ int faar_model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, c
   size_t need = 0, scratch = 0;
   if ((st = faar_model_sizes(m, batch, seq, keep, &need, &scratch))) return st;
   if (arena_bytes < need) return FAAR_ERR_WORKSPACE;
+  if ((st = check_stats(ctx, m, batch, seq, stats))) return st;
   Device dev(ctx->device);
   if (dev.err) return status(ctx, dev.err);
   uint8_t* const at = reinterpret_cast<uint8_t*>(arena);
   const int e = begin(ctx, m, batch, seq, tokens, positions, keep != 0, at);
-  return status(ctx, e ? e : forward(ctx, m, batch, seq, quantised != 0, beta, keep != 0, at, at, Z, H, workspace));
+  return status(ctx, e ? e : forward(ctx, m, batch, seq, quantised != 0, beta, keep != 0, at, at, Z, H, stats, workspace));
+}
+int faar_model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, int quantised,
+                       float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, void* workspace,
+                       size_t workspace_bytes) {
+  return model_forward(ctx, m, batch, seq, tokens, positions, quantised, beta, keep, arena, arena_bytes, Z, H, {1.f, nullptr}, workspace,
+                       workspace_bytes);
+}
+int faar_model_forward_stats(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, int quantised,
+                             float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, float tau, void* stats, void* workspace,
+                             size_t workspace_bytes) {
+  if (!stats) return FAAR_ERR_INVALID_ARG;
+  return model_forward(ctx, m, batch, seq, tokens, positions, quantised, beta, keep, arena, arena_bytes, Z, H, {tau, stats}, workspace,
+                       workspace_bytes);
 }
 
 // Overlap pays while the passes are chains of launches that leave much of the GPU idle.  Whole alignment step, one pass after
@@ -435,9 +471,9 @@ int faar_model_overlap(const faar_model* m, int batch, int seq, int* overlap) {
   return FAAR_OK;
 }
 
-int faar_model_forward_both(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, float beta,
-                            void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp, void* arena, size_t arena_bytes, void* Z,
-                            void* H, void* workspace, size_t workspace_bytes) {
+static int model_forward_both(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, float beta,
+                              void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp, void* arena, size_t arena_bytes, void* Z, void* H,
+                              const Stats& stats_fp, const Stats& stats, void* workspace, size_t workspace_bytes) {
   int st = check_model(ctx, m, batch, seq, false, nullptr, workspace, workspace_bytes);
   if (!st) st = check_model(ctx, m, batch, seq, true, nullptr, workspace, workspace_bytes);
   if (st) return st;
@@ -449,10 +485,25 @@ int faar_model_forward_both(faar_ctx* ctx, const faar_model* m, int batch, int s
   if ((st = faar_model_sizes(m, batch, seq, 0, &need_fp, &scratch))) return st;
   if ((st = faar_model_sizes(m, batch, seq, 1, &need, &scratch))) return st;
   if (arena_fp_bytes < need_fp || arena_bytes < need) return FAAR_ERR_WORKSPACE;
+  if ((st = check_stats(ctx, m, batch, seq, stats_fp)) || (st = check_stats(ctx, m, batch, seq, stats))) return st;
   Device dev(ctx->device);
   if (dev.err) return status(ctx, dev.err);
   return status(ctx, forward_both(ctx, m, batch, seq, tokens, positions, beta, reinterpret_cast<uint8_t*>(arena_fp), Z_fp, H_fp,
-                                  reinterpret_cast<uint8_t*>(arena), Z, H, workspace));
+                                  reinterpret_cast<uint8_t*>(arena), Z, H, stats_fp, stats, workspace));
+}
+
+int faar_model_forward_both(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, float beta,
+                            void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp, void* arena, size_t arena_bytes, void* Z,
+                            void* H, void* workspace, size_t workspace_bytes) {
+  return model_forward_both(ctx, m, batch, seq, tokens, positions, beta, arena_fp, arena_fp_bytes, Z_fp, H_fp, arena, arena_bytes, Z, H,
+                            {1.f, nullptr}, {1.f, nullptr}, workspace, workspace_bytes);
+}
+int faar_model_forward_both_stats(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, float beta,
+                                  void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp, void* arena, size_t arena_bytes, void* Z,
+                                  void* H, float tau, void* stats_fp, void* stats, void* workspace, size_t workspace_bytes) {
+  if (!stats_fp || !stats) return FAAR_ERR_INVALID_ARG;
+  return model_forward_both(ctx, m, batch, seq, tokens, positions, beta, arena_fp, arena_fp_bytes, Z_fp, H_fp, arena, arena_bytes, Z, H,
+                            {tau, stats_fp}, {tau, stats}, workspace, workspace_bytes);
 }
 
 int faar_model_backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* positions, const faar_hparams* hp,

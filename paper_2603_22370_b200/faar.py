@@ -59,6 +59,8 @@ SIGNATURES = {
     "faar_harden_pack": (_I, [_P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _I]),
     "faar_align_loss_workspace_size": (_I, [_I, _I, _P]),
     "faar_align_loss": (_I, [_P, _I, _I, _I, _P, _P, _L, _P, _P, _L, _F, _F, _P, _P, _P, _P, _Z]),
+    "faar_logit_stats_size": (_I, [_P, _I, _I, _P]),
+    "faar_align_loss_stats": (_I, [_P, _I, _I, _I, _P, _P, _L, _P, _P, _L, _F, _F, _P, _P, _P, _P, _P, _P, _Z]),
     "faar_swizzle_scales": (_I, [_P, _I, _I, _P, _P, _Z]),
     "faar_silu_mul": (_I, [_P, _I, _I, _P, _L, _P, _L, _P, _L]),
     "faar_rmsnorm": (_I, [_P, _I, _I, _P, _L, _P, _F, _P, _L, _P]),
@@ -78,6 +80,8 @@ SIGNATURES = {
     "faar_model_forward": (_I, [_P, _P, _I, _I, _P, _P, _I, _F, _I, _P, _Z, _P, _P, _P, _Z]),
     "faar_model_overlap": (_I, [_P, _I, _I, _P]),
     "faar_model_forward_both": (_I, [_P, _P, _I, _I, _P, _P, _F, _P, _Z, _P, _P, _P, _Z, _P, _P, _P, _Z]),
+    "faar_model_forward_stats": (_I, [_P, _P, _I, _I, _P, _P, _I, _F, _I, _P, _Z, _P, _P, _F, _P, _P, _Z]),
+    "faar_model_forward_both_stats": (_I, [_P, _P, _I, _I, _P, _P, _F, _P, _Z, _P, _P, _P, _Z, _P, _P, _F, _P, _P, _P, _Z]),
     "faar_model_backward": (_I, [_P, _P, _I, _I, _P, _P, _P, _Z, _P, _L, _P, _P, _Z, _P, _Z]),
     "faar_nvfp4_gemm": (_I, [_P, _I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _L, _P, _Z]),
 }
@@ -303,6 +307,17 @@ def align_loss(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambd
            dH_q, loss_out2, ws, ws.numel()), "faar_align_loss")
 
 
+def logit_stats_size(ctx, T, vocab) -> int:
+    n = C.c_size_t(0)
+    _check(lib().faar_logit_stats_size(ctx._h, T, vocab, C.byref(n)), "faar_logit_stats_size")
+    return n.value
+
+
+def align_loss_stats(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, stats_fp, stats_q, dZ_q, dH_q, loss_out2, ws):
+    _check(_fast().faar_align_loss_stats(ctx._n, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, stats_fp, stats_q, dZ_q,
+                                         dH_q, loss_out2, ws, ws.numel()), "faar_align_loss_stats")
+
+
 def swizzle_scales(ctx, rows, cols, scales, scales_tiled):
     _check(_fast().faar_swizzle_scales(ctx._n, rows, cols, scales, scales_tiled, scales_tiled.numel()),
            "faar_swizzle_scales")
@@ -414,6 +429,17 @@ def model_overlap(model: Model, batch: int, seq: int) -> bool:
 def model_forward_both(ctx, model, batch, seq, tokens, positions, beta, arena_fp, Z_fp, H_fp, arena, Z, H, ws):
     _check(_fast().faar_model_forward_both(ctx._n, model, batch, seq, tokens, positions, beta, arena_fp, arena_fp.numel(), Z_fp, H_fp,
                                            arena, arena.numel(), Z, H, ws, ws.numel()), "faar_model_forward_both")
+
+
+def model_forward_stats(ctx, model, batch, seq, tokens, positions, quantised, beta, keep, arena, Z, H, tau, stats, ws):
+    _check(_fast().faar_model_forward_stats(ctx._n, model, batch, seq, tokens, positions, int(quantised), beta, int(keep), arena,
+                                            arena.numel(), Z, H, tau, stats, ws, ws.numel()), "faar_model_forward_stats")
+
+
+def model_forward_both_stats(ctx, model, batch, seq, tokens, positions, beta, arena_fp, Z_fp, H_fp, arena, Z, H, tau, stats_fp, stats, ws):
+    _check(_fast().faar_model_forward_both_stats(ctx._n, model, batch, seq, tokens, positions, beta, arena_fp, arena_fp.numel(), Z_fp, H_fp,
+                                                 arena, arena.numel(), Z, H, tau, stats_fp, stats, ws, ws.numel()),
+           "faar_model_forward_both_stats")
 
 
 def model_backward(ctx, model, batch, seq, positions, hp, arena, dZ, ldz, dH, scratch, ws):

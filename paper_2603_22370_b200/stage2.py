@@ -120,9 +120,10 @@ class Stage2Model:
     def _plan_regions(self):
         """Where the buffers of a small model's step lie in its one allocation: (name, first byte, bytes)."""
         z, h = 2 * self.T * self.cfg.vocab, 2 * self.T * self.cfg.hidden
+        stats = faar.logit_stats_size(self.ctx, self.T, self.cfg.vocab)
         self._regions, at = [], 0
         for name, n in (("fp", self.arena_bytes[False]), ("q", self.arena_bytes[True]), ("scratch", self.scratch_bytes), ("Z_fp", z),
-                        ("H_fp", h), ("Z_q", z), ("H_q", h), ("dZ", z), ("dH", h)):
+                        ("H_fp", h), ("Z_q", z), ("H_q", h), ("dZ", z), ("dH", h), ("stats_fp", stats), ("stats_q", stats)):
             self._regions.append((name, at, n))
             at += (n + 255) // 256 * 256
         self._region_bytes, self._regions_of = at, (self.cfg.vocab, self.cfg.hidden)
@@ -171,10 +172,14 @@ class Stage2Model:
         """tokens: [batch*seq] int32 on the device.  Returns (Z [T, vocab], H [T, hidden], activations or None)."""
         return self._forward(self._table(), tokens, quantised, beta, keep)
 
-    def _forward(self, model: faar.Model, tokens, quantised, beta=4.0, keep=False):
+    def _forward(self, model: faar.Model, tokens, quantised, beta=4.0, keep=False, tau=1.0, stats=None):
         arena = torch.empty(self.arena_bytes[bool(keep)], dtype=torch.uint8, device=self.dev)
         Z, H = self._new(self.cfg.vocab), self._new(self.cfg.hidden)
-        faar.model_forward(self.ctx, model, self.batch, self.seq, tokens, self.pos, quantised, beta, keep, arena, Z, H, self.ws)
+        args = (self.ctx, model, self.batch, self.seq, tokens, self.pos, quantised, beta, keep, arena, Z, H)
+        if stats is None:
+            faar.model_forward(*args, self.ws)
+        else:
+            faar.model_forward_stats(*args, tau, stats, self.ws)
         return Z, H, (arena if keep else None)
 
     def _forward_both(self, model: faar.Model, tokens, beta):
@@ -231,21 +236,32 @@ class Stage2Model:
             memory = torch.empty(self._region_bytes, dtype=torch.uint8, device=self.dev)
             base = memory.data_ptr()
             r = {name: faar.Region(base + at, n) for name, at, n in self._regions}
-            faar.model_forward_both(self.ctx, model, self.batch, self.seq, tokens, self.pos, beta, r["fp"], r["Z_fp"], r["H_fp"], r["q"], r["Z_q"],
-                                    r["H_q"], self.ws)
-            faar.align_loss(self.ctx, self.T, c.vocab, c.hidden, r["Z_fp"], r["Z_q"], c.vocab, r["H_fp"], r["H_q"], c.hidden, tau, lambda_kl,
-                            r["dZ"], r["dH"], self.loss, self.aws)
+            passes = (self.ctx, model, self.batch, self.seq, tokens, self.pos, beta, r["fp"], r["Z_fp"], r["H_fp"], r["q"], r["Z_q"], r["H_q"])
+            loss = (self.ctx, self.T, c.vocab, c.hidden, r["Z_fp"], r["Z_q"], c.vocab, r["H_fp"], r["H_q"], c.hidden, tau, lambda_kl)
+            if r["stats_q"].numel():
+                faar.model_forward_both_stats(*passes, tau, r["stats_fp"], r["stats_q"], self.ws)
+                faar.align_loss_stats(*loss, r["stats_fp"], r["stats_q"], r["dZ"], r["dH"], self.loss, self.aws)
+            else:
+                faar.model_forward_both(*passes, self.ws)
+                faar.align_loss(*loss, r["dZ"], r["dH"], self.loss, self.aws)
             faar.model_backward(self.ctx, model, self.batch, self.seq, self.pos, hp, r["q"], r["dZ"], c.vocab, r["dH"], r["scratch"], self.ws)
             return None
+        c, T = self.cfg, self.T
+        stats = ()                             # of both passes' logits, where their products leave them
         if fp_outputs is None and self.overlap:
             Z_fp, H_fp, Z_q, H_q, saved = self._forward_both(model, tokens, beta)
-        else:
-            Z_fp, H_fp = fp_outputs if fp_outputs is not None else self._forward(model, tokens, quantised=False)[:2]
+        elif fp_outputs is not None:
+            Z_fp, H_fp = fp_outputs
             Z_q, H_q, saved = self._forward(model, tokens, quantised=True, beta=beta, keep=True)
-        c, T = self.cfg, self.T
+        else:
+            n = faar.logit_stats_size(self.ctx, T, c.vocab)
+            if n:
+                stats = tuple(torch.empty(n, dtype=torch.uint8, device=self.dev) for _ in range(2))
+            Z_fp, H_fp = self._forward(model, tokens, quantised=False, tau=tau, stats=stats[0] if n else None)[:2]
+            Z_q, H_q, saved = self._forward(model, tokens, quantised=True, beta=beta, keep=True, tau=tau, stats=stats[1] if n else None)
         dZ, dH = torch.empty_like(Z_q), torch.empty_like(H_q)
-        faar.align_loss(self.ctx, T, c.vocab, c.hidden, Z_fp, Z_q, Z_q.shape[1], H_fp, H_q, c.hidden, tau, lambda_kl, dZ, dH,
-                        self.loss, self.aws)
+        loss = faar.align_loss_stats if stats else faar.align_loss
+        loss(self.ctx, T, c.vocab, c.hidden, Z_fp, Z_q, Z_q.shape[1], H_fp, H_q, c.hidden, tau, lambda_kl, *stats, dZ, dH, self.loss, self.aws)
         grads = self._backward(model, dZ, dH, saved, hp, want_dv)
         return {"Z_q": Z_q, "H_q": H_q, "dZ": dZ, "dH": dH, "dV": grads} if want_dv else None
 
