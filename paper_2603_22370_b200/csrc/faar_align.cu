@@ -10,6 +10,7 @@
 // together with the first pass of the next one.  Two tokens' rows per SM would be more than L2 holds at a 128 K vocabulary,
 // so there two CTAs (a cluster on two SMs) share a token, half a row each, and exchange maxima and sums through
 // distributed shared memory.
+// Where the products that wrote the logits left the maxima and sums of the rows' parts as well, the first pass is over those.
 // One token after the other, each pass for itself -> this, us: 2000 tokens, vocabulary 32000 144 -> 122; 512, 8000 23.7 ->
 // 16.6; 3000, 50000 298 -> 251; 8192, 128256 1590 -> 1568 (6.3 GB).
 #include <cuda_bf16.h>

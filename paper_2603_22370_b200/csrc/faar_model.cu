@@ -1,10 +1,10 @@
 // Forward and backward passes of a whole decoder model (full-model alignment, Procedure steps 16-17 and 21-23): the
 // sequence of kernel launches for every block, enqueued by one call.  No arithmetic here and no kernels of its own.
 //
-// Why native: a pass is a chain of 25 launches per block, many of a few microseconds each.  Issued one by one from Python
-// they cost 7.5 us of host time each, more than the kernels of a small model take: an alignment step of two 128-wide blocks
-// on 192 tokens took 770 us for 500 us of device time.  Activations live in one caller-owned arena per pass at
-// offsets that depend on the sizes alone.
+// Why native: a step is a chain of 28 launches per block (7 in each forward pass, 13 in the backward pass, soft weights), many
+// of a few microseconds each.  Issued one by one from Python a launch cost 7.5 us of host time, more than the kernels of a small
+// model take: an alignment step of two 128-wide blocks on 192 tokens took 770 us for 500 us of device time (177 us as it is
+// now).  Activations live in one caller-owned arena per pass at offsets that depend on the sizes alone.
 #include <math.h>
 
 #include "faar_internal.cuh"
