@@ -174,7 +174,8 @@ attn_fwd_kernel(const AttnParams p) {
 // ---- backward, step 0: dsum[b, h, t] = sum_d dO[t, h, d] * O[t, h, d] ------------------------------------------
 // D / 8 lanes share one (token, head) row, 16 bytes of O and of dO each, so a warp takes 256 / D consecutive tokens
 // of one head per pass; consecutive warps take the heads of the same tokens (whole rows of O and dO are read
-// together), and a warp's results are consecutive floats of dsum.
+// together), and a warp's results are consecutive floats of dsum.  (A model's pass of more than 128 tokens has them from the product
+// that forms dO.)
 template <int D>
 __global__ void __launch_bounds__(ATT_THREADS)
 attn_dsum_kernel(const AttnParams p, float* dsum) {
@@ -862,15 +863,19 @@ int launch_fwd(faar_ctx* ctx, const AttnParams& p) {
 }
 
 template <int D>
-int launch_bwd(faar_ctx* ctx, const AttnParams& p, float* dsum, const float2* rope) {
+int launch_bwd(faar_ctx* ctx, const AttnParams& p, float* dsum, const float2* rope, int sum_parts) {
   faar_prof_scope ps(ctx, FAAR_K_ATTENTION);
+  if (sum_parts)                                               // the product that wrote dO left its row sums, too
+    return ctx->tune_attention_fragments ? (int)cudaErrorInvalidValue
+                                         : faar_launch_attention_bwd_tc(ctx, p.B, p.S, p.H, p.Hkv, D, p.q, p.ldq, p.k, p.v, p.ldk, p.dout, p.ldo,
+                                                                        p.lse, dsum, sum_parts, p.dq, p.dk, p.dv, p.scale_log2, rope);
   long long rows = (long long)p.B * p.H * ((p.S + 256 / D - 1) / (256 / D));      // warp passes of the row-sum kernel
   long long blocks = (rows + 3) / 4;
   if (blocks > (long long)ctx->num_sms * 16) blocks = (long long)ctx->num_sms * 16;
   faar_launch_pdl(ctx, attn_dsum_kernel<D>, dim3((int)blocks), dim3(ATT_THREADS), 0, p, dsum);
   const int tiles = (p.S + AT - 1) / AT;
   if (ctx->tune_attention_fragments == 0)
-    return faar_launch_attention_bwd_tc(ctx, p.B, p.S, p.H, p.Hkv, D, p.q, p.ldq, p.k, p.v, p.ldk, p.dout, p.ldo, p.lse, dsum,
+    return faar_launch_attention_bwd_tc(ctx, p.B, p.S, p.H, p.Hkv, D, p.q, p.ldq, p.k, p.v, p.ldk, p.dout, p.ldo, p.lse, dsum, 0,
                                         p.dq, p.dk, p.dv, p.scale_log2, rope);
   if (rope) return (int)cudaErrorInvalidValue;
   if (D == HD && ctx->tune_attention_fragments == 2) {
@@ -903,7 +908,7 @@ int faar_launch_attention_fwd(faar_ctx* ctx, int B, int S, int H, int Hkv, int D
 
 int faar_launch_attention_bwd(faar_ctx* ctx, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                               const void* v, int64_t ldk, const void* out, const void* dout, int64_t ldo, const float* lse,
-                              float* dsum, void* dq, void* dk, void* dv, const float2* rope) {
+                              float* dsum, void* dq, void* dk, void* dv, const float2* rope, int sum_parts) {
   AttnParams p = {};
   p.q = reinterpret_cast<const __nv_bfloat16*>(q); p.k = reinterpret_cast<const __nv_bfloat16*>(k);
   p.v = reinterpret_cast<const __nv_bfloat16*>(v);
@@ -912,5 +917,5 @@ int faar_launch_attention_bwd(faar_ctx* ctx, int B, int S, int H, int Hkv, int D
   p.dq = reinterpret_cast<__nv_bfloat16*>(dq); p.dk = reinterpret_cast<__nv_bfloat16*>(dk); p.dv = reinterpret_cast<__nv_bfloat16*>(dv);
   p.ldq = ldq; p.ldk = ldk; p.ldo = ldo; p.B = B; p.S = S; p.H = H; p.Hkv = Hkv;
   p.scale_log2 = LOG2E / sqrtf((float)D);
-  return D == 64 ? launch_bwd<64>(ctx, p, dsum, rope) : launch_bwd<128>(ctx, p, dsum, rope);
+  return D == 64 ? launch_bwd<64>(ctx, p, dsum, rope, sum_parts) : launch_bwd<128>(ctx, p, dsum, rope, sum_parts);
 }

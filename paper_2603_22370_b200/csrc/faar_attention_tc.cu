@@ -494,8 +494,23 @@ struct TcBwdParams {
   float scale_log2, inv_sqrt_d;
   const float2* rope;              // dq and dk turn back by their row's angles (null: not)
   int parts;                       // dK / dV: CTAs of a cluster that share a key tile's items (1, 2 or 4)
+  int sum_parts;                   // delta's parts: of (b, h, query), part j lies at dsum + j sum_part + h sum_head + b sum_batch + query
+  long long sum_part, sum_head, sum_batch;
   int apart;                       // dQ: its memory may hold what the dK / dV kernel reads, so it waits for that one
 };
+
+// delta of a query, its parts asked for together (8 at most: heads of 128 in units of 16 columns)
+__device__ __forceinline__ float delta_of(const TcBwdParams& p, int b, int h, int q) {
+  const float* at = p.dsum + (long long)h * p.sum_head + (long long)b * p.sum_batch + q;
+  float s = at[0];
+  if (p.sum_parts > 1) {
+    float v[7];
+#pragma unroll
+    for (int j = 0; j < 7; ++j) v[j] = j + 1 < p.sum_parts ? at[(j + 1) * p.sum_part] : 0.f;
+    s = ((s + v[0]) + (v[1] + v[2])) + ((v[3] + v[4]) + (v[5] + v[6]));      // a binary tree, as within the parts
+  }
+  return s;
+}
 
 // A gradient's row towards a head before the rotary embedding: this thread's HD / 4 pairs (elements i and i + HD / 2, from
 // i = HD / 4 * half on), turned back from FP32 accumulators in tensor memory (`t`: the head's first column) by the row's `angles`.
@@ -675,7 +690,7 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const uint32_t t_lane = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
     const long long ro = ((long long)b * p.H + h) * p.S;
     const float lse = qi < p.S ? p.lse[ro + qi] : 0.f;
-    const float nd = qi < p.S ? -p.dsum[ro + qi] * p.inv_sqrt_d : 0.f;
+    const float nd = qi < p.S ? -delta_of(p, b, h, qi) * p.inv_sqrt_d : 0.f;
     bool ok = true;
     for (int j = 0; j < n_kt; ++j) {
       const int k0 = j * KT;
@@ -1016,7 +1031,7 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const long long ro = ((long long)b * p.H + head_of(i)) * p.S;
       const int q = q0_of(i) + (row & (KT - 1));
       if (q >= p.S) return 0.f;
-      return row < KT ? p.lse[ro + q] : -p.dsum[ro + q] * p.inv_sqrt_d;
+      return row < KT ? p.lse[ro + q] : -delta_of(p, b, head_of(i), q) * p.inv_sqrt_d;
     };
     float rv_next = half == 0 && n_it > 0 ? row_value(0) : 0.f;
     for (int i = 0; i < n_it; ++i) {
@@ -1211,11 +1226,14 @@ int faar_launch_attention_fwd_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, in
 
 int faar_launch_attention_bwd_tc(faar_ctx* ctx, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                                  const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
-                                 const float* dsum, void* dq, void* dk, void* dv, float scale_log2, const float2* rope) {
+                                 const float* dsum, int sum_parts, void* dq, void* dk, void* dv, float scale_log2, const float2* rope) {
   if ((long long)B * S > 0x7FFFFFFFll) return (int)cudaErrorInvalidValue;
   TcBwdParams p = {};
   p.rope = rope;
   p.lse = lse; p.dsum = dsum;
+  // attn_dsum_kernel: [B, H, S]; the product that wrote dO: [parts, H, B S]
+  p.sum_parts = sum_parts ? sum_parts : 1;
+  p.sum_head = sum_parts ? (long long)B * S : S; p.sum_batch = sum_parts ? S : (long long)H * S; p.sum_part = (long long)B * S * H;
   p.dq = reinterpret_cast<__nv_bfloat16*>(dq); p.dk = reinterpret_cast<__nv_bfloat16*>(dk); p.dv = reinterpret_cast<__nv_bfloat16*>(dv);
   p.ldq = ldq; p.ldk = ldk; p.B = B; p.S = S; p.H = H; p.Hkv = Hkv; p.scale_log2 = scale_log2;
   p.inv_sqrt_d = scale_log2 / 1.4426950408889634f;

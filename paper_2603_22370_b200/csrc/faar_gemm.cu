@@ -79,7 +79,8 @@ constexpr int PLAIN_TILES = 0, WIDE_TILES = 1, SPLIT_TILES = 2, SHORT_TILES = 3,
 constexpr int SHORT_BLOCKS = 40;
 constexpr int SHORT_SMEM = 387 * 512;          // with the system's 1 KB below the 196 KB carve-out
 constexpr int SHORT_CARVEOUT = 85;             // percent of the 228 KB: 193.8, which is rounded up to the size on offer, 196 KB
-constexpr int GATED_FWD = 8, GATED_BWD = 10, ROPE = 16, STATS = 32;   // MN (see the kernel) of the gated product's launches, of q / k / v's, of logits'
+constexpr int GATED_FWD = 8, GATED_BWD = 10, ROPE = 16, STATS = 32, SUMS = 66;   // MN (see the kernel) of the gated product's launches, of q / k / v's, of
+// logits', of the attention output's gradient
 constexpr int GATE_COLS = 32, GATE_PANEL = 32 * GATE_COLS * 2;        // backward: a warp's 32 rows x 32 columns in BF16
 template <int MODE, int SHAPE = PLAIN_TILES, int MN = 0> struct Cfg {
   static constexpr bool WIDE = SHAPE == WIDE_TILES, SHORT = SHAPE == SHORT_TILES, SPLIT = SHAPE == SPLIT_TILES || SHAPE == SPLIT_NARROW;
@@ -687,6 +688,42 @@ __device__ __forceinline__ void stats_update(const KParams& p, const uint32_t (&
   if (mx > m) { s *= ex2_approx(m - mx); m = mx; }      // 2^-inf = 0 on the first chunk
 #pragma unroll
   for (int j = 0; j < 16; ++j) s += ex2_approx(fmaf(y[j], p.mse2c, -m));
+}
+
+// Attention output's gradient dO = dY W (B untransposed): delta = sum of dO * O over a head's columns, which the attention's backward
+// pass starts from, leaves with it instead of taking a launch of its own in the chain.  A lane's row of O (p.Yref, rows like Yout's)
+// is asked for 32 columns ahead, the first of a tile before the wait for the accumulator.  Whatever widths the launch
+// takes, a warp's columns are whole units of ld_dyt (16 .. head_dim, see launch_variant); every unit's sum is stored for itself,
+// p.partials: [head_dim / unit][heads][M], and the attention kernels add them up.  Sums of 16 columns meet in a binary tree, here as
+// there: the result does not depend on the widths.  The launch that it replaces -> this, alignment
+// step, us: two blocks of 64-element heads on 192 tokens 195 -> 190, four on 1200 371.7 -> 366.0, two of 128-element heads on 400 264.6 ->
+// 260.2; long sequences, whose launches are large, 0.3 % at most.
+__device__ __forceinline__ void load_sum_row(const KParams& p, int row, int col, int end, uint4 (&v)[4]) {
+  if (row >= p.M) return;
+  const uint4* at = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.Yref) + (long long)row * p.ldy + col);
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (col + 8 * q < end) v[q] = at[q];
+}
+__device__ __forceinline__ void sum_update(const KParams& p, int row, int col, const uint32_t (&acc)[16], const uint4& v0, const uint4& v1,
+                                           float (&pending)[3]) {
+  float sum = 0.f;
+  const uint32_t ow[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {                          // dO as it is stored
+    const uint32_t w = pack_bf16x2(__uint_as_float(acc[2 * j]), __uint_as_float(acc[2 * j + 1]));
+    sum = fmaf(__uint_as_float(ow[j] << 16), __uint_as_float(w << 16), sum);
+    sum = fmaf(__uint_as_float(ow[j] & 0xFFFF0000u), __uint_as_float(w & 0xFFFF0000u), sum);
+  }
+  const int unit = (int)p.ld_dyt, dim = p.yref_dtype;    // powers of two
+#pragma unroll
+  for (int level = 0; level < 3; ++level) {
+    if (16 << level >= unit) break;
+    if (!(col >> (4 + level) & 1)) { pending[level] = sum; return; }
+    sum = pending[level] + sum;
+  }
+  const int head = col >> (31 - __clz(dim)), part = (col & (dim - 1)) >> (31 - __clz(unit));
+  if (row < p.M) p.partials[((long long)part * (p.N >> (31 - __clz(dim))) + head) * p.M + row] = sum;
 }
 
 // FWD: residual, sum of squares, dY^T.
@@ -1309,6 +1346,9 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
       float2 angles[MN == ROPE ? 16 : 1];
       if constexpr (MN == ROPE) load_angles(p, o, 16 * cg, angles);
+      uint4 sum_row[MN == SUMS ? 4 : 1];
+      const int sum_end = min(n0 + col_end, p.N);
+      if constexpr (MN == SUMS) load_sum_row(p, o, n0 + col_begin, sum_end, sum_row);
       bool ok = mbar_wait(tfull_bar(acc), acc_phase, ac, 0x400u | acc);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -1432,6 +1472,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           // REF: two chunks' accumulators in flight (a warp's column count is a multiple of 16: the second may be absent)
           constexpr int STEP = MODE == FAAR_GEMM_REF ? 32 : 16;
           float sm = -INFINITY, ssum = 0.f;              // STATS
+          float pending[3];                              // SUMS
           const bool apart = COLUMNS && BN > 128 && k_blocks >= APART_BLOCKS && tile + n_pairs < total_tiles;
 #pragma unroll 1
           for (int c = col_begin; c < col_end; c += STEP) {
@@ -1456,6 +1497,11 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if constexpr (MN == STATS) {
                   stats_update(p, r, sm, ssum);
                   if (second) stats_update(p, r2, sm, ssum);
+                }
+                if constexpr (MN == SUMS) {
+                  sum_update(p, o, n0 + c, r, sum_row[0], sum_row[1], pending);
+                  if (second) sum_update(p, o, n0 + c + 16, r2, sum_row[2], sum_row[3], pending);
+                  load_sum_row(p, o, n0 + c + 32, sum_end, sum_row);
                 }
               }
             } else {
@@ -1765,6 +1811,21 @@ int launch_variant(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_p
     kp.fin_unit = ldexp(1.0, 62 - 2 * FIN_COUNT_BITS - int_bits); kp.fin_inv_unit = 1.0 / kp.fin_unit;
   }
   kp.n_full = WIDE ? 0 : (SPLIT || !halves ? m_tiles * kp.n_main : pick_full(ctx, MODE, m_tiles, kp.n_main, kp.narrow, bn, max_pairs));
+  if constexpr (MN == SUMS) {
+    // the widest unit of which a warp's columns are a multiple, whatever tile (or share of a split one) it has
+    int unit = a->sum_dim;
+    auto fit = [&](int w) {
+      const int per_warp = (w / C::COL_GROUPS + 15) / 16 * 16;
+      while (w % unit || per_warp % unit) unit /= 2;
+    };
+    if (SPLIT) unit = 16;
+    else {
+      fit(bn);
+      if (kp.narrow || kp.n_full < m_tiles * kp.n_main) fit(bn / 2);
+    }
+    kp.Yref = a->sum_with; kp.yref_dtype = a->sum_dim; kp.ld_dyt = unit; kp.partials = a->sums;
+    *a->sum_parts = a->sum_dim / unit;
+  }
   CUtensorMap tmA, tmB, tmBh;
   e = a->a_mn ? make_map_mn(ctx, &tmA, a->A, a->Kc, a->M, a->lda) : make_map(ctx, &tmA, a->A, a->M, a->Kc, a->lda, BM);
   if (e) return e;
@@ -1871,6 +1932,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
       return launch_tiles<MODE, OPT, 4>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
     }
     if (kp.columns && mn == 1) return launch_tiles<MODE, OPT, 5>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
+    if (mn == 2 && a->sums) return launch_tiles<MODE, OPT, SUMS>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
     if (mn == 2) return launch_tiles<MODE, OPT, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
   } else if constexpr (MODE == FAAR_GEMM_BWD) {
     if (mn == 2) return launch_tiles<MODE, OPT, 2>(ctx, a, kp, n_partials_out, bn, max_pairs, cfg);
@@ -1890,7 +1952,7 @@ int launch(faar_ctx* ctx, const faar_gemm_args* a, KParams& kp, int* n_partials_
 // would be padding that is staged all the same.  M on the accumulator's rows -> N, us: 1 row of 8192 over 2048 15.1 -> 10.6,
 // 64 rows 12.8 -> 12.0, 128 rows 13.1 -> 12.2, 160 rows 13.1 -> 13.8; input gradient of 8 rows of 8192 over 2048 14.5 -> 11.9.
 static bool result_columns(const faar_gemm_args* a) {
-  if (a->yref_t || a->gated || a->rope || a->stats) return false;
+  if (a->yref_t || a->gated || a->rope || a->stats || a->sums) return false;
   const long long row = a->ldy * (a->yout_dtype == FAAR_BF16 ? 2 : 4);
   return a->M <= BM || row % 16 != 0 || (reinterpret_cast<uintptr_t>(a->Yout) & 15) != 0;
 }
@@ -1934,6 +1996,10 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
   if (a->rope && (a->mode != FAAR_GEMM_REF || !a->whole || a->a_mn || a->b_mn || a->gated || (a->head_dim != 64 && a->head_dim != 128) ||
                       a->N % a->head_dim || (reinterpret_cast<uintptr_t>(a->rope) & 7) || a->rope_cols % a->head_dim || a->ldy % 16 || (reinterpret_cast<uintptr_t>(a->Yout) & 31) ||
                       a->yout_dtype != FAAR_BF16))
+    return (int)cudaErrorInvalidValue;
+  if (a->sums && (a->mode != FAAR_GEMM_REF || a->a_mn || !a->b_mn || a->gated || a->rope || a->stats || a->yref_t || (a->sum_dim != 64 && a->sum_dim != 128) ||
+                  a->N % a->sum_dim || a->ldy % 8 || ((reinterpret_cast<uintptr_t>(a->Yout) | reinterpret_cast<uintptr_t>(a->sum_with)) & 15) ||
+                  !a->sum_with || !a->sum_parts || a->yout_dtype != FAAR_BF16))
     return (int)cudaErrorInvalidValue;
   kp.M = a->M; kp.N = a->N; kp.Kc = a->Kc; kp.bn = BN_MAX; kp.n_main = kp.narrow = kp.n_full = 0; kp.status = a->status;
   {

@@ -146,7 +146,7 @@ int faar_launch_attention_fwd_tc(faar_ctx*, int B, int S, int H, int Hkv, int D,
 // rope: dq and dk turn back by their row's angles, [D / 2, B S] sines and cosines, on the way out (null: they don't)
 int faar_launch_attention_bwd_tc(faar_ctx*, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                                  const void* v, int64_t ldk, const void* dout, int64_t ldo, const float* lse,
-                                 const float* dsum, void* dq, void* dk, void* dv, float scale_log2, const float2* rope);
+                                 const float* dsum, int sum_parts, void* dq, void* dk, void* dv, float scale_log2, const float2* rope);
 int faar_attention_tc_status(uint32_t* code_out);
 int faar_launch_softquant_eval(faar_ctx*, const faar_shape*, const float* V, const uint8_t* code,
                                const uint8_t* scales, const float* s_global, float beta,
@@ -190,7 +190,7 @@ int faar_launch_attention_fwd(faar_ctx*, int B, int S, int H, int Hkv, int D, co
                               const void* v, int64_t ldk, void* out, int64_t ldo, float* lse);
 int faar_launch_attention_bwd(faar_ctx*, int B, int S, int H, int Hkv, int D, const void* q, int64_t ldq, const void* k,
                               const void* v, int64_t ldk, const void* out, const void* dout, int64_t ldo, const float* lse,
-                              float* dsum, void* dq, void* dk, void* dv, const float2* rope = nullptr);
+                              float* dsum, void* dq, void* dk, void* dv, const float2* rope = nullptr, int sum_parts = 0);
 int faar_launch_nvfp4_gemm(faar_ctx*, int M, int N, int K, const uint8_t* A, const uint8_t* sfa, const float* sa,
                            const uint8_t* B, const uint8_t* sfb, const float* sb, void* C, int64_t ldc, uint32_t* status);
 int faar_launch_round_partials(faar_ctx*, const float* V, int64_t N, float* partials, int* n_partials);
@@ -229,6 +229,8 @@ struct faar_gemm_args {
   int gated;                                   // REF: an epilogue of the gated product, FAAR_GATED_FWD or FAAR_GATED_BWD (0: plain)
   void* act; const void* gate_up;              // and its further tensors (see faar_gemm.cu)
   float2* stats; float stats_c;                // REF: softmax statistics of every row, [M, ceil(N / 128)] (null: not wanted)
+  const void* sum_with; float* sums;           // REF: sums of the result times sum_with [M, ldy] over the sum_dim columns of each head, as
+  int sum_dim; int* sum_parts;                 // sum_parts parts (set by the launch) [parts, heads, M] (sums null: not wanted)
   const float2* rope;                          // REF: the first rope_cols columns of the result are heads that turn by their row's
   int rope_cols, head_dim;                     // angles, [head_dim / 2, M] sines and cosines (null: none do)
   __nv_bfloat16* dYt; int64_t ld_dyt;          // FWD: [M(O), ld_dyt]

@@ -1,7 +1,7 @@
 // Forward and backward passes of a whole decoder model (full-model alignment, Procedure steps 16-17 and 21-23): the
 // sequence of kernel launches for every block, enqueued by one call.  No arithmetic here and no kernels of its own.
 //
-// Why native: a step is a chain of 28 launches per block (7 in each forward pass, 13 in the backward pass, soft weights), many
+// Why native: a step is a chain of 27 launches per block (7 in each forward pass, 12 in the backward pass, soft weights), many
 // of a few microseconds each.  Issued one by one from Python a launch cost 7.5 us of host time, more than the kernels of a small
 // model take: an alignment step of two 128-wide blocks on 192 tokens took 770 us for 500 us of device time (177 us as it is
 // now).  Activations live in one caller-owned arena per pass at offsets that depend on the sizes alone.
@@ -59,7 +59,7 @@ struct Scratch {
     size_t o = 0;
     auto take = [&](size_t n) { const size_t at = o; o += align256(n); return at; };
     dhz = take(s.T * s.d * 2); dx = take(s.T * s.d * 2); dgu = take(s.T * 2 * s.f * 2);
-    dn = take(s.T * s.d * 2); da = take(s.T * s.qd * 2); dqkv = take(s.T * s.qkv * 2); dsum = take(s.seq_rows * 4);
+    dn = take(s.T * s.d * 2); da = take(s.T * s.qd * 2); dqkv = take(s.T * s.qkv * 2); dsum = take(s.seq_rows * 4 * (s.hd / 16));
     total = o;
   }
 };
@@ -114,6 +114,22 @@ int product_gated_bwd(faar_ctx* ctx, size_t T, int f, int K, const void* dY, con
   a.status = reinterpret_cast<uint32_t*>(ws);
   a.Yout = dgu; a.yout_dtype = FAAR_BF16; a.ldy = 2 * f;
   a.gated = FAAR_GATED_BWD; a.gate_up = gu;
+  return faar_launch_gemm(ctx, &a, nullptr);
+}
+
+// dA = dY W_o, the gradient of the attention output a, and the row sums of dA * a by head (*parts of them).  Up to 128 rows such a
+// product is better the other way round (see faar_launch_gemm), without them: *parts = 0.
+int product_sums(faar_ctx* ctx, const Sizes& s, const void* dY, const void* W, const void* a_out, void* dA, float* sums, int* parts, void* ws) {
+  *parts = 0;
+  if (s.T <= 128) return product(ctx, s.T, s.qd, s.d, dY, s.d, W, s.qd, true, dA, s.qd, ws);
+  faar_gemm_args a = {};
+  a.mode = FAAR_GEMM_REF;
+  a.M = (int)s.T; a.N = s.qd; a.Kc = s.d;
+  a.A = dY; a.lda = s.d;
+  a.B = W; a.ldb = s.qd; a.b_mn = 1;
+  a.status = reinterpret_cast<uint32_t*>(ws);
+  a.Yout = dA; a.yout_dtype = FAAR_BF16; a.ldy = s.qd;
+  a.sum_with = a_out; a.sums = sums; a.sum_dim = s.hd; a.sum_parts = parts;
   return faar_launch_gemm(ctx, &a, nullptr);
 }
 
@@ -345,16 +361,20 @@ int backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* 
       e = faar_launch_rmsnorm_bwd(ctx, T, s.d, scratch + S.dn, nullptr, nullptr, s.d, p + A.b.x_mid, s.d, b.mlp_norm,
                                   reinterpret_cast<const float*>(p + A.b.rstd2), dx, s.d, dx, s.d);
     // attention branch: x_mid = x_in + a W_o^T
-    if (!e) e = product(ctx, s.T, s.qd, s.d, dx, s.d, b.o.Wsoft, s.qd, true, scratch + S.da, s.qd, ws);
     const __nv_bfloat16* const qkv = reinterpret_cast<const __nv_bfloat16*>(p + A.b.qkv);
     __nv_bfloat16* const dqkv = reinterpret_cast<__nv_bfloat16*>(scratch + S.dqkv);
     // the tcgen05 kernels turn dq and dk back on the way out; the others leave that to a pass over both, which lie side by side
+    // and take the row sums of dO * O from the product that forms dO
     const bool turned = ctx->tune_attention_fragments == 0;
+    float* const dsum = reinterpret_cast<float*>(scratch + S.dsum);
+    int parts = 0;
+    if (!e && turned) e = product_sums(ctx, s, dx, b.o.Wsoft, p + A.b.a, scratch + S.da, dsum, &parts, ws);
+    if (!e && !turned) e = product(ctx, s.T, s.qd, s.d, dx, s.d, b.o.Wsoft, s.qd, true, scratch + S.da, s.qd, ws);
     if (!e)
       e = faar_launch_attention_bwd(ctx, batch, seq, m->n_heads, m->n_kv_heads, m->head_dim, qkv, s.qkv, qkv + s.qd, qkv + s.qd + s.kvd,
                                     s.qkv, p + A.b.a, scratch + S.da, s.qd, reinterpret_cast<const float*>(p + A.b.lse),
-                                    reinterpret_cast<float*>(scratch + S.dsum), dqkv, dqkv + s.qd, dqkv + s.qd + s.kvd,
-                                    turned ? reinterpret_cast<const float2*>(arena + A.rope) : nullptr);
+                                    dsum, dqkv, dqkv + s.qd, dqkv + s.qd + s.kvd, turned ? reinterpret_cast<const float2*>(arena + A.rope) : nullptr,
+                                    parts);
     if (!e && turned) e = group_update(ctx, b.o, s.T, s.qd, dx, p + A.b.a, hp, ws);          // next to dQ (and so to dK / dV)
     if (!e && !turned) e = group_update(ctx, b.o, s.T, s.qd, dx, p + A.b.a, hp, ws, false);
     if (!e && !turned) e = faar_launch_rope(ctx, T, m->n_heads + m->n_kv_heads, m->head_dim, dqkv, s.qkv, pos, m->theta, 1, dqkv, s.qkv);

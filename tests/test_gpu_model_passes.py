@@ -174,3 +174,34 @@ def test_a_models_passes_are_those_of_its_single_calls(ctx, batch, seq, hidden, 
     # much again wherever one of the gradients formed from them (of the norm, gate / up, the attention output) rounds differently
     assert worst <= 4 * 2.0**-9, worst
     assert max(rel(got[1, n], want[1, n]) for n in ("o_proj", "gate_proj", "up_proj", "down_proj")) <= 1e-5      # (before any attention gradient)
+
+
+@pytest.mark.parametrize("batch,seq,hidden,heads,kv_heads,head_dim,width", [
+    (2, 65, 128, 2, 1, 64, 0),            # 16 columns a warp: four parts
+    (1, 257, 128, 5, 1, 64, 224),         # tiles that are no whole heads, the last column of half of one
+    (1, 128, 192, 3, 1, 64, 0),           # 128 rows: the sums' own launch
+    (3, 100, 1024, 3, 3, 128, 0),         # split contraction: eight parts
+    (2, 700, 2048, 16, 4, 128, 0),
+    (1, 1300, 256, 4, 2, 128, 256),       # whole heads
+])
+def test_row_sums_of_the_attention_gradient(ctx, batch, seq, hidden, heads, kv_heads, head_dim, width):
+    """The sums of dO * O by head leave with the product that forms dO (over 128 rows): in one part a head, in several, of a split contraction."""
+    m, tokens, gen = make_model(ctx, batch, seq, vocab=64, hidden=hidden, n_layers=1, n_heads=heads, n_kv_heads=kv_heads, head_dim=head_dim, ffn=64)
+    faar.tune_tile_n(ctx, width)
+    try:
+        Z, H, arena = m.forward(tokens, quantised=True, beta=6.0, keep=True)
+        dZ, dH = (torch.randn(t.shape, device=t.device, generator=gen).to(torch.bfloat16) for t in (Z, H))
+        V0 = {n: m.lin[0][n].V.clone() for n in stage2.LINEARS}
+        hp = faar.make_hparams(beta=6.0, opt=1, lr=5e-4, step=1)
+        got = m.backward(dZ, dH, arena, hp, want_dv=True)
+        faar.check_status(ctx, m.ws)
+        for n, v in V0.items():
+            m.lin[0][n].V.copy_(v)
+            m.lin[0][n].m.zero_()
+            m.lin[0][n].u.zero_()
+        _, _, kept = forward(m, tokens, True)
+        want = backward(m, dZ, dH, kept, hp)
+    finally:
+        faar.tune_tile_n(ctx, 0)
+    # the bound of the passes' own test, for the gradients that went through the attention's backward pass
+    assert max(rel(got[0, n], want[0, n]) for n in ("q_proj", "k_proj", "v_proj")) <= 4 * 2.0**-9
