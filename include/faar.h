@@ -384,6 +384,12 @@ FAAR_API int faar_layer_step(faar_ctx* ctx, const faar_shape* shape, const faar_
                     const uint8_t* scales, const float* s_global, float* adam_m, float* adam_u,
                     float* loss_out2, void* workspace, size_t workspace_bytes);
 
+/* faar_layer_step without X^T: the dW product reads X [T, ldx] with the token index as its contraction row, which gives
+ * the same bits.  For batches that a few steps use; shape->ldxt is not looked at. */
+FAAR_API int faar_layer_step_rowmajor(faar_ctx* ctx, const faar_shape* shape, const faar_hparams* hp, const void* X,
+                    const void* Y_ref, float* V, const uint8_t* code, const uint8_t* scales, const float* s_global,
+                    float* adam_m, float* adam_u, float* loss_out2, void* workspace, size_t workspace_bytes);
+
 /* faar_layer_step for a calibration batch that lives in HOST memory (ideally
  * pinned): copies X_host[T,K] (ldx) and Y_ref_host (the layout the shape declares)
  * into the caller's device staging buffers X_dev / Yref_dev, rebuilds

@@ -744,9 +744,9 @@ int faar_layer_bwd_rowmajor(faar_ctx* ctx, const faar_shape* s, const faar_hpara
   return cuda_fail(ctx, bwd_impl(ctx, s, hp, dY, X, V, code, scales, s_global, adam_m, adam_u, dV, ws, l, nullptr, 0, 1));
 }
 
-int faar_layer_step(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const void* X, const void* Xt,
-                    const void* Y_ref, float* V, const uint8_t* code, const uint8_t* scales, const float* s_global,
-                    float* adam_m, float* adam_u, float* loss_out2, void* workspace, size_t workspace_bytes) {
+static int layer_step(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const void* X, const void* Xt, const void* Y_ref, float* V,
+                      const uint8_t* code, const uint8_t* scales, const float* s_global, float* adam_m, float* adam_u, float* loss_out2,
+                      void* workspace, size_t workspace_bytes, bool row_major) {
   int st = validate_step(ctx, s, hp, X, Xt, Y_ref, V, code, scales, s_global, adam_m, adam_u, loss_out2, workspace,
                          workspace_bytes);
   if (st) return st;
@@ -757,8 +757,21 @@ int faar_layer_step(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, 
   int np_mse = 0;
   int e = fwd_impl(ctx, s, hp, X, Y_ref, V, code, scales, s_global, dYt, nullptr, ws, l, &np_mse);
   if (e) return cuda_fail(ctx, e);
-  e = bwd_impl(ctx, s, hp, dYt, Xt, V, code, scales, s_global, adam_m, adam_u, nullptr, ws, l, loss_out2, np_mse);
+  e = bwd_impl(ctx, s, hp, dYt, Xt, V, code, scales, s_global, adam_m, adam_u, nullptr, ws, l, loss_out2, np_mse, row_major ? 2 : 0);
   return cuda_fail(ctx, e);
+}
+int faar_layer_step(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const void* X, const void* Xt,
+                    const void* Y_ref, float* V, const uint8_t* code, const uint8_t* scales, const float* s_global,
+                    float* adam_m, float* adam_u, float* loss_out2, void* workspace, size_t workspace_bytes) {
+  return layer_step(ctx, s, hp, X, Xt, Y_ref, V, code, scales, s_global, adam_m, adam_u, loss_out2, workspace, workspace_bytes, false);
+}
+int faar_layer_step_rowmajor(faar_ctx* ctx, const faar_shape* s, const faar_hparams* hp, const void* X, const void* Y_ref, float* V,
+                             const uint8_t* code, const uint8_t* scales, const float* s_global, float* adam_m, float* adam_u,
+                             float* loss_out2, void* workspace, size_t workspace_bytes) {
+  if (!s) return FAAR_ERR_INVALID_ARG;
+  faar_shape shape = *s;
+  shape.ldxt = ((int64_t)s->T + 7) / 8 * 8;                // X^T is not looked at
+  return layer_step(ctx, &shape, hp, X, X, Y_ref, V, code, scales, s_global, adam_m, adam_u, loss_out2, workspace, workspace_bytes, true);
 }
 
 int faar_nvfp4_expand(faar_ctx* ctx, int rows, int K, const void* packed, const void* scales, void* out, int64_t ld) {

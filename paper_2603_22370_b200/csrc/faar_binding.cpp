@@ -90,7 +90,7 @@ template <class T> struct Arg<T, std::enable_if_t<std::is_pointer_v<T>>> {
   X(faar_workspace_init) X(faar_softquant_init) X(faar_softquant_eval) X(faar_softquant_operand_f32)                      \
   X(faar_transpose_bf16) X(faar_act_fakequant) X(faar_layer_ref) X(faar_layer_fwd) X(faar_layer_dx)                       \
   X(faar_layer_dx_operand) X(faar_silu_mul) X(faar_round_loss) X(faar_round_loss_static) X(faar_layer_bwd)                \
-  X(faar_layer_bwd_rowmajor) X(faar_layer_step) X(faar_layer_step_host) X(faar_nvfp4_expand)                              \
+  X(faar_layer_bwd_rowmajor) X(faar_layer_step) X(faar_layer_step_rowmajor) X(faar_layer_step_host) X(faar_nvfp4_expand)                              \
   X(faar_layer_step_host_nvfp4) X(faar_harden_pack) X(faar_align_loss) X(faar_swizzle_scales) X(faar_rmsnorm)             \
   X(faar_rmsnorm_bwd) X(faar_add_rmsnorm) X(faar_rmsnorm_bwd_sum) X(faar_rope) X(faar_silu_mul_bwd) X(faar_embedding)     \
   X(faar_add) X(faar_attention_fwd) X(faar_attention_bwd) X(faar_nvfp4_gemm) X(faar_model_forward) X(faar_model_forward_both) X(faar_model_backward) \

@@ -53,6 +53,7 @@ SIGNATURES = {
     "faar_layer_bwd": (_I, [_P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _Z]),
     "faar_layer_bwd_rowmajor": (_I, [_P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _Z]),
     "faar_layer_step": (_I, [_P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _Z]),
+    "faar_layer_step_rowmajor": (_I, [_P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _Z]),
     "faar_layer_step_host": (_I, [_P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _Z]),
     "faar_nvfp4_expand": (_I, [_P, _I, _I, _P, _P, _P, _L]),
     "faar_layer_step_host_nvfp4": (_I, [_P] * 19 + [_Z]),
@@ -496,6 +497,11 @@ def layer_bwd_rowmajor(ctx, shape, hp, dY, X, V, code, scales, s_global, adam_m,
 def layer_step(ctx, shape, hp, X, Xt, Y_ref, V, code, scales, s_global, adam_m, adam_u, loss_out2, ws):
     _check(_fast().faar_layer_step(ctx._n, shape, hp, X, Xt, Y_ref, V, code, scales, s_global, adam_m, adam_u,
            loss_out2, ws, ws.numel()), "faar_layer_step")
+
+
+def layer_step_rowmajor(ctx, shape, hp, X, Y_ref, V, code, scales, s_global, adam_m, adam_u, loss_out2, ws):
+    _check(_fast().faar_layer_step_rowmajor(ctx._n, shape, hp, X, Y_ref, V, code, scales, s_global, adam_m, adam_u,
+           loss_out2, ws, ws.numel()), "faar_layer_step_rowmajor")
 
 
 def harden_pack(ctx, shape, V, code, scales, s_global, packed, scales_out, decisions, W_final, wfinal_dtype=F32):
