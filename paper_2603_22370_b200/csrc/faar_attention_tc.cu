@@ -146,6 +146,8 @@ __device__ __forceinline__ void ld32x2(uint32_t ta, uint32_t tb, float (&a)[32],
 #pragma unroll
   for (int i = 0; i < 32; ++i) { a[i] = __uint_as_float(u[i]); b[i] = __uint_as_float(v[i]); }
 }
+// Loads and stores of tensor memory are instructions of the whole warp.  Rows beyond the end of a sequence store nothing, so where
+// another load follows such stores a __syncwarp brings the lanes together: nothing else does.
 __device__ __forceinline__ void ld16(uint32_t ta, float (&a)[16]) {
   uint32_t u[16];
   asm volatile(
@@ -448,6 +450,7 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             dst[4 * half + c] = make_uint4(pack2(t[8 * c] * inv, t[8 * c + 1] * inv), pack2(t[8 * c + 2] * inv, t[8 * c + 3] * inv),
                                            pack2(t[8 * c + 4] * inv, t[8 * c + 5] * inv), pack2(t[8 * c + 6] * inv, t[8 * c + 7] * inv));
         }
+        __syncwarp();
       }
       if (qi < p.S) p.lse[((long long)b * p.H + h) * p.S + qi] = m + log2f(l);
     }
@@ -530,15 +533,17 @@ __device__ __forceinline__ void turn_back(const float2* angles, long long tokens
     ld16x2(t + (uint32_t)c, t + (uint32_t)(c + HD / 2), a, b);
 #pragma unroll
     for (int j = 0; j < 16; ++j) faar_rope_turn(a[j], b[j], -v.sc[j].x, v.sc[j].y);
-    if (c + 16 < HD / 4 * (half + 1) && valid) load_angles(angles, tokens, c + 16, v);
-    if (!valid) continue;
+    if (valid) {
+      if (c + 16 < HD / 4 * (half + 1)) load_angles(angles, tokens, c + 16, v);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      reinterpret_cast<uint4*>(row + c)[h] = make_uint4(pack2(a[8 * h], a[8 * h + 1]), pack2(a[8 * h + 2], a[8 * h + 3]),
-                                                        pack2(a[8 * h + 4], a[8 * h + 5]), pack2(a[8 * h + 6], a[8 * h + 7]));
-      reinterpret_cast<uint4*>(row + HD / 2 + c)[h] = make_uint4(pack2(b[8 * h], b[8 * h + 1]), pack2(b[8 * h + 2], b[8 * h + 3]),
-                                                                 pack2(b[8 * h + 4], b[8 * h + 5]), pack2(b[8 * h + 6], b[8 * h + 7]));
+      for (int h = 0; h < 2; ++h) {
+        reinterpret_cast<uint4*>(row + c)[h] = make_uint4(pack2(a[8 * h], a[8 * h + 1]), pack2(a[8 * h + 2], a[8 * h + 3]),
+                                                          pack2(a[8 * h + 4], a[8 * h + 5]), pack2(a[8 * h + 6], a[8 * h + 7]));
+        reinterpret_cast<uint4*>(row + HD / 2 + c)[h] = make_uint4(pack2(b[8 * h], b[8 * h + 1]), pack2(b[8 * h + 2], b[8 * h + 3]),
+                                                                   pack2(b[8 * h + 4], b[8 * h + 5]), pack2(b[8 * h + 6], b[8 * h + 7]));
+      }
     }
+    __syncwarp();                                           // the next load wants the whole warp (see ld16)
   }
 }
 
@@ -757,6 +762,7 @@ attn_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             dst[c0 / 8 + c] = make_uint4(pack2(t[8 * c], t[8 * c + 1]), pack2(t[8 * c + 2], t[8 * c + 3]),
                                          pack2(t[8 * c + 4], t[8 * c + 5]), pack2(t[8 * c + 6], t[8 * c + 7]));
         }
+        __syncwarp();
       }
     }
   }
@@ -853,21 +859,23 @@ __device__ __noinline__ void finish_parts(uint32_t base, uint32_t t_acc, int row
       }
     }
     const int c = column(rank, pair, 0) - (is_k ? HD : 0);
-    if (!valid) continue;
-    if (is_k && angles) {
-      Angles a;
-      load_angles(angles, tokens, c, a);
+    if (valid) {
+      if (is_k && angles) {
+        Angles a;
+        load_angles(angles, tokens, c, a);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) faar_rope_turn(v[0][j], v[1][j], -a.sc[j].x, a.sc[j].y);
+        for (int j = 0; j < 16; ++j) faar_rope_turn(v[0][j], v[1][j], -a.sc[j].x, a.sc[j].y);
+      }
+#pragma unroll
+      for (int partner = 0; partner < 2; ++partner) {
+        uint4* dst = reinterpret_cast<uint4*>(out + c + partner * (HD / 2));
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          dst[q] = make_uint4(pack2(v[partner][8 * q], v[partner][8 * q + 1]), pack2(v[partner][8 * q + 2], v[partner][8 * q + 3]),
+                              pack2(v[partner][8 * q + 4], v[partner][8 * q + 5]), pack2(v[partner][8 * q + 6], v[partner][8 * q + 7]));
+      }
     }
-#pragma unroll
-    for (int partner = 0; partner < 2; ++partner) {
-      uint4* dst = reinterpret_cast<uint4*>(out + c + partner * (HD / 2));
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-        dst[q] = make_uint4(pack2(v[partner][8 * q], v[partner][8 * q + 1]), pack2(v[partner][8 * q + 2], v[partner][8 * q + 3]),
-                            pack2(v[partner][8 * q + 4], v[partner][8 * q + 5]), pack2(v[partner][8 * q + 6], v[partner][8 * q + 7]));
-    }
+    __syncwarp();                                           // the next load wants the whole warp (see ld16)
   }
 }
 
@@ -1120,6 +1128,7 @@ attn_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
               dst[c0 / 8 + c] = make_uint4(pack2(t[8 * c], t[8 * c + 1]), pack2(t[8 * c + 2], t[8 * c + 3]),
                                            pack2(t[8 * c + 4], t[8 * c + 5]), pack2(t[8 * c + 6], t[8 * c + 7]));
           }
+          __syncwarp();
         }
       }
     }

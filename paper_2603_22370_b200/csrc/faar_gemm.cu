@@ -284,6 +284,8 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t tmem_d, uint64_t desc_a, ui
       "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate) : "memory");
 }
+// An instruction of the whole warp.  Rows beyond the matrix take no part in an epilogue's stores, so a __syncwarp stands between
+// those and the next load.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -667,6 +669,7 @@ __device__ __forceinline__ void epi_rope(const KParams& p, uint32_t trow, int ro
         store_row(p, row, n0 + h + c, lo);
         store_row(p, row, n0 + h + hd / 2 + c, hi);
       }
+      __syncwarp();
     }
   }
 }
@@ -1455,6 +1458,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           tmem_ld16(trow + (uint32_t)(half + c), r2);
           tmem_ld_wait();
           epi_gated_fwd(p, o, f0 + c, r, r2);
+          __syncwarp();
         }
       } else {
         if (MODE == FAAR_GEMM_FWD && yvec) {
@@ -1466,6 +1470,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               tmem_ld16(trow + (uint32_t)c, r);
               tmem_ld_wait();
               warp_acc += epi_fwd_vec(p, o, n0 + c, r, yraw[2 * q], yraw[2 * q + 1]);
+              __syncwarp();
             }
           }
         } else {
@@ -1511,6 +1516,7 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               tmem_ld_wait();
               warp_acc += epi_fwd(p, o, n0 + c, r, yr);
             }
+            __syncwarp();
           }
           if constexpr (MN == STATS) {
             const int slots = (p.N + 127) / 128, slot = (n0 + col_begin) / 128;

@@ -23,6 +23,7 @@ def ctx():
     (1, 449, 1, 1),          # eight: four parts, two of which have nothing of the last key tile's one item
     (2, 130, 4, 1),          # the last key tile holds two keys
     (1, 300, 8, 2),
+    (1, 300, 16, 16),        # heads of 128: two parts, each finishing its columns in two turns, with the last key tile's rows cut inside a warp
 ])
 def test_dealt_key_tiles_match_the_oracle(ctx, B, S, H, HKV, D):
     _attention_case(ctx, B, S, H, HKV, D)
