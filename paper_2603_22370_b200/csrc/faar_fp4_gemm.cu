@@ -65,6 +65,7 @@ struct P4 {
   const float* sa; const float* sb;
   __nv_bfloat16* C; long long ldc;
   uint32_t* status;
+  int one_by_one;                            // the producer's copies (see copies_one_by_one)
 };
 
 __device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -211,25 +212,39 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
+    auto load = [&](int mt, int nt, int ks, int stage) {
+      const uint32_t sa = base + stage * C4::STAGE, sb = sa + C4::A_BYTES, sfa = sb + C4::B_BYTES, sfb = sfa + C4::SFA_BYTES;
+      const uint32_t bar = map_to_leader(full(stage));
+      if (rank == 0) bar_expect(full(stage), 2u * (uint32_t)C4::STAGE);
+      tma_2d(sa, &tmA, ks * ROW_BYTES, mt * 2 * TM + (int)rank * TM, bar);
+      tma_2d(sb, &tmB, ks * ROW_BYTES, nt * BN + (int)rank * (BN / 2), bar);
+      tma_3d(sfa, &tmSA, 0, 4 * ks, 2 * mt + (int)rank, bar);
+      tma_3d(sfb, &tmSB, 0, 4 * ks, nt * C4::N_SFB, bar);
+    };
+    int stage = 0; uint32_t phase = 0; bool ok = true;
+    if (p.one_by_one && lane == 0) {                         // (see copies_one_by_one)
+      for (int t = pair; t < tiles && ok; t += n_pairs) {
+        const int mt = t % m_tiles, nt = t / m_tiles;
+        for (int ks = 0; ks < k_stages; ++ks) {
+          ok = bar_wait(empty(stage), phase ^ 1u, ab, 0x900u | stage);
+          if (!ok) break;
+          load(mt, nt, ks, stage);
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+        }
+      }
+    }
     // the whole warp, converged (see faar_elect_one): four copies a stage under `if (lane == 0)` took about 400 of the 512 clocks
     // that a stage's MMAs take, and a few stages' worth of a short contraction's whole time
-    int stage = 0; uint32_t phase = 0; bool ok = true;
-    for (int t = pair; t < tiles && ok; t += n_pairs) {
-      const int mt = t % m_tiles, nt = t / m_tiles;
-      for (int ks = 0; ks < k_stages; ++ks) {
-        ok = __all_sync(0xffffffffu, bar_wait(empty(stage), phase ^ 1u, ab, 0x900u | stage));
-        if (!ok) break;
-        const uint32_t sa = base + stage * C4::STAGE, sb = sa + C4::A_BYTES, sfa = sb + C4::B_BYTES, sfb = sfa + C4::SFA_BYTES;
-        const uint32_t bar = map_to_leader(full(stage));
-        if (faar_elect_one()) {
-          if (rank == 0) bar_expect(full(stage), 2u * (uint32_t)C4::STAGE);
-          tma_2d(sa, &tmA, ks * ROW_BYTES, mt * 2 * TM + (int)rank * TM, bar);
-          tma_2d(sb, &tmB, ks * ROW_BYTES, nt * BN + (int)rank * (BN / 2), bar);
-          tma_3d(sfa, &tmSA, 0, 4 * ks, 2 * mt + (int)rank, bar);
-          tma_3d(sfb, &tmSB, 0, 4 * ks, nt * C4::N_SFB, bar);
+    if (!p.one_by_one) {
+      for (int t = pair; t < tiles && ok; t += n_pairs) {
+        const int mt = t % m_tiles, nt = t / m_tiles;
+        for (int ks = 0; ks < k_stages; ++ks) {
+          ok = __all_sync(0xffffffffu, bar_wait(empty(stage), phase ^ 1u, ab, 0x900u | stage));
+          if (!ok) break;
+          if (faar_elect_one()) load(mt, nt, ks, stage);
+          __syncwarp();
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        __syncwarp();
-        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
     }
     if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) {} }
@@ -406,8 +421,18 @@ bool pick_wide4(int M, int N, int pairs) {
   return (long long)((M + 2 * TM - 1) / (2 * TM)) * ((N + 255) / 256) >= pairs;
 }
 
+// Where one lane issues the producer's copies one by one, about 0.2 us a stage, instead of an elected lane of the converged warp
+// all at once.  Everywhere else the latter is 3 to 13 % faster; but with fewer than 128 rows of A and less than 128 KB of them in
+// all, and more pairs at work (in the last wave) than one die has, pairs that ask for a whole ring at a time hold one another up.
+// One by one / at once, us: 8 rows, 8192 x 2048 5.8 / 6.3, x 8192 13.1 / 16.0, 16384 x 8192 23.0 / 31.4; 64 rows, 8192 x 2048 5.8 / 6.3,
+// x 4096 (128 KB) 8.1 / 7.5; 127 rows, 8192 x 2048 6.45 / 6.86, 128 rows 6.4 / 6.1; 8 rows, 4736 x 2048 (one die's pairs) 5.7 / 5.4,
+// 11008 x 2048 (86 tiles, 12 in the last wave) 8.2 / 7.7.
+bool copies_one_by_one(int M, int K, long long tiles, int pairs) {
+  return M < TM && (long long)M * K < 2 * 131072 && (tiles - 1) % pairs >= pairs / 2;
+}
+
 template <int BN>
-int launch4(faar_ctx* ctx, const uint8_t* A, const uint8_t* sfa, const uint8_t* B, const uint8_t* sfb, const P4& p) {
+int launch4(faar_ctx* ctx, const uint8_t* A, const uint8_t* sfa, const uint8_t* B, const uint8_t* sfb, P4& p) {
   using C4 = Cfg4<BN>;
   auto kern = nvfp4_gemm_kernel<BN>;
   cudaLaunchConfig_t cfg = {};
@@ -433,6 +458,7 @@ int launch4(faar_ctx* ctx, const uint8_t* A, const uint8_t* sfa, const uint8_t* 
   if (!e) e = scale_map(ctx, &tmSB, sfb, (p.N + 127) / 128, p.k_tiles, C4::N_SFB);
   if (e) return e;
   const long long tiles = (long long)((p.M + 2 * TM - 1) / (2 * TM)) * ((p.N + BN - 1) / BN);
+  p.one_by_one = BN == 128 && copies_one_by_one(p.M, p.K, tiles, ctx->num_sms / 2);
   cfg.gridDim = dim3(2 * (unsigned)(tiles < max_pairs ? tiles : max_pairs), 1, 1);
   faar_prof_scope ps(ctx, FAAR_K_NVFP4_GEMM);
   cudaError_t ce = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmSA, tmSB, p);

@@ -138,6 +138,12 @@ def test_own_nvfp4_gemm_with_wide_tiles(ctx, O, K, T):
     _check_nvfp4_gemm(ctx, O, K, T, seed=O + K, sample=128)
 
 
+@pytest.mark.parametrize("O,K,T", [(4736, 544, 8), (4737, 544, 8), (4864, 2048, 127), (4864, 2048, 128), (4864, 2080, 126), (9473, 288, 1)])
+def test_own_nvfp4_gemm_of_few_rows(ctx, O, K, T):
+    """Both ways to issue the copies on either side of their lines: 37 and 38 tiles, 127 and 128 rows, 128 KB of activations, a second wave."""
+    _check_nvfp4_gemm(ctx, O, K, T, seed=T, sample=min(T, 16))
+
+
 def test_own_nvfp4_gemm_agrees_with_the_layer_path(ctx):
     """X_q W_final^T computed two ways by this library: the FP4 GEMM on the packed operands, and the BF16
     tensor-core GEMM (frozen-target call) on the same values written out in BF16 (activations: units times
