@@ -363,6 +363,7 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               if (col + q < p.N) out[q] = __float2bfloat16_rn(__uint_as_float(r[q]) * alpha);
           }
         }
+        __syncwarp();                                        // the next load of tensor memory wants the whole warp
       }
       fence_before();
       __syncwarp();
