@@ -466,13 +466,15 @@ FAAR_API int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const 
                              void* dZ_q, void* dH_q, float* loss_out2, void* workspace, size_t workspace_bytes);
 
 /* The same loss from softmax statistics that the logits' products left behind (faar_model_forward_stats,
- * faar_model_forward_both_stats, at the same tau): stats_fp, stats_q, of the size that faar_logit_stats_size
- * gives (0: the product is too small for them to pay, and the forward calls refuse to take them), 16-byte aligned.
- * The logits are then read once instead of twice. */
+ * faar_model_forward_both_stats): the logits are then read once instead of twice.  stats_fp, stats_q: stats_bytes each, at least
+ * what faar_logit_stats_size gives (FAAR_ERR_WORKSPACE), 16-byte aligned.  A size of 0 says that the product is too small for
+ * them to pay: the forward calls don't take them and this call refuses, too (FAAR_ERR_SHAPE).  They belong to the logits and
+ * to the tau that they were formed with; with another tau here the loss and its gradient are wrong, which no call can see. */
 FAAR_API int faar_logit_stats_size(faar_ctx* ctx, int T, int vocab, size_t* bytes);
 FAAR_API int faar_align_loss_stats(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
                                    const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, const void* stats_fp,
-                                   const void* stats_q, void* dZ_q, void* dH_q, float* loss_out2, void* workspace, size_t workspace_bytes);
+                                   const void* stats_q, size_t stats_bytes, void* dZ_q, void* dH_q, float* loss_out2, void* workspace,
+                                   size_t workspace_bytes);
 
 /* ---- deployable scale-factor layout ---------------------------------------
  * "Hardening and Inference": the final weights are "directly deployable on NVFP4
@@ -618,13 +620,13 @@ FAAR_API int faar_model_overlap(const faar_model* model, int batch, int seq, int
 FAAR_API int faar_model_forward_both(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* tokens, const int* positions,
                                      float beta, void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp, void* arena,
                                      size_t arena_bytes, void* Z, void* H, void* workspace, size_t workspace_bytes);
-/* Both with the logits' softmax statistics at temperature tau (see faar_align_loss_stats). */
+/* Both with the logits' softmax statistics at temperature tau, stats_bytes each (see faar_align_loss_stats). */
 FAAR_API int faar_model_forward_stats(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* tokens, const int* positions,
                                       int quantised, float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, float tau,
-                                      void* stats, void* workspace, size_t workspace_bytes);
+                                      void* stats, size_t stats_bytes, void* workspace, size_t workspace_bytes);
 FAAR_API int faar_model_forward_both_stats(faar_ctx* ctx, const faar_model* model, int batch, int seq, const int* tokens,
                                            const int* positions, float beta, void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp,
-                                           void* arena, size_t arena_bytes, void* Z, void* H, float tau, void* stats_fp, void* stats,
+                                           void* arena, size_t arena_bytes, void* Z, void* H, float tau, void* stats_fp, void* stats, size_t stats_bytes,
                                            void* workspace, size_t workspace_bytes);
 /* From the loss gradients at the logits (dZ, row stride ldz) and at the last hidden state (dH) back to every V, which is
  * updated in place.  arena: of the quantised forward pass with keep != 0 of the same step. */

@@ -209,6 +209,16 @@ faar_prof_scope::faar_prof_scope(faar_ctx* ctx, int kernel_id) : c(ctx), pair(-1
   pair = i;
 }
 
+int faar_check_logit_stats(faar_ctx* ctx, int T, int vocab, const void* stats, size_t stats_bytes) {
+  if (!stats) return FAAR_ERR_INVALID_ARG;
+  size_t need = 0;
+  const int st = faar_logit_stats_size(ctx, T, vocab, &need);
+  if (st) return st;
+  if (need == 0) return FAAR_ERR_SHAPE;
+  if (!aligned16(stats)) return FAAR_ERR_ALIGN;
+  return stats_bytes < need ? FAAR_ERR_WORKSPACE : FAAR_OK;
+}
+
 int faar_check_hparams(const faar_hparams* hp, bool need_opt) { return check_hp(hp, need_opt); }
 
 int faar_bwd_group(faar_ctx* ctx, int n_seg, faar_bwd_state* seg, int T, int K, const faar_hparams* hp, const void* dY, int64_t ldy,
@@ -1076,20 +1086,22 @@ int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_f
                     workspace_bytes);
 }
 
-int faar_align_loss_stats(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz, const void* H_fp,
-                          const void* H_q, int64_t ldh, float tau, float lambda_kl, const void* stats_fp, const void* stats_q, void* dZ_q,
-                          void* dH_q, float* loss_out2, void* workspace, size_t workspace_bytes) {
-  if (!stats_fp || !stats_q) return FAAR_ERR_INVALID_ARG;
-  if (!aligned16(stats_fp) || !aligned16(stats_q)) return FAAR_ERR_ALIGN;
-  return align_loss(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, stats_fp, stats_q, dZ_q, dH_q, loss_out2, workspace,
-                    workspace_bytes);
-}
-
 int faar_logit_stats_size(faar_ctx* ctx, int T, int vocab, size_t* bytes) {
   if (!ctx || !bytes) return FAAR_ERR_INVALID_ARG;
   if (T <= 0 || vocab <= 0) return FAAR_ERR_SHAPE;
   *bytes = vocab % 16 == 0 && faar_logit_stats_pay(ctx, T, vocab) ? (size_t)T * (size_t)((vocab + 127) / 128) * sizeof(float2) : 0;
   return FAAR_OK;
+}
+
+int faar_align_loss_stats(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz, const void* H_fp,
+                          const void* H_q, int64_t ldh, float tau, float lambda_kl, const void* stats_fp, const void* stats_q,
+                          size_t stats_bytes, void* dZ_q, void* dH_q, float* loss_out2, void* workspace, size_t workspace_bytes) {
+  if (!stats_fp || !stats_q) return FAAR_ERR_INVALID_ARG;
+  int st = faar_check_logit_stats(ctx, T, vocab, stats_fp, stats_bytes);
+  if (!st) st = faar_check_logit_stats(ctx, T, vocab, stats_q, stats_bytes);
+  if (st) return st;
+  return align_loss(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, stats_fp, stats_q, dZ_q, dH_q, loss_out2, workspace,
+                    workspace_bytes);
 }
 
 int faar_harden_pack(faar_ctx* ctx, const faar_shape* s, const float* V, const uint8_t* code, const uint8_t* scales,

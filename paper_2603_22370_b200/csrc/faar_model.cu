@@ -134,7 +134,7 @@ int product_sums(faar_ctx* ctx, const Sizes& s, const void* dY, const void* W, c
 }
 
 // Logits and, if wanted, their rows' softmax statistics at temperature tau
-struct Stats { float tau; void* out; };
+struct Stats { float tau; void* out; size_t bytes; };
 int product_logits(faar_ctx* ctx, const faar_model* m, size_t T, const void* H, void* Z, const Stats& st, void* ws) {
   if (!st.out) return product(ctx, T, m->vocab, m->hidden, H, m->hidden, m->lm_head, m->hidden, false, Z, m->vocab, ws);
   faar_gemm_args a = {};
@@ -443,8 +443,7 @@ int faar_model_sizes(const faar_model* m, int batch, int seq, int keep, size_t* 
 static int check_stats(faar_ctx* ctx, const faar_model* m, int batch, int seq, const Stats& st) {
   if (!st.out) return FAAR_OK;
   if (!(st.tau > 0.f) || !isfinite(st.tau)) return FAAR_ERR_INVALID_ARG;
-  if (!aligned(st.out)) return FAAR_ERR_ALIGN;
-  return faar_logit_stats_pay(ctx, batch * seq, m->vocab) ? FAAR_OK : FAAR_ERR_SHAPE;
+  return faar_check_logit_stats(ctx, batch * seq, m->vocab, st.out, st.bytes);
 }
 static int model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, int quantised,
                          float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, const Stats& stats, void* workspace,
@@ -467,14 +466,14 @@ static int model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq,
 int faar_model_forward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, int quantised,
                        float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, void* workspace,
                        size_t workspace_bytes) {
-  return model_forward(ctx, m, batch, seq, tokens, positions, quantised, beta, keep, arena, arena_bytes, Z, H, {1.f, nullptr}, workspace,
+  return model_forward(ctx, m, batch, seq, tokens, positions, quantised, beta, keep, arena, arena_bytes, Z, H, {1.f, nullptr, 0}, workspace,
                        workspace_bytes);
 }
 int faar_model_forward_stats(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, int quantised,
-                             float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, float tau, void* stats, void* workspace,
+                             float beta, int keep, void* arena, size_t arena_bytes, void* Z, void* H, float tau, void* stats, size_t stats_bytes, void* workspace,
                              size_t workspace_bytes) {
   if (!stats) return FAAR_ERR_INVALID_ARG;
-  return model_forward(ctx, m, batch, seq, tokens, positions, quantised, beta, keep, arena, arena_bytes, Z, H, {tau, stats}, workspace,
+  return model_forward(ctx, m, batch, seq, tokens, positions, quantised, beta, keep, arena, arena_bytes, Z, H, {tau, stats, stats_bytes}, workspace,
                        workspace_bytes);
 }
 
@@ -516,14 +515,14 @@ int faar_model_forward_both(faar_ctx* ctx, const faar_model* m, int batch, int s
                             void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp, void* arena, size_t arena_bytes, void* Z,
                             void* H, void* workspace, size_t workspace_bytes) {
   return model_forward_both(ctx, m, batch, seq, tokens, positions, beta, arena_fp, arena_fp_bytes, Z_fp, H_fp, arena, arena_bytes, Z, H,
-                            {1.f, nullptr}, {1.f, nullptr}, workspace, workspace_bytes);
+                            {1.f, nullptr, 0}, {1.f, nullptr, 0}, workspace, workspace_bytes);
 }
 int faar_model_forward_both_stats(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* tokens, const int* positions, float beta,
                                   void* arena_fp, size_t arena_fp_bytes, void* Z_fp, void* H_fp, void* arena, size_t arena_bytes, void* Z,
-                                  void* H, float tau, void* stats_fp, void* stats, void* workspace, size_t workspace_bytes) {
+                                  void* H, float tau, void* stats_fp, void* stats, size_t stats_bytes, void* workspace, size_t workspace_bytes) {
   if (!stats_fp || !stats) return FAAR_ERR_INVALID_ARG;
   return model_forward_both(ctx, m, batch, seq, tokens, positions, beta, arena_fp, arena_fp_bytes, Z_fp, H_fp, arena, arena_bytes, Z, H,
-                            {tau, stats_fp}, {tau, stats}, workspace, workspace_bytes);
+                            {tau, stats_fp, stats_bytes}, {tau, stats, stats_bytes}, workspace, workspace_bytes);
 }
 
 int faar_model_backward(faar_ctx* ctx, const faar_model* m, int batch, int seq, const int* positions, const faar_hparams* hp,

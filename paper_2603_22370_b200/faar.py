@@ -61,7 +61,7 @@ SIGNATURES = {
     "faar_align_loss_workspace_size": (_I, [_I, _I, _P]),
     "faar_align_loss": (_I, [_P, _I, _I, _I, _P, _P, _L, _P, _P, _L, _F, _F, _P, _P, _P, _P, _Z]),
     "faar_logit_stats_size": (_I, [_P, _I, _I, _P]),
-    "faar_align_loss_stats": (_I, [_P, _I, _I, _I, _P, _P, _L, _P, _P, _L, _F, _F, _P, _P, _P, _P, _P, _P, _Z]),
+    "faar_align_loss_stats": (_I, [_P, _I, _I, _I, _P, _P, _L, _P, _P, _L, _F, _F, _P, _P, _Z, _P, _P, _P, _P, _Z]),
     "faar_swizzle_scales": (_I, [_P, _I, _I, _P, _P, _Z]),
     "faar_silu_mul": (_I, [_P, _I, _I, _P, _L, _P, _L, _P, _L]),
     "faar_rmsnorm": (_I, [_P, _I, _I, _P, _L, _P, _F, _P, _L, _P]),
@@ -81,8 +81,8 @@ SIGNATURES = {
     "faar_model_forward": (_I, [_P, _P, _I, _I, _P, _P, _I, _F, _I, _P, _Z, _P, _P, _P, _Z]),
     "faar_model_overlap": (_I, [_P, _I, _I, _P]),
     "faar_model_forward_both": (_I, [_P, _P, _I, _I, _P, _P, _F, _P, _Z, _P, _P, _P, _Z, _P, _P, _P, _Z]),
-    "faar_model_forward_stats": (_I, [_P, _P, _I, _I, _P, _P, _I, _F, _I, _P, _Z, _P, _P, _F, _P, _P, _Z]),
-    "faar_model_forward_both_stats": (_I, [_P, _P, _I, _I, _P, _P, _F, _P, _Z, _P, _P, _P, _Z, _P, _P, _F, _P, _P, _P, _Z]),
+    "faar_model_forward_stats": (_I, [_P, _P, _I, _I, _P, _P, _I, _F, _I, _P, _Z, _P, _P, _F, _P, _Z, _P, _Z]),
+    "faar_model_forward_both_stats": (_I, [_P, _P, _I, _I, _P, _P, _F, _P, _Z, _P, _P, _P, _Z, _P, _P, _F, _P, _P, _Z, _P, _Z]),
     "faar_model_backward": (_I, [_P, _P, _I, _I, _P, _P, _P, _Z, _P, _L, _P, _P, _Z, _P, _Z]),
     "faar_nvfp4_gemm": (_I, [_P, _I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _L, _P, _Z]),
 }
@@ -314,9 +314,14 @@ def logit_stats_size(ctx, T, vocab) -> int:
     return n.value
 
 
+def _stats_bytes(*stats) -> int:
+    """Bytes of the smallest of the buffers; none for one that is missing, which the call refuses."""
+    return min(0 if s is None else s.nbytes for s in stats)
+
+
 def align_loss_stats(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, stats_fp, stats_q, dZ_q, dH_q, loss_out2, ws):
-    _check(_fast().faar_align_loss_stats(ctx._n, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, stats_fp, stats_q, dZ_q,
-                                         dH_q, loss_out2, ws, ws.numel()), "faar_align_loss_stats")
+    _check(_fast().faar_align_loss_stats(ctx._n, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, stats_fp, stats_q,
+                                         _stats_bytes(stats_fp, stats_q), dZ_q, dH_q, loss_out2, ws, ws.numel()), "faar_align_loss_stats")
 
 
 def swizzle_scales(ctx, rows, cols, scales, scales_tiled):
@@ -404,15 +409,15 @@ def model_sizes(model: Model, batch: int, seq: int, keep: int) -> tuple[int, int
 
 
 class Region(int):
-    """Device memory by its address, `bytes` long: stands for a tensor in the calls of a model's passes."""
+    """Device memory by its address, `nbytes` long: stands for a tensor in the calls of a model's passes."""
 
-    def __new__(cls, address: int, bytes: int):
+    def __new__(cls, address: int, nbytes: int):
         r = int.__new__(cls, address)
-        r.bytes = bytes
+        r.nbytes = nbytes
         return r
 
     def numel(self) -> int:
-        return self.bytes
+        return self.nbytes
 
 
 def model_forward(ctx, model, batch, seq, tokens, positions, quantised, beta, keep, arena, Z, H, ws):
@@ -434,12 +439,14 @@ def model_forward_both(ctx, model, batch, seq, tokens, positions, beta, arena_fp
 
 def model_forward_stats(ctx, model, batch, seq, tokens, positions, quantised, beta, keep, arena, Z, H, tau, stats, ws):
     _check(_fast().faar_model_forward_stats(ctx._n, model, batch, seq, tokens, positions, int(quantised), beta, int(keep), arena,
-                                            arena.numel(), Z, H, tau, stats, ws, ws.numel()), "faar_model_forward_stats")
+                                            arena.numel(), Z, H, tau, stats, _stats_bytes(stats), ws, ws.numel()),
+           "faar_model_forward_stats")
 
 
 def model_forward_both_stats(ctx, model, batch, seq, tokens, positions, beta, arena_fp, Z_fp, H_fp, arena, Z, H, tau, stats_fp, stats, ws):
     _check(_fast().faar_model_forward_both_stats(ctx._n, model, batch, seq, tokens, positions, beta, arena_fp, arena_fp.numel(), Z_fp, H_fp,
-                                                 arena, arena.numel(), Z, H, tau, stats_fp, stats, ws, ws.numel()),
+                                                 arena, arena.numel(), Z, H, tau, stats_fp, stats, _stats_bytes(stats_fp, stats), ws,
+                                                 ws.numel()),
            "faar_model_forward_both_stats")
 
 

@@ -52,3 +52,36 @@ def test_small_products_leave_none(ctx):  # noqa: F811
     with pytest.raises(faar.FaarError) as e:
         m._forward(m._table(), tokens, False, tau=0.0, stats=stats)
     assert e.value.status == faar.ERR_INVALID_ARG
+
+
+def test_buffers_and_products_that_the_statistics_calls_refuse(ctx):  # noqa: F811
+    """A buffer for fewer tokens or a smaller vocabulary, in any of the calls, and a loss on statistics that no product leaves.  Every
+    refusal comes from a comparison on the host: nothing is launched."""
+    batch, seq, vocab, d = 1, 257, 18944, 64
+    m, tokens, _ = make_model(ctx, batch, seq, vocab=vocab, hidden=d, n_layers=1, n_heads=1, n_kv_heads=1, head_dim=64, ffn=64)
+    n = faar.logit_stats_size(ctx, seq, vocab)
+    Z, H = (torch.zeros((seq, c), dtype=torch.bfloat16, device=DEV) for c in (vocab, d))
+    arena = {k: torch.empty(m.arena_bytes[k], dtype=torch.uint8, device=DEV) for k in (False, True)}
+    whole, short = (torch.zeros(k, dtype=torch.uint8, device=DEV) for k in (n, n - 1))
+    table, loss = m._table(), torch.zeros(2, device=DEV)
+
+    def forward(s):
+        faar.model_forward_stats(ctx, table, batch, seq, tokens, m.pos, False, 4.0, False, arena[False], Z, H, 1.0, s, m.ws)
+
+    def both(s_fp, s):
+        faar.model_forward_both_stats(ctx, table, batch, seq, tokens, m.pos, 4.0, arena[False], Z, H, arena[True], Z, H, 1.0, s_fp, s, m.ws)
+
+    def align(s_fp, s, T=seq, V=vocab):
+        faar.align_loss_stats(ctx, T, V, d, Z, Z, vocab, H, H, d, 1.0, 1.0, s_fp, s, None, None, loss, m.aws)
+
+    for call, status in [(lambda: forward(short), faar.ERR_WORKSPACE), (lambda: both(whole, short), faar.ERR_WORKSPACE),
+                         (lambda: both(short, whole), faar.ERR_WORKSPACE), (lambda: align(whole, short), faar.ERR_WORKSPACE),
+                         (lambda: align(short, whole), faar.ERR_WORKSPACE), (lambda: align(whole, None), faar.ERR_INVALID_ARG),
+                         (lambda: forward(None), faar.ERR_INVALID_ARG), (lambda: align(whole, whole, T=128), faar.ERR_SHAPE),
+                         (lambda: align(whole, whole, V=vocab - 8), faar.ERR_SHAPE), (lambda: align(whole[8:], whole), faar.ERR_ALIGN)]:
+        with pytest.raises(faar.FaarError) as e:
+            call()
+        assert e.value.status == status
+    align(whole, whole)
+    torch.cuda.synchronize()
+    faar.check_status(ctx, m.ws)
