@@ -467,10 +467,12 @@ FAAR_API int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const 
 
 /* The same loss from softmax statistics that the logits' products left behind (faar_model_forward_stats,
  * faar_model_forward_both_stats): the logits are then read once instead of twice.  stats_fp, stats_q: stats_bytes each, at least
- * what faar_logit_stats_size gives (FAAR_ERR_WORKSPACE), 16-byte aligned.  A size of 0 says that the product is too small for
- * them to pay: the forward calls don't take them and this call refuses, too (FAAR_ERR_SHAPE).  They belong to the logits and
+ * what faar_logit_stats_size gives (FAAR_ERR_WORKSPACE), 16-byte aligned.  A size of 0 says that the product is too small to
+ * leave them: the forward calls don't take them and this call refuses, too (FAAR_ERR_SHAPE).  faar_logit_stats_pay says whether a
+ * step with them is faster: few tokens are better off without.  They belong to the logits and
  * to the tau that they were formed with; with another tau here the loss and its gradient are wrong, which no call can see. */
 FAAR_API int faar_logit_stats_size(faar_ctx* ctx, int T, int vocab, size_t* bytes);
+FAAR_API int faar_logit_stats_pay(faar_ctx* ctx, int T, int vocab, int* pay);
 FAAR_API int faar_align_loss_stats(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
                                    const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, const void* stats_fp,
                                    const void* stats_q, size_t stats_bytes, void* dZ_q, void* dH_q, float* loss_out2, void* workspace,

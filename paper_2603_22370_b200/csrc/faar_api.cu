@@ -1089,8 +1089,16 @@ int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_f
 int faar_logit_stats_size(faar_ctx* ctx, int T, int vocab, size_t* bytes) {
   if (!ctx || !bytes) return FAAR_ERR_INVALID_ARG;
   if (T <= 0 || vocab <= 0) return FAAR_ERR_SHAPE;
-  *bytes = vocab % 16 == 0 && faar_logit_stats_pay(ctx, T, vocab) ? (size_t)T * (size_t)((vocab + 127) / 128) * sizeof(float2) : 0;
+  *bytes = vocab % 16 == 0 && faar_logit_stats_fit(ctx, T, vocab) ? (size_t)T * (size_t)((vocab + 127) / 128) * sizeof(float2) : 0;
   return FAAR_OK;
+}
+
+int faar_logit_stats_pay(faar_ctx* ctx, int T, int vocab, int* pay) {
+  if (!pay) return FAAR_ERR_INVALID_ARG;
+  size_t bytes = 0;
+  const int st = faar_logit_stats_size(ctx, T, vocab, &bytes);
+  if (!st) *pay = bytes != 0 && faar_logit_stats_pays(ctx, T, vocab);
+  return st;
 }
 
 int faar_align_loss_stats(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz, const void* H_fp,

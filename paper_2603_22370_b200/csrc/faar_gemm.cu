@@ -1963,11 +1963,17 @@ static bool result_columns(const faar_gemm_args* a) {
   return a->M <= BM || row % 16 != 0 || (reinterpret_cast<uintptr_t>(a->Yout) & 15) != 0;
 }
 
-// Whether the logits' statistics are worth taking: where every CTA pair has 256-wide tiles anyway (and more than a half-empty row
-// block); a smaller product is better cut into narrower ones.
-bool faar_logit_stats_pay(const faar_ctx* ctx, int T, int vocab) {
-  const long long tiles = (long long)((T + 2 * BM - 1) / (2 * BM)) * ((vocab + BN_MAX - 1) / BN_MAX);
-  return T > BM && tiles >= ctx->num_sms / 2;
+// Which products leave statistics at all: those where every CTA pair has 256-wide tiles anyway (and more than a half-empty row
+// block); a smaller one is better cut into narrower tiles.
+static long long wide_tiles(int T, int vocab) { return (long long)((T + 2 * BM - 1) / (2 * BM)) * ((vocab + BN_MAX - 1) / BN_MAX); }
+bool faar_logit_stats_fit(const faar_ctx* ctx, int T, int vocab) { return T > BM && wide_tiles(T, vocab) >= ctx->num_sms / 2; }
+// And where they save time: such a product has no half-width tiles to even out its last wave, which both passes pay for, and the
+// loss gains with the tokens.  Both forward passes of one block, 2048 wide, and the loss, without statistics -> with them, us:
+// tokens x vocabulary 129 x 128256 344 -> 361, 150 x 20480 187 -> 191, 200 x 25600 197 -> 204, 256 x 50000 243 -> 247, 300 x 12800 193
+// -> 198, 300 x 32000 245 -> 248, 600 x 6400 (75 tiles) 203 -> 206, 1000 x 4864 (76) 243 -> 243; 512 x 16000 223 -> 216, 600 x 9600 220 ->
+// 211, 600 x 128256 786 -> 786, 1000 x 9600 272 -> 267, 2000 x 2560 311 -> 302, 2000 x 32000 667 -> 663, 4096 x 8192 728 -> 674.
+bool faar_logit_stats_pays(const faar_ctx* ctx, int T, int vocab) {
+  return T >= 1000 ? faar_logit_stats_fit(ctx, T, vocab) : T >= 512 && 3 * wide_tiles(T, vocab) >= 2 * ctx->num_sms;
 }
 
 int faar_launch_wait_selftest(faar_ctx* ctx, uint32_t* status, unsigned long long limit_ns) {

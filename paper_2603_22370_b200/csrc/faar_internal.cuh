@@ -248,7 +248,8 @@ struct faar_gemm_args {
 };
 // n_partials_out: number of floats a FWD launch writes to args.partials
 int faar_launch_gemm(faar_ctx*, const faar_gemm_args*, int* n_partials_out);
-bool faar_logit_stats_pay(const faar_ctx*, int T, int vocab);
+bool faar_logit_stats_fit(const faar_ctx*, int T, int vocab);
+bool faar_logit_stats_pays(const faar_ctx*, int T, int vocab);
 int faar_check_logit_stats(faar_ctx*, int T, int vocab, const void* stats, size_t stats_bytes);      // a caller's buffer of them
 int faar_gemm_max_partials(const faar_ctx*, int M, int N);
 int faar_launch_wait_selftest(faar_ctx*, uint32_t* status, unsigned long long limit_ns);

@@ -61,6 +61,7 @@ SIGNATURES = {
     "faar_align_loss_workspace_size": (_I, [_I, _I, _P]),
     "faar_align_loss": (_I, [_P, _I, _I, _I, _P, _P, _L, _P, _P, _L, _F, _F, _P, _P, _P, _P, _Z]),
     "faar_logit_stats_size": (_I, [_P, _I, _I, _P]),
+    "faar_logit_stats_pay": (_I, [_P, _I, _I, _P]),
     "faar_align_loss_stats": (_I, [_P, _I, _I, _I, _P, _P, _L, _P, _P, _L, _F, _F, _P, _P, _Z, _P, _P, _P, _P, _Z]),
     "faar_swizzle_scales": (_I, [_P, _I, _I, _P, _P, _Z]),
     "faar_silu_mul": (_I, [_P, _I, _I, _P, _L, _P, _L, _P, _L]),
@@ -312,6 +313,12 @@ def logit_stats_size(ctx, T, vocab) -> int:
     n = C.c_size_t(0)
     _check(lib().faar_logit_stats_size(ctx._h, T, vocab, C.byref(n)), "faar_logit_stats_size")
     return n.value
+
+
+def logit_stats_pay(ctx, T, vocab) -> bool:
+    n = C.c_int(0)
+    _check(lib().faar_logit_stats_pay(ctx._h, T, vocab, C.byref(n)), "faar_logit_stats_pay")
+    return bool(n.value)
 
 
 def _stats_bytes(*stats) -> int:

@@ -117,10 +117,15 @@ class Stage2Model:
     def _new(self, cols, dtype=torch.bfloat16):
         return torch.empty((self.T, cols), dtype=dtype, device=self.dev)
 
+    def _stats_bytes(self) -> int:
+        """Bytes of the statistics that a pass's logits leave for the loss, 0 where a step is faster without."""
+        T, vocab = self.T, self.cfg.vocab
+        return faar.logit_stats_size(self.ctx, T, vocab) if faar.logit_stats_pay(self.ctx, T, vocab) else 0
+
     def _plan_regions(self):
         """Where the buffers of a small model's step lie in its one allocation: (name, first byte, bytes)."""
         z, h = 2 * self.T * self.cfg.vocab, 2 * self.T * self.cfg.hidden
-        stats = faar.logit_stats_size(self.ctx, self.T, self.cfg.vocab)
+        stats = self._stats_bytes()
         self._regions, at = [], 0
         for name, n in (("fp", self.arena_bytes[False]), ("q", self.arena_bytes[True]), ("scratch", self.scratch_bytes), ("Z_fp", z),
                         ("H_fp", h), ("Z_q", z), ("H_q", h), ("dZ", z), ("dH", h), ("stats_fp", stats), ("stats_q", stats)):
@@ -254,7 +259,7 @@ class Stage2Model:
             Z_fp, H_fp = fp_outputs
             Z_q, H_q, saved = self._forward(model, tokens, quantised=True, beta=beta, keep=True)
         else:
-            n = faar.logit_stats_size(self.ctx, T, c.vocab)
+            n = self._stats_bytes()
             if n:
                 stats = tuple(torch.empty(n, dtype=torch.uint8, device=self.dev) for _ in range(2))
             Z_fp, H_fp = self._forward(model, tokens, quantised=False, tau=tau, stats=stats[0] if n else None)[:2]

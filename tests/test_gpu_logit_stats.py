@@ -85,3 +85,16 @@ def test_buffers_and_products_that_the_statistics_calls_refuse(ctx):  # noqa: F8
     align(whole, whole)
     torch.cuda.synchronize()
     faar.check_status(ctx, m.ws)
+
+
+@pytest.mark.parametrize("T,vocab,fit,pay", [
+    (511, 128256, True, False),           # few tokens, whatever the vocabulary
+    (512, 12544, True, False),            # 98 tiles of 256 x 256
+    (512, 12800, True, True),             # 100
+    (999, 6144, True, False),
+    (1000, 4736, True, True),             # 76
+    (1000, 4608, False, False),           # 72: not a tile for every CTA pair
+    (4096, 1192, False, False),           # not a multiple of 16
+])
+def test_where_statistics_pay(ctx, T, vocab, fit, pay):  # noqa: F811
+    assert (faar.logit_stats_size(ctx, T, vocab) > 0, faar.logit_stats_pay(ctx, T, vocab)) == (fit, pay)
