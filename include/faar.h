@@ -473,6 +473,9 @@ FAAR_API int faar_align_loss(faar_ctx* ctx, int T, int vocab, int hidden, const 
  * to the tau that they were formed with; with another tau here the loss and its gradient are wrong, which no call can see. */
 FAAR_API int faar_logit_stats_size(faar_ctx* ctx, int T, int vocab, size_t* bytes);
 FAAR_API int faar_logit_stats_pay(faar_ctx* ctx, int T, int vocab, int* pay);
+/* The statistics of logits Z [T, ldz] that are there already (a frozen model's outputs that are used for several steps): bit for
+ * bit what their product leaves, so that a step on them gives the bits of one that forms them again. */
+FAAR_API int faar_logit_stats(faar_ctx* ctx, int T, int vocab, const void* Z, int64_t ldz, float tau, void* stats, size_t stats_bytes);
 FAAR_API int faar_align_loss_stats(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz,
                                    const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, const void* stats_fp,
                                    const void* stats_q, size_t stats_bytes, void* dZ_q, void* dH_q, float* loss_out2, void* workspace,

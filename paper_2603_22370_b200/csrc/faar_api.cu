@@ -1101,6 +1101,17 @@ int faar_logit_stats_pay(faar_ctx* ctx, int T, int vocab, int* pay) {
   return st;
 }
 
+int faar_logit_stats(faar_ctx* ctx, int T, int vocab, const void* Z, int64_t ldz, float tau, void* stats, size_t stats_bytes) {
+  if (!ctx || !Z) return FAAR_ERR_INVALID_ARG;
+  if (!(tau > 0.f) || !isfinite(tau)) return FAAR_ERR_INVALID_ARG;
+  const int st = faar_check_logit_stats(ctx, T, vocab, stats, stats_bytes);
+  if (st) return st;
+  if (ldz < vocab) return FAAR_ERR_SHAPE;
+  if (ldz % 8 || !aligned16(Z)) return FAAR_ERR_ALIGN;
+  FAAR_DEVICE_GUARD(ctx);
+  return cuda_fail(ctx, faar_launch_logit_stats(ctx, T, vocab, Z, ldz, tau, reinterpret_cast<float2*>(stats)));
+}
+
 int faar_align_loss_stats(faar_ctx* ctx, int T, int vocab, int hidden, const void* Z_fp, const void* Z_q, int64_t ldz, const void* H_fp,
                           const void* H_q, int64_t ldh, float tau, float lambda_kl, const void* stats_fp, const void* stats_q,
                           size_t stats_bytes, void* dZ_q, void* dH_q, float* loss_out2, void* workspace, size_t workspace_bytes) {

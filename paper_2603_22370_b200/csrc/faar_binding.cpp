@@ -94,7 +94,7 @@ template <class T> struct Arg<T, std::enable_if_t<std::is_pointer_v<T>>> {
   X(faar_layer_step_host_nvfp4) X(faar_harden_pack) X(faar_align_loss) X(faar_swizzle_scales) X(faar_rmsnorm)             \
   X(faar_rmsnorm_bwd) X(faar_add_rmsnorm) X(faar_rmsnorm_bwd_sum) X(faar_rope) X(faar_silu_mul_bwd) X(faar_embedding)     \
   X(faar_add) X(faar_attention_fwd) X(faar_attention_bwd) X(faar_nvfp4_gemm) X(faar_model_forward) X(faar_model_forward_both) X(faar_model_backward) \
-  X(faar_model_forward_stats) X(faar_model_forward_both_stats) X(faar_align_loss_stats)
+  X(faar_model_forward_stats) X(faar_model_forward_both_stats) X(faar_logit_stats) X(faar_align_loss_stats)
 
 enum {
 #define SLOT(name) SLOT_##name,

@@ -434,11 +434,6 @@ __device__ __forceinline__ int tile_count(const KParams& p, int m_tiles) {
   return 2 * m_tiles * p.n_main - p.n_full + (p.narrow ? m_tiles : 0);
 }
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&p);
@@ -679,18 +674,14 @@ __device__ __forceinline__ void epi_rope(const KParams& p, uint32_t trow, int ro
 // of its own over the logits.  A warp's 128 columns are one slot; its lanes keep (m, s) of their rows over the 32 columns in
 // registers.  Under the main loop: [8192, 128256] over 2048 2.85 ms either way, [2000, 32000] 150 us.
 __device__ __forceinline__ void stats_update(const KParams& p, const uint32_t (&acc)[16], float& m, float& s) {
-  float y[16], mx = -INFINITY;
+  float z[16];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
+  for (int j = 0; j < 8; ++j) {                          // as they are stored
     const uint32_t w = pack_bf16x2(__uint_as_float(acc[2 * j]), __uint_as_float(acc[2 * j + 1]));
-    y[2 * j] = __uint_as_float(w << 16);
-    y[2 * j + 1] = __uint_as_float(w & 0xFFFF0000u);
-    mx = fmaxf(mx, fmaxf(y[2 * j], y[2 * j + 1]));
+    z[2 * j] = __uint_as_float(w << 16);
+    z[2 * j + 1] = __uint_as_float(w & 0xFFFF0000u);
   }
-  mx *= p.mse2c;                                        // c > 0: scaling keeps the order
-  if (mx > m) { s *= ex2_approx(m - mx); m = mx; }      // 2^-inf = 0 on the first chunk
-#pragma unroll
-  for (int j = 0; j < 16; ++j) s += ex2_approx(fmaf(y[j], p.mse2c, -m));
+  faar_stats_update(z, p.mse2c, m, s);
 }
 
 // Attention output's gradient dO = dY W (B untransposed): delta = sum of dO * O over a head's columns, which the attention's backward
@@ -946,7 +937,7 @@ __device__ __forceinline__ float epi_bwd_rows(const KParams& p, const Segment& s
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         float& v = cur.v[4 * h + j];
-        const float ex = ex2_approx(-fabsf(fmaf(p.bl, v, p.hbl)));         // e^-|beta (v - 0.5)|
+        const float ex = faar_ex2(-fabsf(fmaf(p.bl, v, p.hbl)));         // e^-|beta (v - 0.5)|
         const float hs = rcp_approx(1.0f + ex);
         const float dh = ex * hs * hs;                                     // h (1 - h)
         // dh times the width factor by an add to its exponent field (a dh flushed to 0 becomes ~1e-38), then

@@ -167,6 +167,8 @@ int faar_launch_align_loss(faar_ctx*, int T, int vocab, int hidden, const void* 
                            const void* H_fp, const void* H_q, int64_t ldh, float tau, float lambda_kl, void* dZ_q,
                            void* dH_q, float* kl_partials, float* mse_partials, uint32_t* finished, float* loss_out2,
                            const float2* stats_fp = nullptr, const float2* stats_q = nullptr);      // of the logits' products, both or none
+// The statistics that a product of these logits leaves, [T, ceil(vocab / 128)]
+int faar_launch_logit_stats(faar_ctx*, int T, int vocab, const void* Z, int64_t ldz, float tau, float2* stats);
 int faar_launch_silu_mul(faar_ctx*, int rows, int cols, const void* gate, int64_t ldg, const void* up, int64_t ldu,
                          void* out, int64_t ldo);
 int faar_launch_rmsnorm(faar_ctx*, int rows, int cols, const void* x, int64_t ldx, const void* b, int64_t ldb,
@@ -393,6 +395,23 @@ __device__ __forceinline__ void faar_rope_turn(float& a, float& b, float sn, flo
   const float x = fmaf(a, cs, -(b * sn)), y = fmaf(b, cs, a * sn);
   a = x;
   b = y;
+}
+
+__device__ __forceinline__ float faar_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// Maximum m of c z and sum s of 2^(c z - m) over a row's values z so far, 16 more of them taken in; before the first, m = -inf, s = 0.
+// One order of every sum wherever a row's statistics are formed: 128 columns in turn.
+__device__ __forceinline__ void faar_stats_update(const float (&z)[16], float c, float& m, float& s) {
+  float mx = -INFINITY;
+#pragma unroll
+  for (int j = 0; j < 16; j += 2) mx = fmaxf(mx, fmaxf(z[j], z[j + 1]));
+  mx *= c;                                            // c > 0: scaling keeps the order
+  if (mx > m) { s *= faar_ex2(m - mx); m = mx; }      // 2^-inf = 0 on the first 16
+#pragma unroll
+  for (int j = 0; j < 16; ++j) s += faar_ex2(fmaf(z[j], c, -m));
 }
 
 __device__ __forceinline__ float faar_warp_sum(float v) {

@@ -62,6 +62,7 @@ SIGNATURES = {
     "faar_align_loss": (_I, [_P, _I, _I, _I, _P, _P, _L, _P, _P, _L, _F, _F, _P, _P, _P, _P, _Z]),
     "faar_logit_stats_size": (_I, [_P, _I, _I, _P]),
     "faar_logit_stats_pay": (_I, [_P, _I, _I, _P]),
+    "faar_logit_stats": (_I, [_P, _I, _I, _P, _L, _F, _P, _Z]),
     "faar_align_loss_stats": (_I, [_P, _I, _I, _I, _P, _P, _L, _P, _P, _L, _F, _F, _P, _P, _Z, _P, _P, _P, _P, _Z]),
     "faar_swizzle_scales": (_I, [_P, _I, _I, _P, _P, _Z]),
     "faar_silu_mul": (_I, [_P, _I, _I, _P, _L, _P, _L, _P, _L]),
@@ -324,6 +325,10 @@ def logit_stats_pay(ctx, T, vocab) -> bool:
 def _stats_bytes(*stats) -> int:
     """Bytes of the smallest of the buffers; none for one that is missing, which the call refuses."""
     return min(0 if s is None else s.nbytes for s in stats)
+
+
+def logit_stats(ctx, T, vocab, Z, ldz, tau, stats):
+    _check(_fast().faar_logit_stats(ctx._n, T, vocab, Z, ldz, tau, stats, _stats_bytes(stats)), "faar_logit_stats")
 
 
 def align_loss_stats(ctx, T, vocab, hidden, Z_fp, Z_q, ldz, H_fp, H_q, ldh, tau, lambda_kl, stats_fp, stats_q, dZ_q, dH_q, loss_out2, ws):

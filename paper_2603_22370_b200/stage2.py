@@ -187,10 +187,14 @@ class Stage2Model:
             faar.model_forward_stats(*args, tau, stats, self.ws)
         return Z, H, (arena if keep else None)
 
-    def _forward_both(self, model: faar.Model, tokens, beta):
+    def _forward_both(self, model: faar.Model, tokens, beta, tau=1.0, stats=None):
         fp, q = (torch.empty(self.arena_bytes[k], dtype=torch.uint8, device=self.dev) for k in (False, True))
         Z_fp, H_fp, Z, H = self._new(self.cfg.vocab), self._new(self.cfg.hidden), self._new(self.cfg.vocab), self._new(self.cfg.hidden)
-        faar.model_forward_both(self.ctx, model, self.batch, self.seq, tokens, self.pos, beta, fp, Z_fp, H_fp, q, Z, H, self.ws)
+        args = (self.ctx, model, self.batch, self.seq, tokens, self.pos, beta, fp, Z_fp, H_fp, q, Z, H)
+        if stats is None:
+            faar.model_forward_both(*args, self.ws)
+        else:
+            faar.model_forward_both_stats(*args, tau, *stats, self.ws)
         return Z_fp, H_fp, Z, H, q
 
     # ---- backward ------------------------------------------------------------------------------------
@@ -252,18 +256,19 @@ class Stage2Model:
             faar.model_backward(self.ctx, model, self.batch, self.seq, self.pos, hp, r["q"], r["dZ"], c.vocab, r["dH"], r["scratch"], self.ws)
             return None
         c, T = self.cfg, self.T
-        stats = ()                             # of both passes' logits, where their products leave them
+        n = self._stats_bytes()                # as above: the step is the same, bit for bit, whatever is handed in or out
+        stats = tuple(torch.empty(n, dtype=torch.uint8, device=self.dev) for _ in range(2)) if n else ()
+        st_fp, st_q = stats or (None, None)
         if fp_outputs is None and self.overlap:
-            Z_fp, H_fp, Z_q, H_q, saved = self._forward_both(model, tokens, beta)
-        elif fp_outputs is not None:
-            Z_fp, H_fp = fp_outputs
-            Z_q, H_q, saved = self._forward(model, tokens, quantised=True, beta=beta, keep=True)
+            Z_fp, H_fp, Z_q, H_q, saved = self._forward_both(model, tokens, beta, tau, stats or None)
         else:
-            n = self._stats_bytes()
-            if n:
-                stats = tuple(torch.empty(n, dtype=torch.uint8, device=self.dev) for _ in range(2))
-            Z_fp, H_fp = self._forward(model, tokens, quantised=False, tau=tau, stats=stats[0] if n else None)[:2]
-            Z_q, H_q, saved = self._forward(model, tokens, quantised=True, beta=beta, keep=True, tau=tau, stats=stats[1] if n else None)
+            if fp_outputs is None:
+                Z_fp, H_fp = self._forward(model, tokens, quantised=False, tau=tau, stats=st_fp)[:2]
+            else:
+                Z_fp, H_fp = fp_outputs
+                if n:
+                    faar.logit_stats(self.ctx, T, c.vocab, Z_fp, c.vocab, tau, st_fp)
+            Z_q, H_q, saved = self._forward(model, tokens, quantised=True, beta=beta, keep=True, tau=tau, stats=st_q)
         dZ, dH = torch.empty_like(Z_q), torch.empty_like(H_q)
         loss = faar.align_loss_stats if stats else faar.align_loss
         loss(self.ctx, T, c.vocab, c.hidden, Z_fp, Z_q, Z_q.shape[1], H_fp, H_q, c.hidden, tau, lambda_kl, *stats, dZ, dH, self.loss, self.aws)

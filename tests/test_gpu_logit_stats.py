@@ -98,3 +98,43 @@ def test_buffers_and_products_that_the_statistics_calls_refuse(ctx):  # noqa: F8
 ])
 def test_where_statistics_pay(ctx, T, vocab, fit, pay):  # noqa: F811
     assert (faar.logit_stats_size(ctx, T, vocab) > 0, faar.logit_stats_pay(ctx, T, vocab)) == (fit, pay)
+
+
+@pytest.mark.parametrize("tau", [1.0, 1.7])
+@pytest.mark.parametrize("T,vocab", [(513, 8720), (1000, 4736)])      # a last slot of 16 columns; whole slots
+def test_a_step_is_the_same_whatever_is_handed_in_or_out(ctx, T, vocab, tau):  # noqa: F811
+    """Losses and every V of a plain step, passes next to one another or in turn, of one that returns its gradients, and of one on frozen
+    outputs formed before: statistics or not is one choice for all."""
+    assert faar.logit_stats_pay(ctx, T, vocab)
+    runs = []
+    for overlap, want_dv, given in [(True, False, False), (False, False, False), (True, True, False), (False, True, False), (True, False, True),
+                                    (False, True, True)]:
+        m, tokens, _ = make_model(ctx, 1, T, vocab=vocab, hidden=64, n_layers=1, n_heads=1, n_kv_heads=1, head_dim=64, ffn=64)
+        m.overlap = overlap
+        fp = m.forward(tokens, quantised=False)[:2] if given else None
+        m.step(tokens, beta=6.0, tau=tau, lambda_kl=0.9, want_dv=want_dv, fp_outputs=fp)
+        faar.check_status(ctx, m.ws)
+        runs.append([m.loss.clone()] + [x.V for lins in m.lin for x in lins.values()])
+    for other in runs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(runs[0], other))
+
+
+@pytest.mark.parametrize("T,vocab,ldz", [(257, 18960, 18960), (300, 9472, 9480)])
+def test_statistics_of_logits_that_are_there(ctx, T, vocab, ldz):  # noqa: F811
+    """Maximum and sum of every 128 columns against 64 bits, with a minute and an infinite logit and a row that is all alike."""
+    gen = torch.Generator(device=DEV).manual_seed(T)
+    Z = torch.full((T, ldz), float("nan"), dtype=torch.bfloat16, device=DEV)
+    Z[:, :vocab] = (torch.randn((T, vocab), device=DEV, generator=gen) * 4).to(torch.bfloat16)
+    Z[0, 5], Z[1, 130], Z[2, :vocab] = -3.0e38, float("-inf"), 1.5
+    stats = torch.full((faar.logit_stats_size(ctx, T, vocab),), 0xFF, dtype=torch.uint8, device=DEV)
+    faar.logit_stats(ctx, T, vocab, Z, ldz, 1.7, stats)
+    got = stats.view(torch.float32).view(T, -1, 2).double()
+    y = torch.full((T, got.shape[1] * 128), float("-inf"), dtype=torch.float64, device=DEV)
+    y[:, :vocab] = Z[:, :vocab].double() * (1.4426950408889634 / 1.7)
+    y = y.view(T, -1, 128)
+    m = y.max(-1).values
+    # the maximum is one rounding of the product with a rounded constant (2^-23 of it); the sum has that error in each of its exponents, the
+    # hardware exponential's (2^-22) and up to 128 additions (2^-17)
+    assert torch.all((got[..., 0] - m).abs() <= 2.0**-23 * m.abs())
+    s = torch.exp2(y - got[..., :1]).sum(-1)
+    assert torch.all((got[..., 1] - s).abs() <= (2.0**-17 + 2.0**-21 + 2.0**-22 * y[y.isfinite()].abs().clamp(max=2.0**7).max()) * s)
