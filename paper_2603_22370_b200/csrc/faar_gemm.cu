@@ -366,6 +366,7 @@ struct KParams {
   int n_full;             // the first n_full tiles of the main columns are bn wide, the others come as two halves (tail split)
   uint32_t* status;
   long long ext_yout, ext_dyt, ext_state, ext_wsoft;   // bytes of Yout, dYt, each of V / m / u / dV, wsoft_next (debug checks)
+  long long ext_partials;                              // and of partials: loss sums, softmax statistics or row sums
   // REF / FWD
   void* Yout; int yout_dtype; long long ldy;
   const void* Yref; int yref_dtype;
@@ -717,7 +718,8 @@ __device__ __forceinline__ void sum_update(const KParams& p, int row, int col, c
     sum = pending[level] + sum;
   }
   const int head = col >> (31 - __clz(dim)), part = (col & (dim - 1)) >> (31 - __clz(unit));
-  if (row < p.M) p.partials[((long long)part * (p.N >> (31 - __clz(dim))) + head) * p.M + row] = sum;
+  float* at = p.partials + ((long long)part * (p.N >> (31 - __clz(dim))) + head) * p.M + row;
+  if (row < p.M && FAAR_DBG_OK(p, at, 4, p.partials, p.ext_partials, 5u)) *at = sum;
 }
 
 // FWD: residual, sum of squares, dY^T.
@@ -1052,7 +1054,7 @@ __device__ __forceinline__ void add_parts(uint32_t (&r)[16], uint32_t parts, int
 // a compile-time choice, so that the K-major kernels carry no trace of the other layout in their issue loops.  Bit 2 (REF): the
 // accumulator's rows are the result's columns; compiled in as well (as a branch it cost 0.1 us in every small product).  Bit 3
 // (REF): the gated product's epilogue, forward, or backward where B is N-contiguous.  Bit 4 (REF): heads turn by their position.  Bit 5
-// (REF): each row's softmax statistics leave with it.
+// (REF): each row's softmax statistics leave with it.  Bit 6 (REF, B untransposed): so do the row sums of the attention's gradient.
 // SHAPE: one of the tile forms (see Cfg).
 constexpr int MIN_SPLIT_BLOCKS = 12;            // contractions of fewer k blocks stay whole (see pick_splits)
 template <int MODE, int OPT, int SHAPE, int MN>
@@ -1511,7 +1513,8 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           }
           if constexpr (MN == STATS) {
             const int slots = (p.N + 127) / 128, slot = (n0 + col_begin) / 128;
-            if (o < p.M && n0 + col_begin < p.N) reinterpret_cast<float2*>(p.partials)[(long long)o * slots + slot] = make_float2(sm, ssum);
+            float2* at = reinterpret_cast<float2*>(p.partials) + (long long)o * slots + slot;
+            if (o < p.M && n0 + col_begin < p.N && FAAR_DBG_OK(p, at, 8, p.partials, p.ext_partials, 5u)) *at = make_float2(sm, ssum);
           }
         }
       }
@@ -1522,8 +1525,10 @@ faar_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     if (MODE == FAAR_GEMM_FWD || (MODE == FAAR_GEMM_BWD && p.fin_out2 != nullptr)) {
       warp_acc = faar_warp_sum(warp_acc);
       if (lane == 0) {
-        if (MODE == FAAR_GEMM_FWD) p.partials[blockIdx.x * C::EPI_WARPS + ew] = warp_acc;
-        else {
+        if (MODE == FAAR_GEMM_FWD) {
+          float* at = p.partials + blockIdx.x * C::EPI_WARPS + ew;
+          if (FAAR_DBG_OK(p, at, 4, p.partials, p.ext_partials, 5u)) *at = warp_acc;
+        } else {
           fin_warp[ew] = warp_acc;
           // one per weight that the warp may have had
           const int columns = SPLIT ? share_begin(BN, splits, split + 1) - share_begin(BN, splits, split) : BN;
@@ -2017,6 +2022,8 @@ int faar_launch_gemm(faar_ctx* ctx, const faar_gemm_args* args, int* n_partials_
     kp.ext_dyt = a->dYt ? ((long long)(a->M - 1) * a->ld_dyt + a->N) * 2 : 0;
     kp.ext_state = (long long)a->M * a->N * 4;
     kp.ext_wsoft = (long long)a->M * a->N * 2;
+    kp.ext_partials = a->stats ? (long long)a->M * ((a->N + 127) / 128) * (long long)sizeof(float2)
+                               : (a->sums ? (long long)a->M * (a->N / 16) * 4 : FAAR_MAX_PARTIALS * 4ll);
   }
   kp.Yout = a->Yout; kp.yout_dtype = a->yout_dtype; kp.ldy = a->ldy;
   kp.Yref = a->Yref; kp.yref_dtype = a->yref_dtype; kp.yref_t = a->yref_t;
