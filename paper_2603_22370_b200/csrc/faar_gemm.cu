@@ -366,7 +366,6 @@ struct KParams {
   int n_full;             // the first n_full tiles of the main columns are bn wide, the others come as two halves (tail split)
   uint32_t* status;
   long long ext_yout, ext_dyt, ext_state, ext_wsoft;   // bytes of Yout, dYt, each of V / m / u / dV, wsoft_next (debug checks)
-  long long ext_partials;                              // and of partials: loss sums, softmax statistics or row sums
   // REF / FWD
   void* Yout; int yout_dtype; long long ldy;
   const void* Yref; int yref_dtype;
@@ -398,6 +397,7 @@ struct KParams {
   double* fin_far_sums;             // and those sums, by CTA
   const float* fin_mse_partials; int fin_n_mse; float fin_scale_mse;
   float fin_scale_round; float* fin_out2;   // {L_MSE, L_round}; null = no final sums here
+  long long ext_partials;           // bytes of partials: loss sums, softmax statistics or row sums (debug checks)
 };
 
 // Tile t of the launch: the first n_full tiles of the raster are bn wide, each of the others is taken as two tiles of
