@@ -441,16 +441,18 @@ attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const float inv = l > 0.f ? 1.0f / l : 0.f;
       uint4* dst = reinterpret_cast<uint4*>(p.out + (seq0 + qi) * p.ldo + h * HD);
 #pragma unroll
-      for (int half = 0; half < HD / 32; ++half) {
-        float t[32];
-        ld32(t_o + 32u * half, t);
+      for (int pair = 0; pair < HD / 64; ++pair) {
+        float t[2][32];
+        ld32x2(t_o + 64u * pair, t_o + 64u * pair + 32u, t[0], t[1]);
         if (qi < p.S) {
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            dst[4 * half + c] = make_uint4(pack2(t[8 * c] * inv, t[8 * c + 1] * inv), pack2(t[8 * c + 2] * inv, t[8 * c + 3] * inv),
-                                           pack2(t[8 * c + 4] * inv, t[8 * c + 5] * inv), pack2(t[8 * c + 6] * inv, t[8 * c + 7] * inv));
+          for (int c = 0; c < 8; ++c) {
+            const float* v = &t[c >> 2][8 * (c & 3)];
+            dst[8 * pair + c] = make_uint4(pack2(v[0] * inv, v[1] * inv), pack2(v[2] * inv, v[3] * inv), pack2(v[4] * inv, v[5] * inv),
+                                           pack2(v[6] * inv, v[7] * inv));
+          }
         }
-        __syncwarp();
+        if (pair + 1 < HD / 64) __syncwarp();
       }
       if (qi < p.S) p.lse[((long long)b * p.H + h) * p.S + qi] = m + log2f(l);
     }
