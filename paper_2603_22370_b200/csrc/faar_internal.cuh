@@ -205,7 +205,7 @@ int faar_launch_harden_pack(faar_ctx*, const faar_shape*, const float* V, const 
 
 // dW products with chain rule and update on row-major operands dY [T, ldy], X [T, ldx]; the segments' rows stacked in dY's
 // columns.  hp has been checked.
-// beside: the launch before it on the stream is the input gradient of the same dY (a plain product), which it runs next to
+// beside: it runs next to the launches before it (see faar_gemm_args)
 int faar_bwd_group(faar_ctx*, int n_seg, faar_bwd_state* seg, int T, int K, const faar_hparams* hp, const void* dY, int64_t ldy,
                    const void* X, int64_t ldx, void* workspace, bool beside = false);
 int faar_check_hparams(const faar_hparams* hp, bool need_opt);
@@ -218,7 +218,10 @@ struct faar_gemm_args {
   int M, N, Kc;           // C[M,N] = A[M,Kc] * B[N,Kc]^T, both operands bf16 with Kc contiguous (REF: the launch may exchange them)
   const void* A; int64_t lda;
   const void* B; int64_t ldb;
-  int beside;             // BWD: 1: needs nothing of the launch before it, a plain product (see faar_pdl_wait_first)
+  int beside;             // BWD: 1: starts next to the launches before it, back to the last one that waits first (faar_pdl_wait_first).  Its
+                          // inputs must be complete when that one's wait is, nothing since may write what it reads or read what it
+                          // writes, and each launch since must join its predecessor before it ends: a plain product or dK / dV first, then
+                          // dQ and dW products in any number
   int ahead;              // FWD, BWD: 1: of what the launch before it on the stream writes it needs the A operand alone, and that launch lets
                           // it start once all before is complete (faar_pdl_wait_first)
   int whole;              // 1: the contraction is not split over CTA pairs (the order of its sums is that of one pair)

@@ -18,8 +18,9 @@ def beta_schedule(t: int, steps: int, beta0: float = 4.0, beta1: float = 32.0) -
     return beta0 if steps <= 1 else beta0 * (beta1 / beta0) ** (t / (steps - 1))
 
 
-#: runs of up to this many steps read X as it is (the same bits): the transposed copy costs 10 us at 512 x 2048 and 4096 tokens (more
-#: for larger batches) and gives at most 0.1 us a step back (30.62 against 30.70 us there; 72.5 against 72.1 at 2048 x 2048)
+#: runs of up to this many steps read X as it is (the same bits): the transposed copy costs about 10 us, more for larger batches, and
+#: gives up to 0.2 us a step back (1000 x 1040 at 777 tokens, 300 x 6976 at 500).  Whole runs, transposed -> as it is, us: 512 x 2048 at 4096
+#: tokens, 12 steps 479 -> 472, 100 steps 3049 -> 3042; 1000 x 1040 at 777 368 -> 354, 2084 -> 2085; 2048 x 2048 at 4096 996 -> 982, 8316 -> 8342
 ROW_MAJOR_STEPS = 100
 
 
