@@ -423,13 +423,16 @@ bool pick_wide4(int M, int N, int pairs) {
 }
 
 // Where one lane issues the producer's copies one by one, about 0.2 us a stage, instead of an elected lane of the converged warp
-// all at once.  Everywhere else the latter is 3 to 13 % faster; but with fewer than 128 rows of A and less than 128 KB of them in
-// all, and more pairs at work (in the last wave) than one die has, pairs that ask for a whole ring at a time hold one another up.
+// all at once, which is 3 to 13 % faster in general.  Up to three stages a tile: there is nothing to get ahead of (200 products of up to 300 rows,
+// at once 1.0 to 1.5 % slower, 4.9 % at most).  And with fewer than 128 rows of A and less than 128 KB of them in all, where pairs that
+// ask for a whole ring at a time hold one another up once more pairs are at work (in the last wave) than one die has, with up to 8 rows,
+// depending on the addresses, from a third of the pairs on (1 to 8 rows, 25 to 37 tiles, 0.90 to 1.12, on average 1.01 times as long).
 // One by one / at once, us: 8 rows, 8192 x 2048 5.8 / 6.3, x 8192 13.1 / 16.0, 16384 x 8192 23.0 / 31.4; 64 rows, 8192 x 2048 5.8 / 6.3,
-// x 4096 (128 KB) 8.1 / 7.5; 127 rows, 8192 x 2048 6.45 / 6.86, 128 rows 6.4 / 6.1; 8 rows, 4736 x 2048 (one die's pairs) 5.7 / 5.4,
+// x 4096 (128 KB) 8.1 / 7.5; 127 rows, 8192 x 2048 6.45 / 6.86, 128 rows 6.4 / 6.1; 1 row, 4096 x 2048 5.9 / 6.5, 64 rows 5.7 / 5.4,
 // 11008 x 2048 (86 tiles, 12 in the last wave) 8.2 / 7.7.
-bool copies_one_by_one(int M, int K, long long tiles, int pairs) {
-  return M < TM && (long long)M * K < 2 * 131072 && (tiles - 1) % pairs >= pairs / 2;
+bool copies_one_by_one(int M, int K, int bn, long long tiles, int pairs) {
+  if (K <= 3 * KS) return true;
+  return bn == 128 && M < TM && (long long)M * K < 2 * 131072 && (tiles - 1) % pairs >= (M <= 8 ? pairs / 3 : pairs / 2);
 }
 
 template <int BN>
@@ -459,7 +462,7 @@ int launch4(faar_ctx* ctx, const uint8_t* A, const uint8_t* sfa, const uint8_t* 
   if (!e) e = scale_map(ctx, &tmSB, sfb, (p.N + 127) / 128, p.k_tiles, C4::N_SFB);
   if (e) return e;
   const long long tiles = (long long)((p.M + 2 * TM - 1) / (2 * TM)) * ((p.N + BN - 1) / BN);
-  p.one_by_one = BN == 128 && copies_one_by_one(p.M, p.K, tiles, ctx->num_sms / 2);
+  p.one_by_one = copies_one_by_one(p.M, p.K, BN, tiles, ctx->num_sms / 2);
   cfg.gridDim = dim3(2 * (unsigned)(tiles < max_pairs ? tiles : max_pairs), 1, 1);
   faar_prof_scope ps(ctx, FAAR_K_NVFP4_GEMM);
   cudaError_t ce = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmSA, tmSB, p);

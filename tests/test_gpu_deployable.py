@@ -138,9 +138,11 @@ def test_own_nvfp4_gemm_with_wide_tiles(ctx, O, K, T):
     _check_nvfp4_gemm(ctx, O, K, T, seed=O + K, sample=128)
 
 
-@pytest.mark.parametrize("O,K,T", [(4736, 544, 8), (4737, 544, 8), (4864, 2048, 127), (4864, 2048, 128), (4864, 2080, 126), (9473, 288, 1)])
+@pytest.mark.parametrize("O,K,T", [(4736, 800, 9), (4737, 800, 9), (4864, 2048, 127), (4864, 2048, 128), (4864, 2080, 126), (9473, 800, 1),
+                                   (3072, 800, 8), (3073, 800, 8), (300, 768, 130), (300, 800, 130), (2560, 768, 2200)])
 def test_own_nvfp4_gemm_of_few_rows(ctx, O, K, T):
-    """Both ways to issue the copies on either side of their lines: 37 and 38 tiles, 127 and 128 rows, 128 KB of activations, a second wave."""
+    """Both ways to issue the copies on either side of their lines: 24 and 25, 37 and 38 tiles, 127 and 128 rows, 128 KB of activations, a second
+    wave, three stages and four, wide tiles."""
     _check_nvfp4_gemm(ctx, O, K, T, seed=T, sample=min(T, 16))
 
 
