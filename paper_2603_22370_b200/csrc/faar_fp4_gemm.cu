@@ -56,6 +56,7 @@ template <int BN> struct Cfg4 {
   static constexpr int COL_SF = COL_ACC1 + BN;
   static constexpr int SF_COLS = 4 * (KS / KI) * (1 + N_SFB);                // one stage's scales: 48 or 32 columns
   static_assert(COL_SF + 2 * SF_COLS <= TMEM_COLS, "tensor memory budget");
+  static_assert(BN % 64 == 0 && OVERLAP % 32 == 0, "the epilogue's pairs of chunks");
 };
 constexpr unsigned long long LIMIT_NS = 2000000000ull;
 
@@ -313,17 +314,8 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * C4::COL_ACC1);
       // the half whose columns the other accumulator shares starts at its shared end and reports when they are read
       const bool owner = C4::OVERLAP && half == (acc ^ 1);
-#pragma unroll 1
-      for (int i = 0; i < BN / 32; ++i) {
-        const int c = half == 0 ? 16 * i : BN - 16 - 16 * i;
+      auto store = [&](int c, const uint32_t (&r)[16]) {
         const int col = nt * BN + c;
-        uint32_t r[16];
-        ld16(trow + (uint32_t)c, r);
-        if (owner && i == C4::OVERLAP / 16 - 1) {
-          fence_before();
-          __syncwarp();
-          if (next && lane == 0) bar_arrive_cluster(map_to_leader(shared_free));
-        }
         if (row < p.M && col < p.N) {
           __nv_bfloat16* out = p.C + (long long)row * p.ldc + col;
           if (col + 16 <= p.N && ((reinterpret_cast<uintptr_t>(out) & 15) == 0)) {
@@ -363,6 +355,20 @@ nvfp4_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               if (col + q < p.N) out[q] = __float2bfloat16_rn(__uint_as_float(r[q]) * alpha);
           }
         }
+      };
+#pragma unroll 1
+      for (int i = 0; i < BN / 32; i += 2) {                 // two loads, then both chunks' stores: 64 rows, 28672 x 256 7.0 -> 6.3 us
+        const int c0 = half == 0 ? 16 * i : BN - 16 - 16 * i, c1 = half == 0 ? c0 + 16 : c0 - 16;
+        uint32_t r0[16], r1[16];
+        ld16(trow + (uint32_t)c0, r0);
+        ld16(trow + (uint32_t)c1, r1);
+        if (owner && i == C4::OVERLAP / 16 - 2) {
+          fence_before();
+          __syncwarp();
+          if (next && lane == 0) bar_arrive_cluster(map_to_leader(shared_free));
+        }
+        store(c0, r0);
+        store(c1, r1);
         __syncwarp();                                        // the next load of tensor memory wants the whole warp
       }
       fence_before();
