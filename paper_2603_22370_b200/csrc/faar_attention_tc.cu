@@ -1177,13 +1177,12 @@ int launch_fwd(faar_ctx* ctx, const TcParams& p, const void* q, int64_t ldq, con
 
 // Over how many CTAs the items of a key tile are dealt: up to `most` CTAs in all (four an SM with heads of 64, of which two run at
 // a time; one with heads of 128, where dQ next to this kernel has use for what is left), while the first key tile leaves each two
-// items, with heads of 128, whose exchange is twice as long, three of the first two CTAs (four items there, one CTA -> two, us: 8 heads on 4 x 32
-// tokens in groups of 4 15.0 -> 15.4, 8 on 2 x 96 in groups of 2 11.8 -> 12.0; six items, 4 heads on 192 in groups of 2 14.6 -> 13.0).  Backward call, one CTA a key tile -> two -> four, us: 32 / 8 heads of 64, 2 x 1000 tokens (128 key tiles) 112 -> 73 -> 70,
+// items.  Backward call, one CTA a key tile -> two -> four, us: 32 / 8 heads of 64, 2 x 1000 tokens (128 key tiles) 112 -> 73 -> 70,
 // 1 x 300 36 -> 24.6 -> 19, 4 x 2048 (512; one) 338 -> 361 -> 408; 16 / 8 heads of 128, 2 x 1000 (128; one) 64 -> 62.4 -> 81, in an
 // alignment step 2882 -> 2905 with two; 3 x 2048 (384; one) 250 -> 275 -> 343.
-int pick_parts(int head_dim, int most, int tiles, int longest) {
+int pick_parts(int most, int tiles, int longest) {
   int parts = 1;
-  while (parts < 4 && 2 * parts * tiles <= most && longest >= 4 * parts + (head_dim == 128 ? 2 : 0)) parts *= 2;
+  while (parts < 4 && 2 * parts * tiles <= most && longest >= 4 * parts) parts *= 2;
   return parts;
 }
 
@@ -1204,7 +1203,7 @@ int launch_bwd(faar_ctx* ctx, TcBwdParams& p, const void* q, int64_t ldq, const 
   if (!e) e = faar_allow_smem(ctx, (const void*)attn_dq_tc_kernel<HD>, Dq<HD>::SMEM);
   if (e) return e;
   const int tiles = (p.S + QT - 1) / QT;
-  p.parts = pick_parts(HD, ctx->num_sms * Dkv<HD>::CTAS * Dkv<HD>::CTAS, tiles * p.Hkv * p.B, p.H / p.Hkv * ((p.S + KT - 1) / KT));
+  p.parts = pick_parts(ctx->num_sms * Dkv<HD>::CTAS * Dkv<HD>::CTAS, tiles * p.Hkv * p.B, p.H / p.Hkv * ((p.S + KT - 1) / KT));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
