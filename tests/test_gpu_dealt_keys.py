@@ -23,7 +23,12 @@ def ctx():
     (1, 449, 1, 1),          # eight: four parts, two of which have nothing of the last key tile's one item
     (2, 130, 4, 1),          # the last key tile holds two keys
     (1, 300, 8, 2),
-    (1, 300, 16, 16),        # heads of 128: two parts, each finishing its columns in two turns, with the last key tile's rows cut inside a warp
 ])
 def test_dealt_key_tiles_match_the_oracle(ctx, B, S, H, HKV, D):
     _attention_case(ctx, B, S, H, HKV, D)
+
+
+def test_two_parts_whose_columns_take_two_turns(ctx):
+    """Heads of 128 and as many key tiles as leave room for two parts: each finishes its columns in two turns, here with the last key
+    tile's rows ending inside a warp."""
+    _attention_case(ctx, 1, 300, 16, 16, 128)
